@@ -85,9 +85,9 @@ attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CU
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(sgen + SM::bar_off + kBarBytes);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(sgen + SM::bar_off + kBarBytes + 4);
 
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = warp_index(), lane = threadIdx.x & 31;
   const int h = blockIdx.y;
-  const int L = c.len[h];
+  const int L = __shfl_sync(0xffffffffu, c.len[h], 0);      // warp-uniform for the role loops
 
   // ---- which rows and which key tiles ---------------------------------------------------------
   int q0, valid_rows, nt;
@@ -102,7 +102,7 @@ attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CU
       ntc = (L + BKT - 1) / BKT;
       list = nullptr;
     } else {
-      ntc = a.nsel[h];
+      ntc = __shfl_sync(0xffffffffu, a.nsel[h], 0);
       list = a.sel + static_cast<int64_t>(h) * a.sel_head_stride + static_cast<int64_t>(qa) * a.sel_stride;
     }
     nt = ntc + (SEG ? a.seg_tiles : 0);
@@ -110,7 +110,7 @@ attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CU
     const int f = blockIdx.z;
     q0 = f * a.rows_per_frame + blockIdx.x * 128;
     valid_rows = min(128, min(a.rows_per_frame - static_cast<int>(blockIdx.x) * 128, a.nq - q0));
-    if (a.keep_frames) keep_n = a.keep_frames[static_cast<int64_t>(h) * a.keep_frames_stride + f];
+    if (a.keep_frames) keep_n = __shfl_sync(0xffffffffu, a.keep_frames[static_cast<int64_t>(h) * a.keep_frames_stride + f], 0);
     nt = (keep_n + BKT - 1) / BKT;
     list = a.sel + static_cast<int64_t>(h) * a.sel_head_stride + static_cast<int64_t>(f) * a.sel_stride;
   }
@@ -306,25 +306,26 @@ attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CU
     }
   } else if (warp == kMmaWarp) {
     // ================================================================== MMA issue
-    if (lane == 0 && nt > 0) {
+    if (nt > 0) {
+      const uint32_t lead = elect_lane();
       constexpr uint32_t idesc_qk = make_idesc_bf16(128, BKT, 0);
       constexpr uint32_t idesc_pv = make_idesc_bf16(128, D, 1);
-      bool ok = mbar_wait(bar_q_full, 0, abort_flag, c.status);
+      bool ok = mbar_wait_warp(bar_q_full, 0, abort_flag, c.status);
       auto issue_s = [&](int j) -> bool {
         const int s = j & 1, g = j & 1, i = j >> 1;      // key stage, softmax group, tile index inside the group
-        if (!mbar_wait(bar_r_full + 8 * s, i & 1, abort_flag, c.status)) return false;
+        if (!mbar_wait_warp(bar_r_full + 8 * s, i & 1, abort_flag, c.status)) return false;
         // S[g] is free once group g holds the logits of its previous tile (j - 2) in registers
-        if (i > 0 && !mbar_wait(bar_s_empty + 8 * g, (i - 1) & 1, abort_flag, c.status)) return false;
+        if (i > 0 && !mbar_wait_warp(bar_s_empty + 8 * g, (i - 1) & 1, abort_flag, c.status)) return false;
         tc_fence_after();
         const uint32_t kt = ring_s + s * SM::kv_bytes;
 #pragma unroll
         for (int kk = 0; kk < D / 16; ++kk) {
           const uint64_t ad = make_smem_desc(q_s + (kk >> 2) * kQChunk + (kk & 3) * 32, 16, 1024);
           const uint64_t bd = make_smem_desc(kt + (kk >> 2) * (BKT * 128) + (kk & 3) * 32, 16, 1024);
-          umma_ss(tmem + g * BKT, ad, bd, idesc_qk, kk != 0);
+          umma_ss(tmem + g * BKT, ad, bd, idesc_qk, kk != 0, lead);
         }
-        umma_commit(bar_r_empty + 8 * s);
-        umma_commit(bar_s_full + 8 * g);
+        umma_commit(bar_r_empty + 8 * s, lead);
+        umma_commit(bar_s_full + 8 * g, lead);
         return true;
       };
       if (ok) ok = issue_s(0);
@@ -332,9 +333,9 @@ attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CU
       for (int j = 0; j < nt && ok; ++j) {
         if (j + 2 < nt) { ok = issue_s(j + 2); if (!ok) break; }
         const int s = 2 + (j & 1), g = j & 1, i = j >> 1;   // value stage, softmax group, tile index inside the group
-        ok = mbar_wait(bar_p_full + 8 * g, i & 1, abort_flag, c.status);
+        ok = mbar_wait_warp(bar_p_full + 8 * g, i & 1, abort_flag, c.status);
         if (!ok) break;
-        ok = mbar_wait(bar_r_full + 8 * s, i & 1, abort_flag, c.status);
+        ok = mbar_wait_warp(bar_r_full + 8 * s, i & 1, abort_flag, c.status);
         if (!ok) break;
         tc_fence_after();
         const uint32_t vt = ring_s + s * SM::kv_bytes;
@@ -343,10 +344,10 @@ attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CU
         for (int ks16 = 0; ks16 < BKT / 16; ++ks16) {
           const uint64_t ad = make_smem_desc(pt + (ks16 >> 2) * kQChunk + (ks16 & 3) * 32, 16, 1024);
           const uint64_t bd = make_smem_desc(vt + ks16 * 2048, BKT * 128, 1024);
-          umma_ss(tmem_o + g * D, ad, bd, idesc_pv, (i | ks16) != 0);
+          umma_ss(tmem_o + g * D, ad, bd, idesc_pv, (i | ks16) != 0, lead);
         }
-        umma_commit(bar_r_empty + 8 * s);
-        umma_commit(bar_pv_done + 8 * g);
+        umma_commit(bar_r_empty + 8 * s, lead);
+        umma_commit(bar_pv_done + 8 * g, lead);
       }
     }
   } else {

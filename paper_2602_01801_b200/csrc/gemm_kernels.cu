@@ -78,10 +78,10 @@ gemm_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__ CU
   constexpr int kCols = kTmemCols;                   // A_TMEM: one accumulator (128 columns) + A (64 columns)
   constexpr int kAcol = 128;                         // first TMEM column of A (A_TMEM)
 
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = warp_index(), lane = threadIdx.x & 31;
   const int h = blockIdx.y;
   const int m0 = blockIdx.x * 128;
-  const int L = c.len[h];
+  const int L = __shfl_sync(0xffffffffu, c.len[h], 0);
 
   // ---- tile range of this CTA ----------------------------------------------------------------
   int n_tiles;
@@ -172,21 +172,22 @@ gemm_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__ CU
         for (int k = max(0, it - NST); k < it; ++k) mbar_wait<kIssueWaitHintNs>(bar_full + 8 * (k % NST), (k / NST) & 1, abort_flag, c.status);
     } else if (warp == kGemmMmaWarp) {
       // ------------------------------------------------------------------ MMA issue
-      if (lane == 0) {
+      {
+        const uint32_t lead = elect_lane();
         constexpr uint32_t idesc = make_idesc_bf16(128, 128, 0);
         bool ok = true;
-        if (A_RES) ok = mbar_wait<kIssueWaitHintNs>(bar_afull, 0, abort_flag, c.status);
-        if (A_TMEM && ok) ok = mbar_wait<kIssueWaitHintNs>(bar_atm, 0, abort_flag, c.status);
+        if (A_RES) ok = mbar_wait_warp<kIssueWaitHintNs>(bar_afull, 0, abort_flag, c.status);
+        if (A_TMEM && ok) ok = mbar_wait_warp<kIssueWaitHintNs>(bar_atm, 0, abort_flag, c.status);
         int it = 0;
         for (int tl = 0; tl < ntl && ok; ++tl) {
           const int buf = A_TMEM ? 0 : (tl & 1), bph = A_TMEM ? (tl & 1) : ((tl >> 1) & 1);
-          ok = mbar_wait<kIssueWaitHintNs>(bar_tempty + 8 * buf, bph ^ 1, abort_flag, c.status);
+          ok = mbar_wait_warp<kIssueWaitHintNs>(bar_tempty + 8 * buf, bph ^ 1, abort_flag, c.status);
           if (!ok) break;
           tc_fence_after();
           const uint32_t d_t = tmem + buf * 128;
           for (int kc = 0; kc < nkc; ++kc, ++it) {
             const int s = it % NST;
-            ok = mbar_wait<kIssueWaitHintNs>(bar_full + 8 * s, (it / NST) & 1, abort_flag, c.status);
+            ok = mbar_wait_warp<kIssueWaitHintNs>(bar_full + 8 * s, (it / NST) & 1, abort_flag, c.status);
             if (!ok) break;
             tc_fence_after();
             const uint32_t st_s = ring_s + s * SM::stage_bytes;
@@ -196,12 +197,12 @@ gemm_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__ CU
             for (int k4 = 0; k4 < 4; ++k4) {
               const uint64_t ad = make_smem_desc(a_c + k4 * 32, 16, 1024);
               const uint64_t bd = make_smem_desc(b_c + k4 * 32, 16, 1024);
-              if (A_TMEM) umma_ts(d_t, tmem + kAcol + kc * 32 + k4 * 8, bd, idesc, (kc | k4) != 0);
-              else umma_ss(d_t, ad, bd, idesc, (kc | k4) != 0);
+              if (A_TMEM) umma_ts(d_t, tmem + kAcol + kc * 32 + k4 * 8, bd, idesc, (kc | k4) != 0, lead);
+              else umma_ss(d_t, ad, bd, idesc, (kc | k4) != 0, lead);
             }
-            umma_commit(bar_empty + 8 * s);
+            umma_commit(bar_empty + 8 * s, lead);
           }
-          if (ok) umma_commit(bar_tfull + 8 * buf);
+          if (ok) umma_commit(bar_tfull + 8 * buf, lead);
         }
       }
     } else {
@@ -398,11 +399,11 @@ t1_pair_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
   volatile int* abort_flag = reinterpret_cast<volatile int*>(sgen + SM::bar_off + 16 * NST + 44);
   static_assert(16 * NST + 48 <= 256, "barrier area");
 
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = warp_index(), lane = threadIdx.x & 31;
   const uint32_t rank = cluster_ctarank();            // 0: issues the MMAs, 1: its peer
   const int h = blockIdx.y;
   const int m0 = blockIdx.x * 128;
-  const int L = c.len[h];
+  const int L = __shfl_sync(0xffffffffu, c.len[h], 0);
 
   const int n_tiles = (L + 127) >> 7;
   const int per = (n_tiles + gridDim.z - 1) / gridDim.z;
@@ -475,19 +476,20 @@ t1_pair_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
       }
     } else if (warp == kGemmMmaWarp) {
       // ------------------------------------------------------------------ MMA issue (even CTA only)
-      if (lane == 0 && rank == 0) {
+      if (rank == 0) {
+        const uint32_t lead = elect_lane();
         constexpr uint32_t idesc = make_idesc_bf16(256, 128, 0);
-        bool ok = mbar_wait<kIssueWaitHintNs>(bar_afull, 0, abort_flag, c.status);
+        bool ok = mbar_wait_warp<kIssueWaitHintNs>(bar_afull, 0, abort_flag, c.status);
         int it = 0;
         for (int tl = 0; tl < ntl && ok; ++tl) {
           const int buf = tl & 1;
-          ok = mbar_wait<kIssueWaitHintNs>(bar_tempty + 8 * buf, ((tl >> 1) & 1) ^ 1, abort_flag, c.status);
+          ok = mbar_wait_warp<kIssueWaitHintNs>(bar_tempty + 8 * buf, ((tl >> 1) & 1) ^ 1, abort_flag, c.status);
           if (!ok) break;
           tc_fence_after();
           const uint32_t d_t = tmem + buf * 128;
           for (int kc = 0; kc < nkc; ++kc, ++it) {
             const int s = it % NST;
-            ok = mbar_wait<kIssueWaitHintNs>(bar_full + 8 * s, (it / NST) & 1, abort_flag, c.status);
+            ok = mbar_wait_warp<kIssueWaitHintNs>(bar_full + 8 * s, (it / NST) & 1, abort_flag, c.status);
             if (!ok) break;
             tc_fence_after();
             const uint32_t a_c = a_s + kc * kChunkBytes;
@@ -496,11 +498,11 @@ t1_pair_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
             for (int k4 = 0; k4 < 4; ++k4) {
               const uint64_t ad = make_smem_desc(a_c + k4 * 32, 16, 1024);
               const uint64_t bd = make_smem_desc(b_c + k4 * 32, 16, 1024);
-              umma_ss_pair(d_t, ad, bd, idesc, (kc | k4) != 0);
+              umma_ss_pair(d_t, ad, bd, idesc, (kc | k4) != 0, lead);
             }
-            umma_commit_pair(bar_empty + 8 * s);
+            umma_commit_pair(bar_empty + 8 * s, lead);
           }
-          if (ok) umma_commit_pair(bar_tfull + 8 * buf);
+          if (ok) umma_commit_pair(bar_tfull + 8 * buf, lead);
         }
       }
     } else {

@@ -42,12 +42,14 @@ struct Smem {
 __host__ __device__ constexpr uint32_t make_idesc_e4m3(int m, int n) {
   return (1u << 4) | (static_cast<uint32_t>(n >> 3) << 17) | (static_cast<uint32_t>(m >> 4) << 24);
 }
-__device__ __forceinline__ void umma_ss_f8(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc, uint32_t accumulate) {
+__device__ __forceinline__ void umma_ss_f8(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc, uint32_t accumulate,
+                                           uint32_t lead) {
   asm volatile(
-      "{\n\t.reg .pred p;\n\t"
+      "{\n\t.reg .pred p, q;\n\t"
       "setp.ne.b32 p, %4, 0;\n\t"
-      "tcgen05.mma.cta_group::1.kind::f8f6f4 [%0], %1, %2, %3, p;\n\t}"
-      ::"r"(d_tmem), "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
+      "setp.ne.b32 q, %5, 0;\n\t"
+      "@q tcgen05.mma.cta_group::1.kind::f8f6f4 [%0], %1, %2, %3, p;\n\t}"
+      ::"r"(d_tmem), "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate), "r"(lead)
       : "memory");
 }
 
@@ -212,10 +214,10 @@ search8_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
   float* kn_s = reinterpret_cast<float*>(sgen + Smem::kn_off);
   static_assert(16 * kStages + 48 <= 256, "barrier area");
 
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = warp_index(), lane = threadIdx.x & 31;
   const int h = blockIdx.y;
   const int m0 = blockIdx.x * 128;
-  const int L = COLMAX ? g.cols_b : c.len[h];
+  const int L = COLMAX ? g.cols_b : __shfl_sync(0xffffffffu, c.len[h], 0);
   const int n_tiles = (L + 127) >> 7;
   const int per = (n_tiles + gridDim.z - 1) / gridDim.z;
   const int t0 = blockIdx.z * per;
@@ -287,13 +289,14 @@ search8_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
         for (int k = max(0, ntl - kStages); k < ntl; ++k) mbar_wait(bar_full + 8 * (k % kStages), (k / kStages) & 1, abort_flag, c.status);
     } else if (warp == kMma) {
       // ------------------------------------------------------------------ MMA issue
-      if (lane == 0) {
+      {
+        const uint32_t lead = elect_lane();
         constexpr uint32_t idesc = make_idesc_e4m3(128, 128);
-        bool ok = mbar_wait(bar_afull, 0, abort_flag, c.status);
+        bool ok = mbar_wait_warp(bar_afull, 0, abort_flag, c.status);
         for (int tl = 0; tl < ntl && ok; ++tl) {
           const int buf = tl & 1, s = tl % kStages;
-          ok = mbar_wait(bar_tempty + 8 * buf, ((tl >> 1) & 1) ^ 1, abort_flag, c.status) &&
-               mbar_wait(bar_full + 8 * s, (tl / kStages) & 1, abort_flag, c.status);
+          ok = mbar_wait_warp(bar_tempty + 8 * buf, ((tl >> 1) & 1) ^ 1, abort_flag, c.status) &&
+               mbar_wait_warp(bar_full + 8 * s, (tl / kStages) & 1, abort_flag, c.status);
           if (!ok) break;
           tc_fence_after();
           const uint32_t b_c = ring_s + s * kTile;
@@ -301,10 +304,10 @@ search8_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
           for (int k4 = 0; k4 < 4; ++k4) {                       // 32 code bytes (K = 32) per instruction
             const uint64_t ad = make_smem_desc(a_s + k4 * 32, 16, 1024);
             const uint64_t bd = make_smem_desc(b_c + k4 * 32, 16, 1024);
-            umma_ss_f8(tmem + buf * 128, ad, bd, idesc, k4 != 0);
+            umma_ss_f8(tmem + buf * 128, ad, bd, idesc, k4 != 0, lead);
           }
-          umma_commit(bar_empty + 8 * s);
-          umma_commit(bar_tfull + 8 * buf);
+          umma_commit(bar_empty + 8 * s, lead);
+          umma_commit(bar_tfull + 8 * buf, lead);
         }
       }
     } else {
