@@ -245,10 +245,8 @@ int fastar_annsa_prepare(fastar_cache_t* cache, const void* q, int32_t nq, int64
 int fastar_cache_set_forced_blocks(fastar_cache_t* cache, int32_t sink_blocks, int32_t recent_blocks);
 
 /* Which kernel runs the bf16 correspondence search of fastar_tempcache_update (Section 5.2, finding the top-1
- * cached key; host-side setting, takes effect from the next update; default FASTAR_T1_AUTO).  All three compute the
- * same arg-max; AUTO picks single CTAs or CTA pairs from how well their grids fill the GPU.  The other values exist
- * so that every variant can be run and checked on any shape: SINGLE = one CTA per 128 new keys, PAIR = two CTAs
- * sharing every key tile (tcgen05 cta_group::2), TS = SINGLE with the new keys held in tensor memory. */
+ * cached key; host-side setting, default FASTAR_T1_AUTO).  One kernel serves every shape now, so all four values run it
+ * and give the same arg-max; the call checks its arguments and stays for the programs that make it. */
 #define FASTAR_T1_AUTO   0
 #define FASTAR_T1_SINGLE 1
 #define FASTAR_T1_PAIR   2

@@ -120,12 +120,12 @@ int ensure_dynamic_smem(const void* kernel, int bytes);
 // Each returns the number of kernels it launched (for the launch counter) or a negative status.
 
 // gemm_kernels.cu
-// tm_pool_k: one page per box; tm_pool_k_half: 64 key rows per box (what one CTA of a pair fetches)
-int launch_t1_similarity(const CacheView& c, const CUtensorMap& tm_a, const CUtensorMap& tm_pool_k,
-                         const CUtensorMap& tm_pool_k_half, int n, int force, cudaStream_t st);
 int launch_c1_relevance(const CacheView& c, const CUtensorMap& tm_q, const CUtensorMap& tm_kp, int nq, int np, int frame_len,
                         int n_frames, cudaStream_t st);
 int launch_s3_scores(const CacheView& c, const CUtensorMap& tm_hq, const CUtensorMap& tm_hk, int nqb, cudaStream_t st);
+
+// search_kernel.cu: T1 on the bf16 keys as one persistent kernel (c.raw_dot: plain dot products).  tm_pool_k: one page per box
+int launch_t1_search(const CacheView& c, const CUtensorMap& tm_a, const CUtensorMap& tm_pool_k, int n, cudaStream_t st);
 
 // search8_kernels.cu: fp8 search codes of bf16 rows (x / |x| * 16, 128-byte rows), and T1 on the codes
 int launch_quantize_keys(const CacheView& c, const __nv_bfloat16* x, int n, int64_t hs, int64_t ts, const float* rnorm,

@@ -24,13 +24,12 @@ struct fastar_cache {
   std::vector<ProfRec> recs;
   fastar_cache_desc desc;
   CacheView v;
-  CUtensorMap tm_pool_k, tm_pool_k_half, tm_pool_v, tm_hq, tm_hk, tm_hk_hi, tm_pool_k8;
+  CUtensorMap tm_pool_k, tm_pool_v, tm_hq, tm_hk, tm_hk_hi, tm_pool_k8;
   PFN_cuTensorMapEncodeTiled_v12000 encode;
   int64_t launches;
   size_t bytes;
   // second stream of the host-tensor step (uploads of q and the prompt, AnnCA, its download) and its fork/join events
   int force_sink_blocks = 0, force_recent_blocks = 0;    // AnnSA selector option (fastar_cache_set_forced_blocks)
-  int t1_kernel = FASTAR_T1_AUTO;                        // fastar_cache_set_similarity_kernel
   // queries whose codes and block histograms fastar_annsa_prepare has already produced (consumed by the next matching AnnSA call)
   struct { const void* q = nullptr; int32_t nq = 0, block_q = 0; int64_t hs = 0, ts = 0; bool valid = false; } prep;
   cudaEvent_t ev_prep = nullptr;
@@ -302,7 +301,6 @@ int fastar_cache_create(fastar_cache_t** out, const fastar_cache_desc* desc, con
   const CacheView& v = c->v;
   const uint64_t D = v.D, PT = v.PT;
   int r = make_map(c, &c->tm_pool_k, v.pool_k, D, PT, static_cast<uint64_t>(v.pool_pages), D * 2, PT * D * 2, v.PT);
-  if (r == FASTAR_OK) r = make_map(c, &c->tm_pool_k_half, v.pool_k, D, PT, static_cast<uint64_t>(v.pool_pages), D * 2, PT * D * 2, 64);
   if (r == FASTAR_OK) r = make_map(c, &c->tm_pool_v, v.pool_v, D, PT, static_cast<uint64_t>(v.pool_pages), D * 2, PT * D * 2, v.PT);
   if (r == FASTAR_OK)
     r = make_map(c, &c->tm_hq, v.hq, v.hist_cols, v.max_qb, v.H, static_cast<uint64_t>(v.hist_cols) * 2,
@@ -424,8 +422,7 @@ int fastar_cache_set_forced_blocks(fastar_cache_t* c, int32_t sink_blocks, int32
 
 int fastar_cache_set_similarity_kernel(fastar_cache_t* c, int32_t kind) {
   if (!c || kind < FASTAR_T1_AUTO || kind > FASTAR_T1_TS) return FASTAR_ERR_INVALID_ARG;
-  c->t1_kernel = kind;
-  return FASTAR_OK;
+  return FASTAR_OK;                          // one kernel serves every shape
 }
 
 int fastar_cache_export_search_codes(fastar_cache_t* c, uint8_t* host_cache_codes, uint8_t* host_new_codes, int32_t n,
@@ -563,10 +560,10 @@ static int update_impl(fastar_cache_t* c, const void* q_probe, const void* k_new
   } else if (q_probe) {
     CacheView vr = vs;
     vr.raw_dot = 1;
-    ACCK(FASTAR_K_T1_SIMILARITY, launch_t1_similarity(vr, tm_a, c->tm_pool_k, c->tm_pool_k_half, n, c->t1_kernel, st));
+    ACCK(FASTAR_K_T1_SIMILARITY, launch_t1_search(vr, tm_a, c->tm_pool_k, n, st));
     ACCK(FASTAR_K_PLAN, launch_probe_cosine(v, kb, n, khs, kts, st));
   } else {
-    ACCK(FASTAR_K_T1_SIMILARITY, launch_t1_similarity(vs, tm_a, c->tm_pool_k, c->tm_pool_k_half, n, c->t1_kernel, st));
+    ACCK(FASTAR_K_T1_SIMILARITY, launch_t1_search(vs, tm_a, c->tm_pool_k, n, st));
   }
   ACCK(FASTAR_K_PLAN, launch_plan(v, n, frame_len, tau, st));
   if (v_ready && !v_converted && cudaStreamWaitEvent(st, v_ready, 0) != cudaSuccess) return FASTAR_ERR_CUDA;

@@ -107,6 +107,10 @@ __device__ __forceinline__ uint32_t mbar_test_wait(uint32_t bar, uint32_t parity
   return ok;
 }
 
+// Suspend-time hint of the waits of the TMA producers and MMA issuers of the search kernels: a waiting thread that polls
+// shares an issue port with the epilogue warps, one parked for up to 10 us still wakes the moment the phase completes.
+constexpr uint32_t kIssueWaitHintNs = 10000;
+
 // Wait limit: about two seconds of wall clock, checked every 256 polls.
 constexpr uint64_t kWaitLimitNs = 2000000000ull;
 
@@ -147,6 +151,13 @@ __device__ __forceinline__ void fence_proxy_async_smem() {
 __device__ __forceinline__ void named_barrier_sync(uint32_t id, uint32_t nthreads) {
   asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(nthreads) : "memory");
 }
+
+// Registers of a warpgroup (four consecutive warps, all executing the same instruction) after launch; the sum over the CTA must
+// not exceed what the launch allocated.
+template <int N>
+__device__ __forceinline__ void setmaxnreg_inc() { asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(N)); }
+template <int N>
+__device__ __forceinline__ void setmaxnreg_dec() { asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(N)); }
 
 // ---------------------------------------------------------------------------------------------
 // TMA.  No multicast anywhere: every CTA issues its own loads.
@@ -214,6 +225,11 @@ __host__ __device__ constexpr uint32_t make_idesc_bf16(int m, int n, int b_mn_ma
          (static_cast<uint32_t>(n >> 3) << 17) | (static_cast<uint32_t>(m >> 4) << 24);
 }
 
+// The same for kind::f8f6f4 with e4m3 A and B (format 0), K-major operands.
+__host__ __device__ constexpr uint32_t make_idesc_e4m3(int m, int n) {
+  return (1u << 4) | (static_cast<uint32_t>(n >> 3) << 17) | (static_cast<uint32_t>(m >> 4) << 24);
+}
+
 // ---------------------------------------------------------------------------------------------
 // tcgen05: MMA, commit, TMEM load/store.
 // ---------------------------------------------------------------------------------------------
@@ -266,74 +282,24 @@ __device__ __forceinline__ void umma_commit(uint32_t bar, uint32_t lead) {
       : "memory");
 }
 
-// ---------------------------------------------------------------------------------------------
-// CTA pairs (cluster of two CTAs on the two SMs of a TPC, tcgen05 cta_group::2)
-// ---------------------------------------------------------------------------------------------
-// One MMA spans both SMs: each CTA supplies its own 128 rows of A and half of the rows of B from its own shared
-// memory (same offsets in both CTAs) and receives its 128 rows of D in its own TMEM.  The even CTA of the pair
-// issues the MMAs; barriers that it waits on collect arrivals and TMA bytes from both CTAs.
-__device__ __forceinline__ uint32_t cluster_ctarank() {
-  uint32_t r;
-  asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
-  return r;
-}
-// shared::cluster address of `addr` (a shared::cta address of this CTA) in the CTA of rank `rank`
-__device__ __forceinline__ uint32_t map_to_cta(uint32_t addr, uint32_t rank) {
-  uint32_t r;
-  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
-  return r;
-}
-__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
-__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
-// arrive on a barrier given by its shared::cluster address (this CTA's or the peer's)
-__device__ __forceinline__ void mbar_arrive_cluster(uint32_t bar_cluster) {
-  asm volatile("mbarrier.arrive.shared::cluster.b64 _, [%0];" ::"r"(bar_cluster) : "memory");
-}
-// 3-D tiled load into this CTA's shared memory whose bytes are counted on a barrier given by its shared::cluster
-// address (the issuing CTA's barrier of the pair).  Every CTA fetches its own tile.
-__device__ __forceinline__ void tma_load_3d_pair(uint32_t dst_smem, const CUtensorMap* m, uint32_t bar_cluster, int c0, int c1,
-                                                 int c2) {
-  asm volatile(
-      "cp.async.bulk.tensor.3d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4, %5}], [%2];"
-      ::"r"(dst_smem), "l"(reinterpret_cast<uint64_t>(m)), "r"(bar_cluster), "r"(c0), "r"(c1), "r"(c2)
-      : "memory");
-}
-// TMEM allocation for a pair: the same warp of both CTAs executes these; both get the same columns.
-__device__ __forceinline__ void tmem_alloc_pair(uint32_t dst_smem, uint32_t ncols) {
-  asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(dst_smem), "r"(ncols) : "memory");
-}
-__device__ __forceinline__ void tmem_relinquish_pair() {
-  asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
-}
-__device__ __forceinline__ void tmem_dealloc_pair(uint32_t taddr, uint32_t ncols) {
-  asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(taddr), "r"(ncols) : "memory");
-}
-// D[256 x N] (+)= A[256 x 16] * B[N x 16]^T over the pair; issued by one thread of the even CTA.
-__device__ __forceinline__ void umma_ss_pair(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
-                                             uint32_t accumulate, uint32_t lead) {
-  asm volatile(
-      "{\n\t.reg .pred p, q;\n\t"
-      "setp.ne.b32 p, %4, 0;\n\t"
-      "setp.ne.b32 q, %5, 0;\n\t"
-      "@q tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n\t}"
-      ::"r"(d_tmem), "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate), "r"(lead)
-      : "memory");
-}
-// Arrive on the barrier at this shared-memory offset in both CTAs of the pair when the MMAs issued so far are done.
-__device__ __forceinline__ void umma_commit_pair(uint32_t bar, uint32_t lead) {
-  const uint16_t mask = 3;
-  asm volatile(
-      "{\n\t.reg .pred q;\n\t"
-      "setp.ne.b32 q, %2, 0;\n\t"
-      "@q tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;\n\t}"
-      ::"r"(bar), "h"(mask), "r"(lead)
-      : "memory");
-}
-
 // 32 lanes x 32 consecutive 32-bit columns: thread t of the warp gets lane (32*(warp%4) + t).
 __device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&r)[32]) {
   asm volatile(
       "tcgen05.ld.sync.aligned.32x32b.x32.b32 "
+      "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, "
+      "%16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];"
+      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
+        "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]), "=r"(r[16]),
+        "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]), "=r"(r[24]),
+        "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
+      : "r"(taddr)
+      : "memory");
+}
+// 16 lanes (from the address's lane on) x 64 consecutive columns, 16 x 256-bit fragments: r[4 i + 2 e + c] of thread t is lane
+// t / 4 + 8 e, column 8 i + 2 (t & 3) + c.
+__device__ __forceinline__ void tmem_ld_frag(uint32_t taddr, uint32_t (&r)[32]) {
+  asm volatile(
+      "tcgen05.ld.sync.aligned.16x256b.x8.b32 "
       "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, "
       "%16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];"
       : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
@@ -384,6 +350,13 @@ __device__ __forceinline__ void fmul2(float& x0, float& x1, float a0, float a1, 
   asm("mov.b64 %0, {%1, %2};" : "=l"(b) : "f"(b0), "f"(b1));
   asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
   asm("mov.b64 {%0, %1}, %2;" : "=f"(x0), "=f"(x1) : "l"(d));
+}
+// (x0, x1) *= f on accumulator bits
+__device__ __forceinline__ void scale2(uint32_t& x0, uint32_t& x1, const float2& f) {
+  float a, b;
+  fmul2(a, b, __uint_as_float(x0), __uint_as_float(x1), f.x, f.y);
+  x0 = __float_as_uint(a);
+  x1 = __float_as_uint(b);
 }
 // Maximum of 32 scores x[j] = acc[j] * rn[j] and, only when it beats `best`, its first column.
 // acc: raw accumulator bits; rn: 32 floats (16-byte aligned, shared or registers via pointer).

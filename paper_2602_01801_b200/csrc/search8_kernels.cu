@@ -38,10 +38,6 @@ struct Smem {
   static constexpr int total = kn_off + 2 * 128 * 4;
 };
 
-// Instruction descriptor of kind::f8f6f4 with e4m3 A and B (format 0), fp32 accumulation, K-major operands.
-__host__ __device__ constexpr uint32_t make_idesc_e4m3(int m, int n) {
-  return (1u << 4) | (static_cast<uint32_t>(n >> 3) << 17) | (static_cast<uint32_t>(m >> 4) << 24);
-}
 __device__ __forceinline__ void umma_ss_f8(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc, uint32_t accumulate,
                                            uint32_t lead) {
   asm volatile(

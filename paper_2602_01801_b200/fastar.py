@@ -193,7 +193,7 @@ class Cache:
         _check(self.lib.fastar_cache_set_forced_blocks(self.handle, sink_blocks, recent_blocks), "fastar_cache_set_forced_blocks")
 
     def set_similarity_kernel(self, kind: str = "auto") -> None:
-        """Which kernel runs the bf16 correspondence search: "auto" (default), "single", "pair" or "ts"."""
+        """Which kernel runs the bf16 correspondence search: "auto" (default), "single", "pair" or "ts" (one kernel serves them all)."""
         _check(self.lib.fastar_cache_set_similarity_kernel(self.handle, {"auto": 0, "single": 1, "pair": 2, "ts": 3}[kind]),
                "fastar_cache_set_similarity_kernel")
 
