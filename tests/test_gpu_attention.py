@@ -1,0 +1,51 @@
+"""The attention kernel's tile loop: one to many key tiles (both soft-max groups, the hand-over of the running maximum between them),
+maxima that rise late or by far, dead and weighted slots, an un-cached segment, ragged query blocks."""
+import math
+
+import numpy as np
+import pytest
+
+from paper_2602_01801_b200 import synth
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("rise", [0.0, 6.0, 60.0])
+@pytest.mark.parametrize("d,pt,nq,length,seg", [(128, 128, 1, 1, 0), (128, 128, 129, 128, 0), (128, 64, 200, 65, 0), (64, 128, 128, 300, 7),
+                                                (64, 64, 77, 1000, 130), (128, 128, 300, 4200, 300), (128, 64, 64, 700, 64)])
+def test_tiles_and_maxima(d, pt, nq, length, seg, rise):
+    import torch
+    from paper_2602_01801_b200 import fastar
+    rng = np.random.default_rng(length + d)
+    H, cap = 2, -(-max(length, nq, 128) // 128) * 128 + 128
+    q = synth.round_bf16(rng.standard_normal((H, nq, d)).astype(np.float32))
+    # the logit of key j against every query grows with j by about `rise` from the first key to the last: q . mean direction
+    u = q.mean((0, 1)) / np.linalg.norm(q.mean((0, 1)))
+    q = synth.round_bf16(q + 3.0 * u)
+    ramp = (np.arange(cap + seg) / max(1, length + seg - 1)) * rise * math.sqrt(d) / 3.0
+    k = synth.round_bf16((0.5 * rng.standard_normal((H, cap + seg, d)) + ramp[None, :, None] * u).astype(np.float32))
+    v = synth.round_bf16(rng.standard_normal((H, cap + seg, d)).astype(np.float32))
+    count = rng.integers(1, 9, (H, cap)).astype(np.int32)
+    lens = np.array([length, max(0, length - 61)])
+    cache = fastar.Cache(H, d, cap, pt, rng.standard_normal((32, d)).astype(np.float32), max_tokens=max(nq, seg, 1))
+    cache.import_state(fastar.bf16_bits(k[:, :cap]), fastar.bf16_bits(v[:, :cap]), lens, count)
+    dq = fastar.to_device(q)
+    if seg:
+        out = cache.annsa_segment(dq, fastar.to_device(k[:, cap:]), fastar.to_device(v[:, cap:]), 128, cap // pt)["out"]
+    else:
+        out = cache.annsa(dq, 128, cap // pt)["out"]
+    assert cache.status() == 0
+    for h in range(H):
+        L = int(lens[h])
+        kk = np.concatenate([k[h, :L], k[h, cap:]]).astype(np.float64)
+        vv = np.concatenate([v[h, :L], v[h, cap:]]).astype(np.float64)
+        got = out[h].float().cpu().numpy()
+        if len(kk) == 0:
+            assert (got == 0).all()
+            continue
+        s = q[h].astype(np.float64) @ kk.T / math.sqrt(d) + np.log(np.concatenate([count[h, :L], np.ones(seg)]))
+        p = np.exp(s - s.max(1, keepdims=True))
+        want = (p / p.sum(1, keepdims=True)) @ vv
+        # probabilities and output rounded to 8 significant bits (2^-8 each), sums in fp32: 2^-7 of the largest value averaged
+        assert np.abs(got - want).max() <= 2.0 ** -7 * np.abs(vv).max()
+        assert np.linalg.norm(got - want) <= 1e-2 * np.linalg.norm(want)
