@@ -95,33 +95,12 @@ attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CU
 
   const int warp = warp_index(), lane = threadIdx.x & 31;
   const int h = blockIdx.y;
-  const int L = __shfl_sync(0xffffffffu, c.len[h], 0);      // warp-uniform for the role loops
 
-  // ---- which rows and which key tiles ---------------------------------------------------------
-  int q0, valid_rows, nt;
-  int ntc = 0;                          // paged mode: tiles taken from the cache; tiles [ntc, nt) are segment tiles
-  int keep_n = a.keep;                  // gather mode: kept prompt tokens of this CTA's frame
-  const int32_t* list;
-  if (!GATHER) {
-    const int qa = blockIdx.x;
-    q0 = qa * a.block_q;
-    valid_rows = min(a.block_q, a.nq - q0);
-    if (a.sel == nullptr) {
-      ntc = (L + BKT - 1) / BKT;
-      list = nullptr;
-    } else {
-      ntc = __shfl_sync(0xffffffffu, a.nsel[h], 0);
-      list = a.sel + static_cast<int64_t>(h) * a.sel_head_stride + static_cast<int64_t>(qa) * a.sel_stride;
-    }
-    nt = ntc + (SEG ? a.seg_tiles : 0);
-  } else {
-    const int f = blockIdx.z;
-    q0 = f * a.rows_per_frame + blockIdx.x * 128;
-    valid_rows = min(128, min(a.rows_per_frame - static_cast<int>(blockIdx.x) * 128, a.nq - q0));
-    if (a.keep_frames) keep_n = __shfl_sync(0xffffffffu, a.keep_frames[static_cast<int64_t>(h) * a.keep_frames_stride + f], 0);
-    nt = (keep_n + BKT - 1) / BKT;
-    list = a.sel + static_cast<int64_t>(h) * a.sel_head_stride + static_cast<int64_t>(f) * a.sel_stride;
-  }
+  // ---- which rows ------------------------------------------------------------------------------
+  const int q0 = GATHER ? static_cast<int>(blockIdx.z) * a.rows_per_frame + static_cast<int>(blockIdx.x) * 128
+                        : static_cast<int>(blockIdx.x) * a.block_q;
+  const int valid_rows = GATHER ? min(128, min(a.rows_per_frame - static_cast<int>(blockIdx.x) * 128, a.nq - q0))
+                                : min(a.block_q, a.nq - q0);
   if (valid_rows <= 0) return;          // uniform for the CTA; nothing allocated yet
 
   // one thread per barrier
@@ -144,6 +123,28 @@ attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CU
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = *tmem_slot;
+  chain_wait();
+
+  // ---- which key tiles (warp-uniform for the role loops) --------------------------------------
+  int nt;
+  int ntc = 0;                          // paged mode: tiles taken from the cache; tiles [ntc, nt) are segment tiles
+  int keep_n = a.keep;                  // gather mode: kept prompt tokens of this CTA's frame
+  const int L = GATHER ? 0 : __shfl_sync(0xffffffffu, c.len[h], 0);
+  const int32_t* list = nullptr;
+  if (!GATHER) {
+    if (a.sel == nullptr) {
+      ntc = (L + BKT - 1) / BKT;
+    } else {
+      ntc = __shfl_sync(0xffffffffu, a.nsel[h], 0);
+      list = a.sel + static_cast<int64_t>(h) * a.sel_head_stride + static_cast<int64_t>(blockIdx.x) * a.sel_stride;
+    }
+    nt = ntc + (SEG ? a.seg_tiles : 0);
+  } else {
+    const int f = blockIdx.z;
+    if (a.keep_frames) keep_n = __shfl_sync(0xffffffffu, a.keep_frames[static_cast<int64_t>(h) * a.keep_frames_stride + f], 0);
+    nt = (keep_n + BKT - 1) / BKT;
+    list = a.sel + static_cast<int64_t>(h) * a.sel_head_stride + static_cast<int64_t>(f) * a.sel_stride;
+  }
 
   // Gather mode with a single key tile (the usual AnnCA case, keep <= BKT): all threads fetch the kept rows
   // of K_p and V_p at once, instead of leaving 2 x BKT x D x 2 bytes of 16-byte gathers to one warp.
@@ -535,7 +536,7 @@ static int launch_attn(const CUtensorMap& tq, const CUtensorMap& tk, const CUten
   auto kern = attn_kernel<D, BKT, GATHER, SEG>;
   const int cfg = ensure_dynamic_smem(reinterpret_cast<const void*>(kern), SM::total);
   if (cfg != FASTAR_OK) return cfg;
-  kern<<<grid, kAttnThreads, SM::total, st>>>(tq, tk, tv, tsk, tsv, c, a);
+  launch_chained(kern, grid, kAttnThreads, SM::total, st, tq, tk, tv, tsk, tsv, c, a);
   return cudaGetLastError() == cudaSuccess ? 1 : FASTAR_ERR_CUDA;
 }
 

@@ -56,6 +56,7 @@ template <int D, bool MEANK>
 __global__ void __launch_bounds__(256) commit_kernel(const CacheView c, const __nv_bfloat16* __restrict__ k_new,
                                                      const __nv_bfloat16* __restrict__ v_new, int n, int frame_len, int64_t hs,
                                                      int64_t ts) {
+  chain_wait();
   constexpr int LPR = D / 8;            // lanes per row
   constexpr int GPW = 32 / LPR;         // work items per warp
   const int h = blockIdx.y;
@@ -277,10 +278,10 @@ int launch_commit(const CacheView& c, const __nv_bfloat16* k_new, const __nv_bfl
   if (n <= 0) return 0;
   const int items_per_cta = 8 * (32 / (c.D / 8));
   const dim3 grid((n + items_per_cta - 1) / items_per_cta, c.H);
-  if (c.D == 128 && !c.rep_mean) commit_kernel<128, false><<<grid, 256, 0, st>>>(c, k_new, v_new, n, frame_len, hs, ts);
-  else if (c.D == 128) commit_kernel<128, true><<<grid, 256, 0, st>>>(c, k_new, v_new, n, frame_len, hs, ts);
-  else if (!c.rep_mean) commit_kernel<64, false><<<grid, 256, 0, st>>>(c, k_new, v_new, n, frame_len, hs, ts);
-  else commit_kernel<64, true><<<grid, 256, 0, st>>>(c, k_new, v_new, n, frame_len, hs, ts);
+  if (c.D == 128 && !c.rep_mean) launch_chained(commit_kernel<128, false>, grid, 256, 0, st, c, k_new, v_new, n, frame_len, hs, ts);
+  else if (c.D == 128) launch_chained(commit_kernel<128, true>, grid, 256, 0, st, c, k_new, v_new, n, frame_len, hs, ts);
+  else if (!c.rep_mean) launch_chained(commit_kernel<64, false>, grid, 256, 0, st, c, k_new, v_new, n, frame_len, hs, ts);
+  else launch_chained(commit_kernel<64, true>, grid, 256, 0, st, c, k_new, v_new, n, frame_len, hs, ts);
   return cudaGetLastError() == cudaSuccess ? 1 : FASTAR_ERR_CUDA;
 }
 

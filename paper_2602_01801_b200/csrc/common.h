@@ -112,6 +112,24 @@ inline __host__ __device__ int64_t slot_row_offset(const CacheView& c, const int
   return (static_cast<int64_t>(page) * c.PT + (slot % c.PT)) * c.D;
 }
 
+// Launches a kernel that may start its prologue while the grid in front of it on the stream drains (programmatic stream
+// serialization).  The kernel has to call chain_wait() (ptx.cuh) before it touches global memory; behind a copy, a memset or
+// an event wait the launch is an ordinary one.  A step is 17 to 27 launches, and a gap between two ordinary ones is 2 us.
+template <class... P, class... A>
+inline cudaError_t launch_chained(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A&&... args) {
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cfg.attrs = &at;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+}
+
 // Raises a kernel's dynamic shared-memory limit once per (kernel, device); safe from several host threads.
 // The attribute is per device, so a process that drives several GPUs sets it on each (fastar_api.cu).
 int ensure_dynamic_smem(const void* kernel, int bytes);
@@ -171,14 +189,20 @@ int launch_attention_paged(const CacheView& c, const CUtensorMap& tm_q, const CU
 int launch_attention_gather(const CacheView& c, const CUtensorMap& tm_q, const AttnArgs& a, cudaStream_t st);
 
 // update_kernels.cu
+struct UpdateOut {         // the caller's [H][n] arrays (each may be null)
+  int32_t* match;
+  float* sim;
+  int32_t* dest;
+};
 int launch_convert_f32_to_bf16(const float* src, __nv_bfloat16* dst, int H, int n, int D, int64_t hs, int64_t ts, cudaStream_t st);
 int launch_prep_codes(const CacheView& c, const __nv_bfloat16* x, int n, int64_t hs, int64_t ts, uint32_t* code_out,
                       float* rnorm_out, cudaStream_t st);
+int launch_prep_update(const CacheView& c, const __nv_bfloat16* k_new, int n, int64_t hs, int64_t ts, cudaStream_t st);
 int launch_prep_codes_strided(const CacheView& c, const __nv_bfloat16* x, int n, int64_t hs, int64_t ts, uint32_t* code_out,
                               int64_t out_stride, cudaStream_t st);
 int launch_bucket_select(const CacheView& c, int nq, int frame_len, int n_frames, int np, cudaStream_t st);
 int launch_probe_cosine(const CacheView& c, const __nv_bfloat16* k_new, int n, int64_t hs, int64_t ts, cudaStream_t st);
-int launch_plan(const CacheView& c, int n, int frame_len, float tau, cudaStream_t st);
+int launch_plan(const CacheView& c, int n, float tau, const UpdateOut& out, cudaStream_t st);
 int launch_commit(const CacheView& c, const __nv_bfloat16* k_new, const __nv_bfloat16* v_new, int n, int frame_len,
                   int64_t hs, int64_t ts, cudaStream_t st);
 int launch_finalize_hist(const CacheView& c, fastar_update_stats* stats_out, int advance_clock, cudaStream_t st);
@@ -188,7 +212,6 @@ int launch_topk_prompt(const CacheView& c, int n_frames, int np, int keep, cudaS
 int launch_reset(const CacheView& c, cudaStream_t st);
 int launch_import_derive(const CacheView& c, cudaStream_t st);
 int launch_bounded_wait_selftest(const CacheView& c, int limit_us, int* released, cudaStream_t st);
-int launch_copy_outputs(const CacheView& c, int n, int32_t* match_out, float* sim_out, int32_t* dest_out, cudaStream_t st);
 int launch_decode_rel(const CacheView& c, int n_frames, int np, float scale, float* rel_out, cudaStream_t st);
 
 }  // namespace fastar

@@ -11,6 +11,7 @@
 #include <vector>
 
 #include "common.h"
+#include "ptx.cuh"
 
 using namespace fastar;
 
@@ -127,7 +128,7 @@ size_t carve(const fastar_cache_desc& d, uint8_t* base, CacheView* v) {
   t.status = reinterpret_cast<int32_t*>(take(4));
   t.lsh = reinterpret_cast<__nv_bfloat16*>(take(32 * D * 2));
   t.best = reinterpret_cast<unsigned long long*>(take(H * MT * 8));
-  t.n_match = reinterpret_cast<int32_t*>(take(H * 4));              // between `best` and `cnt`: one memset clears all three
+  t.n_match = reinterpret_cast<int32_t*>(take(H * 4));              // between `best` and `cnt`: launch_prep_update clears all three
   t.cnt = reinterpret_cast<int32_t*>(take(H * CAP * 4));
   t.cur = reinterpret_cast<int32_t*>(take(H * CAP * 4));
   t.segslot = reinterpret_cast<int32_t*>(take(H * MT * 4));
@@ -209,17 +210,20 @@ int make_map_codes(fastar_cache* c, CUtensorMap* m, const void* ptr, uint64_t d1
 // Block scores of weighted histograms as one number: lo + 256 * hi (exact in fp32 below 2^24).
 __global__ void combine_scores_kernel(const float* __restrict__ lo, const float* __restrict__ hi, int64_t head_stride,
                                       float* __restrict__ out, int per_head) {
+  chain_wait();
   const int h = blockIdx.y;
   for (int q = blockIdx.x * blockDim.x + threadIdx.x; q < per_head; q += gridDim.x * blockDim.x)
     out[static_cast<int64_t>(h) * per_head + q] = lo[h * head_stride + q] + 256.f * hi[h * head_stride + q];
 }
 
 __global__ void seg_bias_kernel(float* __restrict__ bias, int ns, int total) {
+  chain_wait();
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < total; i += gridDim.x * blockDim.x) bias[i] = i < ns ? 0.f : -INFINITY;
 }
 
 __global__ void copy_rows3_kernel(const int32_t* __restrict__ src, int64_t src_hs, int src_rs, int32_t* __restrict__ dst, int rows,
                                   int cols) {
+  chain_wait();
   const int h = blockIdx.y;
   for (int q = blockIdx.x * blockDim.x + threadIdx.x; q < rows * cols; q += gridDim.x * blockDim.x) {
     const int r = q / cols, cidx = q % cols;
@@ -535,10 +539,7 @@ static int update_impl(fastar_cache_t* c, const void* q_probe, const void* k_new
   r = q_probe ? make_map(c, &tm_a, pb, v.D, n, v.H, static_cast<uint64_t>(pts) * 2, static_cast<uint64_t>(phs) * 2, 128)
               : make_map(c, &tm_a, kb, v.D, n, v.H, static_cast<uint64_t>(kts) * 2, static_cast<uint64_t>(khs) * 2, 128);
   if (r != FASTAR_OK) return r;
-  ACCK(FASTAR_K_HASH, launch_prep_codes(v, kb, n, khs, kts, v.code_new, v.rnorm_new, st));
-  // packed arg-max words and per-slot match counts start at zero (adjacent in the workspace: one memset)
-  if (cudaMemsetAsync(v.best, 0, reinterpret_cast<uint8_t*>(v.cnt) - reinterpret_cast<uint8_t*>(v.best) + static_cast<size_t>(v.H) * v.CAP * 4, st) != cudaSuccess)
-    return FASTAR_ERR_CUDA;
+  ACCK(FASTAR_K_HASH, launch_prep_update(v, kb, n, khs, kts, st));
   // A row whose best similarity stays below the threshold is appended whatever its best slot is: the search kernels
   // skip the column search for running maxima below tau minus a margin that covers their rounding (the similarity
   // itself is always exact).  Rankings that a cosine pass follows need the slot in every case.
@@ -565,11 +566,10 @@ static int update_impl(fastar_cache_t* c, const void* q_probe, const void* k_new
   } else {
     ACCK(FASTAR_K_T1_SIMILARITY, launch_t1_search(vs, tm_a, c->tm_pool_k, n, st));
   }
-  ACCK(FASTAR_K_PLAN, launch_plan(v, n, frame_len, tau, st));
+  ACCK(FASTAR_K_PLAN, launch_plan(v, n, tau, UpdateOut{match_out, sim_out, dest_out}, st));
   if (v_ready && !v_converted && cudaStreamWaitEvent(st, v_ready, 0) != cudaSuccess) return FASTAR_ERR_CUDA;
   ACCK(FASTAR_K_COMMIT, launch_commit(v, kb, vb, n, frame_len, khs, kts, st));
   ACCK(FASTAR_K_KEY_HIST, launch_finalize_hist(v, stats_out, 1, st));
-  ACC(launch_copy_outputs(v, n, match_out, sim_out, dest_out, st));
   return FASTAR_OK;
 }
 
@@ -649,7 +649,7 @@ static int annsa_impl(fastar_cache_t* c, const void* q, const void* k_seg, const
     a.sel_head_stride = static_cast<int64_t>(v.max_qb) * v.CAPB;
     a.keep = keep;
     if (sel_out) {
-      copy_rows3_kernel<<<dim3((nqb * keep + 255) / 256, v.H), 256, 0, st>>>(v.sel, a.sel_head_stride, v.CAPB, sel_out, nqb, keep);
+      launch_chained(copy_rows3_kernel, dim3((nqb * keep + 255) / 256, v.H), 256, 0, st, v.sel, a.sel_head_stride, v.CAPB, sel_out, nqb, keep);
       if (cudaGetLastError() != cudaSuccess) return FASTAR_ERR_CUDA;
       c->launches += 1;
     }
@@ -659,7 +659,7 @@ static int annsa_impl(fastar_cache_t* c, const void* q, const void* k_seg, const
                                        static_cast<size_t>(nq) * 4, v.H, cudaMemcpyDeviceToDevice, st) != cudaSuccess)
       return FASTAR_ERR_CUDA;
     if (scores_out && v.hist_weighted) {
-      combine_scores_kernel<<<dim3((nqb * v.CAPB + 255) / 256, v.H), 256, 0, st>>>(v.scores, v.scores_hi, static_cast<int64_t>(v.max_qb) * v.CAPB,
+      launch_chained(combine_scores_kernel, dim3((nqb * v.CAPB + 255) / 256, v.H), 256, 0, st, v.scores, v.scores_hi, static_cast<int64_t>(v.max_qb) * v.CAPB,
                                                                                scores_out, nqb * v.CAPB);
       if (cudaGetLastError() != cudaSuccess) return FASTAR_ERR_CUDA;
       c->launches += 1;
@@ -680,7 +680,7 @@ static int annsa_impl(fastar_cache_t* c, const void* q, const void* k_seg, const
     if (r != FASTAR_OK) return r;
     a.seg_tiles = (ns + v.PT - 1) / v.PT;
     a.seg_bias = v.seg_bias;
-    seg_bias_kernel<<<(a.seg_tiles * v.PT + 255) / 256, 256, 0, st>>>(v.seg_bias, ns, a.seg_tiles * v.PT);
+    launch_chained(seg_bias_kernel, (a.seg_tiles * v.PT + 255) / 256, 256, 0, st, v.seg_bias, ns, a.seg_tiles * v.PT);
     if (cudaGetLastError() != cudaSuccess) return FASTAR_ERR_CUDA;
     c->launches += 1;
   }
@@ -799,7 +799,7 @@ int fastar_annca_attention(fastar_cache_t* c, const void* q, const void* k_promp
     a.sel_stride = v.max_prompt;
     a.sel_head_stride = static_cast<int64_t>(v.max_frames) * v.max_prompt;
     if (sel_out) {
-      copy_rows3_kernel<<<dim3((F * keep + 255) / 256, v.H), 256, 0, st>>>(v.selp, a.sel_head_stride, v.max_prompt, sel_out, F, keep);
+      launch_chained(copy_rows3_kernel, dim3((F * keep + 255) / 256, v.H), 256, 0, st, v.selp, a.sel_head_stride, v.max_prompt, sel_out, F, keep);
       if (cudaGetLastError() != cudaSuccess) return FASTAR_ERR_CUDA;
       c->launches += 1;
     }
@@ -859,7 +859,7 @@ int fastar_annca_attention_lsh(fastar_cache_t* c, const void* q, const void* k_p
   a.sel_stride = v.max_prompt;
   a.sel_head_stride = static_cast<int64_t>(v.max_frames) * v.max_prompt;
   if (sel_out) {
-    copy_rows3_kernel<<<dim3((F * np + 255) / 256, v.H), 256, 0, st>>>(v.selp, a.sel_head_stride, v.max_prompt, sel_out, F, np);
+    launch_chained(copy_rows3_kernel, dim3((F * np + 255) / 256, v.H), 256, 0, st, v.selp, a.sel_head_stride, v.max_prompt, sel_out, F, np);
     if (cudaGetLastError() != cudaSuccess) return FASTAR_ERR_CUDA;
     c->launches += 1;
   }

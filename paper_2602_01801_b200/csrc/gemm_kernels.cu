@@ -65,17 +65,6 @@ gemm_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__ CU
   const int warp = warp_index(), lane = threadIdx.x & 31;
   const int h = blockIdx.y;
   const int m0 = blockIdx.x * 128;
-  const int L = __shfl_sync(0xffffffffu, c.len[h], 0);
-
-  // ---- tile range of this CTA ----------------------------------------------------------------
-  int n_tiles;
-  if (EPI == EPI_COLMAX) n_tiles = (g.cols_b + 127) >> 7;
-  else n_tiles = (((L + c.PT - 1) / c.PT) + 127) >> 7;
-  const int per = (n_tiles + gridDim.z - 1) / gridDim.z;
-  const int t0 = blockIdx.z * per;
-  const int ntl = max(0, min(n_tiles, t0 + per) - t0);
-  const int nkc = g.nkc;
-
   if (threadIdx.x == 0) {
     for (int s = 0; s < NST; ++s) {
       mbar_init(bar_full + 8 * s, 1);
@@ -102,6 +91,16 @@ gemm_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__ CU
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = *tmem_slot;
+  chain_wait();
+
+  // ---- tile range of this CTA ----------------------------------------------------------------
+  int n_tiles;
+  if (EPI == EPI_COLMAX) n_tiles = (g.cols_b + 127) >> 7;
+  else n_tiles = (((__shfl_sync(0xffffffffu, c.len[h], 0) + c.PT - 1) / c.PT) + 127) >> 7;
+  const int per = (n_tiles + gridDim.z - 1) / gridDim.z;
+  const int t0 = blockIdx.z * per;
+  const int ntl = max(0, min(n_tiles, t0 + per) - t0);
+  const int nkc = g.nkc;
 
   if (ntl > 0) {
     if (warp == kGemmProducerWarp) {
@@ -246,7 +245,7 @@ static int launch_gemm(const CUtensorMap& tm_a, const CUtensorMap& tm_b, const C
   auto kern = gemm_kernel<EPI, A_RES, NST>;
   const int cfg = ensure_dynamic_smem(reinterpret_cast<const void*>(kern), SM::total);
   if (cfg != FASTAR_OK) return cfg;
-  kern<<<grid, kGemmThreads, SM::total, st>>>(tm_a, tm_b, c, g);
+  launch_chained(kern, grid, kGemmThreads, SM::total, st, tm_a, tm_b, c, g);
   return cudaGetLastError() == cudaSuccess ? 1 : FASTAR_ERR_CUDA;
 }
 

@@ -37,6 +37,11 @@ __device__ __forceinline__ int checked_index(int idx, int n, int* status) {
 #define FASTAR_IDX(idx, n, status) (idx)
 #endif
 
+// Programmatic dependent launch (launch_chained): the grid may be resident before the grid in front of it on the stream has
+// finished.  chain_wait returns when that grid is complete and its writes are visible; every kernel calls it before it touches
+// memory that another kernel reads or writes.
+__device__ __forceinline__ void chain_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
 __device__ __forceinline__ uint32_t smem_u32(const void* p) {
   return static_cast<uint32_t>(__cvta_generic_to_shared(p));
 }

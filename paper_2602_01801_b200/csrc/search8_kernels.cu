@@ -55,6 +55,7 @@ __device__ __forceinline__ void umma_ss_f8(uint32_t d_tmem, uint64_t adesc, uint
 __global__ void __launch_bounds__(256) quantize_rows_kernel(const __nv_bfloat16* __restrict__ x, int H, int n, int D, int64_t hs,
                                                             int64_t ts, uint8_t* __restrict__ out, int64_t out_rows_per_head,
                                                             float* __restrict__ norm_out, int64_t norm_stride) {
+  chain_wait();
   const int64_t rows = static_cast<int64_t>(H) * n;
   const unsigned hmask = 0xFFFFu << (threadIdx.x & 16);
   for (int64_t q = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x; (q >> 4) < rows;
@@ -97,7 +98,7 @@ int launch_quantize_rows(const CacheView& c, const __nv_bfloat16* x, int n, int6
   if (n <= 0) return 0;
   const int64_t total = static_cast<int64_t>(c.H) * n * 16;
   const int grid = static_cast<int>((total + 255) / 256 < 148 * 8 ? (total + 255) / 256 : 148 * 8);
-  quantize_rows_kernel<<<grid, 256, 0, st>>>(x, c.H, n, c.D, hs, ts, out, out_rows_per_head, norm_out, norm_stride);
+  launch_chained(quantize_rows_kernel, grid, 256, 0, st, x, c.H, n, c.D, hs, ts, out, out_rows_per_head, norm_out, norm_stride);
   return cudaGetLastError() == cudaSuccess ? 1 : FASTAR_ERR_CUDA;
 }
 
@@ -107,6 +108,7 @@ int launch_quantize_rows(const CacheView& c, const __nv_bfloat16* x, int n, int6
 // bytes; bit u of table t sits at bit 8*t + u of the packed code.
 __global__ void __launch_bounds__(256) sign_rows_kernel(const uint32_t* __restrict__ codes, int H, int n, int64_t code_stride, int T,
                                                         int B, uint8_t* __restrict__ out, int64_t out_rows_per_head) {
+  chain_wait();
   const int64_t total = static_cast<int64_t>(H) * n * 16;
   for (int64_t q = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x; q < total;
        q += static_cast<int64_t>(gridDim.x) * blockDim.x) {
@@ -132,7 +134,7 @@ int launch_sign_rows(const CacheView& c, const uint32_t* codes, int n, int64_t c
   if (n <= 0) return 0;
   const int64_t total = static_cast<int64_t>(c.H) * n * 16;
   const int grid = static_cast<int>((total + 255) / 256 < 148 * 8 ? (total + 255) / 256 : 148 * 8);
-  sign_rows_kernel<<<grid, 256, 0, st>>>(codes, c.H, n, code_stride, c.T, c.B, out, out_rows_per_head);
+  launch_chained(sign_rows_kernel, grid, 256, 0, st, codes, c.H, n, code_stride, c.T, c.B, out, out_rows_per_head);
   return cudaGetLastError() == cudaSuccess ? 1 : FASTAR_ERR_CUDA;
 }
 
@@ -140,6 +142,7 @@ int launch_sign_rows(const CacheView& c, const uint32_t* codes, int n, int64_t c
 __global__ void __launch_bounds__(256) quantize_kernel(const __nv_bfloat16* __restrict__ x, int H, int n, int D, int64_t hs,
                                                        int64_t ts, const float* __restrict__ rnorm, int64_t rn_stride,
                                                        uint8_t* __restrict__ out, int64_t out_rows_per_head) {
+  chain_wait();
   const int64_t total = static_cast<int64_t>(H) * n * 16;
   for (int64_t q = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x; q < total;
        q += static_cast<int64_t>(gridDim.x) * blockDim.x) {
@@ -169,7 +172,7 @@ int launch_quantize_keys(const CacheView& c, const __nv_bfloat16* x, int n, int6
   if (n <= 0) return 0;
   const int64_t total = static_cast<int64_t>(c.H) * n * 16;
   const int grid = static_cast<int>((total + 255) / 256 < 148 * 8 ? (total + 255) / 256 : 148 * 8);
-  quantize_kernel<<<grid, 256, 0, st>>>(x, c.H, n, c.D, hs, ts, rnorm, rn_stride, out, out_rows_per_head);
+  launch_chained(quantize_kernel, grid, 256, 0, st, x, c.H, n, c.D, hs, ts, rnorm, rn_stride, out, out_rows_per_head);
   return cudaGetLastError() == cudaSuccess ? 1 : FASTAR_ERR_CUDA;
 }
 
@@ -213,11 +216,6 @@ search8_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
   const int warp = warp_index(), lane = threadIdx.x & 31;
   const int h = blockIdx.y;
   const int m0 = blockIdx.x * 128;
-  const int L = COLMAX ? g.cols_b : __shfl_sync(0xffffffffu, c.len[h], 0);
-  const int n_tiles = (L + 127) >> 7;
-  const int per = (n_tiles + gridDim.z - 1) / gridDim.z;
-  const int t0 = blockIdx.z * per;
-  const int ntl = max(0, min(n_tiles, t0 + per) - t0);
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < kStages; ++s) {
@@ -245,6 +243,12 @@ search8_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = *tmem_slot;
+  chain_wait();
+  const int L = COLMAX ? g.cols_b : __shfl_sync(0xffffffffu, c.len[h], 0);
+  const int n_tiles = (L + 127) >> 7;
+  const int per = (n_tiles + gridDim.z - 1) / gridDim.z;
+  const int t0 = blockIdx.z * per;
+  const int ntl = max(0, min(n_tiles, t0 + per) - t0);
 
   if (ntl > 0) {
     if (warp == kProducer) {
@@ -450,8 +454,8 @@ int launch_t1_similarity_fp8(const CacheView& c, const CUtensorMap& tm_a8, const
   Search8Args g{};
   g.rows_a = n;
   const dim3 grid(row_tiles, c.H, pick_splits8(row_tiles, c.H, c.CAP / 128));
-  if (col_norm) search8_kernel<false, true><<<grid, kThreads, Smem::total, st>>>(tm_a8, tm_pool_k8, c, g);
-  else search8_kernel<false, false><<<grid, kThreads, Smem::total, st>>>(tm_a8, tm_pool_k8, c, g);
+  if (col_norm) launch_chained(search8_kernel<false, true>, grid, kThreads, Smem::total, st, tm_a8, tm_pool_k8, c, g);
+  else launch_chained(search8_kernel<false, false>, grid, kThreads, Smem::total, st, tm_a8, tm_pool_k8, c, g);
   return cudaGetLastError() == cudaSuccess ? 1 : FASTAR_ERR_CUDA;
 }
 
@@ -467,8 +471,7 @@ int launch_c1_relevance_fp8(const CacheView& c, const CUtensorMap& tm_q8, const 
   g.frame_len = frame_len;
   g.qn = qn;
   g.kn = kn;
-  search8_kernel<true><<<dim3(row_tiles, c.H, pick_splits8(row_tiles, c.H, (np + 127) / 128)), kThreads, Smem::total, st>>>(
-      tm_q8, tm_kp8, c, g);
+  launch_chained(search8_kernel<true>, dim3(row_tiles, c.H, pick_splits8(row_tiles, c.H, (np + 127) / 128)), kThreads, Smem::total, st, tm_q8, tm_kp8, c, g);
   return cudaGetLastError() == cudaSuccess ? 1 : FASTAR_ERR_CUDA;
 }
 

@@ -193,6 +193,7 @@ search_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__ 
       tma_prefetch_desc(&tm_b);
       pre[0] = 0;
     }
+    chain_wait();
     int run = 0;
     for (int b = 0; b < heads; b += 32) {
       const int len = b + lane < heads ? c.len[h0 + b + lane] : 0;
@@ -211,6 +212,7 @@ search_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__ 
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = *tmem_slot;
+  chain_wait();
   Seg* seg_s = reinterpret_cast<Seg*>(smem_raw + SM::seg_off);
 
   if (warp >= kEpiWarps) {
@@ -502,7 +504,7 @@ static int launch_search_t(const CacheView& c, const CUtensorMap& tm_a, const CU
     const int heads = min(kMaxHeads, c.H - h0);
     // one CTA per SM; fewer only when the whole search has fewer (row unit, key tile) pairs than that
     const int64_t pairs = static_cast<int64_t>(heads) * ((n + 255) / 256) * (c.CAP / 128);
-    kern<<<static_cast<int>(pairs < sm_count ? pairs : sm_count), kThreads, SM::total, st>>>(tm_a, tm_b, c, n, h0, heads);
+    launch_chained(kern, static_cast<int>(pairs < sm_count ? pairs : sm_count), kThreads, SM::total, st, tm_a, tm_b, c, n, h0, heads);
     if (cudaGetLastError() != cudaSuccess) return FASTAR_ERR_CUDA;
     ++launched;
   }

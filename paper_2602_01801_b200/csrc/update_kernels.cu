@@ -74,6 +74,7 @@ __device__ __forceinline__ void bitonic_sort_smem(unsigned long long* keys, int 
 // ---------------------------------------------------------------------------------------------
 __global__ void convert_kernel(const float* __restrict__ src, __nv_bfloat16* __restrict__ dst, int n, int D, int64_t hs,
                                int64_t ts) {
+  chain_wait();
   const int h = blockIdx.y;
   const int64_t per_head = static_cast<int64_t>(n) * D / 4;
   for (int64_t q = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; q < per_head;
@@ -93,7 +94,7 @@ int launch_convert_f32_to_bf16(const float* src, __nv_bfloat16* dst, int H, int 
   const int64_t per_head = static_cast<int64_t>(n) * D / 4;
   const int64_t want = (per_head + 255) / 256;
   const int bx = static_cast<int>(want < 1024 ? want : 1024);
-  convert_kernel<<<dim3(bx, H), 256, 0, st>>>(src, dst, n, D, hs, ts);
+  launch_chained(convert_kernel, dim3(bx, H), 256, 0, st, src, dst, n, D, hs, ts);
   return cudaGetLastError() == cudaSuccess ? 1 : FASTAR_ERR_CUDA;
 }
 
@@ -109,7 +110,10 @@ template <int D>
 __global__ void __launch_bounds__(256) prep_kernel(const __nv_bfloat16* __restrict__ x, int H, int n, int64_t hs, int64_t ts,
                                                    const __nv_bfloat16* __restrict__ lsh, int T, int B,
                                                    uint32_t* __restrict__ code_out, float* __restrict__ rnorm_out,
-                                                   int64_t out_stride) {
+                                                   int64_t out_stride, uint4* __restrict__ zero, int64_t zero16) {
+  chain_wait();
+  for (int64_t q = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; q < zero16; q += static_cast<int64_t>(gridDim.x) * blockDim.x)
+    zero[q] = make_uint4(0, 0, 0, 0);
   constexpr int KS = D / 16;
   constexpr int RP = D + 8;                    // padded row of the staged projection matrix (bank-conflict free)
   __shared__ __align__(16) __nv_bfloat16 r_s[32 * RP];
@@ -209,17 +213,23 @@ __global__ void __launch_bounds__(256) prep_kernel(const __nv_bfloat16* __restri
   }
 }
 static int launch_prep_generic(const CacheView& c, const __nv_bfloat16* x, int n, int64_t hs, int64_t ts, uint32_t* code_out,
-                               float* rnorm_out, int64_t out_stride, cudaStream_t st) {
+                               float* rnorm_out, int64_t out_stride, cudaStream_t st, uint4* zero = nullptr, int64_t zero16 = 0) {
   if (n <= 0) return 0;
   const int groups = ((n + 15) / 16) * c.H;                      // 16 rows per warp pass
   const dim3 grid(max(1, min((groups + 7) / 8, 2 * 148)));
-  if (c.D == 128) prep_kernel<128><<<grid, 256, 0, st>>>(x, c.H, n, hs, ts, c.lsh, c.T, c.B, code_out, rnorm_out, out_stride);
-  else prep_kernel<64><<<grid, 256, 0, st>>>(x, c.H, n, hs, ts, c.lsh, c.T, c.B, code_out, rnorm_out, out_stride);
+  if (c.D == 128) launch_chained(prep_kernel<128>, grid, 256, 0, st, x, c.H, n, hs, ts, c.lsh, c.T, c.B, code_out, rnorm_out, out_stride, zero, zero16);
+  else launch_chained(prep_kernel<64>, grid, 256, 0, st, x, c.H, n, hs, ts, c.lsh, c.T, c.B, code_out, rnorm_out, out_stride, zero, zero16);
   return cudaGetLastError() == cudaSuccess ? 1 : FASTAR_ERR_CUDA;
 }
 int launch_prep_codes(const CacheView& c, const __nv_bfloat16* x, int n, int64_t hs, int64_t ts, uint32_t* code_out,
                       float* rnorm_out, cudaStream_t st) {
   return launch_prep_generic(c, x, n, hs, ts, code_out, rnorm_out, c.max_tokens, st);
+}
+// The first kernel of an update: codes and reciprocal norms of the new keys, and zeros in the words that the search and the
+// matching accumulate into (best, n_match and cnt lie side by side; a memset of its own cost 4 us with its two gaps).
+int launch_prep_update(const CacheView& c, const __nv_bfloat16* k_new, int n, int64_t hs, int64_t ts, cudaStream_t st) {
+  const int64_t bytes = reinterpret_cast<const uint8_t*>(c.cnt + static_cast<int64_t>(c.H) * c.CAP) - reinterpret_cast<const uint8_t*>(c.best);
+  return launch_prep_generic(c, k_new, n, hs, ts, c.code_new, c.rnorm_new, c.max_tokens, st, reinterpret_cast<uint4*>(c.best), bytes / 16);
 }
 int launch_prep_codes_strided(const CacheView& c, const __nv_bfloat16* x, int n, int64_t hs, int64_t ts, uint32_t* code_out,
                               int64_t out_stride, cudaStream_t st) {
@@ -236,7 +246,8 @@ int launch_prep_codes_strided(const CacheView& c, const __nv_bfloat16* x, int n,
 // Members of a group land in arbitrary order; the commit walks them in ascending token order, so the
 // result does not depend on it.
 // ---------------------------------------------------------------------------------------------
-__global__ void __launch_bounds__(256) match_count_kernel(const CacheView c, int n, float tau) {
+__global__ void __launch_bounds__(256) match_count_kernel(const CacheView c, int n, float tau, const UpdateOut out) {
+  chain_wait();
   const int h = blockIdx.y;
   const int64_t tb = static_cast<int64_t>(h) * c.max_tokens;
   int mine = 0;
@@ -251,6 +262,8 @@ __global__ void __launch_bounds__(256) match_count_kernel(const CacheView c, int
     const bool matched = j >= 0 && s >= tau;
     c.match[tb + i] = matched ? j : -1;
     c.sim[tb + i] = s;
+    if (out.match) out.match[static_cast<int64_t>(h) * n + i] = matched ? j : -1;
+    if (out.sim) out.sim[static_cast<int64_t>(h) * n + i] = s;
     if (matched) atomicAdd(c.cnt + static_cast<int64_t>(h) * c.CAP + j, 1);
     mine += matched ? 1 : 0;
   }
@@ -261,7 +274,8 @@ __global__ void __launch_bounds__(256) match_count_kernel(const CacheView c, int
   }
 }
 
-__global__ void __launch_bounds__(1024) plan_kernel(const CacheView c, int n) {
+__global__ void __launch_bounds__(1024) plan_kernel(const CacheView c, int n, int32_t* __restrict__ dest_out) {
+  chain_wait();
   extern __shared__ unsigned long long keys[];   // victim sort buffer, only touched when evicting
   __shared__ int red[32];
   const int h = blockIdx.x, tid = threadIdx.x;
@@ -465,10 +479,16 @@ __global__ void __launch_bounds__(1024) plan_kernel(const CacheView c, int n) {
   __syncthreads();
   // destinations (matched tokens get theirs in the scatter kernel)
   if (ok) {
-    for (int k = tid; k < U; k += blockDim.x)
-      c.dest[tb + FASTAR_IDX(c.ulist[tb + k], n, c.status)] = FASTAR_IDX(k < A ? L + k : c.victims[tb + k - A], c.CAP, c.status);
+    for (int k = tid; k < U; k += blockDim.x) {
+      const int i = FASTAR_IDX(c.ulist[tb + k], n, c.status), d = FASTAR_IDX(k < A ? L + k : c.victims[tb + k - A], c.CAP, c.status);
+      c.dest[tb + i] = d;
+      if (dest_out) dest_out[static_cast<int64_t>(h) * n + i] = d;
+    }
   } else {
-    for (int i = tid; i < n; i += blockDim.x) c.dest[tb + i] = -1;
+    for (int i = tid; i < n; i += blockDim.x) {
+      c.dest[tb + i] = -1;
+      if (dest_out) dest_out[static_cast<int64_t>(h) * n + i] = -1;
+    }
     if (tid == 0) record_status(c.status, kErrCapacity);
   }
   if (tid == 0) {
@@ -488,7 +508,8 @@ __global__ void __launch_bounds__(1024) plan_kernel(const CacheView c, int n) {
   }
 }
 
-__global__ void __launch_bounds__(256) scatter_kernel(const CacheView c, int n) {
+__global__ void __launch_bounds__(256) scatter_kernel(const CacheView c, int n, int32_t* __restrict__ dest_out) {
+  chain_wait();
   const int h = blockIdx.y;
   if (!c.plan[h].ok) return;
   const int64_t tb = static_cast<int64_t>(h) * c.max_tokens;
@@ -498,6 +519,7 @@ __global__ void __launch_bounds__(256) scatter_kernel(const CacheView c, int n) 
       const int pos = FASTAR_IDX(atomicAdd(c.cur + static_cast<int64_t>(h) * c.CAP + FASTAR_IDX(j, c.CAP, c.status), 1), n, c.status);
       c.order[tb + pos] = i;
       c.dest[tb + i] = j;
+      if (dest_out) dest_out[static_cast<int64_t>(h) * n + i] = j;
     }
   }
 }
@@ -510,6 +532,7 @@ __global__ void __launch_bounds__(256) scatter_kernel(const CacheView c, int n) 
 // ---------------------------------------------------------------------------------------------
 __global__ void __launch_bounds__(256) probe_cosine_kernel(const CacheView c, const __nv_bfloat16* __restrict__ k_new, int n,
                                                            int64_t hs, int64_t ts) {
+  chain_wait();
   const int64_t rows = static_cast<int64_t>(c.H) * n;
   const unsigned hmask = 0xFFFFu << (threadIdx.x & 16);
   for (int64_t q = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x; (q >> 4) < rows;
@@ -546,18 +569,17 @@ __global__ void __launch_bounds__(256) probe_cosine_kernel(const CacheView c, co
 int launch_probe_cosine(const CacheView& c, const __nv_bfloat16* k_new, int n, int64_t hs, int64_t ts, cudaStream_t st) {
   const int64_t total = static_cast<int64_t>(c.H) * n * 16;
   const int grid = static_cast<int>((total + 255) / 256 < 148 * 8 ? (total + 255) / 256 : 148 * 8);
-  probe_cosine_kernel<<<grid, 256, 0, st>>>(c, k_new, n, hs, ts);
+  launch_chained(probe_cosine_kernel, grid, 256, 0, st, c, k_new, n, hs, ts);
   return cudaGetLastError() == cudaSuccess ? 1 : FASTAR_ERR_CUDA;
 }
 
-int launch_plan(const CacheView& c, int n, int frame_len, float tau, cudaStream_t st) {
-  (void)frame_len;
+int launch_plan(const CacheView& c, int n, float tau, const UpdateOut& out, cudaStream_t st) {
   const int cfg = ensure_dynamic_smem(reinterpret_cast<const void*>(plan_kernel), 16384 * 8);
   if (cfg != FASTAR_OK) return cfg;
   const dim3 grid((n + 255) / 256, c.H);
-  match_count_kernel<<<grid, 256, 0, st>>>(c, n, tau);
-  plan_kernel<<<c.H, 1024, 16384 * 8, st>>>(c, n);
-  scatter_kernel<<<grid, 256, 0, st>>>(c, n);
+  launch_chained(match_count_kernel, grid, 256, 0, st, c, n, tau, out);
+  launch_chained(plan_kernel, c.H, 1024, 16384 * 8, st, c, n, out.dest);
+  launch_chained(scatter_kernel, grid, 256, 0, st, c, n, out.dest);
   return cudaGetLastError() == cudaSuccess ? 3 : FASTAR_ERR_CUDA;
 }
 
@@ -566,6 +588,7 @@ int launch_plan(const CacheView& c, int n, int frame_len, float tau, cudaStream_
 // ---------------------------------------------------------------------------------------------
 __global__ void __launch_bounds__(256) key_hist_kernel(const CacheView c, int use_plan, fastar_update_stats* stats_out,
                                                        int advance_clock) {
+  chain_wait();
   extern __shared__ int hist[];          // hist_cols counters
   const int b = blockIdx.x, h = blockIdx.y;
   const int L = use_plan ? c.plan[h].len_new : c.len[h];
@@ -611,13 +634,14 @@ __global__ void __launch_bounds__(256) key_hist_kernel(const CacheView c, int us
   }
 }
 int launch_finalize_hist(const CacheView& c, fastar_update_stats* stats_out, int advance_clock, cudaStream_t st) {
-  key_hist_kernel<<<dim3(c.CAPB, c.H), 256, c.hist_cols * 4, st>>>(c, advance_clock >= 0 ? 1 : 0, stats_out,
+  launch_chained(key_hist_kernel, dim3(c.CAPB, c.H), 256, c.hist_cols * 4, st, c, advance_clock >= 0 ? 1 : 0, stats_out,
                                                                   advance_clock > 0 ? 1 : 0);
   return cudaGetLastError() == cudaSuccess ? 1 : FASTAR_ERR_CUDA;
 }
 
 // S2 (query side)
 __global__ void __launch_bounds__(128) query_hist_kernel(const CacheView c, const uint32_t* __restrict__ codes, int nq, int block_q) {
+  chain_wait();
   extern __shared__ int hist[];
   const int a = blockIdx.x, h = blockIdx.y;
   for (int q = threadIdx.x; q < c.hist_cols; q += blockDim.x) hist[q] = 0;
@@ -634,7 +658,7 @@ __global__ void __launch_bounds__(128) query_hist_kernel(const CacheView c, cons
 }
 int launch_query_hist(const CacheView& c, const uint32_t* codes, int nq, int block_q, cudaStream_t st) {
   const int nqb = (nq + block_q - 1) / block_q;
-  query_hist_kernel<<<dim3(nqb, c.H), 128, c.hist_cols * 4, st>>>(c, codes, nq, block_q);
+  launch_chained(query_hist_kernel, dim3(nqb, c.H), 128, c.hist_cols * 4, st, c, codes, nq, block_q);
   return cudaGetLastError() == cudaSuccess ? 1 : FASTAR_ERR_CUDA;
 }
 
@@ -647,6 +671,7 @@ __global__ void __launch_bounds__(256) topk_kernel(const void* __restrict__ src,
                                                    int32_t* __restrict__ out, int64_t out_head_stride, int out_row_stride,
                                                    int out_fill, int32_t* __restrict__ nsel, int force_first, int force_last,
                                                    const float* __restrict__ src_hi, int* status, int sort_np2) {
+  chain_wait();
   extern __shared__ __align__(16) uint32_t vals[];     // ranking keys: larger key = better entry
   __shared__ int red[32];
   const int row = blockIdx.x, h = blockIdx.y;
@@ -719,7 +744,7 @@ static size_t topk_smem(int n, int np2) { return static_cast<size_t>((n + 3) & ~
 
 int launch_topk_blocks(const CacheView& c, int nqb, int keep, int force_sink, int force_recent, cudaStream_t st) {
   const int np2 = topk_sort_np2(c.CAPB);
-  topk_kernel<false><<<dim3(nqb, c.H), 256, topk_smem(c.CAPB, np2), st>>>(c.scores, static_cast<int64_t>(c.max_qb) * c.CAPB, c.CAPB, c.len,
+  launch_chained(topk_kernel<false>, dim3(nqb, c.H), 256, topk_smem(c.CAPB, np2), st, c.scores, static_cast<int64_t>(c.max_qb) * c.CAPB, c.CAPB, c.len,
                                                             c.PT, 0, keep, c.sel, static_cast<int64_t>(c.max_qb) * c.CAPB, c.CAPB,
                                                             min(keep, c.CAPB), c.nsel, force_sink, force_recent,
                                                             c.hist_weighted ? c.scores_hi : nullptr, c.status, np2);
@@ -732,6 +757,7 @@ int launch_topk_blocks(const CacheView& c, int nqb, int keep, int force_sink, in
 // written in ascending order (block scan) with their count.
 // ---------------------------------------------------------------------------------------------
 __global__ void __launch_bounds__(256) bucket_select_kernel(const CacheView c, int nq, int frame_len, int np) {
+  chain_wait();
   __shared__ uint32_t marks[4 * 8];
   __shared__ int red[32];
   const int f = blockIdx.x, h = blockIdx.y, tid = threadIdx.x;
@@ -769,13 +795,13 @@ __global__ void __launch_bounds__(256) bucket_select_kernel(const CacheView c, i
 }
 
 int launch_bucket_select(const CacheView& c, int nq, int frame_len, int n_frames, int np, cudaStream_t st) {
-  bucket_select_kernel<<<dim3(n_frames, c.H), 256, 0, st>>>(c, nq, frame_len, np);
+  launch_chained(bucket_select_kernel, dim3(n_frames, c.H), 256, 0, st, c, nq, frame_len, np);
   return cudaGetLastError() == cudaSuccess ? 1 : FASTAR_ERR_CUDA;
 }
 
 int launch_topk_prompt(const CacheView& c, int n_frames, int np, int keep, cudaStream_t st) {
   const int np2 = topk_sort_np2(np);
-  topk_kernel<true><<<dim3(n_frames, c.H), 256, topk_smem(np, np2), st>>>(c.rel, static_cast<int64_t>(c.max_frames) * c.max_prompt,
+  launch_chained(topk_kernel<true>, dim3(n_frames, c.H), 256, topk_smem(np, np2), st, c.rel, static_cast<int64_t>(c.max_frames) * c.max_prompt,
                                                                          c.max_prompt, nullptr, 1, np, keep, c.selp,
                                                                          static_cast<int64_t>(c.max_frames) * c.max_prompt, c.max_prompt,
                                                                          min(keep, np), nullptr, 0, 0, nullptr, c.status, np2);
@@ -882,15 +908,8 @@ int launch_bounded_wait_selftest(const CacheView& c, int limit_us, int* released
   return cudaGetLastError() == cudaSuccess ? 1 : FASTAR_ERR_CUDA;
 }
 
-int launch_copy_outputs(const CacheView& c, int n, int32_t* match_out, float* sim_out, int32_t* dest_out, cudaStream_t st) {
-  const size_t w = static_cast<size_t>(n) * 4, sp = static_cast<size_t>(c.max_tokens) * 4;
-  if (match_out && cudaMemcpy2DAsync(match_out, w, c.match, sp, w, c.H, cudaMemcpyDeviceToDevice, st) != cudaSuccess) return FASTAR_ERR_CUDA;
-  if (sim_out && cudaMemcpy2DAsync(sim_out, w, c.sim, sp, w, c.H, cudaMemcpyDeviceToDevice, st) != cudaSuccess) return FASTAR_ERR_CUDA;
-  if (dest_out && cudaMemcpy2DAsync(dest_out, w, c.dest, sp, w, c.H, cudaMemcpyDeviceToDevice, st) != cudaSuccess) return FASTAR_ERR_CUDA;
-  return 0;
-}
-
 __global__ void decode_rel_kernel(const CacheView c, int n_frames, int np, float scale, float* __restrict__ rel_out) {
+  chain_wait();
   const int h = blockIdx.y;
   for (int q = blockIdx.x * blockDim.x + threadIdx.x; q < n_frames * np; q += gridDim.x * blockDim.x) {
     const int f = q / np, p = q % np;
@@ -899,7 +918,7 @@ __global__ void decode_rel_kernel(const CacheView c, int n_frames, int np, float
   }
 }
 int launch_decode_rel(const CacheView& c, int n_frames, int np, float scale, float* rel_out, cudaStream_t st) {
-  decode_rel_kernel<<<dim3((n_frames * np + 255) / 256, c.H), 256, 0, st>>>(c, n_frames, np, scale, rel_out);
+  launch_chained(decode_rel_kernel, dim3((n_frames * np + 255) / 256, c.H), 256, 0, st, c, n_frames, np, scale, rel_out);
   return cudaGetLastError() == cudaSuccess ? 1 : FASTAR_ERR_CUDA;
 }
 

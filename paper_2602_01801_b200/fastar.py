@@ -259,7 +259,7 @@ class Cache:
             res = dict(match=torch.empty((H, n), dtype=torch.int32, device=self.device),
                        sim=torch.empty((H, n), dtype=torch.float32, device=self.device),
                        dest=torch.empty((H, n), dtype=torch.int32, device=self.device),
-                       stats=torch.zeros((H, 8), dtype=torch.int32, device=self.device))
+                       stats=torch.empty((H, 8), dtype=torch.int32, device=self.device))
         if probe is not None:
             _check(self.lib.fastar_tempcache_update_probe(self.handle, probe.data_ptr(), k_new.data_ptr(), v_new.data_ptr(), n,
                                                           frame_len, hs, ts, float(tau), _ptr(res.get("match")),
