@@ -138,8 +138,6 @@ int ensure_dynamic_smem(const void* kernel, int bytes);
 // Each returns the number of kernels it launched (for the launch counter) or a negative status.
 
 // gemm_kernels.cu
-int launch_c1_relevance(const CacheView& c, const CUtensorMap& tm_q, const CUtensorMap& tm_kp, int nq, int np, int frame_len,
-                        int n_frames, cudaStream_t st);
 int launch_s3_scores(const CacheView& c, const CUtensorMap& tm_hq, const CUtensorMap& tm_hk, int nqb, cudaStream_t st);
 
 // search_kernel.cu: T1 on the bf16 keys as one persistent kernel (c.raw_dot: plain dot products).  tm_pool_k: one page per box
@@ -154,6 +152,10 @@ int launch_sign_rows(const CacheView& c, const uint32_t* codes, int n, int64_t c
                      cudaStream_t st);
 int launch_quantize_rows(const CacheView& c, const __nv_bfloat16* x, int n, int64_t hs, int64_t ts, uint8_t* out,
                          int64_t out_rows_per_head, float* norm_out, int64_t norm_stride, cudaStream_t st);
+
+// relevance_kernel.cu: C1 on the bf16 rows and on the 8-bit codes
+int launch_c1_relevance(const CacheView& c, const CUtensorMap& tm_q, const CUtensorMap& tm_kp, int nq, int np, int frame_len,
+                        cudaStream_t st);
 int launch_c1_relevance_fp8(const CacheView& c, const CUtensorMap& tm_q8, const CUtensorMap& tm_kp8, const float* qn,
                             const float* kn, int nq, int np, int frame_len, cudaStream_t st);
 

@@ -33,6 +33,7 @@ struct fastar_cache {
   int force_sink_blocks = 0, force_recent_blocks = 0;    // AnnSA selector option (fastar_cache_set_forced_blocks)
   // queries whose codes and block histograms fastar_annsa_prepare has already produced (consumed by the next matching AnnSA call)
   struct { const void* q = nullptr; int32_t nq = 0, block_q = 0; int64_t hs = 0, ts = 0; bool valid = false; } prep;
+  bool rel_clear = true;     // the relevance maxima are zero (a reset and every prompt top-k leave them so)
   cudaEvent_t ev_prep = nullptr;
   cudaStream_t side = nullptr, copy = nullptr;
   cudaEvent_t ev_fork = nullptr, ev_q = nullptr, ev_join = nullptr, ev_p = nullptr, ev_v = nullptr;
@@ -357,6 +358,7 @@ int fastar_cache_reset(fastar_cache_t* c, void* stream) {
   if (!c) return FASTAR_ERR_INVALID_ARG;
   DeviceGuard guard(c->desc.device);
   ACC(launch_reset(c->v, static_cast<cudaStream_t>(stream)));
+  c->rel_clear = true;
   return FASTAR_OK;
 }
 
@@ -777,7 +779,11 @@ int fastar_annca_attention(fastar_cache_t* c, const void* q, const void* k_promp
     a.sel_stride = keep_tokens;
     a.sel_head_stride = static_cast<int64_t>(F) * keep_tokens;
   } else {
-    if (cudaMemsetAsync(v.rel, 0, static_cast<size_t>(v.H) * v.max_frames * v.max_prompt * 4, st) != cudaSuccess) return FASTAR_ERR_CUDA;
+    // The maxima start at zero (0 is below the word of every float).  The top-k that ranks them puts the zeros back, so a memset is
+    // queued only after a call that failed between the two.
+    if (!c->rel_clear && cudaMemsetAsync(v.rel, 0, static_cast<size_t>(v.H) * v.max_frames * v.max_prompt * 4, st) != cudaSuccess)
+      return FASTAR_ERR_CUDA;
+    c->rel_clear = false;
     float rel_scale = 1.0f / sqrtf(static_cast<float>(v.D));
     if (v.search_bits == 8 && !v.sign_codes) {
       // relevance on the 8-bit codes of the directions, scaled back by the norms (Section 5.1 quantised search)
@@ -792,9 +798,11 @@ int fastar_annca_attention(fastar_cache_t* c, const void* q, const void* k_promp
     } else {
       r = make_map(c, &tm_kp, kpb, v.D, np, v.H, static_cast<uint64_t>(kts) * 2, static_cast<uint64_t>(khs) * 2, 128);
       if (r != FASTAR_OK) return r;
-      ACCK(FASTAR_K_C1_RELEVANCE, launch_c1_relevance(v, tm_q, tm_kp, nq, np, frame_len, F, st));
+      ACCK(FASTAR_K_C1_RELEVANCE, launch_c1_relevance(v, tm_q, tm_kp, nq, np, frame_len, st));
     }
+    if (rel_out) ACC(launch_decode_rel(v, F, np, rel_scale, rel_out, st));
     ACCK(FASTAR_K_TOPK_PROMPT, launch_topk_prompt(v, F, np, keep, st));
+    c->rel_clear = true;
     a.sel = v.selp;
     a.sel_stride = v.max_prompt;
     a.sel_head_stride = static_cast<int64_t>(v.max_frames) * v.max_prompt;
@@ -803,7 +811,6 @@ int fastar_annca_attention(fastar_cache_t* c, const void* q, const void* k_promp
       if (cudaGetLastError() != cudaSuccess) return FASTAR_ERR_CUDA;
       c->launches += 1;
     }
-    if (rel_out) ACC(launch_decode_rel(v, F, np, rel_scale, rel_out, st));
   }
   ACCK(FASTAR_K_C3_ATTENTION, launch_attention_gather(v, tm_q, a, st));
   return FASTAR_OK;

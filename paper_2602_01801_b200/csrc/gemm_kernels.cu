@@ -1,11 +1,8 @@
-// tcgen05 / TMEM / TMA contraction kernel with two fused epilogues:
-//   C1  prompt relevance, column max per frame   (AnnCA, Section 5.3)
-//   S3  bucket-collision scores HQ x HK^T        (AnnSA block selection, Sections 5.1 / 5.4)
-// The score matrix of C1 is never written to memory.
+// S3: bucket-collision scores HQ x HK^T (AnnSA block selection, Sections 5.1 / 5.4) on tcgen05 / TMEM / TMA.
 //
-// One CTA = one 128-row tile of A and a range of 128-row tiles of B; D[128 x 128] fp32 lives in
+// One CTA = one 128-row tile of HQ and a range of 128-row tiles of HK; D[128 x 128] fp32 lives in
 // TMEM, double buffered so the epilogue of tile t overlaps the MMAs of tile t+1.
-// Warp roles: warps 0-7 epilogue (two threads per A row / TMEM lane, one per 64-column half), warp 8 TMA
+// Warp roles: warps 0-7 epilogue (two threads per row / TMEM lane, one per 64-column half), warp 8 TMA
 // producer, warp 9 TMEM allocation + MMA issue.  Operands are bf16, K-major, 128-byte swizzled.
 #include "common.h"
 #include "ptx.cuh"
@@ -13,14 +10,9 @@
 
 namespace fastar {
 
-enum { EPI_COLMAX = 1, EPI_STORE = 2 };
-
 struct GemmArgs {
-  int rows_a;              // valid rows of A per head (nq or nqb)
+  int rows_a;              // valid rows of HQ per head (nqb)
   int nkc;                 // K chunks of 64
-  int frame_len;           // COLMAX
-  int n_frames;            // COLMAX
-  int cols_b;              // COLMAX: np; STORE: unused (uses live blocks)
 };
 
 constexpr int kChunkBytes = 128 * 128;       // 128 rows x 64 bf16
@@ -28,20 +20,17 @@ constexpr int kTmemCols = 256;
 constexpr int kGemmThreads = 320;            // warps 0-7 epilogue, 8 TMA producer, 9 MMA issue
 constexpr int kGemmProducerWarp = 8, kGemmMmaWarp = 9;
 
-template <int EPI, bool A_RES, int NST>
+constexpr int NST = 4;                       // ring stages of a chunk of both operands
 struct GemmSmem {
-  static constexpr int a_bytes = A_RES ? 2 * kChunkBytes : 0;
-  static constexpr int stage_bytes = A_RES ? kChunkBytes : 2 * kChunkBytes;
-  static constexpr int ring_off = a_bytes;
-  static constexpr int bar_off = ring_off + NST * stage_bytes;
+  static constexpr int stage_bytes = 2 * kChunkBytes;
+  static constexpr int bar_off = NST * stage_bytes;
   static constexpr int total = bar_off + 256;
 };
 
-template <int EPI, bool A_RES, int NST>
-__global__ void __launch_bounds__(kGemmThreads, A_RES ? 2 : 1)
+__global__ void __launch_bounds__(kGemmThreads, 1)
 gemm_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__ CUtensorMap tm_b, const CacheView c,
             const GemmArgs g) {
-  using SM = GemmSmem<EPI, A_RES, NST>;
+  using SM = GemmSmem;
   extern __shared__ __align__(1024) uint8_t smem_raw[];
   const uint32_t sbase = smem_u32(smem_raw);
   uint8_t* sgen = smem_raw;
@@ -49,18 +38,16 @@ gemm_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__ CU
     if (threadIdx.x == 0) record_status(c.status, FASTAR_ERR_CUDA);
     return;
   }
-  const uint32_t a_s = sbase;
-  const uint32_t ring_s = sbase + SM::ring_off;
+  const uint32_t ring_s = sbase;
   const uint32_t bar_s = sbase + SM::bar_off;
   // barrier slots (8 bytes each)
   const uint32_t bar_full = bar_s;                   // [NST]
   const uint32_t bar_empty = bar_s + 8 * NST;        // [NST]
   const uint32_t bar_tfull = bar_s + 16 * NST;       // [2]
   const uint32_t bar_tempty = bar_tfull + 16;        // [2]
-  const uint32_t bar_afull = bar_tempty + 16;        // [1]
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(sgen + SM::bar_off + 16 * NST + 40);
-  volatile int* abort_flag = reinterpret_cast<volatile int*>(sgen + SM::bar_off + 16 * NST + 44);
-  static_assert(16 * NST + 48 <= 256, "barrier area");
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(sgen + SM::bar_off + 16 * NST + 32);
+  volatile int* abort_flag = reinterpret_cast<volatile int*>(sgen + SM::bar_off + 16 * NST + 36);
+  static_assert(16 * NST + 40 <= 256, "barrier area");
 
   const int warp = warp_index(), lane = threadIdx.x & 31;
   const int h = blockIdx.y;
@@ -74,7 +61,6 @@ gemm_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__ CU
       mbar_init(bar_tfull + 8 * b, 1);
       mbar_init(bar_tempty + 8 * b, 8);          // one arrival per epilogue warp
     }
-    mbar_init(bar_afull, 1);
     *abort_flag = 0;
     fence_mbar_init();
   }
@@ -94,9 +80,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__ CU
   chain_wait();
 
   // ---- tile range of this CTA ----------------------------------------------------------------
-  int n_tiles;
-  if (EPI == EPI_COLMAX) n_tiles = (g.cols_b + 127) >> 7;
-  else n_tiles = (((__shfl_sync(0xffffffffu, c.len[h], 0) + c.PT - 1) / c.PT) + 127) >> 7;
+  const int n_tiles = (((__shfl_sync(0xffffffffu, c.len[h], 0) + c.PT - 1) / c.PT) + 127) >> 7;
   const int per = (n_tiles + gridDim.z - 1) / gridDim.z;
   const int t0 = blockIdx.z * per;
   const int ntl = max(0, min(n_tiles, t0 + per) - t0);
@@ -106,10 +90,6 @@ gemm_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__ CU
     if (warp == kGemmProducerWarp) {
       // ------------------------------------------------------------------ TMA producer
       bool ok = true;
-      if (A_RES && lane == 0) {
-        mbar_arrive_expect_tx(bar_afull, nkc * kChunkBytes);
-        for (int kc = 0; kc < nkc; ++kc) tma_load_3d(a_s + kc * kChunkBytes, &tm_a, bar_afull, kc * 64, m0, h);
-      }
       int it = 0;
       if (lane == 0) {
         for (int tl = 0; tl < ntl && ok; ++tl) {
@@ -121,8 +101,8 @@ gemm_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__ CU
             if (!ok) break;
             const uint32_t st_s = ring_s + s * SM::stage_bytes;
             mbar_arrive_expect_tx(bar_full + 8 * s, SM::stage_bytes);
-            if (!A_RES) tma_load_3d(st_s, &tm_a, bar_full + 8 * s, kc * 64, m0, h);
-            tma_load_3d(A_RES ? st_s : st_s + kChunkBytes, &tm_b, bar_full + 8 * s, kc * 64, t * 128, h);
+            tma_load_3d(st_s, &tm_a, bar_full + 8 * s, kc * 64, m0, h);
+            tma_load_3d(st_s + kChunkBytes, &tm_b, bar_full + 8 * s, kc * 64, t * 128, h);
           }
         }
       }
@@ -136,7 +116,6 @@ gemm_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__ CU
         const uint32_t lead = elect_lane();
         constexpr uint32_t idesc = make_idesc_bf16(128, 128, 0);
         bool ok = true;
-        if (A_RES) ok = mbar_wait_warp<kIssueWaitHintNs>(bar_afull, 0, abort_flag, c.status);
         int it = 0;
         for (int tl = 0; tl < ntl && ok; ++tl) {
           const int buf = tl & 1, bph = (tl >> 1) & 1;
@@ -150,12 +129,10 @@ gemm_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__ CU
             if (!ok) break;
             tc_fence_after();
             const uint32_t st_s = ring_s + s * SM::stage_bytes;
-            const uint32_t a_c = A_RES ? a_s + kc * kChunkBytes : st_s;
-            const uint32_t b_c = A_RES ? st_s : st_s + kChunkBytes;
 #pragma unroll
             for (int k4 = 0; k4 < 4; ++k4) {
-              const uint64_t ad = make_smem_desc(a_c + k4 * 32, 16, 1024);
-              const uint64_t bd = make_smem_desc(b_c + k4 * 32, 16, 1024);
+              const uint64_t ad = make_smem_desc(st_s + k4 * 32, 16, 1024);
+              const uint64_t bd = make_smem_desc(st_s + kChunkBytes + k4 * 32, 16, 1024);
               umma_ss(d_t, ad, bd, idesc, (kc | k4) != 0, lead);
             }
             umma_commit(bar_empty + 8 * s, lead);
@@ -187,43 +164,11 @@ gemm_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__ CU
 #pragma unroll
         for (int c2 = 0; c2 < 2; ++c2) {
           const int cc = wg * 2 + c2;
-          const uint32_t(&v)[32] = vv[c2];
-          if (EPI == EPI_COLMAX) {
-            const bool rvalid = row < g.rows_a;
-            const int f_r = rvalid ? row / g.frame_len : -1;
-            int f_lo = rvalid ? f_r : 0x7fffffff, f_hi = f_r;
+          if (row < g.rows_a) {
+            float* dst = c.scores + (static_cast<int64_t>(h) * c.max_qb + row) * c.CAPB + t * 128 + cc * 32;
 #pragma unroll
-            for (int o = 16; o >= 1; o >>= 1) {
-              f_lo = min(f_lo, __shfl_xor_sync(0xffffffffu, f_lo, o));
-              f_hi = max(f_hi, __shfl_xor_sync(0xffffffffu, f_hi, o));
-            }
-            for (int f = f_lo; f <= f_hi; ++f) {       // empty when the warp has no valid row
-              float x[32];
-#pragma unroll
-              for (int j = 0; j < 32; ++j) x[j] = (f_r == f) ? __uint_as_float(v[j]) : -INFINITY;
-              // butterfly: after it, lane l holds the maximum of column l over the 32 rows
-#pragma unroll
-              for (int o = 16, w = 32; o >= 1; o >>= 1, w >>= 1) {
-                const bool up = (lane & o) != 0;
-#pragma unroll
-                for (int j = 0; j < w / 2; ++j) {
-                  const float send = up ? x[j] : x[j + w / 2];
-                  const float keep = up ? x[j + w / 2] : x[j];
-                  x[j] = fmaxf(keep, __shfl_xor_sync(0xffffffffu, send, o));
-                }
-              }
-              const int col = t * 128 + cc * 32 + lane;
-              if (col < g.cols_b)
-                atomicMax(c.rel + (static_cast<int64_t>(h) * c.max_frames + f) * c.max_prompt + col,
-                          float_to_ordered(x[0]));
-            }
-          } else {  // EPI_STORE
-            if (row < g.rows_a) {
-              float* dst = c.scores + (static_cast<int64_t>(h) * c.max_qb + row) * c.CAPB + t * 128 + cc * 32;
-#pragma unroll
-              for (int j = 0; j < 32; ++j)
-                if (t * 128 + cc * 32 + j < c.CAPB) dst[j] = __uint_as_float(v[j]);
-            }
+            for (int j = 0; j < 32; ++j)
+              if (t * 128 + cc * 32 + j < c.CAPB) dst[j] = __uint_as_float(vv[c2][j]);
           }
         }
       }
@@ -238,34 +183,15 @@ gemm_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__ CU
   }
 }
 
-template <int EPI, bool A_RES, int NST>
-static int launch_gemm(const CUtensorMap& tm_a, const CUtensorMap& tm_b, const CacheView& c, const GemmArgs& g, dim3 grid,
-                       cudaStream_t st) {
-  using SM = GemmSmem<EPI, A_RES, NST>;
-  auto kern = gemm_kernel<EPI, A_RES, NST>;
-  const int cfg = ensure_dynamic_smem(reinterpret_cast<const void*>(kern), SM::total);
-  if (cfg != FASTAR_OK) return cfg;
-  launch_chained(kern, grid, kGemmThreads, SM::total, st, tm_a, tm_b, c, g);
-  return cudaGetLastError() == cudaSuccess ? 1 : FASTAR_ERR_CUDA;
-}
-
-int launch_c1_relevance(const CacheView& c, const CUtensorMap& tm_q, const CUtensorMap& tm_kp, int nq, int np, int frame_len,
-                        int n_frames, cudaStream_t st) {
-  GemmArgs g{};
-  g.rows_a = nq;
-  g.nkc = c.D / 64;
-  g.frame_len = frame_len;
-  g.n_frames = n_frames;
-  g.cols_b = np;
-  return launch_gemm<EPI_COLMAX, true, 4>(tm_q, tm_kp, c, g, dim3((nq + 127) / 128, c.H, 1), st);
-}
-
 int launch_s3_scores(const CacheView& c, const CUtensorMap& tm_hq, const CUtensorMap& tm_hk, int nqb, cudaStream_t st) {
+  const int cfg = ensure_dynamic_smem(reinterpret_cast<const void*>(gemm_kernel), GemmSmem::total);
+  if (cfg != FASTAR_OK) return cfg;
   GemmArgs g{};
   g.rows_a = nqb;
   g.nkc = c.hist_cols / 64;
   const int col_tiles = (c.CAPB + 127) / 128;
-  return launch_gemm<EPI_STORE, false, 4>(tm_hq, tm_hk, c, g, dim3((nqb + 127) / 128, c.H, col_tiles), st);
+  launch_chained(gemm_kernel, dim3((nqb + 127) / 128, c.H, col_tiles), kGemmThreads, GemmSmem::total, st, tm_hq, tm_hk, c, g);
+  return cudaGetLastError() == cudaSuccess ? 1 : FASTAR_ERR_CUDA;
 }
 
 }  // namespace fastar

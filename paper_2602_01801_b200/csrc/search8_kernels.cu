@@ -10,9 +10,7 @@
 //
 //   quantize_kernel      : bf16 rows + 1/|x|  ->  codes
 //   quantize_rows_kernel : bf16 rows  ->  codes and |x| (AnnCA's queries and prompt keys, Section 5.3)
-//   search8_kernel<false>: codes of the new keys x codes of the cache, row arg-max fused (ties -> lowest slot)
-//   search8_kernel<true> : codes of the queries x codes of the prompt keys, scaled back by |q| |k|, per-frame column
-//                          maximum fused (AnnCA's prompt relevance on the quantised scores)
+//   search8_kernel       : codes of the new keys x codes of the cache, row arg-max fused (ties -> lowest slot)
 // Same CTA layout as the bf16 similarity kernel: 128 new keys per CTA (resident), key tiles streamed through a TMA
 // ring, two fp32 accumulators in TMEM, eight epilogue warps, 2 CTAs per SM.  Every wait is bounded.
 #include <cuda_fp8.h>
@@ -37,17 +35,6 @@ struct Smem {
   static constexpr int kn_off = bar_off + 256;                  // 2 x 128 floats: |k_j| of a tile's keys (query-probe ranking)
   static constexpr int total = kn_off + 2 * 128 * 4;
 };
-
-__device__ __forceinline__ void umma_ss_f8(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc, uint32_t accumulate,
-                                           uint32_t lead) {
-  asm volatile(
-      "{\n\t.reg .pred p, q;\n\t"
-      "setp.ne.b32 p, %4, 0;\n\t"
-      "setp.ne.b32 q, %5, 0;\n\t"
-      "@q tcgen05.mma.cta_group::1.kind::f8f6f4 [%0], %1, %2, %3, p;\n\t}"
-      ::"r"(d_tmem), "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate), "r"(lead)
-      : "memory");
-}
 
 }  // namespace
 
@@ -176,23 +163,12 @@ int launch_quantize_keys(const CacheView& c, const __nv_bfloat16* x, int n, int6
   return cudaGetLastError() == cudaSuccess ? 1 : FASTAR_ERR_CUDA;
 }
 
-// COLMAX = false: B = the paged code pool of the cache, row arg-max.  COLMAX = true: B = `cols_b` prompt-key codes
-// of head h (rows of a dense [H][rows][128] array), per-frame column maximum of score * |q| * |k|.
-struct Search8Args {
-  int rows_a;
-  int cols_b;              // COLMAX
-  int frame_len;           // COLMAX
-  const float* qn;         // COLMAX: |q|, [H][max_tokens]
-  const float* kn;         // COLMAX: |k_p|, [H][max_prompt]
-};
-
-// COLNORM (arg-max only): scores are multiplied by |k_j| before the maximum (query-probe ranking).  A template
+// COLNORM: scores are multiplied by |k_j| before the maximum (query-probe ranking).  A template
 // parameter, so that the plain search keeps its short epilogue.
-template <bool COLMAX, bool COLNORM = false>
+template <bool COLNORM>
 __global__ void __launch_bounds__(kThreads, 2)
 search8_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__ CUtensorMap tm_b, const CacheView c,
-               const Search8Args g) {
-  const int rows_a = g.rows_a;
+               int rows_a) {
   extern __shared__ __align__(1024) uint8_t smem_raw[];
   const uint32_t sbase = smem_u32(smem_raw);
   uint8_t* sgen = smem_raw;
@@ -244,7 +220,7 @@ search8_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
   tc_fence_after();
   const uint32_t tmem = *tmem_slot;
   chain_wait();
-  const int L = COLMAX ? g.cols_b : __shfl_sync(0xffffffffu, c.len[h], 0);
+  const int L = __shfl_sync(0xffffffffu, c.len[h], 0);
   const int n_tiles = (L + 127) >> 7;
   const int per = (n_tiles + gridDim.z - 1) / gridDim.z;
   const int t0 = blockIdx.z * per;
@@ -263,7 +239,7 @@ search8_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
       int pg0 = 0, pg1 = 0;
       for (int tl = 0; tl < ntl; ++tl) {
         const int t = t0 + tl;
-        if (!COLMAX && (tl & 31) == 0 && tl + lane < ntl) {      // page ids of 32 tiles with one coalesced load
+        if ((tl & 31) == 0 && tl + lane < ntl) {      // page ids of 32 tiles with one coalesced load
           pg0 = FASTAR_IDX(pt_h[(t + lane) * pages_per_tile], c.pool_pages, c.status);
           pg1 = pages_per_tile == 2 ? FASTAR_IDX(pt_h[(t + lane) * pages_per_tile + 1], c.pool_pages, c.status) : 0;
         }
@@ -275,12 +251,8 @@ search8_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
           if (ok) {
             const uint32_t b_s = ring_s + s * kTile;
             mbar_arrive_expect_tx(bar_full + 8 * s, kTile);
-            if (COLMAX) {
-              tma_load_3d(b_s, &tm_b, bar_full + 8 * s, 0, t * 128, h);   // rows past cols_b arrive as zeros
-            } else {
-              tma_load_3d(b_s, &tm_b, bar_full + 8 * s, 0, 0, page0);
-              if (pages_per_tile == 2) tma_load_3d(b_s + c.PT * 128, &tm_b, bar_full + 8 * s, 0, 0, page1);
-            }
+            tma_load_3d(b_s, &tm_b, bar_full + 8 * s, 0, 0, page0);
+            if (pages_per_tile == 2) tma_load_3d(b_s + c.PT * 128, &tm_b, bar_full + 8 * s, 0, 0, page1);
           }
         }
       }
@@ -319,26 +291,14 @@ search8_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
       float best = -INFINITY;
       int best_j = -1;
       // the scores are 256 x the quantised similarity (both code rows carry the factor 16)
-      const float need_from = (!COLMAX && !COLNORM && c.search_floor > -INFINITY) ? c.search_floor * (kCodeScale * kCodeScale) : -INFINITY;
+      const float need_from = (!COLNORM && c.search_floor > -INFINITY) ? c.search_floor * (kCodeScale * kCodeScale) : -INFINITY;
       float rn_next = 0.f;
       bool ok = true;
-      // COLMAX: |q| of this thread's row and the range of frames the warp's 32 rows fall in
-      const bool rvalid = row < rows_a;
-      const float qn = (COLMAX && rvalid) ? g.qn[static_cast<int64_t>(h) * c.max_tokens + row] : 0.f;
-      const int f_r = (COLMAX && rvalid) ? row / g.frame_len : -1;
-      int f_lo = (COLMAX && rvalid) ? f_r : 0x7fffffff, f_hi = f_r;
-      if (COLMAX) {
-#pragma unroll
-        for (int o = 16; o >= 1; o >>= 1) {
-          f_lo = min(f_lo, __shfl_xor_sync(0xffffffffu, f_lo, o));
-          f_hi = max(f_hi, __shfl_xor_sync(0xffffffffu, f_hi, o));
-        }
-      }
       for (int tl = 0; tl < ntl && ok; ++tl) {
         const int t = t0 + tl;
         const int buf = tl & 1;
         const int valid_cols = min(128, L - t * 128);
-        if (!COLMAX && COLNORM) {
+        if (COLNORM) {
           // |k_j| of the tile's keys through shared memory: one reciprocal per key, then broadcast reads
           if (wg == 0) {                 // the global load runs one tile ahead of its use
             if (tl == 0) rn_next = (t * 128 + r < L) ? c.rnorm[static_cast<int64_t>(h) * c.CAP + t * 128 + r] : 0.f;
@@ -347,14 +307,6 @@ search8_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
             rn_next = (tl + 1 < ntl && slot < L) ? c.rnorm[static_cast<int64_t>(h) * c.CAP + slot] : 0.f;
           }
           named_barrier_sync(1, 256);
-        }
-        float kn[2] = {0.f, 0.f};
-        if (COLMAX) {
-#pragma unroll
-          for (int c2 = 0; c2 < 2; ++c2) {
-            const int col = t * 128 + (wg * 2 + c2) * 32 + lane;
-            kn[c2] = col < g.cols_b ? g.kn[static_cast<int64_t>(h) * c.max_prompt + col] : 0.f;
-          }
         }
         ok = __all_sync(0xffffffffu, mbar_wait(bar_tfull + 8 * buf, (tl >> 1) & 1, abort_flag, c.status));
         if (!ok) break;                              // warp-uniform: TMEM loads are warp-collective
@@ -365,46 +317,19 @@ search8_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
         tmem_wait_ld();
         tc_fence_before();
         mbar_arrive_warp(bar_tempty + 8 * buf);      // the scores are in registers: release the accumulator
-        if (!COLMAX) {
-          // COLNORM: scores scaled by |k_j| of their column's key (the codes carry directions, the attention score
-          // also depends on the norm).  Only the last tile of a cache has columns to mask.
-          const float4* kn4 = reinterpret_cast<const float4*>(kn_s + buf * 128 + wg * 64);
-          const int jb = t * 128 + wg * 64;
-          if (valid_cols >= 128) {
-            chunk_argmax_t<false, COLNORM>(vv[0], kn4, 32, jb, need_from, best, best_j);
-            chunk_argmax_t<false, COLNORM>(vv[1], kn4 + 8, 32, jb + 32, need_from, best, best_j);
-          } else {
-            chunk_argmax_t<true, COLNORM>(vv[0], kn4, valid_cols - wg * 64, jb, need_from, best, best_j);
-            chunk_argmax_t<true, COLNORM>(vv[1], kn4 + 8, valid_cols - wg * 64 - 32, jb + 32, need_from, best, best_j);
-          }
-          continue;
-        }
-#pragma unroll
-        for (int c2 = 0; c2 < 2; ++c2) {
-          const int cc = wg * 2 + c2;
-          for (int f = f_lo; f <= f_hi; ++f) {         // empty when the warp has no valid row
-            float x[32];
-#pragma unroll
-            for (int j = 0; j < 32; ++j) x[j] = (f_r == f) ? __uint_as_float(vv[c2][j]) * qn : -INFINITY;
-            // butterfly: after it, lane l holds the maximum of column l over the 32 rows
-#pragma unroll
-            for (int o = 16, w = 32; o >= 1; o >>= 1, w >>= 1) {
-              const bool up = (lane & o) != 0;
-#pragma unroll
-              for (int j = 0; j < w / 2; ++j) {
-                const float send = up ? x[j] : x[j + w / 2];
-                const float keep = up ? x[j + w / 2] : x[j];
-                x[j] = fmaxf(keep, __shfl_xor_sync(0xffffffffu, send, o));
-              }
-            }
-            const int col = t * 128 + cc * 32 + lane;
-            if (col < g.cols_b)
-              atomicMax(c.rel + (static_cast<int64_t>(h) * c.max_frames + f) * c.max_prompt + col,
-                        float_to_ordered(x[0] * kn[c2]));
-          }
+        // COLNORM: scores scaled by |k_j| of their column's key (the codes carry directions, the attention score
+        // also depends on the norm).  Only the last tile of a cache has columns to mask.
+        const float4* kn4 = reinterpret_cast<const float4*>(kn_s + buf * 128 + wg * 64);
+        const int jb = t * 128 + wg * 64;
+        if (valid_cols >= 128) {
+          chunk_argmax_t<false, COLNORM>(vv[0], kn4, 32, jb, need_from, best, best_j);
+          chunk_argmax_t<false, COLNORM>(vv[1], kn4 + 8, 32, jb + 32, need_from, best, best_j);
+        } else {
+          chunk_argmax_t<true, COLNORM>(vv[0], kn4, valid_cols - wg * 64, jb, need_from, best, best_j);
+          chunk_argmax_t<true, COLNORM>(vv[1], kn4 + 8, valid_cols - wg * 64 - 32, jb + 32, need_from, best, best_j);
         }
       }
-      if (!COLMAX && ok && row < rows_a && best_j >= 0) {
+      if (ok && row < rows_a && best_j >= 0) {
         const float sim = best * (1.f / (kCodeScale * kCodeScale));
         const unsigned long long key = (static_cast<unsigned long long>(float_to_ordered(sim)) << 32) |
                                        static_cast<unsigned long long>(0xFFFFFFFFu - static_cast<uint32_t>(best_j));
@@ -423,7 +348,6 @@ search8_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
 
 static int configure_search8() {
   int r = ensure_dynamic_smem(reinterpret_cast<const void*>(search8_kernel<false>), Smem::total);
-  if (r == FASTAR_OK) r = ensure_dynamic_smem(reinterpret_cast<const void*>(search8_kernel<false, true>), Smem::total);
   if (r == FASTAR_OK) r = ensure_dynamic_smem(reinterpret_cast<const void*>(search8_kernel<true>), Smem::total);
   return r;
 }
@@ -451,27 +375,9 @@ int launch_t1_similarity_fp8(const CacheView& c, const CUtensorMap& tm_a8, const
                              cudaStream_t st) {
   if (configure_search8() != FASTAR_OK) return FASTAR_ERR_CUDA;
   const int row_tiles = (n + 127) / 128;
-  Search8Args g{};
-  g.rows_a = n;
   const dim3 grid(row_tiles, c.H, pick_splits8(row_tiles, c.H, c.CAP / 128));
-  if (col_norm) launch_chained(search8_kernel<false, true>, grid, kThreads, Smem::total, st, tm_a8, tm_pool_k8, c, g);
-  else launch_chained(search8_kernel<false, false>, grid, kThreads, Smem::total, st, tm_a8, tm_pool_k8, c, g);
-  return cudaGetLastError() == cudaSuccess ? 1 : FASTAR_ERR_CUDA;
-}
-
-// AnnCA prompt relevance on the 8-bit codes: c.rel (cleared by the caller) receives, as ordered integers,
-// max over the frame's queries of code(q) . code(k_p) * |q| * |k_p|; the caller decodes with 1 / (256 sqrt(d)).
-int launch_c1_relevance_fp8(const CacheView& c, const CUtensorMap& tm_q8, const CUtensorMap& tm_kp8, const float* qn,
-                            const float* kn, int nq, int np, int frame_len, cudaStream_t st) {
-  if (configure_search8() != FASTAR_OK) return FASTAR_ERR_CUDA;
-  const int row_tiles = (nq + 127) / 128;
-  Search8Args g{};
-  g.rows_a = nq;
-  g.cols_b = np;
-  g.frame_len = frame_len;
-  g.qn = qn;
-  g.kn = kn;
-  launch_chained(search8_kernel<true>, dim3(row_tiles, c.H, pick_splits8(row_tiles, c.H, (np + 127) / 128)), kThreads, Smem::total, st, tm_q8, tm_kp8, c, g);
+  if (col_norm) launch_chained(search8_kernel<true>, grid, kThreads, Smem::total, st, tm_a8, tm_pool_k8, c, n);
+  else launch_chained(search8_kernel<false>, grid, kThreads, Smem::total, st, tm_a8, tm_pool_k8, c, n);
   return cudaGetLastError() == cudaSuccess ? 1 : FASTAR_ERR_CUDA;
 }
 

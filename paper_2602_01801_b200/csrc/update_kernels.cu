@@ -666,7 +666,7 @@ int launch_query_hist(const CacheView& c, const uint32_t* codes, int nq, int blo
 // S4 / C2: per row keep the k largest entries (ties -> lower index), listed ascending.
 // ---------------------------------------------------------------------------------------------
 template <bool ORDERED_UINT>
-__global__ void __launch_bounds__(256) topk_kernel(const void* __restrict__ src, int64_t src_head_stride, int src_row_stride,
+__global__ void __launch_bounds__(256) topk_kernel(void* __restrict__ src, int64_t src_head_stride, int src_row_stride,
                                                    const int32_t* __restrict__ len, int len_div, int n_fixed, int keep,
                                                    int32_t* __restrict__ out, int64_t out_head_stride, int out_row_stride,
                                                    int out_fill, int32_t* __restrict__ nsel, int force_first, int force_last,
@@ -686,6 +686,7 @@ __global__ void __launch_bounds__(256) topk_kernel(const void* __restrict__ src,
     uint32_t v;
     if (ORDERED_UINT) {
       v = static_cast<const uint32_t*>(src)[so + i];
+      static_cast<uint32_t*>(src)[so + i] = 0u;          // the next call's maxima start there
     } else {
       v = static_cast<uint32_t>(static_cast<const float*>(src)[so + i]);
       if (src_hi) v += 256u * static_cast<uint32_t>(src_hi[so + i]);
@@ -833,6 +834,7 @@ int launch_reset(const CacheView& c, cudaStream_t st) {
   if (cudaMemsetAsync(c.pool_v, 0, pool, st) != cudaSuccess) return FASTAR_ERR_CUDA;
   if (cudaMemsetAsync(c.hk, 0, static_cast<size_t>(c.H) * c.CAPB * c.hist_cols * 2, st) != cudaSuccess) return FASTAR_ERR_CUDA;
   if (c.pool_k8 && cudaMemsetAsync(c.pool_k8, 0, static_cast<size_t>(c.pool_pages) * c.PT * 128, st) != cudaSuccess) return FASTAR_ERR_CUDA;
+  if (cudaMemsetAsync(c.rel, 0, static_cast<size_t>(c.H) * c.max_frames * c.max_prompt * 4, st) != cudaSuccess) return FASTAR_ERR_CUDA;
   reset_meta_kernel<<<296, 256, 0, st>>>(c);
   return cudaGetLastError() == cudaSuccess ? 1 : FASTAR_ERR_CUDA;
 }

@@ -1,0 +1,33 @@
+"""AnnCA at the edges of its tiles: one row, frames shorter than a tile and across tile borders, prompt groups of one to eight tiles,
+more units than CTAs; two calls in a row (the second must not see the first one's maxima)."""
+import numpy as np
+import pytest
+
+from oracle import fastar_oracle as O
+from paper_2602_01801_b200 import synth
+from tests import parity as P
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("heads,d,nq,frame_len,prompt,keep,bits", [
+    (1, 64, 1, 1, 1, 1, 16), (2, 128, 129, 129, 129, 5, 16), (3, 128, 300, 37, 513, 64, 16), (1, 64, 640, 64, 1024, 65, 16),
+    (2, 128, 64, 1, 200, 3, 16), (40, 64, 520, 260, 32, 8, 16), (2, 128, 300, 100, 130, 129, 8), (1, 64, 257, 256, 400, 64, 8)])
+def test_relevance_selection_attention(heads, d, nq, frame_len, prompt, keep, bits):
+    from paper_2602_01801_b200 import fastar
+
+    rng = np.random.default_rng(nq + prompt)
+    frames = -(-nq // frame_len)
+    cache = fastar.Cache(heads, d, 128, 64, rng.standard_normal((32, d)).astype(np.float32), max_tokens=nq, max_prompt_tokens=prompt,
+                         max_frames=frames, search_bits=bits)
+    for scale in (1.0, 0.25):                              # the second call's maxima are the smaller ones
+        Q, Kp, Vp = (synth.round_bf16(scale * rng.standard_normal((heads, n, d)).astype(np.float32)) for n in (nq, prompt, prompt))
+        r = cache.annca(fastar.to_device(Q), fastar.to_device(Kp), fastar.to_device(Vp), frame_len, keep, debug=True)
+        assert cache.status() == fastar.OK
+        codes = cache.export_annca_codes(nq, prompt) if bits == 8 else None
+        out = r["out"].float().cpu().numpy()
+        for h in sorted({0, heads // 2, heads - 1}):
+            sel = r["sel"][h].cpu().numpy()
+            P.check_prompt_selection(Q[h], Kp[h], frame_len, keep, sel, r["rel"][h].cpu().numpy(),
+                                     codes=(codes["q"][h][:, :d], codes["prompt"][h][:, :d]) if bits == 8 else None)
+            P.check_attention(out[h], O.annca(Q[h], Kp[h], Vp[h], frame_len, keep, sel=sel)["out"], f"AnnCA head {h}")
