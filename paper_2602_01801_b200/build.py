@@ -18,7 +18,7 @@ BOUNDS_LIB_PATH = os.path.join(LIB_DIR, "libfastar_bounds.so")
 SAN_LIB_PATH = os.path.join(LIB_DIR, "libfastar_hostsan.so")
 SAN_FLAGS = ["-Xcompiler", "-fsanitize=address", "-Xcompiler", "-fsanitize=undefined", "-Xcompiler", "-fno-omit-frame-pointer",
              "-Xcompiler", "-fno-sanitize-recover=undefined"]
-SOURCES = ["gemm_kernels.cu", "relevance_kernel.cu", "search_kernel.cu", "attn_kernels.cu", "update_kernels.cu", "commit_kernel.cu", "search8_kernels.cu", "fastar_api.cu", "noalloc_select.cu"]
+SOURCES = ["gemm_kernels.cu", "relevance_kernel.cu", "search_kernel.cu", "attn_kernels.cu", "prompt_attn_kernel.cu", "update_kernels.cu", "commit_kernel.cu", "search8_kernels.cu", "fastar_api.cu", "noalloc_select.cu"]
 NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17", "-Xcompiler", "-fPIC"]
 
 

@@ -560,13 +560,11 @@ int launch_attention_paged(const CacheView& c, const CUtensorMap& tm_q, const CU
 }
 
 int launch_attention_gather(const CacheView& c, const CUtensorMap& tm_q, const AttnArgs& a, cudaStream_t st) {
+  // one key tile of 64: a kernel of its own, which keeps the tile and streams the queries (12 x 4680 queries, 64 kept: 34.2 -> 11.5 us)
+  if (a.keep <= 64) return launch_attention_prompt64(c, tm_q, a, st);
   const dim3 grid((a.rows_per_frame + 127) / 128, c.H, a.n_frames);
-  const bool small = a.keep <= 64;
-  if (c.D == 128 && !small) return launch_attn<128, 128, true, false>(tm_q, tm_q, tm_q, tm_q, tm_q, c, a, grid, st);
-  if (c.D == 128 && small) return launch_attn<128, 64, true, false>(tm_q, tm_q, tm_q, tm_q, tm_q, c, a, grid, st);
-  if (c.D == 64 && !small) return launch_attn<64, 128, true, false>(tm_q, tm_q, tm_q, tm_q, tm_q, c, a, grid, st);
-  if (c.D == 64 && small) return launch_attn<64, 64, true, false>(tm_q, tm_q, tm_q, tm_q, tm_q, c, a, grid, st);
-  return FASTAR_ERR_UNSUPPORTED_SHAPE;
+  if (c.D == 128) return launch_attn<128, 128, true, false>(tm_q, tm_q, tm_q, tm_q, tm_q, c, a, grid, st);
+  return launch_attn<64, 128, true, false>(tm_q, tm_q, tm_q, tm_q, tm_q, c, a, grid, st);
 }
 
 }  // namespace fastar

@@ -190,6 +190,9 @@ int launch_attention_paged(const CacheView& c, const CUtensorMap& tm_q, const CU
                            const AttnArgs& a, cudaStream_t st);
 int launch_attention_gather(const CacheView& c, const CUtensorMap& tm_q, const AttnArgs& a, cudaStream_t st);
 
+// prompt_attn_kernel.cu: the gather mode for a.keep <= 64
+int launch_attention_prompt64(const CacheView& c, const CUtensorMap& tm_q, const AttnArgs& a, cudaStream_t st);
+
 // update_kernels.cu
 struct UpdateOut {         // the caller's [H][n] arrays (each may be null)
   int32_t* match;
