@@ -29,6 +29,11 @@ __device__ __forceinline__ void unpack8(const uint4& v, float (&f)[8]) {
   }
 }
 
+// 16 bytes global -> shared, asynchronous
+__device__ __forceinline__ void copy_async16(void* dst, const void* src) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(dst)), "l"(reinterpret_cast<uint64_t>(src)) : "memory");
+}
+
 // The 128-byte search code of a new token goes to the code row of its slot: LPR lanes, 128 / LPR bytes each.  The
 // load is issued with the other row loads (it could alias the pools as far as the compiler knows, so it must not
 // sit behind their stores), the store with the other stores.
@@ -64,6 +69,10 @@ __global__ void __launch_bounds__(256) commit_kernel(const CacheView c, const __
   const int sub = lane / LPR, sl = lane % LPR;
   const unsigned mask = ((LPR == 32) ? 0xffffffffu : ((1u << LPR) - 1u)) << (sub * LPR);
   const int w = (blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)) * GPW + sub;
+  // groups of several members: their tokens in ascending order, and the rows on their way (every lane its own 16 bytes)
+  constexpr int kHeld = 4, kRows = MEANK ? 2 : 4;
+  __shared__ int sorted_s[256 / LPR][kHeld * LPR];
+  __shared__ uint4 rows_s[MEANK ? 2 : 1][kRows][256];
   if (w >= n) return;                   // groups + unmatched tokens <= n
   const int64_t tb = static_cast<int64_t>(h) * c.max_tokens;
   const int64_t sb = static_cast<int64_t>(h) * c.CAP;
@@ -110,9 +119,73 @@ __global__ void __launch_bounds__(256) commit_kernel(const CacheView c, const __
 #pragma unroll
         for (int e = 0; e < 8; ++e) kacc[e] += f[e];
       }
+    } else if (g <= kHeld * LPR) {
+      // Members in ascending token order (the scatter left them unordered).  A member's place is the number of members below it;
+      // with the order known, four rows at a time come in by asynchronous copies, so a member costs a quarter of a load latency
+      // and no search, and no registers while it is under way: occupancy is what the common group of one needs.  12 x 4680 tokens:
+      // 8-bit search (groups of up to 50) 60 -> 27 us, bf16 search (two thirds of the tokens alone) 21.4 -> 21.7; 12 x 1560 by the
+      // probe 20.6 -> 10.4.  (Four rows at a time in registers: 31 us, but 30 with the bf16 search; eight staged: 24.5 and 23.0.)
+      int* order = sorted_s[threadIdx.x / LPR];
+      int best_f = -1;
+      float best_s = -INFINITY;
+      best_i = 0x7fffffff;
+      int tok[kHeld], place[kHeld];
+#pragma unroll
+      for (int q = 0; q < kHeld; ++q) {
+        const bool in = q * LPR + sl < g;
+        tok[q] = q == 0 ? mine : in ? c.order[tb + p0 + q * LPR + sl] : 0x7fffffff;
+        place[q] = 0;
+        if (in) {
+          const int fr = tok[q] / frame_len;
+          const float sm = c.sim[tb + tok[q]];
+          if (fr > best_f || (fr == best_f && (sm > best_s || (sm == best_s && tok[q] < best_i)))) { best_f = fr; best_s = sm; best_i = tok[q]; }
+        }
+      }
+#pragma unroll
+      for (int o = LPR / 2; o >= 1; o >>= 1) {
+        const int f2 = __shfl_xor_sync(mask, best_f, o), i2 = __shfl_xor_sync(mask, best_i, o);
+        const float s2 = __shfl_xor_sync(mask, best_s, o);
+        if (f2 > best_f || (f2 == best_f && (s2 > best_s || (s2 == best_s && i2 < best_i)))) { best_f = f2; best_s = s2; best_i = i2; }
+      }
+#pragma unroll
+      for (int q2 = 0; q2 < kHeld; ++q2) {
+        const int held = min(LPR, g - q2 * LPR);
+        for (int o = 0; o < held; ++o) {
+          const int other = __shfl_sync(mask, tok[q2], sub * LPR + o);
+#pragma unroll
+          for (int q = 0; q < kHeld; ++q) place[q] += other < tok[q] ? 1 : 0;
+        }
+      }
+#pragma unroll
+      for (int q = 0; q < kHeld; ++q)
+        if (q * LPR + sl < g) order[place[q]] = tok[q];
+      __syncwarp(mask);
+      for (int r0 = 0; r0 < g; r0 += kRows) {
+#pragma unroll
+        for (int b = 0; b < kRows; ++b)
+          if (r0 + b < g) {
+            const int64_t off = order[r0 + b] * ts + sl * 8;
+            copy_async16(&rows_s[0][b][threadIdx.x], vh + off);
+            if (MEANK) copy_async16(&rows_s[MEANK ? 1 : 0][b][threadIdx.x], kh + off);
+          }
+        asm volatile("cp.async.wait_all;" ::: "memory");
+#pragma unroll
+        for (int b = 0; b < kRows; ++b)
+          if (r0 + b < g) {
+            float f[8];
+            unpack8(rows_s[0][b][threadIdx.x], f);
+#pragma unroll
+            for (int e = 0; e < 8; ++e) acc[e] += f[e];
+            if (MEANK) {
+              unpack8(rows_s[MEANK ? 1 : 0][b][threadIdx.x], f);
+#pragma unroll
+              for (int e = 0; e < 8; ++e) kacc[e] += f[e];
+            }
+          }
+      }
     } else {
-      // Members in ascending token order (the scatter left them unordered): each round takes the smallest token
-      // index above the previous one.  Lanes hold the first LPR members, larger groups re-read the list.
+      // Larger groups, one member after the other: each round takes the smallest token index above the previous one, from the
+      // lanes (the first LPR members) and the list (the others).
       int best_f = -1, last = -1;
       float best_s = -INFINITY;
       best_i = -1;
