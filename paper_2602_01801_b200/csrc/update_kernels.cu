@@ -14,25 +14,19 @@ namespace fastar {
 // ---------------------------------------------------------------------------------------------
 __device__ __forceinline__ int block_sum(int v, int* red) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-#pragma unroll
-  for (int o = 16; o >= 1; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  v = __reduce_add_sync(0xffffffffu, v);
   __syncthreads();
   if (lane == 0) red[warp] = v;
   __syncthreads();
-  int t = 0;
-  for (int w = 0; w < nw; ++w) t += red[w];
-  return t;
+  return __reduce_add_sync(0xffffffffu, lane < nw ? red[lane] : 0);
 }
 __device__ __forceinline__ int block_max(int v, int* red) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-#pragma unroll
-  for (int o = 16; o >= 1; o >>= 1) v = max(v, __shfl_xor_sync(0xffffffffu, v, o));
+  v = __reduce_max_sync(0xffffffffu, v);
   __syncthreads();
   if (lane == 0) red[warp] = v;
   __syncthreads();
-  int t = red[0];
-  for (int w = 1; w < nw; ++w) t = max(t, red[w]);
-  return t;
+  return __reduce_max_sync(0xffffffffu, red[lane < nw ? lane : 0]);
 }
 // exclusive scan of one value per thread; *total receives the block sum
 __device__ __forceinline__ int block_exscan(int v, int* red, int* total) {
@@ -46,13 +40,9 @@ __device__ __forceinline__ int block_exscan(int v, int* red, int* total) {
   __syncthreads();
   if (lane == 31) red[warp] = inc;
   __syncthreads();
-  int base = 0, tot = 0;
-  for (int w = 0; w < nw; ++w) {
-    const int x = red[w];
-    if (w < warp) base += x;
-    tot += x;
-  }
-  *total = tot;
+  const int x = lane < nw ? red[lane] : 0;
+  const int base = static_cast<int>(__reduce_add_sync(0xffffffffu, lane < warp ? x : 0));
+  *total = static_cast<int>(__reduce_add_sync(0xffffffffu, x));
   return base + inc - v;
 }
 __device__ __forceinline__ void bitonic_sort_smem(unsigned long long* keys, int np2) {
@@ -327,21 +317,6 @@ __global__ void __launch_bounds__(1024) plan_kernel(const CacheView c, int n, in
   const int n_seg = seg_run, M = mem_run;
   if (tid == 0) c.segpos[gb + n_seg] = M;
 
-  // unmatched tokens in token order
-  int u_run = 0;
-  for (int i0 = 0; i0 < n; i0 += 4 * blockDim.x) {
-    const int i = i0 + 4 * tid;
-    int un[4];
-#pragma unroll
-    for (int u = 0; u < 4; ++u) un[u] = (i + u < n && c.match[tb + i + u] < 0) ? 1 : 0;
-    int tot;
-    int k = u_run + block_exscan(un[0] + un[1] + un[2] + un[3], red, &tot);
-#pragma unroll
-    for (int u = 0; u < 4; ++u)
-      if (un[u]) c.ulist[tb + k++] = i + u;
-    u_run += tot;
-  }
-  const int U = u_run;
   // Slot limit of this head.  Shared page pool: the free pages go to the heads in head order, each asking for what its
   // unmatched tokens need up to the capacity.  Every head's planner repeats the same short scan over the heads before
   // it (lengths, matched counts and the pool's fill are only written by the kernels that follow), so the CTAs need no
@@ -368,119 +343,158 @@ __global__ void __launch_bounds__(1024) plan_kernel(const CacheView c, int n, in
     const int held = (L + c.PT - 1) / c.PT;
     for (int p = tid; p < grant; p += blockDim.x) c.page_table[static_cast<int64_t>(h) * c.CAPB + held + p] = s_base + p;
   }
-  const int A = min(U, limit - L);
+
+  // Unmatched tokens in token order.  The first `limit - L` of them are appended; that needs no count of the others.
+  const int room = limit - L;
+  int u_run = 0;
+  for (int i0 = 0; i0 < n; i0 += 4 * blockDim.x) {
+    const int i = i0 + 4 * tid;
+    int un[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) un[u] = (i + u < n && c.match[tb + i + u] < 0) ? 1 : 0;
+    int tot;
+    int k = u_run + block_exscan(un[0] + un[1] + un[2] + un[3], red, &tot);
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+      if (un[u]) {
+        c.ulist[tb + k] = i + u;
+        if (k < room) {
+          c.dest[tb + i + u] = L + k;
+          if (dest_out) dest_out[static_cast<int64_t>(h) * n + i + u] = L + k;
+        }
+        ++k;
+      }
+    u_run += tot;
+  }
+  const int U = u_run;
+  const int A = min(U, room);
   const int E = U - A;
   int ok = 1;
-  // Eviction.  evictable = live, past the sink prefix, stamp < now, not touched by this update (cnt == 0); its key
-  // is its stamp, 0x7fffffff otherwise.  Every pass reads 16 consecutive slots per thread with 128-bit loads (eight
-  // of them in flight), so a pass over a 64k-slot cache is four round trips instead of sixty-four.
-  constexpr int kNever = 0x7fffffff;
-  auto evictable16 = [&](int j, int (&st)[16]) {
-    if (j < L) {                                   // j is a multiple of 16 and the capacity a multiple of 128
-      const int4* pc = reinterpret_cast<const int4*>(c.cnt + sb + j);
-      const int4* ps = reinterpret_cast<const int4*>(c.stamp + sb + j);
-      const int4 c0 = pc[0], c1 = pc[1], c2 = pc[2], c3 = pc[3];
-      const int4 s0 = ps[0], s1 = ps[1], s2 = ps[2], s3 = ps[3];
-      const int cn[16] = {c0.x, c0.y, c0.z, c0.w, c1.x, c1.y, c1.z, c1.w, c2.x, c2.y, c2.z, c2.w, c3.x, c3.y, c3.z, c3.w};
-      const int sp[16] = {s0.x, s0.y, s0.z, s0.w, s1.x, s1.y, s1.z, s1.w, s2.x, s2.y, s2.z, s2.w, s3.x, s3.y, s3.z, s3.w};
-#pragma unroll
-      for (int u = 0; u < 16; ++u)
-        st[u] = (j + u < L && j + u >= c.n_sink && cn[u] == 0 && sp[u] < now) ? sp[u] : kNever;
-    } else {
-#pragma unroll
-      for (int u = 0; u < 16; ++u) st[u] = kNever;
-    }
-  };
-  int smin = kNever, smax = -1;
+  // Eviction.  evictable = live, past the sink prefix, stamp < now, not touched by this update (cnt == 0).  The oldest E go, ties by
+  // slot; what is looked for is the age (now - stamp) that at least E evictable slots reach, the greatest such.
+  int evicted_tokens = 0;
   if (E > 0) {
-    // one pass: how many evictable slots there are, and the range of their stamps
-    int cand = 0;
-    for (int j0 = 0; j0 < L; j0 += 16 * blockDim.x) {
-      int st[16];
-      evictable16(j0 + 16 * tid, st);
+    // The 16 slots of pass p from j = 16 (1024 p + tid) on, read with 128-bit loads: their ages, 0 = not evictable.
+    auto ages16 = [&](int j, int (&age)[16]) {
+      if (j < L) {                                 // j is a multiple of 16 and the capacity a multiple of 128
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          const int4 cn = *reinterpret_cast<const int4*>(c.cnt + sb + j + 4 * q), sp = *reinterpret_cast<const int4*>(c.stamp + sb + j + 4 * q);
+          const int cq[4] = {cn.x, cn.y, cn.z, cn.w}, sq[4] = {sp.x, sp.y, sp.z, sp.w};
+#pragma unroll
+          for (int u = 0; u < 4; ++u) {
+            const int s = j + 4 * q + u;
+            age[4 * q + u] = (s < L && s >= c.n_sink && cq[u] == 0 && sq[u] < now) ? now - sq[u] : 0;
+          }
+        }
+      } else {
+#pragma unroll
+        for (int u = 0; u < 16; ++u) age[u] = 0;
+      }
+    };
+    // Up to 2 x 16384 slots a thread keeps its ages in registers, two to a word, so the search for the age and the compaction read
+    // nothing again (12 heads x 32768 slots at capacity: 87 -> 44 us; longer caches, and ages above 16 bits, go through L2 in every
+    // pass, as all did before).
+    constexpr int kPasses = 2;
+    uint32_t held[kPasses][8];
+    int cand = 0, a_min = 0x7fffffff, a_max = 0;
+    for (int j0 = 0, p = 0; j0 < L; j0 += 16 * blockDim.x, ++p) {
+      int age[16];
+      ages16(j0 + 16 * tid, age);
 #pragma unroll
       for (int u = 0; u < 16; ++u)
-        if (st[u] != kNever) { ++cand; smin = min(smin, st[u]); smax = max(smax, st[u]); }
+        if (age[u] > 0) { ++cand; a_min = min(a_min, age[u]); a_max = max(a_max, age[u]); }
+#pragma unroll
+      for (int q = 0; q < kPasses; ++q)
+        if (p == q)
+#pragma unroll
+          for (int u = 0; u < 8; ++u) held[q][u] = (static_cast<uint32_t>(age[2 * u]) & 0xFFFFu) | (static_cast<uint32_t>(age[2 * u + 1]) << 16);
     }
     cand = block_sum(cand, red);
-    smin = -block_max(-smin, red);
-    smax = block_max(smax, red);
+    a_min = -block_max(-a_min, red);
+    a_max = block_max(a_max, red);
     if (cand < E) ok = 0;
-  }
-  int evicted_tokens = 0;
-  if (ok && E > 0) {
-    // smallest stamp value s* such that at least E evictable slots have stamp <= s*
-    int lo = smin, hi = smax;
-    while (lo < hi) {
-      const int mid = lo + ((hi - lo) >> 1);
+    const bool in_regs = L <= kPasses * 16 * static_cast<int>(blockDim.x) && a_max <= 0xFFFF;
+    auto for_each_pass = [&](auto&& body) {        // body(first slot, ages)
+      int age[16];
+      if (in_regs) {
+#pragma unroll
+        for (int p = 0; p < kPasses; ++p) {
+          const int j0 = p * 16 * blockDim.x;
+          if (j0 >= L) break;
+#pragma unroll
+          for (int u = 0; u < 8; ++u) { age[2 * u] = held[p][u] & 0xFFFFu; age[2 * u + 1] = held[p][u] >> 16; }
+          body(j0 + 16 * tid, age);
+        }
+      } else {
+        for (int j0 = 0; j0 < L; j0 += 16 * blockDim.x) {
+          ages16(j0 + 16 * tid, age);
+          body(j0 + 16 * tid, age);
+        }
+      }
+    };
+    auto reach = [&](int a) {                      // evictable slots of that age or older
       int cn = 0;
-      for (int j0 = 0; j0 < L; j0 += 16 * blockDim.x) {
-        int st[16];
-        evictable16(j0 + 16 * tid, st);
+      for_each_pass([&](int, int (&age)[16]) {
 #pragma unroll
-        for (int u = 0; u < 16; ++u) cn += st[u] <= mid ? 1 : 0;
+        for (int u = 0; u < 16; ++u) cn += age[u] >= a ? 1 : 0;
+      });
+      return block_sum(cn, red);
+    };
+    if (ok) {
+      int lo = a_min, hi = a_max;                  // all reach a_min
+      while (lo < hi) {
+        const int mid = lo + ((hi - lo + 1) >> 1);
+        if (reach(mid) >= E) lo = mid; else hi = mid - 1;
       }
-      cn = block_sum(cn, red);
-      if (cn >= E) hi = mid; else lo = mid + 1;
-    }
-    const int sstar = lo;
-    int c_less = 0;
-    for (int j0 = 0; j0 < L; j0 += 16 * blockDim.x) {
-      int st[16];
-      evictable16(j0 + 16 * tid, st);
+      const int a_star = lo;
+      const int need_eq = E - reach(a_star + 1);
+      // ordered compaction of the victims: all older slots, and the first need_eq slots of that age
+      int eq_run = 0, out_run = 0;
+      for_each_pass([&](int j, int (&age)[16]) {
+        int my_eq = 0;
 #pragma unroll
-      for (int u = 0; u < 16; ++u) c_less += st[u] < sstar ? 1 : 0;
-    }
-    c_less = block_sum(c_less, red);
-    const int need_eq = E - c_less;
-    // ordered compaction of the victims: all slots below s*, and the first need_eq slots at s*
-    int eq_run = 0, out_run = 0;
-    for (int j0 = 0; j0 < L; j0 += 16 * blockDim.x) {
-      const int j = j0 + 16 * tid;
-      int st[16];
-      evictable16(j, st);
-      int my_eq = 0;
+        for (int u = 0; u < 16; ++u) my_eq += age[u] == a_star ? 1 : 0;
+        int tot_eq;
+        int eq_rank = eq_run + block_exscan(my_eq, red, &tot_eq);
+        int my_take = 0;
+        unsigned take_mask = 0;
 #pragma unroll
-      for (int u = 0; u < 16; ++u) my_eq += st[u] == sstar ? 1 : 0;
-      int tot_eq;
-      int eq_rank = eq_run + block_exscan(my_eq, red, &tot_eq);
-      int my_take = 0;
-      unsigned take_mask = 0;
+        for (int u = 0; u < 16; ++u) {
+          const bool is_eq = age[u] == a_star;
+          const bool take = age[u] > a_star || (is_eq && eq_rank < need_eq);
+          eq_rank += is_eq ? 1 : 0;
+          take_mask |= (take ? 1u : 0u) << u;
+          my_take += take ? 1 : 0;
+        }
+        int tot_take;
+        int pos = out_run + block_exscan(my_take, red, &tot_take);
 #pragma unroll
-      for (int u = 0; u < 16; ++u) {
-        const bool is_eq = st[u] == sstar;
-        const bool take = st[u] < sstar || (is_eq && eq_rank < need_eq);
-        eq_rank += is_eq ? 1 : 0;
-        take_mask |= (take ? 1u : 0u) << u;
-        my_take += take ? 1 : 0;
+        for (int u = 0; u < 16; ++u)
+          if ((take_mask >> u) & 1u)
+            keys[pos++] = (static_cast<unsigned long long>(static_cast<uint32_t>(now - age[u])) << 32) | static_cast<uint32_t>(j + u);
+        eq_run += tot_eq;
+        out_run += tot_take;
+      });
+      int e2 = 1;
+      while (e2 < E) e2 <<= 1;
+      for (int p = E + tid; p < e2; p += blockDim.x) keys[p] = ~0ull;
+      __syncthreads();
+      bitonic_sort_smem(keys, e2);
+      int ev = 0;
+      for (int k = tid; k < E; k += blockDim.x) {
+        const int v = static_cast<int>(keys[k] & 0xFFFFFFFFull);
+        c.victims[tb + k] = v;
+        ev += c.count[sb + v];
       }
-      int tot_take;
-      int pos = out_run + block_exscan(my_take, red, &tot_take);
-#pragma unroll
-      for (int u = 0; u < 16; ++u)
-        if ((take_mask >> u) & 1u)
-          keys[pos++] = (static_cast<unsigned long long>(static_cast<uint32_t>(st[u])) << 32) | static_cast<uint32_t>(j + u);
-      eq_run += tot_eq;
-      out_run += tot_take;
+      evicted_tokens = block_sum(ev, red);
     }
-    int e2 = 1;
-    while (e2 < E) e2 <<= 1;
-    for (int p = E + tid; p < e2; p += blockDim.x) keys[p] = ~0ull;
-    __syncthreads();
-    bitonic_sort_smem(keys, e2);
-    int ev = 0;
-    for (int k = tid; k < E; k += blockDim.x) {
-      const int v = static_cast<int>(keys[k] & 0xFFFFFFFFull);
-      c.victims[tb + k] = v;
-      ev += c.count[sb + v];
-    }
-    evicted_tokens = block_sum(ev, red);
   }
   __syncthreads();
-  // destinations (matched tokens get theirs in the scatter kernel)
+  // destinations of the tokens that take a victim's slot (matched tokens get theirs in the scatter kernel)
   if (ok) {
-    for (int k = tid; k < U; k += blockDim.x) {
-      const int i = FASTAR_IDX(c.ulist[tb + k], n, c.status), d = FASTAR_IDX(k < A ? L + k : c.victims[tb + k - A], c.CAP, c.status);
+    for (int k = A + tid; k < U; k += blockDim.x) {
+      const int i = FASTAR_IDX(c.ulist[tb + k], n, c.status), d = FASTAR_IDX(c.victims[tb + k - A], c.CAP, c.status);
       c.dest[tb + i] = d;
       if (dest_out) dest_out[static_cast<int64_t>(h) * n + i] = d;
     }
