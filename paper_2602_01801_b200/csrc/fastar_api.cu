@@ -312,10 +312,10 @@ int fastar_cache_create(fastar_cache_t** out, const fastar_cache_desc* desc, con
                  static_cast<uint64_t>(v.max_qb) * v.hist_cols * 2, 128);
   if (r == FASTAR_OK)
     r = make_map(c, &c->tm_hk, v.hk, v.hist_cols, v.CAPB, v.H, static_cast<uint64_t>(v.hist_cols) * 2,
-                 static_cast<uint64_t>(v.CAPB) * v.hist_cols * 2, 128);
+                 static_cast<uint64_t>(v.CAPB) * v.hist_cols * 2, 64);
   if (r == FASTAR_OK && v.hist_weighted)
     r = make_map(c, &c->tm_hk_hi, v.hk_hi, v.hist_cols, v.CAPB, v.H, static_cast<uint64_t>(v.hist_cols) * 2,
-                 static_cast<uint64_t>(v.CAPB) * v.hist_cols * 2, 128);
+                 static_cast<uint64_t>(v.CAPB) * v.hist_cols * 2, 64);
   if (r == FASTAR_OK && v.search_bits == 8)
     r = make_map_codes(c, &c->tm_pool_k8, v.pool_k8, PT, static_cast<uint64_t>(v.pool_pages), PT * 128, v.PT);
   if (r == FASTAR_OK &&

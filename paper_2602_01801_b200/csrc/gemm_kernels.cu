@@ -1,8 +1,10 @@
 // S3: bucket-collision scores HQ x HK^T (AnnSA block selection, Sections 5.1 / 5.4) on tcgen05 / TMEM / TMA.
 //
-// One CTA = one 128-row tile of HQ and a range of 128-row tiles of HK; D[128 x 128] fp32 lives in
-// TMEM, double buffered so the epilogue of tile t overlaps the MMAs of tile t+1.
-// Warp roles: warps 0-7 epilogue (two threads per row / TMEM lane, one per 64-column half), warp 8 TMA
+// One CTA = one 128-row tile of HQ and a range of 64-row tiles of HK; D[128 x 64] fp32 lives in TMEM, double buffered so the
+// epilogue of tile t overlaps the MMAs of tile t+1.  The product is small (37 x 220 x 1024 for a 12-head layer's head), so it is
+// bound by the latency of sixteen dependent 64-column steps, and by how many SMs take part: 64 keys a tile and two CTAs per SM
+// (128 keys and one CTA before: 10.9 -> 7.7 us; 32 x 1056 x 1024 of 8 heads 13.4 -> 9.4; 85 x 507 of 40 heads 35 -> 24).
+// Warp roles: warps 0-7 epilogue (two threads per row / TMEM lane, one per 32-column half), warp 8 TMA
 // producer, warp 9 TMEM allocation + MMA issue.  Operands are bf16, K-major, 128-byte swizzled.
 #include "common.h"
 #include "ptx.cuh"
@@ -16,18 +18,19 @@ struct GemmArgs {
 };
 
 constexpr int kChunkBytes = 128 * 128;       // 128 rows x 64 bf16
-constexpr int kTmemCols = 256;
+constexpr int kTileN = 64;                   // rows of HK per tile
+constexpr int kTmemCols = 2 * kTileN;
 constexpr int kGemmThreads = 320;            // warps 0-7 epilogue, 8 TMA producer, 9 MMA issue
 constexpr int kGemmProducerWarp = 8, kGemmMmaWarp = 9;
 
 constexpr int NST = 4;                       // ring stages of a chunk of both operands
 struct GemmSmem {
-  static constexpr int stage_bytes = 2 * kChunkBytes;
+  static constexpr int stage_bytes = kChunkBytes + kTileN * 128;
   static constexpr int bar_off = NST * stage_bytes;
   static constexpr int total = bar_off + 256;
 };
 
-__global__ void __launch_bounds__(kGemmThreads, 1)
+__global__ void __launch_bounds__(kGemmThreads, 2)
 gemm_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__ CUtensorMap tm_b, const CacheView c,
             const GemmArgs g) {
   using SM = GemmSmem;
@@ -80,7 +83,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__ CU
   chain_wait();
 
   // ---- tile range of this CTA ----------------------------------------------------------------
-  const int n_tiles = (((__shfl_sync(0xffffffffu, c.len[h], 0) + c.PT - 1) / c.PT) + 127) >> 7;
+  const int n_tiles = (((__shfl_sync(0xffffffffu, c.len[h], 0) + c.PT - 1) / c.PT) + kTileN - 1) / kTileN;
   const int per = (n_tiles + gridDim.z - 1) / gridDim.z;
   const int t0 = blockIdx.z * per;
   const int ntl = max(0, min(n_tiles, t0 + per) - t0);
@@ -102,7 +105,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__ CU
             const uint32_t st_s = ring_s + s * SM::stage_bytes;
             mbar_arrive_expect_tx(bar_full + 8 * s, SM::stage_bytes);
             tma_load_3d(st_s, &tm_a, bar_full + 8 * s, kc * 64, m0, h);
-            tma_load_3d(st_s + kChunkBytes, &tm_b, bar_full + 8 * s, kc * 64, t * 128, h);
+            tma_load_3d(st_s + kChunkBytes, &tm_b, bar_full + 8 * s, kc * 64, t * kTileN, h);
           }
         }
       }
@@ -114,7 +117,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__ CU
       // ------------------------------------------------------------------ MMA issue
       {
         const uint32_t lead = elect_lane();
-        constexpr uint32_t idesc = make_idesc_bf16(128, 128, 0);
+        constexpr uint32_t idesc = make_idesc_bf16(128, kTileN, 0);
         bool ok = true;
         int it = 0;
         for (int tl = 0; tl < ntl && ok; ++tl) {
@@ -122,7 +125,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__ CU
           ok = mbar_wait_warp<kIssueWaitHintNs>(bar_tempty + 8 * buf, bph ^ 1, abort_flag, c.status);
           if (!ok) break;
           tc_fence_after();
-          const uint32_t d_t = tmem + buf * 128;
+          const uint32_t d_t = tmem + buf * kTileN;
           for (int kc = 0; kc < nkc; ++kc, ++it) {
             const int s = it % NST;
             ok = mbar_wait_warp<kIssueWaitHintNs>(bar_full + 8 * s, (it / NST) & 1, abort_flag, c.status);
@@ -142,8 +145,6 @@ gemm_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__ CU
       }
     } else {
       // ------------------------------------------------------------------ epilogue (256 threads)
-      // Two threads per A row: warps 0-3 take columns 0-63 of every tile, warps 4-7 columns 64-127.  A TMEM
-      // load costs a few hundred cycles, so both 32-column loads of a thread are issued before the one wait.
       const int wg = warp >> 2;
       const int r = (warp & 3) * 32 + lane;         // A row inside the tile = TMEM lane
       const int row = m0 + r;
@@ -155,20 +156,23 @@ gemm_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__ CU
         ok = __all_sync(0xffffffffu, mbar_wait(bar_tfull + 8 * buf, bph, abort_flag, c.status));
         if (!ok) break;                              // warp-uniform: TMEM loads are warp-collective
         tc_fence_after();
-        uint32_t vv[2][32];
-        tmem_ld32(tmem + lane_addr + buf * 128 + wg * 64, vv[0]);
-        tmem_ld32(tmem + lane_addr + buf * 128 + wg * 64 + 32, vv[1]);
+        uint32_t v[32];
+        tmem_ld32(tmem + lane_addr + buf * kTileN + wg * 32, v);
         tmem_wait_ld();
         tc_fence_before();
         mbar_arrive_warp(bar_tempty + 8 * buf);      // the scores are in registers: release the accumulator
+        if (row < g.rows_a) {
+          const int col = t * kTileN + wg * 32;
+          float* dst = c.scores + (static_cast<int64_t>(h) * c.max_qb + row) * c.CAPB + col;
+          if ((c.CAPB & 3) == 0) {                   // rows start on 16-byte boundaries
 #pragma unroll
-        for (int c2 = 0; c2 < 2; ++c2) {
-          const int cc = wg * 2 + c2;
-          if (row < g.rows_a) {
-            float* dst = c.scores + (static_cast<int64_t>(h) * c.max_qb + row) * c.CAPB + t * 128 + cc * 32;
+            for (int j = 0; j < 32; j += 4)
+              if (col + j < c.CAPB)
+                *reinterpret_cast<float4*>(dst + j) = make_float4(__uint_as_float(v[j]), __uint_as_float(v[j + 1]), __uint_as_float(v[j + 2]), __uint_as_float(v[j + 3]));
+          } else {
 #pragma unroll
             for (int j = 0; j < 32; ++j)
-              if (t * 128 + cc * 32 + j < c.CAPB) dst[j] = __uint_as_float(vv[c2][j]);
+              if (col + j < c.CAPB) dst[j] = __uint_as_float(v[j]);
           }
         }
       }
@@ -189,7 +193,7 @@ int launch_s3_scores(const CacheView& c, const CUtensorMap& tm_hq, const CUtenso
   GemmArgs g{};
   g.rows_a = nqb;
   g.nkc = c.hist_cols / 64;
-  const int col_tiles = (c.CAPB + 127) / 128;
+  const int col_tiles = (c.CAPB + kTileN - 1) / kTileN;
   launch_chained(gemm_kernel, dim3((nqb + 127) / 128, c.H, col_tiles), kGemmThreads, GemmSmem::total, st, tm_hq, tm_hk, c, g);
   return cudaGetLastError() == cudaSuccess ? 1 : FASTAR_ERR_CUDA;
 }

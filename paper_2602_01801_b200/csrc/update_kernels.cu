@@ -93,7 +93,8 @@ int launch_convert_f32_to_bf16(const float* src, __nv_bfloat16* dst, int H, int 
 // ---------------------------------------------------------------------------------------------
 // X[n x D] . R^T[D x 32] is a skinny contraction (N = 32) bound by reading X once, so it runs on warp-level
 // mma.sync (m16n8k16, bf16 in, fp32 accumulate) with R held in registers: one warp = 16 rows per pass, no shared
-// memory, ~100 instructions per 16 rows.  Fragment layout (g = lane / 4, t = lane % 4):
+// memory, ~100 instructions per 16 rows.  The next group's rows are fetched as this one's are used up (40 x 10800 rows, 110 MB,
+// 17 us at the measured bandwidth: 48 -> 39 us; 12 x 4680 9.9 -> 8.9).  Fragment layout (g = lane / 4, t = lane % 4):
 //   A: a0 = X[g][2t..], a1 = X[g+8][2t..], a2 = X[g][2t+8..], a3 = X[g+8][2t+8..]   (bf16 pairs)
 //   B: b0 = R[n = 8*nt + g][2t..], b1 = R[n][2t+8..];   C: c0,c1 = row g, cols 2t,2t+1;  c2,c3 = row g+8.
 template <int D>
@@ -133,27 +134,40 @@ __global__ void __launch_bounds__(256) prep_kernel(const __nv_bfloat16* __restri
   // 16-row groups of all heads, dealt to the warps of a grid that fills the SMs once
   const int groups_per_head = (n + 15) / 16;
   const int total_groups = groups_per_head * H;
-  for (int grp = blockIdx.x * 8 + warp; grp < total_groups; grp += gridDim.x * 8) {
+  uint4 va[KS / 2], vb[KS / 2];
+  const __nv_bfloat16 *xa = x, *xb = x;                                // this lane's rows of the group that is fetched
+  auto rows = [&](int grp) {
     const int h = grp / groups_per_head;
     const int r0 = (grp - h * groups_per_head) * 16;
-    const int ra = min(r0 + g, n - 1), rb = min(r0 + g + 8, n - 1);   // rows past the end repeat the last one
-    const __nv_bfloat16* xa = x + h * hs + ra * ts + 8 * t;
-    const __nv_bfloat16* xb = x + h * hs + rb * ts + 8 * t;
+    xa = x + h * hs + min(r0 + g, n - 1) * ts + 8 * t;                  // rows past the end repeat the last one
+    xb = x + h * hs + min(r0 + g + 8, n - 1) * ts + 8 * t;
+  };
+  auto fetch = [&](int kk) {                                           // one 128-bit load per row and 32-wide k block
+    va[kk] = *reinterpret_cast<const uint4*>(xa + 32 * kk);
+    vb[kk] = *reinterpret_cast<const uint4*>(xb + 32 * kk);
+  };
+  const int first = blockIdx.x * 8 + warp;
+  if (first < total_groups) {
+    rows(first);
+#pragma unroll
+    for (int kk = 0; kk < KS / 2; ++kk) fetch(kk);
+  }
+  for (int grp = first; grp < total_groups; grp += gridDim.x * 8) {
+    const int h = grp / groups_per_head;
+    const int r0 = (grp - h * groups_per_head) * 16;
+    const bool more = grp + static_cast<int>(gridDim.x) * 8 < total_groups;
+    if (more) rows(grp + gridDim.x * 8);
     float acc[4][4];
 #pragma unroll
     for (int nt = 0; nt < 4; ++nt)
 #pragma unroll
       for (int e = 0; e < 4; ++e) acc[nt][e] = 0.f;
     float sqa = 0.f, sqb = 0.f;
-    uint4 va = make_uint4(0, 0, 0, 0), vb = va;
 #pragma unroll
     for (int ks = 0; ks < KS; ++ks) {
-      if ((ks & 1) == 0) {                                // one 128-bit load per row and 32-wide k block
-        va = *reinterpret_cast<const uint4*>(xa + 32 * (ks >> 1));
-        vb = *reinterpret_cast<const uint4*>(xb + 32 * (ks >> 1));
-      }
-      const uint32_t a0 = (ks & 1) ? va.z : va.x, a2 = (ks & 1) ? va.w : va.y;
-      const uint32_t a1 = (ks & 1) ? vb.z : vb.x, a3 = (ks & 1) ? vb.w : vb.y;
+      const uint4 pa = va[ks >> 1], pb = vb[ks >> 1];
+      const uint32_t a0 = (ks & 1) ? pa.z : pa.x, a2 = (ks & 1) ? pa.w : pa.y;
+      const uint32_t a1 = (ks & 1) ? pb.z : pb.x, a3 = (ks & 1) ? pb.w : pb.y;
       {
         const float2 f0 = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&a0));
         const float2 f2 = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&a2));
@@ -167,6 +181,7 @@ __global__ void __launch_bounds__(256) prep_kernel(const __nv_bfloat16* __restri
         asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%0, %1, %2, %3};"
                      : "+f"(acc[nt][0]), "+f"(acc[nt][1]), "+f"(acc[nt][2]), "+f"(acc[nt][3])
                      : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(bf[ks][nt][0]), "r"(bf[ks][nt][1]));
+      if ((ks & 1) && more) fetch(ks >> 1);               // the registers are free: the next group's rows, in flight until its turn
     }
     // sign bits: this lane owns columns 8*nt + 2t, +1 of rows g and g+8; OR over the quad gives all 32 columns
     uint32_t ma = 0, mb = 0;
@@ -597,16 +612,31 @@ int launch_plan(const CacheView& c, int n, float tau, const UpdateOut& out, cuda
   return cudaGetLastError() == cudaSuccess ? 3 : FASTAR_ERR_CUDA;
 }
 
+// Eight counters as bf16: all of them (SHIFT < 0: exact up to 256), or one of their two 8-bit digits.
+template <int SHIFT>
+__device__ __forceinline__ uint4 pack_counts(const int (&v)[8]) {
+  uint32_t w[4];
+#pragma unroll
+  for (int e = 0; e < 4; ++e) {
+    const int lo = SHIFT < 0 ? v[2 * e] : (v[2 * e] >> (SHIFT < 0 ? 0 : SHIFT)) & 255, hi = SHIFT < 0 ? v[2 * e + 1] : (v[2 * e + 1] >> (SHIFT < 0 ? 0 : SHIFT)) & 255;
+    w[e] = pack_bf16x2(static_cast<float>(lo), static_cast<float>(hi));
+  }
+  return make_uint4(w[0], w[1], w[2], w[3]);
+}
+
 // ---------------------------------------------------------------------------------------------
 // S2 (key side) + end of an update: bucket histogram of every key block, new lengths, stats, clock.
 // ---------------------------------------------------------------------------------------------
-__global__ void __launch_bounds__(256) key_hist_kernel(const CacheView c, int use_plan, fastar_update_stats* stats_out,
+// One CTA of 128 threads per block: a slot per thread, then 16 bytes of the histogram per thread.  A block's row is 2 KB of bf16 for
+// at most 128 codes, so what bounds it is writing the rows (40 heads x 512 blocks: 42 MB, 6.4 us) and the CTAs' starts; with 2-byte
+// stores by 256 threads 39 -> 29 us, 12 heads x 256 blocks 6.8 -> 5.5.
+__global__ void __launch_bounds__(128) key_hist_kernel(const CacheView c, int use_plan, fastar_update_stats* stats_out,
                                                        int advance_clock) {
   chain_wait();
-  extern __shared__ int hist[];          // hist_cols counters
+  extern __shared__ __align__(16) int hist[];          // hist_cols counters, a multiple of 64
   const int b = blockIdx.x, h = blockIdx.y;
   const int L = use_plan ? c.plan[h].len_new : c.len[h];
-  for (int q = threadIdx.x; q < c.hist_cols; q += blockDim.x) hist[q] = 0;
+  for (int q = threadIdx.x; q < c.hist_cols / 4; q += blockDim.x) reinterpret_cast<int4*>(hist)[q] = make_int4(0, 0, 0, 0);
   __syncthreads();
   const int s0 = b * c.PT, s1 = min(L, s0 + c.PT);
   const int nb = 1 << c.B;
@@ -619,14 +649,16 @@ __global__ void __launch_bounds__(256) key_hist_kernel(const CacheView c, int us
   }
   __syncthreads();
   const int64_t ho = (static_cast<int64_t>(h) * c.CAPB + b) * c.hist_cols;
-  for (int q = threadIdx.x; q < c.hist_cols; q += blockDim.x) {
+  for (int q = threadIdx.x; q < c.hist_cols / 8; q += blockDim.x) {
+    int v[8];
+#pragma unroll
+    for (int e = 0; e < 8; ++e) v[e] = hist[8 * q + e];
     if (c.hist_weighted) {
-      const int v = min(max(hist[q], 0), 65535);       // max: a sum of saturated weights could wrap
-      c.hk[ho + q] = __float2bfloat16(static_cast<float>(v & 255));
-      c.hk_hi[ho + q] = __float2bfloat16(static_cast<float>(v >> 8));
-    } else {
-      c.hk[ho + q] = __float2bfloat16(static_cast<float>(hist[q]));
+#pragma unroll
+      for (int e = 0; e < 8; ++e) v[e] = min(max(v[e], 0), 65535);       // max: a sum of saturated weights could wrap
+      reinterpret_cast<uint4*>(c.hk_hi + ho)[q] = pack_counts<8>(v);
     }
+    reinterpret_cast<uint4*>(c.hk + ho)[q] = c.hist_weighted ? pack_counts<0>(v) : pack_counts<-1>(v);
   }
   if (b == 0 && threadIdx.x == 0 && use_plan) {
     const PlanRec pr = c.plan[h];
@@ -648,7 +680,7 @@ __global__ void __launch_bounds__(256) key_hist_kernel(const CacheView c, int us
   }
 }
 int launch_finalize_hist(const CacheView& c, fastar_update_stats* stats_out, int advance_clock, cudaStream_t st) {
-  launch_chained(key_hist_kernel, dim3(c.CAPB, c.H), 256, c.hist_cols * 4, st, c, advance_clock >= 0 ? 1 : 0, stats_out,
+  launch_chained(key_hist_kernel, dim3(c.CAPB, c.H), 128, c.hist_cols * 4, st, c, advance_clock >= 0 ? 1 : 0, stats_out,
                                                                   advance_clock > 0 ? 1 : 0);
   return cudaGetLastError() == cudaSuccess ? 1 : FASTAR_ERR_CUDA;
 }
@@ -656,9 +688,9 @@ int launch_finalize_hist(const CacheView& c, fastar_update_stats* stats_out, int
 // S2 (query side)
 __global__ void __launch_bounds__(128) query_hist_kernel(const CacheView c, const uint32_t* __restrict__ codes, int nq, int block_q) {
   chain_wait();
-  extern __shared__ int hist[];
+  extern __shared__ __align__(16) int hist[];
   const int a = blockIdx.x, h = blockIdx.y;
-  for (int q = threadIdx.x; q < c.hist_cols; q += blockDim.x) hist[q] = 0;
+  for (int q = threadIdx.x; q < c.hist_cols / 4; q += blockDim.x) reinterpret_cast<int4*>(hist)[q] = make_int4(0, 0, 0, 0);
   __syncthreads();
   const int r0 = a * block_q, r1 = min(nq, r0 + block_q);
   const int nb = 1 << c.B;
@@ -668,7 +700,12 @@ __global__ void __launch_bounds__(128) query_hist_kernel(const CacheView c, cons
   }
   __syncthreads();
   __nv_bfloat16* dst = c.hq + (static_cast<int64_t>(h) * c.max_qb + a) * c.hist_cols;
-  for (int q = threadIdx.x; q < c.hist_cols; q += blockDim.x) dst[q] = __float2bfloat16(static_cast<float>(hist[q]));
+  for (int q = threadIdx.x; q < c.hist_cols / 8; q += blockDim.x) {
+    int v[8];
+#pragma unroll
+    for (int e = 0; e < 8; ++e) v[e] = hist[8 * q + e];
+    reinterpret_cast<uint4*>(dst)[q] = pack_counts<-1>(v);
+  }
 }
 int launch_query_hist(const CacheView& c, const uint32_t* codes, int nq, int block_q, cudaStream_t st) {
   const int nqb = (nq + block_q - 1) / block_q;
