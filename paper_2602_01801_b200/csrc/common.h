@@ -199,7 +199,16 @@ struct UpdateOut {         // the caller's [H][n] arrays (each may be null)
   float* sim;
   int32_t* dest;
 };
-int launch_convert_f32_to_bf16(const float* src, __nv_bfloat16* dst, int H, int n, int D, int64_t hs, int64_t ts, cudaStream_t st);
+struct ConvertArgs {
+  struct Tensor {
+    const float* src;
+    __nv_bfloat16* dst;
+    int64_t hs, ts;        // strides of src
+    int n;
+  } t[3];
+  int count;
+};
+int launch_convert_f32_to_bf16(const ConvertArgs& a, int H, int D, cudaStream_t st);
 int launch_prep_codes(const CacheView& c, const __nv_bfloat16* x, int n, int64_t hs, int64_t ts, uint32_t* code_out,
                       float* rnorm_out, cudaStream_t st);
 int launch_prep_update(const CacheView& c, const __nv_bfloat16* k_new, int n, int64_t hs, int64_t ts, cudaStream_t st);

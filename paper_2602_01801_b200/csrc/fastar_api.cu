@@ -258,18 +258,26 @@ __global__ void copy_rows3_kernel(const int32_t* __restrict__ src, int64_t src_h
     c->launches += r__;                                    \
   } while (0)
 
-// Returns a bf16 view of a caller tensor: the tensor itself (bf16) or its converted copy in stage[slot].
-int as_bf16(fastar_cache* c, const void* src, int rows, int64_t* hs, int64_t* ts, int slot, const __nv_bfloat16** out,
-            cudaStream_t st) {
-  if (c->desc.dtype == FASTAR_BF16) {
-    *out = static_cast<const __nv_bfloat16*>(src);
-    return FASTAR_OK;
+// A caller tensor and, behind as_bf16, its bf16 view: the tensor itself (bf16) or its converted copy in stage[slot].
+struct View {
+  const void* src;
+  int rows, slot;
+  int64_t hs, ts;
+  const __nv_bfloat16* p;
+};
+int as_bf16(fastar_cache* c, View* v, int count, cudaStream_t st) {
+  for (int i = 0; i < count; ++i) v[i].p = static_cast<const __nv_bfloat16*>(v[i].src);
+  if (c->desc.dtype == FASTAR_BF16) return FASTAR_OK;
+  ConvertArgs a{};
+  a.count = count;
+  for (int i = 0; i < count; ++i) {
+    if ((reinterpret_cast<uintptr_t>(v[i].src) & 15) || (v[i].hs & 3) || (v[i].ts & 3)) return FASTAR_ERR_INVALID_ARG;
+    a.t[i] = {static_cast<const float*>(v[i].src), c->v.stage[v[i].slot], v[i].hs, v[i].ts, v[i].rows};
+    v[i].p = c->v.stage[v[i].slot];
+    v[i].hs = static_cast<int64_t>(v[i].rows) * c->v.D;
+    v[i].ts = c->v.D;
   }
-  if ((reinterpret_cast<uintptr_t>(src) & 15) || (*hs & 3) || (*ts & 3)) return FASTAR_ERR_INVALID_ARG;
-  ACCK(FASTAR_K_CONVERT, launch_convert_f32_to_bf16(static_cast<const float*>(src), c->v.stage[slot], c->v.H, rows, c->v.D, *hs, *ts, st));
-  *out = c->v.stage[slot];
-  *hs = static_cast<int64_t>(rows) * c->v.D;
-  *ts = c->v.D;
+  ACCK(FASTAR_K_CONVERT, launch_convert_f32_to_bf16(a, c->v.H, c->v.D, st));
   return FASTAR_OK;
 }
 
@@ -525,18 +533,13 @@ static int update_impl(fastar_cache_t* c, const void* q_probe, const void* k_new
   DeviceGuard guard(c->desc.device);
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   const CacheView& v = c->v;
-  const __nv_bfloat16 *kb, *vb, *pb = nullptr;
-  int64_t khs = head_stride, kts = token_stride, vhs = head_stride, vts = token_stride, phs = head_stride, pts = token_stride;
-  int r = as_bf16(c, k_new, n, &khs, &kts, 0, &kb, st);
-  if (r != FASTAR_OK) return r;
   const bool v_converted = c->desc.dtype != FASTAR_BF16;      // the entry conversion already reads v_new
   if (v_ready && v_converted && cudaStreamWaitEvent(st, v_ready, 0) != cudaSuccess) return FASTAR_ERR_CUDA;
-  r = as_bf16(c, v_new, n, &vhs, &vts, 1, &vb, st);
+  View in[3] = {{k_new, n, 0, head_stride, token_stride, nullptr}, {v_new, n, 1, head_stride, token_stride, nullptr}, {q_probe, n, 2, head_stride, token_stride, nullptr}};
+  int r = as_bf16(c, in, q_probe ? 3 : 2, st);
   if (r != FASTAR_OK) return r;
-  if (q_probe) {
-    r = as_bf16(c, q_probe, n, &phs, &pts, 2, &pb, st);
-    if (r != FASTAR_OK) return r;
-  }
+  const __nv_bfloat16 *kb = in[0].p, *vb = in[1].p, *pb = in[2].p;
+  const int64_t khs = in[0].hs, kts = in[0].ts, phs = in[2].hs, pts = in[2].ts;      // K and V alike
   CUtensorMap tm_a;
   r = q_probe ? make_map(c, &tm_a, pb, v.D, n, v.H, static_cast<uint64_t>(pts) * 2, static_cast<uint64_t>(phs) * 2, 128)
               : make_map(c, &tm_a, kb, v.D, n, v.H, static_cast<uint64_t>(kts) * 2, static_cast<uint64_t>(khs) * 2, 128);
@@ -610,10 +613,11 @@ static int annsa_impl(fastar_cache_t* c, const void* q, const void* k_seg, const
   const bool dense = !sel_in && keep_blocks >= v.CAPB;
   const int keep = keep_blocks < v.CAPB ? keep_blocks : v.CAPB;
   if (!dense && !sel_in && v.CAPB > 2048) return FASTAR_ERR_UNSUPPORTED_SHAPE;
-  const __nv_bfloat16* qb;
-  int64_t qhs = head_stride, qts = token_stride;
-  int r = as_bf16(c, q, nq, &qhs, &qts, 2, &qb, st);
+  View in_q{q, nq, 2, head_stride, token_stride, nullptr};
+  int r = as_bf16(c, &in_q, 1, st);
   if (r != FASTAR_OK) return r;
+  const __nv_bfloat16* qb = in_q.p;
+  const int64_t qhs = in_q.hs, qts = in_q.ts;
   CUtensorMap tm_q;
   r = make_map(c, &tm_q, qb, v.D, nq, v.H, static_cast<uint64_t>(qts) * 2, static_cast<uint64_t>(qhs) * 2, 128);
   if (r != FASTAR_OK) return r;
@@ -673,12 +677,11 @@ static int annsa_impl(fastar_cache_t* c, const void* q, const void* k_seg, const
   }
   CUtensorMap tm_sk, tm_sv;
   if (k_seg) {
-    const __nv_bfloat16 *skb, *svb;
-    int64_t khs = seg_head_stride, kts = seg_token_stride, vhs = seg_head_stride, vts = seg_token_stride;
-    r = as_bf16(c, k_seg, ns, &khs, &kts, 0, &skb, st);          // the update's staging slots are free during an attention call
-    if (r == FASTAR_OK) r = as_bf16(c, v_seg, ns, &vhs, &vts, 1, &svb, st);
-    if (r == FASTAR_OK) r = make_map(c, &tm_sk, skb, v.D, ns, v.H, static_cast<uint64_t>(kts) * 2, static_cast<uint64_t>(khs) * 2, v.PT);
-    if (r == FASTAR_OK) r = make_map(c, &tm_sv, svb, v.D, ns, v.H, static_cast<uint64_t>(vts) * 2, static_cast<uint64_t>(vhs) * 2, v.PT);
+    // the update's staging slots are free during an attention call
+    View sg[2] = {{k_seg, ns, 0, seg_head_stride, seg_token_stride, nullptr}, {v_seg, ns, 1, seg_head_stride, seg_token_stride, nullptr}};
+    r = as_bf16(c, sg, 2, st);
+    if (r == FASTAR_OK) r = make_map(c, &tm_sk, sg[0].p, v.D, ns, v.H, static_cast<uint64_t>(sg[0].ts) * 2, static_cast<uint64_t>(sg[0].hs) * 2, v.PT);
+    if (r == FASTAR_OK) r = make_map(c, &tm_sv, sg[1].p, v.D, ns, v.H, static_cast<uint64_t>(sg[1].ts) * 2, static_cast<uint64_t>(sg[1].hs) * 2, v.PT);
     if (r != FASTAR_OK) return r;
     a.seg_tiles = (ns + v.PT - 1) / v.PT;
     a.seg_bias = v.seg_bias;
@@ -705,7 +708,10 @@ int fastar_annsa_prepare(fastar_cache_t* c, const void* q, int32_t nq, int64_t h
   int64_t qhs = head_stride, qts = token_stride;
   if (c->desc.dtype == FASTAR_FP32) {          // own staging buffer: an update or another attention call may be converting too
     if ((reinterpret_cast<uintptr_t>(q) & 15) || (qhs & 3) || (qts & 3)) return FASTAR_ERR_INVALID_ARG;
-    ACCK(FASTAR_K_CONVERT, launch_convert_f32_to_bf16(static_cast<const float*>(q), v.stage_prep, v.H, nq, v.D, qhs, qts, st));
+    ConvertArgs a{};
+    a.count = 1;
+    a.t[0] = {static_cast<const float*>(q), v.stage_prep, qhs, qts, nq};
+    ACCK(FASTAR_K_CONVERT, launch_convert_f32_to_bf16(a, v.H, v.D, st));
     qb = v.stage_prep;
     qhs = static_cast<int64_t>(nq) * v.D;
     qts = v.D;
@@ -747,13 +753,12 @@ int fastar_annca_attention(fastar_cache_t* c, const void* q, const void* k_promp
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   const CacheView& v = c->v;
   const int keep = keep_tokens < np ? keep_tokens : np;
-  const __nv_bfloat16 *qb, *kpb, *vpb;
-  int64_t qhs = head_stride, qts = token_stride, khs = prompt_head_stride, kts = prompt_token_stride, vhs = prompt_head_stride,
-          vts = prompt_token_stride;
-  int r = as_bf16(c, q, nq, &qhs, &qts, 5, &qb, st);   // own staging slot: may run beside an AnnSA call on another stream
-  if (r == FASTAR_OK) r = as_bf16(c, k_prompt, np, &khs, &kts, 3, &kpb, st);
-  if (r == FASTAR_OK) r = as_bf16(c, v_prompt, np, &vhs, &vts, 4, &vpb, st);
+  // own staging slots: may run beside an AnnSA call on another stream
+  View in[3] = {{q, nq, 5, head_stride, token_stride, nullptr}, {k_prompt, np, 3, prompt_head_stride, prompt_token_stride, nullptr}, {v_prompt, np, 4, prompt_head_stride, prompt_token_stride, nullptr}};
+  int r = as_bf16(c, in, 3, st);
   if (r != FASTAR_OK) return r;
+  const __nv_bfloat16 *qb = in[0].p, *kpb = in[1].p, *vpb = in[2].p;
+  const int64_t qhs = in[0].hs, qts = in[0].ts, khs = in[1].hs, kts = in[1].ts;      // K and V alike
   if ((reinterpret_cast<uintptr_t>(kpb) & 15) || (reinterpret_cast<uintptr_t>(vpb) & 15) || ((khs * 2) & 15) || ((kts * 2) & 15))
     return FASTAR_ERR_INVALID_ARG;
   CUtensorMap tm_q, tm_kp;
@@ -829,13 +834,11 @@ int fastar_annca_attention_lsh(fastar_cache_t* c, const void* q, const void* k_p
   DeviceGuard guard(c->desc.device);
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   const CacheView& v = c->v;
-  const __nv_bfloat16 *qb, *kpb, *vpb;
-  int64_t qhs = head_stride, qts = token_stride, khs = prompt_head_stride, kts = prompt_token_stride, vhs = prompt_head_stride,
-          vts = prompt_token_stride;
-  int r = as_bf16(c, q, nq, &qhs, &qts, 5, &qb, st);
-  if (r == FASTAR_OK) r = as_bf16(c, k_prompt, np, &khs, &kts, 3, &kpb, st);
-  if (r == FASTAR_OK) r = as_bf16(c, v_prompt, np, &vhs, &vts, 4, &vpb, st);
+  View in[3] = {{q, nq, 5, head_stride, token_stride, nullptr}, {k_prompt, np, 3, prompt_head_stride, prompt_token_stride, nullptr}, {v_prompt, np, 4, prompt_head_stride, prompt_token_stride, nullptr}};
+  int r = as_bf16(c, in, 3, st);
   if (r != FASTAR_OK) return r;
+  const __nv_bfloat16 *qb = in[0].p, *kpb = in[1].p, *vpb = in[2].p;
+  const int64_t qhs = in[0].hs, qts = in[0].ts, khs = in[1].hs, kts = in[1].ts;      // K and V alike
   if ((reinterpret_cast<uintptr_t>(kpb) & 15) || (reinterpret_cast<uintptr_t>(vpb) & 15) || ((khs * 2) & 15) || ((kts * 2) & 15))
     return FASTAR_ERR_INVALID_ARG;
   CUtensorMap tm_q;

@@ -60,31 +60,33 @@ __device__ __forceinline__ void bitonic_sort_smem(unsigned long long* keys, int 
 }
 
 // ---------------------------------------------------------------------------------------------
-// fp32 -> bf16 entry conversion (strided source, contiguous destination)
+// fp32 -> bf16 entry conversion (strided sources, contiguous destinations): up to three tensors of a call in one launch, one per
+// blockIdx.z (a small call is a chain of launches; one per tensor made six of a step's 21).
 // ---------------------------------------------------------------------------------------------
-__global__ void convert_kernel(const float* __restrict__ src, __nv_bfloat16* __restrict__ dst, int n, int D, int64_t hs,
-                               int64_t ts) {
+__global__ void convert_kernel(const ConvertArgs a, int D) {
   chain_wait();
+  const ConvertArgs::Tensor& x = a.t[blockIdx.z];
   const int h = blockIdx.y;
-  const int64_t per_head = static_cast<int64_t>(n) * D / 4;
+  const int64_t per_head = static_cast<int64_t>(x.n) * D / 4;
   for (int64_t q = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; q < per_head;
        q += static_cast<int64_t>(gridDim.x) * blockDim.x) {
     const int64_t e = q * 4;
     const int row = static_cast<int>(e / D), col = static_cast<int>(e % D);
-    const float4 v = *reinterpret_cast<const float4*>(src + h * hs + row * ts + col);
+    const float4 v = *reinterpret_cast<const float4*>(x.src + h * x.hs + row * x.ts + col);
     uint2 o;
     o.x = pack_bf16x2(v.x, v.y);
     o.y = pack_bf16x2(v.z, v.w);
-    *reinterpret_cast<uint2*>(dst + (static_cast<int64_t>(h) * n + row) * D + col) = o;
+    *reinterpret_cast<uint2*>(x.dst + (static_cast<int64_t>(h) * x.n + row) * D + col) = o;
   }
 }
-int launch_convert_f32_to_bf16(const float* src, __nv_bfloat16* dst, int H, int n, int D, int64_t hs, int64_t ts,
-                               cudaStream_t st) {
-  if (n <= 0) return 0;
-  const int64_t per_head = static_cast<int64_t>(n) * D / 4;
-  const int64_t want = (per_head + 255) / 256;
-  const int bx = static_cast<int>(want < 1024 ? want : 1024);
-  launch_chained(convert_kernel, dim3(bx, H), 256, 0, st, src, dst, n, D, hs, ts);
+int launch_convert_f32_to_bf16(const ConvertArgs& a, int H, int D, cudaStream_t st) {
+  int64_t want = 0;
+  for (int i = 0; i < a.count; ++i) {
+    const int64_t blocks = (static_cast<int64_t>(a.t[i].n) * D / 4 + 255) / 256;
+    want = blocks > want ? blocks : want;
+  }
+  if (want == 0) return 0;
+  launch_chained(convert_kernel, dim3(static_cast<int>(want < 1024 ? want : 1024), H, a.count), 256, 0, st, a, D);
   return cudaGetLastError() == cudaSuccess ? 1 : FASTAR_ERR_CUDA;
 }
 
