@@ -458,7 +458,9 @@ attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CU
         // A logit can make this warp raise the maximum only if it exceeds the last maximum that this warp knows by as much (maxima
         // only grow).  If none does, the hand-over goes on at once, before the maximum is even read: it still cannot change before
         // this sub-tile is through, because whoever raises it waits for P V of all sub-tiles before.
-        bool may = false;
+        // The first sub-tile's warp always goes the long way: it puts the maxima where the others read them, also those of a sub-tile
+        // without a live key (-inf; what lies there is an earlier item's).
+        bool may = t == 0;
 #pragma unroll
         for (int q = 0; q < 4; ++q) may |= mx[q] > m[q] + kLazy;
         may = __any_sync(0xffffffffu, may);
@@ -468,12 +470,12 @@ attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CU
         bool p_free = tg < kGroups || mbar_test_wait(bar_pv_done + 8 * g, (tg / kGroups - 1) & 1);
         const float4 seen = t > 0 ? lds4(max_s) : make_float4(-INFINITY, -INFINITY, -INFINITY, -INFINITY);
         const float cur[4] = {seen.x, seen.y, seen.z, seen.w};
-        bool change = false;
+        bool change = t == 0;
 #pragma unroll
         for (int q = 0; q < 4; ++q) change |= mx[q] > cur[q] + kLazy || cur[q] != m[q];
         if (__any_sync(0xffffffffu, change)) {
           float alpha[4];
-          bool raised = false;
+          bool raised = t == 0;
 #pragma unroll
           for (int q = 0; q < 4; ++q) {
             // the same for the four threads of a row

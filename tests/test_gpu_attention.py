@@ -49,3 +49,41 @@ def test_tiles_and_maxima(d, pt, nq, length, seg, rise):
         # probabilities and output rounded to 8 significant bits (2^-8 each), sums in fp32: 2^-7 of the largest value averaged
         assert np.abs(got - want).max() <= 2.0 ** -7 * np.abs(vv).max()
         assert np.linalg.norm(got - want) <= 1e-2 * np.linalg.norm(want)
+
+
+@pytest.mark.parametrize("d,pt,seg", [(128, 128, 0), (128, 64, 70), (64, 128, 200), (64, 64, 0)])
+def test_listed_blocks_without_a_live_slot(d, pt, seg):
+    """A caller's list may name blocks past a head's live slots: they add nothing, wherever in the list they stand, also for an empty
+    head and where nothing live is listed.  More items than two rounds of the CTAs, so that an item follows others on its CTA."""
+    import torch
+    from oracle import fastar_oracle as O
+    from paper_2602_01801_b200 import fastar
+    rng = np.random.default_rng(d + pt)
+    H, nq, cap, keep = 40, 10 * 128, 1024, 3
+    nb = cap // pt
+    lens = np.resize([cap, 0, 1, 65, pt, 3 * pt + 1, cap - 1], H)
+    q = rng.standard_normal((H, nq // 128, 128, d)) * rng.choice([1.0, 60.0], (H, nq // 128, 1, 1))      # maxima far apart between items
+    q = synth.round_bf16(q.reshape(H, nq, d).astype(np.float32))
+    k, v = (synth.round_bf16(rng.standard_normal((H, cap + seg, d)).astype(np.float32)) for _ in range(2))
+    count = rng.integers(1, 9, (H, cap)).astype(np.int32)
+    cache = fastar.Cache(H, d, cap, pt, rng.standard_normal((32, d)).astype(np.float32), max_tokens=nq)
+    cache.import_state(fastar.bf16_bits(k[:, :cap]), fastar.bf16_bits(v[:, :cap]), lens, count)
+    sel = np.stack([[rng.permutation(nb)[:keep] for _ in range(nq // 128)] for _ in range(H)]).astype(np.int32)
+    sel[:, ::2] = np.sort(sel[:, ::2], axis=2)[:, :, ::-1]                                # dead blocks first
+    sel[3, 1], sel[5, 2] = nb - 1, nb - 1                                                 # nothing but dead blocks
+    args = dict(sel_in=torch.from_numpy(sel).cuda(), nsel_in=torch.full((H,), keep, dtype=torch.int32, device="cuda"))
+    dq = fastar.to_device(q)
+    if seg:
+        out = cache.annsa_segment(dq, fastar.to_device(k[:, cap:]), fastar.to_device(v[:, cap:]), 128, keep, **args)["out"]
+    else:
+        out = cache.annsa(dq, 128, keep, **args)["out"]
+    assert cache.status() == 0
+    for h in range(H):
+        hc = O.HeadCache(cap, d)
+        L = int(lens[h])
+        hc.load(k[h, :L].astype(np.float64), v[h, :L].astype(np.float64), m=count[h, :L].astype(np.int64), now=1)
+        want = O.sparse_attention_with_segment(q[h], hc, sel[h], 128, pt, k[h, cap:], v[h, cap:])
+        got = out[h].float().cpu().numpy()
+        assert np.isfinite(got).all()
+        # as above: rounding of the probabilities and of the output
+        assert np.abs(got - want).max() <= 2.0 ** -7 * np.abs(v).max(), f"head {h}"
