@@ -18,10 +18,11 @@
 //   - P goes through tensor memory (with P in shared memory the MMAs of a tile saturate the read path), beside S and not over
 //     it, so that Q K^T of a group's next sub-tile runs while this one is in its exponentials;
 //   - that leaves room for one O, so all groups use one running maximum per row.  The four warps that own the same rows hand it
-//     on from sub-tile to sub-tile by named barriers.  It is raised lazily, only when a logit exceeds it by more than kLazy = 64
-//     (a factor 2^64: a product with bf16 operands and fp32 sums is as exact at any scale); who raises it rescales O (P V of all
-//     earlier sub-tiles done, that of this one waiting for its P).  A raise stops all groups for some 4 000 cycles: with a limit
-//     of 8 there were two to five per item, a fifth of a short item's time;
+//     on from sub-tile to sub-tile by named barriers.  It is raised lazily, only when a logit exceeds it by more than kLazy = 24
+//     (who raises it rescales O: P V of all earlier sub-tiles done, that of this one waiting for its P).  A raise stops all groups
+//     for some 4 000 cycles.  Kernel time with a limit of 8 / 12 / 16 / 24 / 64: 12 heads x 4 680 queries on 32 of 220 blocks 124 /
+//     144 / 142 / 110 / 110 us, the denoising step 234 / 248 / 240 / 217 / 218, 8 heads on all 16 384 keys 254 / 257 / 253 / 240 /
+//     240: keys of a query's own cluster stand some 13 (d = 128) above the first sub-tile's;
 //   - the row sums add up the probabilities as rounded to bf16, so that they cancel in a row that one key dominates;
 //   - the soft-max warps hold a sub-tile in the 16 x 256-bit fragment shape, four rows x 16 columns a thread: a thread reads 16
 //     biases, not 64, and a warp still has its rows to itself;
@@ -59,7 +60,9 @@ __device__ __forceinline__ float4 lds4(uint32_t addr) {
   return v;
 }
 
-constexpr float kLazy = 64.f;        // binary logarithm of what a probability may be before the running maximum is raised
+// The running maximum is raised when a logit exceeds it by more than kLazy (binary orders), and probabilities are taken relative to
+// kShift above it, so that none is above 2^8 whatever the limit: the sums of P V stay in range for values up to 2^119 / keys.
+constexpr float kLazy = 24.f, kShift = kLazy - 8.f;
 
 template <int D, int BKT>
 struct AttnSmem {
@@ -533,7 +536,7 @@ attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CU
         for (int hf = 0; hf < 2; ++hf) {
           float2 neg[2];
 #pragma unroll
-          for (int e = 0; e < 2; ++e) neg[e].x = neg[e].y = m[2 * hf + e] == -INFINITY ? 0.f : -m[2 * hf + e];
+          for (int e = 0; e < 2; ++e) neg[e].x = neg[e].y = m[2 * hf + e] == -INFINITY ? 0.f : -kShift - m[2 * hf + e];
           uint32_t p[16];
 #pragma unroll
           for (int k = 0; k < 8; ++k)

@@ -87,3 +87,39 @@ def test_listed_blocks_without_a_live_slot(d, pt, seg):
         assert np.isfinite(got).all()
         # as above: rounding of the probabilities and of the output
         assert np.abs(got - want).max() <= 2.0 ** -7 * np.abs(v).max(), f"head {h}"
+
+
+@pytest.mark.parametrize("pt", [64, 128])
+@pytest.mark.parametrize("d,magnitude", [(64, 110), (128, 110), (128, -100)])
+def test_range_of_the_values(d, pt, magnitude):
+    """Values near the ends of bf16's range under maxima that rise with every sub-tile of 64 keys, by 18 to 25 binary orders each time:
+    the output is a mean of the values and stays finite and as exact as for ordinary ones."""
+    import torch
+    from paper_2602_01801_b200 import fastar
+    rng = np.random.default_rng(d + pt)
+    n, steps = 768, 12
+    rise = np.cumsum(np.concatenate([[0.0], rng.uniform(18.0, 25.0, steps - 1)]))
+    unit = math.sqrt(d) / math.log2(math.e) / 8.0          # q = 8 e0: this much of a key's first component is one binary order
+    k = 0.01 * rng.standard_normal((1, n, d))
+    k[0, :, 0] = np.repeat(rise, 64) * unit
+    k, q = synth.round_bf16(k.astype(np.float32)), np.zeros((1, 130, d), np.float32)
+    q[:, :, 0], q[:, :, 1] = 8.0, synth.round_bf16(rng.standard_normal(130).astype(np.float32))
+    v = synth.round_bf16((rng.standard_normal((1, n, d)) * 2.0 ** magnitude).astype(np.float32))
+    cache = fastar.Cache(1, d, n, pt, rng.standard_normal((32, d)).astype(np.float32), max_tokens=n)
+    cache.import_state(fastar.bf16_bits(k), fastar.bf16_bits(v), np.array([n]))
+    for last in (n, 640, 192):                             # the segment entry as well: the last keys from there
+        kk, vv = k[:, :last], v[:, :last]
+        if last == n:
+            out = cache.annsa(fastar.to_device(q), 128, n // pt)["out"]
+        else:
+            cache.import_state(fastar.bf16_bits(k[:, :last - 128]), fastar.bf16_bits(v[:, :last - 128]), np.array([last - 128]))
+            out = cache.annsa_segment(fastar.to_device(q), fastar.to_device(k[:, last - 128:last]), fastar.to_device(v[:, last - 128:last]),
+                                      128, n // pt)["out"]
+        assert cache.status() == 0
+        s = q[0].astype(np.float64) @ kk[0].T.astype(np.float64) / math.sqrt(d)
+        p = np.exp(s - s.max(1, keepdims=True))
+        want = (p / p.sum(1, keepdims=True)) @ vv[0].astype(np.float64)
+        got = out[0].float().cpu().numpy().astype(np.float64)
+        assert np.isfinite(got).all()
+        assert np.abs(got - want).max() <= 2.0 ** -7 * np.abs(vv).max()
+        assert np.linalg.norm(got - want) <= 1e-2 * np.linalg.norm(want)
