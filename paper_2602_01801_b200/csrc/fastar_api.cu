@@ -33,7 +33,7 @@ struct fastar_cache {
   int force_sink_blocks = 0, force_recent_blocks = 0;    // AnnSA selector option (fastar_cache_set_forced_blocks)
   // queries whose codes and block histograms fastar_annsa_prepare has already produced (consumed by the next matching AnnSA call)
   struct { const void* q = nullptr; int32_t nq = 0, block_q = 0; int64_t hs = 0, ts = 0; bool valid = false; } prep;
-  bool rel_clear = true;     // the relevance maxima are zero (a reset and every prompt top-k leave them so)
+  bool rel_clear = true;     // AnnCA's relevance maxima are zero behind all work queued so far (create and every prompt top-k leave them so)
   cudaEvent_t ev_prep = nullptr;
   cudaStream_t side = nullptr, copy = nullptr;
   cudaEvent_t ev_fork = nullptr, ev_q = nullptr, ev_join = nullptr, ev_p = nullptr, ev_v = nullptr;
@@ -352,7 +352,9 @@ int fastar_cache_create(fastar_cache_t** out, const fastar_cache_desc* desc, con
     delete c;
     return FASTAR_ERR_CUDA;
   }
-  r = fastar_cache_reset(c, nullptr);
+  // AnnCA's own scratch: cleared here only, because an AnnCA call may run beside a reset or an import on another stream
+  r = cudaMemsetAsync(v.rel, 0, static_cast<size_t>(v.H) * v.max_frames * v.max_prompt * 4, nullptr) == cudaSuccess ? FASTAR_OK : FASTAR_ERR_CUDA;
+  if (r == FASTAR_OK) r = fastar_cache_reset(c, nullptr);
   if (r == FASTAR_OK && cudaStreamSynchronize(nullptr) != cudaSuccess) r = FASTAR_ERR_CUDA;
   if (r != FASTAR_OK) {
     delete c;
@@ -366,7 +368,6 @@ int fastar_cache_reset(fastar_cache_t* c, void* stream) {
   if (!c) return FASTAR_ERR_INVALID_ARG;
   DeviceGuard guard(c->desc.device);
   ACC(launch_reset(c->v, static_cast<cudaStream_t>(stream)));
-  c->rel_clear = true;
   return FASTAR_OK;
 }
 
@@ -785,7 +786,10 @@ int fastar_annca_attention(fastar_cache_t* c, const void* q, const void* k_promp
     a.sel_head_stride = static_cast<int64_t>(F) * keep_tokens;
   } else {
     // The maxima start at zero (0 is below the word of every float).  The top-k that ranks them puts the zeros back, so a memset is
-    // queued only after a call that failed between the two.
+    // queued only after a call that failed between the two (by each captured call from then on: a graph may never be launched).
+    cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+    if (!c->rel_clear && cudaStreamIsCapturing(st, &capture) != cudaSuccess) return FASTAR_ERR_CUDA;
+    const bool clear_after = c->rel_clear || capture == cudaStreamCaptureStatusNone;
     if (!c->rel_clear && cudaMemsetAsync(v.rel, 0, static_cast<size_t>(v.H) * v.max_frames * v.max_prompt * 4, st) != cudaSuccess)
       return FASTAR_ERR_CUDA;
     c->rel_clear = false;
@@ -807,7 +811,7 @@ int fastar_annca_attention(fastar_cache_t* c, const void* q, const void* k_promp
     }
     if (rel_out) ACC(launch_decode_rel(v, F, np, rel_scale, rel_out, st));
     ACCK(FASTAR_K_TOPK_PROMPT, launch_topk_prompt(v, F, np, keep, st));
-    c->rel_clear = true;
+    c->rel_clear = clear_after;
     a.sel = v.selp;
     a.sel_stride = v.max_prompt;
     a.sel_head_stride = static_cast<int64_t>(v.max_frames) * v.max_prompt;

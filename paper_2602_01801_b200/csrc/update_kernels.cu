@@ -932,7 +932,6 @@ int launch_reset(const CacheView& c, cudaStream_t st) {
   if (cudaMemsetAsync(c.pool_v, 0, pool, st) != cudaSuccess) return FASTAR_ERR_CUDA;
   if (cudaMemsetAsync(c.hk, 0, static_cast<size_t>(c.H) * c.CAPB * c.hist_cols * 2, st) != cudaSuccess) return FASTAR_ERR_CUDA;
   if (c.pool_k8 && cudaMemsetAsync(c.pool_k8, 0, static_cast<size_t>(c.pool_pages) * c.PT * 128, st) != cudaSuccess) return FASTAR_ERR_CUDA;
-  if (cudaMemsetAsync(c.rel, 0, static_cast<size_t>(c.H) * c.max_frames * c.max_prompt * 4, st) != cudaSuccess) return FASTAR_ERR_CUDA;
   reset_meta_kernel<<<296, 256, 0, st>>>(c);
   return cudaGetLastError() == cudaSuccess ? 1 : FASTAR_ERR_CUDA;
 }

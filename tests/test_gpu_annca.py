@@ -31,3 +31,37 @@ def test_relevance_selection_attention(heads, d, nq, frame_len, prompt, keep, bi
             P.check_prompt_selection(Q[h], Kp[h], frame_len, keep, sel, r["rel"][h].cpu().numpy(),
                                      codes=(codes["q"][h][:, :d], codes["prompt"][h][:, :d]) if bits == 8 else None)
             P.check_attention(out[h], O.annca(Q[h], Kp[h], Vp[h], frame_len, keep, sel=sel)["out"], f"AnnCA head {h}")
+
+
+def test_reset_on_another_stream_leaves_the_relevance_alone():
+    """AnnCA uses its own scratch and reads no cache state: a reset (or an import, which begins with one) that runs meanwhile on another
+    stream does not change what it selects."""
+    import torch
+
+    from paper_2602_01801_b200 import fastar
+
+    g = torch.Generator(device="cuda").manual_seed(3)
+    H, d, nq, prompt, keep = 8, 128, 2048, 256, 8
+    q, kp, vp = (torch.randn(H, n, d, generator=g, device="cuda").bfloat16() for n in (nq, prompt, prompt))
+    cache = fastar.Cache(H, d, 256, 128, np.random.default_rng(3).standard_normal((32, d)).astype(np.float32), max_tokens=nq,
+                         max_prompt_tokens=prompt, max_frames=4)
+    def call():
+        return cache.annca(q, kp, vp, nq // 4, keep, debug=True)["sel"]
+
+    want = call()
+    main, side, gate = torch.cuda.current_stream(), torch.cuda.Stream(), torch.cuda.Stream()
+    torch.cuda.synchronize()
+    with torch.cuda.stream(gate):                          # both streams find their work queued when they start
+        torch.cuda._sleep(40_000_000)
+        start = gate.record_event()
+    main.wait_event(start)
+    side.wait_event(start)
+    got = []
+    for _ in range(60):
+        with torch.cuda.stream(side):
+            cache.reset()
+            cache.reset()
+        got.append(call())
+    torch.cuda.synchronize()
+    assert cache.status() == fastar.OK
+    assert all(torch.equal(x, want) for x in got)
