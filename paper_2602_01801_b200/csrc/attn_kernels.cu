@@ -4,7 +4,7 @@
 //            to the key blocks listed in `sel`; one key block = one cache page = one TMA box, looked
 //            up through the page table.
 //   gather : AnnCA's attention over the kept prompt tokens of the query's frame; rows of K_p / V_p
-//            are gathered by index with 128-bit loads into the same swizzled tile layout.
+//            are gathered by index with 16-byte copies into the same swizzled tile layout.
 //
 // One CTA per SM takes (head, query block) items in turn, 128 query rows each (TMEM lanes).  The key tiles are cut into sub-tiles of 64
 // keys, which are dealt in turn to four soft-max groups of four warps (index t, group t % 4): while one is in its exponentials the
@@ -197,39 +197,6 @@ attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CU
     return (a.sel ? __shfl_sync(0xffffffffu, a.nsel[h], 0) : (__shfl_sync(0xffffffffu, c.len[h], 0) + BKT - 1) / BKT) + (SEG ? a.seg_tiles : 0);
   };
 
-  // Gather mode with a single key tile: all threads fetch the kept rows of K_p and V_p at once, instead of leaving
-  // 2 x BKT x D x 2 bytes of 16-byte gathers to one warp.
-  bool prefilled = false;
-  if (GATHER) {
-    const AttnItem w = item_of(blockIdx.x);
-    if (w.nt == 1) {
-      constexpr int CPR = D / 8;                         // 16-byte chunks per row
-      const __nv_bfloat16* kp_h = a.kp + static_cast<int64_t>(w.h) * a.p_head_stride;
-      const __nv_bfloat16* vp_h = a.vp + static_cast<int64_t>(w.h) * a.p_head_stride;
-      for (int q = threadIdx.x; q < 2 * BKT * CPR; q += blockDim.x) {
-        const int which = q / (BKT * CPR), qq = q % (BKT * CPR);
-        const int i = qq / CPR, ch = qq % CPR;
-        uint4 val = make_uint4(0, 0, 0, 0);
-        if (i < w.keep_n) {
-          const int idx = FASTAR_IDX(w.list[i], a.np, c.status);
-          val = *reinterpret_cast<const uint4*>((which ? vp_h : kp_h) + static_cast<int64_t>(idx) * a.p_token_stride + ch * 8);
-        }
-        const uint32_t off = which * RK * SM::kv_bytes + (ch >> 3) * (BKT * 128) + i * 128 + (((ch & 7) ^ (i & 7)) << 4);
-        asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(ring_s + off), "r"(val.x), "r"(val.y), "r"(val.z), "r"(val.w)
-                     : "memory");
-      }
-      for (int i = threadIdx.x; i < BKT; i += blockDim.x)
-        asm volatile("st.shared.f32 [%0], %1;" ::"r"(bias_s + 4 * i), "f"((i < w.keep_n) ? 0.f : -INFINITY) : "memory");
-      fence_proxy_async_smem();
-      __syncthreads();
-      if (threadIdx.x == 0) {
-        mbar_arrive(bar_r_full);                         // K0 -> K stage 0
-        mbar_arrive(bar_r_full + 8 * RK);                // V0 -> V stage 0
-      }
-      prefilled = true;
-    }
-  }
-
   // Everything is counted through the items of a CTA: tile0 key tiles, tile0 * SUB sub-tiles before.  Key tile n is in K stage n % RK
   // and V stage RK + n % RV.
 
@@ -267,61 +234,72 @@ attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CU
             page_n = -1;
           }
         };
+        auto announce = [&](uint32_t stage) {     // gather mode: this warp's copies into the stage have landed
+          fence_proxy_async_smem();
+          __syncwarp();
+          if (lane == 0) mbar_arrive(bar_r_full + 8 * stage);
+        };
+        auto token = [&](int i) { return GATHER && i < w.keep_n ? FASTAR_IDX(w.list[i], a.np, c.status) : 0; };
+        int next = token(lane);                  // gather mode: 32 kept tokens, one per lane
         fetch(0);
         for (int j = 0; j < nt; ++j) {
           if ((j & 31) == 0) {
             blk = blk_n; page = page_n;
             fetch(j + 32);
           }
-          const int b = __shfl_sync(0xffffffffu, blk, j & 31), p = __shfl_sync(0xffffffffu, page, j & 31);
-          if (!(GATHER && prefilled)) {
-            ok = mbar_wait_warp<kIssueWaitHintNs>(bar_r_empty + 8 * st, empty_phase, abort_flag, c.status);
-            if (!ok) break;
-            const uint32_t dst = ring_s + st * SM::kv_bytes;
-            if (!GATHER) {
-              if (lane == 0) {
-                const bool seg = SEG && p < 0;   // rows past the segment's end arrive as zeros and carry a -inf bias
-                const CUtensorMap* tm = seg ? (is_k ? &tm_sk : &tm_sv) : (is_k ? &tm_k : &tm_v);
-                mbar_arrive_expect_tx(bar_r_full + 8 * st, SM::kv_bytes + (is_k ? BKT * 4 : 0));
-                for (int kc = 0; kc < D / 64; ++kc)
-                  tma_load_3d(dst + kc * BKT * 128, tm, bar_r_full + 8 * st, kc * 64, seg ? b * BKT : 0, seg ? w.h : p);
-                if (is_k) {
-                  const float* bias_src = seg ? a.seg_bias + static_cast<int64_t>(b) * BKT : c.log2m + static_cast<int64_t>(w.h) * c.CAP + b * BKT;
-                  bulk_load_1d(bias_s + (copied % NB) * BKT * 4, bias_src, BKT * 4, bar_r_full + 8 * st);
-                }
+          const int b = GATHER ? 0 : __shfl_sync(0xffffffffu, blk, j & 31), p = GATHER ? 0 : __shfl_sync(0xffffffffu, page, j & 31);
+          ok = mbar_wait_warp<kIssueWaitHintNs>(bar_r_empty + 8 * st, empty_phase, abort_flag, c.status);
+          if (!ok) break;
+          const uint32_t dst = ring_s + st * SM::kv_bytes;
+          if (!GATHER) {
+            if (lane == 0) {
+              const bool seg = SEG && p < 0;   // rows past the segment's end arrive as zeros and carry a -inf bias
+              const CUtensorMap* tm = seg ? (is_k ? &tm_sk : &tm_sv) : (is_k ? &tm_k : &tm_v);
+              mbar_arrive_expect_tx(bar_r_full + 8 * st, SM::kv_bytes + (is_k ? BKT * 4 : 0));
+              for (int kc = 0; kc < D / 64; ++kc)
+                tma_load_3d(dst + kc * BKT * 128, tm, bar_r_full + 8 * st, kc * 64, seg ? b * BKT : 0, seg ? w.h : p);
+              if (is_k) {
+                const float* bias_src = seg ? a.seg_bias + static_cast<int64_t>(b) * BKT : c.log2m + static_cast<int64_t>(w.h) * c.CAP + b * BKT;
+                bulk_load_1d(bias_s + (copied % NB) * BKT * 4, bias_src, BKT * 4, bar_r_full + 8 * st);
               }
-            } else {
-              // gather rows of K_p / V_p by index: 16-byte chunks, written at their swizzled position
-              constexpr int CPR = D / 8;                       // 16-byte chunks per row
-              const __nv_bfloat16* src_h = (is_k ? a.kp : a.vp) + static_cast<int64_t>(w.h) * a.p_head_stride;
+            }
+          } else {
+            // Rows of K_p / V_p by index, as asynchronous 16-byte copies to their swizzled position.  A tile is announced when the
+            // copies of the next one are under way (it needs a stage that the tile before the announced one has left).
+            constexpr int CPR = D / 8, RPI = 32 / CPR;       // 16-byte chunks per row, rows per instruction
+            const int ch = lane % CPR;
+            const __nv_bfloat16* src = (is_k ? a.kp : a.vp) + static_cast<int64_t>(w.h) * a.p_head_stride + ch * 8;
 #pragma unroll 1
-              for (int q = lane; q < BKT * CPR; q += 32) {
-                const int i = q / CPR, ch = q % CPR;
-                const int tok = j * BKT + i;
-                uint4 val = make_uint4(0, 0, 0, 0);
-                if (tok < w.keep_n) {
-                  const int idx = FASTAR_IDX(w.list[tok], a.np, c.status);
-                  val = *reinterpret_cast<const uint4*>(src_h + static_cast<int64_t>(idx) * a.p_token_stride + ch * 8);
-                }
-                const uint32_t off = (ch >> 3) * (BKT * 128) + i * 128 + (((ch & 7) ^ (i & 7)) << 4);
-                asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(dst + off), "r"(val.x), "r"(val.y), "r"(val.z),
-                             "r"(val.w)
-                             : "memory");
+            for (int i0 = 0; i0 < BKT; i0 += 32) {
+              const int idx = next;
+              next = token(j * BKT + i0 + 32 + lane);
+#pragma unroll 4
+              for (int r = 0; r < 32; r += RPI) {
+                const int i = i0 + r + lane / CPR;
+                const int tok = __shfl_sync(0xffffffffu, idx, i & 31);
+                cp_async16(dst + (ch >> 3) * (BKT * 128) + i * 128 + (((ch & 7) ^ (i & 7)) << 4),
+                           src + static_cast<int64_t>(tok) * a.p_token_stride, j * BKT + i < w.keep_n);
               }
-              if (is_k)
-                for (int i = lane; i < BKT; i += 32)
-                  asm volatile("st.shared.f32 [%0], %1;" ::"r"(bias_s + ((j % NB) * BKT + i) * 4), "f"((j * BKT + i < w.keep_n) ? 0.f : -INFINITY)
-                               : "memory");
-              fence_proxy_async_smem();
-              __syncwarp();
-              if (lane == 0) mbar_arrive(bar_r_full + 8 * st);
+            }
+            if (is_k)
+              for (int i = lane; i < BKT; i += 32)
+                asm volatile("st.shared.f32 [%0], %1;" ::"r"(bias_s + ((j % NB) * BKT + i) * 4), "f"((j * BKT + i < w.keep_n) ? 0.f : -INFINITY)
+                             : "memory");
+            asm volatile("cp.async.commit_group;" ::: "memory");
+            if (j > 0) asm volatile("cp.async.wait_group 1;" ::: "memory");
+            if (j > 0) announce(st == first ? end - 1 : st - 1);
+            if (j + 1 == nt) {
+              asm volatile("cp.async.wait_all;" ::: "memory");
+              announce(st);
             }
           }
           ++copied;
           if (++st == end) { st = first; empty_phase ^= 1; }
         }
+        if (GATHER) break;                       // one item
       }
       // what is still in flight must land before the CTA may exit (normally the MMAs have consumed all of it)
+      if (GATHER) asm volatile("cp.async.wait_all;" ::: "memory");
       if (lane == 0) {
         if (n_q > 0) mbar_wait(bar_q_full, (n_q - 1) & 1, abort_flag, c.status);
         if (!GATHER)
@@ -638,7 +616,9 @@ static int launch_attn(const CUtensorMap& tq, const CUtensorMap& tk, const CUten
   auto kern = attn_kernel<D, BKT, GATHER, SEG>;
   const int cfg = ensure_dynamic_smem(reinterpret_cast<const void*>(kern), SM::total);
   if (cfg != FASTAR_OK) return cfg;
-  // one CTA per SM takes the items in turn; gather mode (more than 64 kept prompt tokens) fetches its rows per CTA: one item each
+  // One CTA per SM takes the items in turn; gather mode (more than 64 kept prompt tokens, or up to that many by the bucket rule) has
+  // one item per CTA.  Its rows come in by asynchronous copies, a tile ahead: 12 heads x 4680 queries, 512 kept 385 -> 94 us for the
+  // whole call (loads and stores through registers: 385; with 64 registers a thread 286), 40 x 10800 2420 -> 479, 128 kept 71 -> 64.
   int dev = 0, sm_count = 148;
   if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sm_count, cudaDevAttrMultiProcessorCount, dev);
   launch_chained(kern, GATHER ? items : min(items, sm_count), kAttnThreads, SM::total, st, tq, tk, tv, tsk, tsv, c, a);

@@ -30,12 +30,6 @@ struct Cfg {
   static constexpr int total = bar_off + 128;
 };
 
-// 16 bytes global -> shared, or zeros (valid = 0)
-__device__ __forceinline__ void cp_async16(uint32_t dst, const void* src, bool valid) {
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(reinterpret_cast<uint64_t>(src)), "r"(valid ? 16 : 0)
-               : "memory");
-}
-
 template <int D>
 __global__ void __launch_bounds__(kThreads, 2)
 prompt_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const CacheView c, const AttnArgs a, int tiles_per_frame, int tiles_per_head,

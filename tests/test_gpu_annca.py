@@ -12,7 +12,9 @@ pytestmark = pytest.mark.gpu
 
 @pytest.mark.parametrize("heads,d,nq,frame_len,prompt,keep,bits", [
     (1, 64, 1, 1, 1, 1, 16), (2, 128, 129, 129, 129, 5, 16), (3, 128, 300, 37, 513, 64, 16), (1, 64, 640, 64, 1024, 65, 16),
-    (2, 128, 64, 1, 200, 3, 16), (40, 64, 520, 260, 32, 8, 16), (2, 128, 300, 100, 130, 129, 8), (1, 64, 257, 256, 400, 64, 8)])
+    (2, 128, 64, 1, 200, 3, 16), (40, 64, 520, 260, 32, 8, 16), (2, 128, 300, 100, 130, 129, 8), (1, 64, 257, 256, 400, 64, 8),
+    # gathered key tiles: two, a remainder of one token, more than the rings have stages
+    (3, 128, 200, 200, 512, 256, 16), (2, 128, 300, 150, 1024, 1000, 16), (2, 64, 129, 129, 700, 641, 16)])
 def test_relevance_selection_attention(heads, d, nq, frame_len, prompt, keep, bits):
     from paper_2602_01801_b200 import fastar
 
