@@ -18,7 +18,7 @@
 //   - P goes through tensor memory (with P in shared memory the MMAs of a tile saturate the read path), beside S and not over
 //     it, so that Q K^T of a group's next sub-tile runs while this one is in its exponentials;
 //   - that leaves room for one O, so all groups use one running maximum per row.  The four warps that own the same rows hand it
-//     on from sub-tile to sub-tile by named barriers.  It is raised lazily, only when a logit exceeds it by more than kLazy = 24
+//     on from sub-tile to sub-tile by named barriers.  It is raised lazily, only when a logit exceeds it by more than 24 binary orders
 //     (who raises it rescales O: P V of all earlier sub-tiles done, that of this one waiting for its P).  A raise stops all groups
 //     for some 4 000 cycles.  Kernel time with a limit of 8 / 12 / 16 / 24 / 64: 12 heads x 4 680 queries on 32 of 220 blocks 124 /
 //     144 / 142 / 110 / 110 us, the denoising step 234 / 248 / 240 / 217 / 218, 8 heads on all 16 384 keys 254 / 257 / 253 / 240 /
@@ -60,9 +60,10 @@ __device__ __forceinline__ float4 lds4(uint32_t addr) {
   return v;
 }
 
-// The running maximum is raised when a logit exceeds it by more than kLazy (binary orders), and probabilities are taken relative to
-// kShift above it, so that none is above 2^8 whatever the limit: the sums of P V stay in range for values up to 2^119 / keys.
-constexpr float kLazy = 24.f, kShift = kLazy - 8.f;
+// Probabilities are taken relative to kHead binary orders above the running maximum and the maximum is raised when one would exceed
+// 2^kTop, that is when a logit exceeds it by more than kHead + kTop = 24.  So none is above 2^8, and the sums of P V stay in range
+// for values up to 2^119 / keys.  What the code calls the maximum, and the warps hand on, is that reference.
+constexpr float kHead = 16.f, kTop = 8.f;
 
 template <int D, int BKT>
 struct AttnSmem {
@@ -443,7 +444,7 @@ attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CU
         // without a live key (-inf; what lies there is an earlier item's).
         bool may = t == 0;
 #pragma unroll
-        for (int q = 0; q < 4; ++q) may |= mx[q] > m[q] + kLazy;
+        for (int q = 0; q < 4; ++q) may |= mx[q] > m[q] + kTop;
         may = __any_sync(0xffffffffu, may);
         if (t > 0) named_barrier_sync(heard, 64);
         if (!may && t + 1 < ns) named_barrier_arrive(told, 64);
@@ -453,7 +454,7 @@ attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CU
         const float cur[4] = {seen.x, seen.y, seen.z, seen.w};
         bool change = t == 0;
 #pragma unroll
-        for (int q = 0; q < 4; ++q) change |= mx[q] > cur[q] + kLazy || cur[q] != m[q];
+        for (int q = 0; q < 4; ++q) change |= mx[q] > cur[q] + kTop || cur[q] != m[q];
         if (__any_sync(0xffffffffu, change)) {
           float alpha[4];
           bool raised = t == 0;
@@ -464,8 +465,8 @@ attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CU
             mx[q] = fmaxf(mx[q], __shfl_xor_sync(0xffffffffu, mx[q], 2));
             float top = cur[q];
             alpha[q] = 1.f;
-            if (mx[q] > cur[q] + kLazy) {
-              top = mx[q];
+            if (mx[q] > cur[q] + kTop) {
+              top = mx[q] + kHead;
               alpha[q] = cur[q] == -INFINITY ? 0.f : fast_exp2(cur[q] - top);
               raised = true;
             }
@@ -514,7 +515,7 @@ attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CU
         for (int hf = 0; hf < 2; ++hf) {
           float2 neg[2];
 #pragma unroll
-          for (int e = 0; e < 2; ++e) neg[e].x = neg[e].y = m[2 * hf + e] == -INFINITY ? 0.f : -kShift - m[2 * hf + e];
+          for (int e = 0; e < 2; ++e) neg[e].x = neg[e].y = m[2 * hf + e] == -INFINITY ? 0.f : -m[2 * hf + e];
           uint32_t p[16];
 #pragma unroll
           for (int k = 0; k < 8; ++k)
