@@ -223,7 +223,11 @@ static int launch_prep_generic(const CacheView& c, const __nv_bfloat16* x, int n
                                float* rnorm_out, int64_t out_stride, cudaStream_t st, uint4* zero = nullptr, int64_t zero16 = 0) {
   if (n <= 0) return 0;
   const int groups = ((n + 15) / 16) * c.H;                      // 16 rows per warp pass
-  const dim3 grid(max(1, min((groups + 7) / 8, 2 * 148)));
+  // CTAs for the rows (eight warps of 16 a pass) or for the zeros (32 KB each), whichever needs more: a few tokens against many heads
+  // with long caches leave far more to clear than to hash (40 heads x 65536 slots, 1 to 16 tokens: an update of 81 us with CTAs for
+  // the rows only, 50 with these).
+  const int64_t want = max(static_cast<int64_t>(groups + 7) / 8, (zero16 + 2047) / 2048);
+  const dim3 grid(static_cast<unsigned>(max(static_cast<int64_t>(1), min(want, static_cast<int64_t>(2 * 148)))));
   if (c.D == 128) launch_chained(prep_kernel<128>, grid, 256, 0, st, x, c.H, n, hs, ts, c.lsh, c.T, c.B, code_out, rnorm_out, out_stride, zero, zero16);
   else launch_chained(prep_kernel<64>, grid, 256, 0, st, x, c.H, n, hs, ts, c.lsh, c.T, c.B, code_out, rnorm_out, out_stride, zero, zero16);
   return cudaGetLastError() == cudaSuccess ? 1 : FASTAR_ERR_CUDA;

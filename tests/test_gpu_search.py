@@ -58,3 +58,25 @@ def test_search_edges(d, pt, n, lengths, probe):
         assert (score[rows, match] >= score[rows, best] - 2 * slack)[got].all()
         far = np.abs(cos[rows, best] - tau) > 1e-4
         assert np.array_equal(got[far & clear], (cos[rows, best] >= tau)[far & clear])
+
+
+@pytest.mark.parametrize("heads,n,cap", [(1, 1, 128), (1, 1, 32768), (5, 17, 16384), (3, 40, 4224)])
+def test_few_tokens_against_a_long_cache(heads, n, cap):
+    """The words that an update accumulates into are cleared over the whole cache, however few tokens it has: the same tokens are
+    merged again and again into slots from the first to the last of every head, once each time."""
+    from paper_2602_01801_b200 import fastar
+    rng = np.random.default_rng(cap + n)
+    keys = synth.round_bf16(rng.standard_normal((heads, cap, 64)).astype(np.float32))
+    bits = fastar.bf16_bits(keys)
+    cache = fastar.Cache(heads, 64, cap, 64, rng.standard_normal((32, 64)).astype(np.float32), max_tokens=n)
+    cache.import_state(bits, bits, np.full(heads, cap))
+    slots = np.linspace(0, cap - 1, n).astype(int) if n > 1 else np.array([cap - 1])
+    for rep in range(1, 4):
+        new = fastar.to_device(np.ascontiguousarray(keys[:, slots]))
+        res = cache.update(new, new, n, 0.999)
+        assert cache.status() == 0
+        assert (res["match"].cpu().numpy() == slots).all()
+        assert (res["stats"].cpu().numpy()[:, :3] == [n, n, 0]).all()
+        want = np.ones((heads, cap), np.int32)
+        want[:, slots] += rep
+        assert np.array_equal(cache.export_state(kv=False)["count"], want)
