@@ -57,8 +57,13 @@ __device__ __forceinline__ void store_code_part(const CacheView& c, int page, in
   else *reinterpret_cast<uint4*>(dst + sl * 16) = v;
 }
 
+// Two warps a CTA: a CTA keeps its place until its largest group is through, and with eight warps the others wait for that one (20 KB
+// of staging a CTA besides).  Kernel time with 256 / 128 / 64 threads: 40 heads x 10800 tokens 188 / 172 / 160 us, 12 x 4680 25.7 /
+// 24.2 / 23.4, with the 8-bit search 30.5 / 29.3 / 28.3, at capacity 26.0 / 25.3 / 24.3; small calls the same.
+constexpr int kCommitThreads = 64;
+
 template <int D, bool MEANK>
-__global__ void __launch_bounds__(256) commit_kernel(const CacheView c, const __nv_bfloat16* __restrict__ k_new,
+__global__ void __launch_bounds__(kCommitThreads) commit_kernel(const CacheView c, const __nv_bfloat16* __restrict__ k_new,
                                                      const __nv_bfloat16* __restrict__ v_new, int n, int frame_len, int64_t hs,
                                                      int64_t ts) {
   chain_wait();
@@ -71,8 +76,8 @@ __global__ void __launch_bounds__(256) commit_kernel(const CacheView c, const __
   const int w = (blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)) * GPW + sub;
   // groups of several members: their tokens in ascending order, and the rows on their way (every lane its own 16 bytes)
   constexpr int kHeld = 4, kRows = MEANK ? 2 : 4;
-  __shared__ int sorted_s[256 / LPR][kHeld * LPR];
-  __shared__ uint4 rows_s[MEANK ? 2 : 1][kRows][256];
+  __shared__ int sorted_s[kCommitThreads / LPR][kHeld * LPR];
+  __shared__ uint4 rows_s[MEANK ? 2 : 1][kRows][kCommitThreads];
   if (w >= n) return;                   // groups + unmatched tokens <= n
   const int64_t tb = static_cast<int64_t>(h) * c.max_tokens;
   const int64_t sb = static_cast<int64_t>(h) * c.CAP;
@@ -122,7 +127,7 @@ __global__ void __launch_bounds__(256) commit_kernel(const CacheView c, const __
     } else if (g <= kHeld * LPR) {
       // Members in ascending token order (the scatter left them unordered).  A member's place is the number of members below it;
       // with the order known, four rows at a time come in by asynchronous copies, so a member costs a quarter of a load latency
-      // and no search, and no registers while it is under way: occupancy is what the common group of one needs.  12 x 4680 tokens:
+      // and no search, and no registers while it is under way: occupancy is what the common group of one needs.  In CTAs of 256, 12 x 4680 tokens:
       // 8-bit search (groups of up to 50) 60 -> 27 us, bf16 search (two thirds of the tokens alone) 21.4 -> 21.7; 12 x 1560 by the
       // probe 20.6 -> 10.4.  (Four rows at a time in registers: 31 us, but 30 with the bf16 search; eight staged: 24.5 and 23.0.)
       int* order = sorted_s[threadIdx.x / LPR];
@@ -349,12 +354,12 @@ __global__ void __launch_bounds__(256) commit_kernel(const CacheView c, const __
 int launch_commit(const CacheView& c, const __nv_bfloat16* k_new, const __nv_bfloat16* v_new, int n, int frame_len, int64_t hs,
                   int64_t ts, cudaStream_t st) {
   if (n <= 0) return 0;
-  const int items_per_cta = 8 * (32 / (c.D / 8));
+  const int items_per_cta = kCommitThreads / (c.D / 8);
   const dim3 grid((n + items_per_cta - 1) / items_per_cta, c.H);
-  if (c.D == 128 && !c.rep_mean) launch_chained(commit_kernel<128, false>, grid, 256, 0, st, c, k_new, v_new, n, frame_len, hs, ts);
-  else if (c.D == 128) launch_chained(commit_kernel<128, true>, grid, 256, 0, st, c, k_new, v_new, n, frame_len, hs, ts);
-  else if (!c.rep_mean) launch_chained(commit_kernel<64, false>, grid, 256, 0, st, c, k_new, v_new, n, frame_len, hs, ts);
-  else launch_chained(commit_kernel<64, true>, grid, 256, 0, st, c, k_new, v_new, n, frame_len, hs, ts);
+  if (c.D == 128 && !c.rep_mean) launch_chained(commit_kernel<128, false>, grid, kCommitThreads, 0, st, c, k_new, v_new, n, frame_len, hs, ts);
+  else if (c.D == 128) launch_chained(commit_kernel<128, true>, grid, kCommitThreads, 0, st, c, k_new, v_new, n, frame_len, hs, ts);
+  else if (!c.rep_mean) launch_chained(commit_kernel<64, false>, grid, kCommitThreads, 0, st, c, k_new, v_new, n, frame_len, hs, ts);
+  else launch_chained(commit_kernel<64, true>, grid, kCommitThreads, 0, st, c, k_new, v_new, n, frame_len, hs, ts);
   return cudaGetLastError() == cudaSuccess ? 1 : FASTAR_ERR_CUDA;
 }
 
