@@ -745,6 +745,7 @@ int fastar_annca_attention(fastar_cache_t* c, const void* q, const void* k_promp
                            int64_t prompt_head_stride, int64_t prompt_token_stride, int32_t* sel_out, float* rel_out,
                            const int32_t* sel_in, void* stream) {
   if (!c || !q || !k_prompt || !v_prompt || !out || nq < 1 || frame_len < 1 || np < 1 || keep_tokens < 1) return FASTAR_ERR_INVALID_ARG;
+  if (frame_len > nq) frame_len = nq;        // one frame, however long: the tile counts stay small
   const int F = (nq + frame_len - 1) / frame_len;
   if (nq > c->v.max_tokens || np > c->v.max_prompt || F > c->v.max_frames) return FASTAR_ERR_UNSUPPORTED_SHAPE;
   if (token_stride < c->v.D || prompt_token_stride < c->v.D) return FASTAR_ERR_INVALID_ARG;
@@ -830,6 +831,7 @@ int fastar_annca_attention_lsh(fastar_cache_t* c, const void* q, const void* k_p
                                int64_t prompt_token_stride, int32_t* sel_out, int32_t* nsel_out, uint32_t* qcode_out,
                                uint32_t* pcode_out, void* stream) {
   if (!c || !q || !k_prompt || !v_prompt || !out || nq < 1 || frame_len < 1 || np < 1) return FASTAR_ERR_INVALID_ARG;
+  if (frame_len > nq) frame_len = nq;        // one frame, however long: the tile counts stay small
   const int F = (nq + frame_len - 1) / frame_len;
   if (nq > c->v.max_tokens || np > c->v.max_prompt || F > c->v.max_frames) return FASTAR_ERR_UNSUPPORTED_SHAPE;
   if (token_stride < c->v.D || prompt_token_stride < c->v.D) return FASTAR_ERR_INVALID_ARG;

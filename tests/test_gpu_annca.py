@@ -67,3 +67,25 @@ def test_reset_on_another_stream_leaves_the_relevance_alone():
     torch.cuda.synchronize()
     assert cache.status() == fastar.OK
     assert all(torch.equal(x, want) for x in got)
+
+
+@pytest.mark.parametrize("d,keep", [(128, 70), (64, 9)])
+def test_frame_longer_than_the_call(d, keep):
+    """A frame length beyond the queries means one frame, up to the largest integer."""
+    import torch
+
+    from paper_2602_01801_b200 import fastar
+
+    g = torch.Generator(device="cuda").manual_seed(d)
+    H, nq, prompt = 3, 200, 96
+    q, kp, vp = (torch.randn(H, n, d, generator=g, device="cuda").bfloat16() for n in (nq, prompt, prompt))
+    cache = fastar.Cache(H, d, 128, 64, np.random.default_rng(3).standard_normal((32, d)).astype(np.float32), max_tokens=nq,
+                         max_prompt_tokens=prompt, max_frames=2)
+    for call in (lambda f: cache.annca(q, kp, vp, f, keep, debug=True), lambda f: cache.annca_lsh(q, kp, vp, f, debug=True)):
+        want = call(nq)
+        for frame_len in (nq + 1, 2 ** 30, 2 ** 31 - 128, 2 ** 31 - 1):
+            got = call(frame_len)
+            assert cache.status() == fastar.OK
+            assert torch.equal(got["out"], want["out"])
+            n = want["nsel"].max() if "nsel" in want else keep
+            assert torch.equal(got["sel"][..., :n], want["sel"][..., :n])
