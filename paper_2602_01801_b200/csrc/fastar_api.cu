@@ -265,13 +265,20 @@ struct View {
   int64_t hs, ts;
   const __nv_bfloat16* p;
 };
+// Every row must start on a 16-byte boundary: the kernels read them by 128-bit loads, 16-byte copies and TMA.
+bool rows_aligned(const fastar_cache* c, const void* p, int64_t hs, int64_t ts) {
+  const int64_t esz = c->desc.dtype == FASTAR_FP32 ? 4 : 2;
+  return !(reinterpret_cast<uintptr_t>(p) & 15) && !((hs * esz) & 15) && !((ts * esz) & 15);
+}
 int as_bf16(fastar_cache* c, View* v, int count, cudaStream_t st) {
-  for (int i = 0; i < count; ++i) v[i].p = static_cast<const __nv_bfloat16*>(v[i].src);
+  for (int i = 0; i < count; ++i) {
+    if (!rows_aligned(c, v[i].src, v[i].hs, v[i].ts)) return FASTAR_ERR_INVALID_ARG;
+    v[i].p = static_cast<const __nv_bfloat16*>(v[i].src);
+  }
   if (c->desc.dtype == FASTAR_BF16) return FASTAR_OK;
   ConvertArgs a{};
   a.count = count;
   for (int i = 0; i < count; ++i) {
-    if ((reinterpret_cast<uintptr_t>(v[i].src) & 15) || (v[i].hs & 3) || (v[i].ts & 3)) return FASTAR_ERR_INVALID_ARG;
     a.t[i] = {static_cast<const float*>(v[i].src), c->v.stage[v[i].slot], v[i].hs, v[i].ts, v[i].rows};
     v[i].p = c->v.stage[v[i].slot];
     v[i].hs = static_cast<int64_t>(v[i].rows) * c->v.D;
@@ -605,8 +612,7 @@ static int annsa_impl(fastar_cache_t* c, const void* q, const void* k_seg, const
   if (block_q != 64 && block_q != 128) return FASTAR_ERR_UNSUPPORTED_SHAPE;
   if (nq > c->v.max_tokens) return FASTAR_ERR_UNSUPPORTED_SHAPE;
   if (token_stride < c->v.D || head_stride < 0 || (sel_in && !nsel_in)) return FASTAR_ERR_INVALID_ARG;
-  const size_t osz = c->desc.dtype == FASTAR_FP32 ? 4 : 2;
-  if ((reinterpret_cast<uintptr_t>(out) & 15) || ((head_stride * osz) & 15) || ((token_stride * osz) & 15)) return FASTAR_ERR_INVALID_ARG;
+  if (!rows_aligned(c, out, head_stride, token_stride)) return FASTAR_ERR_INVALID_ARG;
   DeviceGuard guard(c->desc.device);
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   const CacheView& v = c->v;
@@ -700,7 +706,7 @@ int fastar_annsa_prepare(fastar_cache_t* c, const void* q, int32_t nq, int64_t h
   if (!c || !q || nq < 1) return FASTAR_ERR_INVALID_ARG;
   if (block_q != 64 && block_q != 128) return FASTAR_ERR_UNSUPPORTED_SHAPE;
   if (nq > c->v.max_tokens) return FASTAR_ERR_UNSUPPORTED_SHAPE;
-  if (token_stride < c->v.D || head_stride < 0) return FASTAR_ERR_INVALID_ARG;
+  if (token_stride < c->v.D || head_stride < 0 || !rows_aligned(c, q, head_stride, token_stride)) return FASTAR_ERR_INVALID_ARG;
   DeviceGuard guard(c->desc.device);
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   const CacheView& v = c->v;
@@ -708,7 +714,6 @@ int fastar_annsa_prepare(fastar_cache_t* c, const void* q, int32_t nq, int64_t h
   const __nv_bfloat16* qb = static_cast<const __nv_bfloat16*>(q);
   int64_t qhs = head_stride, qts = token_stride;
   if (c->desc.dtype == FASTAR_FP32) {          // own staging buffer: an update or another attention call may be converting too
-    if ((reinterpret_cast<uintptr_t>(q) & 15) || (qhs & 3) || (qts & 3)) return FASTAR_ERR_INVALID_ARG;
     ConvertArgs a{};
     a.count = 1;
     a.t[0] = {static_cast<const float*>(q), v.stage_prep, qhs, qts, nq};
@@ -749,8 +754,7 @@ int fastar_annca_attention(fastar_cache_t* c, const void* q, const void* k_promp
   const int F = (nq + frame_len - 1) / frame_len;
   if (nq > c->v.max_tokens || np > c->v.max_prompt || F > c->v.max_frames) return FASTAR_ERR_UNSUPPORTED_SHAPE;
   if (token_stride < c->v.D || prompt_token_stride < c->v.D) return FASTAR_ERR_INVALID_ARG;
-  const size_t osz = c->desc.dtype == FASTAR_FP32 ? 4 : 2;
-  if ((reinterpret_cast<uintptr_t>(out) & 15) || ((head_stride * osz) & 15) || ((token_stride * osz) & 15)) return FASTAR_ERR_INVALID_ARG;
+  if (!rows_aligned(c, out, head_stride, token_stride)) return FASTAR_ERR_INVALID_ARG;
   DeviceGuard guard(c->desc.device);
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   const CacheView& v = c->v;
@@ -761,8 +765,6 @@ int fastar_annca_attention(fastar_cache_t* c, const void* q, const void* k_promp
   if (r != FASTAR_OK) return r;
   const __nv_bfloat16 *qb = in[0].p, *kpb = in[1].p, *vpb = in[2].p;
   const int64_t qhs = in[0].hs, qts = in[0].ts, khs = in[1].hs, kts = in[1].ts;      // K and V alike
-  if ((reinterpret_cast<uintptr_t>(kpb) & 15) || (reinterpret_cast<uintptr_t>(vpb) & 15) || ((khs * 2) & 15) || ((kts * 2) & 15))
-    return FASTAR_ERR_INVALID_ARG;
   CUtensorMap tm_q, tm_kp;
   r = make_map(c, &tm_q, qb, v.D, nq, v.H, static_cast<uint64_t>(qts) * 2, static_cast<uint64_t>(qhs) * 2, 128);
   if (r != FASTAR_OK) return r;
@@ -835,8 +837,7 @@ int fastar_annca_attention_lsh(fastar_cache_t* c, const void* q, const void* k_p
   const int F = (nq + frame_len - 1) / frame_len;
   if (nq > c->v.max_tokens || np > c->v.max_prompt || F > c->v.max_frames) return FASTAR_ERR_UNSUPPORTED_SHAPE;
   if (token_stride < c->v.D || prompt_token_stride < c->v.D) return FASTAR_ERR_INVALID_ARG;
-  const size_t osz = c->desc.dtype == FASTAR_FP32 ? 4 : 2;
-  if ((reinterpret_cast<uintptr_t>(out) & 15) || ((head_stride * osz) & 15) || ((token_stride * osz) & 15)) return FASTAR_ERR_INVALID_ARG;
+  if (!rows_aligned(c, out, head_stride, token_stride)) return FASTAR_ERR_INVALID_ARG;
   DeviceGuard guard(c->desc.device);
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   const CacheView& v = c->v;
@@ -845,8 +846,6 @@ int fastar_annca_attention_lsh(fastar_cache_t* c, const void* q, const void* k_p
   if (r != FASTAR_OK) return r;
   const __nv_bfloat16 *qb = in[0].p, *kpb = in[1].p, *vpb = in[2].p;
   const int64_t qhs = in[0].hs, qts = in[0].ts, khs = in[1].hs, kts = in[1].ts;      // K and V alike
-  if ((reinterpret_cast<uintptr_t>(kpb) & 15) || (reinterpret_cast<uintptr_t>(vpb) & 15) || ((khs * 2) & 15) || ((kts * 2) & 15))
-    return FASTAR_ERR_INVALID_ARG;
   CUtensorMap tm_q;
   r = make_map(c, &tm_q, qb, v.D, nq, v.H, static_cast<uint64_t>(qts) * 2, static_cast<uint64_t>(qhs) * 2, 128);
   if (r != FASTAR_OK) return r;
