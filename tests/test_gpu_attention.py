@@ -1,5 +1,6 @@
-"""The attention kernel's tile loop: one to many key tiles (both soft-max groups, the hand-over of the running maximum between them),
-maxima that rise late or by far, dead and weighted slots, an un-cached segment, ragged query blocks."""
+"""The attention kernel's tile loop: one to many key tiles (the four soft-max groups, the hand-over of the running maximum between
+them), maxima that rise late or by far, weighted slots, an un-cached segment, ragged query blocks; many items per CTA, blocks without a
+live slot, values at the ends of their range."""
 import math
 
 import numpy as np
@@ -49,6 +50,42 @@ def test_tiles_and_maxima(d, pt, nq, length, seg, rise):
         # probabilities and output rounded to 8 significant bits (2^-8 each), sums in fp32: 2^-7 of the largest value averaged
         assert np.abs(got - want).max() <= 2.0 ** -7 * np.abs(vv).max()
         assert np.linalg.norm(got - want) <= 1e-2 * np.linalg.norm(want)
+
+
+@pytest.mark.parametrize("d,pt,seg", [(128, 128, 0), (128, 64, 0), (64, 128, 190), (64, 64, 70), (128, 64, 129)])
+def test_many_items_on_a_cta(d, pt, seg):
+    """400 items on 148 CTAs, with what one item leaves to the next: numbers of sub-tiles that no count of groups or stages divides,
+    empty heads between others, maxima that rise in some items and fall from one item to the next."""
+    import torch
+    from paper_2602_01801_b200 import fastar
+    rng = np.random.default_rng(d + pt + seg)
+    H, nq, cap = 40, 10 * 128 - 50, 1408
+    lens = np.resize([1, 65, 0, 5 * pt, cap, 3 * pt + 1, 700, 129, 0, pt + 64, 11 * 64 + 3], H)
+    q = rng.standard_normal((H, -(-nq // 128), 128, d)) * rng.choice([1.0, 30.0], (H, -(-nq // 128), 1, 1))
+    q = synth.round_bf16(q.reshape(H, -1, d)[:, :nq].astype(np.float32))
+    k, v = (synth.round_bf16(rng.standard_normal((H, cap + seg, d)).astype(np.float32)) for _ in range(2))
+    k[::3] *= (2.0 ** np.linspace(-3, 2, cap + seg).round())[None, :, None].astype(np.float32)      # exact in bf16
+    count = rng.integers(1, 9, (H, cap)).astype(np.int32)
+    cache = fastar.Cache(H, d, cap, pt, rng.standard_normal((32, d)).astype(np.float32), max_tokens=nq)
+    cache.import_state(fastar.bf16_bits(k[:, :cap]), fastar.bf16_bits(v[:, :cap]), lens, count)
+    if seg:
+        out = cache.annsa_segment(fastar.to_device(q), fastar.to_device(k[:, cap:]), fastar.to_device(v[:, cap:]), 128, cap // pt)["out"]
+    else:
+        out = cache.annsa(fastar.to_device(q), 128, cap // pt)["out"]
+    assert cache.status() == 0
+    for h in range(H):
+        L = int(lens[h])
+        got = out[h].float().cpu().numpy()
+        if L + seg == 0:
+            assert (got == 0).all()
+            continue
+        s = q[h].astype(np.float64) @ np.concatenate([k[h, :L], k[h, cap:]]).T / math.sqrt(d)
+        s += np.log(np.concatenate([count[h, :L], np.ones(seg)]))
+        p = np.exp(s - s.max(1, keepdims=True))
+        want = (p / p.sum(1, keepdims=True)) @ np.concatenate([v[h, :L], v[h, cap:]])
+        # as above: rounding of the probabilities and of the output
+        assert np.abs(got - want).max() <= 2.0 ** -7 * np.abs(v).max(), f"head {h}"
+        assert np.linalg.norm(got - want) <= 1e-2 * np.linalg.norm(want), f"head {h}"
 
 
 @pytest.mark.parametrize("d,pt,seg", [(128, 128, 0), (128, 64, 70), (64, 128, 200), (64, 64, 0)])

@@ -26,7 +26,7 @@ T.test_other_tile_shapes(64, 64)
 T.test_eviction_and_sink_and_capacity_error()
 T.test_shared_page_pool_across_ragged_heads(128, 128, 16)
 T.test_eight_bit_quantised_search(128, 128)
-T.test_query_probe_correspondence(128, 128, False, "pair")
+T.test_query_probe_correspondence(128, 128, False)
 T.test_annsa_with_uncached_segment(128, 64, True)
 T.test_annca_lsh_bucket_rule(128, False, 8)
 T.test_random_shapes_and_options(3)

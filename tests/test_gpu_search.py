@@ -25,6 +25,8 @@ def _case(d, pt, n, lengths, seed):
 @pytest.mark.parametrize("d,pt,n,lengths", [
     (128, 128, 1, (1,)), (64, 64, 128, (128, 0, 127)), (128, 64, 129, (129, 640)), (128, 128, 256, (255, 1, 0, 3000)),
     (64, 128, 257, (5000, 129, 4096)), (128, 128, 385, (6000,) * 7), (64, 64, 1000, (2049, 2048, 2047)), (128, 128, 2600, (9000, 12000)),
+    # many heads whose second unit is one tile (the other group of warps sits it out), more keys than one wave may touch (96 MB)
+    (128, 64, 300, (700, 129, 0, 1500) * 10), (128, 128, 300, (52000, 50000, 49999, 51000, 50001, 50000, 52001, 50000)),
 ])
 def test_search_edges(d, pt, n, lengths, probe):
     import torch
