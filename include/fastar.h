@@ -25,7 +25,7 @@
  *     destroyed with it).  Nothing here allocates device memory.
  *   - Tensors are [head][token][channel] with element strides `head_stride`, `token_stride`
  *     (channel stride 1).  Strides in bytes must be multiples of 16 and base pointers 16-byte
- *     aligned (TMA requirement).  Element type is the cache's `dtype`: bf16, or fp32 which is
+ *     aligned, else FASTAR_ERR_INVALID_ARG.  Element type is the cache's `dtype`: bf16, or fp32 which is
  *     rounded to bf16 (nearest-even) on entry; outputs are written in the same type.
  *   - Heads are independent (the paper's formulas are per head); cache lengths are ragged
  *     across heads and live on the device, so no call needs a host round trip.
@@ -274,7 +274,7 @@ int fastar_annsa_attention_segment(fastar_cache_t* cache, const void* q, const v
  *   largest r (ties: lower p); o_i = softmax over the kept p of q_i.k_p/sqrt(d), times v_p.
  * The cache object only supplies H, d, dtype, scratch and the status word; its contents are
  * not touched, and the scratch it uses is its own.  One AnnCA call may therefore run on another
- * stream at the same time as an update or an AnnSA call of the same cache (the step's three calls
+ * stream at the same time as an update, a reset, an import or an AnnSA call of the same cache (the step's three calls
  * are otherwise issued on one stream, or ordered by the caller; two calls of the same kind never
  * overlap).  q, out: dev [H][nq][d]; k_prompt, v_prompt: dev [H][np][d] with their own strides.
  * Optional dev outputs: sel_out [H][F][keep_tokens] (ascending), rel_out [H][F][np] fp32.

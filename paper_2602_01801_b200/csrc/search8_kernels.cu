@@ -11,8 +11,9 @@
 //   quantize_kernel      : bf16 rows + 1/|x|  ->  codes
 //   quantize_rows_kernel : bf16 rows  ->  codes and |x| (AnnCA's queries and prompt keys, Section 5.3)
 //   search8_kernel       : codes of the new keys x codes of the cache, row arg-max fused (ties -> lowest slot)
-// Same CTA layout as the bf16 similarity kernel: 128 new keys per CTA (resident), key tiles streamed through a TMA
-// ring, two fp32 accumulators in TMEM, eight epilogue warps, 2 CTAs per SM.  Every wait is bounded.
+// A CTA keeps 128 new keys in shared memory and streams key tiles past them through a TMA ring; two fp32 accumulators in TMEM, eight
+// epilogue warps (two threads a row), 2 CTAs per SM.  12 heads, 4 680 new against 28 080 cached keys: 164 us, 0.73 of twice the measured
+// bf16 rate; the rest is the arg-max.  Every wait is bounded.
 #include <cuda_fp8.h>
 
 #include "common.h"

@@ -414,8 +414,9 @@ __global__ void __launch_bounds__(1024) plan_kernel(const CacheView c, int n, in
       }
     };
     // Up to 2 x 16384 slots a thread keeps its ages in registers, two to a word, so the search for the age and the compaction read
-    // nothing again (12 heads x 32768 slots at capacity: 87 -> 44 us; longer caches, and ages above 16 bits, go through L2 in every
-    // pass, as all did before).
+    // nothing again (12 heads x 32768 slots at capacity: 87 -> 44 us).  A third pass would be eight more of the 64 registers that 1 024
+    // threads leave each, and two are all that fit (12 bytes spill already): longer caches, and ages above 16 bits, go through L2 in
+    // every pass, as all did before.
     constexpr int kPasses = 2;
     uint32_t held[kPasses][8];
     int cand = 0, a_min = 0x7fffffff, a_max = 0;
@@ -724,8 +725,11 @@ int launch_query_hist(const CacheView& c, const uint32_t* codes, int nq, int blo
 // One warp per row, the row in registers (entry 32 i + lane).  The k-th largest key is found bit by bit, from the highest bit in
 // which the row's keys differ: one count over the row per bit, a dozen instructions per 32 entries, no barrier; the entries above it
 // and the first of those equal to it are then listed in index order by ballots.  Latency-bound (a few thousand dependent
-// instructions).  Measured against a 256-thread bitonic sort of (key, index): 256 rows of 1056 32.0 -> 7.2 us, 3400 rows of 512
-// 78 -> 9.2 us, 444 rows of 256 7.6 -> 4.4 us, 36 rows of 512 prompt tokens 8.4 -> 6.5 us.
+// instructions), and the time follows the registers a lane holds, whatever part of them the row fills: 2.5 us with 4, 3.9 with 16, 6.1
+// with 36, 8.9 with 64 (8 heads x 32 rows of block scores; 1 024 prompt tokens 8.8 with 36, 19.8 with 64).  Hence steps: 4, 16 and 64 are a
+// factor of four apart, and 36 divides the widest of them so that 131 072 keys in 128-slot blocks, or 1 024 prompt tokens, with an eighth
+// to spare, are on the cheap side.  Measured against a 256-thread bitonic sort of (key, index): 256 rows of 1056 32.0 -> 7.2 us, 3400
+// rows of 512 78 -> 9.2 us, 444 rows of 256 7.6 -> 4.4 us, 36 rows of 512 prompt tokens 8.4 -> 6.5 us.
 // ---------------------------------------------------------------------------------------------
 struct TopkArgs {
   void* src;                       // PROMPT: ordered-uint relevance (zeros are put back); else block scores as floats
