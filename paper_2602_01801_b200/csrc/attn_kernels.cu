@@ -26,10 +26,18 @@
 //   - the row sums add up the probabilities as rounded to bf16, so that they cancel in a row that one key dominates;
 //   - the soft-max warps hold a sub-tile in the 16 x 256-bit fragment shape, four rows x 16 columns a thread: a thread reads 16
 //     biases, not 64, and a warp still has its rows to itself;
-//   - Q K^T and P V are issued by two warps, so that a barrier that one of them waits for does not hold back the other;
+//   - Q K^T and P V are issued by two warps, so that a barrier that one of them waits for does not hold back the other, with running
+//     stage numbers and descriptors: what they do between two barriers is on the way of every sub-tile;
+//   - a sub-tile's logits, its biases and the running maximum are asked for together, because each of them takes hundreds of cycles while
+//     Q K^T reads both operands from shared memory (eight 64-bit loads by a warp: 203 cycles, 850-2 600 beside such MMAs).  With the two
+//     points: denoising step of 12 heads 313 -> 298 us, 8 heads, d = 64, 64 of 1 024 blocks 146 -> 142;
+//   - items that do not fill the last round of the SMs are cut by key tiles (see launch_attn), and the soft-max loop is as large as
+//     an SM's instruction caches bear (stalls for instructions: a twentieth of a warp's time, and a sixth with a little more code in the
+//     kernel), so the cut is a variant of its own;
 //   - the CTA stays for its items, and the copies and Q K^T run ahead into the next one, whose first logits are there when the
 //     output of the last has left.
-// TMEM columns: S 4 x 64, P 4 x 32, O 128.  K and V tiles have a TMA ring each.
+// TMEM columns: S 4 x 64, P 4 x 32, O D; with key tiles of 64: S 3 x 64, P, O and Q D / 2 (AttnSmem::QT).  K and V tiles have a TMA ring
+// each.
 // Measured (B200, kernel time; two groups with whole tiles, a CTA per item, a limit of 8 -> this): 12 heads, d = 128, 4 680 queries on
 // 32 of 224 blocks 120.5 -> 105.4 us (0.68 of the measured bf16 peak); the same with the chunk's 4 680 keys beside 241 -> 218 us; 8
 // heads, 4 096 queries on all 16 384 keys 275 -> 246 us (108 of 148 CTAs have two items); d = 64, 64 of 1 024 blocks 142 -> 125 us,
@@ -65,6 +73,8 @@ __device__ __forceinline__ float4 lds4(uint32_t addr) {
 // for values up to 2^119 / keys.  What the code calls the maximum, and the warps hand on, is that reference.
 constexpr float kHead = 16.f, kTop = 8.f;
 
+constexpr float kPartStore = 3.f, kPartAdd = 1.2f, kPartStop = 14.f, kPartGain = 0.05f;     // key tiles, see launch_attn
+
 template <int D, int BKT>
 struct AttnSmem {
   static constexpr int q_bytes = (D / 64) * kQChunk;
@@ -75,7 +85,12 @@ struct AttnSmem {
   static constexpr int RS = 160 * 1024 / kv_bytes > 12 ? 12 : 160 * 1024 / kv_bytes;
   static constexpr int RK = (RS + 1) / 2, RV = RS / 2;
   static constexpr int SUB = BKT / 64;                           // sub-tiles of a key tile
-  static constexpr int NSB = kGroups / SUB;                      // key tiles whose logits are in tensor memory
+  // Q as the MMAs' operand in tensor memory (QT) or in shared memory.  A 128 x 64 x 16 MMA with both operands in shared memory waits for
+  // them (48 cycles, 32 with Q in tensor memory), so tiles of 64 keys take the former, which leaves columns for the logits of three
+  // sub-tiles instead of four; with 128 keys the latter is as fast, and a fourth sub-tile ahead is worth more (denoising step 311 / 298 us
+  // a pass, 161 items of 596 tiles of 64 keys 588 / 633).
+  static constexpr bool QT = BKT == 64;
+  static constexpr int NSB = QT ? 3 : kGroups / SUB;             // sub-tiles (QT) or key tiles whose logits are in tensor memory
   // Bias rows: one is overwritten when NB (16 or 32) tiles later the key tile is fetched, at most six key tiles behind one that is
   // consumed, whose logits went where those of a tile at least two rounds of the groups after this one had been.
   static constexpr int NB = 2048 / BKT;
@@ -86,7 +101,7 @@ struct AttnSmem {
   static constexpr int max_off = xchg_off + 2 * kGroups * 1024;  // [4][8][4] running maxima: warp of the group, lane / 4, row / 8
   static constexpr int bar_off = max_off + 512;
   static constexpr int total = bar_off + 512;
-  static constexpr int p_col = kGroups * 64, o_col = kGroups * 96;       // TMEM columns (S at 0)
+  static constexpr int p_col = (QT ? 3 : kGroups) * 64, o_col = p_col + kGroups * 32, q_col = o_col + D;      // TMEM columns (S at 0)
   static constexpr int tmem_cols = 512;
 };
 
@@ -99,14 +114,115 @@ struct AttnItem {
   const int32_t* list;                  // paged mode: kept blocks (null: all); gather mode: kept tokens
 };
 
-// SEG (paged mode only): tiles of an un-cached K/V segment follow the cache tiles.
-template <int D, int BKT, bool GATHER, bool SEG>
+// SPLIT: the items of the last, partly filled round lie on a line, each as `units` units, and CTA b of `pieces` takes the units
+// [n b / pieces, n (b + 1) / pieces).  An item's tiles are dealt to its units in proportion, so that every role knows its way without
+// the others' tile counts; units is the most tiles that an item can have, and what it has wherever the lists are full.
+struct AttnPart {
+  int item;                             // of the last round's items
+  int lo, hi;                           // its units
+};
+struct AttnPiece {                      // a CTA's piece: stops 0 .. n - 1 are the items first, first + 1, ...
+  int first, n, lo, hi;                 // lo: first unit of the first, hi: end of the last
+};
+__device__ __forceinline__ AttnPiece piece_of_cta(const AttnArgs& a) {      // (the launch keeps these products below 2^31)
+  const unsigned n = a.last_items * a.units, b = blockIdx.x, units = a.units, pieces = a.pieces;
+  const unsigned x0 = n * b / pieces, x1 = n * (b + 1) / pieces;
+  AttnPiece p{};
+  if (b >= pieces || x1 == x0) return p;
+  p.first = x0 / units;
+  p.n = (x1 - 1) / units - p.first + 1;
+  p.lo = x0 - p.first * units;
+  p.hi = x1 - (p.first + p.n - 1) * units;
+  return p;
+}
+__device__ __forceinline__ int piece_at(const AttnArgs& a, int x) {         // the piece that unit x belongs to
+  return (static_cast<unsigned>(x + 1) * a.pieces - 1) / static_cast<unsigned>(a.last_items * a.units);
+}
+__device__ __forceinline__ int tile_at(const AttnArgs& a, int nt, int unit) {       // the tile that a unit of an item of nt tiles begins with
+  return static_cast<unsigned>(nt * unit) / static_cast<unsigned>(a.units);
+}
+// Where a CTA's part of a cut item goes: a piece has two cut items at most, the one that it begins in and the one that it ends in.
+__device__ __forceinline__ int slot_of(int piece, bool begins) { return 2 * piece + (begins ? 1 : 0); }
+
+// A warp's 32 rows x 32 columns of a part (v, relative to the reference m, with the rows' sums) go to memory.
+template <int D>
+__device__ __forceinline__ float4* part_rows(const CacheView& c, int slot, int g, int r) {
+  return reinterpret_cast<float4*>(c.part_o) + (static_cast<int64_t>(slot) * (D / 4) + g * 8) * 128 + r;
+}
+__device__ __forceinline__ float2* part_stat(const CacheView& c, int slot, int g, int r) {
+  return c.part_ml + (static_cast<int64_t>(slot) * kGroups + g) * 128 + r;
+}
+template <int D>
+__device__ __forceinline__ void store_part(const CacheView& c, int slot, int g, int r, const uint32_t (&v)[32], float m, float sum) {
+  float4* dst = part_rows<D>(c, slot, g, r);
+#pragma unroll
+  for (int q = 0; q < 8; ++q)
+    __stcg(dst + q * 128, make_float4(__uint_as_float(v[4 * q]), __uint_as_float(v[4 * q + 1]), __uint_as_float(v[4 * q + 2]), __uint_as_float(v[4 * q + 3])));
+  __stcg(part_stat(c, slot, g, r), make_float2(m, sum));
+}
+// Adds up a warp's share of the `parts` parts of an item, in the order of the pieces; returns the rows' sums.  A part without a live key
+// has a reference of -inf and no rows.
+template <int D>
+__device__ __forceinline__ float merge_parts(const CacheView& c, int first_piece, int parts, int g, int r, uint32_t (&v)[32]) {
+  float m = -INFINITY, sum = 0.f;
+#pragma unroll 4
+  for (int p = 0; p < parts; ++p) m = fmaxf(m, __ldcg(part_stat(c, slot_of(first_piece + p, p == 0), g, r)).x);
+#pragma unroll
+  for (int q = 0; q < 32; ++q) v[q] = 0u;
+#pragma unroll 1
+  for (int p = 0; p < parts; ++p) {
+    const int slot = slot_of(first_piece + p, p == 0);
+    const float2 ml = __ldcg(part_stat(c, slot, g, r));
+    const float4* src = part_rows<D>(c, slot, g, r);
+    float4 x[8];
+#pragma unroll
+    for (int q = 0; q < 8; ++q) x[q] = __ldcg(src + q * 128);
+    if (ml.x == -INFINITY) continue;
+    const float f = fast_exp2(ml.x - m);
+    sum = fmaf(ml.y, f, sum);
+#pragma unroll
+    for (int q = 0; q < 8; ++q) {
+      const float2 a = ffma2(make_float2(x[q].x, x[q].y), make_float2(f, f), make_float2(__uint_as_float(v[4 * q]), __uint_as_float(v[4 * q + 1])));
+      const float2 b = ffma2(make_float2(x[q].z, x[q].w), make_float2(f, f), make_float2(__uint_as_float(v[4 * q + 2]), __uint_as_float(v[4 * q + 3])));
+      v[4 * q] = __float_as_uint(a.x);
+      v[4 * q + 1] = __float_as_uint(a.y);
+      v[4 * q + 2] = __float_as_uint(b.x);
+      v[4 * q + 3] = __float_as_uint(b.y);
+    }
+  }
+  return sum;
+}
+// 32 columns of a row, divided by the row's sum.
+__device__ __forceinline__ void write_row(const AttnArgs& a, int64_t off, const uint32_t (&v)[32], float sum) {
+  const float inv = sum > 0.f ? 1.f / sum : 0.f;
+  if (a.out_fp32) {
+    float4* dst = reinterpret_cast<float4*>(static_cast<float*>(a.out) + off);
+#pragma unroll
+    for (int q = 0; q < 8; ++q)
+      dst[q] = make_float4(__uint_as_float(v[4 * q]) * inv, __uint_as_float(v[4 * q + 1]) * inv, __uint_as_float(v[4 * q + 2]) * inv,
+                           __uint_as_float(v[4 * q + 3]) * inv);
+  } else {
+    uint4* dst = reinterpret_cast<uint4*>(static_cast<__nv_bfloat16*>(a.out) + off);
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      uint32_t o[4];
+#pragma unroll
+      for (int e = 0; e < 4; ++e)
+        o[e] = pack_bf16x2(__uint_as_float(v[8 * q + 2 * e]) * inv, __uint_as_float(v[8 * q + 2 * e + 1]) * inv);
+      dst[q] = make_uint4(o[0], o[1], o[2], o[3]);
+    }
+  }
+}
+
+// SEG (paged mode only): tiles of an un-cached K/V segment follow the cache tiles.  SPLIT (paged mode only): the last round's items are
+// cut by key tiles.
+template <int D, int BKT, bool GATHER, bool SEG, bool SPLIT>
 __global__ void __launch_bounds__(kAttnThreads, 1)
 attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k,
             const __grid_constant__ CUtensorMap tm_v, const __grid_constant__ CUtensorMap tm_sk,
             const __grid_constant__ CUtensorMap tm_sv, const CacheView c, const AttnArgs a) {
   using SM = AttnSmem<D, BKT>;
-  constexpr int RS = SM::RS, RK = SM::RK, RV = SM::RV, NB = SM::NB, SUB = SM::SUB, NSB = SM::NSB;
+  constexpr int RS = SM::RS, RK = SM::RK, RV = SM::RV, NB = SM::NB, SUB = SM::SUB;
   extern __shared__ __align__(1024) uint8_t smem_raw[];
   const uint32_t sbase = smem_u32(smem_raw);
   if (sbase & 1023u) {                  // swizzled tiles need 1024-byte alignment; uniform for the CTA
@@ -128,7 +244,10 @@ attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CU
   const uint32_t bar_xchg = bar_p_full + 32;         // [1] the groups meet here before an item's epilogue
   const uint32_t bar_o_free = bar_xchg + 8;          // [1] the soft-max warps: O of the item has been read
   const uint32_t bar_done = bar_xchg + 16;           // [1] the soft-max warps are through
-  constexpr int kNumBars = 2 + 2 * RS + 19;
+  const uint32_t bar_parts = bar_xchg + 24;          // [1] SPLIT: the warps that store parts are through
+  const uint32_t bar_last = bar_xchg + 32;           // [1] SPLIT: last_s is there
+  const uint32_t bar_qk_done = bar_xchg + 40;        // [1] Q K^T of an item is complete
+  constexpr int kNumBars = 2 + 2 * RS + 22;
   static_assert(kNumBars * 8 + 12 <= 512, "barrier area");
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smem_raw + SM::bar_off + kNumBars * 8);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(smem_raw + SM::bar_off + kNumBars * 8 + 4);
@@ -151,11 +270,15 @@ attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CU
 
   // one thread per barrier
   if (threadIdx.x < kNumBars) {
-    const int i = static_cast<int>(threadIdx.x) - (kNumBars - 19);        // s_full, pv_done, s_empty, p_full, xchg, o_free, done
-    mbar_init(bar + 8 * threadIdx.x, i >= 16 ? kSoftWarps : i >= 12 ? 4 : i >= 8 ? 4 * SUB : i >= 4 || i < 0 ? 1 : 2);
+    const int i = static_cast<int>(threadIdx.x) - (kNumBars - 22);        // s_full, pv_done, s_empty, p_full, xchg, o_free, done, parts, last, qk_done
+    mbar_init(bar + 8 * threadIdx.x, i >= 20 ? 1 : i == 19 ? 4 * (D / 32) : i >= 16 ? kSoftWarps : i >= 12 || (i >= 8 && SM::QT) ? 4 : i >= 8 ? 4 * SUB : i >= 4 || i < 0 ? 1 : 2);
     fence_mbar_init();
   }
   if (threadIdx.x == 0) *abort_flag = *done_flag = 0;
+  AttnPiece* piece_s = reinterpret_cast<AttnPiece*>(smem_raw + SM::bar_off + 480);
+  volatile uint32_t* last_s = reinterpret_cast<volatile uint32_t*>(smem_raw + SM::bar_off + 496);      // cut items that this CTA has the last part of
+  static_assert(kNumBars * 8 + 12 <= 480, "this CTA's piece");
+  if (SPLIT && threadIdx.x == 64) *piece_s = piece_of_cta(a);
   if (warp == kKeyWarp && lane == 0) {
     tma_prefetch_desc(&tm_q);
     if (!GATHER) { tma_prefetch_desc(&tm_k); tma_prefetch_desc(&tm_v); }
@@ -192,10 +315,23 @@ attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CU
     return w;
   };
 
+  // The stops of a CTA: the items it, it + gridDim.x, ...; SPLIT: `rounds` of those, as it = 0, 1, ..., then its piece of the last round.
+  const int it_first = SPLIT ? 0 : blockIdx.x, it_step = SPLIT ? 1 : gridDim.x;
+  auto part_of = [&](int k) {
+    return AttnPart{piece_s->first + k, k == 0 ? piece_s->lo : 0, k + 1 == piece_s->n ? piece_s->hi : a.units};
+  };
+  auto more = [&](int it) { return SPLIT ? __shfl_sync(0xffffffffu, it < a.rounds + piece_s->n ? 1 : 0, 0) != 0 : it < items; };
+  auto item_at = [&](int it) {
+    if (!SPLIT) return it;
+    return __shfl_sync(0xffffffffu, static_cast<int>(it < a.rounds ? blockIdx.x + it * gridDim.x : a.rounds * gridDim.x + piece_s->first + it - a.rounds), 0);
+  };
   auto tiles_of = [&](int it) {
     if (GATHER) return item_of(it).nt;
-    const int h = it / row_blocks % c.H;
-    return (a.sel ? __shfl_sync(0xffffffffu, a.nsel[h], 0) : (__shfl_sync(0xffffffffu, c.len[h], 0) + BKT - 1) / BKT) + (SEG ? a.seg_tiles : 0);
+    const int h = item_at(it) / row_blocks % c.H;
+    const int nt = (a.sel ? __shfl_sync(0xffffffffu, a.nsel[h], 0) : (__shfl_sync(0xffffffffu, c.len[h], 0) + BKT - 1) / BKT) + (SEG ? a.seg_tiles : 0);
+    if (!SPLIT || it < a.rounds) return nt;
+    const AttnPart p = part_of(it - a.rounds);
+    return __shfl_sync(0xffffffffu, tile_at(a, nt, p.hi) - tile_at(a, nt, p.lo), 0);
   };
 
   // Everything is counted through the items of a CTA: tile0 key tiles, tile0 * SUB sub-tiles before.  Key tile n is in K stage n % RK
@@ -209,8 +345,15 @@ attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CU
       const uint32_t first = is_k ? 0 : RK, end = is_k ? RK : RS;
       uint32_t st = first, empty_phase = 1, copied = 0, n_q = 0;
       bool ok = true;
-      for (int it = blockIdx.x; it < items && ok; it += gridDim.x) {
-        const AttnItem w = item_of(it);
+      for (int it = it_first; more(it) && ok; it += it_step) {
+        AttnItem w = item_of(item_at(it));
+        if (SPLIT && it >= a.rounds) {          // tiles [j0, j0 + nt): the list from there, or for all blocks in order the first block itself
+          const AttnPart p = part_of(it - a.rounds);
+          const int j0 = __shfl_sync(0xffffffffu, tile_at(a, w.nt, p.lo), 0);
+          w.list = a.sel ? w.list + j0 : reinterpret_cast<const int32_t*>(static_cast<intptr_t>(j0));
+          w.ntc -= j0;
+          w.nt = __shfl_sync(0xffffffffu, tile_at(a, w.nt, p.hi), 0) - j0;
+        }
         const int nt = w.nt;
         if (nt == 0) continue;
         if (is_k) {
@@ -227,8 +370,9 @@ attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CU
         auto fetch = [&](int j0) {
           const int jj = j0 + lane;
           if (GATHER) return;
+          if (SPLIT && jj >= nt) return;
           if (jj < w.ntc) {
-            blk_n = FASTAR_IDX(w.list ? w.list[jj] : jj, c.CAPB, c.status);
+            blk_n = FASTAR_IDX(a.sel ? w.list[jj] : SPLIT ? static_cast<int>(reinterpret_cast<intptr_t>(w.list)) + jj : jj, c.CAPB, c.status);
             page_n = FASTAR_IDX(c.page_table[static_cast<int64_t>(w.h) * c.CAPB + blk_n], c.pool_pages, c.status);
           } else if (SEG && jj < nt) {        // tile of the un-cached segment: its index, no page
             blk_n = jj - w.ntc;
@@ -312,67 +456,76 @@ attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CU
     } else if (warp == kQkWarp) {
       // ================================================================ S = Q K_j^T
       const uint32_t lead = elect_lane();
-      constexpr uint32_t idesc = make_idesc_bf16(128, BKT, 0);
+      constexpr bool QT = SM::QT;
+      constexpr uint32_t idesc = make_idesc_bf16(128, QT ? 64 : BKT, 0);
+      const uint64_t qd = make_smem_desc(q_s, 16, 1024), kd0 = make_smem_desc(ring_s, 16, 1024);
       bool ok = true;
-      int tile0 = 0, nq_used = 0;
-      for (int it = blockIdx.x; it < items && ok; it += gridDim.x) {
+      uint32_t nq_used = 0, st = 0, r_phase = 0, b = 0, s_phase = 1;       // stage, logits' columns and their barriers' phases
+      for (int it = it_first; more(it) && ok; it += it_step) {
         const int nt = tiles_of(it);
         if (nt == 0) continue;
         ok = mbar_wait_warp<kIssueWaitHintNs>(bar_q_full, nq_used & 1, abort_flag, c.status);
+        if (QT && ok && nq_used > 0) ok = mbar_wait_warp(bar_qk_done, (nq_used - 1) & 1, abort_flag, c.status);
+        if (!ok) break;
         ++nq_used;
+        if (QT) {      // Q to tensor memory; the copies and the MMAs that read them are issued by one thread and execute in order
+          tc_fence_after();
+#pragma unroll
+          for (int kk = 0; kk < D / 16; ++kk) tmem_copy_128x256b(tmem + SM::q_col + kk * 8, qd + (((kk >> 2) * kQChunk + (kk & 3) * 32) >> 4), lead);
+          umma_commit(bar_q_empty, lead);
+        }
         for (int j = 0; j < nt && ok; ++j) {
-          const int jg = tile0 + j, st = jg % RK, b = jg % NSB;
-          // the columns are free once the groups hold the logits of the tile before in registers
-          ok = mbar_wait_warp(bar_r_full + 8 * st, (jg / RK) & 1, abort_flag, c.status) &&
-               (jg < NSB || mbar_wait_warp(bar_s_empty + 8 * b, (jg / NSB - 1) & 1, abort_flag, c.status));
+          // the columns are free once the groups hold the logits before in registers
+          ok = mbar_wait<kIssueWaitHintNs>(bar_r_full + 8 * st, r_phase, abort_flag, c.status) && mbar_wait(bar_s_empty + 8 * b, s_phase, abort_flag, c.status);
+          ok = __all_sync(0xffffffffu, ok);
           if (!ok) break;
           tc_fence_after();
-          const uint32_t kt = ring_s + st * SM::kv_bytes;
+          const uint64_t kd = kd0 + st * (SM::kv_bytes >> 4);
+          const uint32_t s_col = tmem + b * (QT ? 64 : BKT);
 #pragma unroll
           for (int kk = 0; kk < D / 16; ++kk) {
-            const uint64_t ad = make_smem_desc(q_s + (kk >> 2) * kQChunk + (kk & 3) * 32, 16, 1024);
-            const uint64_t bd = make_smem_desc(kt + (kk >> 2) * (BKT * 128) + (kk & 3) * 32, 16, 1024);
-            umma_ss(tmem + b * BKT, ad, bd, idesc, kk != 0, lead);
+            const uint64_t bd = kd + (((kk >> 2) * (BKT * 128) + (kk & 3) * 32) >> 4);
+            if (QT) umma_ts(s_col, tmem + SM::q_col + kk * 8, bd, idesc, kk != 0, lead);
+            else umma_ss(s_col, qd + (((kk >> 2) * kQChunk + (kk & 3) * 32) >> 4), bd, idesc, kk != 0, lead);
           }
           umma_commit(bar_s_full + 8 * b, lead);
           umma_commit(bar_r_empty + 8 * st, lead);
-          if (j + 1 == nt) umma_commit(bar_q_empty, lead);
+          if (j + 1 == nt) umma_commit(QT ? bar_qk_done : bar_q_empty, lead);
           if (lead) mbar_arrive(bar_s_full + 8 * b);     // what this warp has seen land (the biases) is there for the waiting warps
+          if (++st == RK) { st = 0; r_phase ^= 1; }
+          if (++b == SM::NSB) { b = 0; s_phase ^= 1; }
         }
-        tile0 += nt;
       }
     } else if (warp == kPvWarp) {
       // ================================================================ O += P V_j
       const uint32_t lead = elect_lane();
       constexpr uint32_t idesc = make_idesc_bf16(128, D, 1);
+      const uint64_t vd0 = make_smem_desc(ring_s + RK * SM::kv_bytes, BKT * 128, 1024);
       bool ok = true;
-      int tile0 = 0, n_done = 0;
-      for (int it = blockIdx.x; it < items && ok; it += gridDim.x) {
+      uint32_t n_done = 0, st = 0, r_phase = 0, b = 0, p_phase = 0;
+      for (int it = it_first; more(it) && ok; it += it_step) {
         const int nt = tiles_of(it);
         if (nt == 0) continue;
         if (n_done > 0) ok = mbar_wait_warp(bar_o_free, (n_done - 1) & 1, abort_flag, c.status);
         ++n_done;
         for (int j = 0; j < nt && ok; ++j) {
-          const int jg = tile0 + j, st = RK + jg % RV;
-          ok = mbar_wait_warp(bar_r_full + 8 * st, (jg / RV) & 1, abort_flag, c.status);
-          const uint32_t vt = ring_s + st * SM::kv_bytes;
+          ok = mbar_wait_warp(bar_r_full + 8 * (RK + st), r_phase, abort_flag, c.status);
+          const uint64_t vd = vd0 + st * (SM::kv_bytes >> 4);
 #pragma unroll
           for (int sub = 0; sub < SUB; ++sub) {
-            const int tg = jg * SUB + sub, b = tg % kGroups;
-            ok = ok && mbar_wait_warp(bar_p_full + 8 * b, (tg / kGroups) & 1, abort_flag, c.status);
+            ok = ok && mbar_wait_warp(bar_p_full + 8 * b, p_phase, abort_flag, c.status);
             if (!ok) break;
             tc_fence_after();
 #pragma unroll
-            for (int ks = 0; ks < 4; ++ks) {
-              const uint64_t bd = make_smem_desc(vt + (sub * 4 + ks) * 2048, BKT * 128, 1024);
-              umma_ts(tmem + SM::o_col, tmem + SM::p_col + b * 32 + ks * 8, bd, idesc, (j | sub | ks) != 0, lead);
-            }
+            for (int ks = 0; ks < 4; ++ks)
+              umma_ts(tmem + SM::o_col, tmem + SM::p_col + b * 32 + ks * 8, vd + (((sub * 4 + ks) * 2048) >> 4), idesc, (j | sub | ks) != 0, lead);
             umma_commit(bar_pv_done + 8 * b, lead);
+            if (++b == kGroups) { b = 0; p_phase ^= 1; }
           }
           if (!ok) break;
-          umma_commit(bar_r_empty + 8 * st, lead);
+          umma_commit(bar_r_empty + 8 * (RK + st), lead);
+          if (++st == RV) { st = 0; r_phase ^= 1; }
         }
-        tile0 += nt;
       }
       // tensor memory goes back when the soft-max warps are through (all of them get there, none waits for long)
       mbar_wait_warp(bar_done, 0, done_flag, c.status);
@@ -388,7 +541,7 @@ attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CU
     // outlive their loop, which the registers do not allow.)
     bool ok = true, s_ready = false;
     int sub0 = 0, n_done = 0;                           // sub-tiles and items before
-    for (int it = blockIdx.x; it < items; it += gridDim.x) {
+    for (int it = it_first; more(it); it += it_step) {
       const int ns = tiles_of(it) * SUB;
       // what follows from these four is worked out again for every item: kept over the items it would not fit the registers
       uint32_t sb_ = sbase, tm_ = tmem;
@@ -401,7 +554,7 @@ attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CU
       const int g = warp >> 2;                          // soft-max group: sub-tiles with index % kGroups == g
       const uint32_t lane_t = tmem + (static_cast<uint32_t>((warp & 3) * 32) << 16);
       const float scale = rsqrtf(static_cast<float>(D)) * 1.4426950408889634f;
-      const uint32_t s_t = lane_t + g * 64, p_t = lane_t + SM::p_col + g * 32, o_t = lane_t + SM::o_col;
+      const uint32_t p_t = lane_t + SM::p_col + g * 32, o_t = lane_t + SM::o_col;
       const uint32_t max_s = sbase + SM::max_off + ((warp & 3) * 8 + (lane >> 2)) * 16;
       const uint32_t bias_t = sbase + SM::bias_off + 8 * (lane & 3);
       // the barriers of the hand-over (all sixteen: nothing else uses one after the roles part): this warp waits for the look at the
@@ -412,45 +565,50 @@ attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CU
 #pragma unroll
       for (int q = 0; q < 4; ++q) { m[q] = -INFINITY; l[q] = make_float2(0.f, 0.f); }
       for (int t = (g - sub0) & (kGroups - 1); t < ns; t += kGroups) {
-        const int tg = sub0 + t, jg = tg / SUB, sb = jg % NSB;
-        if (!s_ready) ok = ok && mbar_wait_warp(bar_s_full + 8 * sb, (jg / NSB) & 1, abort_flag, c.status);
+        const int tg = sub0 + t, jg = tg / SUB;
+        const uint32_t sn = SM::QT ? tg : jg, sb = sn % SM::NSB;       // barrier of the logits
+        // QT: the group before has been told of its logits, so those of the three sub-tiles before are complete: a barrier's parity tells
+        // two phases apart, and the one before this sub-tile's is that of t - 3.  (At an item's first the groups have just met.)
+        if (SM::QT && t > 0) named_barrier_sync(heard, 64);
+        if (SM::QT || !s_ready) ok = ok && mbar_wait_warp(bar_s_full + 8 * sb, (sn / SM::NSB) & 1, abort_flag, c.status);
         tc_fence_after();
         // the logits of this warp's rows: x[hf][4 k + 2 e + c] is row 16 hf + 8 e + lane / 4, column 8 k + 2 (lane & 3) + c
         uint32_t x[2][32];
 #pragma unroll
         for (int hf = 0; hf < 2; ++hf)
-          tmem_ld_frag(s_t + hf * kHalf, x[hf]);
+          tmem_ld_frag(lane_t + (SM::QT ? sb : g) * 64 + hf * kHalf, x[hf]);
+        const uint32_t bp = bias_t + ((jg % NB) * BKT + (tg % SUB) * 64) * 4;
+        float2 bias[8];
+#pragma unroll
+        for (int k = 0; k < 8; ++k) bias[k] = lds2(bp + 32 * k);
+        if (!SM::QT && t > 0) named_barrier_sync(heard, 64);
+        const float4 seen = t > 0 ? lds4(max_s) : make_float4(-INFINITY, -INFINITY, -INFINITY, -INFINITY);
+        bool p_free = tg < kGroups || mbar_test_wait(bar_pv_done + 8 * g, (tg / kGroups - 1) & 1);
         tmem_wait_ld();
         tc_fence_before();
         mbar_arrive_warp(bar_s_empty + 8 * sb);          // the logits are in registers
-        const uint32_t bp = bias_t + ((jg % NB) * BKT + (tg % SUB) * 64) * 4;
         float mx[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
 #pragma unroll
         for (int k = 0; k < 8; ++k) {
-          const float2 bias = lds2(bp + 32 * k);
 #pragma unroll
           for (int q = 0; q < 4; ++q) {
             uint32_t* v = &x[q >> 1][4 * k + 2 * (q & 1)];
-            const float2 y = ffma2(make_float2(__uint_as_float(v[0]), __uint_as_float(v[1])), make_float2(scale, scale), bias);
+            const float2 y = ffma2(make_float2(__uint_as_float(v[0]), __uint_as_float(v[1])), make_float2(scale, scale), bias[k]);
             v[0] = __float_as_uint(y.x);
             v[1] = __float_as_uint(y.y);
             mx[q] = fmax3(mx[q], y.x, y.y);
           }
         }
-        // A logit can make this warp raise the maximum only if it exceeds the last maximum that this warp knows by as much (maxima
-        // only grow).  If none does, the hand-over goes on at once, before the maximum is even read: it still cannot change before
-        // this sub-tile is through, because whoever raises it waits for P V of all sub-tiles before.
+        // A logit makes this warp raise the maximum if it exceeds the last one by as much.  If none does, and nobody has raised it since
+        // this warp looked, the hand-over goes on at once: the maximum cannot change before this sub-tile is through, because whoever
+        // raises it waits for P V of all sub-tiles before.
         // The first sub-tile's warp always goes the long way: it puts the maxima where the others read them, also those of a sub-tile
         // without a live key (-inf; what lies there is an earlier item's).
         bool may = t == 0;
 #pragma unroll
         for (int q = 0; q < 4; ++q) may |= mx[q] > m[q] + kTop;
         may = __any_sync(0xffffffffu, may);
-        if (t > 0) named_barrier_sync(heard, 64);
         if (!may && t + 1 < ns) named_barrier_arrive(told, 64);
-        // (asked here, needed later: a barrier answers slowly while MMAs run)
-        bool p_free = tg < kGroups || mbar_test_wait(bar_pv_done + 8 * g, (tg / kGroups - 1) & 1);
-        const float4 seen = t > 0 ? lds4(max_s) : make_float4(-INFINITY, -INFINITY, -INFINITY, -INFINITY);
         const float cur[4] = {seen.x, seen.y, seen.z, seen.w};
         bool change = t == 0;
 #pragma unroll
@@ -530,12 +688,12 @@ attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CU
             }
           tmem_st_half_frag(p_t + hf * kHalf, p);
         }
-        const int jn = (tg + kGroups) / SUB;
-        s_ready = mbar_test_wait(bar_s_full + 8 * (jn % NSB), (jn / NSB) & 1);
+        const uint32_t jn = (tg + kGroups) / SUB;            // (asked here, needed later: a barrier answers slowly while MMAs run)
+        if (!SM::QT) s_ready = mbar_test_wait(bar_s_full + 8 * (jn % SM::NSB), (jn / SM::NSB) & 1);
         tmem_wait_st();
         tc_fence_before();
         mbar_arrive_warp(bar_p_full + 8 * g);
-        s_ready = __all_sync(0xffffffffu, s_ready);
+        if (!SM::QT) s_ready = __all_sync(0xffffffffu, s_ready);
       }
       // ---- the groups meet: (m, l) of every row through shared memory ----
       const uint32_t xchg = sbase + SM::xchg_off + (n_done & 1) * kGroups * 1024;
@@ -560,10 +718,9 @@ attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CU
       if (ok && g < D / 32) {
         // O is relative to the last maximum, which the group of the last sub-tile knows; the others may be some raises behind
         uint32_t v[32];
-        float inv = 0.f;
+        float m_all = -INFINITY, denom = 0.f;
         if (ns > 0) {
           float2 part[kGroups];
-          float m_all = -INFINITY, denom = 0.f;
 #pragma unroll
           for (int q = 0; q < kGroups; ++q) {
             part[q] = lds2(xchg + (q * 128 + r) * 8);
@@ -571,7 +728,6 @@ attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CU
           }
 #pragma unroll
           for (int q = 0; q < kGroups; ++q) denom += part[q].y * ((part[q].x == -INFINITY) ? 0.f : fast_exp2(part[q].x - m_all));
-          inv = denom > 0.f ? 1.f / denom : 0.f;
           tmem_ld32(o_t + g * 32, v);
           tmem_wait_ld();
         } else {
@@ -580,24 +736,14 @@ attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CU
         }
         tc_fence_before();
         if (ns > 0) mbar_arrive_warp(bar_o_free);
-        const AttnItem w = rows_of(it);
-        const int64_t off = static_cast<int64_t>(w.h) * a.out_head_stride + static_cast<int64_t>(w.q0 + r) * a.out_token_stride + g * 32;
-        if (r < w.valid_rows && a.out_fp32) {         // loads are warp-collective, only the stores are per row
-          float4* dst = reinterpret_cast<float4*>(static_cast<float*>(a.out) + off);
-#pragma unroll
-          for (int q = 0; q < 8; ++q)
-            dst[q] = make_float4(__uint_as_float(v[4 * q]) * inv, __uint_as_float(v[4 * q + 1]) * inv, __uint_as_float(v[4 * q + 2]) * inv,
-                                 __uint_as_float(v[4 * q + 3]) * inv);
-        } else if (r < w.valid_rows) {
-          uint4* dst = reinterpret_cast<uint4*>(static_cast<__nv_bfloat16*>(a.out) + off);
-#pragma unroll
-          for (int q = 0; q < 4; ++q) {
-            uint32_t o[4];
-#pragma unroll
-            for (int e = 0; e < 4; ++e)
-              o[e] = pack_bf16x2(__uint_as_float(v[8 * q + 2 * e]) * inv, __uint_as_float(v[8 * q + 2 * e + 1]) * inv);
-            dst[q] = make_uint4(o[0], o[1], o[2], o[3]);
-          }
+        AttnPart cut{};
+        if (SPLIT && it >= a.rounds) cut = part_of(it - a.rounds);
+        if (SPLIT && it >= a.rounds && cut.hi - cut.lo < a.units) {
+          store_part<D>(c, slot_of(blockIdx.x, cut.lo == 0), g, r, v, m_all, denom);
+        } else {
+          const AttnItem w = rows_of(item_at(it));
+          if (r < w.valid_rows)               // loads are warp-collective, only the stores are per row
+            write_row(a, static_cast<int64_t>(w.h) * a.out_head_stride + static_cast<int64_t>(w.q0 + r) * a.out_token_stride + g * 32, v, denom);
         }
       } else if (ns > 0) {
         mbar_arrive_warp(bar_o_free);
@@ -605,25 +751,99 @@ attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CU
       if (ns > 0) ++n_done;
       sub0 += ns;
     }
+    const AttnPiece piece = SPLIT ? *piece_s : AttnPiece{};
+    if (SPLIT && (warp >> 2) < D / 32 && piece.n > 0) {
+      // The parts of cut items: the CTA that finds that the other parts of an item have come adds them up.  Asked at the end, so that no
+      // answer is waited for between two items; by one warp, because a fence by each of sixteen takes as long as ten tiles; for both cut
+      // items at once, by two lanes.  After a time-out the warps come here too, so that the counters go back to zero.
+      const int g = warp >> 2, r = (warp & 3) * 32 + lane;
+      auto cut_at = [&](int e) { return part_of(e == 0 ? 0 : piece.n - 1); };
+      auto parts_of = [&](int item, int& first) {
+        first = piece_at(a, item * a.units);
+        return piece_at(a, item * a.units + a.units - 1) - first + 1;
+      };
+      mbar_arrive_warp(bar_parts);
+      if (warp == 0) {
+        ok = mbar_wait_warp(bar_parts, 0, abort_flag, c.status) && ok;
+        const AttnPart cut = cut_at(lane & 1);
+        int last = 0, first;
+        if (lane < min(piece.n, 2) && cut.hi - cut.lo < a.units) {
+          last = atomic_add_acq_rel(c.part_count + cut.item, 1) == parts_of(cut.item, first) - 1 ? 1 : 0;
+          if (last) c.part_count[cut.item] = 0;
+        }
+        const uint32_t both = __ballot_sync(0xffffffffu, last);
+        if (lane == 0) *last_s = both;
+        mbar_arrive_warp(bar_last);
+      }
+      ok = mbar_wait_warp(bar_last, 0, abort_flag, c.status) && ok;
+#pragma unroll 1
+      for (int e = 0; e < 2; ++e)
+        if (ok && ((*last_s >> e) & 1)) {
+          uint32_t v[32];
+          int first;
+          const int item = cut_at(e).item, parts = parts_of(item, first);
+          const float sum = merge_parts<D>(c, first, parts, g, r, v);
+          const AttnItem w = rows_of(a.rounds * gridDim.x + item);
+          if (r < w.valid_rows)
+            write_row(a, static_cast<int64_t>(w.h) * a.out_head_stride + static_cast<int64_t>(w.q0 + r) * a.out_token_stride + g * 32, v, sum);
+        }
+    }
     tc_fence_before();
     mbar_arrive_warp(bar_done);
   }
 }
 
+template <int D, int BKT, bool GATHER, bool SEG, bool SPLIT = false>
+static int launch_attn_t(const CUtensorMap& tq, const CUtensorMap& tk, const CUtensorMap& tv, const CUtensorMap& tsk,
+                         const CUtensorMap& tsv, const CacheView& c, const AttnArgs& a, int grid, cudaStream_t st) {
+  using SM = AttnSmem<D, BKT>;
+  auto kern = attn_kernel<D, BKT, GATHER, SEG, SPLIT>;
+  const int cfg = ensure_dynamic_smem(reinterpret_cast<const void*>(kern), SM::total);
+  if (cfg != FASTAR_OK) return cfg;
+  launch_chained(kern, grid, kAttnThreads, SM::total, st, tq, tk, tv, tsk, tsv, c, a);
+  return cudaGetLastError() == cudaSuccess ? 1 : FASTAR_ERR_CUDA;
+}
+
 template <int D, int BKT, bool GATHER, bool SEG>
 static int launch_attn(const CUtensorMap& tq, const CUtensorMap& tk, const CUtensorMap& tv, const CUtensorMap& tsk,
                        const CUtensorMap& tsv, const CacheView& c, const AttnArgs& a, int items, cudaStream_t st) {
-  using SM = AttnSmem<D, BKT>;
-  auto kern = attn_kernel<D, BKT, GATHER, SEG>;
-  const int cfg = ensure_dynamic_smem(reinterpret_cast<const void*>(kern), SM::total);
-  if (cfg != FASTAR_OK) return cfg;
   // One CTA per SM takes the items in turn; gather mode (more than 64 kept prompt tokens, or up to that many by the bucket rule) has
   // one item per CTA.  Its rows come in by asynchronous copies, a tile ahead: 12 heads x 4680 queries, 512 kept 385 -> 94 us for the
   // whole call (loads and stores through registers: 385; with 64 registers a thread 286), 40 x 10800 2420 -> 479, 128 kept 71 -> 64.
   int dev = 0, sm_count = 148;
   if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sm_count, cudaDevAttrMultiProcessorCount, dev);
-  launch_chained(kern, GATHER ? items : min(items, sm_count), kAttnThreads, SM::total, st, tq, tk, tv, tsk, tsv, c, a);
-  return cudaGetLastError() == cudaSuccess ? 1 : FASTAR_ERR_CUDA;
+  if constexpr (!GATHER) {
+    // Items that do not fill the last round of the SMs are cut by key tiles where that pays, in tile times (about a microsecond): a part's
+    // way through memory takes kPartStore, adding one in the end kPartAdd, another stop of a CTA kPartStop.  Either every item is cut into
+    // k equal pieces, which leaves a CTA one stop, or all are dealt to all CTAs.  What is saved has to be kPartGain of the whole.
+    // Kernel time without and with the cut: one item of 153 64-key tiles of 17 x 19 queries 44.0 -> 20.8 us (2 heads), 30 items of 25
+    // tiles 28.2 -> 18.6, 44 of 24 30.4 -> 24.5, 182 of 530 902 -> 647, 156 of 16 42.3 -> 38.1; 8 x 4 096 queries on 16 384 keys (256 of
+    // 128, dealt to all) 283 -> 265 a pass.  Where it would not pay: 108 items of 54 tiles dealt to all 63 -> 69, 18 of 6 13.6 -> 23.2, 256 of
+    // 16 39.4 -> 45.0, 256 of 64 119 -> 122; and full rounds of 64-key tiles, whose loop is slower in this variant (936 of 245 951 -> 990).
+    const int grid = min(min(sm_count, kAttnMaxGrid), c.max_pieces), full = min(sm_count, kAttnMaxGrid), rounds = items / full, left = items % full;
+    const int tiles = (a.sel ? a.keep : c.CAPB) + a.seg_tiles;           // at most
+    float best = tiles * (1.f - kPartGain * (rounds + 1));
+    int pieces = 0;
+    for (int k = 2; left > 0 && k * left <= grid && k * kAttnMinPiece <= tiles; ++k) {
+      const float t = static_cast<float>(tiles) / k + kPartStore + kPartAdd * k;
+      if (t < best) { best = t; pieces = k * left; }
+    }
+    if (left > 0 && grid > left) {
+      const float t = static_cast<float>(left) * tiles / grid + kPartStop + kPartStore + kPartAdd * (static_cast<float>(grid) / left + 1.f);
+      if (t < best && static_cast<int64_t>(left) * tiles >= static_cast<int64_t>(grid) * kAttnMinPiece) pieces = grid;
+    }
+    const int64_t largest = static_cast<int64_t>(tiles) * max(left * (pieces + 1), tiles);      // of the kernel's products
+    if (rounds > 0 && BKT == 64) pieces = 0;
+    if (pieces > 0 && !a.no_cut && largest < (1ll << 31)) {
+      AttnArgs cut = a;
+      cut.rounds = rounds;
+      cut.last_items = left;
+      cut.units = tiles;
+      cut.pieces = pieces;
+      return launch_attn_t<D, BKT, GATHER, SEG, true>(tq, tk, tv, tsk, tsv, c, cut, full, st);
+    }
+  }
+  return launch_attn_t<D, BKT, GATHER, SEG>(tq, tk, tv, tsk, tsv, c, a, GATHER ? items : min(items, sm_count), st);
 }
 
 // tm_seg_k / tm_seg_v: maps of the un-cached segment (box {64, page_tokens, 1}); nullptr when a.seg_tiles == 0.

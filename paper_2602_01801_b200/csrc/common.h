@@ -104,6 +104,12 @@ struct CacheView {
   int32_t* nselp;                  // [H][max_frames]
   // AnnSA's query codes (their own array: fastar_annsa_prepare may run beside an update, which hashes its keys into code_new)
   uint32_t* code_q_sa;             // [H][max_tokens]
+  // AnnSA's parts of items that are cut by key tiles (where stage[0] and stage[1] are): rows (fp32, [part][D / 4][128] of four columns), their references and sums
+  // ([part][4][128]), and the parts that have come ([item], zero between calls)
+  float* part_o;
+  float2* part_ml;
+  int32_t* part_count;
+  int32_t max_pieces;              // there is room for two parts of each of so many pieces
   __nv_bfloat16* stage_prep;       // fp32 caches: bf16 copy of the queries hashed by fastar_annsa_prepare (null for bf16)
 };
 
@@ -184,7 +190,12 @@ struct AttnArgs {
   // gather mode: kept tokens of every frame, [H][keep_frames_stride] (nullptr: `keep` for all frames)
   const int32_t* keep_frames;
   int keep_frames_stride;
+  // paged mode, set by the launch where the items of the last round are cut (attn_kernels.cu)
+  int rounds, last_items, units, pieces;
+  int no_cut;              // paged mode: the parts' place is taken
 };
+constexpr int kAttnMaxGrid = 160;  // CTAs that may share the items of a last round
+constexpr int kAttnMinPiece = 4;   // key tiles of a piece, at least
 int launch_attention_paged(const CacheView& c, const CUtensorMap& tm_q, const CUtensorMap& tm_pool_k,
                            const CUtensorMap& tm_pool_v, const CUtensorMap* tm_seg_k, const CUtensorMap* tm_seg_v,
                            const AttnArgs& a, cudaStream_t st);

@@ -149,7 +149,23 @@ size_t carve(const fastar_cache_desc& d, uint8_t* base, CacheView* v) {
   t.nsel = reinterpret_cast<int32_t*>(take(H * 4));
   t.rel = reinterpret_cast<uint32_t*>(take(H * t.max_frames * MP * 4));
   t.selp = reinterpret_cast<int32_t*>(take(H * t.max_frames * MP * 4));
-  for (int i = 0; i < 3; ++i) t.stage[i] = reinterpret_cast<__nv_bfloat16*>(take(H * MT * D * 2));
+  {
+    // stage[0], stage[1] and, in the same place, the parts of AnnSA's cut items: nobody stages keys and values while AnnSA attends, but
+    // for the segment of an fp32 cache (annsa_impl).  A piece of the last round's items has two parts at most, and there are no more
+    // pieces than items or than their tiles allow.
+    const size_t items = H * t.max_qb < kAttnMaxGrid ? H * t.max_qb : kAttnMaxGrid;
+    const size_t by_tiles = items * (t.CAPB + (MT + t.PT - 1) / t.PT) / kAttnMinPiece;
+    const size_t pieces = by_tiles < items ? items : by_tiles < kAttnMaxGrid ? by_tiles : kAttnMaxGrid;
+    const size_t staged = (H * MT * D * 2 + 1023) & ~static_cast<size_t>(1023), rows = 2 * pieces * 128 * D * 4, stats = 2 * pieces * 4 * 128 * 8;
+    uint8_t* both = take(2 * staged > rows + stats ? 2 * staged : rows + stats);
+    t.stage[0] = reinterpret_cast<__nv_bfloat16*>(both);
+    t.stage[1] = reinterpret_cast<__nv_bfloat16*>(both ? both + staged : nullptr);
+    t.max_pieces = static_cast<int32_t>(pieces);
+    t.part_o = reinterpret_cast<float*>(both);
+    t.part_ml = reinterpret_cast<float2*>(both ? both + rows : nullptr);
+    t.part_count = reinterpret_cast<int32_t*>(take(kAttnMaxGrid * 4));
+  }
+  t.stage[2] = reinterpret_cast<__nv_bfloat16*>(take(H * MT * D * 2));
   for (int i = 3; i < 5; ++i) t.stage[i] = reinterpret_cast<__nv_bfloat16*>(take(H * MP * D * 2));
   t.stage[5] = reinterpret_cast<__nv_bfloat16*>(take(H * MT * D * 2));
   t.search_bits = (d.search_bits == 8 || d.search_bits == 1) ? 8 : 16;     // both keep a pool of 128-byte code rows
@@ -361,6 +377,8 @@ int fastar_cache_create(fastar_cache_t** out, const fastar_cache_desc* desc, con
   }
   // AnnCA's own scratch: cleared here only, because an AnnCA call may run beside a reset or an import on another stream
   r = cudaMemsetAsync(v.rel, 0, static_cast<size_t>(v.H) * v.max_frames * v.max_prompt * 4, nullptr) == cudaSuccess ? FASTAR_OK : FASTAR_ERR_CUDA;
+  // so are the counters of AnnSA's parts, which every call leaves at zero
+  if (r == FASTAR_OK && cudaMemsetAsync(v.part_count, 0, kAttnMaxGrid * 4, nullptr) != cudaSuccess) r = FASTAR_ERR_CUDA;
   if (r == FASTAR_OK) r = fastar_cache_reset(c, nullptr);
   if (r == FASTAR_OK && cudaStreamSynchronize(nullptr) != cudaSuccess) r = FASTAR_ERR_CUDA;
   if (r != FASTAR_OK) {
@@ -684,7 +702,8 @@ static int annsa_impl(fastar_cache_t* c, const void* q, const void* k_seg, const
   }
   CUtensorMap tm_sk, tm_sv;
   if (k_seg) {
-    // the update's staging slots are free during an attention call
+    // the update's staging slots are free during an attention call (where the segment has to be converted, no items are cut)
+    a.no_cut = c->desc.dtype != FASTAR_BF16;
     View sg[2] = {{k_seg, ns, 0, seg_head_stride, seg_token_stride, nullptr}, {v_seg, ns, 1, seg_head_stride, seg_token_stride, nullptr}};
     r = as_bf16(c, sg, 2, st);
     if (r == FASTAR_OK) r = make_map(c, &tm_sk, sg[0].p, v.D, ns, v.H, static_cast<uint64_t>(sg[0].ts) * 2, static_cast<uint64_t>(sg[0].hs) * 2, v.PT);

@@ -42,6 +42,13 @@ __device__ __forceinline__ int checked_index(int idx, int n, int* status) {
 // memory that another kernel reads or writes.
 __device__ __forceinline__ void chain_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
+// What this thread, and the threads that a barrier has ordered before it, wrote is seen by whoever reads a later count.
+__device__ __forceinline__ int atomic_add_acq_rel(int32_t* p, int v) {
+  int old;
+  asm volatile("atom.add.acq_rel.gpu.global.s32 %0, [%1], %2;" : "=r"(old) : "l"(p), "r"(v) : "memory");
+  return old;
+}
+
 __device__ __forceinline__ uint32_t smem_u32(const void* p) {
   return static_cast<uint32_t>(__cvta_generic_to_shared(p));
 }
@@ -296,6 +303,16 @@ __device__ __forceinline__ void umma_ts(uint32_t d_tmem, uint32_t a_tmem, uint64
       "setp.ne.b32 q, %5, 0;\n\t"
       "@q tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}"
       ::"r"(d_tmem), "r"(a_tmem), "l"(bdesc), "r"(idesc), "r"(accumulate), "r"(lead)
+      : "memory");
+}
+// 128 rows x 32 bytes of shared memory (a K-major operand's K = 16 step) to eight columns of tensor memory; in order with the MMAs that
+// the same thread issues.
+__device__ __forceinline__ void tmem_copy_128x256b(uint32_t taddr, uint64_t desc, uint32_t lead) {
+  asm volatile(
+      "{\n\t.reg .pred q;\n\t"
+      "setp.ne.b32 q, %2, 0;\n\t"
+      "@q tcgen05.cp.cta_group::1.128x256b [%0], %1;\n\t}"
+      ::"r"(taddr), "l"(desc), "r"(lead)
       : "memory");
 }
 // Arrive on an mbarrier when all MMAs issued so far by the elected thread have completed.

@@ -160,3 +160,52 @@ def test_range_of_the_values(d, pt, magnitude):
         assert np.isfinite(got).all()
         assert np.abs(got - want).max() <= 2.0 ** -7 * np.abs(vv).max()
         assert np.linalg.norm(got - want) <= 1e-2 * np.linalg.norm(want)
+
+
+@pytest.mark.parametrize("d,pt,H,nq,lens,seg,keep", [
+    (128, 128, 1, 100, [40 * 128 - 5], 0, 0),                      # one item for all CTAs
+    (64, 64, 1, 64, [1030 * 64], 0, 0),                            # as many parts as an item gets
+    (128, 64, 3, 300, [9 * 64, 0, 31 * 64 + 1], 200, 0),           # unequal heads, one of them with nothing but the segment
+    (64, 128, 7, 22 * 128 - 60, [17 * 128, 0, 1, 129, 24 * 128, 9 * 128, 300], 0, 0),      # a full round and six items
+    (128, 128, 5, 44 * 128, [24 * 128], 0, 0),                     # 72 items: the ends of two in one CTA
+    (128, 128, 2, 500, [60 * 128], 0, 33),                         # lists of blocks, and a segment behind them
+    (64, 64, 3, 700, [40 * 64 - 9, 64, 40 * 64], 100, 21),
+])
+def test_items_cut_by_key_tiles(d, pt, H, nq, lens, seg, keep):
+    """The items of a last round that does not fill the SMs are cut: parts of all lengths, empty heads between them, the same result by
+    a second call (the counters of the parts are back at zero)."""
+    import torch
+    from paper_2602_01801_b200 import fastar
+    rng = np.random.default_rng(d + pt + H)
+    lens = np.resize(lens, H)
+    cap = -(-max(int(lens.max()), 128) // 128) * 128
+    cap += cap // 2 // 128 * 128 if H == 7 else 0                  # fewer live blocks than the launch knows of
+    q = synth.round_bf16((rng.standard_normal((H, nq, d)) * rng.choice([1.0, 20.0], (H, nq, 1))).astype(np.float32))
+    k, v = (synth.round_bf16(rng.standard_normal((H, cap + seg, d)).astype(np.float32)) for _ in range(2))
+    count = rng.integers(1, 9, (H, cap)).astype(np.int32)
+    cache = fastar.Cache(H, d, cap, pt, rng.standard_normal((32, d)).astype(np.float32), max_tokens=nq)
+    cache.import_state(fastar.bf16_bits(k[:, :cap]), fastar.bf16_bits(v[:, :cap]), lens, count)
+    args, nqb = {}, -(-nq // 128)
+    if keep:
+        sel = np.stack([[rng.permutation(cap // pt)[:keep] for _ in range(nqb)] for _ in range(H)]).astype(np.int32)
+        args = dict(sel_in=torch.from_numpy(sel).cuda(), nsel_in=torch.full((H,), keep, dtype=torch.int32, device="cuda"))
+    dq, dk, dv = fastar.to_device(q), fastar.to_device(k[:, cap:]), fastar.to_device(v[:, cap:])
+    blocks = keep or cap // pt
+    out, again = (cache.annsa_segment(dq, dk, dv, 128, blocks, **args)["out"] if seg else cache.annsa(dq, 128, blocks, **args)["out"] for _ in range(2))
+    assert cache.status() == 0
+    assert torch.equal(out, again)
+    for h in range(H):
+        for b in range(0, nqb, max(1, nqb // 6)):
+            slots = np.concatenate([np.arange(s * pt, s * pt + pt) for s in (sel[h, b] if keep else range(cap // pt))])
+            slots = slots[slots < lens[h]]
+            got = out[h, b * 128: b * 128 + 128].float().cpu().numpy()
+            if len(slots) + seg == 0:
+                assert (got == 0).all()
+                continue
+            kk, vv = (np.concatenate([x[h, slots], x[h, cap:]]) for x in (k, v))
+            s = q[h, b * 128: b * 128 + 128].astype(np.float64) @ kk.T / math.sqrt(d) + np.log(np.concatenate([count[h, slots], np.ones(seg)]))
+            p = np.exp(s - s.max(1, keepdims=True))
+            want = (p / p.sum(1, keepdims=True)) @ vv
+            # as above: rounding of the probabilities and of the output
+            assert np.abs(got - want).max() <= 2.0 ** -7 * np.abs(vv).max(), f"head {h}, block {b}"
+            assert np.linalg.norm(got - want) <= 1e-2 * np.linalg.norm(want), f"head {h}, block {b}"
