@@ -220,8 +220,7 @@ struct ConvertArgs {
   int count;
 };
 int launch_convert_f32_to_bf16(const ConvertArgs& a, int H, int D, cudaStream_t st);
-int launch_prep_codes(const CacheView& c, const __nv_bfloat16* x, int n, int64_t hs, int64_t ts, uint32_t* code_out,
-                      float* rnorm_out, cudaStream_t st);
+int launch_query_blocks(const CacheView& c, const __nv_bfloat16* q, int nq, int64_t hs, int64_t ts, int block_q, cudaStream_t st);
 int launch_prep_update(const CacheView& c, const __nv_bfloat16* k_new, int n, int64_t hs, int64_t ts, cudaStream_t st);
 int launch_prep_codes_strided(const CacheView& c, const __nv_bfloat16* x, int n, int64_t hs, int64_t ts, uint32_t* code_out,
                               int64_t out_stride, cudaStream_t st);
@@ -231,7 +230,6 @@ int launch_plan(const CacheView& c, int n, float tau, const UpdateOut& out, cuda
 int launch_commit(const CacheView& c, const __nv_bfloat16* k_new, const __nv_bfloat16* v_new, int n, int frame_len,
                   int64_t hs, int64_t ts, cudaStream_t st);
 int launch_finalize_hist(const CacheView& c, fastar_update_stats* stats_out, int advance_clock, cudaStream_t st);
-int launch_query_hist(const CacheView& c, const uint32_t* codes, int nq, int block_q, cudaStream_t st);
 int launch_topk_blocks(const CacheView& c, int nqb, int keep, int force_sink, int force_recent, cudaStream_t st);
 int launch_topk_prompt(const CacheView& c, int n_frames, int np, int keep, cudaStream_t st);
 int launch_reset(const CacheView& c, cudaStream_t st);

@@ -664,8 +664,7 @@ static int annsa_impl(fastar_cache_t* c, const void* q, const void* k_seg, const
                           c->prep.hs == head_stride && c->prep.ts == token_stride;
     c->prep.valid = false;
     if (!prepared) {
-      ACCK(FASTAR_K_HASH, launch_prep_codes(v, qb, nq, qhs, qts, v.code_q_sa, nullptr, st));
-      ACCK(FASTAR_K_QUERY_HIST, launch_query_hist(v, v.code_q_sa, nq, block_q, st));
+      ACCK(FASTAR_K_HASH, launch_query_blocks(v, qb, nq, qhs, qts, block_q, st));
     }
     ACCK(FASTAR_K_S3_SCORES, launch_s3_scores(v, c->tm_hq, c->tm_hk, nqb, st));
     if (v.hist_weighted) {                   // the high digits of the weighted histograms, into their own score array
@@ -741,8 +740,7 @@ int fastar_annsa_prepare(fastar_cache_t* c, const void* q, int32_t nq, int64_t h
     qhs = static_cast<int64_t>(nq) * v.D;
     qts = v.D;
   }
-  ACCK(FASTAR_K_HASH, launch_prep_codes(v, qb, nq, qhs, qts, v.code_q_sa, nullptr, st));
-  ACCK(FASTAR_K_QUERY_HIST, launch_query_hist(v, v.code_q_sa, nq, block_q, st));
+  ACCK(FASTAR_K_HASH, launch_query_blocks(v, qb, nq, qhs, qts, block_q, st));
   c->prep.q = q; c->prep.nq = nq; c->prep.block_q = block_q; c->prep.hs = head_stride; c->prep.ts = token_stride;
   c->prep.valid = true;
   return FASTAR_OK;

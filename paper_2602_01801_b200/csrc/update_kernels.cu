@@ -90,6 +90,18 @@ int launch_convert_f32_to_bf16(const ConvertArgs& a, int H, int D, cudaStream_t 
   return cudaGetLastError() == cudaSuccess ? 1 : FASTAR_ERR_CUDA;
 }
 
+// Eight counters as bf16: all of them (SHIFT < 0: exact up to 256), or one of their two 8-bit digits.
+template <int SHIFT>
+__device__ __forceinline__ uint4 pack_counts(const int (&v)[8]) {
+  uint32_t w[4];
+#pragma unroll
+  for (int e = 0; e < 4; ++e) {
+    const int lo = SHIFT < 0 ? v[2 * e] : (v[2 * e] >> (SHIFT < 0 ? 0 : SHIFT)) & 255, hi = SHIFT < 0 ? v[2 * e + 1] : (v[2 * e + 1] >> (SHIFT < 0 ? 0 : SHIFT)) & 255;
+    w[e] = pack_bf16x2(static_cast<float>(lo), static_cast<float>(hi));
+  }
+  return make_uint4(w[0], w[1], w[2], w[3]);
+}
+
 // ---------------------------------------------------------------------------------------------
 // S1: codes (and reciprocal norms).
 // ---------------------------------------------------------------------------------------------
@@ -99,11 +111,18 @@ int launch_convert_f32_to_bf16(const ConvertArgs& a, int H, int D, cudaStream_t 
 // 17 us at the measured bandwidth: 48 -> 39 us; 12 x 4680 9.9 -> 8.9).  Fragment layout (g = lane / 4, t = lane % 4):
 //   A: a0 = X[g][2t..], a1 = X[g+8][2t..], a2 = X[g][2t+8..], a3 = X[g+8][2t+8..]   (bf16 pairs)
 //   B: b0 = R[n = 8*nt + g][2t..], b1 = R[n][2t+8..];   C: c0,c1 = row g, cols 2t,2t+1;  c2,c3 = row g+8.
-template <int D>
-__global__ void __launch_bounds__(256) prep_kernel(const __nv_bfloat16* __restrict__ x, int H, int n, int64_t hs, int64_t ts,
+// BLOCKS (the query side of S2 in the same launch: 12 x 4680 rows 9.2 + 2.7 -> 10.2 us, 2 x 600 4.1 + 2.3 -> 4.4): a CTA's warps take the
+// 16-row groups of one block of block_rows rows (64 or 128), and the CTA writes the block's bucket histogram.
+struct BlockHist {
+  __nv_bfloat16* hist;         // [H][max_qb][hist_cols]
+  int block_rows, max_qb, hist_cols;
+};
+template <int D, bool BLOCKS>
+__global__ void __launch_bounds__(256, 2) prep_kernel(const __nv_bfloat16* __restrict__ x, int H, int n, int64_t hs, int64_t ts,
                                                    const __nv_bfloat16* __restrict__ lsh, int T, int B,
                                                    uint32_t* __restrict__ code_out, float* __restrict__ rnorm_out,
-                                                   int64_t out_stride, uint4* __restrict__ zero, int64_t zero16) {
+                                                   int64_t out_stride, uint4* __restrict__ zero, int64_t zero16, BlockHist bh) {
+  __shared__ __align__(16) int hist[BLOCKS ? 1024 : 4];
   chain_wait();
   for (int64_t q = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; q < zero16; q += static_cast<int64_t>(gridDim.x) * blockDim.x)
     zero[q] = make_uint4(0, 0, 0, 0);
@@ -134,8 +153,13 @@ __global__ void __launch_bounds__(256) prep_kernel(const __nv_bfloat16* __restri
       bf[ks][nt][1] = *reinterpret_cast<const uint32_t*>(rp + 2);
     }
   // 16-row groups of all heads, dealt to the warps of a grid that fills the SMs once
-  const int groups_per_head = (n + 15) / 16;
+  // BLOCKS: groups are numbered through whole blocks, so that a CTA's eight warps have the groups of one block, or of two of 64 rows of
+  // which the second waits for the CTA's next pass
+  const int per_block = BLOCKS ? bh.block_rows / 16 : 1;
+  const int groups_per_head = BLOCKS ? (n + bh.block_rows - 1) / bh.block_rows * per_block : (n + 15) / 16;
   const int total_groups = groups_per_head * H;
+  const int stride = BLOCKS ? static_cast<int>(gridDim.x) * per_block : static_cast<int>(gridDim.x) * 8;
+  const bool idle = BLOCKS && warp >= per_block;         // 64-row blocks: four warps have rows
   uint4 va[KS / 2], vb[KS / 2];
   const __nv_bfloat16 *xa = x, *xb = x;                                // this lane's rows of the group that is fetched
   auto rows = [&](int grp) {
@@ -148,17 +172,22 @@ __global__ void __launch_bounds__(256) prep_kernel(const __nv_bfloat16* __restri
     va[kk] = *reinterpret_cast<const uint4*>(xa + 32 * kk);
     vb[kk] = *reinterpret_cast<const uint4*>(xb + 32 * kk);
   };
-  const int first = blockIdx.x * 8 + warp;
-  if (first < total_groups) {
+  const int first = BLOCKS ? blockIdx.x * per_block + (idle ? 0 : warp) : blockIdx.x * 8 + warp;
+  if (first < total_groups && !idle) {
     rows(first);
 #pragma unroll
     for (int kk = 0; kk < KS / 2; ++kk) fetch(kk);
   }
-  for (int grp = first; grp < total_groups; grp += gridDim.x * 8) {
+  for (int grp = first; grp < total_groups; grp += stride) {
     const int h = grp / groups_per_head;
     const int r0 = (grp - h * groups_per_head) * 16;
-    const bool more = grp + static_cast<int>(gridDim.x) * 8 < total_groups;
-    if (more) rows(grp + gridDim.x * 8);
+    const bool more = grp + stride < total_groups && !idle;
+    if (more) rows(grp + stride);
+    if (BLOCKS) {
+      reinterpret_cast<int4*>(hist)[threadIdx.x] = make_int4(0, 0, 0, 0);
+      __syncthreads();
+    }
+    if (!idle) {
     float acc[4][4];
 #pragma unroll
     for (int nt = 0; nt < 4; ++nt)
@@ -202,12 +231,17 @@ __global__ void __launch_bounds__(256) prep_kernel(const __nv_bfloat16* __restri
       sqa += __shfl_xor_sync(0xffffffffu, sqa, o);
       sqb += __shfl_xor_sync(0xffffffffu, sqb, o);
     }
-    if (t == 0) {
-      uint32_t ca = 0, cb = 0;
-      for (int tt = 0; tt < T; ++tt) {
-        ca |= ((ma >> (tt * B)) & ((1u << B) - 1u)) << (8 * tt);
-        cb |= ((mb >> (tt * B)) & ((1u << B) - 1u)) << (8 * tt);
+    uint32_t ca = 0, cb = 0;
+    for (int tt = 0; tt < T; ++tt) {
+      ca |= ((ma >> (tt * B)) & ((1u << B) - 1u)) << (8 * tt);
+      cb |= ((mb >> (tt * B)) & ((1u << B) - 1u)) << (8 * tt);
+    }
+    if (BLOCKS)                              // table t of rows g and g + 8
+      if (t < T) {
+        if (r0 + g < n) atomicAdd(&hist[(t << B) + ((ca >> (8 * t)) & 0xFFu)], 1);
+        if (r0 + g + 8 < n) atomicAdd(&hist[(t << B) + ((cb >> (8 * t)) & 0xFFu)], 1);
       }
+    if (t == 0) {
       if (r0 + g < n) {
         code_out[h * out_stride + r0 + g] = ca;
         if (rnorm_out) rnorm_out[h * out_stride + r0 + g] = sqa > 0.f ? 1.f / sqrtf(sqa) : 0.f;
@@ -216,6 +250,19 @@ __global__ void __launch_bounds__(256) prep_kernel(const __nv_bfloat16* __restri
         code_out[h * out_stride + r0 + g + 8] = cb;
         if (rnorm_out) rnorm_out[h * out_stride + r0 + g + 8] = sqb > 0.f ? 1.f / sqrtf(sqb) : 0.f;
       }
+    }
+    }
+    if (BLOCKS) {
+      __syncthreads();
+      const int blk = (grp - h * groups_per_head) / per_block;
+      uint4* dst = reinterpret_cast<uint4*>(bh.hist + (static_cast<int64_t>(h) * bh.max_qb + blk) * bh.hist_cols);
+      if (threadIdx.x < bh.hist_cols / 8) {
+        int v[8];
+#pragma unroll
+        for (int e = 0; e < 8; ++e) v[e] = hist[8 * threadIdx.x + e];
+        dst[threadIdx.x] = pack_counts<-1>(v);
+      }
+      __syncthreads();
     }
   }
 }
@@ -228,18 +275,28 @@ static int launch_prep_generic(const CacheView& c, const __nv_bfloat16* x, int n
   // the rows only, 50 with these).
   const int64_t want = max(static_cast<int64_t>(groups + 7) / 8, (zero16 + 2047) / 2048);
   const dim3 grid(static_cast<unsigned>(max(static_cast<int64_t>(1), min(want, static_cast<int64_t>(2 * 148)))));
-  if (c.D == 128) launch_chained(prep_kernel<128>, grid, 256, 0, st, x, c.H, n, hs, ts, c.lsh, c.T, c.B, code_out, rnorm_out, out_stride, zero, zero16);
-  else launch_chained(prep_kernel<64>, grid, 256, 0, st, x, c.H, n, hs, ts, c.lsh, c.T, c.B, code_out, rnorm_out, out_stride, zero, zero16);
+  if (c.D == 128) launch_chained(prep_kernel<128, false>, grid, 256, 0, st, x, c.H, n, hs, ts, c.lsh, c.T, c.B, code_out, rnorm_out, out_stride, zero, zero16, BlockHist{});
+  else launch_chained(prep_kernel<64, false>, grid, 256, 0, st, x, c.H, n, hs, ts, c.lsh, c.T, c.B, code_out, rnorm_out, out_stride, zero, zero16, BlockHist{});
   return cudaGetLastError() == cudaSuccess ? 1 : FASTAR_ERR_CUDA;
 }
-int launch_prep_codes(const CacheView& c, const __nv_bfloat16* x, int n, int64_t hs, int64_t ts, uint32_t* code_out,
-                      float* rnorm_out, cudaStream_t st) {
-  return launch_prep_generic(c, x, n, hs, ts, code_out, rnorm_out, c.max_tokens, st);
+// Codes of the queries and the bucket histograms of their blocks of block_q rows.
+int launch_query_blocks(const CacheView& c, const __nv_bfloat16* q, int nq, int64_t hs, int64_t ts, int block_q, cudaStream_t st) {
+  if (nq <= 0) return 0;
+  const int64_t blocks = static_cast<int64_t>((nq + block_q - 1) / block_q) * c.H;
+  const int grid = static_cast<int>(min(blocks, static_cast<int64_t>(2 * 148)));
+  const BlockHist bh{c.hq, block_q, c.max_qb, c.hist_cols};
+  if (c.D == 128) launch_chained(prep_kernel<128, true>, grid, 256, 0, st, q, c.H, nq, hs, ts, c.lsh, c.T, c.B, c.code_q_sa, nullptr, c.max_tokens, nullptr, 0, bh);
+  else launch_chained(prep_kernel<64, true>, grid, 256, 0, st, q, c.H, nq, hs, ts, c.lsh, c.T, c.B, c.code_q_sa, nullptr, c.max_tokens, nullptr, 0, bh);
+  return cudaGetLastError() == cudaSuccess ? 1 : FASTAR_ERR_CUDA;
 }
+bool plan_is_fused(const CacheView& c, int n);
+int plan_fused_smem(const CacheView& c, int n);
 // The first kernel of an update: codes and reciprocal norms of the new keys, and zeros in the words that the search and the
 // matching accumulate into (best, n_match and cnt lie side by side; a memset of its own cost 4 us with its two gaps).
 int launch_prep_update(const CacheView& c, const __nv_bfloat16* k_new, int n, int64_t hs, int64_t ts, cudaStream_t st) {
-  const int64_t bytes = reinterpret_cast<const uint8_t*>(c.cnt + static_cast<int64_t>(c.H) * c.CAP) - reinterpret_cast<const uint8_t*>(c.best);
+  const uint8_t* end = plan_is_fused(c, n) ? reinterpret_cast<const uint8_t*>(c.best + ((static_cast<int64_t>(c.H) * c.max_tokens + 1) & ~1ll))
+                                           : reinterpret_cast<const uint8_t*>(c.cnt + static_cast<int64_t>(c.H) * c.CAP);
+  const int64_t bytes = end - reinterpret_cast<const uint8_t*>(c.best);
   return launch_prep_generic(c, k_new, n, hs, ts, c.code_new, c.rnorm_new, c.max_tokens, st, reinterpret_cast<uint4*>(c.best), bytes / 16);
 }
 int launch_prep_codes_strided(const CacheView& c, const __nv_bfloat16* x, int n, int64_t hs, int64_t ts, uint32_t* code_out,
@@ -283,6 +340,136 @@ __global__ void __launch_bounds__(256) match_count_kernel(const CacheView c, int
     for (int o = 16; o > 0; o >>= 1) mine += __shfl_xor_sync(0xFFFFFFFFu, mine, o);
     if ((threadIdx.x & 31) == 0 && mine > 0) atomicAdd(c.n_match + h, mine);
   }
+}
+
+// Eviction.  evictable = live, past the sink prefix, stamp < now, not touched by this update.  The oldest E go, ties by slot; what is
+// looked for is the age (now - stamp) that at least E evictable slots reach, the greatest such.  False: there are fewer than E.
+// untouched(j, free): whether slots j .. j + 15 are matched by no token; keys: room for the victims, up to a power of two.
+template <class Untouched>
+__device__ __forceinline__ bool choose_victims(const CacheView& c, int h, int L, int now, int E, unsigned long long* keys, int* red,
+                                               int& evicted_tokens, const Untouched& untouched) {
+  const int tid = threadIdx.x;
+  const int64_t tb = static_cast<int64_t>(h) * c.max_tokens, sb = static_cast<int64_t>(h) * c.CAP;
+  bool ok = true;
+  // The 16 slots of pass p from j = 16 (1024 p + tid) on, read with 128-bit loads: their ages, 0 = not evictable.
+  auto ages16 = [&](int j, int (&age)[16]) {
+    if (j < L) {                                 // j is a multiple of 16 and the capacity a multiple of 128
+      bool free[16];
+      untouched(j, free);
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        const int4 sp = *reinterpret_cast<const int4*>(c.stamp + sb + j + 4 * q);
+        const int sq[4] = {sp.x, sp.y, sp.z, sp.w};
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          const int s = j + 4 * q + u;
+          age[4 * q + u] = (s < L && s >= c.n_sink && free[4 * q + u] && sq[u] < now) ? now - sq[u] : 0;
+        }
+      }
+    } else {
+#pragma unroll
+      for (int u = 0; u < 16; ++u) age[u] = 0;
+    }
+  };
+  // Up to 2 x 16384 slots a thread keeps its ages in registers, two to a word, so the search for the age and the compaction read
+  // nothing again (12 heads x 32768 slots at capacity: 87 -> 44 us).  A third pass would be eight more of the 64 registers that 1 024
+  // threads leave each, and two are all that fit (12 bytes spill already): longer caches, and ages above 16 bits, go through L2 in
+  // every pass, as all did before.
+  constexpr int kPasses = 2;
+  uint32_t held[kPasses][8];
+  int cand = 0, a_min = 0x7fffffff, a_max = 0;
+  for (int j0 = 0, p = 0; j0 < L; j0 += 16 * blockDim.x, ++p) {
+    int age[16];
+    ages16(j0 + 16 * tid, age);
+#pragma unroll
+    for (int u = 0; u < 16; ++u)
+      if (age[u] > 0) { ++cand; a_min = min(a_min, age[u]); a_max = max(a_max, age[u]); }
+#pragma unroll
+    for (int q = 0; q < kPasses; ++q)
+      if (p == q)
+#pragma unroll
+        for (int u = 0; u < 8; ++u) held[q][u] = (static_cast<uint32_t>(age[2 * u]) & 0xFFFFu) | (static_cast<uint32_t>(age[2 * u + 1]) << 16);
+  }
+  cand = block_sum(cand, red);
+  a_min = -block_max(-a_min, red);
+  a_max = block_max(a_max, red);
+  if (cand < E) ok = false;
+  const bool in_regs = L <= kPasses * 16 * static_cast<int>(blockDim.x) && a_max <= 0xFFFF;
+  auto for_each_pass = [&](auto&& body) {        // body(first slot, ages)
+    int age[16];
+    if (in_regs) {
+#pragma unroll
+      for (int p = 0; p < kPasses; ++p) {
+        const int j0 = p * 16 * blockDim.x;
+        if (j0 >= L) break;
+#pragma unroll
+        for (int u = 0; u < 8; ++u) { age[2 * u] = held[p][u] & 0xFFFFu; age[2 * u + 1] = held[p][u] >> 16; }
+        body(j0 + 16 * tid, age);
+      }
+    } else {
+      for (int j0 = 0; j0 < L; j0 += 16 * blockDim.x) {
+        ages16(j0 + 16 * tid, age);
+        body(j0 + 16 * tid, age);
+      }
+    }
+  };
+  auto reach = [&](int a) {                      // evictable slots of that age or older
+    int cn = 0;
+    for_each_pass([&](int, int (&age)[16]) {
+#pragma unroll
+      for (int u = 0; u < 16; ++u) cn += age[u] >= a ? 1 : 0;
+    });
+    return block_sum(cn, red);
+  };
+  if (ok) {
+    int lo = a_min, hi = a_max;                  // all reach a_min
+    while (lo < hi) {
+      const int mid = lo + ((hi - lo + 1) >> 1);
+      if (reach(mid) >= E) lo = mid; else hi = mid - 1;
+    }
+    const int a_star = lo;
+    const int need_eq = E - reach(a_star + 1);
+    // ordered compaction of the victims: all older slots, and the first need_eq slots of that age
+    int eq_run = 0, out_run = 0;
+    for_each_pass([&](int j, int (&age)[16]) {
+      int my_eq = 0;
+#pragma unroll
+      for (int u = 0; u < 16; ++u) my_eq += age[u] == a_star ? 1 : 0;
+      int tot_eq;
+      int eq_rank = eq_run + block_exscan(my_eq, red, &tot_eq);
+      int my_take = 0;
+      unsigned take_mask = 0;
+#pragma unroll
+      for (int u = 0; u < 16; ++u) {
+        const bool is_eq = age[u] == a_star;
+        const bool take = age[u] > a_star || (is_eq && eq_rank < need_eq);
+        eq_rank += is_eq ? 1 : 0;
+        take_mask |= (take ? 1u : 0u) << u;
+        my_take += take ? 1 : 0;
+      }
+      int tot_take;
+      int pos = out_run + block_exscan(my_take, red, &tot_take);
+#pragma unroll
+      for (int u = 0; u < 16; ++u)
+        if ((take_mask >> u) & 1u)
+          keys[pos++] = (static_cast<unsigned long long>(static_cast<uint32_t>(now - age[u])) << 32) | static_cast<uint32_t>(j + u);
+      eq_run += tot_eq;
+      out_run += tot_take;
+    });
+    int e2 = 1;
+    while (e2 < E) e2 <<= 1;
+    for (int p = E + tid; p < e2; p += blockDim.x) keys[p] = ~0ull;
+    __syncthreads();
+    bitonic_sort_smem(keys, e2);
+    int ev = 0;
+    for (int k = tid; k < E; k += blockDim.x) {
+      const int v = static_cast<int>(keys[k] & 0xFFFFFFFFull);
+      c.victims[tb + k] = v;
+      ev += c.count[sb + v];
+    }
+    evicted_tokens = block_sum(ev, red);
+  }
+  return ok;
 }
 
 __global__ void __launch_bounds__(1024) plan_kernel(const CacheView c, int n, int32_t* __restrict__ dest_out) {
@@ -391,126 +578,16 @@ __global__ void __launch_bounds__(1024) plan_kernel(const CacheView c, int n, in
   const int A = min(U, room);
   const int E = U - A;
   int ok = 1;
-  // Eviction.  evictable = live, past the sink prefix, stamp < now, not touched by this update (cnt == 0).  The oldest E go, ties by
-  // slot; what is looked for is the age (now - stamp) that at least E evictable slots reach, the greatest such.
   int evicted_tokens = 0;
   if (E > 0) {
-    // The 16 slots of pass p from j = 16 (1024 p + tid) on, read with 128-bit loads: their ages, 0 = not evictable.
-    auto ages16 = [&](int j, int (&age)[16]) {
-      if (j < L) {                                 // j is a multiple of 16 and the capacity a multiple of 128
+    ok = choose_victims(c, h, L, now, E, keys, red, evicted_tokens, [&](int j, bool (&free)[16]) {
+      const int4* p = reinterpret_cast<const int4*>(c.cnt + sb + j);
 #pragma unroll
-        for (int q = 0; q < 4; ++q) {
-          const int4 cn = *reinterpret_cast<const int4*>(c.cnt + sb + j + 4 * q), sp = *reinterpret_cast<const int4*>(c.stamp + sb + j + 4 * q);
-          const int cq[4] = {cn.x, cn.y, cn.z, cn.w}, sq[4] = {sp.x, sp.y, sp.z, sp.w};
-#pragma unroll
-          for (int u = 0; u < 4; ++u) {
-            const int s = j + 4 * q + u;
-            age[4 * q + u] = (s < L && s >= c.n_sink && cq[u] == 0 && sq[u] < now) ? now - sq[u] : 0;
-          }
-        }
-      } else {
-#pragma unroll
-        for (int u = 0; u < 16; ++u) age[u] = 0;
+      for (int q = 0; q < 4; ++q) {
+        const int4 cn = p[q];
+        free[4 * q] = cn.x == 0; free[4 * q + 1] = cn.y == 0; free[4 * q + 2] = cn.z == 0; free[4 * q + 3] = cn.w == 0;
       }
-    };
-    // Up to 2 x 16384 slots a thread keeps its ages in registers, two to a word, so the search for the age and the compaction read
-    // nothing again (12 heads x 32768 slots at capacity: 87 -> 44 us).  A third pass would be eight more of the 64 registers that 1 024
-    // threads leave each, and two are all that fit (12 bytes spill already): longer caches, and ages above 16 bits, go through L2 in
-    // every pass, as all did before.
-    constexpr int kPasses = 2;
-    uint32_t held[kPasses][8];
-    int cand = 0, a_min = 0x7fffffff, a_max = 0;
-    for (int j0 = 0, p = 0; j0 < L; j0 += 16 * blockDim.x, ++p) {
-      int age[16];
-      ages16(j0 + 16 * tid, age);
-#pragma unroll
-      for (int u = 0; u < 16; ++u)
-        if (age[u] > 0) { ++cand; a_min = min(a_min, age[u]); a_max = max(a_max, age[u]); }
-#pragma unroll
-      for (int q = 0; q < kPasses; ++q)
-        if (p == q)
-#pragma unroll
-          for (int u = 0; u < 8; ++u) held[q][u] = (static_cast<uint32_t>(age[2 * u]) & 0xFFFFu) | (static_cast<uint32_t>(age[2 * u + 1]) << 16);
-    }
-    cand = block_sum(cand, red);
-    a_min = -block_max(-a_min, red);
-    a_max = block_max(a_max, red);
-    if (cand < E) ok = 0;
-    const bool in_regs = L <= kPasses * 16 * static_cast<int>(blockDim.x) && a_max <= 0xFFFF;
-    auto for_each_pass = [&](auto&& body) {        // body(first slot, ages)
-      int age[16];
-      if (in_regs) {
-#pragma unroll
-        for (int p = 0; p < kPasses; ++p) {
-          const int j0 = p * 16 * blockDim.x;
-          if (j0 >= L) break;
-#pragma unroll
-          for (int u = 0; u < 8; ++u) { age[2 * u] = held[p][u] & 0xFFFFu; age[2 * u + 1] = held[p][u] >> 16; }
-          body(j0 + 16 * tid, age);
-        }
-      } else {
-        for (int j0 = 0; j0 < L; j0 += 16 * blockDim.x) {
-          ages16(j0 + 16 * tid, age);
-          body(j0 + 16 * tid, age);
-        }
-      }
-    };
-    auto reach = [&](int a) {                      // evictable slots of that age or older
-      int cn = 0;
-      for_each_pass([&](int, int (&age)[16]) {
-#pragma unroll
-        for (int u = 0; u < 16; ++u) cn += age[u] >= a ? 1 : 0;
-      });
-      return block_sum(cn, red);
-    };
-    if (ok) {
-      int lo = a_min, hi = a_max;                  // all reach a_min
-      while (lo < hi) {
-        const int mid = lo + ((hi - lo + 1) >> 1);
-        if (reach(mid) >= E) lo = mid; else hi = mid - 1;
-      }
-      const int a_star = lo;
-      const int need_eq = E - reach(a_star + 1);
-      // ordered compaction of the victims: all older slots, and the first need_eq slots of that age
-      int eq_run = 0, out_run = 0;
-      for_each_pass([&](int j, int (&age)[16]) {
-        int my_eq = 0;
-#pragma unroll
-        for (int u = 0; u < 16; ++u) my_eq += age[u] == a_star ? 1 : 0;
-        int tot_eq;
-        int eq_rank = eq_run + block_exscan(my_eq, red, &tot_eq);
-        int my_take = 0;
-        unsigned take_mask = 0;
-#pragma unroll
-        for (int u = 0; u < 16; ++u) {
-          const bool is_eq = age[u] == a_star;
-          const bool take = age[u] > a_star || (is_eq && eq_rank < need_eq);
-          eq_rank += is_eq ? 1 : 0;
-          take_mask |= (take ? 1u : 0u) << u;
-          my_take += take ? 1 : 0;
-        }
-        int tot_take;
-        int pos = out_run + block_exscan(my_take, red, &tot_take);
-#pragma unroll
-        for (int u = 0; u < 16; ++u)
-          if ((take_mask >> u) & 1u)
-            keys[pos++] = (static_cast<unsigned long long>(static_cast<uint32_t>(now - age[u])) << 32) | static_cast<uint32_t>(j + u);
-        eq_run += tot_eq;
-        out_run += tot_take;
-      });
-      int e2 = 1;
-      while (e2 < E) e2 <<= 1;
-      for (int p = E + tid; p < e2; p += blockDim.x) keys[p] = ~0ull;
-      __syncthreads();
-      bitonic_sort_smem(keys, e2);
-      int ev = 0;
-      for (int k = tid; k < E; k += blockDim.x) {
-        const int v = static_cast<int>(keys[k] & 0xFFFFFFFFull);
-        c.victims[tb + k] = v;
-        ev += c.count[sb + v];
-      }
-      evicted_tokens = block_sum(ev, red);
-    }
+    }) ? 1 : 0;
   }
   __syncthreads();
   // destinations of the tokens that take a victim's slot (matched tokens get theirs in the scatter kernel)
@@ -539,6 +616,149 @@ __global__ void __launch_bounds__(1024) plan_kernel(const CacheView c, int n, in
     pr.len_new = ok ? L + A : L;
     pr.evicted_tokens = evicted_tokens;
     pr.pages_granted = grant;
+    pr.pad[0] = pr.pad[1] = 0;
+    c.plan[h] = pr;
+  }
+}
+
+// The three steps in one CTA per head, for caches and calls whose counters fit its shared memory: what each slot is matched by is
+// counted there (16 bits a slot), the counter's old value is a token's rank in its group, and the groups' starts replace the counters,
+// so that neither counts nor positions go through memory, nothing has to be cleared for them and two launches are saved.  A thread's
+// tokens (i = tid, tid + 1024, ... up to K of them) stay in its registers.  Bound by the latencies of a few dependent steps of one CTA.
+template <int K>
+__global__ void __launch_bounds__(1024) plan_fused_kernel(const CacheView c, int n, float tau, const UpdateOut out) {
+  chain_wait();
+  extern __shared__ unsigned long long plan_s[];       // [CAP / 4] counters, then the victim sort buffer
+  __shared__ int red[32];
+  __shared__ int fresh_s[K * 32];                      // unmatched tokens of (pass, warp), then of those before
+  const int h = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int64_t tb = static_cast<int64_t>(h) * c.max_tokens, gb = static_cast<int64_t>(h) * (c.max_tokens + 1), ob = static_cast<int64_t>(h) * n;
+  uint32_t* cnt = reinterpret_cast<uint32_t*>(plan_s); // slots 2 q and 2 q + 1
+  unsigned long long* keys = plan_s + c.CAP / 4;
+  const int L = c.len[h], now = *c.now;
+  unsigned long long best[K];
+#pragma unroll
+  for (int k = 0; k < K; ++k) best[k] = k * 1024 + tid < n ? c.best[tb + k * 1024 + tid] : 0ull;
+  for (int q = tid; q < (L + 15) / 16 * 2; q += 1024) reinterpret_cast<uint4*>(cnt)[q] = make_uint4(0, 0, 0, 0);
+  __syncthreads();
+
+  // a token's slot and its rank among the slot's tokens (below 2^14), or kFresh
+  constexpr uint32_t kFresh = 0xFFFFFFFFu;
+  uint32_t place[K];
+#pragma unroll
+  for (int k = 0; k < K; ++k) {
+    const int i = k * 1024 + tid;
+    int j = -1;
+    float s = 0.f;
+    if (best[k] != 0ull) {
+      j = FASTAR_IDX(static_cast<int>(0xFFFFFFFFu - static_cast<uint32_t>(best[k] & 0xFFFFFFFFull)), c.CAP, c.status);
+      s = ordered_to_float(static_cast<uint32_t>(best[k] >> 32));
+    }
+    const bool matched = j >= 0 && s >= tau;
+    place[k] = kFresh;
+    if (i < n) {
+      c.sim[tb + i] = s;
+      if (out.match) out.match[ob + i] = matched ? j : -1;
+      if (out.sim) out.sim[ob + i] = s;
+      if (matched) place[k] = static_cast<uint32_t>(j) | ((atomicAdd(cnt + (j >> 1), 1u << (16 * (j & 1))) >> (16 * (j & 1))) & 0xFFFFu) << 16;
+    }
+    const uint32_t m = __ballot_sync(0xffffffffu, i < n && !matched);
+    if (lane == 0) fresh_s[k * 32 + warp] = __popc(m);
+  }
+  __syncthreads();
+  int U;
+  const int fresh_before = block_exscan(tid < K * 32 ? fresh_s[tid] : 0, red, &U);
+  if (tid < K * 32) fresh_s[tid] = fresh_before;
+
+  // groups: as in plan_kernel; a touched slot's counter becomes 2^15 + the start of its members
+  int n_seg = 0, M = 0;
+  for (int j0 = 0; j0 < L; j0 += 16 * 1024) {
+    const int j = j0 + 16 * tid;
+    uint4* p = reinterpret_cast<uint4*>(cnt + j / 2);
+    uint32_t w[8] = {0, 0, 0, 0, 0, 0, 0, 0};
+    if (j < L) {
+      const uint4 a = p[0], b = p[1];
+      w[0] = a.x; w[1] = a.y; w[2] = a.z; w[3] = a.w; w[4] = b.x; w[5] = b.y; w[6] = b.z; w[7] = b.w;
+    }
+    int my_seg = 0, my_mem = 0;
+#pragma unroll
+    for (int q = 0; q < 8; ++q) {
+      my_seg += ((w[q] & 0xFFFFu) != 0) + (w[q] >> 16 != 0);
+      my_mem += (w[q] & 0xFFFFu) + (w[q] >> 16);
+    }
+    int tot;
+    const int ex = block_exscan((my_seg << 16) | my_mem, red, &tot);
+    int seg = n_seg + (ex >> 16), mem = M + (ex & 0xFFFF);
+    if (my_seg > 0) {
+#pragma unroll
+      for (int u = 0; u < 16; ++u) {
+        const uint32_t cn = (w[u >> 1] >> (16 * (u & 1))) & 0xFFFFu;
+        if (cn > 0) {
+          c.segslot[tb + seg] = j + u;
+          c.segpos[gb + seg] = mem;
+          w[u >> 1] = (w[u >> 1] & (0xFFFFu << (16 * (~u & 1)))) | ((0x8000u | mem) << (16 * (u & 1)));
+          ++seg;
+          mem += cn;
+        }
+      }
+      p[0] = make_uint4(w[0], w[1], w[2], w[3]);
+      p[1] = make_uint4(w[4], w[5], w[6], w[7]);
+    }
+    n_seg += tot >> 16;
+    M += tot & 0xFFFF;
+  }
+  if (tid == 0) c.segpos[gb + n_seg] = M;
+  __syncthreads();
+
+  const int room = c.CAP - L, A = min(U, room), E = U - A;
+  int evicted_tokens = 0;
+  bool ok = true;
+  if (E > 0)
+    ok = choose_victims(c, h, L, now, E, keys, red, evicted_tokens, [&](int j, bool (&free)[16]) {
+#pragma unroll
+      for (int q = 0; q < 8; ++q) {
+        const uint32_t w = cnt[j / 2 + q];
+        free[2 * q] = (w & 0xFFFFu) == 0;
+        free[2 * q + 1] = w >> 16 == 0;
+      }
+    });
+  __syncthreads();
+
+  // members into their groups' ranges; unmatched tokens, in token order, appended or into the victims' slots
+#pragma unroll
+  for (int k = 0; k < K; ++k) {
+    const int i = k * 1024 + tid;
+    const bool fresh = i < n && place[k] == kFresh;
+    const uint32_t m = __ballot_sync(0xffffffffu, fresh);
+    int d = -1;
+    if (fresh) {
+      const int r = fresh_s[k * 32 + warp] + __popc(m & ((1u << lane) - 1u));
+      c.ulist[tb + r] = i;
+      if (ok) d = r < A ? L + r : FASTAR_IDX(c.victims[tb + r - A], c.CAP, c.status);
+    } else if (i < n && ok) {
+      const int j = place[k] & 0xFFFFu;
+      d = j;
+      const uint32_t start = (cnt[j >> 1] >> (16 * (j & 1))) & 0x7FFFu;
+      c.order[tb + FASTAR_IDX(static_cast<int>(start + (place[k] >> 16)), n, c.status)] = i;
+    }
+    if (i < n) {
+      c.dest[tb + i] = d;
+      if (out.dest) out.dest[ob + i] = d;
+    }
+  }
+  if (tid == 0) {
+    if (!ok) record_status(c.status, kErrCapacity);
+    PlanRec pr;
+    pr.ok = ok ? 1 : 0;
+    pr.n_matched = M;
+    pr.n_seg = n_seg;
+    pr.n_unmatched = U;
+    pr.n_append = ok ? A : 0;
+    pr.n_evict = ok ? E : 0;
+    pr.len_old = L;
+    pr.len_new = ok ? L + A : L;
+    pr.evicted_tokens = evicted_tokens;
+    pr.pages_granted = 0;
     pr.pad[0] = pr.pad[1] = 0;
     c.plan[h] = pr;
   }
@@ -609,7 +829,31 @@ int launch_probe_cosine(const CacheView& c, const __nv_bfloat16* k_new, int n, i
   return cudaGetLastError() == cudaSuccess ? 1 : FASTAR_ERR_CUDA;
 }
 
+template <int K>
+static int launch_plan_fused(const CacheView& c, int n, float tau, const UpdateOut& out, int smem, cudaStream_t st) {
+  const int cfg = ensure_dynamic_smem(reinterpret_cast<const void*>(plan_fused_kernel<K>), smem);
+  if (cfg != FASTAR_OK) return cfg;
+  launch_chained(plan_fused_kernel<K>, c.H, 1024, smem, st, c, n, tau, out);
+  return cudaGetLastError() == cudaSuccess ? 1 : FASTAR_ERR_CUDA;
+}
+
+bool plan_is_fused(const CacheView& c, int n) {
+  return !c.pool_shared && n <= 8192 && c.CAP <= 65536 && plan_fused_smem(c, n) <= 220 * 1024;
+}
+int plan_fused_smem(const CacheView& c, int n) {
+  int room = 1;                              // victims, up to a power of two
+  while (room < n) room <<= 1;
+  return c.CAP * 2 + room * 8;
+}
+
 int launch_plan(const CacheView& c, int n, float tau, const UpdateOut& out, cudaStream_t st) {
+  if (plan_is_fused(c, n)) {
+    const int smem = plan_fused_smem(c, n);
+    if (n <= 1024) return launch_plan_fused<1>(c, n, tau, out, smem, st);
+    if (n <= 2048) return launch_plan_fused<2>(c, n, tau, out, smem, st);
+    if (n <= 4096) return launch_plan_fused<4>(c, n, tau, out, smem, st);
+    return launch_plan_fused<8>(c, n, tau, out, smem, st);
+  }
   const int cfg = ensure_dynamic_smem(reinterpret_cast<const void*>(plan_kernel), 16384 * 8);
   if (cfg != FASTAR_OK) return cfg;
   const dim3 grid((n + 255) / 256, c.H);
@@ -617,18 +861,6 @@ int launch_plan(const CacheView& c, int n, float tau, const UpdateOut& out, cuda
   launch_chained(plan_kernel, c.H, 1024, 16384 * 8, st, c, n, out.dest);
   launch_chained(scatter_kernel, grid, 256, 0, st, c, n, out.dest);
   return cudaGetLastError() == cudaSuccess ? 3 : FASTAR_ERR_CUDA;
-}
-
-// Eight counters as bf16: all of them (SHIFT < 0: exact up to 256), or one of their two 8-bit digits.
-template <int SHIFT>
-__device__ __forceinline__ uint4 pack_counts(const int (&v)[8]) {
-  uint32_t w[4];
-#pragma unroll
-  for (int e = 0; e < 4; ++e) {
-    const int lo = SHIFT < 0 ? v[2 * e] : (v[2 * e] >> (SHIFT < 0 ? 0 : SHIFT)) & 255, hi = SHIFT < 0 ? v[2 * e + 1] : (v[2 * e + 1] >> (SHIFT < 0 ? 0 : SHIFT)) & 255;
-    w[e] = pack_bf16x2(static_cast<float>(lo), static_cast<float>(hi));
-  }
-  return make_uint4(w[0], w[1], w[2], w[3]);
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -689,34 +921,6 @@ __global__ void __launch_bounds__(128) key_hist_kernel(const CacheView c, int us
 int launch_finalize_hist(const CacheView& c, fastar_update_stats* stats_out, int advance_clock, cudaStream_t st) {
   launch_chained(key_hist_kernel, dim3(c.CAPB, c.H), 128, c.hist_cols * 4, st, c, advance_clock >= 0 ? 1 : 0, stats_out,
                                                                   advance_clock > 0 ? 1 : 0);
-  return cudaGetLastError() == cudaSuccess ? 1 : FASTAR_ERR_CUDA;
-}
-
-// S2 (query side)
-__global__ void __launch_bounds__(128) query_hist_kernel(const CacheView c, const uint32_t* __restrict__ codes, int nq, int block_q) {
-  chain_wait();
-  extern __shared__ __align__(16) int hist[];
-  const int a = blockIdx.x, h = blockIdx.y;
-  for (int q = threadIdx.x; q < c.hist_cols / 4; q += blockDim.x) reinterpret_cast<int4*>(hist)[q] = make_int4(0, 0, 0, 0);
-  __syncthreads();
-  const int r0 = a * block_q, r1 = min(nq, r0 + block_q);
-  const int nb = 1 << c.B;
-  for (int r = r0 + threadIdx.x; r < r1; r += blockDim.x) {
-    const uint32_t code = codes[static_cast<int64_t>(h) * c.max_tokens + r];
-    for (int t = 0; t < c.T; ++t) atomicAdd(&hist[t * nb + ((code >> (8 * t)) & 0xFFu)], 1);
-  }
-  __syncthreads();
-  __nv_bfloat16* dst = c.hq + (static_cast<int64_t>(h) * c.max_qb + a) * c.hist_cols;
-  for (int q = threadIdx.x; q < c.hist_cols / 8; q += blockDim.x) {
-    int v[8];
-#pragma unroll
-    for (int e = 0; e < 8; ++e) v[e] = hist[8 * q + e];
-    reinterpret_cast<uint4*>(dst)[q] = pack_counts<-1>(v);
-  }
-}
-int launch_query_hist(const CacheView& c, const uint32_t* codes, int nq, int block_q, cudaStream_t st) {
-  const int nqb = (nq + block_q - 1) / block_q;
-  launch_chained(query_hist_kernel, dim3(nqb, c.H), 128, c.hist_cols * 4, st, c, codes, nq, block_q);
   return cudaGetLastError() == cudaSuccess ? 1 : FASTAR_ERR_CUDA;
 }
 
@@ -790,7 +994,7 @@ __global__ void __launch_bounds__(32 * kTopkWarps) topk_kernel(const TopkArgs a)
   }
   hi = __reduce_max_sync(0xffffffffu, hi);
   lo = __reduce_min_sync(0xffffffffu, lo);
-  // t: the largest value that at least k keys reach.  Entries past the row are 0 and every candidate is above 0.
+  // t: the largest value that at least k keys reach, or a lower one that no other key reaches.  Entries past the row are 0 and every candidate is above 0.
   const int bits = 32 - __clz(hi ^ lo);
   uint32_t t = bits >= 32 ? 0u : hi & ~((1u << bits) - 1u);
   for (int bit = bits - 1; bit >= 0; --bit) {
@@ -798,7 +1002,9 @@ __global__ void __launch_bounds__(32 * kTopkWarps) topk_kernel(const TopkArgs a)
     int cnt[4] = {0, 0, 0, 0};
 #pragma unroll
     for (int q = 0; q < NV; ++q) cnt[q & 3] += v[q] >= cand ? 1 : 0;
-    if (static_cast<int>(__reduce_add_sync(0xffffffffu, (cnt[0] + cnt[1]) + (cnt[2] + cnt[3]))) >= k) t = cand;
+    const int reach = static_cast<int>(__reduce_add_sync(0xffffffffu, (cnt[0] + cnt[1]) + (cnt[2] + cnt[3])));
+    if (reach >= k) t = cand;
+    if (reach == k) break;                 // the k keys are told apart from the others: the lower bits do not matter
   }
   int above = 0;
 #pragma unroll
