@@ -670,42 +670,44 @@ __global__ void __launch_bounds__(1024) plan_fused_kernel(const CacheView c, int
   const int fresh_before = block_exscan(tid < K * 32 ? fresh_s[tid] : 0, red, &U);
   if (tid < K * 32) fresh_s[tid] = fresh_before;
 
-  // groups: as in plan_kernel; a touched slot's counter becomes 2^15 + the start of its members
+  // Groups, 16 consecutive slots per thread and pass; a touched slot's counter becomes 2^15 + the start of its members.  The tables are
+  // put together in shared memory (slot and start in one word, where the victims come later) and leave in order: a scattered 4-byte store
+  // takes an SM a cycle per lane, and there is one SM per head.
+  uint32_t* table = reinterpret_cast<uint32_t*>(keys);
+  uint16_t* slot16 = reinterpret_cast<uint16_t*>(cnt);
   int n_seg = 0, M = 0;
   for (int j0 = 0; j0 < L; j0 += 16 * 1024) {
     const int j = j0 + 16 * tid;
-    uint4* p = reinterpret_cast<uint4*>(cnt + j / 2);
     uint32_t w[8] = {0, 0, 0, 0, 0, 0, 0, 0};
     if (j < L) {
-      const uint4 a = p[0], b = p[1];
+      const uint4 a = reinterpret_cast<const uint4*>(cnt + j / 2)[0], b = reinterpret_cast<const uint4*>(cnt + j / 2)[1];
       w[0] = a.x; w[1] = a.y; w[2] = a.z; w[3] = a.w; w[4] = b.x; w[5] = b.y; w[6] = b.z; w[7] = b.w;
     }
-    int my_seg = 0, my_mem = 0;
+    uint32_t touched = 0;
+    int my_mem = 0;
 #pragma unroll
     for (int q = 0; q < 8; ++q) {
-      my_seg += ((w[q] & 0xFFFFu) != 0) + (w[q] >> 16 != 0);
+      touched |= ((w[q] & 0xFFFFu) != 0 ? 1u : 0u) << (2 * q) | (w[q] >> 16 != 0 ? 2u : 0u) << (2 * q);
       my_mem += (w[q] & 0xFFFFu) + (w[q] >> 16);
     }
     int tot;
-    const int ex = block_exscan((my_seg << 16) | my_mem, red, &tot);
+    const int ex = block_exscan((__popc(touched) << 16) | my_mem, red, &tot);
     int seg = n_seg + (ex >> 16), mem = M + (ex & 0xFFFF);
-    if (my_seg > 0) {
-#pragma unroll
-      for (int u = 0; u < 16; ++u) {
-        const uint32_t cn = (w[u >> 1] >> (16 * (u & 1))) & 0xFFFFu;
-        if (cn > 0) {
-          c.segslot[tb + seg] = j + u;
-          c.segpos[gb + seg] = mem;
-          w[u >> 1] = (w[u >> 1] & (0xFFFFu << (16 * (~u & 1)))) | ((0x8000u | mem) << (16 * (u & 1)));
-          ++seg;
-          mem += cn;
-        }
-      }
-      p[0] = make_uint4(w[0], w[1], w[2], w[3]);
-      p[1] = make_uint4(w[4], w[5], w[6], w[7]);
+    for (; touched; touched &= touched - 1) {            // a few of the sixteen
+      const int slot = j + __ffs(touched) - 1;
+      const int members = slot16[slot];
+      table[seg++] = static_cast<uint32_t>(slot) | static_cast<uint32_t>(mem) << 16;
+      slot16[slot] = static_cast<uint16_t>(0x8000 | mem);
+      mem += members;
     }
     n_seg += tot >> 16;
     M += tot & 0xFFFF;
+  }
+  __syncthreads();
+  for (int q = tid; q < n_seg; q += 1024) {
+    const uint32_t e = table[q];
+    c.segslot[tb + q] = e & 0xFFFFu;
+    c.segpos[gb + q] = e >> 16;
   }
   if (tid == 0) c.segpos[gb + n_seg] = M;
   __syncthreads();
@@ -724,7 +726,9 @@ __global__ void __launch_bounds__(1024) plan_fused_kernel(const CacheView c, int
     });
   __syncthreads();
 
-  // members into their groups' ranges; unmatched tokens, in token order, appended or into the victims' slots
+  // members into their groups' ranges (through shared memory, as above); unmatched tokens, in token order, appended or into the victims'
+  // slots
+  uint16_t* members = reinterpret_cast<uint16_t*>(keys);
 #pragma unroll
   for (int k = 0; k < K; ++k) {
     const int i = k * 1024 + tid;
@@ -738,14 +742,16 @@ __global__ void __launch_bounds__(1024) plan_fused_kernel(const CacheView c, int
     } else if (i < n && ok) {
       const int j = place[k] & 0xFFFFu;
       d = j;
-      const uint32_t start = (cnt[j >> 1] >> (16 * (j & 1))) & 0x7FFFu;
-      c.order[tb + FASTAR_IDX(static_cast<int>(start + (place[k] >> 16)), n, c.status)] = i;
+      members[FASTAR_IDX(static_cast<int>((slot16[j] & 0x7FFFu) + (place[k] >> 16)), n, c.status)] = static_cast<uint16_t>(i);
     }
     if (i < n) {
       c.dest[tb + i] = d;
       if (out.dest) out.dest[ob + i] = d;
     }
   }
+  __syncthreads();
+  if (ok)
+    for (int q = tid; q < M; q += 1024) c.order[tb + q] = members[q];
   if (tid == 0) {
     if (!ok) record_status(c.status, kErrCapacity);
     PlanRec pr;
