@@ -69,6 +69,7 @@ struct CacheView {
   int32_t* sel;                    // [H][max_qb][CAPB]
   int32_t* nsel;                   // [H]
   uint32_t* rel;                   // [H][max_frames][max_prompt]  ordered-uint relevance
+  int32_t* rel_count;              // [H]  CTAs of the relevance kernel that are through with the head (zero between calls)
   int32_t* selp;                   // [H][max_frames][max_prompt]
   // staging (fp32 entry conversion and the host-tensor step)
   __nv_bfloat16* stage[6];         // k, v, q (AnnSA), kp, vp, q (AnnCA)  ([H][max_tokens][D] / [H][max_prompt][D])
@@ -161,9 +162,9 @@ int launch_quantize_rows(const CacheView& c, const __nv_bfloat16* x, int n, int6
 
 // relevance_kernel.cu: C1 on the bf16 rows and on the 8-bit codes
 int launch_c1_relevance(const CacheView& c, const CUtensorMap& tm_q, const CUtensorMap& tm_kp, int nq, int np, int frame_len,
-                        cudaStream_t st);
+                        int keep, cudaStream_t st);
 int launch_c1_relevance_fp8(const CacheView& c, const CUtensorMap& tm_q8, const CUtensorMap& tm_kp8, const float* qn,
-                            const float* kn, int nq, int np, int frame_len, cudaStream_t st);
+                            const float* kn, int nq, int np, int frame_len, int keep, cudaStream_t st);
 
 // attn_kernels.cu
 struct AttnArgs {

@@ -148,6 +148,7 @@ size_t carve(const fastar_cache_desc& d, uint8_t* base, CacheView* v) {
   t.sel = reinterpret_cast<int32_t*>(take(H * t.max_qb * t.CAPB * 4));
   t.nsel = reinterpret_cast<int32_t*>(take(H * 4));
   t.rel = reinterpret_cast<uint32_t*>(take(H * t.max_frames * MP * 4));
+  t.rel_count = reinterpret_cast<int32_t*>(take(H * 4));
   t.selp = reinterpret_cast<int32_t*>(take(H * t.max_frames * MP * 4));
   {
     // stage[0], stage[1] and, in the same place, the parts of AnnSA's cut items: nobody stages keys and values while AnnSA attends, but
@@ -378,6 +379,7 @@ int fastar_cache_create(fastar_cache_t** out, const fastar_cache_desc* desc, con
   // AnnCA's own scratch: cleared here only, because an AnnCA call may run beside a reset or an import on another stream
   r = cudaMemsetAsync(v.rel, 0, static_cast<size_t>(v.H) * v.max_frames * v.max_prompt * 4, nullptr) == cudaSuccess ? FASTAR_OK : FASTAR_ERR_CUDA;
   // so are the counters of AnnSA's parts, which every call leaves at zero
+  if (r == FASTAR_OK && cudaMemsetAsync(v.rel_count, 0, static_cast<size_t>(v.H) * 4, nullptr) != cudaSuccess) r = FASTAR_ERR_CUDA;
   if (r == FASTAR_OK && cudaMemsetAsync(v.part_count, 0, kAttnMaxGrid * 4, nullptr) != cudaSuccess) r = FASTAR_ERR_CUDA;
   if (r == FASTAR_OK) r = fastar_cache_reset(c, nullptr);
   if (r == FASTAR_OK && cudaStreamSynchronize(nullptr) != cudaSuccess) r = FASTAR_ERR_CUDA;
@@ -813,6 +815,7 @@ int fastar_annca_attention(fastar_cache_t* c, const void* q, const void* k_promp
     if (!c->rel_clear && cudaMemsetAsync(v.rel, 0, static_cast<size_t>(v.H) * v.max_frames * v.max_prompt * 4, st) != cudaSuccess)
       return FASTAR_ERR_CUDA;
     c->rel_clear = false;
+    const int ranked = rel_out ? 0 : keep;     // the maxima are wanted: they are ranked (and cleared) by a kernel behind their decoding
     float rel_scale = 1.0f / sqrtf(static_cast<float>(v.D));
     if (v.search_bits == 8 && !v.sign_codes) {
       // relevance on the 8-bit codes of the directions, scaled back by the norms (Section 5.1 quantised search)
@@ -822,15 +825,17 @@ int fastar_annca_attention(fastar_cache_t* c, const void* q, const void* k_promp
       if (r != FASTAR_OK) return r;
       ACCK(FASTAR_K_HASH, launch_quantize_rows(v, qb, nq, qhs, qts, v.q8_ca, v.max_tokens, v.qn_ca, v.max_tokens, st));
       ACCK(FASTAR_K_HASH, launch_quantize_rows(v, kpb, np, khs, kts, v.kp8_ca, v.max_prompt, v.kpn_ca, v.max_prompt, st));
-      ACCK(FASTAR_K_C1_RELEVANCE, launch_c1_relevance_fp8(v, tm_q8, tm_kp8, v.qn_ca, v.kpn_ca, nq, np, frame_len, st));
+      ACCK(FASTAR_K_C1_RELEVANCE, launch_c1_relevance_fp8(v, tm_q8, tm_kp8, v.qn_ca, v.kpn_ca, nq, np, frame_len, ranked, st));
       rel_scale *= 1.0f / 256.0f;
     } else {
       r = make_map(c, &tm_kp, kpb, v.D, np, v.H, static_cast<uint64_t>(kts) * 2, static_cast<uint64_t>(khs) * 2, 128);
       if (r != FASTAR_OK) return r;
-      ACCK(FASTAR_K_C1_RELEVANCE, launch_c1_relevance(v, tm_q, tm_kp, nq, np, frame_len, st));
+      ACCK(FASTAR_K_C1_RELEVANCE, launch_c1_relevance(v, tm_q, tm_kp, nq, np, frame_len, ranked, st));
     }
-    if (rel_out) ACC(launch_decode_rel(v, F, np, rel_scale, rel_out, st));
-    ACCK(FASTAR_K_TOPK_PROMPT, launch_topk_prompt(v, F, np, keep, st));
+    if (rel_out) {
+      ACC(launch_decode_rel(v, F, np, rel_scale, rel_out, st));
+      ACCK(FASTAR_K_TOPK_PROMPT, launch_topk_prompt(v, F, np, keep, st));
+    }
     c->rel_clear = clear_after;
     a.sel = v.selp;
     a.sel_stride = v.max_prompt;

@@ -169,7 +169,7 @@ extern "C" int fastar_annca_select_noalloc(const void* q, const void* k_prompt, 
   if (r != FASTAR_OK) return r;
   // the accumulators are maxima: the part this call uses must start at zero (0 is below the word of every float)
   if (cudaMemsetAsync(v.rel, 0, static_cast<size_t>(num_heads) * F * np * 4, st) != cudaSuccess) return FASTAR_ERR_CUDA;
-  r = launch_c1_relevance(v, tm_q, tm_kp, nq, np, frame_len, st);
+  r = launch_c1_relevance(v, tm_q, tm_kp, nq, np, frame_len, 0, st);
   if (r < 0) return r;
   noalloc_topk_kernel<<<dim3(static_cast<unsigned>(F), num_heads), 256, np * 4, st>>>(kNoAllocHeaderWords, static_cast<int>(F), np,
                                                                                     keep_tokens, sel_out);

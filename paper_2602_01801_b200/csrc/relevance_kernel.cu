@@ -16,8 +16,11 @@
 // (18 and 19 only make up the warpgroup whose registers the epilogue takes over).
 #include "common.h"
 #include "ptx.cuh"
+#include "topk.cuh"
 
 namespace fastar {
+
+TopkArgs prompt_topk_args(const CacheView& c, int n_frames, int np, int keep);      // update_kernels.cu
 
 namespace {
 
@@ -34,6 +37,7 @@ struct RelArgs {
   int units;               // heads * prompt_groups * query_tiles
   const float* qn;         // CODE8: |q|, [H][max_tokens]
   const float* kn;         // CODE8: |k_p|, [H][max_prompt]
+  TopkArgs top;            // NV > 0: the ranking of a head's rows
 };
 
 template <int NKC>
@@ -45,7 +49,10 @@ struct Cfg {
 };
 
 // NKC: 128-byte chunks of a row (bf16: d / 64, codes: 1)
-template <int NKC, bool CODE8>
+// NV > 0: the CTA that finishes a head ranks its frames' tokens too (topk_row with NV registers), which saves a launch: as long on
+// the device (2 x 600 queries 6.5 + 2.4 -> 9.5 us, 12 x 4680 18.5 + 6.0 -> 24.6, its codes 18.0 + 7.3 -> 23.5, 40 x 10800 75.5 + 8.9 -> 83.0), but
+// a small step is bound by what the host spends on its launches (75.4 -> 71.2 us a pass).
+template <int NKC, bool CODE8, int NV>
 __global__ void __launch_bounds__(kThreads, 1)
 relevance_kernel(const __grid_constant__ CUtensorMap tm_p, const __grid_constant__ CUtensorMap tm_q, const CacheView c, const RelArgs g) {
   using SM = Cfg<NKC>;
@@ -65,9 +72,10 @@ relevance_kernel(const __grid_constant__ CUtensorMap tm_p, const __grid_constant
   const uint32_t bar_pfull = bar_tempty + 8 * kBuffers;
   const uint32_t bar_pempty = bar_pfull + 8;
   constexpr int kNumBars = 2 * S + 2 * kBuffers + 2;
-  static_assert(kNumBars * 8 + 8 <= SM::bars, "barrier area");
+  static_assert(kNumBars * 8 + 12 <= SM::bars, "barrier area");
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smem_raw + bar_off + kNumBars * 8);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(smem_raw + bar_off + kNumBars * 8 + 4);
+  volatile int* last_s = abort_flag + 1;
   const int warp = warp_index(), lane = threadIdx.x & 31;
 
   if (threadIdx.x < kNumBars) {
@@ -272,6 +280,24 @@ relevance_kernel(const __grid_constant__ CUtensorMap tm_p, const __grid_constant
       if (any) f_cur = f_last;
     }
     if (ok && f_cur >= 0) flush_all(cur, f_cur);
+    if constexpr (NV > 0) {
+      // A head's units are those of consecutive CTAs; each tells, after its last report, and the last one of a head has all maxima.  (Also
+      // after a time-out, so that the counters go back to zero.)
+      const int per_head = g.prompt_groups * g.query_tiles, h0 = u0 / per_head, h1 = (u1 - 1) / per_head;
+      auto cta_of = [&](int u) { return static_cast<int>((static_cast<int64_t>(u + 1) * gridDim.x - 1) / g.units); };
+      for (int h = h0; h <= h1; ++h) {
+        named_barrier_sync(1, kEpiWarps * 32);
+        if (threadIdx.x == 0) {
+          const int ctas = cta_of((h + 1) * per_head - 1) - cta_of(h * per_head) + 1;
+          const int last = atomic_add_acq_rel(c.rel_count + h, 1) == ctas - 1 ? 1 : 0;
+          if (last) c.rel_count[h] = 0;
+          *last_s = last;
+        }
+        named_barrier_sync(1, kEpiWarps * 32);
+        if (*last_s)
+          for (int row = warp; row < g.top.rows; row += kEpiWarps) topk_row<true, NV>(g.top, h, row);
+      }
+    }
   }
 
   tc_fence_before();
@@ -282,10 +308,10 @@ relevance_kernel(const __grid_constant__ CUtensorMap tm_p, const __grid_constant
   }
 }
 
-template <int NKC, bool CODE8>
-int launch_relevance(const CUtensorMap& tm_p, const CUtensorMap& tm_q, const CacheView& c, RelArgs g, cudaStream_t st) {
+template <int NKC, bool CODE8, int NV>
+int launch_relevance_t(const CUtensorMap& tm_p, const CUtensorMap& tm_q, const CacheView& c, RelArgs g, cudaStream_t st) {
   using SM = Cfg<NKC>;
-  auto kern = relevance_kernel<NKC, CODE8>;
+  auto kern = relevance_kernel<NKC, CODE8, NV>;
   const int cfg = ensure_dynamic_smem(reinterpret_cast<const void*>(kern), SM::total(kMaxGroup));
   if (cfg != FASTAR_OK) return cfg;
   int dev = 0, sm_count = 148;
@@ -310,28 +336,38 @@ int launch_relevance(const CUtensorMap& tm_p, const CUtensorMap& tm_q, const Cac
   return cudaGetLastError() == cudaSuccess ? 1 : FASTAR_ERR_CUDA;
 }
 
+// keep = 0: the maxima only; else the kept tokens of every frame too, by the steps of launch_topk.
+template <int NKC, bool CODE8>
+int launch_relevance(const CUtensorMap& tm_p, const CUtensorMap& tm_q, const CacheView& c, RelArgs g, int keep, cudaStream_t st) {
+  if (keep == 0) return launch_relevance_t<NKC, CODE8, 0>(tm_p, tm_q, c, g, st);
+  g.top = prompt_topk_args(c, (g.nq + g.frame_len - 1) / g.frame_len, g.np, keep);
+  if (g.np <= 128) return launch_relevance_t<NKC, CODE8, 4>(tm_p, tm_q, c, g, st);
+  if (g.np <= 512) return launch_relevance_t<NKC, CODE8, 16>(tm_p, tm_q, c, g, st);
+  return launch_relevance_t<NKC, CODE8, 36>(tm_p, tm_q, c, g, st);
+}
+
 }  // namespace
 
 // c.rel (zero before the call where it is used) receives the maxima as ordered integers.
 int launch_c1_relevance(const CacheView& c, const CUtensorMap& tm_q, const CUtensorMap& tm_kp, int nq, int np, int frame_len,
-                        cudaStream_t st) {
+                        int keep, cudaStream_t st) {
   RelArgs g{};
   g.nq = nq;
   g.np = np;
   g.frame_len = frame_len;
-  return c.D == 128 ? launch_relevance<2, false>(tm_kp, tm_q, c, g, st) : launch_relevance<1, false>(tm_kp, tm_q, c, g, st);
+  return c.D == 128 ? launch_relevance<2, false>(tm_kp, tm_q, c, g, keep, st) : launch_relevance<1, false>(tm_kp, tm_q, c, g, keep, st);
 }
 
 // The same on the 8-bit codes of the directions: code(q) . code(k_p) * |q| * |k_p|; the caller decodes with 1 / (256 sqrt(d)).
 int launch_c1_relevance_fp8(const CacheView& c, const CUtensorMap& tm_q8, const CUtensorMap& tm_kp8, const float* qn,
-                            const float* kn, int nq, int np, int frame_len, cudaStream_t st) {
+                            const float* kn, int nq, int np, int frame_len, int keep, cudaStream_t st) {
   RelArgs g{};
   g.nq = nq;
   g.np = np;
   g.frame_len = frame_len;
   g.qn = qn;
   g.kn = kn;
-  return launch_relevance<1, true>(tm_kp8, tm_q8, c, g, st);
+  return launch_relevance<1, true>(tm_kp8, tm_q8, c, g, keep, st);
 }
 
 }  // namespace fastar
