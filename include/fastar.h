@@ -21,7 +21,7 @@
  *     void* (0 = the legacy default stream).  All work is enqueued on that stream and the
  *     call returns without synchronising unless stated otherwise.
  *   - Ownership: the caller owns every tensor and the workspace buffer; the library owns only
- *     the small host object behind fastar_cache_t (with two CUDA streams and six events created and
+ *     the small host object behind fastar_cache_t (with four CUDA streams and their events created and
  *     destroyed with it).  Nothing here allocates device memory.
  *   - Tensors are [head][token][channel] with element strides `head_stride`, `token_stride`
  *     (channel stride 1).  Strides in bytes must be multiples of 16 and base pointers 16-byte
@@ -302,11 +302,12 @@ int fastar_annca_attention_lsh(fastar_cache_t* cache, const void* q, const void*
 /* One whole attention step with HOST tensors (contiguous [H][n][d] / [H][np][d], cache dtype):
  * copies the inputs to the device, runs update -> AnnSA -> AnnCA (same arguments as above, the
  * chunk's n tokens being both the new keys/values and the queries), copies both outputs back and
- * synchronises the stream.  Staging buffers live in the workspace.  The uploads of q and of the
- * prompt, AnnCA and the download of its output run on a second stream owned by the cache object,
- * beside the update, and the new values are uploaded last, on a third stream, while the
- * correspondence search (which reads only the keys) already runs; those streams start after the
- * work already queued on `stream` and are idle again when the call returns.
+ * synchronises the stream.  Staging buffers live in the workspace.  Copies and kernels go by
+ * slices of heads where the tensors are large, on streams owned by the cache object beside `stream`: the
+ * prompt, the keys, the queries and the values are uploaded in that order (the queries first where they are
+ * the probe), and each part starts when what it reads is there.  Those streams start after the work already
+ * queued on `stream` and are idle again when the call returns.  Arguments that one of the calls would refuse
+ * are refused before anything is queued.
  * flags: 0, or FASTAR_STEP_QUERY_PROBE to run the update as
  * fastar_tempcache_update_probe with q as the probe. */
 #define FASTAR_STEP_QUERY_PROBE 1

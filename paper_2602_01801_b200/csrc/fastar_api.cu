@@ -20,32 +20,52 @@ struct ProfRec {
   cudaEvent_t a, b;
 };
 
+// A range of heads as the kernels see it: the view whose arrays begin at its first head, and the maps that have a head coordinate.
+struct HeadRange {
+  CacheView v;
+  CUtensorMap tm_hq, tm_hk, tm_hk_hi;
+};
+constexpr int kMaxSlices = 4;                // of the host-tensor step
+
 struct fastar_cache {
   bool prof = false;
   std::vector<ProfRec> recs;
   fastar_cache_desc desc;
   CacheView v;
-  CUtensorMap tm_pool_k, tm_pool_v, tm_hq, tm_hk, tm_hk_hi, tm_pool_k8;
+  HeadRange all;
+  CUtensorMap tm_pool_k, tm_pool_v, tm_pool_k8;
   PFN_cuTensorMapEncodeTiled_v12000 encode;
   int64_t launches;
   size_t bytes;
-  // second stream of the host-tensor step (uploads of q and the prompt, AnnCA, its download) and its fork/join events
   int force_sink_blocks = 0, force_recent_blocks = 0;    // AnnSA selector option (fastar_cache_set_forced_blocks)
   // queries whose codes and block histograms fastar_annsa_prepare has already produced (consumed by the next matching AnnSA call)
   struct { const void* q = nullptr; int32_t nq = 0, block_q = 0; int64_t hs = 0, ts = 0; bool valid = false; } prep;
   bool rel_clear = true;     // AnnCA's relevance maxima are zero behind all work queued so far (create and every prompt top-k leave them so)
-  cudaEvent_t ev_prep = nullptr;
-  cudaStream_t side = nullptr, copy = nullptr;
-  cudaEvent_t ev_fork = nullptr, ev_q = nullptr, ev_join = nullptr, ev_p = nullptr, ev_v = nullptr;
+  // the host-tensor step's streams and events (fastar_attention_step_host); the events of a slice: its keys, queries and values are up,
+  // planned, queries hashed, AnnCA's and AnnSA's outputs are there
+  enum { kUp = 0, kSide, kAttend, kDown, kStreams };
+  enum { kKeysUp = 0, kQueriesUp, kValuesUp, kPlanned, kHashed, kCrossDone, kSelfDone, kSliceEvents };
+  cudaStream_t streams[kStreams] = {};
+  cudaEvent_t slice_ev[kMaxSlices][kSliceEvents] = {};
+  cudaEvent_t ev_fork = nullptr, ev_prompt = nullptr, ev_join = nullptr;
+  bool make_streams() {
+    for (cudaStream_t& s : streams)
+      if (cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking) != cudaSuccess) return false;
+    for (cudaEvent_t* e : {&ev_fork, &ev_prompt, &ev_join})
+      if (cudaEventCreateWithFlags(e, cudaEventDisableTiming) != cudaSuccess) return false;
+    for (auto& slice : slice_ev)
+      for (cudaEvent_t& e : slice)
+        if (cudaEventCreateWithFlags(&e, cudaEventDisableTiming) != cudaSuccess) return false;
+    return true;
+  }
   ~fastar_cache() {
-    if (ev_fork) cudaEventDestroy(ev_fork);
-    if (ev_q) cudaEventDestroy(ev_q);
-    if (ev_join) cudaEventDestroy(ev_join);
-    if (ev_p) cudaEventDestroy(ev_p);
-    if (ev_v) cudaEventDestroy(ev_v);
-    if (ev_prep) cudaEventDestroy(ev_prep);
-    if (side) cudaStreamDestroy(side);
-    if (copy) cudaStreamDestroy(copy);
+    for (cudaEvent_t e : {ev_fork, ev_prompt, ev_join})
+      if (e) cudaEventDestroy(e);
+    for (auto& slice : slice_ev)
+      for (cudaEvent_t e : slice)
+        if (e) cudaEventDestroy(e);
+    for (cudaStream_t s : streams)
+      if (s) cudaStreamDestroy(s);
   }
 };
 
@@ -225,6 +245,44 @@ int make_map_codes(fastar_cache* c, CUtensorMap* m, const void* ptr, uint64_t d1
   return r == CUDA_SUCCESS ? FASTAR_OK : FASTAR_ERR_CUDA;
 }
 
+// Heads [h0, h0 + count) of the cache.
+int make_range(fastar_cache* c, int h0, int count, HeadRange* out) {
+  CacheView v = c->v;
+  const int64_t h = h0, cap = h * v.CAP, mt = h * v.max_tokens, mp = h * v.max_prompt;
+  v.H = count;
+  v.page_table += h * v.CAPB;
+  v.n_match += h;
+  v.count += cap; v.stamp += cap; v.log2m += cap; v.rnorm += cap; v.kcode += cap; v.cnt += cap; v.cur += cap;
+  v.hk += h * v.CAPB * v.hist_cols;
+  v.len += h;
+  v.best += mt; v.segslot += mt; v.ulist += mt; v.rnorm_new += mt; v.code_new += mt; v.match += mt; v.sim += mt; v.order += mt;
+  v.dest += mt; v.victims += mt; v.code_q_ca += mt; v.code_q_sa += mt;
+  v.segpos += h * (v.max_tokens + 1);
+  v.plan += h;
+  v.hq += h * v.max_qb * v.hist_cols;
+  v.scores += h * v.max_qb * v.CAPB;
+  v.sel += h * v.max_qb * v.CAPB;
+  v.nsel += h;
+  v.rel += h * v.max_frames * v.max_prompt;
+  v.rel_count += h;
+  v.selp += h * v.max_frames * v.max_prompt;
+  v.nselp += h * v.max_frames;
+  v.code_p_ca += mp;
+  for (int i = 0; i < 6; ++i) v.stage[i] += (i == 3 || i == 4 ? mp : mt) * v.D;
+  if (v.stage_prep) v.stage_prep += mt * v.D;
+  if (v.hk_hi) { v.hk_hi += h * v.CAPB * v.hist_cols; v.scores_hi += h * v.max_qb * v.CAPB; }
+  if (v.k8_new) {
+    v.k8_new += mt * 128; v.q8_ca += mt * 128; v.q8_probe += mt * 128; v.kp8_ca += mp * 128;
+    v.qn_ca += mt; v.qn_probe += mt; v.kpn_ca += mp;
+  }
+  out->v = v;
+  const uint64_t row = static_cast<uint64_t>(v.hist_cols) * 2;
+  int r = make_map(c, &out->tm_hq, v.hq, v.hist_cols, v.max_qb, v.H, row, static_cast<uint64_t>(v.max_qb) * row, 128);
+  if (r == FASTAR_OK) r = make_map(c, &out->tm_hk, v.hk, v.hist_cols, v.CAPB, v.H, row, static_cast<uint64_t>(v.CAPB) * row, 64);
+  if (r == FASTAR_OK && v.hist_weighted) r = make_map(c, &out->tm_hk_hi, v.hk_hi, v.hist_cols, v.CAPB, v.H, row, static_cast<uint64_t>(v.CAPB) * row, 64);
+  return r;
+}
+
 // Block scores of weighted histograms as one number: lo + 256 * hi (exact in fp32 below 2^24).
 __global__ void combine_scores_kernel(const float* __restrict__ lo, const float* __restrict__ hi, int64_t head_stride,
                                       float* __restrict__ out, int per_head) {
@@ -287,7 +345,7 @@ bool rows_aligned(const fastar_cache* c, const void* p, int64_t hs, int64_t ts) 
   const int64_t esz = c->desc.dtype == FASTAR_FP32 ? 4 : 2;
   return !(reinterpret_cast<uintptr_t>(p) & 15) && !((hs * esz) & 15) && !((ts * esz) & 15);
 }
-int as_bf16(fastar_cache* c, View* v, int count, cudaStream_t st) {
+int as_bf16(fastar_cache* c, const CacheView& cv, View* v, int count, cudaStream_t st) {
   for (int i = 0; i < count; ++i) {
     if (!rows_aligned(c, v[i].src, v[i].hs, v[i].ts)) return FASTAR_ERR_INVALID_ARG;
     v[i].p = static_cast<const __nv_bfloat16*>(v[i].src);
@@ -296,12 +354,12 @@ int as_bf16(fastar_cache* c, View* v, int count, cudaStream_t st) {
   ConvertArgs a{};
   a.count = count;
   for (int i = 0; i < count; ++i) {
-    a.t[i] = {static_cast<const float*>(v[i].src), c->v.stage[v[i].slot], v[i].hs, v[i].ts, v[i].rows};
-    v[i].p = c->v.stage[v[i].slot];
-    v[i].hs = static_cast<int64_t>(v[i].rows) * c->v.D;
-    v[i].ts = c->v.D;
+    a.t[i] = {static_cast<const float*>(v[i].src), cv.stage[v[i].slot], v[i].hs, v[i].ts, v[i].rows};
+    v[i].p = cv.stage[v[i].slot];
+    v[i].hs = static_cast<int64_t>(v[i].rows) * cv.D;
+    v[i].ts = cv.D;
   }
-  ACCK(FASTAR_K_CONVERT, launch_convert_f32_to_bf16(a, c->v.H, c->v.D, st));
+  ACCK(FASTAR_K_CONVERT, launch_convert_f32_to_bf16(a, cv.H, cv.D, st));
   return FASTAR_OK;
 }
 
@@ -339,26 +397,10 @@ int fastar_cache_create(fastar_cache_t** out, const fastar_cache_desc* desc, con
   const uint64_t D = v.D, PT = v.PT;
   int r = make_map(c, &c->tm_pool_k, v.pool_k, D, PT, static_cast<uint64_t>(v.pool_pages), D * 2, PT * D * 2, v.PT);
   if (r == FASTAR_OK) r = make_map(c, &c->tm_pool_v, v.pool_v, D, PT, static_cast<uint64_t>(v.pool_pages), D * 2, PT * D * 2, v.PT);
-  if (r == FASTAR_OK)
-    r = make_map(c, &c->tm_hq, v.hq, v.hist_cols, v.max_qb, v.H, static_cast<uint64_t>(v.hist_cols) * 2,
-                 static_cast<uint64_t>(v.max_qb) * v.hist_cols * 2, 128);
-  if (r == FASTAR_OK)
-    r = make_map(c, &c->tm_hk, v.hk, v.hist_cols, v.CAPB, v.H, static_cast<uint64_t>(v.hist_cols) * 2,
-                 static_cast<uint64_t>(v.CAPB) * v.hist_cols * 2, 64);
-  if (r == FASTAR_OK && v.hist_weighted)
-    r = make_map(c, &c->tm_hk_hi, v.hk_hi, v.hist_cols, v.CAPB, v.H, static_cast<uint64_t>(v.hist_cols) * 2,
-                 static_cast<uint64_t>(v.CAPB) * v.hist_cols * 2, 64);
+  if (r == FASTAR_OK) r = make_range(c, 0, v.H, &c->all);
   if (r == FASTAR_OK && v.search_bits == 8)
     r = make_map_codes(c, &c->tm_pool_k8, v.pool_k8, PT, static_cast<uint64_t>(v.pool_pages), PT * 128, v.PT);
-  if (r == FASTAR_OK &&
-      (cudaStreamCreateWithFlags(&c->side, cudaStreamNonBlocking) != cudaSuccess ||
-       cudaStreamCreateWithFlags(&c->copy, cudaStreamNonBlocking) != cudaSuccess ||
-       cudaEventCreateWithFlags(&c->ev_p, cudaEventDisableTiming) != cudaSuccess ||
-       cudaEventCreateWithFlags(&c->ev_v, cudaEventDisableTiming) != cudaSuccess ||
-       cudaEventCreateWithFlags(&c->ev_prep, cudaEventDisableTiming) != cudaSuccess ||
-       cudaEventCreateWithFlags(&c->ev_fork, cudaEventDisableTiming) != cudaSuccess ||
-       cudaEventCreateWithFlags(&c->ev_q, cudaEventDisableTiming) != cudaSuccess ||
-       cudaEventCreateWithFlags(&c->ev_join, cudaEventDisableTiming) != cudaSuccess))
+  if (r == FASTAR_OK && !c->make_streams())
     r = FASTAR_ERR_CUDA;
   if (r != FASTAR_OK) {
     delete c;
@@ -547,27 +589,41 @@ int fastar_cache_import(fastar_cache_t* c, const uint16_t* host_k, const uint16_
   return cudaStreamSynchronize(st) == cudaSuccess ? FASTAR_OK : FASTAR_ERR_CUDA;
 }
 
-// One update; q_probe == nullptr is the key -> key cosine search, otherwise the cached keys are ranked by their dot
+// What update_impl does of an update: the search and the planning, which read only the keys, the commit, or both.  kCommitKeep leaves
+// the clock as it is (a range of heads that is not the last of an update).
+enum UpdatePart { kWhole, kSearch, kCommit, kCommitKeep };
+
+// One update of a range of heads; q_probe == nullptr is the key -> key cosine search, otherwise the cached keys are ranked by their dot
 // product with the probe rows and the threshold is applied to the key cosine of the winner.
-// v_ready (may be null): an event after which v_new may be read; the search and the planning, which read only the
-// keys, are queued before the wait.
-static int update_impl(fastar_cache_t* c, const void* q_probe, const void* k_new, const void* v_new, int32_t n, int32_t frame_len,
-                       int64_t head_stride, int64_t token_stride, float tau, int32_t* match_out, float* sim_out,
-                       int32_t* dest_out, fastar_update_stats* stats_out, void* stream, cudaEvent_t v_ready = nullptr) {
+static int update_impl(fastar_cache_t* c, const HeadRange& range, UpdatePart part, const void* q_probe, const void* k_new, const void* v_new,
+                       int32_t n, int32_t frame_len, int64_t head_stride, int64_t token_stride, float tau, int32_t* match_out,
+                       float* sim_out, int32_t* dest_out, fastar_update_stats* stats_out, void* stream) {
   if (!c || !k_new || !v_new || n < 1 || frame_len < 1) return FASTAR_ERR_INVALID_ARG;
   if (n > c->v.max_tokens || n > 16384 || n > c->v.CAP) return FASTAR_ERR_UNSUPPORTED_SHAPE;
   if (token_stride < c->v.D || head_stride < 0) return FASTAR_ERR_INVALID_ARG;
   if (q_probe && c->v.sign_codes) return FASTAR_ERR_UNSUPPORTED_SHAPE;      // the Hamming search compares keys with keys
   DeviceGuard guard(c->desc.device);
   cudaStream_t st = static_cast<cudaStream_t>(stream);
-  const CacheView& v = c->v;
-  const bool v_converted = c->desc.dtype != FASTAR_BF16;      // the entry conversion already reads v_new
-  if (v_ready && v_converted && cudaStreamWaitEvent(st, v_ready, 0) != cudaSuccess) return FASTAR_ERR_CUDA;
+  const CacheView& v = range.v;
+  // keys and values together (one stride for both); in parts, the search converts keys and probe and the commit the values
   View in[3] = {{k_new, n, 0, head_stride, token_stride, nullptr}, {v_new, n, 1, head_stride, token_stride, nullptr}, {q_probe, n, 2, head_stride, token_stride, nullptr}};
-  int r = as_bf16(c, in, q_probe ? 3 : 2, st);
+  int r;
+  if (part == kWhole) r = as_bf16(c, v, in, q_probe ? 3 : 2, st);
+  else r = as_bf16(c, v, part == kSearch ? in : in + 1, 1, st);
+  if (r == FASTAR_OK && part == kSearch && q_probe) r = as_bf16(c, v, in + 2, 1, st);
   if (r != FASTAR_OK) return r;
+  if (part == kCommit || part == kCommitKeep) {              // the keys were converted by the search
+    in[0].p = c->desc.dtype == FASTAR_BF16 ? static_cast<const __nv_bfloat16*>(k_new) : v.stage[0];
+    in[0].hs = in[1].hs;
+    in[0].ts = in[1].ts;
+  }
   const __nv_bfloat16 *kb = in[0].p, *vb = in[1].p, *pb = in[2].p;
   const int64_t khs = in[0].hs, kts = in[0].ts, phs = in[2].hs, pts = in[2].ts;      // K and V alike
+  if (part == kCommit || part == kCommitKeep) {
+    ACCK(FASTAR_K_COMMIT, launch_commit(v, kb, vb, n, frame_len, khs, kts, st));
+    ACCK(FASTAR_K_KEY_HIST, launch_finalize_hist(v, stats_out, part == kCommit ? 1 : 0, st));
+    return FASTAR_OK;
+  }
   CUtensorMap tm_a;
   r = q_probe ? make_map(c, &tm_a, pb, v.D, n, v.H, static_cast<uint64_t>(pts) * 2, static_cast<uint64_t>(phs) * 2, 128)
               : make_map(c, &tm_a, kb, v.D, n, v.H, static_cast<uint64_t>(kts) * 2, static_cast<uint64_t>(khs) * 2, 128);
@@ -600,7 +656,7 @@ static int update_impl(fastar_cache_t* c, const void* q_probe, const void* k_new
     ACCK(FASTAR_K_T1_SIMILARITY, launch_t1_search(vs, tm_a, c->tm_pool_k, n, st));
   }
   ACCK(FASTAR_K_PLAN, launch_plan(v, n, tau, UpdateOut{match_out, sim_out, dest_out}, st));
-  if (v_ready && !v_converted && cudaStreamWaitEvent(st, v_ready, 0) != cudaSuccess) return FASTAR_ERR_CUDA;
+  if (part == kSearch) return FASTAR_OK;
   ACCK(FASTAR_K_COMMIT, launch_commit(v, kb, vb, n, frame_len, khs, kts, st));
   ACCK(FASTAR_K_KEY_HIST, launch_finalize_hist(v, stats_out, 1, st));
   return FASTAR_OK;
@@ -609,20 +665,22 @@ static int update_impl(fastar_cache_t* c, const void* q_probe, const void* k_new
 int fastar_tempcache_update(fastar_cache_t* c, const void* k_new, const void* v_new, int32_t n, int32_t frame_len,
                             int64_t head_stride, int64_t token_stride, float tau, int32_t* match_out, float* sim_out,
                             int32_t* dest_out, fastar_update_stats* stats_out, void* stream) {
-  return update_impl(c, nullptr, k_new, v_new, n, frame_len, head_stride, token_stride, tau, match_out, sim_out, dest_out, stats_out,
+  if (!c) return FASTAR_ERR_INVALID_ARG;
+  return update_impl(c, c->all, kWhole, nullptr, k_new, v_new, n, frame_len, head_stride, token_stride, tau, match_out, sim_out, dest_out, stats_out,
                      stream);
 }
 
 int fastar_tempcache_update_probe(fastar_cache_t* c, const void* q_probe, const void* k_new, const void* v_new, int32_t n,
                                   int32_t frame_len, int64_t head_stride, int64_t token_stride, float tau, int32_t* match_out,
                                   float* sim_out, int32_t* dest_out, fastar_update_stats* stats_out, void* stream) {
-  if (!q_probe) return FASTAR_ERR_INVALID_ARG;
-  return update_impl(c, q_probe, k_new, v_new, n, frame_len, head_stride, token_stride, tau, match_out, sim_out, dest_out, stats_out,
+  if (!c || !q_probe) return FASTAR_ERR_INVALID_ARG;
+  return update_impl(c, c->all, kWhole, q_probe, k_new, v_new, n, frame_len, head_stride, token_stride, tau, match_out, sim_out, dest_out, stats_out,
                      stream);
 }
 
 // AnnSA; k_seg != nullptr adds the ns tokens of an un-cached K/V segment to every query's candidate set.
-static int annsa_impl(fastar_cache_t* c, const void* q, const void* k_seg, const void* v_seg, int32_t ns, int64_t seg_head_stride,
+// prepared: the queries' codes and block histograms are there.  cut: the place of the attention's parts is free.
+static int annsa_impl(fastar_cache_t* c, const HeadRange& range, bool prepared, bool cut, const void* q, const void* k_seg, const void* v_seg, int32_t ns, int64_t seg_head_stride,
                       int64_t seg_token_stride, void* out, int32_t nq, int64_t head_stride, int64_t token_stride, int32_t block_q,
                       int32_t keep_blocks, int32_t* sel_out, int32_t* nsel_out, uint32_t* qcode_out, float* scores_out,
                       const int32_t* sel_in, const int32_t* nsel_in, void* stream) {
@@ -635,13 +693,13 @@ static int annsa_impl(fastar_cache_t* c, const void* q, const void* k_seg, const
   if (!rows_aligned(c, out, head_stride, token_stride)) return FASTAR_ERR_INVALID_ARG;
   DeviceGuard guard(c->desc.device);
   cudaStream_t st = static_cast<cudaStream_t>(stream);
-  const CacheView& v = c->v;
+  const CacheView& v = range.v;
   const int nqb = (nq + block_q - 1) / block_q;
   const bool dense = !sel_in && keep_blocks >= v.CAPB;
   const int keep = keep_blocks < v.CAPB ? keep_blocks : v.CAPB;
   if (!dense && !sel_in && v.CAPB > 2048) return FASTAR_ERR_UNSUPPORTED_SHAPE;
   View in_q{q, nq, 2, head_stride, token_stride, nullptr};
-  int r = as_bf16(c, &in_q, 1, st);
+  int r = as_bf16(c, v, &in_q, 1, st);
   if (r != FASTAR_OK) return r;
   const __nv_bfloat16* qb = in_q.p;
   const int64_t qhs = in_q.hs, qts = in_q.ts;
@@ -650,6 +708,7 @@ static int annsa_impl(fastar_cache_t* c, const void* q, const void* k_seg, const
   if (r != FASTAR_OK) return r;
   AttnArgs a{};
   a.nq = nq;
+  a.no_cut = !cut;
   a.block_q = block_q;
   a.out = out;
   a.out_fp32 = c->desc.dtype == FASTAR_FP32;
@@ -662,17 +721,14 @@ static int annsa_impl(fastar_cache_t* c, const void* q, const void* k_seg, const
     a.sel_head_stride = static_cast<int64_t>(nqb) * keep_blocks;
     a.keep = keep_blocks;
   } else if (!dense) {
-    const bool prepared = c->prep.valid && c->prep.q == q && c->prep.nq == nq && c->prep.block_q == block_q &&
-                          c->prep.hs == head_stride && c->prep.ts == token_stride;
-    c->prep.valid = false;
     if (!prepared) {
       ACCK(FASTAR_K_HASH, launch_query_blocks(v, qb, nq, qhs, qts, block_q, st));
     }
-    ACCK(FASTAR_K_S3_SCORES, launch_s3_scores(v, c->tm_hq, c->tm_hk, nqb, st));
+    ACCK(FASTAR_K_S3_SCORES, launch_s3_scores(v, range.tm_hq, range.tm_hk, nqb, st));
     if (v.hist_weighted) {                   // the high digits of the weighted histograms, into their own score array
       CacheView vh = v;
       vh.scores = v.scores_hi;
-      ACCK(FASTAR_K_S3_SCORES, launch_s3_scores(vh, c->tm_hq, c->tm_hk_hi, nqb, st));
+      ACCK(FASTAR_K_S3_SCORES, launch_s3_scores(vh, range.tm_hq, range.tm_hk_hi, nqb, st));
     }
     ACCK(FASTAR_K_TOPK_BLOCKS, launch_topk_blocks(v, nqb, keep, c->force_sink_blocks, c->force_recent_blocks, st));
     a.sel = v.sel;
@@ -704,9 +760,9 @@ static int annsa_impl(fastar_cache_t* c, const void* q, const void* k_seg, const
   CUtensorMap tm_sk, tm_sv;
   if (k_seg) {
     // the update's staging slots are free during an attention call (where the segment has to be converted, no items are cut)
-    a.no_cut = c->desc.dtype != FASTAR_BF16;
+    a.no_cut = a.no_cut || c->desc.dtype != FASTAR_BF16;
     View sg[2] = {{k_seg, ns, 0, seg_head_stride, seg_token_stride, nullptr}, {v_seg, ns, 1, seg_head_stride, seg_token_stride, nullptr}};
-    r = as_bf16(c, sg, 2, st);
+    r = as_bf16(c, v, sg, 2, st);
     if (r == FASTAR_OK) r = make_map(c, &tm_sk, sg[0].p, v.D, ns, v.H, static_cast<uint64_t>(sg[0].ts) * 2, static_cast<uint64_t>(sg[0].hs) * 2, v.PT);
     if (r == FASTAR_OK) r = make_map(c, &tm_sv, sg[1].p, v.D, ns, v.H, static_cast<uint64_t>(sg[1].ts) * 2, static_cast<uint64_t>(sg[1].hs) * 2, v.PT);
     if (r != FASTAR_OK) return r;
@@ -721,16 +777,9 @@ static int annsa_impl(fastar_cache_t* c, const void* q, const void* k_seg, const
   return FASTAR_OK;
 }
 
-int fastar_annsa_prepare(fastar_cache_t* c, const void* q, int32_t nq, int64_t head_stride, int64_t token_stride, int32_t block_q,
-                         void* stream) {
-  if (!c || !q || nq < 1) return FASTAR_ERR_INVALID_ARG;
-  if (block_q != 64 && block_q != 128) return FASTAR_ERR_UNSUPPORTED_SHAPE;
-  if (nq > c->v.max_tokens) return FASTAR_ERR_UNSUPPORTED_SHAPE;
-  if (token_stride < c->v.D || head_stride < 0 || !rows_aligned(c, q, head_stride, token_stride)) return FASTAR_ERR_INVALID_ARG;
-  DeviceGuard guard(c->desc.device);
-  cudaStream_t st = static_cast<cudaStream_t>(stream);
-  const CacheView& v = c->v;
-  c->prep.valid = false;
+static int prepare_impl(fastar_cache_t* c, const HeadRange& range, const void* q, int32_t nq, int64_t head_stride, int64_t token_stride,
+                        int32_t block_q, cudaStream_t st) {
+  const CacheView& v = range.v;
   const __nv_bfloat16* qb = static_cast<const __nv_bfloat16*>(q);
   int64_t qhs = head_stride, qts = token_stride;
   if (c->desc.dtype == FASTAR_FP32) {          // own staging buffer: an update or another attention call may be converting too
@@ -743,28 +792,53 @@ int fastar_annsa_prepare(fastar_cache_t* c, const void* q, int32_t nq, int64_t h
     qts = v.D;
   }
   ACCK(FASTAR_K_HASH, launch_query_blocks(v, qb, nq, qhs, qts, block_q, st));
+  return FASTAR_OK;
+}
+
+int fastar_annsa_prepare(fastar_cache_t* c, const void* q, int32_t nq, int64_t head_stride, int64_t token_stride, int32_t block_q,
+                         void* stream) {
+  if (!c || !q || nq < 1) return FASTAR_ERR_INVALID_ARG;
+  if (block_q != 64 && block_q != 128) return FASTAR_ERR_UNSUPPORTED_SHAPE;
+  if (nq > c->v.max_tokens) return FASTAR_ERR_UNSUPPORTED_SHAPE;
+  if (token_stride < c->v.D || head_stride < 0 || !rows_aligned(c, q, head_stride, token_stride)) return FASTAR_ERR_INVALID_ARG;
+  DeviceGuard guard(c->desc.device);
+  cudaStream_t st = static_cast<cudaStream_t>(stream);
+  c->prep.valid = false;
+  const int r = prepare_impl(c, c->all, q, nq, head_stride, token_stride, block_q, st);
+  if (r != FASTAR_OK) return r;
   c->prep.q = q; c->prep.nq = nq; c->prep.block_q = block_q; c->prep.hs = head_stride; c->prep.ts = token_stride;
   c->prep.valid = true;
   return FASTAR_OK;
 }
 
+// Whether the prepared queries (fastar_annsa_prepare) are these; they serve one call that selects blocks.
+static bool take_prepared(fastar_cache_t* c, const void* q, int32_t nq, int64_t head_stride, int64_t token_stride, int32_t block_q,
+                          int32_t keep_blocks, const int32_t* sel_in) {
+  if (sel_in || keep_blocks >= c->v.CAPB) return false;
+  const bool prepared = c->prep.valid && c->prep.q == q && c->prep.nq == nq && c->prep.block_q == block_q && c->prep.hs == head_stride &&
+                        c->prep.ts == token_stride;
+  c->prep.valid = false;
+  return prepared;
+}
+
 int fastar_annsa_attention(fastar_cache_t* c, const void* q, void* out, int32_t nq, int64_t head_stride, int64_t token_stride,
                            int32_t block_q, int32_t keep_blocks, int32_t* sel_out, int32_t* nsel_out, uint32_t* qcode_out,
                            float* scores_out, const int32_t* sel_in, const int32_t* nsel_in, void* stream) {
-  return annsa_impl(c, q, nullptr, nullptr, 0, 0, 0, out, nq, head_stride, token_stride, block_q, keep_blocks, sel_out, nsel_out,
-                    qcode_out, scores_out, sel_in, nsel_in, stream);
+  if (!c) return FASTAR_ERR_INVALID_ARG;
+  return annsa_impl(c, c->all, take_prepared(c, q, nq, head_stride, token_stride, block_q, keep_blocks, sel_in), true, q, nullptr, nullptr, 0, 0, 0,
+                    out, nq, head_stride, token_stride, block_q, keep_blocks, sel_out, nsel_out, qcode_out, scores_out, sel_in, nsel_in, stream);
 }
 
 int fastar_annsa_attention_segment(fastar_cache_t* c, const void* q, const void* k_seg, const void* v_seg, void* out, int32_t nq,
                                    int32_t ns, int64_t head_stride, int64_t token_stride, int64_t seg_head_stride,
                                    int64_t seg_token_stride, int32_t block_q, int32_t keep_blocks, const int32_t* sel_in,
                                    const int32_t* nsel_in, void* stream) {
-  if (!k_seg || !v_seg) return FASTAR_ERR_INVALID_ARG;
-  return annsa_impl(c, q, k_seg, v_seg, ns, seg_head_stride, seg_token_stride, out, nq, head_stride, token_stride, block_q,
+  if (!c || !k_seg || !v_seg) return FASTAR_ERR_INVALID_ARG;
+  return annsa_impl(c, c->all, take_prepared(c, q, nq, head_stride, token_stride, block_q, keep_blocks, sel_in), true, q, k_seg, v_seg, ns, seg_head_stride, seg_token_stride, out, nq, head_stride, token_stride, block_q,
                     keep_blocks, nullptr, nullptr, nullptr, nullptr, sel_in, nsel_in, stream);
 }
 
-int fastar_annca_attention(fastar_cache_t* c, const void* q, const void* k_prompt, const void* v_prompt, void* out, int32_t nq,
+static int annca_impl(fastar_cache_t* c, const HeadRange& range, const void* q, const void* k_prompt, const void* v_prompt, void* out, int32_t nq,
                            int32_t frame_len, int32_t np, int32_t keep_tokens, int64_t head_stride, int64_t token_stride,
                            int64_t prompt_head_stride, int64_t prompt_token_stride, int32_t* sel_out, float* rel_out,
                            const int32_t* sel_in, void* stream) {
@@ -776,11 +850,11 @@ int fastar_annca_attention(fastar_cache_t* c, const void* q, const void* k_promp
   if (!rows_aligned(c, out, head_stride, token_stride)) return FASTAR_ERR_INVALID_ARG;
   DeviceGuard guard(c->desc.device);
   cudaStream_t st = static_cast<cudaStream_t>(stream);
-  const CacheView& v = c->v;
+  const CacheView& v = range.v;
   const int keep = keep_tokens < np ? keep_tokens : np;
   // own staging slots: may run beside an AnnSA call on another stream
   View in[3] = {{q, nq, 5, head_stride, token_stride, nullptr}, {k_prompt, np, 3, prompt_head_stride, prompt_token_stride, nullptr}, {v_prompt, np, 4, prompt_head_stride, prompt_token_stride, nullptr}};
-  int r = as_bf16(c, in, 3, st);
+  int r = as_bf16(c, v, in, 3, st);
   if (r != FASTAR_OK) return r;
   const __nv_bfloat16 *qb = in[0].p, *kpb = in[1].p, *vpb = in[2].p;
   const int64_t qhs = in[0].hs, qts = in[0].ts, khs = in[1].hs, kts = in[1].ts;      // K and V alike
@@ -812,7 +886,7 @@ int fastar_annca_attention(fastar_cache_t* c, const void* q, const void* k_promp
     cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
     if (!c->rel_clear && cudaStreamIsCapturing(st, &capture) != cudaSuccess) return FASTAR_ERR_CUDA;
     const bool clear_after = c->rel_clear || capture == cudaStreamCaptureStatusNone;
-    if (!c->rel_clear && cudaMemsetAsync(v.rel, 0, static_cast<size_t>(v.H) * v.max_frames * v.max_prompt * 4, st) != cudaSuccess)
+    if (!c->rel_clear && cudaMemsetAsync(c->v.rel, 0, static_cast<size_t>(c->v.H) * v.max_frames * v.max_prompt * 4, st) != cudaSuccess)
       return FASTAR_ERR_CUDA;
     c->rel_clear = false;
     const int ranked = rel_out ? 0 : keep;     // the maxima are wanted: they are ranked (and cleared) by a kernel behind their decoding
@@ -850,6 +924,15 @@ int fastar_annca_attention(fastar_cache_t* c, const void* q, const void* k_promp
   return FASTAR_OK;
 }
 
+int fastar_annca_attention(fastar_cache_t* c, const void* q, const void* k_prompt, const void* v_prompt, void* out, int32_t nq,
+                           int32_t frame_len, int32_t np, int32_t keep_tokens, int64_t head_stride, int64_t token_stride,
+                           int64_t prompt_head_stride, int64_t prompt_token_stride, int32_t* sel_out, float* rel_out,
+                           const int32_t* sel_in, void* stream) {
+  if (!c) return FASTAR_ERR_INVALID_ARG;
+  return annca_impl(c, c->all, q, k_prompt, v_prompt, out, nq, frame_len, np, keep_tokens, head_stride, token_stride, prompt_head_stride,
+                    prompt_token_stride, sel_out, rel_out, sel_in, stream);
+}
+
 int fastar_annca_attention_lsh(fastar_cache_t* c, const void* q, const void* k_prompt, const void* v_prompt, void* out, int32_t nq,
                                int32_t frame_len, int32_t np, int64_t head_stride, int64_t token_stride, int64_t prompt_head_stride,
                                int64_t prompt_token_stride, int32_t* sel_out, int32_t* nsel_out, uint32_t* qcode_out,
@@ -864,7 +947,7 @@ int fastar_annca_attention_lsh(fastar_cache_t* c, const void* q, const void* k_p
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   const CacheView& v = c->v;
   View in[3] = {{q, nq, 5, head_stride, token_stride, nullptr}, {k_prompt, np, 3, prompt_head_stride, prompt_token_stride, nullptr}, {v_prompt, np, 4, prompt_head_stride, prompt_token_stride, nullptr}};
-  int r = as_bf16(c, in, 3, st);
+  int r = as_bf16(c, v, in, 3, st);
   if (r != FASTAR_OK) return r;
   const __nv_bfloat16 *qb = in[0].p, *kpb = in[1].p, *vpb = in[2].p;
   const int64_t qhs = in[0].hs, qts = in[0].ts, khs = in[1].hs, kts = in[1].ts;      // K and V alike
@@ -920,62 +1003,122 @@ int fastar_attention_step_host(fastar_cache_t* c, const void* k_new_host, const 
   if (!c || !k_new_host || !v_new_host || !q_host || !k_prompt_host || !v_prompt_host || !out_sa_host || !out_ca_host)
     return FASTAR_ERR_INVALID_ARG;
   if (n < 1 || n > c->v.max_tokens || np < 1 || np > c->v.max_prompt) return FASTAR_ERR_UNSUPPORTED_SHAPE;
+  // what the calls below would refuse is refused before anything is queued
+  const CacheView& v = c->v;
+  const bool f32 = c->desc.dtype == FASTAR_FP32, probe = (flags & FASTAR_STEP_QUERY_PROBE) != 0, sparse = keep_blocks < v.CAPB;
+  if (frame_len < 1 || keep_blocks < 1 || keep_tokens < 1) return FASTAR_ERR_INVALID_ARG;
+  if ((block_q != 64 && block_q != 128) || n > v.CAP || n > 16384 || (sparse && v.CAPB > 2048) || (probe && v.sign_codes) ||
+      (n + min(frame_len, n) - 1) / min(frame_len, n) > v.max_frames)
+    return FASTAR_ERR_UNSUPPORTED_SHAPE;
   DeviceGuard guard(c->desc.device);
   cudaStream_t st = static_cast<cudaStream_t>(stream);
-  const CacheView& v = c->v;
-  const bool f32 = c->desc.dtype == FASTAR_FP32;
+  if (sparse) c->prep.valid = false;             // the queries of this call take the place of prepared ones
   const size_t esz = f32 ? 4 : 2;
   const void* hsrc[5] = {k_new_host, v_new_host, q_host, k_prompt_host, v_prompt_host};
   void* dsrc[5];
   for (int i = 0; i < 5; ++i) dsrc[i] = f32 ? v.stage_in_raw[i] : static_cast<void*>(v.stage[i]);
-  auto upload = [&](int i, cudaStream_t s) {
-    const size_t bytes = static_cast<size_t>(v.H) * (i < 3 ? n : np) * v.D * esz;
-    return cudaMemcpyAsync(dsrc[i], hsrc[i], bytes, cudaMemcpyHostToDevice, s) == cudaSuccess;
-  };
-  // Three streams, so that the copies and the two attentions overlap the cache update instead of queueing behind it.
-  // The host link is the bottleneck of this call, so the uploads are ordered by when their consumer can start:
-  // K first (the correspondence search and the planning read only the keys), then q and the prompt (AnnCA), V last
-  // (read by the merge at the end of the update).
-  //   caller's stream : upload K -> update [search, plan | wait V | merge] -> (q uploaded) AnnSA -> download its output
-  //   side stream     : upload q, prompt K/V -> AnnCA (reads no cache state) -> download its output
-  //   copy stream     : (prompt uploaded) upload V
-  // The owned streams start after everything already queued on the caller's stream and are joined before returning.
-  cudaStream_t sd = c->side, sc = c->copy;
-  const int64_t hs = static_cast<int64_t>(n) * v.D, ts = v.D, phs = static_cast<int64_t>(np) * v.D;
-  const size_t obytes = static_cast<size_t>(v.H) * n * v.D * esz;
-  if (cudaEventRecord(c->ev_fork, st) != cudaSuccess || cudaStreamWaitEvent(sd, c->ev_fork, 0) != cudaSuccess) return FASTAR_ERR_CUDA;
+  // The host link is the bottleneck of this call, so the work goes by slices of heads (heads are independent; a shared page pool has one
+  // slice) and every slice starts when its tensors are up, while the next ones still come and the outputs of those before leave:
+  //   up      : prompt, the keys of all slices, the queries, the values (the search and the planning read only the keys; the queries come
+  //             first where they are the probe)
+  //   caller's: (keys up) search, planning, slice by slice
+  //   side    : (queries up) their hash for AnnSA's selector, AnnCA
+  //   attend  : (planned, values up) commit, (hashed) AnnSA
+  //   down    : AnnCA's outputs, AnnSA's outputs
+  // 12 heads x 4680 tokens against 28 080 keys, bf16: 1 366 -> 1 190 us with four slices (46.3 MB up and 28.8 down take 952 at once), 1 277
+  // with two, 1 274 with six; 1 225 with the queries before the keys, 1 277 with AnnCA's output in one copy, 1 345 with the queries in one.
+  // A slice below 3 MB a tensor is not worth its launches (11 heads x 1 120, fp32, 6 MB: 660 -> 636 with two slices, 713 with three).  The
+  // owned streams start behind what the caller's stream holds and are joined before the call returns.
+  const size_t token_bytes = static_cast<size_t>(n) * v.D * esz, prompt_bytes = static_cast<size_t>(np) * v.D * esz, all_bytes = token_bytes * v.H;
+  int slices = static_cast<int>(all_bytes / (3u << 20));
+  slices = v.pool_shared || slices < 1 ? 1 : slices < kMaxSlices ? slices : kMaxSlices;
+  slices = slices < v.H ? slices : v.H;
+  HeadRange ranges[kMaxSlices];
+  int first[kMaxSlices + 1];
   int r = FASTAR_OK;
-  bool copies_ok = upload(0, st) && upload(2, sd);
-  copies_ok = copies_ok && cudaEventRecord(c->ev_q, sd) == cudaSuccess && upload(3, sd) && upload(4, sd) &&
-              cudaEventRecord(c->ev_p, sd) == cudaSuccess && cudaStreamWaitEvent(sc, c->ev_p, 0) == cudaSuccess && upload(1, sc);
-  // the query-side selector work (codes, block histograms) needs only q: it runs on the side stream, behind the uploads
-  // (the host link is the bottleneck) and before AnnCA
-  const bool sparse_sa = keep_blocks < v.CAPB;
-  if (copies_ok && sparse_sa && fastar_annsa_prepare(c, dsrc[2], n, static_cast<int64_t>(n) * v.D, v.D, block_q, sd) != FASTAR_OK) copies_ok = false;
-  if (cudaEventRecord(c->ev_prep, sd) != cudaSuccess) copies_ok = false;
-  // recorded even after a failed copy: the update below waits on it
-  copies_ok = (cudaEventRecord(c->ev_v, sc) == cudaSuccess) && copies_ok;
-  if (!copies_ok) r = FASTAR_ERR_CUDA;
-  const bool probe = (flags & FASTAR_STEP_QUERY_PROBE) != 0;
-  if (r == FASTAR_OK && probe && cudaStreamWaitEvent(st, c->ev_q, 0) != cudaSuccess) r = FASTAR_ERR_CUDA;   // the update reads q
-  if (r == FASTAR_OK)
-    r = update_impl(c, probe ? dsrc[2] : nullptr, dsrc[0], dsrc[1], n, frame_len, hs, ts, tau, nullptr, nullptr, nullptr, nullptr, st,
-                    c->ev_v);
-  if (r == FASTAR_OK)
-    r = fastar_annca_attention(c, dsrc[2], dsrc[3], dsrc[4], v.stage_out[1], n, frame_len, np, keep_tokens, hs, ts, phs, ts, nullptr,
-                               nullptr, nullptr, sd);
-  if (r == FASTAR_OK && cudaMemcpyAsync(out_ca_host, v.stage_out[1], obytes, cudaMemcpyDeviceToHost, sd) != cudaSuccess) r = FASTAR_ERR_CUDA;
-  if (r == FASTAR_OK && cudaStreamWaitEvent(st, c->ev_prep, 0) != cudaSuccess) r = FASTAR_ERR_CUDA;
-  if (r == FASTAR_OK)
-    r = fastar_annsa_attention(c, dsrc[2], v.stage_out[0], n, hs, ts, block_q, keep_blocks, nullptr, nullptr, nullptr, nullptr, nullptr,
-                               nullptr, st);
-  if (r == FASTAR_OK && cudaMemcpyAsync(out_sa_host, v.stage_out[0], obytes, cudaMemcpyDeviceToHost, st) != cudaSuccess) r = FASTAR_ERR_CUDA;
+  for (int i = 0; i <= slices; ++i) first[i] = v.H * i / slices;
+  for (int i = 0; i < slices && r == FASTAR_OK; ++i) r = make_range(c, first[i], first[i + 1] - first[i], &ranges[i]);
+  if (r != FASTAR_OK) return r;
+  cudaStream_t up = c->streams[c->kUp], side = c->streams[c->kSide], attend = c->streams[c->kAttend], down = c->streams[c->kDown];
+  auto try_cuda = [&](cudaError_t e) { if (e != cudaSuccess && r == FASTAR_OK) r = FASTAR_ERR_CUDA; };
+  auto at = [&](const void* base, int h, size_t head_bytes) { return static_cast<uint8_t*>(const_cast<void*>(base)) + h * head_bytes; };
+  auto upload = [&](int i, int h0, int h1, size_t head_bytes) {
+    try_cuda(cudaMemcpyAsync(at(dsrc[i], h0, head_bytes), at(hsrc[i], h0, head_bytes), (h1 - h0) * head_bytes, cudaMemcpyHostToDevice, up));
+  };
+  const int64_t hs = static_cast<int64_t>(n) * v.D, ts = v.D, phs = static_cast<int64_t>(np) * v.D;
+  try_cuda(cudaEventRecord(c->ev_fork, st));
+  for (cudaStream_t s : c->streams) try_cuda(cudaStreamWaitEvent(s, c->ev_fork, 0));
+  auto upload_prompt = [&]() {
+    upload(3, 0, v.H, prompt_bytes);
+    upload(4, 0, v.H, prompt_bytes);
+    try_cuda(cudaEventRecord(c->ev_prompt, up));
+  };
+  if (slices > 1) upload_prompt();
+  const int order[3] = {probe ? 2 : 0, probe ? 0 : 2, 1};                  // of the tensors of a slice: 0 keys, 1 values, 2 queries
+  constexpr int event_of[3] = {fastar_cache::kKeysUp, fastar_cache::kValuesUp, fastar_cache::kQueriesUp};
+  for (int t : order) {
+    if (slices == 1 && t == 1) upload_prompt();                            // one slice: whatever starts earliest first
+    for (int i = 0; i < slices; ++i) {
+      upload(t, first[i], first[i + 1], token_bytes);
+      try_cuda(cudaEventRecord(c->slice_ev[i][event_of[t]], up));
+    }
+  }
+  auto search = [&](int i) {
+    cudaEvent_t* ev = c->slice_ev[i];
+    void *k = at(dsrc[0], first[i], token_bytes), *vv = at(dsrc[1], first[i], token_bytes), *q = at(dsrc[2], first[i], token_bytes);
+    try_cuda(cudaStreamWaitEvent(st, ev[c->kKeysUp], 0));
+    if (probe) try_cuda(cudaStreamWaitEvent(st, ev[c->kQueriesUp], 0));
+    if (r == FASTAR_OK) r = update_impl(c, ranges[i], kSearch, probe ? q : nullptr, k, vv, n, frame_len, hs, ts, tau, nullptr, nullptr, nullptr, nullptr, st);
+    try_cuda(cudaEventRecord(ev[c->kPlanned], st));
+  };
+  auto cross = [&](int i) {
+    cudaEvent_t* ev = c->slice_ev[i];
+    void* q = at(dsrc[2], first[i], token_bytes);
+    if (i == 0) try_cuda(cudaStreamWaitEvent(side, c->ev_prompt, 0));
+    try_cuda(cudaStreamWaitEvent(side, ev[c->kQueriesUp], 0));
+    if (r == FASTAR_OK && sparse) r = prepare_impl(c, ranges[i], q, n, hs, ts, block_q, side);
+    try_cuda(cudaEventRecord(ev[c->kHashed], side));
+    if (r == FASTAR_OK)
+      r = annca_impl(c, ranges[i], q, at(dsrc[3], first[i], prompt_bytes), at(dsrc[4], first[i], prompt_bytes), at(v.stage_out[1], first[i], token_bytes), n,
+                     frame_len, np, keep_tokens, hs, ts, phs, ts, nullptr, nullptr, nullptr, side);
+    try_cuda(cudaEventRecord(ev[c->kCrossDone], side));
+  };
+  auto download = [&](int which, int i) {                                  // 0 AnnSA's output, 1 AnnCA's
+    try_cuda(cudaStreamWaitEvent(down, c->slice_ev[i][which ? c->kCrossDone : c->kSelfDone], 0));
+    try_cuda(cudaMemcpyAsync(at(which ? out_ca_host : out_sa_host, first[i], token_bytes), at(v.stage_out[which], first[i], token_bytes),
+                             (first[i + 1] - first[i]) * token_bytes, cudaMemcpyDeviceToHost, down));
+  };
+  // Issued in the order in which they can start: the host is only just ahead.  A copy to memory that is not pinned would hold the host
+  // until it is done, so such copies are issued last.
+  cudaPointerAttributes attr{};
+  const bool pinned = cudaPointerGetAttributes(&attr, out_ca_host) == cudaSuccess && attr.type != cudaMemoryTypeUnregistered;
+  for (int i = 0; i < slices && r == FASTAR_OK; ++i) search(i);
+  for (int i = 0; i < slices && r == FASTAR_OK; ++i) {
+    cross(i);
+    if (pinned) download(1, i);
+  }
+  for (int i = 0; i < slices && r == FASTAR_OK; ++i) {
+    cudaEvent_t* ev = c->slice_ev[i];
+    void *k = at(dsrc[0], first[i], token_bytes), *vv = at(dsrc[1], first[i], token_bytes), *q = at(dsrc[2], first[i], token_bytes);
+    try_cuda(cudaStreamWaitEvent(attend, ev[c->kPlanned], 0));
+    try_cuda(cudaStreamWaitEvent(attend, ev[c->kValuesUp], 0));
+    if (r == FASTAR_OK)
+      r = update_impl(c, ranges[i], i + 1 < slices ? kCommitKeep : kCommit, nullptr, k, vv, n, frame_len, hs, ts, tau, nullptr, nullptr, nullptr, nullptr, attend);
+    try_cuda(cudaStreamWaitEvent(attend, ev[c->kHashed], 0));
+    // (the attention's parts lie where the other slices' keys and values are)
+    if (r == FASTAR_OK)
+      r = annsa_impl(c, ranges[i], sparse, slices == 1, q, nullptr, nullptr, 0, 0, 0, at(v.stage_out[0], first[i], token_bytes), n, hs, ts, block_q, keep_blocks,
+                     nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, attend);
+    try_cuda(cudaEventRecord(ev[c->kSelfDone], attend));
+  }
+  for (int i = 0; i < slices && r == FASTAR_OK && !pinned; ++i) download(1, i);
+  for (int i = 0; i < slices && r == FASTAR_OK; ++i) download(0, i);
   // always join: the owned streams must be idle when this call returns, whatever happened above
-  const bool joined = cudaEventRecord(c->ev_join, sd) == cudaSuccess && cudaStreamWaitEvent(st, c->ev_join, 0) == cudaSuccess &&
-                      cudaStreamWaitEvent(st, c->ev_v, 0) == cudaSuccess && cudaStreamSynchronize(st) == cudaSuccess;
+  bool joined = true;
+  for (cudaStream_t s : c->streams) joined = cudaEventRecord(c->ev_join, s) == cudaSuccess && cudaStreamWaitEvent(st, c->ev_join, 0) == cudaSuccess && joined;
+  joined = cudaStreamSynchronize(st) == cudaSuccess && joined;
   if (!joined) {
-    cudaStreamSynchronize(sd);
-    cudaStreamSynchronize(sc);
+    for (cudaStream_t s : c->streams) cudaStreamSynchronize(s);
     return r != FASTAR_OK ? r : FASTAR_ERR_CUDA;
   }
   return r;

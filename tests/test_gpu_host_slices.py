@@ -1,0 +1,37 @@
+"""The host-tensor step in slices of heads: outputs and cache as by the device calls, bit for bit, where the heads do not divide evenly, with
+every search and a probe, over two steps (one clock for all slices).
+(Even numbers of key tiles: which of the attention's four groups adds up a sub-tile depends on the sub-tiles of the items before.)"""
+import numpy as np
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("H,n,d,fp32,bits,probe,capacity,keep", [(12, 4200, 128, False, 16, False, 8448, 8), (5, 5000, 128, True, 16, True, 10112, 10),
+                                                                 (3, 8200, 128, False, 8, False, 8448, 6), (1, 4096, 64, True, 8, True, 4352, 99)])
+def test_host_step_by_slices_equals_the_device_calls(H, n, d, fp32, bits, probe, capacity, keep):
+    import torch
+    from paper_2602_01801_b200 import fastar
+    g = torch.Generator().manual_seed(H * n)
+    dtype, np_, frame = (torch.float32 if fp32 else torch.bfloat16), 70, n // 2
+    lsh = np.random.default_rng(n).standard_normal((32, d)).astype(np.float32)
+    host, dev = (fastar.Cache(H, d, capacity, 128, lsh, max_tokens=n, max_prompt_tokens=np_, max_frames=3, fp32=fp32, search_bits=bits) for _ in range(2))
+    rand = lambda m: torch.randn(H, m, d, generator=g).to(dtype).pin_memory()
+    kp, vp = rand(np_), rand(np_)
+    k0 = rand(n)
+    for step in range(2):
+        # the second step finds most of the first one's keys again, appends a few and, where the cache is full, evicts
+        k, v, q = (k0 if step == 0 else torch.where(torch.rand(H, n, 1, generator=g) < 0.9, k0, rand(n)).pin_memory()), rand(n), rand(n)
+        sa, ca = torch.empty_like(q).pin_memory(), torch.empty_like(q).pin_memory()
+        host.step_host(k, v, q, kp, vp, sa, ca, frame, 0.9, 128, keep, 20, probe=probe)
+        dk, dv, dq = k.cuda(), v.cuda(), q.cuda()
+        dev.update(dk, dv, frame, 0.9, probe=dq if probe else None)
+        assert torch.equal(sa, dev.annsa(dq, 128, keep)["out"].cpu())
+        assert torch.equal(ca, dev.annca(dq, kp.cuda(), vp.cuda(), frame, 20)["out"].cpu())
+        assert host.status() == dev.status()
+        a, b = host.export_state(), dev.export_state()
+        assert all(np.array_equal(a[x], b[x]) for x in a)
+    with pytest.raises(fastar.FastarError):
+        host.step_host(k, v, q, kp, vp, sa, ca, frame, 0.9, 96, keep, 20)
+    c = host.export_state()
+    assert all(np.array_equal(a[x], c[x]) for x in a)          # refused before anything was queued
