@@ -146,6 +146,9 @@ int ensure_dynamic_smem(const void* kernel, int bytes);
 
 // gemm_kernels.cu
 int launch_s3_scores(const CacheView& c, const CUtensorMap& tm_hq, const CUtensorMap& tm_hk, int nqb, cudaStream_t st);
+bool s3_ranks(const CacheView& c, int nqb);
+int launch_s3_topk(const CacheView& c, const CUtensorMap& tm_hq, const CUtensorMap& tm_hk, int nqb, int keep, int force_sink, int force_recent,
+                   cudaStream_t st);
 
 // search_kernel.cu: T1 on the bf16 keys as one persistent kernel (c.raw_dot: plain dot products).  tm_pool_k: one page per box
 int launch_t1_search(const CacheView& c, const CUtensorMap& tm_a, const CUtensorMap& tm_pool_k, int n, cudaStream_t st);

@@ -724,13 +724,17 @@ static int annsa_impl(fastar_cache_t* c, const HeadRange& range, bool prepared, 
     if (!prepared) {
       ACCK(FASTAR_K_HASH, launch_query_blocks(v, qb, nq, qhs, qts, block_q, st));
     }
-    ACCK(FASTAR_K_S3_SCORES, launch_s3_scores(v, range.tm_hq, range.tm_hk, nqb, st));
-    if (v.hist_weighted) {                   // the high digits of the weighted histograms, into their own score array
-      CacheView vh = v;
-      vh.scores = v.scores_hi;
-      ACCK(FASTAR_K_S3_SCORES, launch_s3_scores(vh, range.tm_hq, range.tm_hk_hi, nqb, st));
+    if (s3_ranks(v, nqb)) {
+      ACCK(FASTAR_K_S3_SCORES, launch_s3_topk(v, range.tm_hq, range.tm_hk, nqb, keep, c->force_sink_blocks, c->force_recent_blocks, st));
+    } else {
+      ACCK(FASTAR_K_S3_SCORES, launch_s3_scores(v, range.tm_hq, range.tm_hk, nqb, st));
+      if (v.hist_weighted) {                   // the high digits of the weighted histograms, into their own score array
+        CacheView vh = v;
+        vh.scores = v.scores_hi;
+        ACCK(FASTAR_K_S3_SCORES, launch_s3_scores(vh, range.tm_hq, range.tm_hk_hi, nqb, st));
+      }
+      ACCK(FASTAR_K_TOPK_BLOCKS, launch_topk_blocks(v, nqb, keep, c->force_sink_blocks, c->force_recent_blocks, st));
     }
-    ACCK(FASTAR_K_TOPK_BLOCKS, launch_topk_blocks(v, nqb, keep, c->force_sink_blocks, c->force_recent_blocks, st));
     a.sel = v.sel;
     a.nsel = v.nsel;
     a.sel_stride = v.CAPB;

@@ -8,6 +8,7 @@
 // producer, warp 9 TMEM allocation + MMA issue.  Operands are bf16, K-major, 128-byte swizzled.
 #include "common.h"
 #include "ptx.cuh"
+#include "topk.cuh"
 
 
 namespace fastar {
@@ -15,6 +16,7 @@ namespace fastar {
 struct GemmArgs {
   int rows_a;              // valid rows of HQ per head (nqb)
   int nkc;                 // K chunks of 64
+  TopkArgs top;            // RANK: the ranking of the rows
 };
 
 constexpr int kChunkBytes = 128 * 128;       // 128 rows x 64 bf16
@@ -30,6 +32,9 @@ struct GemmSmem {
   static constexpr int total = bar_off + 256;
 };
 
+// RANK: a head's key blocks fit one tile and its query blocks are few, so the CTA has whole rows and ranks them too (a launch less: 2 heads,
+// 5 x 10 blocks 6.4 + 2.5 -> 7.8 us).
+template <bool RANK>
 __global__ void __launch_bounds__(kGemmThreads, 2)
 gemm_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__ CUtensorMap tm_b, const CacheView c,
             const GemmArgs g) {
@@ -185,17 +190,36 @@ gemm_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__ CU
     tc_fence_after();
     tmem_dealloc(tmem, kTmemCols);
   }
+  if (RANK)
+    for (int row = warp; row < g.rows_a; row += kGemmThreads / 32) topk_row<false, kTileN / 32>(g.top, h, row);
+}
+
+template <bool RANK>
+static int launch_gemm(const CacheView& c, const CUtensorMap& tm_hq, const CUtensorMap& tm_hk, const GemmArgs& g, cudaStream_t st) {
+  const int cfg = ensure_dynamic_smem(reinterpret_cast<const void*>(gemm_kernel<RANK>), GemmSmem::total);
+  if (cfg != FASTAR_OK) return cfg;
+  const int col_tiles = (c.CAPB + kTileN - 1) / kTileN;
+  launch_chained(gemm_kernel<RANK>, dim3((g.rows_a + 127) / 128, c.H, col_tiles), kGemmThreads, GemmSmem::total, st, tm_hq, tm_hk, c, g);
+  return cudaGetLastError() == cudaSuccess ? 1 : FASTAR_ERR_CUDA;
 }
 
 int launch_s3_scores(const CacheView& c, const CUtensorMap& tm_hq, const CUtensorMap& tm_hk, int nqb, cudaStream_t st) {
-  const int cfg = ensure_dynamic_smem(reinterpret_cast<const void*>(gemm_kernel), GemmSmem::total);
-  if (cfg != FASTAR_OK) return cfg;
   GemmArgs g{};
   g.rows_a = nqb;
   g.nkc = c.hist_cols / 64;
-  const int col_tiles = (c.CAPB + kTileN - 1) / kTileN;
-  launch_chained(gemm_kernel, dim3((nqb + 127) / 128, c.H, col_tiles), kGemmThreads, GemmSmem::total, st, tm_hq, tm_hk, c, g);
-  return cudaGetLastError() == cudaSuccess ? 1 : FASTAR_ERR_CUDA;
+  return launch_gemm<false>(c, tm_hq, tm_hk, g, st);
 }
+
+// Scores and the kept blocks.  One launch where a head's blocks fit one tile and a warp has two rows at most; more rows would wait for one
+// another in the few CTAs (a row is 1.5 us), and weighted histograms have two products to rank.
+int launch_s3_topk(const CacheView& c, const CUtensorMap& tm_hq, const CUtensorMap& tm_hk, int nqb, int keep, int force_sink, int force_recent,
+                   cudaStream_t st) {
+  GemmArgs g{};
+  g.rows_a = nqb;
+  g.nkc = c.hist_cols / 64;
+  g.top = block_topk_args(c, nqb, keep, force_sink, force_recent);
+  return launch_gemm<true>(c, tm_hq, tm_hk, g, st);
+}
+bool s3_ranks(const CacheView& c, int nqb) { return c.CAPB <= kTileN && nqb <= 2 * (kGemmThreads / 32) && !c.hist_weighted; }
 
 }  // namespace fastar

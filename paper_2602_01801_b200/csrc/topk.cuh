@@ -29,6 +29,8 @@ struct TopkArgs {
   int force_first, force_last;
   int* status;
 };
+TopkArgs block_topk_args(const CacheView& c, int nqb, int keep, int force_sink, int force_recent);      // update_kernels.cu
+
 // One row by one warp.
 template <bool PROMPT, int NV>
 __device__ __forceinline__ void topk_row(const TopkArgs& a, int h, int row) {

@@ -951,7 +951,7 @@ static int launch_topk(const TopkArgs& a, int columns, int H, cudaStream_t st) {
   return cudaGetLastError() == cudaSuccess ? 1 : FASTAR_ERR_CUDA;
 }
 
-int launch_topk_blocks(const CacheView& c, int nqb, int keep, int force_sink, int force_recent, cudaStream_t st) {
+TopkArgs block_topk_args(const CacheView& c, int nqb, int keep, int force_sink, int force_recent) {
   TopkArgs a{};
   a.src = c.scores;
   a.src_hi = c.hist_weighted ? c.scores_hi : nullptr;
@@ -967,7 +967,10 @@ int launch_topk_blocks(const CacheView& c, int nqb, int keep, int force_sink, in
   a.force_first = force_sink;
   a.force_last = force_recent;
   a.status = c.status;
-  return launch_topk<false>(a, c.CAPB, c.H, st);
+  return a;
+}
+int launch_topk_blocks(const CacheView& c, int nqb, int keep, int force_sink, int force_recent, cudaStream_t st) {
+  return launch_topk<false>(block_topk_args(c, nqb, keep, force_sink, force_recent), c.CAPB, c.H, st);
 }
 // ---------------------------------------------------------------------------------------------
 // AnnCA with the LSH bucket rule (Section 5.3): a prompt token is kept for a frame iff, in at least one table, a
