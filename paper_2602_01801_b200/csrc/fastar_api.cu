@@ -1095,7 +1095,8 @@ int fastar_attention_step_host(fastar_cache_t* c, const void* k_new_host, const 
   // Issued in the order in which they can start: the host is only just ahead.  A copy to memory that is not pinned would hold the host
   // until it is done, so such copies are issued last.
   cudaPointerAttributes attr{};
-  const bool pinned = cudaPointerGetAttributes(&attr, out_ca_host) == cudaSuccess && attr.type != cudaMemoryTypeUnregistered;
+  const bool known = cudaPointerGetAttributes(&attr, out_ca_host) == cudaSuccess, pinned = known && attr.type != cudaMemoryTypeUnregistered;
+  if (!known) cudaGetLastError();                // (not an error of the launches that follow)
   for (int i = 0; i < slices && r == FASTAR_OK; ++i) search(i);
   for (int i = 0; i < slices && r == FASTAR_OK; ++i) {
     cross(i);
