@@ -342,6 +342,7 @@ int launch_relevance(const CUtensorMap& tm_p, const CUtensorMap& tm_q, const Cac
   if (keep == 0) return launch_relevance_t<NKC, CODE8, 0>(tm_p, tm_q, c, g, st);
   g.top = prompt_topk_args(c, (g.nq + g.frame_len - 1) / g.frame_len, g.np, keep);
   if (g.np <= 128) return launch_relevance_t<NKC, CODE8, 4>(tm_p, tm_q, c, g, st);
+  if (g.np <= 256) return launch_relevance_t<NKC, CODE8, 8>(tm_p, tm_q, c, g, st);
   if (g.np <= 512) return launch_relevance_t<NKC, CODE8, 16>(tm_p, tm_q, c, g, st);
   return launch_relevance_t<NKC, CODE8, 36>(tm_p, tm_q, c, g, st);
 }

@@ -856,10 +856,15 @@ int plan_fused_smem(const CacheView& c, int n) {
 int launch_plan(const CacheView& c, int n, float tau, const UpdateOut& out, cudaStream_t st) {
   if (plan_is_fused(c, n)) {
     const int smem = plan_fused_smem(c, n);
-    if (n <= 1024) return launch_plan_fused<1>(c, n, tau, out, smem, st);
-    if (n <= 2048) return launch_plan_fused<2>(c, n, tau, out, smem, st);
-    if (n <= 4096) return launch_plan_fused<4>(c, n, tau, out, smem, st);
-    return launch_plan_fused<8>(c, n, tau, out, smem, st);
+    switch ((n + 1023) / 1024) {             // every pass over the tokens counts (12 x 4680 with 8 for 5: 14.8 us, with 5 12.0)
+      case 1: return launch_plan_fused<1>(c, n, tau, out, smem, st);
+      case 2: return launch_plan_fused<2>(c, n, tau, out, smem, st);
+      case 3: return launch_plan_fused<3>(c, n, tau, out, smem, st);
+      case 4: return launch_plan_fused<4>(c, n, tau, out, smem, st);
+      case 5: return launch_plan_fused<5>(c, n, tau, out, smem, st);
+      case 6: return launch_plan_fused<6>(c, n, tau, out, smem, st);
+      default: return launch_plan_fused<8>(c, n, tau, out, smem, st);
+    }
   }
   const int cfg = ensure_dynamic_smem(reinterpret_cast<const void*>(plan_kernel), 16384 * 8);
   if (cfg != FASTAR_OK) return cfg;
@@ -944,6 +949,7 @@ static int launch_topk(const TopkArgs& a, int columns, int H, cudaStream_t st) {
   const dim3 grid((a.rows + kTopkWarps - 1) / kTopkWarps, H);
   const int threads = 32 * kTopkWarps;
   if (columns <= 128) launch_chained(topk_kernel<PROMPT, 4>, grid, threads, 0, st, a);
+  else if (columns <= 256) launch_chained(topk_kernel<PROMPT, 8>, grid, threads, 0, st, a);
   else if (columns <= 512) launch_chained(topk_kernel<PROMPT, 16>, grid, threads, 0, st, a);
   else if (columns <= 1152) launch_chained(topk_kernel<PROMPT, 36>, grid, threads, 0, st, a);
   else if (columns <= 2048) launch_chained(topk_kernel<PROMPT, 64>, grid, threads, 0, st, a);
