@@ -55,7 +55,7 @@ struct CacheView {
   uint32_t* code_new;              // [H][max_tokens]  codes of new keys / of queries
   int32_t* match;                  // [H][max_tokens]
   float* sim;                      // [H][max_tokens]
-  int32_t* cnt;                    // [H][CAP]         tokens matched to each slot by this update (zeroed with `best`)
+  int32_t* cnt;                    // [H][CAP]         tokens matched to each slot by this update (cleared where the planner counts here)
   int32_t* cur;                    // [H][CAP]         scatter cursor of each touched slot
   int32_t* order;                  // [H][max_tokens]  matched token ids, grouped by slot (unordered inside a group)
   int32_t* segpos;                 // [H][max_tokens+1] start of each group in `order` (+ end sentinel)
@@ -225,6 +225,15 @@ struct ConvertArgs {
 };
 int launch_convert_f32_to_bf16(const ConvertArgs& a, int H, int D, cudaStream_t st);
 int launch_query_blocks(const CacheView& c, const __nv_bfloat16* q, int nq, int64_t hs, int64_t ts, int block_q, cudaStream_t st);
+struct UpdateScratch {               // what the first kernel of an update clears; a part that is not used is null and empty
+  unsigned long long* best;
+  int64_t n_best;                    // words
+  uint4* cnt;
+  int64_t n_cnt16;                   // 16-byte pieces
+  int32_t* n_match;
+  int32_t n_heads;
+};
+UpdateScratch update_scratch(const CacheView& c, int n);
 int launch_prep_update(const CacheView& c, const __nv_bfloat16* k_new, int n, int64_t hs, int64_t ts, cudaStream_t st);
 int launch_prep_codes_strided(const CacheView& c, const __nv_bfloat16* x, int n, int64_t hs, int64_t ts, uint32_t* code_out,
                               int64_t out_stride, cudaStream_t st);

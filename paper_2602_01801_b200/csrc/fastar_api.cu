@@ -149,7 +149,7 @@ size_t carve(const fastar_cache_desc& d, uint8_t* base, CacheView* v) {
   t.status = reinterpret_cast<int32_t*>(take(4));
   t.lsh = reinterpret_cast<__nv_bfloat16*>(take(32 * D * 2));
   t.best = reinterpret_cast<unsigned long long*>(take(H * MT * 8));
-  t.n_match = reinterpret_cast<int32_t*>(take(H * 4));              // between `best` and `cnt`: launch_prep_update clears all three
+  t.n_match = reinterpret_cast<int32_t*>(take(H * 4));
   t.cnt = reinterpret_cast<int32_t*>(take(H * CAP * 4));
   t.cur = reinterpret_cast<int32_t*>(take(H * CAP * 4));
   t.segslot = reinterpret_cast<int32_t*>(take(H * MT * 4));

@@ -122,11 +122,13 @@ template <int D, bool BLOCKS>
 __global__ void __launch_bounds__(256, 2) prep_kernel(const __nv_bfloat16* __restrict__ x, int H, int n, int64_t hs, int64_t ts,
                                                    const __nv_bfloat16* __restrict__ lsh, int T, int B,
                                                    uint32_t* __restrict__ code_out, float* __restrict__ rnorm_out,
-                                                   int64_t out_stride, uint4* __restrict__ zero, int64_t zero16, BlockHist bh) {
+                                                   int64_t out_stride, UpdateScratch clear, BlockHist bh) {
   __shared__ __align__(16) int hist[BLOCKS ? 1024 : 4];
   chain_wait();
-  for (int64_t q = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; q < zero16; q += static_cast<int64_t>(gridDim.x) * blockDim.x)
-    zero[q] = make_uint4(0, 0, 0, 0);
+  const int64_t thread = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x, threads = static_cast<int64_t>(gridDim.x) * blockDim.x;
+  for (int64_t q = thread; q < clear.n_best; q += threads) clear.best[q] = 0ull;
+  for (int64_t q = thread; q < clear.n_cnt16; q += threads) clear.cnt[q] = make_uint4(0, 0, 0, 0);
+  for (int64_t q = thread; q < clear.n_heads; q += threads) clear.n_match[q] = 0;
   constexpr int KS = D / 16;
   constexpr int RP = D + 8;                    // padded row of the staged projection matrix (bank-conflict free)
   __shared__ __align__(16) __nv_bfloat16 r_s[32 * RP];
@@ -268,16 +270,16 @@ __global__ void __launch_bounds__(256, 2) prep_kernel(const __nv_bfloat16* __res
   }
 }
 static int launch_prep_generic(const CacheView& c, const __nv_bfloat16* x, int n, int64_t hs, int64_t ts, uint32_t* code_out,
-                               float* rnorm_out, int64_t out_stride, cudaStream_t st, uint4* zero = nullptr, int64_t zero16 = 0) {
+                               float* rnorm_out, int64_t out_stride, cudaStream_t st, const UpdateScratch& clear = UpdateScratch{}) {
   if (n <= 0) return 0;
   const int groups = ((n + 15) / 16) * c.H;                      // 16 rows per warp pass
   // CTAs for the rows (eight warps of 16 a pass) or for the zeros (32 KB each), whichever needs more: a few tokens against many heads
   // with long caches leave far more to clear than to hash (40 heads x 65536 slots, 1 to 16 tokens: an update of 81 us with CTAs for
   // the rows only, 50 with these).
-  const int64_t want = max(static_cast<int64_t>(groups + 7) / 8, (zero16 + 2047) / 2048);
+  const int64_t want = max(static_cast<int64_t>(groups + 7) / 8, (clear.n_best / 2 + clear.n_cnt16 + 2047) / 2048);
   const dim3 grid(static_cast<unsigned>(max(static_cast<int64_t>(1), min(want, static_cast<int64_t>(2 * 148)))));
-  if (c.D == 128) launch_chained(prep_kernel<128, false>, grid, 256, 0, st, x, c.H, n, hs, ts, c.lsh, c.T, c.B, code_out, rnorm_out, out_stride, zero, zero16, BlockHist{});
-  else launch_chained(prep_kernel<64, false>, grid, 256, 0, st, x, c.H, n, hs, ts, c.lsh, c.T, c.B, code_out, rnorm_out, out_stride, zero, zero16, BlockHist{});
+  if (c.D == 128) launch_chained(prep_kernel<128, false>, grid, 256, 0, st, x, c.H, n, hs, ts, c.lsh, c.T, c.B, code_out, rnorm_out, out_stride, clear, BlockHist{});
+  else launch_chained(prep_kernel<64, false>, grid, 256, 0, st, x, c.H, n, hs, ts, c.lsh, c.T, c.B, code_out, rnorm_out, out_stride, clear, BlockHist{});
   return cudaGetLastError() == cudaSuccess ? 1 : FASTAR_ERR_CUDA;
 }
 // Codes of the queries and the bucket histograms of their blocks of block_q rows.
@@ -286,19 +288,30 @@ int launch_query_blocks(const CacheView& c, const __nv_bfloat16* q, int nq, int6
   const int64_t blocks = static_cast<int64_t>((nq + block_q - 1) / block_q) * c.H;
   const int grid = static_cast<int>(min(blocks, static_cast<int64_t>(2 * 148)));
   const BlockHist bh{c.hq, block_q, c.max_qb, c.hist_cols};
-  if (c.D == 128) launch_chained(prep_kernel<128, true>, grid, 256, 0, st, q, c.H, nq, hs, ts, c.lsh, c.T, c.B, c.code_q_sa, nullptr, c.max_tokens, nullptr, 0, bh);
-  else launch_chained(prep_kernel<64, true>, grid, 256, 0, st, q, c.H, nq, hs, ts, c.lsh, c.T, c.B, c.code_q_sa, nullptr, c.max_tokens, nullptr, 0, bh);
+  if (c.D == 128) launch_chained(prep_kernel<128, true>, grid, 256, 0, st, q, c.H, nq, hs, ts, c.lsh, c.T, c.B, c.code_q_sa, nullptr, c.max_tokens, UpdateScratch{}, bh);
+  else launch_chained(prep_kernel<64, true>, grid, 256, 0, st, q, c.H, nq, hs, ts, c.lsh, c.T, c.B, c.code_q_sa, nullptr, c.max_tokens, UpdateScratch{}, bh);
   return cudaGetLastError() == cudaSuccess ? 1 : FASTAR_ERR_CUDA;
 }
 bool plan_is_fused(const CacheView& c, int n);
 int plan_fused_smem(const CacheView& c, int n);
-// The first kernel of an update: codes and reciprocal norms of the new keys, and zeros in the words that the search and the
-// matching accumulate into (best, n_match and cnt lie side by side; a memset of its own cost 4 us with its two gaps).
+// The words that the search and the matching of an update accumulate into, as zeros (by a memset of their own they cost 4 us with its
+// two gaps): those of the view's heads and no others, because the view may be a range of heads whose neighbours are at work.  The
+// rows of `best` are max_tokens words of 8 bytes, so a range's first word may lie between two 16-byte boundaries.
+UpdateScratch update_scratch(const CacheView& c, int n) {
+  UpdateScratch z{};
+  z.best = c.best;
+  z.n_best = static_cast<int64_t>(c.H) * c.max_tokens;
+  if (!plan_is_fused(c, n)) {                // the planner in one kernel counts in its shared memory
+    z.cnt = reinterpret_cast<uint4*>(c.cnt);             // the capacity is a multiple of 128
+    z.n_cnt16 = static_cast<int64_t>(c.H) * c.CAP / 4;
+    z.n_match = c.n_match;
+    z.n_heads = c.H;
+  }
+  return z;
+}
+// The first kernel of an update: codes and reciprocal norms of the new keys, and the zeros.
 int launch_prep_update(const CacheView& c, const __nv_bfloat16* k_new, int n, int64_t hs, int64_t ts, cudaStream_t st) {
-  const uint8_t* end = plan_is_fused(c, n) ? reinterpret_cast<const uint8_t*>(c.best + ((static_cast<int64_t>(c.H) * c.max_tokens + 1) & ~1ll))
-                                           : reinterpret_cast<const uint8_t*>(c.cnt + static_cast<int64_t>(c.H) * c.CAP);
-  const int64_t bytes = end - reinterpret_cast<const uint8_t*>(c.best);
-  return launch_prep_generic(c, k_new, n, hs, ts, c.code_new, c.rnorm_new, c.max_tokens, st, reinterpret_cast<uint4*>(c.best), bytes / 16);
+  return launch_prep_generic(c, k_new, n, hs, ts, c.code_new, c.rnorm_new, c.max_tokens, st, update_scratch(c, n));
 }
 int launch_prep_codes_strided(const CacheView& c, const __nv_bfloat16* x, int n, int64_t hs, int64_t ts, uint32_t* code_out,
                               int64_t out_stride, cudaStream_t st) {
