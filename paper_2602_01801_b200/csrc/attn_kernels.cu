@@ -161,7 +161,7 @@ __device__ __forceinline__ void store_part(const CacheView& c, int slot, int g, 
   __stcg(part_stat(c, slot, g, r), make_float2(m, sum));
 }
 // Adds up a warp's share of the `parts` parts of an item, in the order of the pieces; returns the rows' sums.  A part without a live key
-// has a reference of -inf and no rows.
+// has a reference of -inf, a sum of 0 and no rows; one whose logits are NaN has the same reference and a sum of NaN, which has to reach the row.
 template <int D>
 __device__ __forceinline__ float merge_parts(const CacheView& c, int first_piece, int parts, int g, int r, uint32_t (&v)[32]) {
   float m = -INFINITY, sum = 0.f;
@@ -177,7 +177,7 @@ __device__ __forceinline__ float merge_parts(const CacheView& c, int first_piece
     float4 x[8];
 #pragma unroll
     for (int q = 0; q < 8; ++q) x[q] = __ldcg(src + q * 128);
-    if (ml.x == -INFINITY) continue;
+    if (ml.x == -INFINITY && ml.y == 0.f) continue;
     const float f = fast_exp2(ml.x - m);
     sum = fmaf(ml.y, f, sum);
 #pragma unroll

@@ -209,3 +209,43 @@ def test_items_cut_by_key_tiles(d, pt, H, nq, lens, seg, keep):
             # as above: rounding of the probabilities and of the output
             assert np.abs(got - want).max() <= 2.0 ** -7 * np.abs(vv).max(), f"head {h}, block {b}"
             assert np.linalg.norm(got - want) <= 1e-2 * np.linalg.norm(want), f"head {h}, block {b}"
+
+
+@pytest.mark.parametrize("d,pt", [(64, 64), (64, 128), (128, 64), (128, 128)])
+@pytest.mark.parametrize("whole_rounds", [False, True])
+def test_not_a_number_stays_in_its_rows(d, pt, whole_rounds):
+    """A query of NaN, a cached key of NaN: exactly the rows that they reach are NaN, whether items are cut by key tiles (a few of them) or not
+    (as many as there are SMs)."""
+    import torch
+    from paper_2602_01801_b200 import fastar
+    rng = np.random.default_rng(d + pt)
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    H, keep, blocks = 2, 33, 60
+    nq = 128 * (sms // H if whole_rounds else 3) - 28
+    nqb = -(-nq // 128)
+    q, k, v = (synth.round_bf16(rng.standard_normal((H, m, d)).astype(np.float32)) for m in (nq, blocks * pt, blocks * pt))
+    q[0, 5, 3] = np.nan
+    q[1, nq - 1] = np.inf
+    k[1, 7 * pt + 9, d - 1] = np.nan
+    lens = np.array([blocks * pt - 3, blocks * pt])
+    cap = -(-blocks * pt // 128) * 128
+    cache = fastar.Cache(H, d, cap, pt, rng.standard_normal((32, d)).astype(np.float32), max_tokens=nq)
+    cache.import_state(fastar.bf16_bits(k), fastar.bf16_bits(v), lens)
+    sel = np.stack([[np.sort(rng.permutation(blocks)[:keep]) for _ in range(nqb)] for _ in range(H)]).astype(np.int32)
+    nsel = torch.full((H,), keep, dtype=torch.int32, device="cuda")
+    out = cache.annsa(fastar.to_device(q), 128, keep, sel_in=torch.from_numpy(sel).cuda(), nsel_in=nsel)["out"].float().cpu().numpy()
+    assert cache.status() == 0
+    with np.errstate(invalid="ignore"):
+        for h in range(H):
+            for b in {0, 1, nqb // 2, nqb - 1}:
+                rows = slice(b * 128, min(nq, b * 128 + 128))
+                at = (sel[h, b][:, None] * pt + np.arange(pt)).reshape(-1)
+                at = at[at < lens[h]]
+                s = q[h, rows].astype(np.float64) @ k[h, at].T.astype(np.float64) / math.sqrt(d)
+                p = np.exp(s - s.max(1, keepdims=True))
+                want = (p / p.sum(1, keepdims=True)) @ v[h, at]
+                nan = np.isnan(want)
+                assert nan.any() == (7 in sel[1, b] if h == 1 and b < nqb - 1 else h == 1 or b == 0)
+                assert np.array_equal(np.isnan(out[h, rows]), nan)
+                # rounding of the probabilities and of the output
+                assert np.abs(out[h, rows] - want)[~nan].max(initial=0) <= 2.0 ** -7 * np.abs(v[h]).max()
