@@ -678,12 +678,20 @@ int fastar_tempcache_update_probe(fastar_cache_t* c, const void* q_probe, const 
                      stream);
 }
 
+// Whether the prepared queries (fastar_annsa_prepare) are these; they serve one call that selects blocks.
+static bool take_prepared(fastar_cache_t* c, const void* q, int32_t nq, int64_t head_stride, int64_t token_stride, int32_t block_q) {
+  const bool prepared = c->prep.valid && c->prep.q == q && c->prep.nq == nq && c->prep.block_q == block_q && c->prep.hs == head_stride &&
+                        c->prep.ts == token_stride;
+  c->prep.valid = false;
+  return prepared;
+}
+
 // AnnSA; k_seg != nullptr adds the ns tokens of an un-cached K/V segment to every query's candidate set.
-// prepared: the queries' codes and block histograms are there.  cut: the place of the attention's parts is free.
-static int annsa_impl(fastar_cache_t* c, const HeadRange& range, bool prepared, bool cut, const void* q, const void* k_seg, const void* v_seg, int32_t ns, int64_t seg_head_stride,
-                      int64_t seg_token_stride, void* out, int32_t nq, int64_t head_stride, int64_t token_stride, int32_t block_q,
-                      int32_t keep_blocks, int32_t* sel_out, int32_t* nsel_out, uint32_t* qcode_out, float* scores_out,
-                      const int32_t* sel_in, const int32_t* nsel_in, void* stream) {
+// hashed: the codes and block histograms of the range's queries are there.  cut: the place of the attention's parts is free.
+static int annsa_impl(fastar_cache_t* c, const HeadRange& range, bool hashed, bool cut, const void* q, const void* k_seg, const void* v_seg,
+                      int32_t ns, int64_t seg_head_stride, int64_t seg_token_stride, void* out, int32_t nq, int64_t head_stride,
+                      int64_t token_stride, int32_t block_q, int32_t keep_blocks, int32_t* sel_out, int32_t* nsel_out,
+                      uint32_t* qcode_out, float* scores_out, const int32_t* sel_in, const int32_t* nsel_in, void* stream) {
   if (!c || !q || !out || nq < 1 || keep_blocks < 1) return FASTAR_ERR_INVALID_ARG;
   if (k_seg && (!v_seg || ns < 1 || seg_token_stride < c->v.D || seg_head_stride < 0)) return FASTAR_ERR_INVALID_ARG;
   if (k_seg && ns > c->v.max_tokens) return FASTAR_ERR_UNSUPPORTED_SHAPE;
@@ -721,9 +729,8 @@ static int annsa_impl(fastar_cache_t* c, const HeadRange& range, bool prepared, 
     a.sel_head_stride = static_cast<int64_t>(nqb) * keep_blocks;
     a.keep = keep_blocks;
   } else if (!dense) {
-    if (!prepared) {
+    if (!hashed && !take_prepared(c, q, nq, head_stride, token_stride, block_q))
       ACCK(FASTAR_K_HASH, launch_query_blocks(v, qb, nq, qhs, qts, block_q, st));
-    }
     if (s3_ranks(v, nqb)) {
       ACCK(FASTAR_K_S3_SCORES, launch_s3_topk(v, range.tm_hq, range.tm_hk, nqb, keep, c->force_sink_blocks, c->force_recent_blocks, st));
     } else {
@@ -815,22 +822,12 @@ int fastar_annsa_prepare(fastar_cache_t* c, const void* q, int32_t nq, int64_t h
   return FASTAR_OK;
 }
 
-// Whether the prepared queries (fastar_annsa_prepare) are these; they serve one call that selects blocks.
-static bool take_prepared(fastar_cache_t* c, const void* q, int32_t nq, int64_t head_stride, int64_t token_stride, int32_t block_q,
-                          int32_t keep_blocks, const int32_t* sel_in) {
-  if (sel_in || keep_blocks >= c->v.CAPB) return false;
-  const bool prepared = c->prep.valid && c->prep.q == q && c->prep.nq == nq && c->prep.block_q == block_q && c->prep.hs == head_stride &&
-                        c->prep.ts == token_stride;
-  c->prep.valid = false;
-  return prepared;
-}
-
 int fastar_annsa_attention(fastar_cache_t* c, const void* q, void* out, int32_t nq, int64_t head_stride, int64_t token_stride,
                            int32_t block_q, int32_t keep_blocks, int32_t* sel_out, int32_t* nsel_out, uint32_t* qcode_out,
                            float* scores_out, const int32_t* sel_in, const int32_t* nsel_in, void* stream) {
   if (!c) return FASTAR_ERR_INVALID_ARG;
-  return annsa_impl(c, c->all, take_prepared(c, q, nq, head_stride, token_stride, block_q, keep_blocks, sel_in), true, q, nullptr, nullptr, 0, 0, 0,
-                    out, nq, head_stride, token_stride, block_q, keep_blocks, sel_out, nsel_out, qcode_out, scores_out, sel_in, nsel_in, stream);
+  return annsa_impl(c, c->all, false, true, q, nullptr, nullptr, 0, 0, 0, out, nq, head_stride, token_stride, block_q, keep_blocks, sel_out,
+                    nsel_out, qcode_out, scores_out, sel_in, nsel_in, stream);
 }
 
 int fastar_annsa_attention_segment(fastar_cache_t* c, const void* q, const void* k_seg, const void* v_seg, void* out, int32_t nq,
@@ -838,8 +835,8 @@ int fastar_annsa_attention_segment(fastar_cache_t* c, const void* q, const void*
                                    int64_t seg_token_stride, int32_t block_q, int32_t keep_blocks, const int32_t* sel_in,
                                    const int32_t* nsel_in, void* stream) {
   if (!c || !k_seg || !v_seg) return FASTAR_ERR_INVALID_ARG;
-  return annsa_impl(c, c->all, take_prepared(c, q, nq, head_stride, token_stride, block_q, keep_blocks, sel_in), true, q, k_seg, v_seg, ns, seg_head_stride, seg_token_stride, out, nq, head_stride, token_stride, block_q,
-                    keep_blocks, nullptr, nullptr, nullptr, nullptr, sel_in, nsel_in, stream);
+  return annsa_impl(c, c->all, false, true, q, k_seg, v_seg, ns, seg_head_stride, seg_token_stride, out, nq, head_stride, token_stride,
+                    block_q, keep_blocks, nullptr, nullptr, nullptr, nullptr, sel_in, nsel_in, stream);
 }
 
 static int annca_impl(fastar_cache_t* c, const HeadRange& range, const void* q, const void* k_prompt, const void* v_prompt, void* out, int32_t nq,

@@ -48,3 +48,32 @@ def test_rows_off_a_boundary_are_refused(fp32, search_bits):
         if name != "annsa":
             call(*[rows(0, good)] * args)
     assert cache.status() == fastar.OK
+
+
+@pytest.mark.parametrize("fp32", [False, True])
+def test_a_refused_call_leaves_the_prepared_queries(fp32):
+    import torch
+
+    from paper_2602_01801_b200 import fastar
+
+    H, d, n = 2, 64, 70
+    q = torch.randn(H, n, d, device="cuda", dtype=torch.float32 if fp32 else torch.bfloat16)
+    cache = fastar.Cache(H, d, 512, 64, np.random.default_rng(1).standard_normal((32, d)).astype(np.float32), max_tokens=n, fp32=fp32)
+    cache.update(q, q, n, 2.0)
+
+    def launches(call):
+        before = cache.launch_count()
+        out = call()["out"]
+        return cache.launch_count() - before, out
+
+    off = torch.empty(H * n * d + 1, device="cuda", dtype=q.dtype)[1:].view(H, n, d)
+    plain, want = launches(lambda: cache.annsa(q, 64, 3))
+    for refused in (lambda: cache.annsa(q, 96, 3), lambda: cache.annsa(q, 64, 0), lambda: cache.annsa(q, 64, 3, out=off),
+                    lambda: cache.annsa_segment(q, q[:, :0], q[:, :0], 64, 3)):
+        cache.annsa_prepare(q, 64)
+        with pytest.raises(fastar.FastarError):
+            refused()
+        prepared, out = launches(lambda: cache.annsa(q, 64, 3))
+        assert prepared == plain - 1
+        assert torch.equal(out, want)
+    assert cache.status() == fastar.OK
