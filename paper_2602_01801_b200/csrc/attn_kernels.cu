@@ -47,6 +47,8 @@
 #include "common.h"
 #include "ptx.cuh"
 
+#include <type_traits>
+
 namespace fastar {
 
 constexpr int kQChunk = 128 * 128;   // bytes of one 128-row x 64-column bf16 chunk
@@ -73,7 +75,13 @@ __device__ __forceinline__ float4 lds4(uint32_t addr) {
 // for values up to 2^119 / keys.  What the code calls the maximum, and the warps hand on, is that reference.
 constexpr float kHead = 16.f, kTop = 8.f;
 
-constexpr float kPartStore = 3.f, kPartAdd = 1.2f, kPartStop = 14.f, kPartGain = 0.05f;     // key tiles, see launch_attn
+// What a cut costs, in times of a tile of BKT keys (0.78 us with 128, 0.40 with 64): a part's way through memory, adding it up, another stop
+// of a CTA; a tile in the variant with the cut; and the share of the whole that has to be saved (see launch_attn).
+template <int BKT>
+struct CutCost {
+  static constexpr float store = BKT == 64 ? 6.f : 3.f, add = BKT == 64 ? 1.5f : 1.2f, stop = BKT == 64 ? 20.f : 14.f;
+  static constexpr float loop = BKT == 64 ? 1.2f : 1.f, gain = 0.05f;
+};
 
 template <int D, int BKT>
 struct AttnSmem {
@@ -214,9 +222,10 @@ __device__ __forceinline__ void write_row(const AttnArgs& a, int64_t off, const 
   }
 }
 
-// SEG (paged mode only): tiles of an un-cached K/V segment follow the cache tiles.  SPLIT (paged mode only): the last round's items are
-// cut by key tiles.
-template <int D, int BKT, bool GATHER, bool SEG, bool SPLIT>
+// SEG (paged mode only): tiles of an un-cached K/V segment follow the cache tiles.  CUT (paged mode only): the last round's items are
+// cut by key tiles if the longest of all items has `whole_below` tiles at least.  The launch knows how many tiles there can be, the device how
+// many there are; the kernel has both ways through it, and a CTA runs one of them.
+template <int D, int BKT, bool GATHER, bool SEG, bool CUT>
 __global__ void __launch_bounds__(kAttnThreads, 1)
 attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k,
             const __grid_constant__ CUtensorMap tm_v, const __grid_constant__ CUtensorMap tm_sk,
@@ -278,7 +287,7 @@ attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CU
   AttnPiece* piece_s = reinterpret_cast<AttnPiece*>(smem_raw + SM::bar_off + 480);
   volatile uint32_t* last_s = reinterpret_cast<volatile uint32_t*>(smem_raw + SM::bar_off + 496);      // cut items that this CTA has the last part of
   static_assert(kNumBars * 8 + 12 <= 480, "this CTA's piece");
-  if (SPLIT && threadIdx.x == 64) *piece_s = piece_of_cta(a);
+  if (CUT && threadIdx.x == 64) *piece_s = piece_of_cta(a);
   if (warp == kKeyWarp && lane == 0) {
     tma_prefetch_desc(&tm_q);
     if (!GATHER) { tma_prefetch_desc(&tm_k); tma_prefetch_desc(&tm_v); }
@@ -294,510 +303,523 @@ attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CU
   const uint32_t tmem = *tmem_slot;
   chain_wait();
 
-  // The item with its key tiles (warp-uniform)
-  auto item_of = [&](int it) {
-    AttnItem w = rows_of(it);
-    if (!GATHER) {
-      if (a.sel == nullptr) {
-        w.ntc = (__shfl_sync(0xffffffffu, c.len[w.h], 0) + BKT - 1) / BKT;
+  auto run = [&](auto way) {
+    constexpr bool SPLIT = decltype(way)::value;
+    // The item with its key tiles (warp-uniform)
+    auto item_of = [&](int it) {
+      AttnItem w = rows_of(it);
+      if (!GATHER) {
+        if (a.sel == nullptr) {
+          w.ntc = (__shfl_sync(0xffffffffu, c.len[w.h], 0) + BKT - 1) / BKT;
+        } else {
+          w.ntc = __shfl_sync(0xffffffffu, a.nsel[w.h], 0);
+          w.list = a.sel + static_cast<int64_t>(w.h) * a.sel_head_stride + static_cast<int64_t>(it % row_blocks) * a.sel_stride;
+        }
+        w.nt = w.ntc + (SEG ? a.seg_tiles : 0);
       } else {
-        w.ntc = __shfl_sync(0xffffffffu, a.nsel[w.h], 0);
-        w.list = a.sel + static_cast<int64_t>(w.h) * a.sel_head_stride + static_cast<int64_t>(it % row_blocks) * a.sel_stride;
+        const int f = it / (row_blocks * c.H);
+        w.keep_n = a.keep;
+        if (a.keep_frames) w.keep_n = __shfl_sync(0xffffffffu, a.keep_frames[static_cast<int64_t>(w.h) * a.keep_frames_stride + f], 0);
+        w.nt = (w.keep_n + BKT - 1) / BKT;
+        w.list = a.sel + static_cast<int64_t>(w.h) * a.sel_head_stride + static_cast<int64_t>(f) * a.sel_stride;
       }
-      w.nt = w.ntc + (SEG ? a.seg_tiles : 0);
-    } else {
-      const int f = it / (row_blocks * c.H);
-      w.keep_n = a.keep;
-      if (a.keep_frames) w.keep_n = __shfl_sync(0xffffffffu, a.keep_frames[static_cast<int64_t>(w.h) * a.keep_frames_stride + f], 0);
-      w.nt = (w.keep_n + BKT - 1) / BKT;
-      w.list = a.sel + static_cast<int64_t>(w.h) * a.sel_head_stride + static_cast<int64_t>(f) * a.sel_stride;
-    }
-    return w;
-  };
+      return w;
+    };
 
-  // The stops of a CTA: the items it, it + gridDim.x, ...; SPLIT: `rounds` of those, as it = 0, 1, ..., then its piece of the last round.
-  const int it_first = SPLIT ? 0 : blockIdx.x, it_step = SPLIT ? 1 : gridDim.x;
-  auto part_of = [&](int k) {
-    return AttnPart{piece_s->first + k, k == 0 ? piece_s->lo : 0, k + 1 == piece_s->n ? piece_s->hi : a.units};
-  };
-  auto more = [&](int it) { return SPLIT ? __shfl_sync(0xffffffffu, it < a.rounds + piece_s->n ? 1 : 0, 0) != 0 : it < items; };
-  auto item_at = [&](int it) {
-    if (!SPLIT) return it;
-    return __shfl_sync(0xffffffffu, static_cast<int>(it < a.rounds ? blockIdx.x + it * gridDim.x : a.rounds * gridDim.x + piece_s->first + it - a.rounds), 0);
-  };
-  auto tiles_of = [&](int it) {
-    if (GATHER) return item_of(it).nt;
-    const int h = item_at(it) / row_blocks % c.H;
-    const int nt = (a.sel ? __shfl_sync(0xffffffffu, a.nsel[h], 0) : (__shfl_sync(0xffffffffu, c.len[h], 0) + BKT - 1) / BKT) + (SEG ? a.seg_tiles : 0);
-    if (!SPLIT || it < a.rounds) return nt;
-    const AttnPart p = part_of(it - a.rounds);
-    return __shfl_sync(0xffffffffu, tile_at(a, nt, p.hi) - tile_at(a, nt, p.lo), 0);
-  };
+    // The stops of a CTA: the items it, it + gridDim.x, ...; SPLIT: `rounds` of those, as it = 0, 1, ..., then its piece of the last round.
+    const int it_first = SPLIT ? 0 : blockIdx.x, it_step = SPLIT ? 1 : gridDim.x;
+    auto part_of = [&](int k) {
+      return AttnPart{piece_s->first + k, k == 0 ? piece_s->lo : 0, k + 1 == piece_s->n ? piece_s->hi : a.units};
+    };
+    auto more = [&](int it) { return SPLIT ? __shfl_sync(0xffffffffu, it < a.rounds + piece_s->n ? 1 : 0, 0) != 0 : it < items; };
+    auto item_at = [&](int it) {
+      if (!SPLIT) return it;
+      return __shfl_sync(0xffffffffu, static_cast<int>(it < a.rounds ? blockIdx.x + it * gridDim.x : a.rounds * gridDim.x + piece_s->first + it - a.rounds), 0);
+    };
+    auto tiles_of = [&](int it) {
+      if (GATHER) return item_of(it).nt;
+      const int h = item_at(it) / row_blocks % c.H;
+      const int nt = (a.sel ? __shfl_sync(0xffffffffu, a.nsel[h], 0) : (__shfl_sync(0xffffffffu, c.len[h], 0) + BKT - 1) / BKT) + (SEG ? a.seg_tiles : 0);
+      if (!SPLIT || it < a.rounds) return nt;
+      const AttnPart p = part_of(it - a.rounds);
+      return __shfl_sync(0xffffffffu, tile_at(a, nt, p.hi) - tile_at(a, nt, p.lo), 0);
+    };
 
-  // Everything is counted through the items of a CTA: tile0 key tiles, tile0 * SUB sub-tiles before.  Key tile n is in K stage n % RK
-  // and V stage RK + n % RV.
+    // Everything is counted through the items of a CTA: tile0 key tiles, tile0 * SUB sub-tiles before.  Key tile n is in K stage n % RK
+    // and V stage RK + n % RV.
 
-  if (warp >= kSoftWarps) {
-    setmaxnreg_dec<kIssueRegs>();
-    if (warp == kKeyWarp || warp == kValueWarp) {
-      // ================================================================ copies: Q, K and the biases, or V
-      const bool is_k = warp == kKeyWarp;
-      const uint32_t first = is_k ? 0 : RK, end = is_k ? RK : RS;
-      uint32_t st = first, empty_phase = 1, copied = 0, n_q = 0;
-      bool ok = true;
-      for (int it = it_first; more(it) && ok; it += it_step) {
-        AttnItem w = item_of(item_at(it));
-        if (SPLIT && it >= a.rounds) {          // tiles [j0, j0 + nt): the list from there, or for all blocks in order the first block itself
-          const AttnPart p = part_of(it - a.rounds);
-          const int j0 = __shfl_sync(0xffffffffu, tile_at(a, w.nt, p.lo), 0);
-          w.list = a.sel ? w.list + j0 : reinterpret_cast<const int32_t*>(static_cast<intptr_t>(j0));
-          w.ntc -= j0;
-          w.nt = __shfl_sync(0xffffffffu, tile_at(a, w.nt, p.hi), 0) - j0;
-        }
-        const int nt = w.nt;
-        if (nt == 0) continue;
-        if (is_k) {
-          if (n_q > 0) ok = mbar_wait_warp<kIssueWaitHintNs>(bar_q_empty, (n_q - 1) & 1, abort_flag, c.status);
-          if (!ok) break;
-          if (lane == 0) {
-            mbar_arrive_expect_tx(bar_q_full, SM::q_bytes);
-            for (int kc = 0; kc < D / 64; ++kc) tma_load_3d(q_s + kc * kQChunk, &tm_q, bar_q_full, kc * 64, w.q0, w.h);
+    if (warp >= kSoftWarps) {
+      setmaxnreg_dec<kIssueRegs>();
+      if (warp == kKeyWarp || warp == kValueWarp) {
+        // ================================================================ copies: Q, K and the biases, or V
+        const bool is_k = warp == kKeyWarp;
+        const uint32_t first = is_k ? 0 : RK, end = is_k ? RK : RS;
+        uint32_t st = first, empty_phase = 1, copied = 0, n_q = 0;
+        bool ok = true;
+        for (int it = it_first; more(it) && ok; it += it_step) {
+          AttnItem w = item_of(item_at(it));
+          if (SPLIT && it >= a.rounds) {          // tiles [j0, j0 + nt): the list from there, or for all blocks in order the first block itself
+            const AttnPart p = part_of(it - a.rounds);
+            const int j0 = __shfl_sync(0xffffffffu, tile_at(a, w.nt, p.lo), 0);
+            w.list = a.sel ? w.list + j0 : reinterpret_cast<const int32_t*>(static_cast<intptr_t>(j0));
+            w.ntc -= j0;
+            w.nt = __shfl_sync(0xffffffffu, tile_at(a, w.nt, p.hi), 0) - j0;
           }
-          ++n_q;
-        }
-        // paged mode: block ids and page ids of 32 tiles at a time, one coalesced load each and one window ahead; lane 0 copies
-        int blk = 0, page = 0, blk_n = 0, page_n = 0;
-        auto fetch = [&](int j0) {
-          const int jj = j0 + lane;
-          if (GATHER) return;
-          if (SPLIT && jj >= nt) return;
-          if (jj < w.ntc) {
-            blk_n = FASTAR_IDX(a.sel ? w.list[jj] : SPLIT ? static_cast<int>(reinterpret_cast<intptr_t>(w.list)) + jj : jj, c.CAPB, c.status);
-            page_n = FASTAR_IDX(c.page_table[static_cast<int64_t>(w.h) * c.CAPB + blk_n], c.pool_pages, c.status);
-          } else if (SEG && jj < nt) {        // tile of the un-cached segment: its index, no page
-            blk_n = jj - w.ntc;
-            page_n = -1;
-          }
-        };
-        auto announce = [&](uint32_t stage) {     // gather mode: this warp's copies into the stage have landed
-          fence_proxy_async_smem();
-          __syncwarp();
-          if (lane == 0) mbar_arrive(bar_r_full + 8 * stage);
-        };
-        auto token = [&](int i) { return GATHER && i < w.keep_n ? FASTAR_IDX(w.list[i], a.np, c.status) : 0; };
-        int next = token(lane);                  // gather mode: 32 kept tokens, one per lane
-        fetch(0);
-        for (int j = 0; j < nt; ++j) {
-          if ((j & 31) == 0) {
-            blk = blk_n; page = page_n;
-            fetch(j + 32);
-          }
-          const int b = GATHER ? 0 : __shfl_sync(0xffffffffu, blk, j & 31), p = GATHER ? 0 : __shfl_sync(0xffffffffu, page, j & 31);
-          ok = mbar_wait_warp<kIssueWaitHintNs>(bar_r_empty + 8 * st, empty_phase, abort_flag, c.status);
-          if (!ok) break;
-          const uint32_t dst = ring_s + st * SM::kv_bytes;
-          if (!GATHER) {
-            if (lane == 0) {
-              const bool seg = SEG && p < 0;   // rows past the segment's end arrive as zeros and carry a -inf bias
-              const CUtensorMap* tm = seg ? (is_k ? &tm_sk : &tm_sv) : (is_k ? &tm_k : &tm_v);
-              mbar_arrive_expect_tx(bar_r_full + 8 * st, SM::kv_bytes + (is_k ? BKT * 4 : 0));
-              for (int kc = 0; kc < D / 64; ++kc)
-                tma_load_3d(dst + kc * BKT * 128, tm, bar_r_full + 8 * st, kc * 64, seg ? b * BKT : 0, seg ? w.h : p);
-              if (is_k) {
-                const float* bias_src = seg ? a.seg_bias + static_cast<int64_t>(b) * BKT : c.log2m + static_cast<int64_t>(w.h) * c.CAP + b * BKT;
-                bulk_load_1d(bias_s + (copied % NB) * BKT * 4, bias_src, BKT * 4, bar_r_full + 8 * st);
-              }
-            }
-          } else {
-            // Rows of K_p / V_p by index, as asynchronous 16-byte copies to their swizzled position.  A tile is announced when the
-            // copies of the next one are under way (it needs a stage that the tile before the announced one has left).
-            constexpr int CPR = D / 8, RPI = 32 / CPR;       // 16-byte chunks per row, rows per instruction
-            const int ch = lane % CPR;
-            const __nv_bfloat16* src = (is_k ? a.kp : a.vp) + static_cast<int64_t>(w.h) * a.p_head_stride + ch * 8;
-#pragma unroll 1
-            for (int i0 = 0; i0 < BKT; i0 += 32) {
-              const int idx = next;
-              next = token(j * BKT + i0 + 32 + lane);
-#pragma unroll 4
-              for (int r = 0; r < 32; r += RPI) {
-                const int i = i0 + r + lane / CPR;
-                const int tok = __shfl_sync(0xffffffffu, idx, i & 31);
-                cp_async16(dst + (ch >> 3) * (BKT * 128) + i * 128 + (((ch & 7) ^ (i & 7)) << 4),
-                           src + static_cast<int64_t>(tok) * a.p_token_stride, j * BKT + i < w.keep_n);
-              }
-            }
-            if (is_k)
-              for (int i = lane; i < BKT; i += 32)
-                asm volatile("st.shared.f32 [%0], %1;" ::"r"(bias_s + ((j % NB) * BKT + i) * 4), "f"((j * BKT + i < w.keep_n) ? 0.f : -INFINITY)
-                             : "memory");
-            asm volatile("cp.async.commit_group;" ::: "memory");
-            if (j > 0) asm volatile("cp.async.wait_group 1;" ::: "memory");
-            if (j > 0) announce(st == first ? end - 1 : st - 1);
-            if (j + 1 == nt) {
-              asm volatile("cp.async.wait_all;" ::: "memory");
-              announce(st);
-            }
-          }
-          ++copied;
-          if (++st == end) { st = first; empty_phase ^= 1; }
-        }
-        if (GATHER) break;                       // one item
-      }
-      // what is still in flight must land before the CTA may exit (normally the MMAs have consumed all of it)
-      if (GATHER) asm volatile("cp.async.wait_all;" ::: "memory");
-      if (lane == 0) {
-        if (n_q > 0) mbar_wait(bar_q_full, (n_q - 1) & 1, abort_flag, c.status);
-        if (!GATHER)
-          for (uint32_t s = first; s < end; ++s) {           // the last tile of stage s, if it has had one
-            const uint32_t r = end - first, had = (copied + r - 1 - (s - first)) / r;
-            if (had > 0) mbar_wait(bar_r_full + 8 * s, (had - 1) & 1, abort_flag, c.status);
-          }
-      }
-    } else if (warp == kQkWarp) {
-      // ================================================================ S = Q K_j^T
-      const uint32_t lead = elect_lane();
-      constexpr bool QT = SM::QT;
-      constexpr uint32_t idesc = make_idesc_bf16(128, QT ? 64 : BKT, 0);
-      const uint64_t qd = make_smem_desc(q_s, 16, 1024), kd0 = make_smem_desc(ring_s, 16, 1024);
-      bool ok = true;
-      uint32_t nq_used = 0, st = 0, r_phase = 0, b = 0, s_phase = 1;       // stage, logits' columns and their barriers' phases
-      for (int it = it_first; more(it) && ok; it += it_step) {
-        const int nt = tiles_of(it);
-        if (nt == 0) continue;
-        ok = mbar_wait_warp<kIssueWaitHintNs>(bar_q_full, nq_used & 1, abort_flag, c.status);
-        if (QT && ok && nq_used > 0) ok = mbar_wait_warp(bar_qk_done, (nq_used - 1) & 1, abort_flag, c.status);
-        if (!ok) break;
-        ++nq_used;
-        if (QT) {      // Q to tensor memory; the copies and the MMAs that read them are issued by one thread and execute in order
-          tc_fence_after();
-#pragma unroll
-          for (int kk = 0; kk < D / 16; ++kk) tmem_copy_128x256b(tmem + SM::q_col + kk * 8, qd + (((kk >> 2) * kQChunk + (kk & 3) * 32) >> 4), lead);
-          umma_commit(bar_q_empty, lead);
-        }
-        for (int j = 0; j < nt && ok; ++j) {
-          // the columns are free once the groups hold the logits before in registers
-          ok = mbar_wait<kIssueWaitHintNs>(bar_r_full + 8 * st, r_phase, abort_flag, c.status) && mbar_wait(bar_s_empty + 8 * b, s_phase, abort_flag, c.status);
-          ok = __all_sync(0xffffffffu, ok);
-          if (!ok) break;
-          tc_fence_after();
-          const uint64_t kd = kd0 + st * (SM::kv_bytes >> 4);
-          const uint32_t s_col = tmem + b * (QT ? 64 : BKT);
-#pragma unroll
-          for (int kk = 0; kk < D / 16; ++kk) {
-            const uint64_t bd = kd + (((kk >> 2) * (BKT * 128) + (kk & 3) * 32) >> 4);
-            if (QT) umma_ts(s_col, tmem + SM::q_col + kk * 8, bd, idesc, kk != 0, lead);
-            else umma_ss(s_col, qd + (((kk >> 2) * kQChunk + (kk & 3) * 32) >> 4), bd, idesc, kk != 0, lead);
-          }
-          umma_commit(bar_s_full + 8 * b, lead);
-          umma_commit(bar_r_empty + 8 * st, lead);
-          if (j + 1 == nt) umma_commit(QT ? bar_qk_done : bar_q_empty, lead);
-          if (lead) mbar_arrive(bar_s_full + 8 * b);     // what this warp has seen land (the biases) is there for the waiting warps
-          if (++st == RK) { st = 0; r_phase ^= 1; }
-          if (++b == SM::NSB) { b = 0; s_phase ^= 1; }
-        }
-      }
-    } else if (warp == kPvWarp) {
-      // ================================================================ O += P V_j
-      const uint32_t lead = elect_lane();
-      constexpr uint32_t idesc = make_idesc_bf16(128, D, 1);
-      const uint64_t vd0 = make_smem_desc(ring_s + RK * SM::kv_bytes, BKT * 128, 1024);
-      bool ok = true;
-      uint32_t n_done = 0, st = 0, r_phase = 0, b = 0, p_phase = 0;
-      for (int it = it_first; more(it) && ok; it += it_step) {
-        const int nt = tiles_of(it);
-        if (nt == 0) continue;
-        if (n_done > 0) ok = mbar_wait_warp(bar_o_free, (n_done - 1) & 1, abort_flag, c.status);
-        ++n_done;
-        for (int j = 0; j < nt && ok; ++j) {
-          ok = mbar_wait_warp(bar_r_full + 8 * (RK + st), r_phase, abort_flag, c.status);
-          const uint64_t vd = vd0 + st * (SM::kv_bytes >> 4);
-#pragma unroll
-          for (int sub = 0; sub < SUB; ++sub) {
-            ok = ok && mbar_wait_warp(bar_p_full + 8 * b, p_phase, abort_flag, c.status);
+          const int nt = w.nt;
+          if (nt == 0) continue;
+          if (is_k) {
+            if (n_q > 0) ok = mbar_wait_warp<kIssueWaitHintNs>(bar_q_empty, (n_q - 1) & 1, abort_flag, c.status);
             if (!ok) break;
+            if (lane == 0) {
+              mbar_arrive_expect_tx(bar_q_full, SM::q_bytes);
+              for (int kc = 0; kc < D / 64; ++kc) tma_load_3d(q_s + kc * kQChunk, &tm_q, bar_q_full, kc * 64, w.q0, w.h);
+            }
+            ++n_q;
+          }
+          // paged mode: block ids and page ids of 32 tiles at a time, one coalesced load each and one window ahead; lane 0 copies
+          int blk = 0, page = 0, blk_n = 0, page_n = 0;
+          auto fetch = [&](int j0) {
+            const int jj = j0 + lane;
+            if (GATHER) return;
+            if (SPLIT && jj >= nt) return;
+            if (jj < w.ntc) {
+              blk_n = FASTAR_IDX(a.sel ? w.list[jj] : SPLIT ? static_cast<int>(reinterpret_cast<intptr_t>(w.list)) + jj : jj, c.CAPB, c.status);
+              page_n = FASTAR_IDX(c.page_table[static_cast<int64_t>(w.h) * c.CAPB + blk_n], c.pool_pages, c.status);
+            } else if (SEG && jj < nt) {        // tile of the un-cached segment: its index, no page
+              blk_n = jj - w.ntc;
+              page_n = -1;
+            }
+          };
+          auto announce = [&](uint32_t stage) {     // gather mode: this warp's copies into the stage have landed
+            fence_proxy_async_smem();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(bar_r_full + 8 * stage);
+          };
+          auto token = [&](int i) { return GATHER && i < w.keep_n ? FASTAR_IDX(w.list[i], a.np, c.status) : 0; };
+          int next = token(lane);                  // gather mode: 32 kept tokens, one per lane
+          fetch(0);
+          for (int j = 0; j < nt; ++j) {
+            if ((j & 31) == 0) {
+              blk = blk_n; page = page_n;
+              fetch(j + 32);
+            }
+            const int b = GATHER ? 0 : __shfl_sync(0xffffffffu, blk, j & 31), p = GATHER ? 0 : __shfl_sync(0xffffffffu, page, j & 31);
+            ok = mbar_wait_warp<kIssueWaitHintNs>(bar_r_empty + 8 * st, empty_phase, abort_flag, c.status);
+            if (!ok) break;
+            const uint32_t dst = ring_s + st * SM::kv_bytes;
+            if (!GATHER) {
+              if (lane == 0) {
+                const bool seg = SEG && p < 0;   // rows past the segment's end arrive as zeros and carry a -inf bias
+                const CUtensorMap* tm = seg ? (is_k ? &tm_sk : &tm_sv) : (is_k ? &tm_k : &tm_v);
+                mbar_arrive_expect_tx(bar_r_full + 8 * st, SM::kv_bytes + (is_k ? BKT * 4 : 0));
+                for (int kc = 0; kc < D / 64; ++kc)
+                  tma_load_3d(dst + kc * BKT * 128, tm, bar_r_full + 8 * st, kc * 64, seg ? b * BKT : 0, seg ? w.h : p);
+                if (is_k) {
+                  const float* bias_src = seg ? a.seg_bias + static_cast<int64_t>(b) * BKT : c.log2m + static_cast<int64_t>(w.h) * c.CAP + b * BKT;
+                  bulk_load_1d(bias_s + (copied % NB) * BKT * 4, bias_src, BKT * 4, bar_r_full + 8 * st);
+                }
+              }
+            } else {
+              // Rows of K_p / V_p by index, as asynchronous 16-byte copies to their swizzled position.  A tile is announced when the
+              // copies of the next one are under way (it needs a stage that the tile before the announced one has left).
+              constexpr int CPR = D / 8, RPI = 32 / CPR;       // 16-byte chunks per row, rows per instruction
+              const int ch = lane % CPR;
+              const __nv_bfloat16* src = (is_k ? a.kp : a.vp) + static_cast<int64_t>(w.h) * a.p_head_stride + ch * 8;
+#pragma unroll 1
+              for (int i0 = 0; i0 < BKT; i0 += 32) {
+                const int idx = next;
+                next = token(j * BKT + i0 + 32 + lane);
+#pragma unroll 4
+                for (int r = 0; r < 32; r += RPI) {
+                  const int i = i0 + r + lane / CPR;
+                  const int tok = __shfl_sync(0xffffffffu, idx, i & 31);
+                  cp_async16(dst + (ch >> 3) * (BKT * 128) + i * 128 + (((ch & 7) ^ (i & 7)) << 4),
+                             src + static_cast<int64_t>(tok) * a.p_token_stride, j * BKT + i < w.keep_n);
+                }
+              }
+              if (is_k)
+                for (int i = lane; i < BKT; i += 32)
+                  asm volatile("st.shared.f32 [%0], %1;" ::"r"(bias_s + ((j % NB) * BKT + i) * 4), "f"((j * BKT + i < w.keep_n) ? 0.f : -INFINITY)
+                               : "memory");
+              asm volatile("cp.async.commit_group;" ::: "memory");
+              if (j > 0) asm volatile("cp.async.wait_group 1;" ::: "memory");
+              if (j > 0) announce(st == first ? end - 1 : st - 1);
+              if (j + 1 == nt) {
+                asm volatile("cp.async.wait_all;" ::: "memory");
+                announce(st);
+              }
+            }
+            ++copied;
+            if (++st == end) { st = first; empty_phase ^= 1; }
+          }
+          if (GATHER) break;                       // one item
+        }
+        // what is still in flight must land before the CTA may exit (normally the MMAs have consumed all of it)
+        if (GATHER) asm volatile("cp.async.wait_all;" ::: "memory");
+        if (lane == 0) {
+          if (n_q > 0) mbar_wait(bar_q_full, (n_q - 1) & 1, abort_flag, c.status);
+          if (!GATHER)
+            for (uint32_t s = first; s < end; ++s) {           // the last tile of stage s, if it has had one
+              const uint32_t r = end - first, had = (copied + r - 1 - (s - first)) / r;
+              if (had > 0) mbar_wait(bar_r_full + 8 * s, (had - 1) & 1, abort_flag, c.status);
+            }
+        }
+      } else if (warp == kQkWarp) {
+        // ================================================================ S = Q K_j^T
+        const uint32_t lead = elect_lane();
+        constexpr bool QT = SM::QT;
+        constexpr uint32_t idesc = make_idesc_bf16(128, QT ? 64 : BKT, 0);
+        const uint64_t qd = make_smem_desc(q_s, 16, 1024), kd0 = make_smem_desc(ring_s, 16, 1024);
+        bool ok = true;
+        uint32_t nq_used = 0, st = 0, r_phase = 0, b = 0, s_phase = 1;       // stage, logits' columns and their barriers' phases
+        for (int it = it_first; more(it) && ok; it += it_step) {
+          const int nt = tiles_of(it);
+          if (nt == 0) continue;
+          ok = mbar_wait_warp<kIssueWaitHintNs>(bar_q_full, nq_used & 1, abort_flag, c.status);
+          if (QT && ok && nq_used > 0) ok = mbar_wait_warp(bar_qk_done, (nq_used - 1) & 1, abort_flag, c.status);
+          if (!ok) break;
+          ++nq_used;
+          if (QT) {      // Q to tensor memory; the copies and the MMAs that read them are issued by one thread and execute in order
             tc_fence_after();
 #pragma unroll
-            for (int ks = 0; ks < 4; ++ks)
-              umma_ts(tmem + SM::o_col, tmem + SM::p_col + b * 32 + ks * 8, vd + (((sub * 4 + ks) * 2048) >> 4), idesc, (j | sub | ks) != 0, lead);
-            umma_commit(bar_pv_done + 8 * b, lead);
-            if (++b == kGroups) { b = 0; p_phase ^= 1; }
+            for (int kk = 0; kk < D / 16; ++kk) tmem_copy_128x256b(tmem + SM::q_col + kk * 8, qd + (((kk >> 2) * kQChunk + (kk & 3) * 32) >> 4), lead);
+            umma_commit(bar_q_empty, lead);
           }
-          if (!ok) break;
-          umma_commit(bar_r_empty + 8 * (RK + st), lead);
-          if (++st == RV) { st = 0; r_phase ^= 1; }
-        }
-      }
-      // tensor memory goes back when the soft-max warps are through (all of them get there, none waits for long)
-      mbar_wait_warp(bar_done, 0, done_flag, c.status);
-      tc_fence_after();
-      tmem_dealloc(tmem, SM::tmem_cols);
-    }
-  } else {
-    // ================================================================== soft-max groups + epilogue (512 threads)
-    setmaxnreg_inc<kSoftRegs>();
-    constexpr uint32_t kHalf = 16u << 16;               // the second sixteen lanes
-    // After a time-out a warp goes on to its last sub-tile without waiting, so that no other is ever left at a named barrier.
-    // (It reads and writes its columns of tensor memory all the same: with the loads behind `if (ok)` the logits would have to
-    // outlive their loop, which the registers do not allow.)
-    bool ok = true, s_ready = false;
-    int sub0 = 0, n_done = 0;                           // sub-tiles and items before
-    for (int it = it_first; more(it); it += it_step) {
-      const int ns = tiles_of(it) * SUB;
-      // what follows from these four is worked out again for every item: kept over the items it would not fit the registers
-      uint32_t sb_ = sbase, tm_ = tmem;
-      int wp_ = warp, ln_ = lane;
-      asm volatile("" : "+r"(sb_), "+r"(tm_), "+r"(wp_), "+r"(ln_));
-      const uint32_t sbase = sb_, tmem = tm_;
-      const int warp = wp_, lane = ln_;
-      const uint32_t bar_s_full = sbase + SM::bar_off + 16 + 16 * RS, bar_pv_done = bar_s_full + 32, bar_s_empty = bar_pv_done + 32;
-      const uint32_t bar_p_full = bar_s_empty + 32, bar_xchg = bar_p_full + 32, bar_o_free = bar_xchg + 8;
-      const int g = warp >> 2;                          // soft-max group: sub-tiles with index % kGroups == g
-      const uint32_t lane_t = tmem + (static_cast<uint32_t>((warp & 3) * 32) << 16);
-      const float scale = rsqrtf(static_cast<float>(D)) * 1.4426950408889634f;
-      const uint32_t p_t = lane_t + SM::p_col + g * 32, o_t = lane_t + SM::o_col;
-      const uint32_t max_s = sbase + SM::max_off + ((warp & 3) * 8 + (lane >> 2)) * 16;
-      const uint32_t bias_t = sbase + SM::bias_off + 8 * (lane & 3);
-      // the barriers of the hand-over (all sixteen: nothing else uses one after the roles part): this warp waits for the look at the
-      // sub-tile before, and tells of its own
-      const uint32_t heard = 4 * g + (warp & 3), told = 4 * ((g + 1) % kGroups) + (warp & 3);
-      float m[4];
-      float2 l[4];                                      // running maxima of rows 8 q + lane / 4; sums over the even and the odd columns
+          for (int j = 0; j < nt && ok; ++j) {
+            // the columns are free once the groups hold the logits before in registers
+            ok = mbar_wait<kIssueWaitHintNs>(bar_r_full + 8 * st, r_phase, abort_flag, c.status) && mbar_wait(bar_s_empty + 8 * b, s_phase, abort_flag, c.status);
+            ok = __all_sync(0xffffffffu, ok);
+            if (!ok) break;
+            tc_fence_after();
+            const uint64_t kd = kd0 + st * (SM::kv_bytes >> 4);
+            const uint32_t s_col = tmem + b * (QT ? 64 : BKT);
 #pragma unroll
-      for (int q = 0; q < 4; ++q) { m[q] = -INFINITY; l[q] = make_float2(0.f, 0.f); }
-      for (int t = (g - sub0) & (kGroups - 1); t < ns; t += kGroups) {
-        const int tg = sub0 + t, jg = tg / SUB;
-        const uint32_t sn = SM::QT ? tg : jg, sb = sn % SM::NSB;       // barrier of the logits
-        // QT: the group before has been told of its logits, so those of the three sub-tiles before are complete: a barrier's parity tells
-        // two phases apart, and the one before this sub-tile's is that of t - 3.  (At an item's first the groups have just met.)
-        if (SM::QT && t > 0) named_barrier_sync(heard, 64);
-        if (SM::QT || !s_ready) ok = ok && mbar_wait_warp(bar_s_full + 8 * sb, (sn / SM::NSB) & 1, abort_flag, c.status);
-        tc_fence_after();
-        // the logits of this warp's rows: x[hf][4 k + 2 e + c] is row 16 hf + 8 e + lane / 4, column 8 k + 2 (lane & 3) + c
-        uint32_t x[2][32];
-#pragma unroll
-        for (int hf = 0; hf < 2; ++hf)
-          tmem_ld_frag(lane_t + (SM::QT ? sb : g) * 64 + hf * kHalf, x[hf]);
-        const uint32_t bp = bias_t + ((jg % NB) * BKT + (tg % SUB) * 64) * 4;
-        float2 bias[8];
-#pragma unroll
-        for (int k = 0; k < 8; ++k) bias[k] = lds2(bp + 32 * k);
-        if (!SM::QT && t > 0) named_barrier_sync(heard, 64);
-        const float4 seen = t > 0 ? lds4(max_s) : make_float4(-INFINITY, -INFINITY, -INFINITY, -INFINITY);
-        bool p_free = tg < kGroups || mbar_test_wait(bar_pv_done + 8 * g, (tg / kGroups - 1) & 1);
-        tmem_wait_ld();
-        tc_fence_before();
-        mbar_arrive_warp(bar_s_empty + 8 * sb);          // the logits are in registers
-        float mx[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
-#pragma unroll
-        for (int k = 0; k < 8; ++k) {
-#pragma unroll
-          for (int q = 0; q < 4; ++q) {
-            uint32_t* v = &x[q >> 1][4 * k + 2 * (q & 1)];
-            const float2 y = ffma2(make_float2(__uint_as_float(v[0]), __uint_as_float(v[1])), make_float2(scale, scale), bias[k]);
-            v[0] = __float_as_uint(y.x);
-            v[1] = __float_as_uint(y.y);
-            mx[q] = fmax3(mx[q], y.x, y.y);
+            for (int kk = 0; kk < D / 16; ++kk) {
+              const uint64_t bd = kd + (((kk >> 2) * (BKT * 128) + (kk & 3) * 32) >> 4);
+              if (QT) umma_ts(s_col, tmem + SM::q_col + kk * 8, bd, idesc, kk != 0, lead);
+              else umma_ss(s_col, qd + (((kk >> 2) * kQChunk + (kk & 3) * 32) >> 4), bd, idesc, kk != 0, lead);
+            }
+            umma_commit(bar_s_full + 8 * b, lead);
+            umma_commit(bar_r_empty + 8 * st, lead);
+            if (j + 1 == nt) umma_commit(QT ? bar_qk_done : bar_q_empty, lead);
+            if (lead) mbar_arrive(bar_s_full + 8 * b);     // what this warp has seen land (the biases) is there for the waiting warps
+            if (++st == RK) { st = 0; r_phase ^= 1; }
+            if (++b == SM::NSB) { b = 0; s_phase ^= 1; }
           }
         }
-        // A logit makes this warp raise the maximum if it exceeds the last one by as much.  If none does, and nobody has raised it since
-        // this warp looked, the hand-over goes on at once: the maximum cannot change before this sub-tile is through, because whoever
-        // raises it waits for P V of all sub-tiles before.
-        // The first sub-tile's warp always goes the long way: it puts the maxima where the others read them, also those of a sub-tile
-        // without a live key (-inf; what lies there is an earlier item's).
-        bool may = t == 0;
+      } else if (warp == kPvWarp) {
+        // ================================================================ O += P V_j
+        const uint32_t lead = elect_lane();
+        constexpr uint32_t idesc = make_idesc_bf16(128, D, 1);
+        const uint64_t vd0 = make_smem_desc(ring_s + RK * SM::kv_bytes, BKT * 128, 1024);
+        bool ok = true;
+        uint32_t n_done = 0, st = 0, r_phase = 0, b = 0, p_phase = 0;
+        for (int it = it_first; more(it) && ok; it += it_step) {
+          const int nt = tiles_of(it);
+          if (nt == 0) continue;
+          if (n_done > 0) ok = mbar_wait_warp(bar_o_free, (n_done - 1) & 1, abort_flag, c.status);
+          ++n_done;
+          for (int j = 0; j < nt && ok; ++j) {
+            ok = mbar_wait_warp(bar_r_full + 8 * (RK + st), r_phase, abort_flag, c.status);
+            const uint64_t vd = vd0 + st * (SM::kv_bytes >> 4);
 #pragma unroll
-        for (int q = 0; q < 4; ++q) may |= mx[q] > m[q] + kTop;
-        may = __any_sync(0xffffffffu, may);
-        if (!may && t + 1 < ns) named_barrier_arrive(told, 64);
-        const float cur[4] = {seen.x, seen.y, seen.z, seen.w};
-        bool change = t == 0;
-#pragma unroll
-        for (int q = 0; q < 4; ++q) change |= mx[q] > cur[q] + kTop || cur[q] != m[q];
-        if (__any_sync(0xffffffffu, change)) {
-          float alpha[4];
-          bool raised = t == 0;
-#pragma unroll
-          for (int q = 0; q < 4; ++q) {
-            // the same for the four threads of a row
-            mx[q] = fmaxf(mx[q], __shfl_xor_sync(0xffffffffu, mx[q], 1));
-            mx[q] = fmaxf(mx[q], __shfl_xor_sync(0xffffffffu, mx[q], 2));
-            float top = cur[q];
-            alpha[q] = 1.f;
-            if (mx[q] > cur[q] + kTop) {
-              top = mx[q] + kHead;
-              alpha[q] = cur[q] == -INFINITY ? 0.f : fast_exp2(cur[q] - top);
-              raised = true;
-            }
-            // this thread's sum follows both the others' raises and its own
-            if (m[q] != top) {
-              const float f = m[q] == -INFINITY ? 0.f : fast_exp2(m[q] - top);
-              l[q].x *= f;
-              l[q].y *= f;
-            }
-            m[q] = top;
-          }
-          if (__any_sync(0xffffffffu, raised)) {
-            if (t > 0) {
-              // O is relative to the old maxima: P V of the sub-tile before must be in it, that of this one follows its P.
-              // (A parity tells only two phases apart, so the phase before has to be over: P V of sub-tile t - 4, which this group
-              // has to see done in any case, comes after that of t - 5.)
-              if (!__all_sync(0xffffffffu, p_free)) ok = ok && mbar_wait_warp(bar_pv_done + 8 * g, (tg / kGroups - 1) & 1, abort_flag, c.status);
-              p_free = true;
-              ok = ok && mbar_wait_warp(bar_pv_done + 8 * ((tg - 1) % kGroups), ((tg - 1) / kGroups) & 1, abort_flag, c.status);
+            for (int sub = 0; sub < SUB; ++sub) {
+              ok = ok && mbar_wait_warp(bar_p_full + 8 * b, p_phase, abort_flag, c.status);
+              if (!ok) break;
               tc_fence_after();
-              if (ok)
-#pragma unroll 1
-                for (int cc = 0; cc < 2 * (D / 32); ++cc) {
-                  const int hf = cc & 1;
-                  const uint32_t o_c = o_t + hf * kHalf + (cc >> 1) * 32;
-                  const float a0 = hf ? alpha[2] : alpha[0], a1 = hf ? alpha[3] : alpha[1];
-                  uint32_t v[16];
-                  tmem_ld_frag16(o_c, v);
-                  tmem_wait_ld();
 #pragma unroll
-                  for (int q = 0; q < 16; ++q) v[q] = __float_as_uint(__uint_as_float(v[q]) * ((q & 2) ? a1 : a0));
-                  tmem_st_frag16(o_c, v);
-                }
+              for (int ks = 0; ks < 4; ++ks)
+                umma_ts(tmem + SM::o_col, tmem + SM::p_col + b * 32 + ks * 8, vd + (((sub * 4 + ks) * 2048) >> 4), idesc, (j | sub | ks) != 0, lead);
+              umma_commit(bar_pv_done + 8 * b, lead);
+              if (++b == kGroups) { b = 0; p_phase ^= 1; }
             }
-            if ((lane & 3) == 0)
-              asm volatile("st.shared.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(max_s), "f"(m[0]), "f"(m[1]), "f"(m[2]), "f"(m[3]) : "memory");
-            __syncwarp();
+            if (!ok) break;
+            umma_commit(bar_r_empty + 8 * (RK + st), lead);
+            if (++st == RV) { st = 0; r_phase ^= 1; }
           }
         }
-        if (may && t + 1 < ns) named_barrier_arrive(told, 64);
-        // P is free once P V of the group's last sub-tile has read it
-        if (!__all_sync(0xffffffffu, p_free)) ok = ok && mbar_wait_warp(bar_pv_done + 8 * g, (tg / kGroups - 1) & 1, abort_flag, c.status);
+        // tensor memory goes back when the soft-max warps are through (all of them get there, none waits for long)
+        mbar_wait_warp(bar_done, 0, done_flag, c.status);
         tc_fence_after();
-        // exponentials -> bf16 P
-#pragma unroll
-        for (int hf = 0; hf < 2; ++hf) {
-          float2 neg[2];
-#pragma unroll
-          for (int e = 0; e < 2; ++e) neg[e].x = neg[e].y = m[2 * hf + e] == -INFINITY ? 0.f : -m[2 * hf + e];
-          uint32_t p[16];
-#pragma unroll
-          for (int k = 0; k < 8; ++k)
-#pragma unroll
-            for (int e = 0; e < 2; ++e) {
-              const uint32_t* v = &x[hf][4 * k + 2 * e];
-              const float2 u = fadd2(make_float2(__uint_as_float(v[0]), __uint_as_float(v[1])), neg[e]);
-              const float2 pr = make_float2(fast_exp2(u.x), fast_exp2(u.y));
-              const uint32_t b = pack_bf16x2(pr.x, pr.y);
-              p[2 * k + e] = b;
-              l[2 * hf + e] = fadd2(l[2 * hf + e], make_float2(__uint_as_float(b << 16), __uint_as_float(b & 0xFFFF0000u)));
-            }
-          tmem_st_half_frag(p_t + hf * kHalf, p);
-        }
-        const uint32_t jn = (tg + kGroups) / SUB;            // (asked here, needed later: a barrier answers slowly while MMAs run)
-        if (!SM::QT) s_ready = mbar_test_wait(bar_s_full + 8 * (jn % SM::NSB), (jn / SM::NSB) & 1);
-        tmem_wait_st();
-        tc_fence_before();
-        mbar_arrive_warp(bar_p_full + 8 * g);
-        if (!SM::QT) s_ready = __all_sync(0xffffffffu, s_ready);
+        tmem_dealloc(tmem, SM::tmem_cols);
       }
-      // ---- the groups meet: (m, l) of every row through shared memory ----
-      const uint32_t xchg = sbase + SM::xchg_off + (n_done & 1) * kGroups * 1024;
-      if (ns > 0) {
-        // the group of the last sub-tile waits for the last P V, the others for that group
-        const int last = sub0 + ns - 1;
-        if (g == last % kGroups) ok = ok && mbar_wait_warp(bar_pv_done + 8 * g, (last / kGroups) & 1, abort_flag, c.status);
+    } else {
+      // ================================================================== soft-max groups + epilogue (512 threads)
+      setmaxnreg_inc<kSoftRegs>();
+      constexpr uint32_t kHalf = 16u << 16;               // the second sixteen lanes
+      // After a time-out a warp goes on to its last sub-tile without waiting, so that no other is ever left at a named barrier.
+      // (It reads and writes its columns of tensor memory all the same: with the loads behind `if (ok)` the logits would have to
+      // outlive their loop, which the registers do not allow.)
+      bool ok = true, s_ready = false;
+      int sub0 = 0, n_done = 0;                           // sub-tiles and items before
+      for (int it = it_first; more(it); it += it_step) {
+        const int ns = tiles_of(it) * SUB;
+        // what follows from these four is worked out again for every item: kept over the items it would not fit the registers
+        uint32_t sb_ = sbase, tm_ = tmem;
+        int wp_ = warp, ln_ = lane;
+        asm volatile("" : "+r"(sb_), "+r"(tm_), "+r"(wp_), "+r"(ln_));
+        const uint32_t sbase = sb_, tmem = tm_;
+        const int warp = wp_, lane = ln_;
+        const uint32_t bar_s_full = sbase + SM::bar_off + 16 + 16 * RS, bar_pv_done = bar_s_full + 32, bar_s_empty = bar_pv_done + 32;
+        const uint32_t bar_p_full = bar_s_empty + 32, bar_xchg = bar_p_full + 32, bar_o_free = bar_xchg + 8;
+        const int g = warp >> 2;                          // soft-max group: sub-tiles with index % kGroups == g
+        const uint32_t lane_t = tmem + (static_cast<uint32_t>((warp & 3) * 32) << 16);
+        const float scale = rsqrtf(static_cast<float>(D)) * 1.4426950408889634f;
+        const uint32_t p_t = lane_t + SM::p_col + g * 32, o_t = lane_t + SM::o_col;
+        const uint32_t max_s = sbase + SM::max_off + ((warp & 3) * 8 + (lane >> 2)) * 16;
+        const uint32_t bias_t = sbase + SM::bias_off + 8 * (lane & 3);
+        // the barriers of the hand-over (all sixteen: nothing else uses one after the roles part): this warp waits for the look at the
+        // sub-tile before, and tells of its own
+        const uint32_t heard = 4 * g + (warp & 3), told = 4 * ((g + 1) % kGroups) + (warp & 3);
+        float m[4];
+        float2 l[4];                                      // running maxima of rows 8 q + lane / 4; sums over the even and the odd columns
 #pragma unroll
-        for (int q = 0; q < 4; ++q) {
-          float sum = l[q].x + l[q].y;
-          sum += __shfl_xor_sync(0xffffffffu, sum, 1);
-          sum += __shfl_xor_sync(0xffffffffu, sum, 2);
-          if ((lane & 3) == 0)
-            asm volatile("st.shared.v2.f32 [%0], {%1, %2};" ::"r"(xchg + (g * 128 + (warp & 3) * 32 + (lane >> 2) + 8 * q) * 8), "f"(m[q]), "f"(sum)
-                         : "memory");
-        }
-        mbar_arrive_warp(bar_xchg);
-        ok = mbar_wait_warp(bar_xchg, n_done & 1, abort_flag, c.status) && ok;
-        tc_fence_after();
-      }
-      const int r = (warp & 3) * 32 + lane;         // from here on a thread owns one row, 32 of its columns
-      if (ok && g < D / 32) {
-        // O is relative to the last maximum, which the group of the last sub-tile knows; the others may be some raises behind
-        uint32_t v[32];
-        float m_all = -INFINITY, denom = 0.f;
-        if (ns > 0) {
-          float2 part[kGroups];
+        for (int q = 0; q < 4; ++q) { m[q] = -INFINITY; l[q] = make_float2(0.f, 0.f); }
+        for (int t = (g - sub0) & (kGroups - 1); t < ns; t += kGroups) {
+          const int tg = sub0 + t, jg = tg / SUB;
+          const uint32_t sn = SM::QT ? tg : jg, sb = sn % SM::NSB;       // barrier of the logits
+          // QT: the group before has been told of its logits, so those of the three sub-tiles before are complete: a barrier's parity tells
+          // two phases apart, and the one before this sub-tile's is that of t - 3.  (At an item's first the groups have just met.)
+          if (SM::QT && t > 0) named_barrier_sync(heard, 64);
+          if (SM::QT || !s_ready) ok = ok && mbar_wait_warp(bar_s_full + 8 * sb, (sn / SM::NSB) & 1, abort_flag, c.status);
+          tc_fence_after();
+          // the logits of this warp's rows: x[hf][4 k + 2 e + c] is row 16 hf + 8 e + lane / 4, column 8 k + 2 (lane & 3) + c
+          uint32_t x[2][32];
 #pragma unroll
-          for (int q = 0; q < kGroups; ++q) {
-            part[q] = lds2(xchg + (q * 128 + r) * 8);
-            m_all = fmaxf(m_all, part[q].x);
-          }
+          for (int hf = 0; hf < 2; ++hf)
+            tmem_ld_frag(lane_t + (SM::QT ? sb : g) * 64 + hf * kHalf, x[hf]);
+          const uint32_t bp = bias_t + ((jg % NB) * BKT + (tg % SUB) * 64) * 4;
+          float2 bias[8];
 #pragma unroll
-          for (int q = 0; q < kGroups; ++q) denom += part[q].y * ((part[q].x == -INFINITY) ? 0.f : fast_exp2(part[q].x - m_all));
-          tmem_ld32(o_t + g * 32, v);
+          for (int k = 0; k < 8; ++k) bias[k] = lds2(bp + 32 * k);
+          if (!SM::QT && t > 0) named_barrier_sync(heard, 64);
+          const float4 seen = t > 0 ? lds4(max_s) : make_float4(-INFINITY, -INFINITY, -INFINITY, -INFINITY);
+          bool p_free = tg < kGroups || mbar_test_wait(bar_pv_done + 8 * g, (tg / kGroups - 1) & 1);
           tmem_wait_ld();
-        } else {
+          tc_fence_before();
+          mbar_arrive_warp(bar_s_empty + 8 * sb);          // the logits are in registers
+          float mx[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
 #pragma unroll
-          for (int q = 0; q < 32; ++q) v[q] = 0u;
-        }
-        tc_fence_before();
-        if (ns > 0) mbar_arrive_warp(bar_o_free);
-        AttnPart cut{};
-        if (SPLIT && it >= a.rounds) cut = part_of(it - a.rounds);
-        if (SPLIT && it >= a.rounds && cut.hi - cut.lo < a.units) {
-          store_part<D>(c, slot_of(blockIdx.x, cut.lo == 0), g, r, v, m_all, denom);
-        } else {
-          const AttnItem w = rows_of(item_at(it));
-          if (r < w.valid_rows)               // loads are warp-collective, only the stores are per row
-            write_row(a, static_cast<int64_t>(w.h) * a.out_head_stride + static_cast<int64_t>(w.q0 + r) * a.out_token_stride + g * 32, v, denom);
-        }
-      } else if (ns > 0) {
-        mbar_arrive_warp(bar_o_free);
-      }
-      if (ns > 0) ++n_done;
-      sub0 += ns;
-    }
-    const AttnPiece piece = SPLIT ? *piece_s : AttnPiece{};
-    if (SPLIT && (warp >> 2) < D / 32 && piece.n > 0) {
-      // The parts of cut items: the CTA that finds that the other parts of an item have come adds them up.  Asked at the end, so that no
-      // answer is waited for between two items; by one warp, because a fence by each of sixteen takes as long as ten tiles; for both cut
-      // items at once, by two lanes.  After a time-out the warps come here too, so that the counters go back to zero.
-      const int g = warp >> 2, r = (warp & 3) * 32 + lane;
-      auto cut_at = [&](int e) { return part_of(e == 0 ? 0 : piece.n - 1); };
-      auto parts_of = [&](int item, int& first) {
-        first = piece_at(a, item * a.units);
-        return piece_at(a, item * a.units + a.units - 1) - first + 1;
-      };
-      mbar_arrive_warp(bar_parts);
-      if (warp == 0) {
-        ok = mbar_wait_warp(bar_parts, 0, abort_flag, c.status) && ok;
-        const AttnPart cut = cut_at(lane & 1);
-        int last = 0, first;
-        if (lane < min(piece.n, 2) && cut.hi - cut.lo < a.units) {
-          last = atomic_add_acq_rel(c.part_count + cut.item, 1) == parts_of(cut.item, first) - 1 ? 1 : 0;
-          if (last) c.part_count[cut.item] = 0;
-        }
-        const uint32_t both = __ballot_sync(0xffffffffu, last);
-        if (lane == 0) *last_s = both;
-        mbar_arrive_warp(bar_last);
-      }
-      ok = mbar_wait_warp(bar_last, 0, abort_flag, c.status) && ok;
+          for (int k = 0; k < 8; ++k) {
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+              uint32_t* v = &x[q >> 1][4 * k + 2 * (q & 1)];
+              const float2 y = ffma2(make_float2(__uint_as_float(v[0]), __uint_as_float(v[1])), make_float2(scale, scale), bias[k]);
+              v[0] = __float_as_uint(y.x);
+              v[1] = __float_as_uint(y.y);
+              mx[q] = fmax3(mx[q], y.x, y.y);
+            }
+          }
+          // A logit makes this warp raise the maximum if it exceeds the last one by as much.  If none does, and nobody has raised it since
+          // this warp looked, the hand-over goes on at once: the maximum cannot change before this sub-tile is through, because whoever
+          // raises it waits for P V of all sub-tiles before.
+          // The first sub-tile's warp always goes the long way: it puts the maxima where the others read them, also those of a sub-tile
+          // without a live key (-inf; what lies there is an earlier item's).
+          bool may = t == 0;
+#pragma unroll
+          for (int q = 0; q < 4; ++q) may |= mx[q] > m[q] + kTop;
+          may = __any_sync(0xffffffffu, may);
+          if (!may && t + 1 < ns) named_barrier_arrive(told, 64);
+          const float cur[4] = {seen.x, seen.y, seen.z, seen.w};
+          bool change = t == 0;
+#pragma unroll
+          for (int q = 0; q < 4; ++q) change |= mx[q] > cur[q] + kTop || cur[q] != m[q];
+          if (__any_sync(0xffffffffu, change)) {
+            float alpha[4];
+            bool raised = t == 0;
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+              // the same for the four threads of a row
+              mx[q] = fmaxf(mx[q], __shfl_xor_sync(0xffffffffu, mx[q], 1));
+              mx[q] = fmaxf(mx[q], __shfl_xor_sync(0xffffffffu, mx[q], 2));
+              float top = cur[q];
+              alpha[q] = 1.f;
+              if (mx[q] > cur[q] + kTop) {
+                top = mx[q] + kHead;
+                alpha[q] = cur[q] == -INFINITY ? 0.f : fast_exp2(cur[q] - top);
+                raised = true;
+              }
+              // this thread's sum follows both the others' raises and its own
+              if (m[q] != top) {
+                const float f = m[q] == -INFINITY ? 0.f : fast_exp2(m[q] - top);
+                l[q].x *= f;
+                l[q].y *= f;
+              }
+              m[q] = top;
+            }
+            if (__any_sync(0xffffffffu, raised)) {
+              if (t > 0) {
+                // O is relative to the old maxima: P V of the sub-tile before must be in it, that of this one follows its P.
+                // (A parity tells only two phases apart, so the phase before has to be over: P V of sub-tile t - 4, which this group
+                // has to see done in any case, comes after that of t - 5.)
+                if (!__all_sync(0xffffffffu, p_free)) ok = ok && mbar_wait_warp(bar_pv_done + 8 * g, (tg / kGroups - 1) & 1, abort_flag, c.status);
+                p_free = true;
+                ok = ok && mbar_wait_warp(bar_pv_done + 8 * ((tg - 1) % kGroups), ((tg - 1) / kGroups) & 1, abort_flag, c.status);
+                tc_fence_after();
+                if (ok)
 #pragma unroll 1
-      for (int e = 0; e < 2; ++e)
-        if (ok && ((*last_s >> e) & 1)) {
-          uint32_t v[32];
-          int first;
-          const int item = cut_at(e).item, parts = parts_of(item, first);
-          const float sum = merge_parts<D>(c, first, parts, g, r, v);
-          const AttnItem w = rows_of(a.rounds * gridDim.x + item);
-          if (r < w.valid_rows)
-            write_row(a, static_cast<int64_t>(w.h) * a.out_head_stride + static_cast<int64_t>(w.q0 + r) * a.out_token_stride + g * 32, v, sum);
+                  for (int cc = 0; cc < 2 * (D / 32); ++cc) {
+                    const int hf = cc & 1;
+                    const uint32_t o_c = o_t + hf * kHalf + (cc >> 1) * 32;
+                    const float a0 = hf ? alpha[2] : alpha[0], a1 = hf ? alpha[3] : alpha[1];
+                    uint32_t v[16];
+                    tmem_ld_frag16(o_c, v);
+                    tmem_wait_ld();
+#pragma unroll
+                    for (int q = 0; q < 16; ++q) v[q] = __float_as_uint(__uint_as_float(v[q]) * ((q & 2) ? a1 : a0));
+                    tmem_st_frag16(o_c, v);
+                  }
+              }
+              if ((lane & 3) == 0)
+                asm volatile("st.shared.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(max_s), "f"(m[0]), "f"(m[1]), "f"(m[2]), "f"(m[3]) : "memory");
+              __syncwarp();
+            }
+          }
+          if (may && t + 1 < ns) named_barrier_arrive(told, 64);
+          // P is free once P V of the group's last sub-tile has read it
+          if (!__all_sync(0xffffffffu, p_free)) ok = ok && mbar_wait_warp(bar_pv_done + 8 * g, (tg / kGroups - 1) & 1, abort_flag, c.status);
+          tc_fence_after();
+          // exponentials -> bf16 P
+#pragma unroll
+          for (int hf = 0; hf < 2; ++hf) {
+            float2 neg[2];
+#pragma unroll
+            for (int e = 0; e < 2; ++e) neg[e].x = neg[e].y = m[2 * hf + e] == -INFINITY ? 0.f : -m[2 * hf + e];
+            uint32_t p[16];
+#pragma unroll
+            for (int k = 0; k < 8; ++k)
+#pragma unroll
+              for (int e = 0; e < 2; ++e) {
+                const uint32_t* v = &x[hf][4 * k + 2 * e];
+                const float2 u = fadd2(make_float2(__uint_as_float(v[0]), __uint_as_float(v[1])), neg[e]);
+                const float2 pr = make_float2(fast_exp2(u.x), fast_exp2(u.y));
+                const uint32_t b = pack_bf16x2(pr.x, pr.y);
+                p[2 * k + e] = b;
+                l[2 * hf + e] = fadd2(l[2 * hf + e], make_float2(__uint_as_float(b << 16), __uint_as_float(b & 0xFFFF0000u)));
+              }
+            tmem_st_half_frag(p_t + hf * kHalf, p);
+          }
+          const uint32_t jn = (tg + kGroups) / SUB;            // (asked here, needed later: a barrier answers slowly while MMAs run)
+          if (!SM::QT) s_ready = mbar_test_wait(bar_s_full + 8 * (jn % SM::NSB), (jn / SM::NSB) & 1);
+          tmem_wait_st();
+          tc_fence_before();
+          mbar_arrive_warp(bar_p_full + 8 * g);
+          if (!SM::QT) s_ready = __all_sync(0xffffffffu, s_ready);
         }
-    }
-    tc_fence_before();
-    mbar_arrive_warp(bar_done);
+        // ---- the groups meet: (m, l) of every row through shared memory ----
+        const uint32_t xchg = sbase + SM::xchg_off + (n_done & 1) * kGroups * 1024;
+        if (ns > 0) {
+          // the group of the last sub-tile waits for the last P V, the others for that group
+          const int last = sub0 + ns - 1;
+          if (g == last % kGroups) ok = ok && mbar_wait_warp(bar_pv_done + 8 * g, (last / kGroups) & 1, abort_flag, c.status);
+#pragma unroll
+          for (int q = 0; q < 4; ++q) {
+            float sum = l[q].x + l[q].y;
+            sum += __shfl_xor_sync(0xffffffffu, sum, 1);
+            sum += __shfl_xor_sync(0xffffffffu, sum, 2);
+            if ((lane & 3) == 0)
+              asm volatile("st.shared.v2.f32 [%0], {%1, %2};" ::"r"(xchg + (g * 128 + (warp & 3) * 32 + (lane >> 2) + 8 * q) * 8), "f"(m[q]), "f"(sum)
+                           : "memory");
+          }
+          mbar_arrive_warp(bar_xchg);
+          ok = mbar_wait_warp(bar_xchg, n_done & 1, abort_flag, c.status) && ok;
+          tc_fence_after();
+        }
+        const int r = (warp & 3) * 32 + lane;         // from here on a thread owns one row, 32 of its columns
+        if (ok && g < D / 32) {
+          // O is relative to the last maximum, which the group of the last sub-tile knows; the others may be some raises behind
+          uint32_t v[32];
+          float m_all = -INFINITY, denom = 0.f;
+          if (ns > 0) {
+            float2 part[kGroups];
+#pragma unroll
+            for (int q = 0; q < kGroups; ++q) {
+              part[q] = lds2(xchg + (q * 128 + r) * 8);
+              m_all = fmaxf(m_all, part[q].x);
+            }
+#pragma unroll
+            for (int q = 0; q < kGroups; ++q) denom += part[q].y * ((part[q].x == -INFINITY) ? 0.f : fast_exp2(part[q].x - m_all));
+            tmem_ld32(o_t + g * 32, v);
+            tmem_wait_ld();
+          } else {
+#pragma unroll
+            for (int q = 0; q < 32; ++q) v[q] = 0u;
+          }
+          tc_fence_before();
+          if (ns > 0) mbar_arrive_warp(bar_o_free);
+          AttnPart cut{};
+          if (SPLIT && it >= a.rounds) cut = part_of(it - a.rounds);
+          if (SPLIT && it >= a.rounds && cut.hi - cut.lo < a.units) {
+            store_part<D>(c, slot_of(blockIdx.x, cut.lo == 0), g, r, v, m_all, denom);
+          } else {
+            const AttnItem w = rows_of(item_at(it));
+            if (r < w.valid_rows)               // loads are warp-collective, only the stores are per row
+              write_row(a, static_cast<int64_t>(w.h) * a.out_head_stride + static_cast<int64_t>(w.q0 + r) * a.out_token_stride + g * 32, v, denom);
+          }
+        } else if (ns > 0) {
+          mbar_arrive_warp(bar_o_free);
+        }
+        if (ns > 0) ++n_done;
+        sub0 += ns;
+      }
+      const AttnPiece piece = SPLIT ? *piece_s : AttnPiece{};
+      if (SPLIT && (warp >> 2) < D / 32 && piece.n > 0) {
+        // The parts of cut items: the CTA that finds that the other parts of an item have come adds them up.  Asked at the end, so that no
+        // answer is waited for between two items; by one warp, because a fence by each of sixteen takes as long as ten tiles; for both cut
+        // items at once, by two lanes.  After a time-out the warps come here too, so that the counters go back to zero.
+        const int g = warp >> 2, r = (warp & 3) * 32 + lane;
+        auto cut_at = [&](int e) { return part_of(e == 0 ? 0 : piece.n - 1); };
+        auto parts_of = [&](int item, int& first) {
+          first = piece_at(a, item * a.units);
+          return piece_at(a, item * a.units + a.units - 1) - first + 1;
+        };
+        mbar_arrive_warp(bar_parts);
+        if (warp == 0) {
+          ok = mbar_wait_warp(bar_parts, 0, abort_flag, c.status) && ok;
+          const AttnPart cut = cut_at(lane & 1);
+          int last = 0, first;
+          if (lane < min(piece.n, 2) && cut.hi - cut.lo < a.units) {
+            last = atomic_add_acq_rel(c.part_count + cut.item, 1) == parts_of(cut.item, first) - 1 ? 1 : 0;
+            if (last) c.part_count[cut.item] = 0;
+          }
+          const uint32_t both = __ballot_sync(0xffffffffu, last);
+          if (lane == 0) *last_s = both;
+          mbar_arrive_warp(bar_last);
+        }
+        ok = mbar_wait_warp(bar_last, 0, abort_flag, c.status) && ok;
+#pragma unroll 1
+        for (int e = 0; e < 2; ++e)
+          if (ok && ((*last_s >> e) & 1)) {
+            uint32_t v[32];
+            int first;
+            const int item = cut_at(e).item, parts = parts_of(item, first);
+            const float sum = merge_parts<D>(c, first, parts, g, r, v);
+            const AttnItem w = rows_of(a.rounds * gridDim.x + item);
+            if (r < w.valid_rows)
+              write_row(a, static_cast<int64_t>(w.h) * a.out_head_stride + static_cast<int64_t>(w.q0 + r) * a.out_token_stride + g * 32, v, sum);
+          }
+      }
+      tc_fence_before();
+      mbar_arrive_warp(bar_done);
+    }  };
+  if constexpr (CUT) {
+    const int32_t* live = a.sel ? a.nsel : c.len;            // tiles, or keys
+    int longest = live[min(lane, c.H - 1)];
+#pragma unroll 1
+    for (int h = lane + 32; h < c.H; h += 32) longest = max(longest, live[h]);
+    longest = __reduce_max_sync(0xffffffffu, longest);
+    if ((a.sel ? longest : (longest + BKT - 1) / BKT) + (SEG ? a.seg_tiles : 0) >= a.whole_below) run(std::true_type{});
+    else run(std::false_type{});
+  } else {
+    run(std::false_type{});
   }
 }
 
-template <int D, int BKT, bool GATHER, bool SEG, bool SPLIT = false>
+template <int D, int BKT, bool GATHER, bool SEG, bool CUT = false>
 static int launch_attn_t(const CUtensorMap& tq, const CUtensorMap& tk, const CUtensorMap& tv, const CUtensorMap& tsk,
                          const CUtensorMap& tsv, const CacheView& c, const AttnArgs& a, int grid, cudaStream_t st) {
   using SM = AttnSmem<D, BKT>;
-  auto kern = attn_kernel<D, BKT, GATHER, SEG, SPLIT>;
+  auto kern = attn_kernel<D, BKT, GATHER, SEG, CUT>;
   const int cfg = ensure_dynamic_smem(reinterpret_cast<const void*>(kern), SM::total);
   if (cfg != FASTAR_OK) return cfg;
   launch_chained(kern, grid, kAttnThreads, SM::total, st, tq, tk, tv, tsk, tsv, c, a);
@@ -813,35 +835,38 @@ static int launch_attn(const CUtensorMap& tq, const CUtensorMap& tk, const CUten
   int dev = 0, sm_count = 148;
   if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sm_count, cudaDevAttrMultiProcessorCount, dev);
   if constexpr (!GATHER) {
-    // Items that do not fill the last round of the SMs are cut by key tiles where that pays, in tile times (about a microsecond): a part's
-    // way through memory takes kPartStore, adding one in the end kPartAdd, another stop of a CTA kPartStop.  Either every item is cut into
-    // k equal pieces, which leaves a CTA one stop, or all are dealt to all CTAs.  What is saved has to be kPartGain of the whole.
+    // Items that do not fill the last round of the SMs are cut by key tiles where that pays by CutCost: either every item into k equal
+    // pieces, which leaves a CTA one stop, or all are dealt to all CTAs.  What is decided here for the most tiles that an item can have, the
+    // kernel does if there is an item of so many (whole_below) that it pays: a cache that is a tenth full is attended as if it had no more room.
     // Kernel time without and with the cut: one item of 153 64-key tiles of 17 x 19 queries 44.0 -> 20.8 us (2 heads), 30 items of 25
     // tiles 28.2 -> 18.6, 44 of 24 30.4 -> 24.5, 182 of 530 902 -> 647, 156 of 16 42.3 -> 38.1; 8 x 4 096 queries on 16 384 keys (256 of
     // 128, dealt to all) 283 -> 265 a pass.  Where it would not pay: 108 items of 54 tiles dealt to all 63 -> 69, 18 of 6 13.6 -> 23.2, 256 of
     // 16 39.4 -> 45.0, 256 of 64 119 -> 122; and full rounds of 64-key tiles, whose loop is slower in this variant (936 of 245 951 -> 990).
+    // With room for more keys than there are: 4 x 1 024 queries on 512 keys in a cache of 32 768, 64-key tiles 10.9 us, cut by the room 21.9, now
+    // 11.6 (the look at the lengths is 0.4 of it); 8 x 1 560 on 2 048, 128-key tiles 21.9, 30.5, 21.8.
+    using Cost = CutCost<BKT>;
     const int grid = min(min(sm_count, kAttnMaxGrid), c.max_pieces), full = min(sm_count, kAttnMaxGrid), rounds = items / full, left = items % full;
     const int tiles = (a.sel ? a.keep : c.CAPB) + a.seg_tiles;           // at most
-    float best = tiles * (1.f - kPartGain * (rounds + 1));
-    int pieces = 0;
+    const float share = 1.f - Cost::gain * (rounds + 1);                 // of its tiles' time that a cut item may take
+    AttnArgs cut = a;
+    cut.rounds = rounds;
+    cut.last_items = left;
+    cut.units = tiles;
+    float best = tiles * share;
     for (int k = 2; left > 0 && k * left <= grid && k * kAttnMinPiece <= tiles; ++k) {
-      const float t = static_cast<float>(tiles) / k + kPartStore + kPartAdd * k;
-      if (t < best) { best = t; pieces = k * left; }
+      const float dealt = Cost::loop / k, cost = Cost::store + Cost::add * k, t = tiles * dealt + cost;
+      if (t < best) { best = t; cut.pieces = k * left; cut.whole_below = static_cast<int>(cost / (share - dealt)) + 1; }
     }
     if (left > 0 && grid > left) {
-      const float t = static_cast<float>(left) * tiles / grid + kPartStop + kPartStore + kPartAdd * (static_cast<float>(grid) / left + 1.f);
-      if (t < best && static_cast<int64_t>(left) * tiles >= static_cast<int64_t>(grid) * kAttnMinPiece) pieces = grid;
+      const float dealt = Cost::loop * left / grid, cost = Cost::stop + Cost::store + Cost::add * (static_cast<float>(grid) / left + 1.f);
+      if (tiles * dealt + cost < best && static_cast<int64_t>(left) * tiles >= static_cast<int64_t>(grid) * kAttnMinPiece) {
+        cut.pieces = grid;
+        cut.whole_below = static_cast<int>(cost / (share - dealt)) + 1;
+      }
     }
-    const int64_t largest = static_cast<int64_t>(tiles) * max(left * (pieces + 1), tiles);      // of the kernel's products
-    if (rounds > 0 && BKT == 64) pieces = 0;
-    if (pieces > 0 && !a.no_cut && largest < (1ll << 31)) {
-      AttnArgs cut = a;
-      cut.rounds = rounds;
-      cut.last_items = left;
-      cut.units = tiles;
-      cut.pieces = pieces;
-      return launch_attn_t<D, BKT, GATHER, SEG, true>(tq, tk, tv, tsk, tsv, c, cut, full, st);
-    }
+    const int64_t largest = static_cast<int64_t>(tiles) * max(left * (cut.pieces + 1), tiles);      // of the kernel's products
+    if (rounds > 0 && BKT == 64) cut.pieces = 0;
+    if (cut.pieces > 0 && !a.no_cut && largest < (1ll << 31)) return launch_attn_t<D, BKT, GATHER, SEG, true>(tq, tk, tv, tsk, tsv, c, cut, full, st);
   }
   return launch_attn_t<D, BKT, GATHER, SEG>(tq, tk, tv, tsk, tsv, c, a, GATHER ? items : min(items, sm_count), st);
 }

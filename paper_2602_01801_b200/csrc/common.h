@@ -195,7 +195,7 @@ struct AttnArgs {
   const int32_t* keep_frames;
   int keep_frames_stride;
   // paged mode, set by the launch where the items of the last round are cut (attn_kernels.cu)
-  int rounds, last_items, units, pieces;
+  int rounds, last_items, units, pieces, whole_below;
   int no_cut;              // paged mode: the parts' place is taken
 };
 constexpr int kAttnMaxGrid = 160;  // CTAs that may share the items of a last round

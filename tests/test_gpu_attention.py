@@ -249,3 +249,43 @@ def test_not_a_number_stays_in_its_rows(d, pt, whole_rounds):
                 assert np.array_equal(np.isnan(out[h, rows]), nan)
                 # rounding of the probabilities and of the output
                 assert np.abs(out[h, rows] - want)[~nan].max(initial=0) <= 2.0 ** -7 * np.abs(v[h]).max()
+
+
+@pytest.mark.parametrize("d,pt,H,nqb,tiles,lens,seg", [
+    (128, 128, 1, 3, 128, [512], 0),                               # room for 128 tiles, four are there
+    (128, 128, 1, 3, 128, [17 * 128], 0),                          # the most that is not cut, and the least that is
+    (128, 128, 1, 3, 128, [17 * 128 + 1], 0),
+    (64, 64, 6, 3, 160, [0, 1, 64 * 7, 64 * 19, 64 * 15 - 1, 64 * 4], 0),
+    (64, 64, 6, 3, 160, [0, 1, 64 * 7, 64 * 60, 64 * 15 - 1, 64 * 160], 0),        # cut, heads of nothing and of a few keys too
+    (128, 64, 6, 3, 100, [64 * 9, 0, 5, 64 * 7, 0, 64 * 3 + 3], 130),
+    (128, 64, 6, 3, 100, [64 * 9, 64 * 100, 5, 64 * 40, 0, 64 * 30 + 3], 130),
+    (128, 128, 8, 11, 80, [128 * 50, 128 * 5 - 1, 128 * 3, 100, 128 * 40, 0, 128 * 6, 128], 0),      # 88 items, cut if dealt to all CTAs
+    (128, 128, 8, 11, 80, [128 * 80, 128 * 56 - 1, 128 * 57, 100, 128 * 80, 0, 128 * 56, 128 * 70], 0),
+    (64, 64, 11, 9, 140, [64 * 140, 64, 64 * 127, 64 * 128, 64 * 100, 64 * 140, 64 * 3, 0, 64 * 140, 64 * 130, 64 * 135], 0),      # 99 items
+    (64, 128, 11, 17, 40, [128 * 9, 128 * 10, 128 * 2, 1, 0, 1, 128 * 3, 128 * 4, 128 * 8, 128 * 4, 128 * 3], 0),      # a full round and 39
+    (64, 128, 11, 17, 40, [128 * 40, 128 * 11, 128 * 12, 128 * 12 + 1, 0, 1, 128 * 30, 128 * 40, 128 * 8, 128 * 40, 128 * 13], 0),
+])
+def test_items_of_caches_that_are_not_full(d, pt, H, nqb, tiles, lens, seg):
+    """Whether items are cut is decided by the keys that are there, not by the room for them: on both sides of the decision, with heads of no,
+    few and many tiles in one call; the same by a second call."""
+    import torch
+    from paper_2602_01801_b200 import fastar
+    g = torch.Generator(device="cuda").manual_seed(d + H * tiles)
+    cap, nq = -(-tiles * pt // 128) * 128, nqb * 128 - 31
+    normal = lambda *shape: torch.randn(*shape, generator=g, device="cuda").bfloat16()
+    q, k, v, sk, sv = (normal(H, m, d) for m in (nq, cap, cap, max(seg, 1), max(seg, 1)))
+    cache = fastar.Cache(H, d, cap, pt, np.random.default_rng(1).standard_normal((32, d)).astype(np.float32), max_tokens=nq)
+    cache.import_state(fastar.bf16_bits(k.float().cpu().numpy()), fastar.bf16_bits(v.float().cpu().numpy()), np.array(lens))
+    call = (lambda: cache.annsa_segment(q, sk, sv, 128, cap // pt)["out"]) if seg else (lambda: cache.annsa(q, 128, cap // pt)["out"])
+    out, again = call(), call()
+    assert cache.status() == 0
+    assert torch.equal(out, again)
+    for h in range(H):
+        kk, vv = (torch.cat([x[h, : lens[h]], y[h, :seg]]).double() for x, y in ((k, sk), (v, sv)))
+        if len(kk) == 0:
+            assert (out[h] == 0).all()
+            continue
+        want = torch.softmax(q[h].double() @ kk.T / math.sqrt(d), -1) @ vv
+        # rounding of the probabilities and of the output
+        assert (out[h].double() - want).abs().max() <= 2.0 ** -7 * vv.abs().max()
+        assert (out[h].double() - want).norm() <= 1e-2 * want.norm()
