@@ -578,9 +578,11 @@ attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CU
         for (int t = (g - sub0) & (kGroups - 1); t < ns; t += kGroups) {
           const int tg = sub0 + t, jg = tg / SUB;
           const uint32_t sn = SM::QT ? tg : jg, sb = sn % SM::NSB;       // barrier of the logits
-          // QT: the group before has been told of its logits, so those of the three sub-tiles before are complete: a barrier's parity tells
-          // two phases apart, and the one before this sub-tile's is that of t - 3.  (At an item's first the groups have just met.)
-          if (SM::QT && t > 0) named_barrier_sync(heard, 64);
+          // QT: a barrier's parity tells two phases apart, and the one before this sub-tile's is that of t - 3, which has to be complete.  From
+          // the fourth on that is known from the group before, which has been told of its own logits; at an item's first three, whose t - 3 is
+          // of an item before, from the groups' meeting, and there the hand-over waits until the logits are under way (64 keys a tile, four tiles
+          // an item, 256 and 444 items 13.6 -> 13.1 and 18.8 -> 18.0 us, sixteen 33.1 -> 32.7; sixty-four 89.1 -> 90.0).
+          if (SM::QT && t > 2) named_barrier_sync(heard, 64);
           if (SM::QT || !s_ready) ok = ok && mbar_wait_warp(bar_s_full + 8 * sb, (sn / SM::NSB) & 1, abort_flag, c.status);
           tc_fence_after();
           // the logits of this warp's rows: x[hf][4 k + 2 e + c] is row 16 hf + 8 e + lane / 4, column 8 k + 2 (lane & 3) + c
@@ -592,7 +594,7 @@ attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CU
           float2 bias[8];
 #pragma unroll
           for (int k = 0; k < 8; ++k) bias[k] = lds2(bp + 32 * k);
-          if (!SM::QT && t > 0) named_barrier_sync(heard, 64);
+          if (t > 0 && (!SM::QT || t <= 2)) named_barrier_sync(heard, 64);
           const float4 seen = t > 0 ? lds4(max_s) : make_float4(-INFINITY, -INFINITY, -INFINITY, -INFINITY);
           bool p_free = tg < kGroups || mbar_test_wait(bar_pv_done + 8 * g, (tg / kGroups - 1) & 1);
           tmem_wait_ld();
