@@ -890,7 +890,8 @@ static int annca_impl(fastar_cache_t* c, const HeadRange& range, const void* q, 
     if (!c->rel_clear && cudaMemsetAsync(c->v.rel, 0, static_cast<size_t>(c->v.H) * v.max_frames * v.max_prompt * 4, st) != cudaSuccess)
       return FASTAR_ERR_CUDA;
     c->rel_clear = false;
-    const int ranked = rel_out ? 0 : keep;     // the maxima are wanted: they are ranked (and cleared) by a kernel behind their decoding
+    // Where the maxima are wanted they are ranked (and cleared) by a kernel behind their decoding.
+    const int ranked = !rel_out && c1_ranks(v, nq, F, np) ? keep : 0;
     float rel_scale = 1.0f / sqrtf(static_cast<float>(v.D));
     if (v.search_bits == 8 && !v.sign_codes) {
       // relevance on the 8-bit codes of the directions, scaled back by the norms (Section 5.1 quantised search)
@@ -907,10 +908,8 @@ static int annca_impl(fastar_cache_t* c, const HeadRange& range, const void* q, 
       if (r != FASTAR_OK) return r;
       ACCK(FASTAR_K_C1_RELEVANCE, launch_c1_relevance(v, tm_q, tm_kp, nq, np, frame_len, ranked, st));
     }
-    if (rel_out) {
-      ACC(launch_decode_rel(v, F, np, rel_scale, rel_out, st));
-      ACCK(FASTAR_K_TOPK_PROMPT, launch_topk_prompt(v, F, np, keep, st));
-    }
+    if (rel_out) ACC(launch_decode_rel(v, F, np, rel_scale, rel_out, st));
+    if (ranked == 0) ACCK(FASTAR_K_TOPK_PROMPT, launch_topk_prompt(v, F, np, keep, st));
     c->rel_clear = clear_after;
     a.sel = v.selp;
     a.sel_stride = v.max_prompt;

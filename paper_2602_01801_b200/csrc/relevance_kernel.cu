@@ -49,9 +49,7 @@ struct Cfg {
 };
 
 // NKC: 128-byte chunks of a row (bf16: d / 64, codes: 1)
-// NV > 0: the CTA that finishes a head ranks its frames' tokens too (topk_row with NV registers), which saves a launch: as long on
-// the device (2 x 600 queries 6.5 + 2.4 -> 9.5 us, 12 x 4680 18.5 + 6.0 -> 24.6, its codes 18.0 + 7.3 -> 23.5, 40 x 10800 75.5 + 8.9 -> 83.0), but
-// a small step is bound by what the host spends on its launches (75.4 -> 71.2 us a pass).
+// NV > 0: the CTA that finishes a head ranks its frames' tokens too (topk_row with NV registers), which saves a launch (see c1_ranks).
 template <int NKC, bool CODE8, int NV>
 __global__ void __launch_bounds__(kThreads, 1)
 relevance_kernel(const __grid_constant__ CUtensorMap tm_p, const __grid_constant__ CUtensorMap tm_q, const CacheView c, const RelArgs g) {
@@ -343,11 +341,19 @@ int launch_relevance(const CUtensorMap& tm_p, const CUtensorMap& tm_q, const Cac
   g.top = prompt_topk_args(c, (g.nq + g.frame_len - 1) / g.frame_len, g.np, keep);
   if (g.np <= 128) return launch_relevance_t<NKC, CODE8, 4>(tm_p, tm_q, c, g, st);
   if (g.np <= 256) return launch_relevance_t<NKC, CODE8, 8>(tm_p, tm_q, c, g, st);
-  if (g.np <= 512) return launch_relevance_t<NKC, CODE8, 16>(tm_p, tm_q, c, g, st);
-  return launch_relevance_t<NKC, CODE8, 36>(tm_p, tm_q, c, g, st);
+  return launch_relevance_t<NKC, CODE8, 16>(tm_p, tm_q, c, g, st);
 }
 
 }  // namespace
+
+// Whether a head's frames are ranked by the CTA that finishes it.  On the device that is no gain: one CTA ranks a head, sixteen rows at a time,
+// where the top-k has an SM for every two rows.  It pays where a call is short enough to be bound by its launches (one head, 640 queries, 512
+// prompt tokens 17.1 -> 14.6 us a call, 2 x 1200 17.1 -> 14.9, 12 x 1200 and 256 tokens 17.3 -> 17.4), and there only for few rows, short ones
+// (16 frames of 512 tokens 17.3 -> 18.6, 32 17.2 -> 18.7, one of 1 024 17.1 -> 19.2); 12 x 4680 queries 20.4 -> 23.2, 40 x 10800 and 1 024
+// tokens 158 -> 168.
+bool c1_ranks(const CacheView& c, int nq, int n_frames, int np) {
+  return n_frames <= 8 && np <= 512 && static_cast<int64_t>(c.H) * ((nq + 127) / 128) <= 148;
+}
 
 // c.rel (zero before the call where it is used) receives the maxima as ordered integers.
 int launch_c1_relevance(const CacheView& c, const CUtensorMap& tm_q, const CUtensorMap& tm_kp, int nq, int np, int frame_len,

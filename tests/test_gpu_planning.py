@@ -91,3 +91,35 @@ def test_block_scores_ranked_by_their_own_kernel_or_behind_it(nq, blocks, forced
                 rank[max(0, live - forced):] = np.where(rank[max(0, live - forced):] < 1e9, rank[max(0, live - forced):] + 1e9, rank[max(0, live - forced):])
             want = np.sort(np.lexsort((np.arange(live), -rank))[:kept])
             assert np.array_equal(sel[b, :kept], want)
+
+
+@pytest.mark.parametrize("H,nq,frame,n_prompt,keep", [(1, 1, 1, 1, 1), (4, 4736, 592, 512, 33), (4, 4737, 4737, 300, 20), (2, 80, 10, 128, 17), (2, 90, 10, 129, 40),
+                                                      (3, 700, 233, 257, 64), (3, 700, 234, 513, 24), (37, 512, 256, 256, 9), (1, 640, 10, 1024, 30)])
+def test_kept_prompt_tokens_are_those_of_the_largest_relevance(H, nq, frame, n_prompt, keep):
+    """On both sides of where the relevance kernel ranks (8 frames, 512 tokens, 148 tiles): attention over the tokens that the relevances in 64 bits
+    keep.  Frames whose last kept token is ahead by less than fp32 sums can tell are left out."""
+    import math
+
+    import torch
+    from paper_2602_01801_b200 import fastar
+    g = torch.Generator(device="cuda").manual_seed(nq + n_prompt)
+    d = 128
+    cache = fastar.Cache(H, d, 1024, 128, np.random.default_rng(1).standard_normal((32, d)).astype(np.float32), max_tokens=nq, max_prompt_tokens=n_prompt, max_frames=64)
+    q, k, v = (torch.randn(H, m, d, device="cuda", generator=g).bfloat16() for m in (nq, n_prompt, n_prompt))
+    out, again = (cache.annca(q, k, v, frame, keep)["out"] for _ in range(2))          # the maxima and the counters are back at zero
+    assert cache.status() == 0 and torch.equal(out, again)
+    compared = frames = 0
+    for f in range(-(-nq // frame)):
+        s = q[:, f * frame: f * frame + frame].double() @ k.double().transpose(1, 2) / math.sqrt(d)
+        rel, kept = torch.sort(s.amax(1), dim=1, descending=True)
+        for h in range(H):
+            frames += 1
+            if keep < n_prompt and rel[h, keep - 1] - rel[h, keep] < 1e-5:       # sums of 128 products of size 1: 128 * 2^-24
+                continue
+            compared += 1
+            at = kept[h, :keep]
+            want = torch.softmax(s[h][:, at], -1) @ v[h, at].double()
+            got = out[h, f * frame: f * frame + frame].double()
+            # rounding of the probabilities and of the output
+            assert (got - want).abs().max() <= 2.0 ** -7 * v[h].abs().max()
+    assert compared >= 0.9 * frames
