@@ -112,18 +112,23 @@ __device__ __forceinline__ uint4 pack_counts(const int (&v)[8]) {
 // 17 us at the measured bandwidth: 48 -> 39 us; 12 x 4680 9.9 -> 8.9).  Fragment layout (g = lane / 4, t = lane % 4):
 //   A: a0 = X[g][2t..], a1 = X[g+8][2t..], a2 = X[g][2t+8..], a3 = X[g+8][2t+8..]   (bf16 pairs)
 //   B: b0 = R[n = 8*nt + g][2t..], b1 = R[n][2t+8..];   C: c0,c1 = row g, cols 2t,2t+1;  c2,c3 = row g+8.
-// BLOCKS (the query side of S2 in the same launch: 12 x 4680 rows 9.2 + 2.7 -> 10.2 us, 2 x 600 4.1 + 2.3 -> 4.4): a CTA's warps take the
-// 16-row groups of one block of block_rows rows (64 or 128), and the CTA writes the block's bucket histogram.
+// ROWS > 0 (the query side of S2 in the same launch: 12 x 4680 rows 9.2 + 2.7 -> 10.2 us, 2 x 600 4.1 + 2.3 -> 4.4): blocks of 64 or 128 rows,
+// whose bucket histograms the CTA writes.  With four of eight warps idle for blocks of 64, 40 x 10800 rows took 45 us, with two blocks a pass 37
+// (d = 64 29 -> 22); with a launch of their own for the histograms 33 (26).  Blocks of 128: 34 (21) us, 31 (24) with that launch.
 struct BlockHist {
   __nv_bfloat16* hist;         // [H][max_qb][hist_cols]
-  int block_rows, max_qb, hist_cols;
+  int max_qb, hist_cols;
 };
-template <int D, bool BLOCKS>
+template <int D, int ROWS>
 __global__ void __launch_bounds__(256, 2) prep_kernel(const __nv_bfloat16* __restrict__ x, int H, int n, int64_t hs, int64_t ts,
                                                    const __nv_bfloat16* __restrict__ lsh, int T, int B,
                                                    uint32_t* __restrict__ code_out, float* __restrict__ rnorm_out,
                                                    int64_t out_stride, UpdateScratch clear, BlockHist bh) {
-  __shared__ __align__(16) int hist[BLOCKS ? 1024 : 4];
+  constexpr bool BLOCKS = ROWS > 0;
+  constexpr int per_block = BLOCKS ? ROWS / 16 : 1, blocks_a_pass = BLOCKS ? 8 / per_block : 1;
+  __shared__ __align__(16) int hist[BLOCKS ? 2 : 1][blocks_a_pass][BLOCKS ? 1024 : 4];      // [pass & 1][block of the pass]
+  if (BLOCKS)
+    for (int q = threadIdx.x; q < 2 * blocks_a_pass * 1024 / 4; q += 256) reinterpret_cast<int4*>(&hist[0][0][0])[q] = make_int4(0, 0, 0, 0);
   chain_wait();
   const int64_t thread = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x, threads = static_cast<int64_t>(gridDim.x) * blockDim.x;
   for (int64_t q = thread; q < clear.n_best; q += threads) clear.best[q] = 0ull;
@@ -155,14 +160,12 @@ __global__ void __launch_bounds__(256, 2) prep_kernel(const __nv_bfloat16* __res
       bf[ks][nt][0] = *reinterpret_cast<const uint32_t*>(rp);
       bf[ks][nt][1] = *reinterpret_cast<const uint32_t*>(rp + 2);
     }
-  // 16-row groups of all heads, dealt to the warps of a grid that fills the SMs once
-  // BLOCKS: groups are numbered through whole blocks, so that a CTA's eight warps have the groups of one block, or of two of 64 rows of
-  // which the second waits for the CTA's next pass
-  const int per_block = BLOCKS ? bh.block_rows / 16 : 1;
-  const int groups_per_head = BLOCKS ? (n + bh.block_rows - 1) / bh.block_rows * per_block : (n + 15) / 16;
+  // 16-row groups of all heads, dealt to the warps of a grid that fills the SMs once, eight to a CTA's pass
+  // BLOCKS: groups are numbered through whole blocks, so that a pass has one block of 128 rows or two of 64.  The histograms of two passes
+  // take turns: a thread that has written its columns of one clears them at once, and by the barrier of the next pass they are free.
+  const int groups_per_head = BLOCKS ? (n + ROWS - 1) / ROWS * per_block : (n + 15) / 16;
   const int total_groups = groups_per_head * H;
-  const int stride = BLOCKS ? static_cast<int>(gridDim.x) * per_block : static_cast<int>(gridDim.x) * 8;
-  const bool idle = BLOCKS && warp >= per_block;         // 64-row blocks: four warps have rows
+  const int stride = static_cast<int>(gridDim.x) * 8;
   uint4 va[KS / 2], vb[KS / 2];
   const __nv_bfloat16 *xa = x, *xb = x;                                // this lane's rows of the group that is fetched
   auto rows = [&](int grp) {
@@ -175,97 +178,95 @@ __global__ void __launch_bounds__(256, 2) prep_kernel(const __nv_bfloat16* __res
     va[kk] = *reinterpret_cast<const uint4*>(xa + 32 * kk);
     vb[kk] = *reinterpret_cast<const uint4*>(xb + 32 * kk);
   };
-  const int first = BLOCKS ? blockIdx.x * per_block + (idle ? 0 : warp) : blockIdx.x * 8 + warp;
-  if (first < total_groups && !idle) {
+  const int first = blockIdx.x * 8 + warp;
+  if (first < total_groups) {
     rows(first);
 #pragma unroll
     for (int kk = 0; kk < KS / 2; ++kk) fetch(kk);
   }
-  for (int grp = first; grp < total_groups; grp += stride) {
+  int buffer = 0;
+  for (int grp = first; BLOCKS ? grp - warp < total_groups : grp < total_groups; grp += stride) {
     const int h = grp / groups_per_head;
     const int r0 = (grp - h * groups_per_head) * 16;
-    const bool more = grp + stride < total_groups && !idle;
+    const bool more = grp + stride < total_groups;
     if (more) rows(grp + stride);
-    if (BLOCKS) {
-      reinterpret_cast<int4*>(hist)[threadIdx.x] = make_int4(0, 0, 0, 0);
-      __syncthreads();
-    }
-    if (!idle) {
-    float acc[4][4];
-#pragma unroll
-    for (int nt = 0; nt < 4; ++nt)
-#pragma unroll
-      for (int e = 0; e < 4; ++e) acc[nt][e] = 0.f;
-    float sqa = 0.f, sqb = 0.f;
-#pragma unroll
-    for (int ks = 0; ks < KS; ++ks) {
-      const uint4 pa = va[ks >> 1], pb = vb[ks >> 1];
-      const uint32_t a0 = (ks & 1) ? pa.z : pa.x, a2 = (ks & 1) ? pa.w : pa.y;
-      const uint32_t a1 = (ks & 1) ? pb.z : pb.x, a3 = (ks & 1) ? pb.w : pb.y;
-      {
-        const float2 f0 = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&a0));
-        const float2 f2 = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&a2));
-        const float2 f1 = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&a1));
-        const float2 f3 = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&a3));
-        sqa = fmaf(f0.x, f0.x, fmaf(f0.y, f0.y, fmaf(f2.x, f2.x, fmaf(f2.y, f2.y, sqa))));
-        sqb = fmaf(f1.x, f1.x, fmaf(f1.y, f1.y, fmaf(f3.x, f3.x, fmaf(f3.y, f3.y, sqb))));
-      }
+    if (!BLOCKS || grp < total_groups) {         // (the last pass may have a block less)
+      float acc[4][4];
 #pragma unroll
       for (int nt = 0; nt < 4; ++nt)
-        asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%0, %1, %2, %3};"
-                     : "+f"(acc[nt][0]), "+f"(acc[nt][1]), "+f"(acc[nt][2]), "+f"(acc[nt][3])
-                     : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(bf[ks][nt][0]), "r"(bf[ks][nt][1]));
-      if ((ks & 1) && more) fetch(ks >> 1);               // the registers are free: the next group's rows, in flight until its turn
-    }
-    // sign bits: this lane owns columns 8*nt + 2t, +1 of rows g and g+8; OR over the quad gives all 32 columns
-    uint32_t ma = 0, mb = 0;
 #pragma unroll
-    for (int nt = 0; nt < 4; ++nt) {
-      const int c0 = 8 * nt + 2 * t;
-      ma |= (acc[nt][0] > 0.f ? 1u : 0u) << c0;
-      ma |= (acc[nt][1] > 0.f ? 1u : 0u) << (c0 + 1);
-      mb |= (acc[nt][2] > 0.f ? 1u : 0u) << c0;
-      mb |= (acc[nt][3] > 0.f ? 1u : 0u) << (c0 + 1);
-    }
+        for (int e = 0; e < 4; ++e) acc[nt][e] = 0.f;
+      float sqa = 0.f, sqb = 0.f;
 #pragma unroll
-    for (int o = 1; o <= 2; o <<= 1) {
-      ma |= __shfl_xor_sync(0xffffffffu, ma, o);
-      mb |= __shfl_xor_sync(0xffffffffu, mb, o);
-      sqa += __shfl_xor_sync(0xffffffffu, sqa, o);
-      sqb += __shfl_xor_sync(0xffffffffu, sqb, o);
-    }
-    uint32_t ca = 0, cb = 0;
-    for (int tt = 0; tt < T; ++tt) {
-      ca |= ((ma >> (tt * B)) & ((1u << B) - 1u)) << (8 * tt);
-      cb |= ((mb >> (tt * B)) & ((1u << B) - 1u)) << (8 * tt);
-    }
-    if (BLOCKS)                              // table t of rows g and g + 8
-      if (t < T) {
-        if (r0 + g < n) atomicAdd(&hist[(t << B) + ((ca >> (8 * t)) & 0xFFu)], 1);
-        if (r0 + g + 8 < n) atomicAdd(&hist[(t << B) + ((cb >> (8 * t)) & 0xFFu)], 1);
+      for (int ks = 0; ks < KS; ++ks) {
+        const uint4 pa = va[ks >> 1], pb = vb[ks >> 1];
+        const uint32_t a0 = (ks & 1) ? pa.z : pa.x, a2 = (ks & 1) ? pa.w : pa.y;
+        const uint32_t a1 = (ks & 1) ? pb.z : pb.x, a3 = (ks & 1) ? pb.w : pb.y;
+        {
+          const float2 f0 = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&a0));
+          const float2 f2 = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&a2));
+          const float2 f1 = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&a1));
+          const float2 f3 = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&a3));
+          sqa = fmaf(f0.x, f0.x, fmaf(f0.y, f0.y, fmaf(f2.x, f2.x, fmaf(f2.y, f2.y, sqa))));
+          sqb = fmaf(f1.x, f1.x, fmaf(f1.y, f1.y, fmaf(f3.x, f3.x, fmaf(f3.y, f3.y, sqb))));
+        }
+#pragma unroll
+        for (int nt = 0; nt < 4; ++nt)
+          asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%0, %1, %2, %3};"
+                       : "+f"(acc[nt][0]), "+f"(acc[nt][1]), "+f"(acc[nt][2]), "+f"(acc[nt][3])
+                       : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(bf[ks][nt][0]), "r"(bf[ks][nt][1]));
+        if ((ks & 1) && more) fetch(ks >> 1);               // the registers are free: the next group's rows, in flight until its turn
       }
-    if (t == 0) {
-      if (r0 + g < n) {
-        code_out[h * out_stride + r0 + g] = ca;
-        if (rnorm_out) rnorm_out[h * out_stride + r0 + g] = sqa > 0.f ? 1.f / sqrtf(sqa) : 0.f;
+      // sign bits: this lane owns columns 8*nt + 2t, +1 of rows g and g+8; OR over the quad gives all 32 columns
+      uint32_t ma = 0, mb = 0;
+#pragma unroll
+      for (int nt = 0; nt < 4; ++nt) {
+        const int c0 = 8 * nt + 2 * t;
+        ma |= (acc[nt][0] > 0.f ? 1u : 0u) << c0;
+        ma |= (acc[nt][1] > 0.f ? 1u : 0u) << (c0 + 1);
+        mb |= (acc[nt][2] > 0.f ? 1u : 0u) << c0;
+        mb |= (acc[nt][3] > 0.f ? 1u : 0u) << (c0 + 1);
       }
-      if (r0 + g + 8 < n) {
-        code_out[h * out_stride + r0 + g + 8] = cb;
-        if (rnorm_out) rnorm_out[h * out_stride + r0 + g + 8] = sqb > 0.f ? 1.f / sqrtf(sqb) : 0.f;
+#pragma unroll
+      for (int o = 1; o <= 2; o <<= 1) {
+        ma |= __shfl_xor_sync(0xffffffffu, ma, o);
+        mb |= __shfl_xor_sync(0xffffffffu, mb, o);
+        sqa += __shfl_xor_sync(0xffffffffu, sqa, o);
+        sqb += __shfl_xor_sync(0xffffffffu, sqb, o);
       }
-    }
+      uint32_t ca = 0, cb = 0;
+      for (int tt = 0; tt < T; ++tt) {
+        ca |= ((ma >> (tt * B)) & ((1u << B) - 1u)) << (8 * tt);
+        cb |= ((mb >> (tt * B)) & ((1u << B) - 1u)) << (8 * tt);
+      }
+      if (BLOCKS && t < T) {                   // table t of rows g and g + 8
+        int* counts = hist[buffer][warp / per_block] + (t << B);
+        if (r0 + g < n) atomicAdd(counts + ((ca >> (8 * t)) & 0xFFu), 1);
+        if (r0 + g + 8 < n) atomicAdd(counts + ((cb >> (8 * t)) & 0xFFu), 1);
+      }
+      if (t == 0) {
+        if (r0 + g < n) {
+          code_out[h * out_stride + r0 + g] = ca;
+          if (rnorm_out) rnorm_out[h * out_stride + r0 + g] = sqa > 0.f ? 1.f / sqrtf(sqa) : 0.f;
+        }
+        if (r0 + g + 8 < n) {
+          code_out[h * out_stride + r0 + g + 8] = cb;
+          if (rnorm_out) rnorm_out[h * out_stride + r0 + g + 8] = sqb > 0.f ? 1.f / sqrtf(sqb) : 0.f;
+        }
+      }
     }
     if (BLOCKS) {
       __syncthreads();
-      const int blk = (grp - h * groups_per_head) / per_block;
-      uint4* dst = reinterpret_cast<uint4*>(bh.hist + (static_cast<int64_t>(h) * bh.max_qb + blk) * bh.hist_cols);
-      if (threadIdx.x < bh.hist_cols / 8) {
+      const int half = threadIdx.x >> 7, column = 8 * (threadIdx.x & 127), block = (grp - warp) / per_block + half;       // of all heads
+      if (half < blocks_a_pass && block * per_block < total_groups && column < bh.hist_cols) {
+        const int blocks = groups_per_head / per_block;
+        int* counts = &hist[buffer][half][column];
         int v[8];
 #pragma unroll
-        for (int e = 0; e < 8; ++e) v[e] = hist[8 * threadIdx.x + e];
-        dst[threadIdx.x] = pack_counts<-1>(v);
+        for (int e = 0; e < 8; ++e) { v[e] = counts[e]; counts[e] = 0; }
+        *reinterpret_cast<uint4*>(bh.hist + (static_cast<int64_t>(block / blocks) * bh.max_qb + block % blocks) * bh.hist_cols + column) = pack_counts<-1>(v);
       }
-      __syncthreads();
+      buffer ^= 1;
     }
   }
 }
@@ -278,18 +279,20 @@ static int launch_prep_generic(const CacheView& c, const __nv_bfloat16* x, int n
   // the rows only, 50 with these).
   const int64_t want = max(static_cast<int64_t>(groups + 7) / 8, (clear.n_best / 2 + clear.n_cnt16 + 2047) / 2048);
   const dim3 grid(static_cast<unsigned>(max(static_cast<int64_t>(1), min(want, static_cast<int64_t>(2 * 148)))));
-  if (c.D == 128) launch_chained(prep_kernel<128, false>, grid, 256, 0, st, x, c.H, n, hs, ts, c.lsh, c.T, c.B, code_out, rnorm_out, out_stride, clear, BlockHist{});
-  else launch_chained(prep_kernel<64, false>, grid, 256, 0, st, x, c.H, n, hs, ts, c.lsh, c.T, c.B, code_out, rnorm_out, out_stride, clear, BlockHist{});
+  if (c.D == 128) launch_chained(prep_kernel<128, 0>, grid, 256, 0, st, x, c.H, n, hs, ts, c.lsh, c.T, c.B, code_out, rnorm_out, out_stride, clear, BlockHist{});
+  else launch_chained(prep_kernel<64, 0>, grid, 256, 0, st, x, c.H, n, hs, ts, c.lsh, c.T, c.B, code_out, rnorm_out, out_stride, clear, BlockHist{});
   return cudaGetLastError() == cudaSuccess ? 1 : FASTAR_ERR_CUDA;
 }
 // Codes of the queries and the bucket histograms of their blocks of block_q rows.
 int launch_query_blocks(const CacheView& c, const __nv_bfloat16* q, int nq, int64_t hs, int64_t ts, int block_q, cudaStream_t st) {
   if (nq <= 0) return 0;
-  const int64_t blocks = static_cast<int64_t>((nq + block_q - 1) / block_q) * c.H;
-  const int grid = static_cast<int>(min(blocks, static_cast<int64_t>(2 * 148)));
-  const BlockHist bh{c.hq, block_q, c.max_qb, c.hist_cols};
-  if (c.D == 128) launch_chained(prep_kernel<128, true>, grid, 256, 0, st, q, c.H, nq, hs, ts, c.lsh, c.T, c.B, c.code_q_sa, nullptr, c.max_tokens, UpdateScratch{}, bh);
-  else launch_chained(prep_kernel<64, true>, grid, 256, 0, st, q, c.H, nq, hs, ts, c.lsh, c.T, c.B, c.code_q_sa, nullptr, c.max_tokens, UpdateScratch{}, bh);
+  const int64_t groups = static_cast<int64_t>((nq + block_q - 1) / block_q) * c.H * (block_q / 16);
+  const int grid = static_cast<int>(min((groups + 7) / 8, static_cast<int64_t>(2 * 148)));
+  auto launch = [&](auto kernel) {
+    launch_chained(kernel, grid, 256, 0, st, q, c.H, nq, hs, ts, c.lsh, c.T, c.B, c.code_q_sa, nullptr, c.max_tokens, UpdateScratch{}, BlockHist{c.hq, c.max_qb, c.hist_cols});
+  };
+  if (c.D == 128) block_q == 128 ? launch(prep_kernel<128, 128>) : launch(prep_kernel<128, 64>);
+  else block_q == 128 ? launch(prep_kernel<64, 128>) : launch(prep_kernel<64, 64>);
   return cudaGetLastError() == cudaSuccess ? 1 : FASTAR_ERR_CUDA;
 }
 bool plan_is_fused(const CacheView& c, int n);

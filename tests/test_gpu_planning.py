@@ -123,3 +123,31 @@ def test_kept_prompt_tokens_are_those_of_the_largest_relevance(H, nq, frame, n_p
             # rounding of the probabilities and of the output
             assert (got - want).abs().max() <= 2.0 ** -7 * v[h].abs().max()
     assert compared >= 0.9 * frames
+
+
+@pytest.mark.parametrize("H,nq,block_q,tables,bits", [(1, 1, 64, 4, 8), (3, 320, 64, 4, 8), (40, 1000, 64, 1, 3), (39, 1010, 64, 4, 8), (40, 1200, 128, 4, 8), (3, 129, 128, 2, 5)])
+def test_histograms_of_query_blocks(H, nq, block_q, tables, bits):
+    """One block, an odd number of them (a pass of two has one), more than a CTA has in one pass; the scores are the products of the blocks'
+    histograms by the codes of queries and keys."""
+    import torch
+    from paper_2602_01801_b200 import fastar
+    g = torch.Generator(device="cuda").manual_seed(nq)
+    d, cap = 64, 256
+    cache = fastar.Cache(H, d, cap, 64, np.random.default_rng(1).standard_normal((tables * bits, d)).astype(np.float32), tables, bits, max_tokens=max(nq, cap))
+    k, q = (torch.randn(H, m, d, device="cuda", generator=g).bfloat16() for m in (cap, nq))
+    cache.update(k, k, cap, 2.0)
+    for _ in range(2):
+        r = cache.annsa(q, block_q, 2, debug=True)
+        keys = torch.from_numpy(cache.export_state(kv=False)["code"].astype(np.int64)).cuda()
+
+        def histogram(codes, rows):
+            n = -(-codes.shape[1] // rows)
+            h = torch.zeros(H, n, tables << bits, device="cuda", dtype=torch.float64)
+            for t in range(tables):
+                at = (torch.arange(codes.shape[1], device="cuda") // rows * (tables << bits) + (t << bits))[None] + ((codes >> 8 * t) & 255)
+                h.view(H, -1).scatter_add_(1, at, torch.ones_like(at, dtype=torch.float64))
+            return h
+
+        want = histogram(r["qcode"].long() & 0xFFFFFFFF, block_q) @ histogram(keys, 64).transpose(1, 2)
+        assert torch.equal(r["scores"].double(), want)
+    assert cache.status() == 0
