@@ -79,7 +79,7 @@ constexpr float kHead = 16.f, kTop = 8.f;
 // of a CTA; a tile in the variant with the cut; and the share of the whole that has to be saved (see launch_attn).
 template <int BKT>
 struct CutCost {
-  static constexpr float store = BKT == 64 ? 6.f : 3.f, add = BKT == 64 ? 1.5f : 1.2f, stop = BKT == 64 ? 20.f : 14.f;
+  static constexpr float store = BKT == 64 ? 6.f : 3.2f, add = BKT == 64 ? 1.7f : 0.95f, stop = BKT == 64 ? 20.f : 14.f;
   static constexpr float loop = BKT == 64 ? 1.2f : 1.f, gain = 0.05f;
 };
 
@@ -844,8 +844,10 @@ static int launch_attn(const CUtensorMap& tq, const CUtensorMap& tk, const CUten
     // tiles 28.2 -> 18.6, 44 of 24 30.4 -> 24.5, 182 of 530 902 -> 647, 156 of 16 42.3 -> 38.1; 8 x 4 096 queries on 16 384 keys (256 of
     // 128, dealt to all) 283 -> 265 a pass.  Where it would not pay: 108 items of 54 tiles dealt to all 63 -> 69, 18 of 6 13.6 -> 23.2, 256 of
     // 16 39.4 -> 45.0, 256 of 64 119 -> 122; and full rounds of 64-key tiles, whose loop is slower in this variant (936 of 245 951 -> 990).
-    // With room for more keys than there are: 4 x 1 024 queries on 512 keys in a cache of 32 768, 64-key tiles 10.9 us, cut by the room 21.9, now
-    // 11.6 (the look at the lengths is 0.4 of it); 8 x 1 560 on 2 048, 128-key tiles 21.9, 30.5, 21.8.
+    // With room for more keys than there are: 4 x 1 024 queries on 512 keys in a cache of 32 768, 64-key tiles 10.8 us, cut by the room 21.6, now
+    // 11.3 (the look at the lengths is 0.4 of it); 8 x 1 560 on 2 048, 128-key tiles 21.9, 30.5, 21.8.  One head, 1 560 queries on 8 to 48 tiles of 128
+    // with room for 64, what the cut gives: decided by the room -3.5 to +22.0 us, now -0.5 to +22.7; d = 64 and 64-key tiles -3.1 to +8.8, now +0.1
+    // to +9.7.
     using Cost = CutCost<BKT>;
     const int grid = min(min(sm_count, kAttnMaxGrid), c.max_pieces), full = min(sm_count, kAttnMaxGrid), rounds = items / full, left = items % full;
     const int tiles = (a.sel ? a.keep : c.CAPB) + a.seg_tiles;           // at most

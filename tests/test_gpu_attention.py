@@ -253,8 +253,8 @@ def test_not_a_number_stays_in_its_rows(d, pt, whole_rounds):
 
 @pytest.mark.parametrize("d,pt,H,nqb,tiles,lens,seg", [
     (128, 128, 1, 3, 128, [512], 0),                               # room for 128 tiles, four are there
-    (128, 128, 1, 3, 128, [17 * 128], 0),                          # the most that is not cut, and the least that is
-    (128, 128, 1, 3, 128, [17 * 128 + 1], 0),
+    (128, 128, 1, 3, 128, [15 * 128], 0),                          # the most that is not cut, and the least that is
+    (128, 128, 1, 3, 128, [15 * 128 + 1], 0),
     (64, 64, 6, 3, 160, [0, 1, 64 * 7, 64 * 19, 64 * 15 - 1, 64 * 4], 0),
     (64, 64, 6, 3, 160, [0, 1, 64 * 7, 64 * 60, 64 * 15 - 1, 64 * 160], 0),        # cut, heads of nothing and of a few keys too
     (128, 64, 6, 3, 100, [64 * 9, 0, 5, 64 * 7, 0, 64 * 3 + 3], 130),
