@@ -306,7 +306,9 @@ int fastar_annca_attention_lsh(fastar_cache_t* cache, const void* q, const void*
  * slices of heads where the tensors are large, on streams owned by the cache object beside `stream`: the
  * prompt, the keys, the queries and the values are uploaded in that order (the queries first where they are
  * the probe), and each part starts when what it reads is there.  Those streams start after the work already
- * queued on `stream` and are idle again when the call returns.  Arguments that one of the calls would refuse
+ * queued on `stream` and are idle again when the call returns.  The cache ends up as by the calls on the device,
+ * bit for bit; the outputs may differ from theirs by rounding, because the order in which AnnSA adds up a row depends
+ * on which other rows are in the launch.  Arguments that one of the calls would refuse
  * are refused before anything is queued.
  * flags: 0, or FASTAR_STEP_QUERY_PROBE to run the update as
  * fastar_tempcache_update_probe with q as the probe. */

@@ -121,7 +121,7 @@ inline __host__ __device__ int64_t slot_row_offset(const CacheView& c, const int
 
 // Launches a kernel that may start its prologue while the grid in front of it on the stream drains (programmatic stream
 // serialization).  The kernel has to call chain_wait() (ptx.cuh) before it touches global memory; behind a copy, a memset or
-// an event wait the launch is an ordinary one.  A step is 15 to 18 launches, and a gap between two ordinary ones is 2 us.
+// an event wait the launch is an ordinary one.  A step is 10 to 14 launches, and a gap between two ordinary ones is 2 us.
 template <class... P, class... A>
 inline cudaError_t launch_chained(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A&&... args) {
   cudaLaunchAttribute at{};

@@ -1025,8 +1025,9 @@ int fastar_attention_step_host(fastar_cache_t* c, const void* k_new_host, const 
   //   side    : (queries up) their hash for AnnSA's selector, AnnCA
   //   attend  : (planned, values up) commit, (hashed) AnnSA
   //   down    : AnnCA's outputs, AnnSA's outputs
-  // 12 heads x 4680 tokens against 28 080 keys, bf16: 1 366 -> 1 190 us with four slices (46.3 MB up and 28.8 down take 952 at once), 1 277
-  // with two, 1 274 with six; 1 225 with the queries before the keys, 1 277 with AnnCA's output in one copy, 1 345 with the queries in one.
+  // 12 heads x 4680 tokens against 28 080 keys, bf16: 1 368 -> 1 223 us with four slices (46.3 MB up and 28.8 down take 952 at once).  Against
+  // 1 190 on another box: 1 277 with two, 1 274 with six; 1 225 with the queries before the keys, 1 277 with AnnCA's output in one copy, 1 345
+  // with the queries in one.  With 4 of 147 blocks kept against 9 360 keys it is 1 225 -> 1 266: little computing to hide.
   // A slice below 3 MB a tensor is not worth its launches (11 heads x 1 120, fp32, 6 MB: 660 -> 636 with two slices, 713 with three).  The
   // owned streams start behind what the caller's stream holds and are joined before the call returns.
   const size_t token_bytes = static_cast<size_t>(n) * v.D * esz, prompt_bytes = static_cast<size_t>(np) * v.D * esz, all_bytes = token_bytes * v.H;

@@ -7,14 +7,15 @@
 namespace fastar {
 
 // S4 / C2: per row keep the k largest entries (ties -> lower index), listed ascending.
-// One warp per row, the row in registers (entry 32 i + lane).  The k-th largest key is found bit by bit, from the highest bit in
-// which the row's keys differ: one count over the row per bit, a dozen instructions per 32 entries, no barrier; the entries above it
-// and the first of those equal to it are then listed in index order by ballots.  Latency-bound (a few thousand dependent
-// instructions), and the time follows the registers a lane holds, whatever part of them the row fills: 2.5 us with 4, 3.9 with 16, 6.1
-// with 36, 8.9 with 64 (8 heads x 32 rows of block scores; 1 024 prompt tokens 8.8 with 36, 19.8 with 64).  Hence steps: 4, 16 and 64 are a
-// factor of four apart, 8 halves the second (220 blocks of 12 heads 5.6 -> 4.5 us, 128 of 8 4.4 -> 3.5), and 36 divides the widest of them so that 131 072 keys in 128-slot blocks, or 1 024 prompt tokens, with an eighth
-// to spare, are on the cheap side.  Measured against a 256-thread bitonic sort of (key, index): 256 rows of 1056 32.0 -> 7.2 us, 3400
-// rows of 512 78 -> 9.2 us, 444 rows of 256 7.6 -> 4.4 us, 36 rows of 512 prompt tokens 8.4 -> 6.5 us.
+// One warp per row, the row in registers (entry 32 i + lane).  The k-th largest key is found bit by bit, from the highest bit in which the
+// row's keys differ: one count over the row per bit, a dozen instructions per 32 entries, no barrier; the entries above it and the first of
+// those equal to it are then listed in index order by ballots.  Latency-bound (a few thousand dependent instructions), and the time
+// follows the registers a lane holds, whatever part of them the row fills: 2.5 us with 4, 3.9 with 16, 6.1 with 36, 8.9 with 64 (8 heads x
+// 32 rows of block scores; 1 024 prompt tokens 8.8 with 36, 19.8 with 64).  Hence steps: 4, 16 and 64 are a factor of four apart, 8 halves
+// the second (220 blocks of 12 heads 5.6 -> 4.5 us, 128 of 8 4.4 -> 3.5), and 36 divides the widest of them so that 131 072 keys in 128-slot
+// blocks, or 1 024 prompt tokens, with an eighth to spare, are on the cheap side.  Measured against a 256-thread bitonic sort of (key,
+// index): 256 rows of 1056 32.0 -> 7.2 us, 3400 rows of 512 78 -> 9.2 us, 444 rows of 256 7.6 -> 4.4 us, 36 rows of 512 prompt tokens 8.4 ->
+// 6.5 us.
 struct TopkArgs {
   void* src;                       // PROMPT: ordered-uint relevance (zeros are put back); else block scores as floats
   const float* src_hi;             // high digits of weighted scores, or nullptr

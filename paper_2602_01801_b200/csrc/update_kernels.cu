@@ -322,7 +322,8 @@ int launch_prep_codes_strided(const CacheView& c, const __nv_bfloat16* x, int n,
 }
 
 // ---------------------------------------------------------------------------------------------
-// T2-T4 planning in three small kernels (all work O(n + L), no sort):
+// T2-T4 planning: one kernel where its counters fit a CTA's shared memory (plan_fused_kernel, plan_is_fused), else three; all work
+// O(n + L), no sort:
 //   match_count : decode the packed arg-max, threshold (T2), count the tokens matched to each slot
 //   plan        : one CTA per head: scan the slot counts -> groups (touched slots) and their member
 //                 ranges; scan the tokens -> unmatched tokens in token order; place them (append, then
@@ -872,7 +873,7 @@ int plan_fused_smem(const CacheView& c, int n) {
 int launch_plan(const CacheView& c, int n, float tau, const UpdateOut& out, cudaStream_t st) {
   if (plan_is_fused(c, n)) {
     const int smem = plan_fused_smem(c, n);
-    switch ((n + 1023) / 1024) {             // every pass over the tokens counts (12 x 4680 with 8 for 5: 14.8 us, with 5 12.0)
+    switch ((n + 1023) / 1024) {             // every pass over the tokens counts (12 x 4680 with 8 for 5: 14.8 us, with 5 12.0; seven run as eight)
       case 1: return launch_plan_fused<1>(c, n, tau, out, smem, st);
       case 2: return launch_plan_fused<2>(c, n, tau, out, smem, st);
       case 3: return launch_plan_fused<3>(c, n, tau, out, smem, st);
