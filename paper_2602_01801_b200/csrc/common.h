@@ -164,7 +164,7 @@ int launch_quantize_rows(const CacheView& c, const __nv_bfloat16* x, int n, int6
                          int64_t out_rows_per_head, float* norm_out, int64_t norm_stride, cudaStream_t st);
 
 // relevance_kernel.cu: C1 on the bf16 rows and on the 8-bit codes; with the ranking if keep > 0, where c1_ranks says that it pays
-bool c1_ranks(const CacheView& c, int nq, int n_frames, int np);
+bool c1_ranks(const CacheView& c, int nq, int n_frames, int np, bool beside);
 int launch_c1_relevance(const CacheView& c, const CUtensorMap& tm_q, const CUtensorMap& tm_kp, int nq, int np, int frame_len,
                         int keep, cudaStream_t st);
 int launch_c1_relevance_fp8(const CacheView& c, const CUtensorMap& tm_q8, const CUtensorMap& tm_kp8, const float* qn,

@@ -839,7 +839,8 @@ int fastar_annsa_attention_segment(fastar_cache_t* c, const void* q, const void*
                     block_q, keep_blocks, nullptr, nullptr, nullptr, nullptr, sel_in, nsel_in, stream);
 }
 
-static int annca_impl(fastar_cache_t* c, const HeadRange& range, const void* q, const void* k_prompt, const void* v_prompt, void* out, int32_t nq,
+// beside: the call runs beside kernels that fill the SMs (c1_ranks).
+static int annca_impl(fastar_cache_t* c, const HeadRange& range, bool beside, const void* q, const void* k_prompt, const void* v_prompt, void* out, int32_t nq,
                            int32_t frame_len, int32_t np, int32_t keep_tokens, int64_t head_stride, int64_t token_stride,
                            int64_t prompt_head_stride, int64_t prompt_token_stride, int32_t* sel_out, float* rel_out,
                            const int32_t* sel_in, void* stream) {
@@ -891,7 +892,7 @@ static int annca_impl(fastar_cache_t* c, const HeadRange& range, const void* q, 
       return FASTAR_ERR_CUDA;
     c->rel_clear = false;
     // Where the maxima are wanted they are ranked (and cleared) by a kernel behind their decoding.
-    const int ranked = !rel_out && c1_ranks(v, nq, F, np) ? keep : 0;
+    const int ranked = !rel_out && c1_ranks(v, nq, F, np, beside) ? keep : 0;
     float rel_scale = 1.0f / sqrtf(static_cast<float>(v.D));
     if (v.search_bits == 8 && !v.sign_codes) {
       // relevance on the 8-bit codes of the directions, scaled back by the norms (Section 5.1 quantised search)
@@ -929,7 +930,7 @@ int fastar_annca_attention(fastar_cache_t* c, const void* q, const void* k_promp
                            int64_t prompt_head_stride, int64_t prompt_token_stride, int32_t* sel_out, float* rel_out,
                            const int32_t* sel_in, void* stream) {
   if (!c) return FASTAR_ERR_INVALID_ARG;
-  return annca_impl(c, c->all, q, k_prompt, v_prompt, out, nq, frame_len, np, keep_tokens, head_stride, token_stride, prompt_head_stride,
+  return annca_impl(c, c->all, false, q, k_prompt, v_prompt, out, nq, frame_len, np, keep_tokens, head_stride, token_stride, prompt_head_stride,
                     prompt_token_stride, sel_out, rel_out, sel_in, stream);
 }
 
@@ -1080,7 +1081,7 @@ int fastar_attention_step_host(fastar_cache_t* c, const void* k_new_host, const 
     if (r == FASTAR_OK && sparse) r = prepare_impl(c, ranges[i], q, n, hs, ts, block_q, side);
     try_cuda(cudaEventRecord(ev[c->kHashed], side));
     if (r == FASTAR_OK)
-      r = annca_impl(c, ranges[i], q, at(dsrc[3], first[i], prompt_bytes), at(dsrc[4], first[i], prompt_bytes), at(v.stage_out[1], first[i], token_bytes), n,
+      r = annca_impl(c, ranges[i], true, q, at(dsrc[3], first[i], prompt_bytes), at(dsrc[4], first[i], prompt_bytes), at(v.stage_out[1], first[i], token_bytes), n,
                      frame_len, np, keep_tokens, hs, ts, phs, ts, nullptr, nullptr, nullptr, side);
     try_cuda(cudaEventRecord(ev[c->kCrossDone], side));
   };

@@ -350,9 +350,11 @@ int launch_relevance(const CUtensorMap& tm_p, const CUtensorMap& tm_q, const Cac
 // where the top-k has an SM for every two rows.  It pays where a call is short enough to be bound by its launches (one head, 640 queries, 512
 // prompt tokens 17.1 -> 14.6 us a call, 2 x 1200 17.1 -> 14.9, 12 x 1200 and 256 tokens 17.3 -> 17.4), and there only for few rows, short ones
 // (16 frames of 512 tokens 17.3 -> 18.6, 32 17.2 -> 18.7, one of 1 024 17.1 -> 19.2); 12 x 4680 queries 20.4 -> 23.2, 40 x 10800 and 1 024
-// tokens 158 -> 168.
-bool c1_ranks(const CacheView& c, int nq, int n_frames, int np) {
-  return n_frames <= 8 && np <= 512 && static_cast<int64_t>(c.H) * ((nq + 127) / 128) <= 148;
+// tokens 158 -> 168.  Beside kernels that fill the SMs (the host-tensor step) the size does not matter: between the two kernels the next one
+// of the others takes the SMs, and with the top-k there are two such places (25 heads x 9 222 tokens, a host call 4 320 us, with the top-k
+// 4 398).
+bool c1_ranks(const CacheView& c, int nq, int n_frames, int np, bool beside) {
+  return n_frames <= 8 && np <= 512 && (beside || static_cast<int64_t>(c.H) * ((nq + 127) / 128) <= 148);
 }
 
 // c.rel (zero before the call where it is used) receives the maxima as ordered integers.
