@@ -260,7 +260,7 @@ def run_ours(args, cfg):
         cache.workspace.copy_(snap)
         step()
     barrier()
-    # The step is a fixed sequence of 11 to 15 short launches: replay it as one CUDA graph (tensor maps and
+    # The step is a fixed sequence of 12 to 15 short launches: replay it as one CUDA graph (tensor maps and
     # arguments are baked in at capture; the cache state they act on is restored before every replay).
     graph = None
     if not args.no_graph:
