@@ -34,6 +34,8 @@
 //   - items that do not fill the last round of the SMs are cut by key tiles (see launch_attn), and the soft-max loop is as large as
 //     an SM's instruction caches bear (stalls for instructions: a twentieth of a warp's time, and a sixth with a little more code in the
 //     kernel), so the cut is a variant of its own;
+//   - items whose logits a bound keeps near the first sub-tile's need no maximum at all (see kFlatMin): the loop for them is what the
+//     arithmetic needs, 245 instructions, and the exponentials and the tensor core bound it (0.74 and 0.73 of the time at d = 128);
 //   - the CTA stays for its items, and the copies and Q K^T run ahead into the next one, whose first logits are there when the
 //     output of the last has left.
 // TMEM columns: S 4 x 64, P 4 x 32, O D; with key tiles of 64: S 3 x 64, P, O and Q D / 2 (AttnSmem::QT).  K and V tiles have a TMA ring
@@ -41,9 +43,11 @@
 // Measured (B200, kernel time; two groups with whole tiles, a CTA per item, a limit of 8 -> this): 12 heads, d = 128, 4 680 queries on
 // 32 of 224 blocks 120.5 -> 105.4 us (0.68 of the measured bf16 peak); the same with the chunk's 4 680 keys beside 241 -> 218 us; 8
 // heads, 4 096 queries on all 16 384 keys 275 -> 246 us (108 of 148 CTAs have two items); d = 64, 64 of 1 024 blocks 142 -> 125 us,
-// 16 of 160 blocks 49 -> 39.5 us.  Row sums by a warp-level product with ones instead of adds: 311 us for 242 (it takes the tensor
+// 16 of 160 blocks 49 -> 39.5 us.  With flat items: the first three 99 -> 88, 194 -> 166 and 226 -> 192 us, the last two 118 -> 91 and
+// 37.8 -> 31.2.  Row sums by a warp-level product with ones instead of adds: 311 us for 242 (it takes the tensor
 // core); sums of the unrounded probabilities: 4 % faster, not as exact.
 // Warp roles: warps 0-15 soft-max groups 0-3, 16 copies Q and K (TMA or gather), 17 Q K^T, 18 P V, 19 copies V.
+#include "bound.cuh"
 #include "common.h"
 #include "ptx.cuh"
 
@@ -83,6 +87,45 @@ struct CutCost {
   static constexpr float loop = BKT == 64 ? 1.2f : 1.f, gain = 0.05f;
 };
 
+__device__ __forceinline__ float lds1(uint32_t addr) {
+  float v;
+  asm volatile("ld.shared.f32 %0, [%1];" : "=f"(v) : "r"(addr));
+  return v;
+}
+// 2^u of two logits on the FMA units, u < 2^22; 0 from -127 down, as the special-function units give it for a logit of -inf.  2^f on
+// [-1/2, 1/2] by a polynomial of degree 5, fitted to the least relative error (9.2e-8; that of ex2.approx is 1.2e-7) with 2^0 = 1.
+__device__ __forceinline__ float2 poly_exp2(float2 u) {
+  auto both = [](float v) { return make_float2(v, v); };
+  constexpr float kRound = 12582912.f;                     // 1.5 x 2^23: the sum's last bits are the nearest integer
+  u.x = fmaxf(u.x, -127.f);
+  u.y = fmaxf(u.y, -127.f);
+  const float2 r = fadd2(u, both(kRound)), f = ffma2(fadd2(r, both(-kRound)), both(-1.f), u);
+  float2 y = both(0x1.5bba14p-10f);
+  y = ffma2(y, f, both(0x1.3cea88p-7f));
+  y = ffma2(y, f, both(0x1.c6b752p-5f));
+  y = ffma2(y, f, both(0x1.ebf9bcp-3f));
+  y = ffma2(y, f, both(0x1.62e42ap-1f));
+  y = ffma2(y, f, both(1.f));
+  return make_float2(__uint_as_float(__float_as_uint(y.x) + (__float_as_uint(r.x) << 23)), __uint_as_float(__float_as_uint(y.y) + (__float_as_uint(r.y) << 23)));
+}
+// Both halves of a bf16 pair to a sum each, as they are.
+__device__ __forceinline__ void add_bf16x2(float2& s, uint32_t b) {
+  asm("{.reg .b16 l, h; mov.b32 {l, h}, %2; add.f32.bf16 %0, l, %0; add.f32.bf16 %1, h, %1;}" : "+f"(s.x), "+f"(s.y) : "r"(b));
+}
+// Flat items.  A logit is at most |q| max |k| / sqrt(d) + log2 max m; the cache keeps the largest of each head (HeadBound), a segment's come
+// with the call, and |q| is worked out here.  If that, for the rows of a warp, is not more than T above the reference that an item's first
+// sub-tile gives, nothing after it can ask for another reference: the sub-tiles that follow need no maximum, no look at the others' and no
+// hand-over, which are 160 of the loop's 440 instructions; and one reference for the four rows of a thread (the lowest of theirs, so that
+// a row's largest probability is 2^-kHead at least, as ever) goes into the biases.  T is as large as the sums of P V allow: keys x 2^T x
+// max |v| is below 2^118, or T is kTop, as where the maximum is looked for.  Items of fewer sub-tiles than kFlatMin don't ask.
+constexpr int kFlatMin = 8;
+constexpr float kFlatTop = 96.f, kFlatSum = 118.f;
+// Pairs of every sixteen whose exponentials the FMA units work out: the special-function units take 512 cycles for a sub-tile's, the tensor
+// core 270 at d = 64 and 540 at 128.  Kernel time with 0 / 2 / 4 of sixteen: d = 64, 256 items of 128 sub-tiles 96.0 / 91.2 / 90.0 us; d = 128, 256 of
+// 256 194 / 192 / 196, 444 of 138 170 / 170 / 174.
+template <int D>
+constexpr int kPolyPairs = D == 64 ? 4 : 2;
+
 template <int D, int BKT>
 struct AttnSmem {
   static constexpr int q_bytes = (D / 64) * kQChunk;
@@ -107,7 +150,8 @@ struct AttnSmem {
   static constexpr int bias_off = ring_off + RS * kv_bytes;
   static constexpr int xchg_off = bias_off + NB * BKT * 4;       // [2][kGroups][128] (maximum, sum) of the groups' rows, by item
   static constexpr int max_off = xchg_off + 2 * kGroups * 1024;  // [4][8][4] running maxima: warp of the group, lane / 4, row / 8
-  static constexpr int bar_off = max_off + 512;
+  static constexpr int flat_off = max_off + 512;                 // [4] by warp of the group: the item is flat (see kFlatMin)
+  static constexpr int bar_off = flat_off + 64;
   static constexpr int total = bar_off + 512;
   static constexpr int p_col = (QT ? 3 : kGroups) * 64, o_col = p_col + kGroups * 32, q_col = o_col + D;      // TMEM columns (S at 0)
   static constexpr int tmem_cols = 512;
@@ -231,6 +275,7 @@ attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CU
             const __grid_constant__ CUtensorMap tm_v, const __grid_constant__ CUtensorMap tm_sk,
             const __grid_constant__ CUtensorMap tm_sv, const CacheView c, const AttnArgs a) {
   using SM = AttnSmem<D, BKT>;
+  constexpr bool FLAT = !GATHER;                     // prompt tokens have no bounds, and few tiles
   constexpr int RS = SM::RS, RK = SM::RK, RV = SM::RV, NB = SM::NB, SUB = SM::SUB;
   extern __shared__ __align__(1024) uint8_t smem_raw[];
   const uint32_t sbase = smem_u32(smem_raw);
@@ -243,7 +288,7 @@ attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CU
   const uint32_t bias_s = sbase + SM::bias_off;
   const uint32_t bar = sbase + SM::bar_off;
   const uint32_t bar_q_full = bar;
-  const uint32_t bar_q_empty = bar + 8;
+  const uint32_t bar_q_empty = bar + 8;              // the MMAs (or copies) that read Q, and the warps that look at it (FLAT)
   const uint32_t bar_r_full = bar + 16;              // [RS] the K stages, then the V stages
   const uint32_t bar_r_empty = bar_r_full + 8 * RS;  // [RS]
   const uint32_t bar_s_full = bar_r_empty + 8 * RS;  // [4] by key tile: the MMAs' commit, and the issuing warp once the biases are there
@@ -280,7 +325,7 @@ attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CU
   // one thread per barrier
   if (threadIdx.x < kNumBars) {
     const int i = static_cast<int>(threadIdx.x) - (kNumBars - 22);        // s_full, pv_done, s_empty, p_full, xchg, o_free, done, parts, last, qk_done
-    mbar_init(bar + 8 * threadIdx.x, i >= 20 ? 1 : i == 19 ? 4 * (D / 32) : i >= 16 ? kSoftWarps : i >= 12 || (i >= 8 && SM::QT) ? 4 : i >= 8 ? 4 * SUB : i >= 4 || i < 0 ? 1 : 2);
+    mbar_init(bar + 8 * threadIdx.x, FLAT && threadIdx.x == 1 ? 5 : i >= 20 ? 1 : i == 19 ? 4 * (D / 32) : i >= 16 ? kSoftWarps : i >= 12 || (i >= 8 && SM::QT) ? 4 : i >= 8 ? 4 * SUB : i >= 4 || i < 0 ? 1 : 2);
     fence_mbar_init();
   }
   if (threadIdx.x == 0) *abort_flag = *done_flag = 0;
@@ -471,7 +516,7 @@ attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CU
         constexpr uint32_t idesc = make_idesc_bf16(128, QT ? 64 : BKT, 0);
         const uint64_t qd = make_smem_desc(q_s, 16, 1024), kd0 = make_smem_desc(ring_s, 16, 1024);
         bool ok = true;
-        uint32_t nq_used = 0, st = 0, r_phase = 0, b = 0, s_phase = 1;       // stage, logits' columns and their barriers' phases
+        uint32_t nq_used = 0, st = 0, r_phase = 0, b = 0, s_phase = 1, full_b = 0;       // stage, logits' columns and their barriers
         for (int it = it_first; more(it) && ok; it += it_step) {
           const int nt = tiles_of(it);
           if (nt == 0) continue;
@@ -499,10 +544,12 @@ attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CU
               if (QT) umma_ts(s_col, tmem + SM::q_col + kk * 8, bd, idesc, kk != 0, lead);
               else umma_ss(s_col, qd + (((kk >> 2) * kQChunk + (kk & 3) * 32) >> 4), bd, idesc, kk != 0, lead);
             }
-            umma_commit(bar_s_full + 8 * b, lead);
+            const uint32_t full = bar_s_full + 8 * (QT ? full_b : b);
+            umma_commit(full, lead);
             umma_commit(bar_r_empty + 8 * st, lead);
             if (j + 1 == nt) umma_commit(QT ? bar_qk_done : bar_q_empty, lead);
-            if (lead) mbar_arrive(bar_s_full + 8 * b);     // what this warp has seen land (the biases) is there for the waiting warps
+            if (lead) mbar_arrive(full);                   // what this warp has seen land (the biases) is there for the waiting warps
+            full_b = (full_b + 1) % kGroups;
             if (++st == RK) { st = 0; r_phase ^= 1; }
             if (++b == SM::NSB) { b = 0; s_phase ^= 1; }
           }
@@ -567,7 +614,7 @@ attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CU
         const float scale = rsqrtf(static_cast<float>(D)) * 1.4426950408889634f;
         const uint32_t p_t = lane_t + SM::p_col + g * 32, o_t = lane_t + SM::o_col;
         const uint32_t max_s = sbase + SM::max_off + ((warp & 3) * 8 + (lane >> 2)) * 16;
-        const uint32_t bias_t = sbase + SM::bias_off + 8 * (lane & 3);
+        const uint32_t bias_t = sbase + SM::bias_off + 8 * (lane & 3), flat_s = sbase + SM::flat_off + 4 * (warp & 3);
         // the barriers of the hand-over (all sixteen: nothing else uses one after the roles part): this warp waits for the look at the
         // sub-tile before, and tells of its own
         const uint32_t heard = 4 * g + (warp & 3), told = 4 * ((g + 1) % kGroups) + (warp & 3);
@@ -575,15 +622,51 @@ attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CU
         float2 l[4];                                      // running maxima of rows 8 q + lane / 4; sums over the even and the odd columns
 #pragma unroll
         for (int q = 0; q < 4; ++q) { m[q] = -INFINITY; l[q] = make_float2(0.f, 0.f); }
-        for (int t = (g - sub0) & (kGroups - 1); t < ns; t += kGroups) {
+        // the logits' barriers: QT has one per group for their arrival (a barrier's parity tells two phases apart) and one per place for their leaving
+        const uint32_t full = bar_s_full + 8 * (SM::QT ? g : g / SUB), empty = bar_s_empty + 8 * (SM::QT ? 0 : g / SUB);
+        int t = (g - sub0) & (kGroups - 1);
+        bool flat = false, heard_it = false;
+        float need[4];                                    // t = 0: what a logit of the rows may be, less T
+        if (FLAT && t == 0 && ns > 0) {
+          if (ns >= kFlatMin) {
+            ok = ok && mbar_wait_warp(sbase + SM::bar_off, n_done & 1, abort_flag, c.status);
+            const int h = item_at(it) / row_blocks % c.H;
+            HeadBound b = c.bound[h];
+            if (SEG) {
+              const HeadBound p = a.seg_bound[h * kSegParts + lane];
+              b.key = max(b.key, __reduce_max_sync(0xffffffffu, p.key));
+              b.value = max(b.value, __reduce_max_sync(0xffffffffu, p.value));
+            }
+            const uint32_t row = sbase + SM::q_off + ((warp & 3) * 32 + lane) * 128;
+            float sq = 0.f;
+#pragma unroll
+            for (int ch = 0; ch < D / 8; ++ch) {
+              uint4 v;
+              asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(row + (ch >> 3) * kQChunk + (((ch & 7) ^ (lane & 7)) << 4)));
+              sq = square_sum8(v, sq);
+            }
+            // (1.001: the roundings of the norms, of the products' sums and of what follows; 1e-20: components whose squares are below the
+            // smallest float)
+            const float most = (sqrtf(sq) + 1e-20f) * ((sqrtf(__uint_as_float(b.key)) + 1e-20f) * scale * 1.001f) + log2f(static_cast<float>(max(b.count, 1)));
+            const float top = fmaxf(kTop, fminf(kFlatTop, kFlatSum - log2f(static_cast<float>(ns * 64)) - log2f(__uint_as_float(b.value))));
+#pragma unroll
+            for (int q = 0; q < 4; ++q) need[q] = __shfl_sync(0xffffffffu, most, (lane >> 2) + 8 * q) - top;
+          }
+          mbar_arrive_warp(sbase + SM::bar_off + 8);
+        }
+        if (FLAT && ns >= kFlatMin && t > 0) {            // the first sub-tile's warp has said whether the item is flat
+          named_barrier_sync(heard, 64);
+          heard_it = true;
+          flat = lds1(flat_s) != 0.f;
+          if (flat) {
+            if (t + 1 < kGroups) named_barrier_arrive(told, 64);
+            m[0] = m[1] = m[2] = m[3] = lds1(max_s);
+          }
+        }
+        for (; t < ns && !flat; t += kGroups) {
           const int tg = sub0 + t, jg = tg / SUB;
-          const uint32_t sn = SM::QT ? tg : jg, sb = sn % SM::NSB;       // barrier of the logits
-          // QT: a barrier's parity tells two phases apart, and the one before this sub-tile's is that of t - 3, which has to be complete.  From
-          // the fourth on that is known from the group before, which has been told of its own logits; at an item's first three, whose t - 3 is
-          // of an item before, from the groups' meeting, and there the hand-over waits until the logits are under way (64 keys a tile, four tiles
-          // an item, 256 and 444 items 13.6 -> 13.1 and 18.8 -> 18.0 us, sixteen 33.1 -> 32.7; sixty-four 89.1 -> 90.0).
-          if (SM::QT && t > 2) named_barrier_sync(heard, 64);
-          if (SM::QT || !s_ready) ok = ok && mbar_wait_warp(bar_s_full + 8 * sb, (sn / SM::NSB) & 1, abort_flag, c.status);
+          const uint32_t sb = SM::QT ? tg % SM::NSB : 0;
+          if (!s_ready) ok = ok && mbar_wait_warp(full, (tg / kGroups) & 1, abort_flag, c.status);
           tc_fence_after();
           // the logits of this warp's rows: x[hf][4 k + 2 e + c] is row 16 hf + 8 e + lane / 4, column 8 k + 2 (lane & 3) + c
           uint32_t x[2][32];
@@ -594,12 +677,13 @@ attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CU
           float2 bias[8];
 #pragma unroll
           for (int k = 0; k < 8; ++k) bias[k] = lds2(bp + 32 * k);
-          if (t > 0 && (!SM::QT || t <= 2)) named_barrier_sync(heard, 64);
+          if (t > 0 && !heard_it) named_barrier_sync(heard, 64);
+          heard_it = false;
           const float4 seen = t > 0 ? lds4(max_s) : make_float4(-INFINITY, -INFINITY, -INFINITY, -INFINITY);
           bool p_free = tg < kGroups || mbar_test_wait(bar_pv_done + 8 * g, (tg / kGroups - 1) & 1);
           tmem_wait_ld();
           tc_fence_before();
-          mbar_arrive_warp(bar_s_empty + 8 * sb);          // the logits are in registers
+          mbar_arrive_warp(empty + 8 * sb);                // the logits are in registers
           float mx[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
 #pragma unroll
           for (int k = 0; k < 8; ++k) {
@@ -648,6 +732,12 @@ attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CU
                 l[q].y *= f;
               }
               m[q] = top;
+            }
+            if (FLAT && t == 0 && ns >= kFlatMin) {
+              const float low = fminf(fminf(m[0], m[1]), fminf(m[2], m[3]));
+              flat = __all_sync(0xffffffffu, need[0] <= low && need[1] <= low && need[2] <= low && need[3] <= low && low > -INFINITY);
+              if (flat) m[0] = m[1] = m[2] = m[3] = low;
+              if (lane == 0) asm volatile("st.shared.f32 [%0], %1;" ::"r"(flat_s), "f"(flat ? 1.f : 0.f) : "memory");
             }
             if (__any_sync(0xffffffffu, raised)) {
               if (t > 0) {
@@ -701,12 +791,60 @@ attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CU
               }
             tmem_st_half_frag(p_t + hf * kHalf, p);
           }
-          const uint32_t jn = (tg + kGroups) / SUB;            // (asked here, needed later: a barrier answers slowly while MMAs run)
-          if (!SM::QT) s_ready = mbar_test_wait(bar_s_full + 8 * (jn % SM::NSB), (jn / SM::NSB) & 1);
+          s_ready = mbar_test_wait(full, (tg / kGroups + 1) & 1);      // (asked here, needed later: a barrier answers slowly while MMAs run)
           tmem_wait_st();
           tc_fence_before();
           mbar_arrive_warp(bar_p_full + 8 * g);
-          if (!SM::QT) s_ready = __all_sync(0xffffffffu, s_ready);
+          s_ready = __all_sync(0xffffffffu, s_ready);
+        }
+        if (FLAT) {
+          const float2 ref = make_float2(-m[0], -m[0]), scale2 = make_float2(scale, scale);
+          for (; t < ns; t += kGroups) {
+            const int tg = sub0 + t, jg = tg / SUB;
+            const uint32_t phase = (tg / kGroups) & 1, sb = SM::QT ? tg % SM::NSB : 0;
+            if (!s_ready) ok = ok && mbar_wait_warp(full, phase, abort_flag, c.status);
+            tc_fence_after();
+            uint32_t x[2][32];
+#pragma unroll
+            for (int hf = 0; hf < 2; ++hf) tmem_ld_frag(lane_t + (SM::QT ? sb : g) * 64 + hf * kHalf, x[hf]);
+            const uint32_t bp = bias_t + ((jg % NB) * BKT + (tg % SUB) * 64) * 4;
+            float2 bias[8];
+#pragma unroll
+            for (int k = 0; k < 8; ++k) bias[k] = lds2(bp + 32 * k);
+            const bool p_free = mbar_test_wait(bar_pv_done + 8 * g, phase ^ 1);
+#pragma unroll
+            for (int k = 0; k < 8; ++k) bias[k] = fadd2(bias[k], ref);
+            tmem_wait_ld();
+            tc_fence_before();
+            mbar_arrive_warp(empty + 8 * sb);
+            uint32_t p[2][16];
+#pragma unroll
+            for (int hf = 0; hf < 2; ++hf) {
+#pragma unroll
+              for (int k = 0; k < 8; ++k)
+#pragma unroll
+                for (int e = 0; e < 2; ++e) {
+                  const uint32_t* v = &x[hf][4 * k + 2 * e];
+                  const float2 u = ffma2(make_float2(__uint_as_float(v[0]), __uint_as_float(v[1])), scale2, bias[k]);
+                  float2 pr;
+                  if (2 * k + e < kPolyPairs<D>) pr = poly_exp2(u);
+                  else pr = make_float2(fast_exp2(u.x), fast_exp2(u.y));
+                  const uint32_t b = pack_bf16x2(pr.x, pr.y);
+                  p[hf][2 * k + e] = b;
+                  add_bf16x2(l[2 * hf + e], b);
+                }
+            }
+            // P is free once P V of the group's last sub-tile has read it; waited for here, behind the exponentials
+            if (!__all_sync(0xffffffffu, p_free)) ok = ok && mbar_wait_warp(bar_pv_done + 8 * g, phase ^ 1, abort_flag, c.status);
+            tc_fence_after();
+            tmem_st_half_frag(p_t, p[0]);
+            tmem_st_half_frag(p_t + kHalf, p[1]);
+            s_ready = mbar_test_wait(full, phase ^ 1);
+            tmem_wait_st();
+            tc_fence_before();
+            mbar_arrive_warp(bar_p_full + 8 * g);
+            s_ready = __all_sync(0xffffffffu, s_ready);
+          }
         }
         // ---- the groups meet: (m, l) of every row through shared memory ----
         const uint32_t xchg = sbase + SM::xchg_off + (n_done & 1) * kGroups * 1024;

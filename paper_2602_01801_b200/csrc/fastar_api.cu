@@ -145,6 +145,7 @@ size_t carve(const fastar_cache_desc& d, uint8_t* base, CacheView* v) {
   t.kcode = reinterpret_cast<uint32_t*>(take(H * CAP * 4));
   t.hk = reinterpret_cast<__nv_bfloat16*>(take(H * t.CAPB * t.hist_cols * 2));
   t.len = reinterpret_cast<int32_t*>(take(H * 4));
+  t.bound = reinterpret_cast<HeadBound*>(take(H * sizeof(HeadBound)));
   t.now = reinterpret_cast<int32_t*>(take(4));
   t.status = reinterpret_cast<int32_t*>(take(4));
   t.lsh = reinterpret_cast<__nv_bfloat16*>(take(32 * D * 2));
@@ -205,6 +206,7 @@ size_t carve(const fastar_cache_desc& d, uint8_t* base, CacheView* v) {
   t.q8_probe = t.search_bits == 8 ? take(H * MT * 128) : nullptr;
   t.qn_probe = t.search_bits == 8 ? reinterpret_cast<float*>(take(H * MT * 4)) : nullptr;
   t.seg_bias = reinterpret_cast<float*>(take((MT + 128) * 4));
+  t.seg_bound = reinterpret_cast<HeadBound*>(take(H * kSegParts * sizeof(HeadBound)));
   t.code_q_ca = reinterpret_cast<uint32_t*>(take(H * MT * 4));
   t.code_p_ca = reinterpret_cast<uint32_t*>(take(H * MP * 4));
   t.nselp = reinterpret_cast<int32_t*>(take(H * t.max_frames * 4));
@@ -255,6 +257,8 @@ int make_range(fastar_cache* c, int h0, int count, HeadRange* out) {
   v.count += cap; v.stamp += cap; v.log2m += cap; v.rnorm += cap; v.kcode += cap; v.cnt += cap; v.cur += cap;
   v.hk += h * v.CAPB * v.hist_cols;
   v.len += h;
+  v.bound += h;
+  v.seg_bound += h * kSegParts;
   v.best += mt; v.segslot += mt; v.ulist += mt; v.rnorm_new += mt; v.code_new += mt; v.match += mt; v.sim += mt; v.order += mt;
   v.dest += mt; v.victims += mt; v.code_q_ca += mt; v.code_q_sa += mt;
   v.segpos += h * (v.max_tokens + 1);
@@ -290,11 +294,6 @@ __global__ void combine_scores_kernel(const float* __restrict__ lo, const float*
   const int h = blockIdx.y;
   for (int q = blockIdx.x * blockDim.x + threadIdx.x; q < per_head; q += gridDim.x * blockDim.x)
     out[static_cast<int64_t>(h) * per_head + q] = lo[h * head_stride + q] + 256.f * hi[h * head_stride + q];
-}
-
-__global__ void seg_bias_kernel(float* __restrict__ bias, int ns, int total) {
-  chain_wait();
-  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < total; i += gridDim.x * blockDim.x) bias[i] = i < ns ? 0.f : -INFINITY;
 }
 
 __global__ void copy_rows3_kernel(const int32_t* __restrict__ src, int64_t src_hs, int src_rs, int32_t* __restrict__ dst, int rows,
@@ -779,9 +778,8 @@ static int annsa_impl(fastar_cache_t* c, const HeadRange& range, bool hashed, bo
     if (r != FASTAR_OK) return r;
     a.seg_tiles = (ns + v.PT - 1) / v.PT;
     a.seg_bias = v.seg_bias;
-    launch_chained(seg_bias_kernel, (a.seg_tiles * v.PT + 255) / 256, 256, 0, st, v.seg_bias, ns, a.seg_tiles * v.PT);
-    if (cudaGetLastError() != cudaSuccess) return FASTAR_ERR_CUDA;
-    c->launches += 1;
+    a.seg_bound = v.seg_bound;
+    ACC(launch_segment(v, sg[0].p, sg[0].hs, sg[0].ts, sg[1].p, sg[1].hs, sg[1].ts, ns, a.seg_tiles, st));
   }
   ACCK(FASTAR_K_S5_ATTENTION, launch_attention_paged(v, tm_q, c->tm_pool_k, c->tm_pool_v, k_seg ? &tm_sk : nullptr,
                                                      k_seg ? &tm_sv : nullptr, a, st));

@@ -6,6 +6,7 @@
 //   S2  per-block bucket histograms, S4 / C2 top-k with ties to the lower index   Sections 5.3, 5.4
 #include "common.h"
 #include "ptx.cuh"
+#include "bound.cuh"
 #include "topk.cuh"
 
 namespace fastar {
@@ -123,7 +124,7 @@ template <int D, int ROWS>
 __global__ void __launch_bounds__(256, 2) prep_kernel(const __nv_bfloat16* __restrict__ x, int H, int n, int64_t hs, int64_t ts,
                                                    const __nv_bfloat16* __restrict__ lsh, int T, int B,
                                                    uint32_t* __restrict__ code_out, float* __restrict__ rnorm_out,
-                                                   int64_t out_stride, UpdateScratch clear, BlockHist bh) {
+                                                   int64_t out_stride, HeadBound* bound, UpdateScratch clear, BlockHist bh) {
   constexpr bool BLOCKS = ROWS > 0;
   constexpr int per_block = BLOCKS ? ROWS / 16 : 1, blocks_a_pass = BLOCKS ? 8 / per_block : 1;
   __shared__ __align__(16) int hist[BLOCKS ? 2 : 1][blocks_a_pass][BLOCKS ? 1024 : 4];      // [pass & 1][block of the pass]
@@ -189,6 +190,7 @@ __global__ void __launch_bounds__(256, 2) prep_kernel(const __nv_bfloat16* __res
     const int h = grp / groups_per_head;
     const int r0 = (grp - h * groups_per_head) * 16;
     const bool more = grp + stride < total_groups;
+    const uint32_t had = !BLOCKS && bound ? bound[h].key : 0xFFFFFFFFu;
     if (more) rows(grp + stride);
     if (!BLOCKS || grp < total_groups) {         // (the last pass may have a block less)
       float acc[4][4];
@@ -234,6 +236,7 @@ __global__ void __launch_bounds__(256, 2) prep_kernel(const __nv_bfloat16* __res
         sqa += __shfl_xor_sync(0xffffffffu, sqa, o);
         sqb += __shfl_xor_sync(0xffffffffu, sqb, o);
       }
+      if (!BLOCKS && bound) raise_bound_warp(&bound[h].key, had, max(__float_as_uint(sqa), __float_as_uint(sqb)));
       uint32_t ca = 0, cb = 0;
       for (int tt = 0; tt < T; ++tt) {
         ca |= ((ma >> (tt * B)) & ((1u << B) - 1u)) << (8 * tt);
@@ -273,14 +276,15 @@ __global__ void __launch_bounds__(256, 2) prep_kernel(const __nv_bfloat16* __res
 static int launch_prep_generic(const CacheView& c, const __nv_bfloat16* x, int n, int64_t hs, int64_t ts, uint32_t* code_out,
                                float* rnorm_out, int64_t out_stride, cudaStream_t st, const UpdateScratch& clear = UpdateScratch{}) {
   if (n <= 0) return 0;
+  HeadBound* bound = rnorm_out ? c.bound : nullptr;               // cached keys, or keys that will be
   const int groups = ((n + 15) / 16) * c.H;                      // 16 rows per warp pass
   // CTAs for the rows (eight warps of 16 a pass) or for the zeros (32 KB each), whichever needs more: a few tokens against many heads
   // with long caches leave far more to clear than to hash (40 heads x 65536 slots, 1 to 16 tokens: an update of 81 us with CTAs for
   // the rows only, 50 with these).
   const int64_t want = max(static_cast<int64_t>(groups + 7) / 8, (clear.n_best / 2 + clear.n_cnt16 + 2047) / 2048);
   const dim3 grid(static_cast<unsigned>(max(static_cast<int64_t>(1), min(want, static_cast<int64_t>(2 * 148)))));
-  if (c.D == 128) launch_chained(prep_kernel<128, 0>, grid, 256, 0, st, x, c.H, n, hs, ts, c.lsh, c.T, c.B, code_out, rnorm_out, out_stride, clear, BlockHist{});
-  else launch_chained(prep_kernel<64, 0>, grid, 256, 0, st, x, c.H, n, hs, ts, c.lsh, c.T, c.B, code_out, rnorm_out, out_stride, clear, BlockHist{});
+  if (c.D == 128) launch_chained(prep_kernel<128, 0>, grid, 256, 0, st, x, c.H, n, hs, ts, c.lsh, c.T, c.B, code_out, rnorm_out, out_stride, bound, clear, BlockHist{});
+  else launch_chained(prep_kernel<64, 0>, grid, 256, 0, st, x, c.H, n, hs, ts, c.lsh, c.T, c.B, code_out, rnorm_out, out_stride, bound, clear, BlockHist{});
   return cudaGetLastError() == cudaSuccess ? 1 : FASTAR_ERR_CUDA;
 }
 // Codes of the queries and the bucket histograms of their blocks of block_q rows.
@@ -289,7 +293,7 @@ int launch_query_blocks(const CacheView& c, const __nv_bfloat16* q, int nq, int6
   const int64_t groups = static_cast<int64_t>((nq + block_q - 1) / block_q) * c.H * (block_q / 16);
   const int grid = static_cast<int>(min((groups + 7) / 8, static_cast<int64_t>(2 * 148)));
   auto launch = [&](auto kernel) {
-    launch_chained(kernel, grid, 256, 0, st, q, c.H, nq, hs, ts, c.lsh, c.T, c.B, c.code_q_sa, nullptr, c.max_tokens, UpdateScratch{}, BlockHist{c.hq, c.max_qb, c.hist_cols});
+    launch_chained(kernel, grid, 256, 0, st, q, c.H, nq, hs, ts, c.lsh, c.T, c.B, c.code_q_sa, nullptr, c.max_tokens, nullptr, UpdateScratch{}, BlockHist{c.hq, c.max_qb, c.hist_cols});
   };
   if (c.D == 128) block_q == 128 ? launch(prep_kernel<128, 128>) : launch(prep_kernel<128, 64>);
   else block_q == 128 ? launch(prep_kernel<64, 128>) : launch(prep_kernel<64, 64>);
@@ -931,6 +935,7 @@ __global__ void __launch_bounds__(128) key_hist_kernel(const CacheView c, int us
   if (b == 0 && threadIdx.x == 0 && use_plan) {
     const PlanRec pr = c.plan[h];
     c.len[h] = pr.len_new;
+    c.bound[h].count = min(max(c.bound[h].count, 1) + pr.n_matched, 1 << 30);          // a slot of m takes no more than all that matched
     if (c.pool_shared && pr.pages_granted > 0) atomicAdd(c.next_free, pr.pages_granted);
     if (stats_out) {
       fastar_update_stats s;
@@ -950,6 +955,53 @@ __global__ void __launch_bounds__(128) key_hist_kernel(const CacheView c, int us
 int launch_finalize_hist(const CacheView& c, fastar_update_stats* stats_out, int advance_clock, cudaStream_t st) {
   launch_chained(key_hist_kernel, dim3(c.CAPB, c.H), 128, c.hist_cols * 4, st, c, advance_clock >= 0 ? 1 : 0, stats_out,
                                                                   advance_clock > 0 ? 1 : 0);
+  return cudaGetLastError() == cudaSuccess ? 1 : FASTAR_ERR_CUDA;
+}
+
+// ---------------------------------------------------------------------------------------------
+// An un-cached segment of an attention call: the biases of its rows, and what its keys and values do not exceed, by kSegParts parts of the
+// tokens of a head, which the attention puts together (so there is nothing to clear and no atomic).  Half a warp (a quarter at d = 64) has a row.
+// ---------------------------------------------------------------------------------------------
+template <int D>
+__global__ void __launch_bounds__(256) segment_kernel(const CacheView c, const __nv_bfloat16* __restrict__ k, int64_t khs, int64_t kts,
+                                                      const __nv_bfloat16* __restrict__ v, int64_t vhs, int64_t vts, int ns, int total) {
+  constexpr int LPR = D / 8, RPC = 256 / LPR;          // lanes a row, rows a CTA's pass
+  __shared__ HeadBound part;
+  if (threadIdx.x == 0) part = HeadBound{};
+  __syncthreads();
+  chain_wait();
+  const int h = blockIdx.y, sl = threadIdx.x % LPR;
+  for (int i = (h * kSegParts + blockIdx.x) * 256 + threadIdx.x; i < total; i += c.H * kSegParts * 256) c.seg_bias[i] = i < ns ? 0.f : -INFINITY;
+  const int r0 = static_cast<int>(static_cast<int64_t>(ns) * blockIdx.x / kSegParts), r1 = static_cast<int>(static_cast<int64_t>(ns) * (blockIdx.x + 1) / kSegParts);
+  uint32_t kmost = 0, vmost = 0;
+  constexpr int RPW = 32 / LPR, B = 4;                 // rows a warp, rows of a thread that are under way
+  for (int rb = r0 + (threadIdx.x >> 5) * RPW; rb < r1; rb += B * RPC) {
+    uint4 kr[B], vr[B];
+#pragma unroll
+    for (int b = 0; b < B; ++b) {                        // past the end the last row again
+      const int row = min(rb + b * RPC + (threadIdx.x & 31) / LPR, r1 - 1);
+      kr[b] = *reinterpret_cast<const uint4*>(k + h * khs + row * kts + sl * 8);
+      vr[b] = *reinterpret_cast<const uint4*>(v + h * vhs + row * vts + sl * 8);
+    }
+#pragma unroll
+    for (int b = 0; b < B; ++b) {
+      vmost = max(vmost, largest8(vr[b]));
+      float sq = square_sum8(kr[b], 0.f);
+#pragma unroll
+      for (int o = LPR / 2; o >= 1; o >>= 1) sq += __shfl_xor_sync(0xffffffffu, sq, o);
+      kmost = max(kmost, __float_as_uint(sq));
+    }
+  }
+  raise_bound_warp(&part.key, 0, kmost);
+  raise_bound_warp(&part.value, 0, vmost);
+  __syncthreads();
+  if (threadIdx.x == 0) c.seg_bound[h * kSegParts + blockIdx.x] = part;
+}
+int launch_segment(const CacheView& c, const __nv_bfloat16* k, int64_t khs, int64_t kts, const __nv_bfloat16* v, int64_t vhs, int64_t vts, int ns,
+                   int tiles, cudaStream_t st) {
+  const dim3 grid(kSegParts, c.H);
+  if (c.D == 128) launch_chained(segment_kernel<128>, grid, 256, 0, st, c, k, khs, kts, v, vhs, vts, ns, tiles * c.PT);
+  else launch_chained(segment_kernel<64>, grid, 256, 0, st, c, k, khs, kts, v, vhs, vts, ns, tiles * c.PT);
   return cudaGetLastError() == cudaSuccess ? 1 : FASTAR_ERR_CUDA;
 }
 
@@ -1077,6 +1129,7 @@ __global__ void reset_meta_kernel(const CacheView c) {
     // does not hold stay at page 0, a valid address that only masked-out slots ever read)
     if (q < static_cast<int64_t>(c.H) * c.CAPB) c.page_table[q] = c.pool_shared ? 0 : static_cast<int32_t>(q);
     if (q < c.H) c.len[q] = 0;
+    if (q < c.H) c.bound[q] = HeadBound{0u, __float_as_uint(64.f), 0, 0};      // (ordinary values are below 64: an update raises nothing)
     if (q == 0) { *c.now = 0; *c.status = 0; *c.next_free = 0; }
   }
 }
@@ -1097,8 +1150,13 @@ __global__ void import_fix_kernel(const CacheView c) {
   const int L = c.len[h];
   const int lane = threadIdx.x & 31;
   const int32_t* pt_h = c.page_table + static_cast<int64_t>(h) * c.CAPB;
+  uint32_t vmost = 0, cmost = 1;
   for (int s = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); s < c.CAP; s += gridDim.x * (blockDim.x >> 5)) {
     const int64_t q = static_cast<int64_t>(h) * c.CAP + s;
+    if (s < L) {
+      vmost = max(vmost, largest8(*reinterpret_cast<const uint4*>(c.pool_v + slot_row_offset(c, pt_h, s) + (lane & (D / 8 - 1)) * 8)));
+      cmost = max(cmost, static_cast<uint32_t>(max(c.count[q], 1)));
+    }
     if (s >= L) {
       const int64_t ro = slot_row_offset(c, pt_h, s);
       for (int e = lane * 2; e < D; e += 64) {
@@ -1110,6 +1168,8 @@ __global__ void import_fix_kernel(const CacheView c) {
       c.log2m[q] = log2f(static_cast<float>(max(1, c.count[q])));
     }
   }
+  raise_bound_warp(&c.bound[h].value, 0, vmost);
+  if (lane == 0) atomicMax(&c.bound[h].count, static_cast<int>(cmost));
 }
 int launch_import_derive(const CacheView& c, cudaStream_t st) {
   // codes and reciprocal norms of every slot (the pools are [H][CAP][D] under the identity page table)

@@ -289,3 +289,61 @@ def test_items_of_caches_that_are_not_full(d, pt, H, nqb, tiles, lens, seg):
         # rounding of the probabilities and of the output
         assert (out[h].double() - want).abs().max() <= 2.0 ** -7 * vv.abs().max()
         assert (out[h].double() - want).norm() <= 1e-2 * want.norm()
+
+
+@pytest.mark.parametrize("d,pt", [(64, 64), (64, 128), (128, 64), (128, 128)])
+@pytest.mark.parametrize("tiles", [7, 8, 9, 21])
+def test_bounds_of_the_logits(d, pt, tiles):
+    """Heads whose largest norms, values and multiplicities bound every logit near an item's first ones, and heads where they do not: a last key
+    that towers over the others, values near the end of bf16's range, rows of very unequal norms, keys and values of zero.  The same for keys
+    that came by updates, by an import, and as a segment."""
+    import torch
+    from paper_2602_01801_b200 import fastar
+    rng = np.random.default_rng(d + pt + tiles)
+    H, nq, n = 8, 200, tiles * 64
+    cap = -(-n // 128) * 128 + 128
+    q, k, v = (rng.standard_normal((H, m, d)).astype(np.float32) for m in (nq, n, n))
+    count = np.ones((H, n), np.int32)
+    q[1, ::3] *= 30.0                                      # rows of a warp far apart
+    q[2, :, 0] = np.abs(q[2, :, 0]) + 4.0
+    k[2, n - 1] = 0.0
+    k[2, n - 1, 0] = 12.0 * math.sqrt(d)                   # the last key, 50 binary orders and more above the others
+    v[3] *= 2.0 ** 100                                     # 8 binary orders of room, and logits that rise by about 20
+    q[3, :, 0], k[3, :, 0] = 4.0, np.linspace(0.0, 3.5 * math.sqrt(d) / math.log2(math.e), n)
+    count[4] = rng.integers(1, 5000, n)
+    k[5, n // 2:], v[5, : n // 2] = 0.0, 0.0
+    v[6] = 0.0
+    v[7] *= 2.0 ** -100
+    k[7] *= 3.0
+    q, k, v = (synth.round_bf16(x) for x in (q, k, v))
+    lsh = rng.standard_normal((32, d)).astype(np.float32)
+    dq, dk, dv = (fastar.to_device(x) for x in (q, k, v))
+
+    def check(out, times, but=-1):
+        for h in range(H):
+            if h == but:
+                continue
+            s = q[h].astype(np.float64) @ k[h].T.astype(np.float64) / math.sqrt(d) + np.log(times[h])
+            p = np.exp(s - s.max(1, keepdims=True))
+            want = (p / p.sum(1, keepdims=True)) @ v[h].astype(np.float64)
+            got = out[h].float().cpu().numpy().astype(np.float64)
+            assert np.isfinite(got).all(), f"head {h}"
+            # as above: rounding of the probabilities and of the output
+            assert np.abs(got - want).max() <= 2.0 ** -7 * np.abs(v[h]).max(), f"head {h}"
+            assert np.linalg.norm(got - want) <= 1e-2 * np.linalg.norm(want), f"head {h}"
+
+    def new():
+        return fastar.Cache(H, d, cap, pt, lsh, max_tokens=max(n, nq))
+    cache = new()
+    cache.import_state(fastar.bf16_bits(k), fastar.bf16_bits(v), np.full(H, n), count)
+    check(cache.annsa(dq, 128, cap // pt)["out"], count)
+    cut = n // 2 + 5
+    cache.import_state(fastar.bf16_bits(k[:, :cut]), fastar.bf16_bits(v[:, :cut]), np.full(H, cut), count[:, :cut])
+    check(cache.annsa_segment(dq, dk[:, cut:], dv[:, cut:], 128, cap // pt)["out"], np.where(np.arange(n) < cut, count, 1))
+    cache = new()
+    for a, b in ((0, cut), (cut, n)):                      # (a threshold that nothing reaches: appended)
+        cache.update(dk[:, a:b], dv[:, a:b], n, 2.0)
+    check(cache.annsa(dq, 128, cap // pt)["out"], np.ones((H, n)))
+    cache.update(dk[:, :cut], dv[:, :cut], n, 0.999)       # every key finds itself: multiplicities of two, the same mean values
+    check(cache.annsa(dq, 128, cap // pt)["out"], np.broadcast_to(np.where(np.arange(n) < cut, 2, 1), (H, n)), but=5)      # (keys of zero find nothing)
+    assert cache.status() == 0
