@@ -35,7 +35,7 @@
 //     an SM's instruction caches bear (stalls for instructions: a twentieth of a warp's time, and a sixth with a little more code in the
 //     kernel), so the cut is a variant of its own;
 //   - items whose logits a bound keeps near the first sub-tile's need no maximum at all (see kFlatMin): the loop for them is what the
-//     arithmetic needs, 245 instructions, and the exponentials and the tensor core bound it (0.74 and 0.73 of the time at d = 128);
+//     arithmetic needs, 270 instructions, and the exponentials and the tensor core bound it (0.74 and 0.73 of the time at d = 128);
 //   - the CTA stays for its items, and the copies and Q K^T run ahead into the next one, whose first logits are there when the
 //     output of the last has left.
 // TMEM columns: S 4 x 64, P 4 x 32, O D; with key tiles of 64: S 3 x 64, P, O and Q D / 2 (AttnSmem::QT).  K and V tiles have a TMA ring
@@ -43,8 +43,8 @@
 // Measured (B200, kernel time; two groups with whole tiles, a CTA per item, a limit of 8 -> this): 12 heads, d = 128, 4 680 queries on
 // 32 of 224 blocks 120.5 -> 105.4 us (0.68 of the measured bf16 peak); the same with the chunk's 4 680 keys beside 241 -> 218 us; 8
 // heads, 4 096 queries on all 16 384 keys 275 -> 246 us (108 of 148 CTAs have two items); d = 64, 64 of 1 024 blocks 142 -> 125 us,
-// 16 of 160 blocks 49 -> 39.5 us.  With flat items: the first three 99 -> 88, 194 -> 166 and 226 -> 192 us, the last two 118 -> 91 and
-// 37.8 -> 31.2.  Row sums by a warp-level product with ones instead of adds: 311 us for 242 (it takes the tensor
+// 16 of 160 blocks 49 -> 39.5 us.  With flat items: the first three 99 -> 89, 194 -> 174 and 226 -> 199 us, the last two 118 -> 95 and
+// 37.8 -> 32.1.  Row sums by a warp-level product with ones instead of adds: 311 us for 242 (it takes the tensor
 // core); sums of the unrounded probabilities: 4 % faster, not as exact.
 // Warp roles: warps 0-15 soft-max groups 0-3, 16 copies Q and K (TMA or gather), 17 Q K^T, 18 P V, 19 copies V.
 #include "bound.cuh"
@@ -79,14 +79,17 @@ __device__ __forceinline__ float4 lds4(uint32_t addr) {
 // for values up to 2^119 / keys.  What the code calls the maximum, and the warps hand on, is that reference.
 constexpr float kHead = 16.f, kTop = 8.f;
 
-// What a cut costs, in times of a tile of BKT keys (0.78 us with 128, 0.40 with 64): a part's way through memory, adding it up, another stop
-// of a CTA; a tile in the variant with the cut; and the share of the whole that has to be saved (see launch_attn).
+// What a cut costs, in times of a tile of BKT keys (0.60 us with 128, 0.32 with 64): a part's way through memory, which is longer by `part`
+// for every part there is, adding one up, another stop of a CTA; and the share of the whole that has to be saved (see launch_attn).
 template <int BKT>
 struct CutCost {
-  static constexpr float store = BKT == 64 ? 6.f : 3.2f, add = BKT == 64 ? 1.7f : 0.95f, stop = BKT == 64 ? 20.f : 14.f;
-  static constexpr float loop = BKT == 64 ? 1.2f : 1.f, gain = 0.05f;
+  static constexpr float store = BKT == 64 ? 6.2f : 3.2f, part = BKT == 64 ? 0.066f : 0.029f, add = BKT == 64 ? 1.45f : 0.8f, stop = BKT == 64 ? 14.f : 8.3f;
+  static constexpr float gain = 0.05f;
 };
 
+__device__ __forceinline__ void sts4(uint32_t addr, const float (&v)[4]) {
+  asm volatile("st.shared.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "f"(v[0]), "f"(v[1]), "f"(v[2]), "f"(v[3]) : "memory");
+}
 __device__ __forceinline__ float lds1(uint32_t addr) {
   float v;
   asm volatile("ld.shared.f32 %0, [%1];" : "=f"(v) : "r"(addr));
@@ -115,8 +118,9 @@ __device__ __forceinline__ void add_bf16x2(float2& s, uint32_t b) {
 // Flat items.  A logit is at most |q| max |k| / sqrt(d) + log2 max m; the cache keeps the largest of each head (HeadBound), a segment's come
 // with the call, and |q| is worked out here.  If that, for the rows of a warp, is not more than T above the reference that an item's first
 // sub-tile gives, nothing after it can ask for another reference: the sub-tiles that follow need no maximum, no look at the others' and no
-// hand-over, which are 160 of the loop's 440 instructions; and one reference for the four rows of a thread (the lowest of theirs, so that
-// a row's largest probability is 2^-kHead at least, as ever) goes into the biases.  T is as large as the sums of P V allow: keys x 2^T x
+// hand-over, which are 160 of the loop's 440 instructions.  (One reference for the four rows of a thread, within the biases, would spare 24
+// more and is 1 to 3 % faster, but then the largest probabilities no longer lie just below a power of two, where bf16 is finest: error against
+// 64 bits 0.00230 -> 0.00233.)  T is as large as the sums of P V allow: keys x 2^T x
 // max |v| is below 2^118, or T is kTop, as where the maximum is looked for.  Items of fewer sub-tiles than kFlatMin don't ask.
 constexpr int kFlatMin = 8;
 constexpr float kFlatTop = 96.f, kFlatSum = 118.f;
@@ -626,7 +630,6 @@ attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CU
         const uint32_t full = bar_s_full + 8 * (SM::QT ? g : g / SUB), empty = bar_s_empty + 8 * (SM::QT ? 0 : g / SUB);
         int t = (g - sub0) & (kGroups - 1);
         bool flat = false, heard_it = false;
-        float need[4];                                    // t = 0: what a logit of the rows may be, less T
         if (FLAT && t == 0 && ns > 0) {
           if (ns >= kFlatMin) {
             ok = ok && mbar_wait_warp(sbase + SM::bar_off, n_done & 1, abort_flag, c.status);
@@ -649,8 +652,11 @@ attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CU
             // smallest float)
             const float most = (sqrtf(sq) + 1e-20f) * ((sqrtf(__uint_as_float(b.key)) + 1e-20f) * scale * 1.001f) + log2f(static_cast<float>(max(b.count, 1)));
             const float top = fmaxf(kTop, fminf(kFlatTop, kFlatSum - log2f(static_cast<float>(ns * 64)) - log2f(__uint_as_float(b.value))));
+            // what the rows' logits may be, less T, to where the maxima will be: nobody looks there yet, and it would not fit the registers
+            float need[4];
 #pragma unroll
             for (int q = 0; q < 4; ++q) need[q] = __shfl_sync(0xffffffffu, most, (lane >> 2) + 8 * q) - top;
+            if ((lane & 3) == 0) sts4(max_s, need);
           }
           mbar_arrive_warp(sbase + SM::bar_off + 8);
         }
@@ -660,7 +666,8 @@ attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CU
           flat = lds1(flat_s) != 0.f;
           if (flat) {
             if (t + 1 < kGroups) named_barrier_arrive(told, 64);
-            m[0] = m[1] = m[2] = m[3] = lds1(max_s);
+            const float4 ref = lds4(max_s);
+            m[0] = ref.x; m[1] = ref.y; m[2] = ref.z; m[3] = ref.w;
           }
         }
         for (; t < ns && !flat; t += kGroups) {
@@ -734,9 +741,9 @@ attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CU
               m[q] = top;
             }
             if (FLAT && t == 0 && ns >= kFlatMin) {
-              const float low = fminf(fminf(m[0], m[1]), fminf(m[2], m[3]));
-              flat = __all_sync(0xffffffffu, need[0] <= low && need[1] <= low && need[2] <= low && need[3] <= low && low > -INFINITY);
-              if (flat) m[0] = m[1] = m[2] = m[3] = low;
+              const float4 need = lds4(max_s);
+              flat = need.x <= m[0] && need.y <= m[1] && need.z <= m[2] && need.w <= m[3] && fminf(fminf(m[0], m[1]), fminf(m[2], m[3])) > -INFINITY;
+              flat = __all_sync(0xffffffffu, flat);
               if (lane == 0) asm volatile("st.shared.f32 [%0], %1;" ::"r"(flat_s), "f"(flat ? 1.f : 0.f) : "memory");
             }
             if (__any_sync(0xffffffffu, raised)) {
@@ -762,8 +769,7 @@ attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CU
                     tmem_st_frag16(o_c, v);
                   }
               }
-              if ((lane & 3) == 0)
-                asm volatile("st.shared.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(max_s), "f"(m[0]), "f"(m[1]), "f"(m[2]), "f"(m[3]) : "memory");
+              if ((lane & 3) == 0) sts4(max_s, m);
               __syncwarp();
             }
           }
@@ -798,7 +804,7 @@ attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CU
           s_ready = __all_sync(0xffffffffu, s_ready);
         }
         if (FLAT) {
-          const float2 ref = make_float2(-m[0], -m[0]), scale2 = make_float2(scale, scale);
+          const float2 scale2 = make_float2(scale, scale);
           for (; t < ns; t += kGroups) {
             const int tg = sub0 + t, jg = tg / SUB;
             const uint32_t phase = (tg / kGroups) & 1, sb = SM::QT ? tg % SM::NSB : 0;
@@ -812,8 +818,6 @@ attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CU
 #pragma unroll
             for (int k = 0; k < 8; ++k) bias[k] = lds2(bp + 32 * k);
             const bool p_free = mbar_test_wait(bar_pv_done + 8 * g, phase ^ 1);
-#pragma unroll
-            for (int k = 0; k < 8; ++k) bias[k] = fadd2(bias[k], ref);
             tmem_wait_ld();
             tc_fence_before();
             mbar_arrive_warp(empty + 8 * sb);
@@ -825,7 +829,8 @@ attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CU
 #pragma unroll
                 for (int e = 0; e < 2; ++e) {
                   const uint32_t* v = &x[hf][4 * k + 2 * e];
-                  const float2 u = ffma2(make_float2(__uint_as_float(v[0]), __uint_as_float(v[1])), scale2, bias[k]);
+                  const float ref = -m[2 * hf + e];
+                  const float2 u = fadd2(ffma2(make_float2(__uint_as_float(v[0]), __uint_as_float(v[1])), scale2, bias[k]), make_float2(ref, ref));
                   float2 pr;
                   if (2 * k + e < kPolyPairs<D>) pr = poly_exp2(u);
                   else pr = make_float2(fast_exp2(u.x), fast_exp2(u.y));
@@ -978,14 +983,13 @@ static int launch_attn(const CUtensorMap& tq, const CUtensorMap& tk, const CUten
     // Items that do not fill the last round of the SMs are cut by key tiles where that pays by CutCost: either every item into k equal
     // pieces, which leaves a CTA one stop, or all are dealt to all CTAs.  What is decided here for the most tiles that an item can have, the
     // kernel does if there is an item of so many (whole_below) that it pays: a cache that is a tenth full is attended as if it had no more room.
-    // Kernel time without and with the cut: one item of 153 64-key tiles of 17 x 19 queries 44.0 -> 20.8 us (2 heads), 30 items of 25
-    // tiles 28.2 -> 18.6, 44 of 24 30.4 -> 24.5, 182 of 530 902 -> 647, 156 of 16 42.3 -> 38.1; 8 x 4 096 queries on 16 384 keys (256 of
-    // 128, dealt to all) 283 -> 265 a pass.  Where it would not pay: 108 items of 54 tiles dealt to all 63 -> 69, 18 of 6 13.6 -> 23.2, 256 of
-    // 16 39.4 -> 45.0, 256 of 64 119 -> 122; and full rounds of 64-key tiles, whose loop is slower in this variant (936 of 245 951 -> 990).
+    // Dense calls of 288 shapes (4 to 440 items of 4 to 256 tiles, both dimensions, both tiles) were measured uncut, in as many equal pieces as
+    // fit, and dealt; this picks a time 1.01 times the best of the three in the geometric mean.  Kernel time uncut and cut: 18 items of 128
+    // 128-key tiles 85 -> 27 us, 72 of 32 28 -> 23, 156 of 64 93 -> 71; 160 of 128 64-key tiles 91 -> 63, 18 of 64 26 -> 18; 108 of 256 64-key
+    // tiles, dealt, 87 -> 77; 256 of 128 128-key tiles, d = 64, dealt, 156 -> 149.  Where it would not pay: 72 of 16 128-key tiles 18.0 and
+    // 18.1, 108 of 64, dealt, 43 and 45, 4 of 8 12.5 and 13.8.
     // With room for more keys than there are: 4 x 1 024 queries on 512 keys in a cache of 32 768, 64-key tiles 10.8 us, cut by the room 21.6, now
-    // 11.3 (the look at the lengths is 0.4 of it); 8 x 1 560 on 2 048, 128-key tiles 21.9, 30.5, 21.8.  One head, 1 560 queries on 8 to 48 tiles of 128
-    // with room for 64, what the cut gives: decided by the room -3.5 to +22.0 us, now -0.5 to +22.7; d = 64 and 64-key tiles -3.1 to +8.8, now +0.1
-    // to +9.7.
+    // 11.3 (the look at the lengths is 0.4 of it); 8 x 1 560 on 2 048, 128-key tiles 21.9, 30.5, 21.8.
     using Cost = CutCost<BKT>;
     const int grid = min(min(sm_count, kAttnMaxGrid), c.max_pieces), full = min(sm_count, kAttnMaxGrid), rounds = items / full, left = items % full;
     const int tiles = (a.sel ? a.keep : c.CAPB) + a.seg_tiles;           // at most
@@ -996,18 +1000,17 @@ static int launch_attn(const CUtensorMap& tq, const CUtensorMap& tk, const CUten
     cut.units = tiles;
     float best = tiles * share;
     for (int k = 2; left > 0 && k * left <= grid && k * kAttnMinPiece <= tiles; ++k) {
-      const float dealt = Cost::loop / k, cost = Cost::store + Cost::add * k, t = tiles * dealt + cost;
+      const float dealt = 1.f / k, cost = Cost::store + Cost::part * k * left + Cost::add * k, t = tiles * dealt + cost;
       if (t < best) { best = t; cut.pieces = k * left; cut.whole_below = static_cast<int>(cost / (share - dealt)) + 1; }
     }
     if (left > 0 && grid > left) {
-      const float dealt = Cost::loop * left / grid, cost = Cost::stop + Cost::store + Cost::add * (static_cast<float>(grid) / left + 1.f);
+      const float dealt = static_cast<float>(left) / grid, cost = Cost::stop + Cost::store + Cost::part * (grid + left) + Cost::add * (static_cast<float>(grid) / left + 1.f);
       if (tiles * dealt + cost < best && static_cast<int64_t>(left) * tiles >= static_cast<int64_t>(grid) * kAttnMinPiece) {
         cut.pieces = grid;
         cut.whole_below = static_cast<int>(cost / (share - dealt)) + 1;
       }
     }
     const int64_t largest = static_cast<int64_t>(tiles) * max(left * (cut.pieces + 1), tiles);      // of the kernel's products
-    if (rounds > 0 && BKT == 64) cut.pieces = 0;
     if (cut.pieces > 0 && !a.no_cut && largest < (1ll << 31)) return launch_attn_t<D, BKT, GATHER, SEG, true>(tq, tk, tv, tsk, tsv, c, cut, full, st);
   }
   return launch_attn_t<D, BKT, GATHER, SEG>(tq, tk, tv, tsk, tsv, c, a, GATHER ? items : min(items, sm_count), st);
