@@ -83,14 +83,14 @@ __device__ __forceinline__ float row_max(const Frag& f) {
   }
   return fmax3(fmax3(m[0], m[1], m[2]), fmaxf(m[3], m[4]), __uint_as_float(f.x[HALF][28 + 2 * E + 1]));
 }
-// A thread's new maximum cm (> thr) of one of its rows, and the slot of it: the lowest column, looked for only when the maximum
-// reaches *need (below it the thread's first slot stands in).  row_best: the row's maximum over all threads that share the row,
-// as far as known, in shared memory (-inf or positive); a maximum below it is another thread's to report.
+// The maximum cm of a thread's columns of one of its rows, and the slot of it: the lowest column, looked for only when the maximum
+// reaches *need (below it the thread's first slot stands in).  row_best: the row's maximum over all threads that share the row, as far as
+// known, in shared memory (-inf or positive), `seen` what was read of it; a maximum below it is another thread's to report, an equal one
+// may be the lower slot.
 template <int HALF, int E>
-__device__ __forceinline__ void take_max(const Frag& f, float cm, int jb, const float* need, int* row_best, float& thr, float& best,
-                                         int& best_j) {
-  if (cm > thr) {
-    thr = best = cm;
+__device__ __forceinline__ void take_max(const Frag& f, float cm, int jb, const float* need, int* row_best, float seen, float& best, int& best_j) {
+  if (cm > best && cm >= seen) {
+    best = cm;
     best_j = jb;
     if (cm > 0.f) atomicMax(row_best, __float_as_int(cm));
     if (cm >= *need) {
@@ -106,7 +106,6 @@ __device__ __forceinline__ void take_max(const Frag& f, float cm, int jb, const 
     }
   }
 }
-
 // This CTA's segments.  pre[h] = key tiles of the heads before h.  The line counts a key tile once per row unit: the last unit
 // of a head may hold one A tile only, but a key tile costs it as much (4680 rows: 0.90 against 0.92 us).
 struct SegIter {
@@ -342,7 +341,8 @@ search_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__ 
     const int rq = (warp & 3) * 32 + (lane >> 2);  // this thread's rows: rq, rq + 8, rq + 16, rq + 24
     const uint32_t lane_addr = static_cast<uint32_t>((warp & 3) * 32) << 16;
     bool ok = true;
-    int it = 0, acc = 0;                           // key tiles, accumulators so far (of both groups)
+    int it = 0;                                    // key tiles so far
+    int b = grp, bph = 0;                          // this group's next accumulator, and its barriers' phase
     int* row_s = reinterpret_cast<int*>(smem_raw + SM::row_off);
     if (threadIdx.x < 256) row_s[threadIdx.x] = __float_as_int(-INFINITY);
     named_barrier_sync(1, kEpiWarps * 32);
@@ -356,7 +356,7 @@ search_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__ 
       const Seg sg = seg_s[nseg & 1];
       // The threads of a row share its running maximum, so that one looks for the column of a new maximum only when the row's
       // other columns do not beat it already.  Warps are at most one segment apart: three generations.
-      int* best_s = row_s + slot3 * 256 + grp * 128 + rq;
+      int* best_s = row_s + slot3 * 256 + grp * 128 + ((warp & 3) * 8 + (lane >> 2)) * 4;      // a thread's four rows side by side
       slot3 = slot3 == 2 ? 0 : slot3 + 1;
       if (cg == 0) row_s[slot3 * 256 + grp * 128 + r] = __float_as_int(-INFINITY);
       if (sg.h < 0) {
@@ -387,22 +387,29 @@ search_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__ 
       if (!ok) break;
       skipped = !mine;
       const int ntl = sg.t1 - sg.t0;
+      // accumulators go round by three; the groups take turns, or the first has them all
+      auto advance = [&](int n) {
+        b += n;
+        if (b >= kAccs) { b -= kAccs; bph ^= 1; }
+      };
       if (!mine) {                                 // a unit of one A tile: nothing for the second group
         it += ntl;
-        acc += ntl;
+        const int on = b + ntl;
+        bph ^= (on / kAccs) & 1;
+        b = on % kAccs;
         continue;
       }
       const int row0 = sg.u * 256 + grp * 128 + rq;
       const float* rn_new = c.rnorm_new + static_cast<int64_t>(h) * c.max_tokens;
-      float best[4], thr[4];
+      float best[4];
       int bj[4];
 #pragma unroll
       for (int q = 0; q < 4; ++q) {
-        best[q] = thr[q] = -INFINITY;
+        best[q] = -INFINITY;
         bj[q] = -1;
       }
       // What a score must reach for its slot to matter (it lacks the row's own factor).  In shared memory, because it is read
-      // rarely; the two warps of a row write the same values, each reads its own.
+      // rarely; the two warps of a row write the same values, each reads its own.  Rows past the end have nothing to look for.
       float* need_s = reinterpret_cast<float*>(smem_raw + SM::need_off) + (best_s - row_s);
       if ((lane & 3) == 0)
 #pragma unroll
@@ -412,19 +419,17 @@ search_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__ 
             const float rn = row0 + 8 * q < n ? rn_new[row0 + 8 * q] : 0.f;
             if (rn > 0.f) need = c.search_floor / rn;
           }
-          need_s[8 * q] = need;
+          need_s[q] = need;
+          if (row0 + 8 * q >= n) best_s[q] = __float_as_int(INFINITY);
         }
       __syncwarp();
-      acc += grp;
       for (int t = sg.t0; t < sg.t1; ++t, ++it) {
-        const int b = acc % kAccs, bph = (acc / kAccs) & 1;
-        acc += sg.two ? 2 : 1;
         Frag f;
         ok = mbar_wait_warp(bar_tfull + 8 * b, bph, abort_flag, c.status);
         if (!ok) break;                            // warp-uniform: TMEM loads are warp-collective
         tc_fence_after();
-        // The scores, the factors of this thread's columns and the rows' maxima are asked for together (one after the other they took half
-        // of a tile's time: 8 heads, d = 64, 4 096 new against 16 384 keys 100.1 -> 92.6 us, 12 x 4680, d = 128, 328 -> 320).
+        // The scores and the rows' maxima are asked for together (one after the other they took half of a tile's time: 8 heads, d = 64,
+        // 4 096 new against 16 384 keys 100.1 -> 92.6 us, 12 x 4680, d = 128, 328 -> 320).
         tmem_ld_frag(tmem + lane_addr + b * 128 + cg * 64, f.x[0]);
         tmem_ld_frag(tmem + lane_addr + (16u << 16) + b * 128 + cg * 64, f.x[1]);
         float2 rn[8];
@@ -433,16 +438,12 @@ search_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__ 
 #pragma unroll
           for (int i = 0; i < 8; ++i) rn[i] = rn2[4 * i];
         }
-        // A row's maximum has to exceed this thread's last one and reach the row's (an equal score may be the lower slot): the
-        // float below it, and below -inf the lowest finite one, which only columns past the cache's end do not exceed.
-        int seen[4];
-#pragma unroll
-        for (int q = 0; q < 4; ++q) seen[q] = *static_cast<volatile int*>(best_s + 8 * q);
+        int seen_w[4];
+        asm volatile("ld.volatile.shared.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(seen_w[0]), "=r"(seen_w[1]), "=r"(seen_w[2]), "=r"(seen_w[3]) : "r"(smem_u32(best_s)));
         tmem_wait_ld();
         tc_fence_before();
         mbar_arrive_warp(bar_tempty + 8 * b);      // the scores are in registers: release the accumulator
-#pragma unroll
-        for (int q = 0; q < 4; ++q) thr[q] = fmaxf(thr[q], __int_as_float(seen[q] - 1));
+        advance(sg.two ? 2 : 1);
         if (SCORE == SCORE_COS) {
 #pragma unroll
           for (int i = 0; i < 8; ++i) {
@@ -463,20 +464,20 @@ search_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__ 
                 f.x[hf][4 * (i >> 1) + (i & 1)] = f.x[hf][4 * (i >> 1) + 2 + (i & 1)] = __float_as_uint(-INFINITY);
         }
         const float m0 = row_max<0, 0>(f), m1 = row_max<0, 1>(f), m2 = row_max<1, 0>(f), m3 = row_max<1, 1>(f);
-        if (m0 > thr[0] || m1 > thr[1] || m2 > thr[2] || m3 > thr[3]) {
-          take_max<0, 0>(f, m0, jb, need_s + 0, best_s, thr[0], best[0], bj[0]);
-          take_max<0, 1>(f, m1, jb, need_s + 8, best_s + 8, thr[1], best[1], bj[1]);
-          take_max<1, 0>(f, m2, jb, need_s + 16, best_s + 16, thr[2], best[2], bj[2]);
-          take_max<1, 1>(f, m3, jb, need_s + 24, best_s + 24, thr[3], best[3], bj[3]);
+        const float s0 = __int_as_float(seen_w[0]), s1 = __int_as_float(seen_w[1]), s2 = __int_as_float(seen_w[2]), s3 = __int_as_float(seen_w[3]);
+        if (m0 >= s0 || m1 >= s1 || m2 >= s2 || m3 >= s3) {
+          take_max<0, 0>(f, m0, jb, need_s + 0, best_s + 0, s0, best[0], bj[0]);
+          take_max<0, 1>(f, m1, jb, need_s + 1, best_s + 1, s1, best[1], bj[1]);
+          take_max<1, 0>(f, m2, jb, need_s + 2, best_s + 2, s2, best[2], bj[2]);
+          take_max<1, 1>(f, m3, jb, need_s + 3, best_s + 3, s3, best[3], bj[3]);
         }
       }
       if (!ok) break;
-      if (sg.two) acc -= grp;                      // both groups leave the segment with the same count
       unsigned long long* out = c.best + static_cast<int64_t>(h) * c.max_tokens;
 #pragma unroll
       for (int q = 0; q < 4; ++q) {
         const int row = row0 + 8 * q;
-        if (row >= n || bj[q] < 0 || best[q] < __int_as_float(*static_cast<volatile int*>(best_s + 8 * q))) continue;
+        if (row >= n || bj[q] < 0 || best[q] < __int_as_float(*static_cast<volatile int*>(best_s + q))) continue;
         const float sim = SCORE == SCORE_COS ? best[q] * rn_new[row] : best[q];
         atomicMax(out + row, (static_cast<unsigned long long>(float_to_ordered(sim)) << 32) |
                                  static_cast<unsigned long long>(0xFFFFFFFFu - static_cast<uint32_t>(bj[q])));
