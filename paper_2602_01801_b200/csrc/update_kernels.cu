@@ -130,11 +130,6 @@ __global__ void __launch_bounds__(256, 2) prep_kernel(const __nv_bfloat16* __res
   __shared__ __align__(16) int hist[BLOCKS ? 2 : 1][blocks_a_pass][BLOCKS ? 1024 : 4];      // [pass & 1][block of the pass]
   if (BLOCKS)
     for (int q = threadIdx.x; q < 2 * blocks_a_pass * 1024 / 4; q += 256) reinterpret_cast<int4*>(&hist[0][0][0])[q] = make_int4(0, 0, 0, 0);
-  chain_wait();
-  const int64_t thread = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x, threads = static_cast<int64_t>(gridDim.x) * blockDim.x;
-  for (int64_t q = thread; q < clear.n_best; q += threads) clear.best[q] = 0ull;
-  for (int64_t q = thread; q < clear.n_cnt16; q += threads) clear.cnt[q] = make_uint4(0, 0, 0, 0);
-  for (int64_t q = thread; q < clear.n_heads; q += threads) clear.n_match[q] = 0;
   constexpr int KS = D / 16;
   constexpr int RP = D + 8;                    // padded row of the staged projection matrix (bank-conflict free)
   __shared__ __align__(16) __nv_bfloat16 r_s[32 * RP];
@@ -148,19 +143,6 @@ __global__ void __launch_bounds__(256, 2) prep_kernel(const __nv_bfloat16* __res
     if (col < ncol) v = *reinterpret_cast<const uint4*>(lsh + col * D + ch * 8);
     *reinterpret_cast<uint4*>(r_s + col * RP + ch * 8) = v;
   }
-  __syncthreads();
-  uint32_t bf[KS][4][2];
-#pragma unroll
-  for (int ks = 0; ks < KS; ++ks)
-#pragma unroll
-    for (int nt = 0; nt < 4; ++nt) {
-      // The contraction index may be permuted freely as long as A and B agree: lane t of a quad reads 8
-      // contiguous elements (one 128-bit load) per 32-wide k block, k = 32*(ks/2) + 8t + 4*(ks%2) + {0,1 | 2,3}.
-      const int col = 8 * nt + g;
-      const __nv_bfloat16* rp = r_s + col * RP + 32 * (ks >> 1) + 8 * t + 4 * (ks & 1);
-      bf[ks][nt][0] = *reinterpret_cast<const uint32_t*>(rp);
-      bf[ks][nt][1] = *reinterpret_cast<const uint32_t*>(rp + 2);
-    }
   // 16-row groups of all heads, dealt to the warps of a grid that fills the SMs once, eight to a CTA's pass
   // BLOCKS: groups are numbered through whole blocks, so that a pass has one block of 128 rows or two of 64.  The histograms of two passes
   // take turns: a thread that has written its columns of one clears them at once, and by the barrier of the next pass they are free.
@@ -180,11 +162,29 @@ __global__ void __launch_bounds__(256, 2) prep_kernel(const __nv_bfloat16* __res
     vb[kk] = *reinterpret_cast<const uint4*>(xb + 32 * kk);
   };
   const int first = blockIdx.x * 8 + warp;
+  chain_wait();                                // (the projection matrix is written when the cache is created)
   if (first < total_groups) {
     rows(first);
 #pragma unroll
     for (int kk = 0; kk < KS / 2; ++kk) fetch(kk);
   }
+  const int64_t thread = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x, threads = static_cast<int64_t>(gridDim.x) * blockDim.x;
+  for (int64_t q = thread; q < clear.n_best; q += threads) clear.best[q] = 0ull;
+  for (int64_t q = thread; q < clear.n_cnt16; q += threads) clear.cnt[q] = make_uint4(0, 0, 0, 0);
+  for (int64_t q = thread; q < clear.n_heads; q += threads) clear.n_match[q] = 0;
+  __syncthreads();
+  uint32_t bf[KS][4][2];
+#pragma unroll
+  for (int ks = 0; ks < KS; ++ks)
+#pragma unroll
+    for (int nt = 0; nt < 4; ++nt) {
+      // The contraction index may be permuted freely as long as A and B agree: lane t of a quad reads 8
+      // contiguous elements (one 128-bit load) per 32-wide k block, k = 32*(ks/2) + 8t + 4*(ks%2) + {0,1 | 2,3}.
+      const int col = 8 * nt + g;
+      const __nv_bfloat16* rp = r_s + col * RP + 32 * (ks >> 1) + 8 * t + 4 * (ks & 1);
+      bf[ks][nt][0] = *reinterpret_cast<const uint32_t*>(rp);
+      bf[ks][nt][1] = *reinterpret_cast<const uint32_t*>(rp + 2);
+    }
   int buffer = 0;
   for (int grp = first; BLOCKS ? grp - warp < total_groups : grp < total_groups; grp += stride) {
     const int h = grp / groups_per_head;
