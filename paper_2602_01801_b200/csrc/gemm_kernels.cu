@@ -25,7 +25,10 @@ constexpr int kTmemCols = 2 * kTileN;
 constexpr int kGemmThreads = 320;            // warps 0-7 epilogue, 8 TMA producer, 9 MMA issue
 constexpr int kGemmProducerWarp = 8, kGemmMmaWarp = 9;
 
-constexpr int NST = 4;                       // ring stages of a chunk of both operands
+// Ring stages of a chunk of both operands.  A CTA's sixteen chunks are a chain of loads, so a grid of one CTA per SM at most takes all the
+// shared memory for its ring: two round trips to L2 instead of four.  A larger grid has two CTAs per SM, each with half of the loads under way.
+constexpr int kFewStages = 4, kManyStages = 9;
+template <int NST>
 struct GemmSmem {
   static constexpr int stage_bytes = kChunkBytes + kTileN * 128;
   static constexpr int bar_off = NST * stage_bytes;
@@ -34,11 +37,11 @@ struct GemmSmem {
 
 // RANK: a head's key blocks fit one tile and its query blocks are few, so the CTA has whole rows and ranks them too (a launch less: 2 heads,
 // 5 x 10 blocks 6.4 + 2.5 -> 7.8 us).
-template <bool RANK>
+template <bool RANK, int NST>
 __global__ void __launch_bounds__(kGemmThreads, 2)
 gemm_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__ CUtensorMap tm_b, const CacheView c,
             const GemmArgs g) {
-  using SM = GemmSmem;
+  using SM = GemmSmem<NST>;
   extern __shared__ __align__(1024) uint8_t smem_raw[];
   const uint32_t sbase = smem_u32(smem_raw);
   uint8_t* sgen = smem_raw;
@@ -194,13 +197,20 @@ gemm_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__ CU
     for (int row = warp; row < g.rows_a; row += kGemmThreads / 32) topk_row<false, kTileN / 32>(g.top, h, row);
 }
 
+template <bool RANK, int NST>
+static int launch_gemm_t(const CacheView& c, const CUtensorMap& tm_hq, const CUtensorMap& tm_hk, const GemmArgs& g, dim3 grid, cudaStream_t st) {
+  const int cfg = ensure_dynamic_smem(reinterpret_cast<const void*>(gemm_kernel<RANK, NST>), GemmSmem<NST>::total);
+  if (cfg != FASTAR_OK) return cfg;
+  launch_chained(gemm_kernel<RANK, NST>, grid, kGemmThreads, GemmSmem<NST>::total, st, tm_hq, tm_hk, c, g);
+  return cudaGetLastError() == cudaSuccess ? 1 : FASTAR_ERR_CUDA;
+}
 template <bool RANK>
 static int launch_gemm(const CacheView& c, const CUtensorMap& tm_hq, const CUtensorMap& tm_hk, const GemmArgs& g, cudaStream_t st) {
-  const int cfg = ensure_dynamic_smem(reinterpret_cast<const void*>(gemm_kernel<RANK>), GemmSmem::total);
-  if (cfg != FASTAR_OK) return cfg;
-  const int col_tiles = (c.CAPB + kTileN - 1) / kTileN;
-  launch_chained(gemm_kernel<RANK>, dim3((g.rows_a + 127) / 128, c.H, col_tiles), kGemmThreads, GemmSmem::total, st, tm_hq, tm_hk, c, g);
-  return cudaGetLastError() == cudaSuccess ? 1 : FASTAR_ERR_CUDA;
+  int dev = 0, sm_count = 148;
+  if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sm_count, cudaDevAttrMultiProcessorCount, dev);
+  const dim3 grid((g.rows_a + 127) / 128, c.H, (c.CAPB + kTileN - 1) / kTileN);
+  if (static_cast<int64_t>(grid.x) * grid.y * grid.z <= sm_count) return launch_gemm_t<RANK, kManyStages>(c, tm_hq, tm_hk, g, grid, st);
+  return launch_gemm_t<RANK, kFewStages>(c, tm_hq, tm_hk, g, grid, st);
 }
 
 int launch_s3_scores(const CacheView& c, const CUtensorMap& tm_hq, const CUtensorMap& tm_hk, int nqb, cudaStream_t st) {

@@ -55,3 +55,27 @@ def test_prompt_topk(prompt, keep):
             want = (q[h, 17 * f: 17 * f + 17] @ kp[h].T).max(0)
             assert np.array_equal(np.rint(r["rel"][h, f].cpu().numpy() * 8.0), want)
             assert np.array_equal(r["sel"][h, f].cpu().numpy(), _kept(want, keep))
+
+
+@pytest.mark.parametrize("H,capacity,nq", [(1, 128, 1), (29, 16640, 130), (40, 16640, 130)])
+def test_block_scores_of_few_and_many_heads(H, capacity, nq):
+    """The grid of the block scores on both sides of one CTA per SM (1, 145 and 200 CTAs): same-bucket pairs counted from the codes."""
+    import torch
+    from paper_2602_01801_b200 import fastar
+    rng = np.random.default_rng(H)
+    d, pt, length = 64, 64, capacity - 7
+    cache = fastar.Cache(H, d, capacity, pt, rng.standard_normal((32, d)).astype(np.float32), max_tokens=nq)
+    k = synth.round_bf16(rng.standard_normal((H, length, d)).astype(np.float32))
+    cache.import_state(fastar.bf16_bits(k), fastar.bf16_bits(k), np.full(H, length))
+    r = cache.annsa(fastar.to_device(synth.round_bf16(rng.standard_normal((H, nq, d)).astype(np.float32))), 128, 1, debug=True)
+    assert cache.status() == 0
+    kc = torch.from_numpy(cache.export_state(kv=False)["code"][:, :length].astype(np.int64)).cuda()
+    qc = r["qcode"].long() & 0xFFFFFFFF
+
+    def histograms(code, block):
+        n = -(-code.shape[1] // block)
+        at = (torch.arange(code.shape[1], device="cuda") // block * 1024)[None, :, None] + 256 * torch.arange(4, device="cuda") + (code[..., None] >> (8 * torch.arange(4, device="cuda")) & 255)
+        out = torch.zeros(H, n * 1024, device="cuda", dtype=torch.float64)
+        return out.scatter_add_(1, at.reshape(H, -1), torch.ones_like(at.reshape(H, -1), dtype=torch.float64)).reshape(H, n, 1024)
+    hk = histograms(kc, pt)
+    assert torch.equal(r["scores"][:, :, : hk.shape[1]].double(), histograms(qc, 128) @ hk.mT)
