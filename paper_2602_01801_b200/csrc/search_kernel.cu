@@ -20,7 +20,11 @@
 // Measured (B200, kernel time, before = CTAs of 128 rows or CTA pairs with both operands in shared memory): 12 heads, d = 128,
 // 4 680 new against 28 080 cached keys 370 -> 308 us (0.80 of the measured bf16 peak); 40 heads, 10 800 against 64 800: 5.78 ->
 // 5.29 ms (1.36 PFLOP/s: the power limit holds the clock at 1.55 GHz there); 8 heads, d = 64, 4 096 against 16 384: 138 ->
-// 103 us.  A key tile takes an SM 1 380-1 460 cycles, its 16 MMAs 1 025.
+// 103 us.  A key tile takes an SM 1 380-1 460 cycles, its 16 MMAs 1 025.  Since then: asking for scores, factors and maxima together 328 -> 303
+// and 100 -> 93; the rows' maxima side by side 303 -> 293 and 93.4 -> 91.4; no slots for maxima that no match can come of 292 -> 293 and
+// 91.9 -> 89.1, by the query probe (12 x 1560 on 14 040) 64.4 -> 62.8.  What was slower: working out scores only where a row's largest dot
+// product times the largest factor of the columns reaches its maximum (308 and 106: some row of a warp's 32 does in most tiles), a tile's halves
+// taking turns in the registers, loads a half ahead (322 and 103), asking for the next accumulator's barrier early (1 to 3 %).
 #include "common.h"
 #include "ptx.cuh"
 
@@ -60,8 +64,7 @@ struct Cfg {
   static constexpr int pre_off = rn_off + (SCORE == SCORE_COS ? factors * 512 : 0);
   static constexpr int len_off = pre_off + (kMaxHeads + 8) * 4;    // live slots of the heads
   static constexpr int row_off = len_off + kMaxHeads * 4;    // [3][256] running row maxima of the last segments
-  static constexpr int need_off = row_off + 3 * 256 * 4;           // [3][256] what their maxima must reach
-  static constexpr int seg_off = need_off + 3 * 256 * 4;           // [2] Seg
+  static constexpr int seg_off = row_off + 3 * 256 * 4;            // [2] Seg
   static constexpr int bar_off = seg_off + 64;
   static constexpr int total = bar_off + 512;
 };
@@ -83,29 +86,25 @@ __device__ __forceinline__ float row_max(const Frag& f) {
   }
   return fmax3(fmax3(m[0], m[1], m[2]), fmaxf(m[3], m[4]), __uint_as_float(f.x[HALF][28 + 2 * E + 1]));
 }
-// The maximum cm of a thread's columns of one of its rows, and the slot of it: the lowest column, looked for only when the maximum
-// reaches *need (below it the thread's first slot stands in).  row_best: the row's maximum over all threads that share the row, as far as
-// known, in shared memory (-inf or positive), `seen` what was read of it; a maximum below it is another thread's to report, an equal one
-// may be the lower slot.
+// The maximum cm of a thread's columns of one of its rows reaches what the row asks for: the slot of it is looked for, the lowest column.
+// row_best: what a slot has to reach to matter, or the row's maximum over all threads that share it if that is more, in shared memory (-inf or
+// positive), `seen` what was read of it; a maximum below it is another thread's to report, an equal one may be the lower slot.
 template <int HALF, int E>
-__device__ __forceinline__ void take_max(const Frag& f, float cm, int jb, const float* need, int* row_best, float seen, float& best, int& best_j) {
+__device__ __forceinline__ void take_max(const Frag& f, float cm, int jb, int* row_best, float seen, float best, int& best_j) {
   if (cm > best && cm >= seen) {
-    best = cm;
-    best_j = jb;
     if (cm > 0.f) atomicMax(row_best, __float_as_int(cm));
-    if (cm >= *need) {
-      int idx[4];                                    // four short chains, the lowest columns in idx[0]
+    int idx[4];                                      // four short chains, the lowest columns in idx[0]
 #pragma unroll
-      for (int k = 0; k < 4; ++k) {
-        idx[k] = 64;
+    for (int k = 0; k < 4; ++k) {
+      idx[k] = 64;
 #pragma unroll
-        for (int q = 4 * k + 3; q >= 4 * k; --q)
-          idx[k] = (__uint_as_float(f.x[HALF][4 * (q >> 1) + 2 * E + (q & 1)]) == cm) ? 8 * (q >> 1) + (q & 1) : idx[k];
-      }
-      best_j = jb + min(min(idx[0], idx[1]), min(idx[2], idx[3]));
+      for (int q = 4 * k + 3; q >= 4 * k; --q)
+        idx[k] = (__uint_as_float(f.x[HALF][4 * (q >> 1) + 2 * E + (q & 1)]) == cm) ? 8 * (q >> 1) + (q & 1) : idx[k];
     }
+    best_j = jb + min(min(idx[0], idx[1]), min(idx[2], idx[3]));
   }
 }
+
 // This CTA's segments.  pre[h] = key tiles of the heads before h.  The line counts a key tile once per row unit: the last unit
 // of a head may hold one A tile only, but a key tile costs it as much (4680 rows: 0.90 against 0.92 us).
 struct SegIter {
@@ -408,19 +407,19 @@ search_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__ 
         best[q] = -INFINITY;
         bj[q] = -1;
       }
-      // What a score must reach for its slot to matter (it lacks the row's own factor).  In shared memory, because it is read
-      // rarely; the two warps of a row write the same values, each reads its own.  Rows past the end have nothing to look for.
-      float* need_s = reinterpret_cast<float*>(smem_raw + SM::need_off) + (best_s - row_s);
+      // What a score must reach for its slot to matter (it lacks the row's own factor): the row's maximum starts there, so that a score that
+      // finds no match, which most do, is a maximum in a register and nothing else.  Rows past the end have nothing to look for.
+      float rn_row[4];                             // (fetched again when the segment is through)
+      auto needed = [&](int q) {
+        rn_row[q] = SCORE == SCORE_COS && row0 + 8 * q < n ? rn_new[row0 + 8 * q] : 1.f;
+        const float need = SCORE == SCORE_COS && rn_row[q] > 0.f ? c.search_floor / rn_row[q] : -INFINITY;
+        return row0 + 8 * q >= n ? INFINITY : need > 0.f ? need : -INFINITY;
+      };
       if ((lane & 3) == 0)
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
-          float need = -INFINITY;
-          if (SCORE == SCORE_COS) {
-            const float rn = row0 + 8 * q < n ? rn_new[row0 + 8 * q] : 0.f;
-            if (rn > 0.f) need = c.search_floor / rn;
-          }
-          need_s[q] = need;
-          if (row0 + 8 * q >= n) best_s[q] = __float_as_int(INFINITY);
+          const float need = needed(q);
+          if (need > 0.f) atomicMax(best_s + q, __float_as_int(need));
         }
       __syncwarp();
       for (int t = sg.t0; t < sg.t1; ++t, ++it) {
@@ -466,21 +465,30 @@ search_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__ 
         const float m0 = row_max<0, 0>(f), m1 = row_max<0, 1>(f), m2 = row_max<1, 0>(f), m3 = row_max<1, 1>(f);
         const float s0 = __int_as_float(seen_w[0]), s1 = __int_as_float(seen_w[1]), s2 = __int_as_float(seen_w[2]), s3 = __int_as_float(seen_w[3]);
         if (m0 >= s0 || m1 >= s1 || m2 >= s2 || m3 >= s3) {
-          take_max<0, 0>(f, m0, jb, need_s + 0, best_s + 0, s0, best[0], bj[0]);
-          take_max<0, 1>(f, m1, jb, need_s + 1, best_s + 1, s1, best[1], bj[1]);
-          take_max<1, 0>(f, m2, jb, need_s + 2, best_s + 2, s2, best[2], bj[2]);
-          take_max<1, 1>(f, m3, jb, need_s + 3, best_s + 3, s3, best[3], bj[3]);
+          take_max<0, 0>(f, m0, jb, best_s + 0, s0, best[0], bj[0]);
+          take_max<0, 1>(f, m1, jb, best_s + 1, s1, best[1], bj[1]);
+          take_max<1, 0>(f, m2, jb, best_s + 2, s2, best[2], bj[2]);
+          take_max<1, 1>(f, m3, jb, best_s + 3, s3, best[3], bj[3]);
         }
+        best[0] = fmaxf(best[0], m0);
+        best[1] = fmaxf(best[1], m1);
+        best[2] = fmaxf(best[2], m2);
+        best[3] = fmaxf(best[3], m3);
       }
       if (!ok) break;
+      // A row that has found nothing has its maximum reported by one thread of a quad, with the segment's first slot in its slot's place.
       unsigned long long* out = c.best + static_cast<int64_t>(h) * c.max_tokens;
 #pragma unroll
       for (int q = 0; q < 4; ++q) {
         const int row = row0 + 8 * q;
-        if (row >= n || bj[q] < 0 || best[q] < __int_as_float(*static_cast<volatile int*>(best_s + q))) continue;
-        const float sim = SCORE == SCORE_COS ? best[q] * rn_new[row] : best[q];
+        const float need = needed(q), row_top = __int_as_float(*static_cast<volatile int*>(best_s + q));
+        float top = fmaxf(best[q], __shfl_xor_sync(0xffffffffu, best[q], 1));
+        top = fmaxf(top, __shfl_xor_sync(0xffffffffu, top, 2));
+        const bool found = bj[q] >= 0 && best[q] >= row_top, none = need > 0.f && row_top == need && (lane & 3) == 0 && top > -INFINITY && top < need;
+        if (row >= n || !(found || none)) continue;
+        const float score = found ? best[q] : top, sim = SCORE == SCORE_COS ? score * rn_row[q] : score;
         atomicMax(out + row, (static_cast<unsigned long long>(float_to_ordered(sim)) << 32) |
-                                 static_cast<unsigned long long>(0xFFFFFFFFu - static_cast<uint32_t>(bj[q])));
+                                 static_cast<unsigned long long>(0xFFFFFFFFu - static_cast<uint32_t>(found ? bj[q] : sg.t0 * 128)));
       }
     }
   }
