@@ -238,7 +238,9 @@ struct ConvertArgs {
   int count;
 };
 int launch_convert_f32_to_bf16(const ConvertArgs& a, int H, int D, cudaStream_t st);
-int launch_query_blocks(const CacheView& c, const __nv_bfloat16* q, int nq, int64_t hs, int64_t ts, int block_q, cudaStream_t st);
+// conv (where a call's tensors are fp32): the rows' source, t[0], and more tensors to convert on the way
+int launch_query_blocks(const CacheView& c, const __nv_bfloat16* q, int nq, int64_t hs, int64_t ts, int block_q, cudaStream_t st,
+                        const ConvertArgs& conv = ConvertArgs{});
 struct UpdateScratch {               // what the first kernel of an update clears; a part that is not used is null and empty
   unsigned long long* best;
   int64_t n_best;                    // words
@@ -248,7 +250,7 @@ struct UpdateScratch {               // what the first kernel of an update clear
   int32_t n_heads;
 };
 UpdateScratch update_scratch(const CacheView& c, int n);
-int launch_prep_update(const CacheView& c, const __nv_bfloat16* k_new, int n, int64_t hs, int64_t ts, cudaStream_t st);
+int launch_prep_update(const CacheView& c, const __nv_bfloat16* k_new, int n, int64_t hs, int64_t ts, cudaStream_t st, const ConvertArgs& conv = ConvertArgs{});
 int launch_prep_codes_strided(const CacheView& c, const __nv_bfloat16* x, int n, int64_t hs, int64_t ts, uint32_t* code_out,
                               int64_t out_stride, cudaStream_t st);
 int launch_bucket_select(const CacheView& c, int nq, int frame_len, int n_frames, int np, cudaStream_t st);

@@ -344,22 +344,26 @@ bool rows_aligned(const fastar_cache* c, const void* p, int64_t hs, int64_t ts) 
   const int64_t esz = c->desc.dtype == FASTAR_FP32 ? 4 : 2;
   return !(reinterpret_cast<uintptr_t>(p) & 15) && !((hs * esz) & 15) && !((ts * esz) & 15);
 }
-int as_bf16(fastar_cache* c, const CacheView& cv, View* v, int count, cudaStream_t st) {
+// The views of tensors that a conversion (a) will have written; nothing is launched.
+int staged(fastar_cache* c, const CacheView& cv, View* v, int count, ConvertArgs& a) {
   for (int i = 0; i < count; ++i) {
     if (!rows_aligned(c, v[i].src, v[i].hs, v[i].ts)) return FASTAR_ERR_INVALID_ARG;
     v[i].p = static_cast<const __nv_bfloat16*>(v[i].src);
   }
   if (c->desc.dtype == FASTAR_BF16) return FASTAR_OK;
-  ConvertArgs a{};
-  a.count = count;
   for (int i = 0; i < count; ++i) {
-    a.t[i] = {static_cast<const float*>(v[i].src), cv.stage[v[i].slot], v[i].hs, v[i].ts, v[i].rows};
+    a.t[a.count++] = {static_cast<const float*>(v[i].src), cv.stage[v[i].slot], v[i].hs, v[i].ts, v[i].rows};
     v[i].p = cv.stage[v[i].slot];
     v[i].hs = static_cast<int64_t>(v[i].rows) * cv.D;
     v[i].ts = cv.D;
   }
-  ACCK(FASTAR_K_CONVERT, launch_convert_f32_to_bf16(a, cv.H, cv.D, st));
   return FASTAR_OK;
+}
+int as_bf16(fastar_cache* c, const CacheView& cv, View* v, int count, cudaStream_t st) {
+  ConvertArgs a{};
+  const int r = staged(c, cv, v, count, a);
+  if (r == FASTAR_OK && a.count > 0) ACCK(FASTAR_K_CONVERT, launch_convert_f32_to_bf16(a, cv.H, cv.D, st));
+  return r;
 }
 
 }  // namespace
@@ -607,9 +611,11 @@ static int update_impl(fastar_cache_t* c, const HeadRange& range, UpdatePart par
   // keys and values together (one stride for both); in parts, the search converts keys and probe and the commit the values
   View in[3] = {{k_new, n, 0, head_stride, token_stride, nullptr}, {v_new, n, 1, head_stride, token_stride, nullptr}, {q_probe, n, 2, head_stride, token_stride, nullptr}};
   int r;
-  if (part == kWhole) r = as_bf16(c, v, in, q_probe ? 3 : 2, st);
-  else r = as_bf16(c, v, part == kSearch ? in : in + 1, 1, st);
-  if (r == FASTAR_OK && part == kSearch && q_probe) r = as_bf16(c, v, in + 2, 1, st);
+  ConvertArgs conv{};                        // by the hash of the keys, on its way
+  if (part == kWhole) r = staged(c, v, in, q_probe ? 3 : 2, conv);
+  else if (part == kSearch) r = staged(c, v, in, 1, conv);
+  else r = as_bf16(c, v, in + 1, 1, st);
+  if (r == FASTAR_OK && part == kSearch && q_probe) r = staged(c, v, in + 2, 1, conv);
   if (r != FASTAR_OK) return r;
   if (part == kCommit || part == kCommitKeep) {              // the keys were converted by the search
     in[0].p = c->desc.dtype == FASTAR_BF16 ? static_cast<const __nv_bfloat16*>(k_new) : v.stage[0];
@@ -627,7 +633,7 @@ static int update_impl(fastar_cache_t* c, const HeadRange& range, UpdatePart par
   r = q_probe ? make_map(c, &tm_a, pb, v.D, n, v.H, static_cast<uint64_t>(pts) * 2, static_cast<uint64_t>(phs) * 2, 128)
               : make_map(c, &tm_a, kb, v.D, n, v.H, static_cast<uint64_t>(kts) * 2, static_cast<uint64_t>(khs) * 2, 128);
   if (r != FASTAR_OK) return r;
-  ACCK(FASTAR_K_HASH, launch_prep_update(v, kb, n, khs, kts, st));
+  ACCK(FASTAR_K_HASH, launch_prep_update(v, kb, n, khs, kts, st, conv));
   // A row whose best similarity stays below the threshold is appended whatever its best slot is: the search kernels
   // skip the column search for running maxima below tau minus a margin that covers their rounding (the similarity
   // itself is always exact).  Rankings that a cosine pass follows need the slot in every case.
@@ -789,18 +795,12 @@ static int annsa_impl(fastar_cache_t* c, const HeadRange& range, bool hashed, bo
 static int prepare_impl(fastar_cache_t* c, const HeadRange& range, const void* q, int32_t nq, int64_t head_stride, int64_t token_stride,
                         int32_t block_q, cudaStream_t st) {
   const CacheView& v = range.v;
-  const __nv_bfloat16* qb = static_cast<const __nv_bfloat16*>(q);
-  int64_t qhs = head_stride, qts = token_stride;
+  ConvertArgs conv{};
   if (c->desc.dtype == FASTAR_FP32) {          // own staging buffer: an update or another attention call may be converting too
-    ConvertArgs a{};
-    a.count = 1;
-    a.t[0] = {static_cast<const float*>(q), v.stage_prep, qhs, qts, nq};
-    ACCK(FASTAR_K_CONVERT, launch_convert_f32_to_bf16(a, v.H, v.D, st));
-    qb = v.stage_prep;
-    qhs = static_cast<int64_t>(nq) * v.D;
-    qts = v.D;
+    conv.count = 1;
+    conv.t[0] = {static_cast<const float*>(q), v.stage_prep, head_stride, token_stride, nq};
   }
-  ACCK(FASTAR_K_HASH, launch_query_blocks(v, qb, nq, qhs, qts, block_q, st));
+  ACCK(FASTAR_K_HASH, launch_query_blocks(v, static_cast<const __nv_bfloat16*>(q), nq, head_stride, token_stride, block_q, st, conv));
   return FASTAR_OK;
 }
 

@@ -9,6 +9,8 @@
 #include "bound.cuh"
 #include "topk.cuh"
 
+#include <type_traits>
+
 namespace fastar {
 
 // ---------------------------------------------------------------------------------------------
@@ -65,13 +67,9 @@ __device__ __forceinline__ void bitonic_sort_smem(unsigned long long* keys, int 
 // fp32 -> bf16 entry conversion (strided sources, contiguous destinations): up to three tensors of a call in one launch, one per
 // blockIdx.z (a small call is a chain of launches; one per tensor made six of a step's 21).
 // ---------------------------------------------------------------------------------------------
-__global__ void convert_kernel(const ConvertArgs a, int D) {
-  chain_wait();
-  const ConvertArgs::Tensor& x = a.t[blockIdx.z];
-  const int h = blockIdx.y;
+__device__ __forceinline__ void convert_rows(const ConvertArgs::Tensor& x, int h, int D, int64_t thread, int64_t threads) {
   const int64_t per_head = static_cast<int64_t>(x.n) * D / 4;
-  for (int64_t q = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; q < per_head;
-       q += static_cast<int64_t>(gridDim.x) * blockDim.x) {
+  for (int64_t q = thread; q < per_head; q += threads) {
     const int64_t e = q * 4;
     const int row = static_cast<int>(e / D), col = static_cast<int>(e % D);
     const float4 v = *reinterpret_cast<const float4*>(x.src + h * x.hs + row * x.ts + col);
@@ -80,6 +78,10 @@ __global__ void convert_kernel(const ConvertArgs a, int D) {
     o.y = pack_bf16x2(v.z, v.w);
     *reinterpret_cast<uint2*>(x.dst + (static_cast<int64_t>(h) * x.n + row) * D + col) = o;
   }
+}
+__global__ void convert_kernel(const ConvertArgs a, int D) {
+  chain_wait();
+  convert_rows(a.t[blockIdx.z], blockIdx.y, D, blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x, static_cast<int64_t>(gridDim.x) * blockDim.x);
 }
 int launch_convert_f32_to_bf16(const ConvertArgs& a, int H, int D, cudaStream_t st) {
   int64_t want = 0;
@@ -116,15 +118,17 @@ __device__ __forceinline__ uint4 pack_counts(const int (&v)[8]) {
 // ROWS > 0 (the query side of S2 in the same launch: 12 x 4680 rows 9.2 + 2.7 -> 10.2 us, 2 x 600 4.1 + 2.3 -> 4.4): blocks of 64 or 128 rows,
 // whose bucket histograms the CTA writes.  With four of eight warps idle for blocks of 64, 40 x 10800 rows took 45 us, with two blocks a pass 37
 // (d = 64 29 -> 22); with a launch of their own for the histograms 33 (26).  Blocks of 128: 34 (21) us, 31 (24) with that launch.
+// F32: the rows are fp32 (conv.t[0]); the kernel rounds them on their way, writes them where the kernels behind it read them, and converts
+// conv's other tensors too (an update's values): one head x 256 rows, d = 64, 2.2 + 3.4 -> 4.9 us and a launch less for the host.
 struct BlockHist {
   __nv_bfloat16* hist;         // [H][max_qb][hist_cols]
   int max_qb, hist_cols;
 };
-template <int D, int ROWS>
+template <int D, int ROWS, bool F32>
 __global__ void __launch_bounds__(256, 2) prep_kernel(const __nv_bfloat16* __restrict__ x, int H, int n, int64_t hs, int64_t ts,
                                                    const __nv_bfloat16* __restrict__ lsh, int T, int B,
                                                    uint32_t* __restrict__ code_out, float* __restrict__ rnorm_out,
-                                                   int64_t out_stride, HeadBound* bound, UpdateScratch clear, BlockHist bh) {
+                                                   int64_t out_stride, HeadBound* bound, UpdateScratch clear, BlockHist bh, const ConvertArgs conv) {
   constexpr bool BLOCKS = ROWS > 0;
   constexpr int per_block = BLOCKS ? ROWS / 16 : 1, blocks_a_pass = BLOCKS ? 8 / per_block : 1;
   __shared__ __align__(16) int hist[BLOCKS ? 2 : 1][blocks_a_pass][BLOCKS ? 1024 : 4];      // [pass & 1][block of the pass]
@@ -150,16 +154,38 @@ __global__ void __launch_bounds__(256, 2) prep_kernel(const __nv_bfloat16* __res
   const int total_groups = groups_per_head * H;
   const int stride = static_cast<int>(gridDim.x) * 8;
   uint4 va[KS / 2], vb[KS / 2];
-  const __nv_bfloat16 *xa = x, *xb = x;                                // this lane's rows of the group that is fetched
+  using Source = std::conditional_t<F32, float, __nv_bfloat16>;
+  const Source* src;
+  if constexpr (F32) src = conv.t[0].src;
+  else src = x;
+  const Source *xa = src, *xb = src;                                   // this lane's rows of the group that is fetched
+  __nv_bfloat16 *oa = nullptr, *ob = nullptr;                          // F32: and where they go
   auto rows = [&](int grp) {
     const int h = grp / groups_per_head;
     const int r0 = (grp - h * groups_per_head) * 16;
-    xa = x + h * hs + min(r0 + g, n - 1) * ts + 8 * t;                  // rows past the end repeat the last one
-    xb = x + h * hs + min(r0 + g + 8, n - 1) * ts + 8 * t;
+    const int ra = min(r0 + g, n - 1), rb = min(r0 + g + 8, n - 1);    // rows past the end repeat the last one
+    const int64_t head = F32 ? conv.t[0].hs : hs, row = F32 ? conv.t[0].ts : ts;
+    xa = src + h * head + ra * row + 8 * t;
+    xb = src + h * head + rb * row + 8 * t;
+    if constexpr (F32) {
+      oa = conv.t[0].dst + (static_cast<int64_t>(h) * n + ra) * D + 8 * t;
+      ob = conv.t[0].dst + (static_cast<int64_t>(h) * n + rb) * D + 8 * t;
+    }
   };
-  auto fetch = [&](int kk) {                                           // one 128-bit load per row and 32-wide k block
-    va[kk] = *reinterpret_cast<const uint4*>(xa + 32 * kk);
-    vb[kk] = *reinterpret_cast<const uint4*>(xb + 32 * kk);
+  auto fetch = [&](int kk) {                                           // one 128-bit load per row and 32-wide k block, F32: two
+    if constexpr (F32) {
+      auto round8 = [](const float* p) {
+        const float4 u = *reinterpret_cast<const float4*>(p), v = *reinterpret_cast<const float4*>(p + 4);
+        return make_uint4(pack_bf16x2(u.x, u.y), pack_bf16x2(u.z, u.w), pack_bf16x2(v.x, v.y), pack_bf16x2(v.z, v.w));
+      };
+      va[kk] = round8(xa + 32 * kk);
+      vb[kk] = round8(xb + 32 * kk);
+      *reinterpret_cast<uint4*>(oa + 32 * kk) = va[kk];
+      *reinterpret_cast<uint4*>(ob + 32 * kk) = vb[kk];
+    } else {
+      va[kk] = *reinterpret_cast<const uint4*>(xa + 32 * kk);
+      vb[kk] = *reinterpret_cast<const uint4*>(xb + 32 * kk);
+    }
   };
   const int first = blockIdx.x * 8 + warp;
   chain_wait();                                // (the projection matrix is written when the cache is created)
@@ -272,31 +298,47 @@ __global__ void __launch_bounds__(256, 2) prep_kernel(const __nv_bfloat16* __res
       buffer ^= 1;
     }
   }
+  if constexpr (F32) {
+    if (conv.count > 1)
+      for (int h = 0; h < H; ++h) convert_rows(conv.t[1], h, D, thread, threads);
+    if (conv.count > 2)
+      for (int h = 0; h < H; ++h) convert_rows(conv.t[2], h, D, thread, threads);
+  }
 }
 static int launch_prep_generic(const CacheView& c, const __nv_bfloat16* x, int n, int64_t hs, int64_t ts, uint32_t* code_out,
-                               float* rnorm_out, int64_t out_stride, cudaStream_t st, const UpdateScratch& clear = UpdateScratch{}) {
+                               float* rnorm_out, int64_t out_stride, cudaStream_t st, const UpdateScratch& clear = UpdateScratch{},
+                               const ConvertArgs& conv = ConvertArgs{}) {
   if (n <= 0) return 0;
   HeadBound* bound = rnorm_out ? c.bound : nullptr;               // cached keys, or keys that will be
   const int groups = ((n + 15) / 16) * c.H;                      // 16 rows per warp pass
   // CTAs for the rows (eight warps of 16 a pass) or for the zeros (32 KB each), whichever needs more: a few tokens against many heads
   // with long caches leave far more to clear than to hash (40 heads x 65536 slots, 1 to 16 tokens: an update of 81 us with CTAs for
   // the rows only, 50 with these).
-  const int64_t want = max(static_cast<int64_t>(groups + 7) / 8, (clear.n_best / 2 + clear.n_cnt16 + 2047) / 2048);
+  int64_t want = max(static_cast<int64_t>(groups + 7) / 8, (clear.n_best / 2 + clear.n_cnt16 + 2047) / 2048);
+  if (conv.count > 1) want = max(want, static_cast<int64_t>(conv.count - 1) * c.H * n * c.D / 4 / 256);      // four numbers a thread
   const dim3 grid(static_cast<unsigned>(max(static_cast<int64_t>(1), min(want, static_cast<int64_t>(2 * 148)))));
-  if (c.D == 128) launch_chained(prep_kernel<128, 0>, grid, 256, 0, st, x, c.H, n, hs, ts, c.lsh, c.T, c.B, code_out, rnorm_out, out_stride, bound, clear, BlockHist{});
-  else launch_chained(prep_kernel<64, 0>, grid, 256, 0, st, x, c.H, n, hs, ts, c.lsh, c.T, c.B, code_out, rnorm_out, out_stride, bound, clear, BlockHist{});
+  auto launch = [&](auto kernel) {
+    launch_chained(kernel, grid, 256, 0, st, x, c.H, n, hs, ts, c.lsh, c.T, c.B, code_out, rnorm_out, out_stride, bound, clear, BlockHist{}, conv);
+  };
+  if (c.D == 128) conv.count > 0 ? launch(prep_kernel<128, 0, true>) : launch(prep_kernel<128, 0, false>);
+  else conv.count > 0 ? launch(prep_kernel<64, 0, true>) : launch(prep_kernel<64, 0, false>);
   return cudaGetLastError() == cudaSuccess ? 1 : FASTAR_ERR_CUDA;
 }
 // Codes of the queries and the bucket histograms of their blocks of block_q rows.
-int launch_query_blocks(const CacheView& c, const __nv_bfloat16* q, int nq, int64_t hs, int64_t ts, int block_q, cudaStream_t st) {
+int launch_query_blocks(const CacheView& c, const __nv_bfloat16* q, int nq, int64_t hs, int64_t ts, int block_q, cudaStream_t st, const ConvertArgs& conv) {
   if (nq <= 0) return 0;
   const int64_t groups = static_cast<int64_t>((nq + block_q - 1) / block_q) * c.H * (block_q / 16);
   const int grid = static_cast<int>(min((groups + 7) / 8, static_cast<int64_t>(2 * 148)));
   auto launch = [&](auto kernel) {
-    launch_chained(kernel, grid, 256, 0, st, q, c.H, nq, hs, ts, c.lsh, c.T, c.B, c.code_q_sa, nullptr, c.max_tokens, nullptr, UpdateScratch{}, BlockHist{c.hq, c.max_qb, c.hist_cols});
+    launch_chained(kernel, grid, 256, 0, st, q, c.H, nq, hs, ts, c.lsh, c.T, c.B, c.code_q_sa, nullptr, c.max_tokens, nullptr, UpdateScratch{}, BlockHist{c.hq, c.max_qb, c.hist_cols}, conv);
   };
-  if (c.D == 128) block_q == 128 ? launch(prep_kernel<128, 128>) : launch(prep_kernel<128, 64>);
-  else block_q == 128 ? launch(prep_kernel<64, 128>) : launch(prep_kernel<64, 64>);
+  if (conv.count > 0) {
+    if (c.D == 128) block_q == 128 ? launch(prep_kernel<128, 128, true>) : launch(prep_kernel<128, 64, true>);
+    else block_q == 128 ? launch(prep_kernel<64, 128, true>) : launch(prep_kernel<64, 64, true>);
+  } else {
+    if (c.D == 128) block_q == 128 ? launch(prep_kernel<128, 128, false>) : launch(prep_kernel<128, 64, false>);
+    else block_q == 128 ? launch(prep_kernel<64, 128, false>) : launch(prep_kernel<64, 64, false>);
+  }
   return cudaGetLastError() == cudaSuccess ? 1 : FASTAR_ERR_CUDA;
 }
 bool plan_is_fused(const CacheView& c, int n);
@@ -317,8 +359,8 @@ UpdateScratch update_scratch(const CacheView& c, int n) {
   return z;
 }
 // The first kernel of an update: codes and reciprocal norms of the new keys, and the zeros.
-int launch_prep_update(const CacheView& c, const __nv_bfloat16* k_new, int n, int64_t hs, int64_t ts, cudaStream_t st) {
-  return launch_prep_generic(c, k_new, n, hs, ts, c.code_new, c.rnorm_new, c.max_tokens, st, update_scratch(c, n));
+int launch_prep_update(const CacheView& c, const __nv_bfloat16* k_new, int n, int64_t hs, int64_t ts, cudaStream_t st, const ConvertArgs& conv) {
+  return launch_prep_generic(c, k_new, n, hs, ts, c.code_new, c.rnorm_new, c.max_tokens, st, update_scratch(c, n), conv);
 }
 int launch_prep_codes_strided(const CacheView& c, const __nv_bfloat16* x, int n, int64_t hs, int64_t ts, uint32_t* code_out,
                               int64_t out_stride, cudaStream_t st) {
