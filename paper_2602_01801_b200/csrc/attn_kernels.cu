@@ -125,10 +125,9 @@ __device__ __forceinline__ void add_bf16x2(float2& s, uint32_t b) {
 constexpr int kFlatMin = 8;
 constexpr float kFlatTop = 96.f, kFlatSum = 118.f;
 // Pairs of every sixteen whose exponentials the FMA units work out: the special-function units take 512 cycles for a sub-tile's, the tensor
-// core 270 at d = 64 and 540 at 128.  Kernel time with 0 / 2 / 4 of sixteen: d = 64, 256 items of 128 sub-tiles 96.0 / 91.2 / 90.0 us; d = 128, 256 of
-// 256 194 / 192 / 196, 444 of 138 170 / 170 / 174.
-template <int D>
-constexpr int kPolyPairs = D == 64 ? 4 : 2;
+// core 270 at d = 64 and 540 at 128.  Kernel time with 0 / 2 / 4 of sixteen: d = 64, 256 items of 128 sub-tiles 97.9 / 94.1 / 95.0 us; d = 128, 256 of
+// 256 201 / 200 / 202.
+constexpr int kPolyPairs = 2;
 
 template <int D, int BKT>
 struct AttnSmem {
@@ -832,7 +831,7 @@ attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CU
                   const float ref = -m[2 * hf + e];
                   const float2 u = fadd2(ffma2(make_float2(__uint_as_float(v[0]), __uint_as_float(v[1])), scale2, bias[k]), make_float2(ref, ref));
                   float2 pr;
-                  if (2 * k + e < kPolyPairs<D>) pr = poly_exp2(u);
+                  if (2 * k + e < kPolyPairs) pr = poly_exp2(u);
                   else pr = make_float2(fast_exp2(u.x), fast_exp2(u.y));
                   const uint32_t b = pack_bf16x2(pr.x, pr.y);
                   p[hf][2 * k + e] = b;
