@@ -635,9 +635,15 @@ attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CU
             const int h = item_at(it) / row_blocks % c.H;
             HeadBound b = c.bound[h];
             if (SEG) {
-              const HeadBound p = a.seg_bound[h * kSegParts + lane];
-              b.key = max(b.key, __reduce_max_sync(0xffffffffu, p.key));
-              b.value = max(b.value, __reduce_max_sync(0xffffffffu, p.value));
+              uint32_t key = 0, value = 0;
+#pragma unroll
+              for (int i = 0; i < kSegParts / 32; ++i) {
+                const HeadBound p = a.seg_bound[h * kSegParts + 32 * i + lane];
+                key = max(key, p.key);
+                value = max(value, p.value);
+              }
+              b.key = max(b.key, __reduce_max_sync(0xffffffffu, key));
+              b.value = max(b.value, __reduce_max_sync(0xffffffffu, value));
             }
             const uint32_t row = sbase + SM::q_off + ((warp & 3) * 32 + lane) * 128;
             float sq = 0.f;

@@ -33,7 +33,7 @@ struct HeadBound {
   int32_t count;          // m
   int32_t pad;
 };
-constexpr int kSegParts = 32;      // parts of the tokens of an un-cached segment whose bounds the attention puts together
+constexpr int kSegParts = 128;     // parts of the tokens of an un-cached segment whose bounds the attention puts together
 
 struct CacheView {
   // shape
@@ -259,9 +259,13 @@ int launch_plan(const CacheView& c, int n, float tau, const UpdateOut& out, cuda
 int launch_commit(const CacheView& c, const __nv_bfloat16* k_new, const __nv_bfloat16* v_new, int n, int frame_len,
                   int64_t hs, int64_t ts, cudaStream_t st);
 int launch_finalize_hist(const CacheView& c, fastar_update_stats* stats_out, int advance_clock, cudaStream_t st);
-int launch_segment(const CacheView& c, const __nv_bfloat16* k, int64_t khs, int64_t kts, const __nv_bfloat16* v, int64_t vhs, int64_t vts, int ns,
-                   int tiles, cudaStream_t st);
-int launch_topk_blocks(const CacheView& c, int nqb, int keep, int force_sink, int force_recent, cudaStream_t st);
+struct SegArgs {           // an un-cached segment of an attention call
+  const __nv_bfloat16 *k, *v;
+  int64_t hs, ts;
+  int ns, total;           // its tokens, and the rows of its tiles
+};
+int launch_segment(const CacheView& c, const SegArgs& s, cudaStream_t st);
+int launch_topk_blocks(const CacheView& c, int nqb, int keep, int force_sink, int force_recent, const SegArgs* seg, cudaStream_t st);      // seg: with its parts, or null
 int launch_topk_prompt(const CacheView& c, int n_frames, int np, int keep, cudaStream_t st);
 int launch_reset(const CacheView& c, cudaStream_t st);
 int launch_import_derive(const CacheView& c, cudaStream_t st);

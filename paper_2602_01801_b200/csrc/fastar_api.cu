@@ -727,6 +727,22 @@ static int annsa_impl(fastar_cache_t* c, const HeadRange& range, bool hashed, bo
   a.out_fp32 = c->desc.dtype == FASTAR_FP32;
   a.out_head_stride = head_stride;
   a.out_token_stride = token_stride;
+  CUtensorMap tm_sk, tm_sv;
+  SegArgs seg{};
+  bool seg_done = false;
+  if (k_seg) {
+    // the update's staging slots are free during an attention call (where the segment has to be converted, no items are cut)
+    a.no_cut = a.no_cut || c->desc.dtype != FASTAR_BF16;
+    View sg[2] = {{k_seg, ns, 0, seg_head_stride, seg_token_stride, nullptr}, {v_seg, ns, 1, seg_head_stride, seg_token_stride, nullptr}};
+    r = as_bf16(c, v, sg, 2, st);
+    if (r == FASTAR_OK) r = make_map(c, &tm_sk, sg[0].p, v.D, ns, v.H, static_cast<uint64_t>(sg[0].ts) * 2, static_cast<uint64_t>(sg[0].hs) * 2, v.PT);
+    if (r == FASTAR_OK) r = make_map(c, &tm_sv, sg[1].p, v.D, ns, v.H, static_cast<uint64_t>(sg[1].ts) * 2, static_cast<uint64_t>(sg[1].hs) * 2, v.PT);
+    if (r != FASTAR_OK) return r;
+    a.seg_tiles = (ns + v.PT - 1) / v.PT;
+    a.seg_bias = v.seg_bias;
+    a.seg_bound = v.seg_bound;
+    seg = SegArgs{sg[0].p, sg[1].p, sg[0].hs, sg[0].ts, ns, a.seg_tiles * v.PT};      // K and V alike
+  }
   if (sel_in) {
     a.sel = sel_in;
     a.nsel = nsel_in;
@@ -745,7 +761,8 @@ static int annsa_impl(fastar_cache_t* c, const HeadRange& range, bool hashed, bo
         vh.scores = v.scores_hi;
         ACCK(FASTAR_K_S3_SCORES, launch_s3_scores(vh, range.tm_hq, range.tm_hk_hi, nqb, st));
       }
-      ACCK(FASTAR_K_TOPK_BLOCKS, launch_topk_blocks(v, nqb, keep, c->force_sink_blocks, c->force_recent_blocks, st));
+      seg_done = k_seg != nullptr;             // (on the SMs that the ranking leaves idle)
+      ACCK(FASTAR_K_TOPK_BLOCKS, launch_topk_blocks(v, nqb, keep, c->force_sink_blocks, c->force_recent_blocks, k_seg ? &seg : nullptr, st));
     }
     a.sel = v.sel;
     a.nsel = v.nsel;
@@ -773,20 +790,7 @@ static int annsa_impl(fastar_cache_t* c, const HeadRange& range, bool hashed, bo
       return FASTAR_ERR_CUDA;
     }
   }
-  CUtensorMap tm_sk, tm_sv;
-  if (k_seg) {
-    // the update's staging slots are free during an attention call (where the segment has to be converted, no items are cut)
-    a.no_cut = a.no_cut || c->desc.dtype != FASTAR_BF16;
-    View sg[2] = {{k_seg, ns, 0, seg_head_stride, seg_token_stride, nullptr}, {v_seg, ns, 1, seg_head_stride, seg_token_stride, nullptr}};
-    r = as_bf16(c, v, sg, 2, st);
-    if (r == FASTAR_OK) r = make_map(c, &tm_sk, sg[0].p, v.D, ns, v.H, static_cast<uint64_t>(sg[0].ts) * 2, static_cast<uint64_t>(sg[0].hs) * 2, v.PT);
-    if (r == FASTAR_OK) r = make_map(c, &tm_sv, sg[1].p, v.D, ns, v.H, static_cast<uint64_t>(sg[1].ts) * 2, static_cast<uint64_t>(sg[1].hs) * 2, v.PT);
-    if (r != FASTAR_OK) return r;
-    a.seg_tiles = (ns + v.PT - 1) / v.PT;
-    a.seg_bias = v.seg_bias;
-    a.seg_bound = v.seg_bound;
-    ACC(launch_segment(v, sg[0].p, sg[0].hs, sg[0].ts, sg[1].p, sg[1].hs, sg[1].ts, ns, a.seg_tiles, st));
-  }
+  if (k_seg && !seg_done) ACC(launch_segment(v, seg, st));
   ACCK(FASTAR_K_S5_ATTENTION, launch_attention_paged(v, tm_q, c->tm_pool_k, c->tm_pool_v, k_seg ? &tm_sk : nullptr,
                                                      k_seg ? &tm_sv : nullptr, a, st));
   return FASTAR_OK;

@@ -1003,27 +1003,25 @@ int launch_finalize_hist(const CacheView& c, fastar_update_stats* stats_out, int
 // ---------------------------------------------------------------------------------------------
 // An un-cached segment of an attention call: the biases of its rows, and what its keys and values do not exceed, by kSegParts parts of the
 // tokens of a head, which the attention puts together (so there is nothing to clear and no atomic).  Half a warp (a quarter at d = 64) has a row.
+// The parts are CTAs of 64 threads, on the SMs that the block top-k leaves idle where there is one (12 heads x 4680 tokens, with the top-k 3.9 + 8.5 -> 9.0 us).
 // ---------------------------------------------------------------------------------------------
 template <int D>
-__global__ void __launch_bounds__(256) segment_kernel(const CacheView c, const __nv_bfloat16* __restrict__ k, int64_t khs, int64_t kts,
-                                                      const __nv_bfloat16* __restrict__ v, int64_t vhs, int64_t vts, int ns, int total) {
-  constexpr int LPR = D / 8, RPC = 256 / LPR;          // lanes a row, rows a CTA's pass
-  __shared__ HeadBound part;
-  if (threadIdx.x == 0) part = HeadBound{};
+__device__ __forceinline__ void segment_part(const CacheView& c, const SegArgs& s, int h, int part) {
+  constexpr int LPR = D / 8, RPW = 32 / LPR, B = 4;    // lanes a row, rows a warp, rows of a thread that are under way
+  __shared__ HeadBound bound;
+  if (threadIdx.x == 0) bound = HeadBound{};
   __syncthreads();
-  chain_wait();
-  const int h = blockIdx.y, sl = threadIdx.x % LPR;
-  for (int i = (h * kSegParts + blockIdx.x) * 256 + threadIdx.x; i < total; i += c.H * kSegParts * 256) c.seg_bias[i] = i < ns ? 0.f : -INFINITY;
-  const int r0 = static_cast<int>(static_cast<int64_t>(ns) * blockIdx.x / kSegParts), r1 = static_cast<int>(static_cast<int64_t>(ns) * (blockIdx.x + 1) / kSegParts);
+  const int sl = threadIdx.x % LPR, rpc = blockDim.x / LPR;
+  for (int i = (h * kSegParts + part) * blockDim.x + threadIdx.x; i < s.total; i += c.H * kSegParts * blockDim.x) c.seg_bias[i] = i < s.ns ? 0.f : -INFINITY;
+  const int r0 = static_cast<int>(static_cast<int64_t>(s.ns) * part / kSegParts), r1 = static_cast<int>(static_cast<int64_t>(s.ns) * (part + 1) / kSegParts);
   uint32_t kmost = 0, vmost = 0;
-  constexpr int RPW = 32 / LPR, B = 4;                 // rows a warp, rows of a thread that are under way
-  for (int rb = r0 + (threadIdx.x >> 5) * RPW; rb < r1; rb += B * RPC) {
+  for (int rb = r0 + (threadIdx.x >> 5) * RPW; rb < r1; rb += B * rpc) {
     uint4 kr[B], vr[B];
 #pragma unroll
-    for (int b = 0; b < B; ++b) {                        // past the end the last row again
-      const int row = min(rb + b * RPC + (threadIdx.x & 31) / LPR, r1 - 1);
-      kr[b] = *reinterpret_cast<const uint4*>(k + h * khs + row * kts + sl * 8);
-      vr[b] = *reinterpret_cast<const uint4*>(v + h * vhs + row * vts + sl * 8);
+    for (int b = 0; b < B; ++b) {                      // past the end the last row again
+      const int row = min(rb + b * rpc + static_cast<int>(threadIdx.x & 31) / LPR, r1 - 1);
+      kr[b] = *reinterpret_cast<const uint4*>(s.k + h * s.hs + row * s.ts + sl * 8);
+      vr[b] = *reinterpret_cast<const uint4*>(s.v + h * s.hs + row * s.ts + sl * 8);
     }
 #pragma unroll
     for (int b = 0; b < B; ++b) {
@@ -1034,16 +1032,20 @@ __global__ void __launch_bounds__(256) segment_kernel(const CacheView c, const _
       kmost = max(kmost, __float_as_uint(sq));
     }
   }
-  raise_bound_warp(&part.key, 0, kmost);
-  raise_bound_warp(&part.value, 0, vmost);
+  raise_bound_warp(&bound.key, 0, kmost);
+  raise_bound_warp(&bound.value, 0, vmost);
   __syncthreads();
-  if (threadIdx.x == 0) c.seg_bound[h * kSegParts + blockIdx.x] = part;
+  if (threadIdx.x == 0) c.seg_bound[h * kSegParts + part] = bound;
 }
-int launch_segment(const CacheView& c, const __nv_bfloat16* k, int64_t khs, int64_t kts, const __nv_bfloat16* v, int64_t vhs, int64_t vts, int ns,
-                   int tiles, cudaStream_t st) {
+template <int D>
+__global__ void __launch_bounds__(64) segment_kernel(const CacheView c, const SegArgs s) {
+  chain_wait();
+  segment_part<D>(c, s, blockIdx.y, blockIdx.x);
+}
+int launch_segment(const CacheView& c, const SegArgs& s, cudaStream_t st) {
   const dim3 grid(kSegParts, c.H);
-  if (c.D == 128) launch_chained(segment_kernel<128>, grid, 256, 0, st, c, k, khs, kts, v, vhs, vts, ns, tiles * c.PT);
-  else launch_chained(segment_kernel<64>, grid, 256, 0, st, c, k, khs, kts, v, vhs, vts, ns, tiles * c.PT);
+  if (c.D == 128) launch_chained(segment_kernel<128>, grid, 64, 0, st, c, s);
+  else launch_chained(segment_kernel<64>, grid, 64, 0, st, c, s);
   return cudaGetLastError() == cudaSuccess ? 1 : FASTAR_ERR_CUDA;
 }
 
@@ -1054,16 +1056,29 @@ __global__ void __launch_bounds__(32 * kTopkWarps) topk_kernel(const TopkArgs a)
   const int row = blockIdx.x * kTopkWarps + (threadIdx.x >> 5);
   if (row < a.rows) topk_row<PROMPT, NV>(a, blockIdx.y, row);
 }
+// The same with the parts of a segment behind the rows' CTAs.
+template <int NV, int D>
+__global__ void __launch_bounds__(32 * kTopkWarps) topk_segment_kernel(const TopkArgs a, const CacheView c, const SegArgs s) {
+  chain_wait();
+  const int ctas = (a.rows + kTopkWarps - 1) / kTopkWarps, row = blockIdx.x * kTopkWarps + (threadIdx.x >> 5);
+  if (static_cast<int>(blockIdx.x) >= ctas) segment_part<D>(c, s, blockIdx.y, blockIdx.x - ctas);
+  else if (row < a.rows) topk_row<false, NV>(a, blockIdx.y, row);
+}
 
 template <bool PROMPT>
-static int launch_topk(const TopkArgs& a, int columns, int H, cudaStream_t st) {
-  const dim3 grid((a.rows + kTopkWarps - 1) / kTopkWarps, H);
-  const int threads = 32 * kTopkWarps;
-  if (columns <= 128) launch_chained(topk_kernel<PROMPT, 4>, grid, threads, 0, st, a);
-  else if (columns <= 256) launch_chained(topk_kernel<PROMPT, 8>, grid, threads, 0, st, a);
-  else if (columns <= 512) launch_chained(topk_kernel<PROMPT, 16>, grid, threads, 0, st, a);
-  else if (columns <= 1152) launch_chained(topk_kernel<PROMPT, 36>, grid, threads, 0, st, a);
-  else if (columns <= 2048) launch_chained(topk_kernel<PROMPT, 64>, grid, threads, 0, st, a);
+static int launch_topk(const TopkArgs& a, int columns, const CacheView& c, const SegArgs* seg, cudaStream_t st) {
+  const int ctas = (a.rows + kTopkWarps - 1) / kTopkWarps, threads = 32 * kTopkWarps;
+  auto launch = [&](auto width) {
+    constexpr int NV = decltype(width)::value;
+    if (PROMPT || !seg) launch_chained(topk_kernel<PROMPT, NV>, dim3(ctas, c.H), threads, 0, st, a);
+    else if (c.D == 128) launch_chained(topk_segment_kernel<NV, 128>, dim3(ctas + kSegParts, c.H), threads, 0, st, a, c, *seg);
+    else launch_chained(topk_segment_kernel<NV, 64>, dim3(ctas + kSegParts, c.H), threads, 0, st, a, c, *seg);
+  };
+  if (columns <= 128) launch(std::integral_constant<int, 4>{});
+  else if (columns <= 256) launch(std::integral_constant<int, 8>{});
+  else if (columns <= 512) launch(std::integral_constant<int, 16>{});
+  else if (columns <= 1152) launch(std::integral_constant<int, 36>{});
+  else if (columns <= 2048) launch(std::integral_constant<int, 64>{});
   else return FASTAR_ERR_UNSUPPORTED_SHAPE;          // the entry points refuse such rows
   return cudaGetLastError() == cudaSuccess ? 1 : FASTAR_ERR_CUDA;
 }
@@ -1086,8 +1101,8 @@ TopkArgs block_topk_args(const CacheView& c, int nqb, int keep, int force_sink, 
   a.status = c.status;
   return a;
 }
-int launch_topk_blocks(const CacheView& c, int nqb, int keep, int force_sink, int force_recent, cudaStream_t st) {
-  return launch_topk<false>(block_topk_args(c, nqb, keep, force_sink, force_recent), c.CAPB, c.H, st);
+int launch_topk_blocks(const CacheView& c, int nqb, int keep, int force_sink, int force_recent, const SegArgs* seg, cudaStream_t st) {
+  return launch_topk<false>(block_topk_args(c, nqb, keep, force_sink, force_recent), c.CAPB, c, seg, st);
 }
 // ---------------------------------------------------------------------------------------------
 // AnnCA with the LSH bucket rule (Section 5.3): a prompt token is kept for a frame iff, in at least one table, a
@@ -1152,7 +1167,7 @@ TopkArgs prompt_topk_args(const CacheView& c, int n_frames, int np, int keep) {
   return a;
 }
 int launch_topk_prompt(const CacheView& c, int n_frames, int np, int keep, cudaStream_t st) {
-  return launch_topk<true>(prompt_topk_args(c, n_frames, np, keep), np, c.H, st);
+  return launch_topk<true>(prompt_topk_args(c, n_frames, np, keep), np, c, nullptr, st);
 }
 
 // ---------------------------------------------------------------------------------------------
