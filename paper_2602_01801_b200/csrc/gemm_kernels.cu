@@ -26,7 +26,9 @@ constexpr int kGemmThreads = 320;            // warps 0-7 epilogue, 8 TMA produc
 constexpr int kGemmProducerWarp = 8, kGemmMmaWarp = 9;
 
 // Ring stages of a chunk of both operands.  A CTA's sixteen chunks are a chain of loads, so a grid of one CTA per SM at most takes all the
-// shared memory for its ring: two round trips to L2 instead of four.  A larger grid has two CTAs per SM, each with half of the loads under way.
+// shared memory for its ring: two round trips to L2 instead of four (48 CTAs 8.0 -> 7.5 us, 128 9.4 -> 8.3, 24 7.3 -> 6.85, 6 7.6 -> 7.45).  A
+// larger grid has two CTAs per SM, each with half of the loads under way, and a few CTAs find L2 idle: they are slower with the long ring (four
+// 6.4 -> 6.85, one that ranks 8.4 -> 8.7).
 constexpr int kFewStages = 4, kManyStages = 9;
 template <int NST>
 struct GemmSmem {
@@ -209,7 +211,9 @@ static int launch_gemm(const CacheView& c, const CUtensorMap& tm_hq, const CUten
   int dev = 0, sm_count = 148;
   if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sm_count, cudaDevAttrMultiProcessorCount, dev);
   const dim3 grid((g.rows_a + 127) / 128, c.H, (c.CAPB + kTileN - 1) / kTileN);
-  if (static_cast<int64_t>(grid.x) * grid.y * grid.z <= sm_count) return launch_gemm_t<RANK, kManyStages>(c, tm_hq, tm_hk, g, grid, st);
+  const int64_t ctas = static_cast<int64_t>(grid.x) * grid.y * grid.z;
+  if constexpr (!RANK)
+    if (ctas >= 6 && ctas <= sm_count) return launch_gemm_t<RANK, kManyStages>(c, tm_hq, tm_hk, g, grid, st);
   return launch_gemm_t<RANK, kFewStages>(c, tm_hq, tm_hk, g, grid, st);
 }
 

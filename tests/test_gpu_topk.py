@@ -57,9 +57,9 @@ def test_prompt_topk(prompt, keep):
             assert np.array_equal(r["sel"][h, f].cpu().numpy(), _kept(want, keep))
 
 
-@pytest.mark.parametrize("H,capacity,nq", [(1, 128, 1), (29, 16640, 130), (40, 16640, 130)])
+@pytest.mark.parametrize("H,capacity,nq", [(1, 4224, 130), (29, 16640, 130), (40, 16640, 130)])
 def test_block_scores_of_few_and_many_heads(H, capacity, nq):
-    """The grid of the block scores on both sides of one CTA per SM (1, 145 and 200 CTAs): same-bucket pairs counted from the codes."""
+    """The grid of the block scores on both sides of one CTA per SM (2, 145 and 200 CTAs): same-bucket pairs counted from the codes."""
     import torch
     from paper_2602_01801_b200 import fastar
     rng = np.random.default_rng(H)
