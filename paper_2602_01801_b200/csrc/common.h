@@ -172,8 +172,15 @@ int launch_t1_similarity_fp8(const CacheView& c, const CUtensorMap& tm_a8, const
                              cudaStream_t st);
 int launch_sign_rows(const CacheView& c, const uint32_t* codes, int n, int64_t code_stride, uint8_t* out, int64_t out_rows_per_head,
                      cudaStream_t st);
-int launch_quantize_rows(const CacheView& c, const __nv_bfloat16* x, int n, int64_t hs, int64_t ts, uint8_t* out,
-                         int64_t out_rows_per_head, float* norm_out, int64_t norm_stride, cudaStream_t st);
+struct QuantizeRows {      // rows to code: their norms and codes at the same places, rows_per_head of them a head
+  const __nv_bfloat16* x;
+  int64_t hs, ts;
+  int n;
+  uint8_t* out;
+  float* norm_out;
+  int64_t rows_per_head;
+};
+int launch_quantize_rows(const CacheView& c, const QuantizeRows& a, const QuantizeRows& b, cudaStream_t st);
 
 // relevance_kernel.cu: C1 on the bf16 rows and on the 8-bit codes; with the ranking if keep > 0, where c1_ranks says that it pays
 bool c1_ranks(const CacheView& c, int nq, int n_frames, int np, bool beside);

@@ -648,7 +648,7 @@ static int update_impl(fastar_cache_t* c, const HeadRange& range, UpdatePart par
     if (r != FASTAR_OK) return r;
     if (v.sign_codes) ACCK(FASTAR_K_HASH, launch_sign_rows(v, v.code_new, n, v.max_tokens, v.k8_new, v.max_tokens, st));
     else ACCK(FASTAR_K_HASH, launch_quantize_keys(v, kb, n, khs, kts, v.rnorm_new, v.max_tokens, v.k8_new, v.max_tokens, st));
-    if (q_probe) ACCK(FASTAR_K_HASH, launch_quantize_rows(v, pb, n, phs, pts, v.q8_probe, v.max_tokens, v.qn_probe, v.max_tokens, st));
+    if (q_probe) ACCK(FASTAR_K_HASH, launch_quantize_rows(v, QuantizeRows{pb, phs, pts, n, v.q8_probe, v.qn_probe, v.max_tokens}, QuantizeRows{}, st));
     ACCK(FASTAR_K_T1_SIMILARITY, launch_t1_similarity_fp8(vs, tm_a8, c->tm_pool_k8, n, q_probe != nullptr, st));
     // query-probe and Hamming rankings are not similarities: the threshold is applied to the exact key cosine of the winner
     if (q_probe || v.sign_codes) ACCK(FASTAR_K_PLAN, launch_probe_cosine(v, kb, n, khs, kts, st));
@@ -902,8 +902,8 @@ static int annca_impl(fastar_cache_t* c, const HeadRange& range, bool beside, co
       r = make_map_codes(c, &tm_q8, v.q8_ca, nq, v.H, static_cast<uint64_t>(v.max_tokens) * 128, 128);
       if (r == FASTAR_OK) r = make_map_codes(c, &tm_kp8, v.kp8_ca, np, v.H, static_cast<uint64_t>(v.max_prompt) * 128, 128);
       if (r != FASTAR_OK) return r;
-      ACCK(FASTAR_K_HASH, launch_quantize_rows(v, qb, nq, qhs, qts, v.q8_ca, v.max_tokens, v.qn_ca, v.max_tokens, st));
-      ACCK(FASTAR_K_HASH, launch_quantize_rows(v, kpb, np, khs, kts, v.kp8_ca, v.max_prompt, v.kpn_ca, v.max_prompt, st));
+      const QuantizeRows queries{qb, qhs, qts, nq, v.q8_ca, v.qn_ca, v.max_tokens}, prompt{kpb, khs, kts, np, v.kp8_ca, v.kpn_ca, v.max_prompt};
+      ACCK(FASTAR_K_HASH, launch_quantize_rows(v, queries, prompt, st));
       ACCK(FASTAR_K_C1_RELEVANCE, launch_c1_relevance_fp8(v, tm_q8, tm_kp8, v.qn_ca, v.kpn_ca, nq, np, frame_len, ranked, st));
       rel_scale *= 1.0f / 256.0f;
     } else {

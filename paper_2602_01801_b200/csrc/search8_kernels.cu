@@ -39,23 +39,21 @@ struct Smem {
 
 }  // namespace
 
-// Half a warp per row: |x|, then the code of x / |x| * 16 (an all-zero row gets an all-zero code and norm 0).
-__global__ void __launch_bounds__(256) quantize_rows_kernel(const __nv_bfloat16* __restrict__ x, int H, int n, int D, int64_t hs,
-                                                            int64_t ts, uint8_t* __restrict__ out, int64_t out_rows_per_head,
-                                                            float* __restrict__ norm_out, int64_t norm_stride) {
+// Half a warp per row: |x|, then the code of x / |x| * 16 (an all-zero row gets an all-zero code and norm 0).  One or two tensors a launch:
+// AnnCA codes its queries and its prompt keys (12 heads x 4680 and 512 rows 11.3 -> 9.8 us).
+__global__ void __launch_bounds__(256) quantize_rows_kernel(const QuantizeRows a, const QuantizeRows b, int H, int D) {
   chain_wait();
-  const int64_t rows = static_cast<int64_t>(H) * n;
+  const int rows_a = H * a.n, rows = rows_a + H * b.n;
   const unsigned hmask = 0xFFFFu << (threadIdx.x & 16);
-  for (int64_t q = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x; (q >> 4) < rows;
-       q += static_cast<int64_t>(gridDim.x) * blockDim.x) {
-    const int e8 = static_cast<int>(q & 15);
-    const int64_t rowid = q >> 4;
-    const int h = static_cast<int>(rowid / n), i = static_cast<int>(rowid % n);
+  const int e8 = threadIdx.x & 15;
+  for (int r = (blockIdx.x * 256 + threadIdx.x) >> 4; r < rows; r += gridDim.x * 16) {
+    const bool first = r < rows_a;
+    const int rowid = first ? r : r - rows_a, n = first ? a.n : b.n, h = rowid / n, i = rowid - h * n;
     float f[8];
 #pragma unroll
     for (int e = 0; e < 8; ++e) f[e] = 0.f;
     if (e8 * 8 < D) {
-      const uint4 v = *reinterpret_cast<const uint4*>(x + h * hs + i * ts + e8 * 8);
+      const uint4 v = *reinterpret_cast<const uint4*>((first ? a.x : b.x) + h * (first ? a.hs : b.hs) + i * (first ? a.ts : b.ts) + e8 * 8);
       const __nv_bfloat162* p = reinterpret_cast<const __nv_bfloat162*>(&v);
 #pragma unroll
       for (int e = 0; e < 4; ++e) {
@@ -75,18 +73,17 @@ __global__ void __launch_bounds__(256) quantize_rows_kernel(const __nv_bfloat16*
 #pragma unroll
     for (int e = 0; e < 4; ++e)
       w[e] = __nv_cvt_float2_to_fp8x2(make_float2(f[2 * e] * s, f[2 * e + 1] * s), __NV_SATFINITE, __NV_E4M3);
-    *reinterpret_cast<uint2*>(out + (static_cast<int64_t>(h) * out_rows_per_head + i) * 128 + e8 * 8) =
-        make_uint2(w[0] | (w[1] << 16), w[2] | (w[3] << 16));
-    if (e8 == 0) norm_out[h * norm_stride + i] = nrm;
+    const int64_t row = static_cast<int64_t>(h) * (first ? a.rows_per_head : b.rows_per_head) + i;
+    *reinterpret_cast<uint2*>((first ? a.out : b.out) + row * 128 + e8 * 8) = make_uint2(w[0] | (w[1] << 16), w[2] | (w[3] << 16));
+    if (e8 == 0) (first ? a.norm_out : b.norm_out)[row] = nrm;
   }
 }
 
-int launch_quantize_rows(const CacheView& c, const __nv_bfloat16* x, int n, int64_t hs, int64_t ts, uint8_t* out,
-                         int64_t out_rows_per_head, float* norm_out, int64_t norm_stride, cudaStream_t st) {
-  if (n <= 0) return 0;
-  const int64_t total = static_cast<int64_t>(c.H) * n * 16;
+int launch_quantize_rows(const CacheView& c, const QuantizeRows& a, const QuantizeRows& b, cudaStream_t st) {
+  const int64_t total = static_cast<int64_t>(c.H) * (a.n + b.n) * 16;
+  if (total <= 0) return 0;
   const int grid = static_cast<int>((total + 255) / 256 < 148 * 8 ? (total + 255) / 256 : 148 * 8);
-  launch_chained(quantize_rows_kernel, grid, 256, 0, st, x, c.H, n, c.D, hs, ts, out, out_rows_per_head, norm_out, norm_stride);
+  launch_chained(quantize_rows_kernel, grid, 256, 0, st, a, b, c.H, c.D);
   return cudaGetLastError() == cudaSuccess ? 1 : FASTAR_ERR_CUDA;
 }
 
