@@ -294,7 +294,7 @@ attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CU
   const uint32_t bar_q_empty = bar + 8;              // the MMAs (or copies) that read Q, and the warps that look at it (FLAT)
   const uint32_t bar_r_full = bar + 16;              // [RS] the K stages, then the V stages
   const uint32_t bar_r_empty = bar_r_full + 8 * RS;  // [RS]
-  const uint32_t bar_s_full = bar_r_empty + 8 * RS;  // [4] by key tile: the MMAs' commit, and the issuing warp once the biases are there
+  const uint32_t bar_s_full = bar_r_empty + 8 * RS;  // [4] by key tile, QT by group: the MMAs' commit, and the issuing warp once the biases are there
   const uint32_t bar_pv_done = bar_s_full + 32;      // [4] by sub-tile
   const uint32_t bar_s_empty = bar_pv_done + 32;     // [4] by key tile: the warps of its groups
   const uint32_t bar_p_full = bar_s_empty + 32;      // [4] by sub-tile: the warps of its group
