@@ -21,7 +21,7 @@
  *     void* (0 = the legacy default stream).  All work is enqueued on that stream and the
  *     call returns without synchronising unless stated otherwise.
  *   - Ownership: the caller owns every tensor and the workspace buffer; the library owns only
- *     the small host object behind fastar_cache_t (with four CUDA streams and their events created and
+ *     the small host object behind fastar_cache_t (with five CUDA streams and their events created and
  *     destroyed with it).  Nothing here allocates device memory.
  *   - Tensors are [head][token][channel] with element strides `head_stride`, `token_stride`
  *     (channel stride 1).  Strides in bytes must be multiples of 16 and base pointers 16-byte

@@ -43,7 +43,7 @@ struct fastar_cache {
   bool rel_clear = true;     // AnnCA's relevance maxima are zero behind all work queued so far (create and every prompt top-k leave them so)
   // the host-tensor step's streams and events (fastar_attention_step_host); the events of a slice: its keys, queries and values are up,
   // planned, queries hashed, AnnCA's and AnnSA's outputs are there
-  enum { kUp = 0, kSide, kAttend, kDown, kStreams };
+  enum { kUp = 0, kSide, kAttend, kDown, kDown2, kStreams };
   enum { kKeysUp = 0, kQueriesUp, kValuesUp, kPlanned, kHashed, kCrossDone, kSelfDone, kSliceEvents };
   cudaStream_t streams[kStreams] = {};
   cudaEvent_t slice_ev[kMaxSlices][kSliceEvents] = {};
@@ -1027,10 +1027,15 @@ int fastar_attention_step_host(fastar_cache_t* c, const void* k_new_host, const 
   //   caller's: (keys up) search, planning, slice by slice
   //   side    : (queries up) their hash for AnnSA's selector, AnnCA
   //   attend  : (planned, values up) commit, (hashed) AnnSA
-  //   down    : AnnCA's outputs, AnnSA's outputs
-  // 12 heads x 4680 tokens against 28 080 keys, bf16: 1 368 -> 1 223 us with four slices (46.3 MB up and 28.8 down take 952 at once).  Against
-  // 1 190 on another box: 1 277 with two, 1 274 with six; 1 225 with the queries before the keys, 1 277 with AnnCA's output in one copy, 1 345
-  // with the queries in one.  With 4 of 147 blocks kept against 9 360 keys it is 1 225 -> 1 266: little computing to hide.
+  //   down    : AnnCA's outputs, AnnSA's outputs (two streams in turn, by slice)
+  // 12 heads x 4680 tokens against 28 080 keys, bf16, four slices: 1 368 -> 1 150 to 1 210 us (46.3 MB up and 28.8 down take 952 at once).  With one
+  // stream for the downloads the call depends on when the kernels between them end: 1 235 to 1 310, but 1 173 to 1 193 with a search that takes
+  // 4 % longer.  (Means of 240 calls; single ones vary by 50 either way.)  Two streams against one, by shape: the same with 8-bit search 0.94, by the
+  // probe 0.94, 4 blocks kept of 147 0.94, 11 heads x 1 120 in fp32 0.94, 25 and 40 heads 1.00, 6 and 8 heads 1.01 and 1.015.  With two: slices
+  // of 4, 4, 2 and 2 heads 1 214, of 4, 3, 3 and 2 1 221, three of 4 1 191; a stream for each download 1 145 to 1 160.  With one, against 1 190: 1 277
+  // with two slices, 1 274 with six; 1 225 with the queries before the keys, 1 277 with AnnCA's output in one copy, 1 345 with the queries in
+  // one.  Uploads through two streams 1 400, and 1 300 if each waits for the one before.  Where there is little computing to hide, slices lose:
+  // 4 of 147 blocks kept against 9 360 keys 1 225 -> 1 266 with one stream of downloads.
   // A slice below 3 MB a tensor is not worth its launches (11 heads x 1 120, fp32, 6 MB: 660 -> 636 with two slices, 713 with three).  The
   // owned streams start behind what the caller's stream holds and are joined before the call returns.
   const size_t token_bytes = static_cast<size_t>(n) * v.D * esz, prompt_bytes = static_cast<size_t>(np) * v.D * esz, all_bytes = token_bytes * v.H;
@@ -1043,7 +1048,7 @@ int fastar_attention_step_host(fastar_cache_t* c, const void* k_new_host, const 
   for (int i = 0; i <= slices; ++i) first[i] = v.H * i / slices;
   for (int i = 0; i < slices && r == FASTAR_OK; ++i) r = make_range(c, first[i], first[i + 1] - first[i], &ranges[i]);
   if (r != FASTAR_OK) return r;
-  cudaStream_t up = c->streams[c->kUp], side = c->streams[c->kSide], attend = c->streams[c->kAttend], down = c->streams[c->kDown];
+  cudaStream_t up = c->streams[c->kUp], side = c->streams[c->kSide], attend = c->streams[c->kAttend];
   auto try_cuda = [&](cudaError_t e) { if (e != cudaSuccess && r == FASTAR_OK) r = FASTAR_ERR_CUDA; };
   auto at = [&](const void* base, int h, size_t head_bytes) { return static_cast<uint8_t*>(const_cast<void*>(base)) + h * head_bytes; };
   auto upload = [&](int i, int h0, int h1, size_t head_bytes) {
@@ -1087,7 +1092,10 @@ int fastar_attention_step_host(fastar_cache_t* c, const void* k_new_host, const 
                      frame_len, np, keep_tokens, hs, ts, phs, ts, nullptr, nullptr, nullptr, side);
     try_cuda(cudaEventRecord(ev[c->kCrossDone], side));
   };
-  auto download = [&](int which, int i) {                                  // 0 AnnSA's output, 1 AnnCA's
+  // 0 AnnSA's output, 1 AnnCA's.  Two streams take turns: a copy's start is then made ready while the one before still runs, and less of the
+  // uploads' time goes by between copies (147 -> 125 us of a call).
+  auto download = [&](int which, int i) {
+    cudaStream_t down = c->streams[i & 1 ? c->kDown2 : c->kDown];
     try_cuda(cudaStreamWaitEvent(down, c->slice_ev[i][which ? c->kCrossDone : c->kSelfDone], 0));
     try_cuda(cudaMemcpyAsync(at(which ? out_ca_host : out_sa_host, first[i], token_bytes), at(v.stage_out[which], first[i], token_bytes),
                              (first[i + 1] - first[i]) * token_bytes, cudaMemcpyDeviceToHost, down));
