@@ -116,14 +116,14 @@ __device__ __forceinline__ void add_bf16x2(float2& s, uint32_t b) {
   asm("{.reg .b16 l, h; mov.b32 {l, h}, %2; add.f32.bf16 %0, l, %0; add.f32.bf16 %1, h, %1;}" : "+f"(s.x), "+f"(s.y) : "r"(b));
 }
 // Flat items.  A logit is at most |q| max |k| / sqrt(d) + log2 max m; the cache keeps the largest of each head (HeadBound), a segment's come
-// with the call, and |q| is worked out here.  If that, for the rows of a warp, is not more than T above the reference that an item's first
+// with the call, and |q| is worked out here.  If that, for the rows of a warp, is not more than kTop above the reference that an item's first
 // sub-tile gives, nothing after it can ask for another reference: the sub-tiles that follow need no maximum, no look at the others' and no
-// hand-over, which are 160 of the loop's 440 instructions.  (One reference for the four rows of a thread, within the biases, would spare 24
+// hand-over, which are 160 of the loop's 440 instructions, and every probability is taken relative to what the loop that looks would take it.  (One reference for the four rows of a thread, within the biases, would spare 24
 // more and is 1 to 3 % faster, but then the largest probabilities no longer lie just below a power of two, where bf16 is finest: error against
-// 64 bits 0.00230 -> 0.00233.)  T is as large as the sums of P V allow: keys x 2^T x
-// max |v| is below 2^118, or T is kTop, as where the maximum is looked for.  Items of fewer sub-tiles than kFlatMin don't ask.
+// 64 bits 0.00230 -> 0.00233.  Nor may the bound be further above: with 96, as far as fp32 sums bear, items stay flat in which the other loop
+// would have raised, and behind a raise the row's largest probability is a power of two.  Keys in the order of their clusters, logits of 1.5 to 4
+// times the usual size: 0.00209-0.00230 where the maximum is looked for, 0.00224-0.00233 so.)  Items of fewer sub-tiles than kFlatMin don't ask.
 constexpr int kFlatMin = 8;
-constexpr float kFlatTop = 96.f, kFlatSum = 118.f;
 // Pairs of every sixteen whose exponentials the FMA units work out: the special-function units take 512 cycles for a sub-tile's, the tensor
 // core 270 at d = 64 and 540 at 128.  Kernel time with 0 / 2 / 4 of sixteen: d = 64, 256 items of 128 sub-tiles 97.9 / 94.1 / 95.0 us; d = 128, 256 of
 // 256 201 / 200 / 202.
@@ -635,15 +635,10 @@ attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CU
             const int h = item_at(it) / row_blocks % c.H;
             HeadBound b = c.bound[h];
             if (SEG) {
-              uint32_t key = 0, value = 0;
+              uint32_t key = 0;
 #pragma unroll
-              for (int i = 0; i < kSegParts / 32; ++i) {
-                const HeadBound p = a.seg_bound[h * kSegParts + 32 * i + lane];
-                key = max(key, p.key);
-                value = max(value, p.value);
-              }
+              for (int i = 0; i < kSegParts / 32; ++i) key = max(key, a.seg_bound[h * kSegParts + 32 * i + lane]);
               b.key = max(b.key, __reduce_max_sync(0xffffffffu, key));
-              b.value = max(b.value, __reduce_max_sync(0xffffffffu, value));
             }
             const uint32_t row = sbase + SM::q_off + ((warp & 3) * 32 + lane) * 128;
             float sq = 0.f;
@@ -656,11 +651,10 @@ attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CU
             // (1.001: the roundings of the norms, of the products' sums and of what follows; 1e-20: components whose squares are below the
             // smallest float)
             const float most = (sqrtf(sq) + 1e-20f) * ((sqrtf(__uint_as_float(b.key)) + 1e-20f) * scale * 1.001f) + log2f(static_cast<float>(max(b.count, 1)));
-            const float top = fmaxf(kTop, fminf(kFlatTop, kFlatSum - log2f(static_cast<float>(ns * 64)) - log2f(__uint_as_float(b.value))));
-            // what the rows' logits may be, less T, to where the maxima will be: nobody looks there yet, and it would not fit the registers
+            // what the rows' logits may be, less kTop, to where the maxima will be: nobody looks there yet, and it would not fit the registers
             float need[4];
 #pragma unroll
-            for (int q = 0; q < 4; ++q) need[q] = __shfl_sync(0xffffffffu, most, (lane >> 2) + 8 * q) - top;
+            for (int q = 0; q < 4; ++q) need[q] = __shfl_sync(0xffffffffu, most, (lane >> 2) + 8 * q) - kTop;
             if ((lane & 3) == 0) sts4(max_s, need);
           }
           mbar_arrive_warp(sbase + SM::bar_off + 8);

@@ -14,7 +14,6 @@
 // recomputed from the rounded mean inside this kernel instead of being copied from the representative token.
 #include <cuda_fp8.h>
 
-#include "bound.cuh"
 #include "common.h"
 #include "ptx.cuh"
 
@@ -219,7 +218,6 @@ __global__ void __launch_bounds__(kCommitThreads) commit_kernel(const CacheView 
         if (fr > best_f || (fr == best_f && s > best_s)) { best_f = fr; best_s = s; best_i = i; }
       }
     }
-    const uint32_t had = c.bound[h].value;
     const float inv = 1.f / static_cast<float>(m_old + g);
     uint4 krow;
     uint4 code8 = make_uint4(0u, 0u, 0u, 0u);
@@ -318,7 +316,6 @@ __global__ void __launch_bounds__(kCommitThreads) commit_kernel(const CacheView 
     vout.w = pack_bf16x2(acc[6] * inv, acc[7] * inv);
     *reinterpret_cast<uint4*>(c.pool_v + ro) = vout;
     *reinterpret_cast<uint4*>(c.pool_k + ro) = krow;
-    raise_bound(&c.bound[h].value, had, largest8(vout));
     if (c.pool_k8) store_code_part<LPR>(c, page, slot % c.PT, sl, code8);
     if (sl == 0) {
       c.count[sb + slot] = m_old + g;
@@ -332,7 +329,6 @@ __global__ void __launch_bounds__(kCommitThreads) commit_kernel(const CacheView 
     const int slot = FASTAR_IDX(c.dest[tb + i], c.CAP, c.status);
     const uint4 krow = *reinterpret_cast<const uint4*>(kh + i * ts + sl * 8);
     const uint4 vrow = *reinterpret_cast<const uint4*>(vh + i * ts + sl * 8);
-    const uint32_t had = c.bound[h].value;
     uint4 code8 = make_uint4(0u, 0u, 0u, 0u);
     if (c.pool_k8) code8 = load_code_part<LPR>(c, h, i, sl);
     float rn = 0.f;
@@ -345,7 +341,6 @@ __global__ void __launch_bounds__(kCommitThreads) commit_kernel(const CacheView 
     const int64_t ro = (static_cast<int64_t>(page) * c.PT + (slot % c.PT)) * c.D + sl * 8;
     *reinterpret_cast<uint4*>(c.pool_k + ro) = krow;
     *reinterpret_cast<uint4*>(c.pool_v + ro) = vrow;
-    raise_bound(&c.bound[h].value, had, largest8(vrow));
     if (c.pool_k8) store_code_part<LPR>(c, page, slot % c.PT, sl, code8);
     if (sl == 0) {
       c.count[sb + slot] = 1;

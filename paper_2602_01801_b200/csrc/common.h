@@ -25,13 +25,11 @@ struct PlanRec {          // per head, written by the planning kernel of an upda
   int32_t pad[2];
 };
 
-// What the rows of a head's slots do not exceed: bounds over all that came since the last reset, so they only rise.  The first two are words
-// of floats that are not negative, which are in the floats' order; one that is not finite, or no number, is above all that are.
+// What the rows of a head's slots do not exceed: bounds over all that came since the last reset, so they only rise.  The first is the word
+// of a float that is not negative, and these words are in the floats' order; one that is not finite, or no number, is above all that are.
 struct HeadBound {
   uint32_t key;           // |k|^2 (squares below the smallest float are not in it)
-  uint32_t value;         // |component of v|
   int32_t count;          // m
-  int32_t pad;
 };
 constexpr int kSegParts = 128;     // parts of the tokens of an un-cached segment whose bounds the attention puts together
 
@@ -110,7 +108,7 @@ struct CacheView {
   int sign_codes;                  // the search code rows hold LSH sign bits as +-1 (Hamming search) instead of fp8 directions
   int rep_mean;                    // representative key of a merged slot: 0 = newest key, 1 = count-weighted mean key
   float* seg_bias;                 // [max_tokens + 128]  bias of the rows of an un-cached attention segment
-  HeadBound* seg_bound;            // [H][kSegParts]  and what its rows do not exceed
+  uint32_t* seg_bound;             // [H][kSegParts]  and what |k|^2 of its rows does not exceed
   // AnnCA with the LSH bucket rule: codes of the queries and of the prompt keys, kept tokens per frame
   uint32_t* code_q_ca;             // [H][max_tokens]
   uint32_t* code_p_ca;             // [H][max_prompt]
@@ -210,7 +208,7 @@ struct AttnArgs {
   // rows (0 for a token, -inf past its end), seg_tiles * page_tokens floats
   int seg_tiles;
   const float* seg_bias;
-  const HeadBound* seg_bound;      // [H][kSegParts]
+  const uint32_t* seg_bound;       // [H][kSegParts]
   int np;                  // gather mode: prompt tokens (range of the kept indices)
   // gather mode: kept tokens of every frame, [H][keep_frames_stride] (nullptr: `keep` for all frames)
   const int32_t* keep_frames;
@@ -267,7 +265,7 @@ int launch_commit(const CacheView& c, const __nv_bfloat16* k_new, const __nv_bfl
                   int64_t hs, int64_t ts, cudaStream_t st);
 int launch_finalize_hist(const CacheView& c, fastar_update_stats* stats_out, int advance_clock, cudaStream_t st);
 struct SegArgs {           // an un-cached segment of an attention call
-  const __nv_bfloat16 *k, *v;
+  const __nv_bfloat16* k;
   int64_t hs, ts;
   int ns, total;           // its tokens, and the rows of its tiles
 };

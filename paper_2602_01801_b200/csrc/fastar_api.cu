@@ -206,7 +206,7 @@ size_t carve(const fastar_cache_desc& d, uint8_t* base, CacheView* v) {
   t.q8_probe = t.search_bits == 8 ? take(H * MT * 128) : nullptr;
   t.qn_probe = t.search_bits == 8 ? reinterpret_cast<float*>(take(H * MT * 4)) : nullptr;
   t.seg_bias = reinterpret_cast<float*>(take((MT + 128) * 4));
-  t.seg_bound = reinterpret_cast<HeadBound*>(take(H * kSegParts * sizeof(HeadBound)));
+  t.seg_bound = reinterpret_cast<uint32_t*>(take(H * kSegParts * 4));
   t.code_q_ca = reinterpret_cast<uint32_t*>(take(H * MT * 4));
   t.code_p_ca = reinterpret_cast<uint32_t*>(take(H * MP * 4));
   t.nselp = reinterpret_cast<int32_t*>(take(H * t.max_frames * 4));
@@ -741,7 +741,7 @@ static int annsa_impl(fastar_cache_t* c, const HeadRange& range, bool hashed, bo
     a.seg_tiles = (ns + v.PT - 1) / v.PT;
     a.seg_bias = v.seg_bias;
     a.seg_bound = v.seg_bound;
-    seg = SegArgs{sg[0].p, sg[1].p, sg[0].hs, sg[0].ts, ns, a.seg_tiles * v.PT};      // K and V alike
+    seg = SegArgs{sg[0].p, sg[0].hs, sg[0].ts, ns, a.seg_tiles * v.PT};
   }
   if (sel_in) {
     a.sel = sel_in;

@@ -1001,39 +1001,36 @@ int launch_finalize_hist(const CacheView& c, fastar_update_stats* stats_out, int
 }
 
 // ---------------------------------------------------------------------------------------------
-// An un-cached segment of an attention call: the biases of its rows, and what its keys and values do not exceed, by kSegParts parts of the
+// An un-cached segment of an attention call: the biases of its rows, and what |k|^2 of its keys does not exceed, by kSegParts parts of the
 // tokens of a head, which the attention puts together (so there is nothing to clear and no atomic).  Half a warp (a quarter at d = 64) has a row.
 // The parts are CTAs of 64 threads, on the SMs that the block top-k leaves idle where there is one (12 heads x 4680 tokens, with the top-k 3.9 + 8.5 -> 9.0 us).
 // ---------------------------------------------------------------------------------------------
 template <int D>
 __device__ __forceinline__ void segment_part(const CacheView& c, const SegArgs& s, int h, int part) {
   constexpr int LPR = D / 8, RPW = 32 / LPR, B = 4;    // lanes a row, rows a warp, rows of a thread that are under way
-  __shared__ HeadBound bound;
-  if (threadIdx.x == 0) bound = HeadBound{};
+  __shared__ uint32_t bound;
+  if (threadIdx.x == 0) bound = 0u;
   __syncthreads();
   const int sl = threadIdx.x % LPR, rpc = blockDim.x / LPR;
   for (int i = (h * kSegParts + part) * blockDim.x + threadIdx.x; i < s.total; i += c.H * kSegParts * blockDim.x) c.seg_bias[i] = i < s.ns ? 0.f : -INFINITY;
   const int r0 = static_cast<int>(static_cast<int64_t>(s.ns) * part / kSegParts), r1 = static_cast<int>(static_cast<int64_t>(s.ns) * (part + 1) / kSegParts);
-  uint32_t kmost = 0, vmost = 0;
+  uint32_t most = 0;
   for (int rb = r0 + (threadIdx.x >> 5) * RPW; rb < r1; rb += B * rpc) {
-    uint4 kr[B], vr[B];
+    uint4 kr[B];
 #pragma unroll
     for (int b = 0; b < B; ++b) {                      // past the end the last row again
       const int row = min(rb + b * rpc + static_cast<int>(threadIdx.x & 31) / LPR, r1 - 1);
       kr[b] = *reinterpret_cast<const uint4*>(s.k + h * s.hs + row * s.ts + sl * 8);
-      vr[b] = *reinterpret_cast<const uint4*>(s.v + h * s.hs + row * s.ts + sl * 8);
     }
 #pragma unroll
     for (int b = 0; b < B; ++b) {
-      vmost = max(vmost, largest8(vr[b]));
       float sq = square_sum8(kr[b], 0.f);
 #pragma unroll
       for (int o = LPR / 2; o >= 1; o >>= 1) sq += __shfl_xor_sync(0xffffffffu, sq, o);
-      kmost = max(kmost, __float_as_uint(sq));
+      most = max(most, __float_as_uint(sq));
     }
   }
-  raise_bound_warp(&bound.key, 0, kmost);
-  raise_bound_warp(&bound.value, 0, vmost);
+  raise_bound_warp(&bound, 0, most);
   __syncthreads();
   if (threadIdx.x == 0) c.seg_bound[h * kSegParts + part] = bound;
 }
@@ -1186,7 +1183,7 @@ __global__ void reset_meta_kernel(const CacheView c) {
     // does not hold stay at page 0, a valid address that only masked-out slots ever read)
     if (q < static_cast<int64_t>(c.H) * c.CAPB) c.page_table[q] = c.pool_shared ? 0 : static_cast<int32_t>(q);
     if (q < c.H) c.len[q] = 0;
-    if (q < c.H) c.bound[q] = HeadBound{0u, __float_as_uint(64.f), 0, 0};      // (ordinary values are below 64: an update raises nothing)
+    if (q < c.H) c.bound[q] = HeadBound{0u, 0};
     if (q == 0) { *c.now = 0; *c.status = 0; *c.next_free = 0; }
   }
 }
@@ -1207,13 +1204,10 @@ __global__ void import_fix_kernel(const CacheView c) {
   const int L = c.len[h];
   const int lane = threadIdx.x & 31;
   const int32_t* pt_h = c.page_table + static_cast<int64_t>(h) * c.CAPB;
-  uint32_t vmost = 0, cmost = 1;
+  int cmost = 1;
   for (int s = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); s < c.CAP; s += gridDim.x * (blockDim.x >> 5)) {
     const int64_t q = static_cast<int64_t>(h) * c.CAP + s;
-    if (s < L) {
-      vmost = max(vmost, largest8(*reinterpret_cast<const uint4*>(c.pool_v + slot_row_offset(c, pt_h, s) + (lane & (D / 8 - 1)) * 8)));
-      cmost = max(cmost, static_cast<uint32_t>(max(c.count[q], 1)));
-    }
+    if (s < L) cmost = max(cmost, c.count[q]);
     if (s >= L) {
       const int64_t ro = slot_row_offset(c, pt_h, s);
       for (int e = lane * 2; e < D; e += 64) {
@@ -1225,8 +1219,7 @@ __global__ void import_fix_kernel(const CacheView c) {
       c.log2m[q] = log2f(static_cast<float>(max(1, c.count[q])));
     }
   }
-  raise_bound_warp(&c.bound[h].value, 0, vmost);
-  if (lane == 0) atomicMax(&c.bound[h].count, static_cast<int>(cmost));
+  if (lane == 0) atomicMax(&c.bound[h].count, cmost);
 }
 int launch_import_derive(const CacheView& c, cudaStream_t st) {
   // codes and reciprocal norms of every slot (the pools are [H][CAP][D] under the identity page table)

@@ -347,3 +347,32 @@ def test_bounds_of_the_logits(d, pt, tiles):
     cache.update(dk[:, :cut], dv[:, :cut], n, 0.999)       # every key finds itself: multiplicities of two, the same mean values
     check(cache.annsa(dq, 128, cap // pt)["out"], np.broadcast_to(np.where(np.arange(n) < cut, 2, 1), (H, n)), but=5)      # (keys of zero find nothing)
     assert cache.status() == 0
+
+
+@pytest.mark.parametrize("d,pt", [(64, 64), (64, 128), (128, 64), (128, 128)])
+@pytest.mark.parametrize("size", [1.0, 1.5, 2.0, 4.0])
+def test_items_without_maxima_are_as_exact_as_with(d, pt, size):
+    """Keys in the order of their clusters, logits of `size` times the usual: a row's own cluster comes late, so where the maximum is looked for it
+    may be raised there, and a row's largest probability is a power of two behind a raise.  Looking for it is forced by one more key, of a norm that
+    no bound admits, against which every query has a logit of minus thousands: the error without that key is not larger than with it."""
+    import torch
+    from paper_2602_01801_b200 import fastar
+    g = torch.Generator(device="cuda").manual_seed(d + pt)
+    normal = lambda *shape: torch.randn(*shape, generator=g, device="cuda")
+    H, n, nq = 2, 4095, 512
+    centre = normal(H, 64, d) * math.sqrt(size)
+    k = centre[:, torch.arange(n + 1, device="cuda") * 64 // (n + 1)] + 0.5 * normal(H, n + 1, d)
+    q = centre[:, torch.randint(0, 64, (nq,), generator=g, device="cuda")] + 0.5 * normal(H, nq, d)
+    q[..., 0], k[..., 0] = 4.0, 0.0
+    k[:, n], k[:, n, 0] = 0.0, -(2.0 ** 20)
+    q, k, v = q.bfloat16(), k.bfloat16(), normal(H, n + 1, d).bfloat16()
+    want = torch.softmax(q.double() @ k[:, :n].double().mT / math.sqrt(d), -1) @ v[:, :n].double()
+    errors = []
+    for m in (n, n + 1):
+        cache = fastar.Cache(H, d, 4096, pt, np.random.default_rng(1).standard_normal((32, d)).astype(np.float32), max_tokens=n + 1)
+        cache.update(k[:, :m], v[:, :m], m, 2.0)
+        out = cache.annsa(q, 128, 4096 // pt)["out"].double()
+        assert cache.status() == 0
+        errors.append(float((out - want).norm() / want.norm()))
+    # the same probabilities up to the exponentials' 2e-7, which round to another bf16 number once in some ten thousand times
+    assert errors[0] <= 1.001 * errors[1]
