@@ -168,6 +168,13 @@ int fastar_cache_export_probe_codes(fastar_cache_t* cache, uint8_t* host_probe_c
 int fastar_cache_export_annca_codes(fastar_cache_t* cache, uint8_t* host_q_codes, uint8_t* host_prompt_codes,
                                     int32_t nq, int32_t np, void* stream);
 
+/* The bounds that AnnSA takes the logits by, of every key block's live slots: the largest |k|, host_norm
+ * [H][capacity/page_tokens] (infinite where a key is not finite), the largest log2 m, host_log2m, and the
+ * largest log2(e) |k| + log2 m, host_joint; zeros for a block without a live slot.  Copied to the host;
+ * synchronises the stream.  An update or an import writes them anew, so a key leaves them when it is
+ * evicted.  What they decide is speed, not results. */
+int fastar_cache_export_bounds(fastar_cache_t* cache, float* host_norm, float* host_log2m, float* host_joint, void* stream);
+
 /* Load a state (same layouts; count/stamp NULL = all ones / all zeros).  Slots >= len[h] are
  * cleared.  Derived per-slot data (1/|k|, log2 m, LSH codes, search codes, histograms) are recomputed on the
  * device.  `now` must exceed every stamp.  Synchronises the stream. */

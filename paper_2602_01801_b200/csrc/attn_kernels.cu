@@ -115,14 +115,17 @@ __device__ __forceinline__ float2 poly_exp2(float2 u) {
 __device__ __forceinline__ void add_bf16x2(float2& s, uint32_t b) {
   asm("{.reg .b16 l, h; mov.b32 {l, h}, %2; add.f32.bf16 %0, l, %0; add.f32.bf16 %1, h, %1;}" : "+f"(s.x), "+f"(s.y) : "r"(b));
 }
-// Flat items.  A logit is at most |q| max |k| / sqrt(d) + log2 max m; the cache keeps the largest of each head (HeadBound), a segment's come
-// with the call, and |q| is worked out here.  If that, for the rows of a warp, is not more than kTop above the reference that an item's first
-// sub-tile gives, nothing after it can ask for another reference: the sub-tiles that follow need no maximum, no look at the others' and no
-// hand-over, which are 160 of the loop's 440 instructions, and every probability is taken relative to what the loop that looks would take it.  (One reference for the four rows of a thread, within the biases, would spare 24
-// more and is 1 to 3 % faster, but then the largest probabilities no longer lie just below a power of two, where bf16 is finest: error against
-// 64 bits 0.00230 -> 0.00233.  Nor may the bound be further above: with 96, as far as fp32 sums bear, items stay flat in which the other loop
-// would have raised, and behind a raise the row's largest probability is a power of two.  Keys in the order of their clusters, logits of 1.5 to 4
-// times the usual size: 0.00209-0.00230 where the maximum is looked for, 0.00224-0.00233 so.)  Items of fewer sub-tiles than kFlatMin don't ask.
+// Flat items.  What a logit can be at most follows from |q| and from the bounds that the cache keeps for the blocks of an item (BlockBound) and
+// that come with a segment.  If that, for the rows of a warp, is not more than kTop above the reference that an item's first sub-tile gives,
+// nothing after it can ask for another reference: the sub-tiles that follow need no maximum, no look at the others' and no hand-over, which are
+// some 170 of the loop's 440 instructions, and every probability is taken relative to the same number as in the loop that looks.  (One reference
+// for the four rows of a thread, within the biases, would spare 24 more and is 1 to 3 % faster, but then the largest probabilities no longer
+// lie just below a power of two, where bf16 is finest: error against 64 bits 0.00230 -> 0.00233.  Nor may the bound be further above: with 96, as
+// far as fp32 sums bear, items stay flat in which the other loop would have raised, and behind a raise the row's largest probability is a power
+// of two.  Keys in the order of their clusters, logits of 1.5 to 4 times the usual size: 0.00209-0.00230 where the maximum is looked for,
+// 0.00224-0.00233 so.)  Items of fewer sub-tiles than kFlatMin don't ask.  The bounds are of the item's own blocks: where tokens have merged into
+// its slots thousands of times (12 heads, 8-bit search, m up to 2^10) 0.89 of the items are flat, by the bounds of a head 0.60, and if |k| and
+// m are bounded apart 0.01.
 constexpr int kFlatMin = 8;
 // Pairs of every sixteen whose exponentials the FMA units work out: the special-function units take 512 cycles for a sub-tile's, the tensor
 // core 270 at d = 64 and 540 at 128.  Kernel time with 0 / 2 / 4 of sixteen: d = 64, 256 items of 128 sub-tiles 97.9 / 94.1 / 95.0 us; d = 128, 256 of
@@ -154,6 +157,7 @@ struct AttnSmem {
   static constexpr int xchg_off = bias_off + NB * BKT * 4;       // [2][kGroups][128] (maximum, sum) of the groups' rows, by item
   static constexpr int max_off = xchg_off + 2 * kGroups * 1024;  // [4][8][4] running maxima: warp of the group, lane / 4, row / 8
   static constexpr int flat_off = max_off + 512;                 // [4] by warp of the group: the item is flat (see kFlatMin)
+  static constexpr int stat_off = flat_off + 16;                 // the bounds of an item's keys: |k|, log2 m, both, |k| of the segment
   static constexpr int bar_off = flat_off + 64;
   static constexpr int total = bar_off + 512;
   static constexpr int p_col = (QT ? 3 : kGroups) * 64, o_col = p_col + kGroups * 32, q_col = o_col + D;      // TMEM columns (S at 0)
@@ -304,11 +308,13 @@ attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CU
   const uint32_t bar_parts = bar_xchg + 24;          // [1] SPLIT: the warps that store parts are through
   const uint32_t bar_last = bar_xchg + 32;           // [1] SPLIT: last_s is there
   const uint32_t bar_qk_done = bar_xchg + 40;        // [1] Q K^T of an item is complete
-  constexpr int kNumBars = 2 + 2 * RS + 22;
+  const uint32_t bar_stat = bar_xchg + 48;           // [1] FLAT: the bounds of an item's keys are there
+  // and [4] FLAT, by warp of a group: the first sub-tile's maxima and what follows from them are there
+  constexpr int kNumBars = 2 + 2 * RS + 27;
   static_assert(kNumBars * 8 + 12 <= 512, "barrier area");
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smem_raw + SM::bar_off + kNumBars * 8);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(smem_raw + SM::bar_off + kNumBars * 8 + 4);
-  volatile int* done_flag = abort_flag + 1;          // stays 0: the wait for the soft-max warps at the end goes on after an abort
+  volatile int* done_flag = abort_flag + 1;          // stays 0: the waits that go on after an abort, for what every soft-max warp gets to
 
   const int warp = warp_index(), lane = threadIdx.x & 31;
   const int row_blocks = GATHER ? (a.rows_per_frame + 127) / 128 : (a.nq + a.block_q - 1) / a.block_q;
@@ -327,7 +333,7 @@ attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CU
 
   // one thread per barrier
   if (threadIdx.x < kNumBars) {
-    const int i = static_cast<int>(threadIdx.x) - (kNumBars - 22);        // s_full, pv_done, s_empty, p_full, xchg, o_free, done, parts, last, qk_done
+    const int i = static_cast<int>(threadIdx.x) - (kNumBars - 27);        // s_full, pv_done, s_empty, p_full, xchg, o_free, done, parts, last, qk_done, stat, looked
     mbar_init(bar + 8 * threadIdx.x, FLAT && threadIdx.x == 1 ? 5 : i >= 20 ? 1 : i == 19 ? 4 * (D / 32) : i >= 16 ? kSoftWarps : i >= 12 || (i >= 8 && SM::QT) ? 4 : i >= 8 ? 4 * SUB : i >= 4 || i < 0 ? 1 : 2);
     fence_mbar_init();
   }
@@ -402,7 +408,7 @@ attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CU
         // ================================================================ copies: Q, K and the biases, or V
         const bool is_k = warp == kKeyWarp;
         const uint32_t first = is_k ? 0 : RK, end = is_k ? RK : RS;
-        uint32_t st = first, empty_phase = 1, copied = 0, n_q = 0;
+        uint32_t st = first, empty_phase = 1, copied = 0, n_q = 0, n_stat = 0;
         bool ok = true;
         for (int it = it_first; more(it) && ok; it += it_step) {
           AttnItem w = item_of(item_at(it));
@@ -415,6 +421,33 @@ attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CU
           }
           const int nt = w.nt;
           if (nt == 0) continue;
+          // The bounds of the item's keys, by the warp that has the most time: the first tile of V is waited for later than Q and K.  They
+          // follow those of the item before once these have been read: a barrier's parity tells two phases apart, and V's ring may have room for
+          // all of an item.
+          if (FLAT && !is_k) {
+            if (n_stat > 0) ok = mbar_wait_warp<kIssueWaitHintNs>(bar_q_empty, (n_stat - 1) & 1, abort_flag, c.status);
+            if (!ok) break;
+            if (nt * SUB >= kFlatMin) {
+              float4 keys = make_float4(0.f, 0.f, 0.f, 0.f);      // |k|, log2 m, both, |k| of the segment
+              uint32_t seg = 0;
+              if (SEG)
+#pragma unroll
+                for (int i = 0; i < kSegParts / 32; ++i) seg = max(seg, a.seg_bound[w.h * kSegParts + 32 * i + lane]);
+#pragma unroll 2
+              for (int jj = lane; jj < min(w.ntc, nt); jj += 32) {
+                const int b = FASTAR_IDX(a.sel ? w.list[jj] : SPLIT ? static_cast<int>(reinterpret_cast<intptr_t>(w.list)) + jj : jj, c.CAPB, c.status);
+                const float4 x = *reinterpret_cast<const float4*>(c.bound + static_cast<int64_t>(w.h) * c.CAPB + b);
+                keys.x = fmaxf(keys.x, x.x);
+                keys.y = fmaxf(keys.y, x.y);
+                keys.z = fmaxf(keys.z, x.z);
+              }
+              auto most = [](float x) { return __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(x))); };      // (none is negative)
+              const float v[4] = {most(keys.x), most(keys.y), most(keys.z), sqrtf(most(__uint_as_float(seg)))};
+              if (lane == 0) sts4(sbase + SM::stat_off, v);
+            }
+            if (lane == 0) mbar_arrive(bar_stat);
+            ++n_stat;
+          }
           if (is_k) {
             if (n_q > 0) ok = mbar_wait_warp<kIssueWaitHintNs>(bar_q_empty, (n_q - 1) & 1, abort_flag, c.status);
             if (!ok) break;
@@ -628,18 +661,10 @@ attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CU
         // the logits' barriers: QT has one per group for their arrival (a barrier's parity tells two phases apart) and one per place for their leaving
         const uint32_t full = bar_s_full + 8 * (SM::QT ? g : g / SUB), empty = bar_s_empty + 8 * (SM::QT ? 0 : g / SUB);
         int t = (g - sub0) & (kGroups - 1);
-        bool flat = false, heard_it = false;
         if (FLAT && t == 0 && ns > 0) {
+          ok = ok && mbar_wait_warp(bar_s_full + 176, n_done & 1, abort_flag, c.status);      // the bounds of the item's keys
           if (ns >= kFlatMin) {
             ok = ok && mbar_wait_warp(sbase + SM::bar_off, n_done & 1, abort_flag, c.status);
-            const int h = item_at(it) / row_blocks % c.H;
-            HeadBound b = c.bound[h];
-            if (SEG) {
-              uint32_t key = 0;
-#pragma unroll
-              for (int i = 0; i < kSegParts / 32; ++i) key = max(key, a.seg_bound[h * kSegParts + 32 * i + lane]);
-              b.key = max(b.key, __reduce_max_sync(0xffffffffu, key));
-            }
             const uint32_t row = sbase + SM::q_off + ((warp & 3) * 32 + lane) * 128;
             float sq = 0.f;
 #pragma unroll
@@ -649,8 +674,12 @@ attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CU
               sq = square_sum8(v, sq);
             }
             // (1.001: the roundings of the norms, of the products' sums and of what follows; 1e-20: components whose squares are below the
-            // smallest float)
-            const float most = (sqrtf(sq) + 1e-20f) * ((sqrtf(__uint_as_float(b.key)) + 1e-20f) * scale * 1.001f) + log2f(static_cast<float>(max(b.count, 1)));
+            // smallest float.  Where q or a key is not finite, `apart` is not either, or no number, and so is the lesser of the two.)
+            const float4 keys = lds4(sbase + SM::stat_off);
+            const float y = (sqrtf(sq) + 1e-20f) * (scale * 1.001f), norm = keys.x + 1e-20f;
+            const float together = keys.z + fmaxf(y - kJoint, 0.f) * norm, apart = y * norm + keys.y;
+            float most = together < apart ? together : apart;
+            if (SEG) most = most >= y * (keys.w + 1e-20f) ? most : y * (keys.w + 1e-20f);
             // what the rows' logits may be, less kTop, to where the maxima will be: nobody looks there yet, and it would not fit the registers
             float need[4];
 #pragma unroll
@@ -659,17 +688,19 @@ attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CU
           }
           mbar_arrive_warp(sbase + SM::bar_off + 8);
         }
-        if (FLAT && ns >= kFlatMin && t > 0) {            // the first sub-tile's warp has said whether the item is flat
-          named_barrier_sync(heard, 64);
-          heard_it = true;
-          flat = lds1(flat_s) != 0.f;
-          if (flat) {
-            if (t + 1 < kGroups) named_barrier_arrive(told, 64);
+        const uint32_t looked = bar_s_full + 184 + 8 * (warp & 3);
+        bool looks = true;
+        if (FLAT && ns >= kFlatMin && t > 0) {            // the first sub-tile's warp says whether the item is flat
+          // (not given up with the other waits: all warps of the rows have to go the same way, and the one that says which gets there)
+          ok = mbar_wait_warp(looked, n_done & 1, done_flag, c.status, 2 * kWaitLimitNs) && ok;
+          looks = lds1(flat_s) == 0.f;
+          if (!looks) {
             const float4 ref = lds4(max_s);
             m[0] = ref.x; m[1] = ref.y; m[2] = ref.z; m[3] = ref.w;
           }
         }
-        for (; t < ns && !flat; t += kGroups) {
+        if (looks)                                        // (a condition of its own: in the loop's it costs a twentieth)
+        for (; t < ns; t += kGroups) {
           const int tg = sub0 + t, jg = tg / SUB;
           const uint32_t sb = SM::QT ? tg % SM::NSB : 0;
           if (!s_ready) ok = ok && mbar_wait_warp(full, (tg / kGroups) & 1, abort_flag, c.status);
@@ -683,8 +714,7 @@ attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CU
           float2 bias[8];
 #pragma unroll
           for (int k = 0; k < 8; ++k) bias[k] = lds2(bp + 32 * k);
-          if (t > 0 && !heard_it) named_barrier_sync(heard, 64);
-          heard_it = false;
+          if (t > 0) named_barrier_sync(heard, 64);
           const float4 seen = t > 0 ? lds4(max_s) : make_float4(-INFINITY, -INFINITY, -INFINITY, -INFINITY);
           bool p_free = tg < kGroups || mbar_test_wait(bar_pv_done + 8 * g, (tg / kGroups - 1) & 1);
           tmem_wait_ld();
@@ -739,10 +769,13 @@ attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CU
               }
               m[q] = top;
             }
-            if (FLAT && t == 0 && ns >= kFlatMin) {
-              const float4 need = lds4(max_s);
-              flat = need.x <= m[0] && need.y <= m[1] && need.z <= m[2] && need.w <= m[3] && fminf(fminf(m[0], m[1]), fminf(m[2], m[3])) > -INFINITY;
-              flat = __all_sync(0xffffffffu, flat);
+            bool flat = false;
+            if (FLAT && t == 0) {
+              if (ns >= kFlatMin) {
+                const float4 need = lds4(max_s);
+                flat = need.x <= m[0] && need.y <= m[1] && need.z <= m[2] && need.w <= m[3] && fminf(fminf(m[0], m[1]), fminf(m[2], m[3])) > -INFINITY;
+                flat = __all_sync(0xffffffffu, flat);
+              }
               if (lane == 0) asm volatile("st.shared.f32 [%0], %1;" ::"r"(flat_s), "f"(flat ? 1.f : 0.f) : "memory");
             }
             if (__any_sync(0xffffffffu, raised)) {
@@ -770,7 +803,9 @@ attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CU
               }
               if ((lane & 3) == 0) sts4(max_s, m);
               __syncwarp();
+              if (FLAT && t == 0) mbar_arrive_warp(looked);
             }
+            if (flat) may = false;                         // nobody hands on in a flat item
           }
           if (may && t + 1 < ns) named_barrier_arrive(told, 64);
           // P is free once P V of the group's last sub-tile has read it
@@ -801,6 +836,10 @@ attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CU
           tc_fence_before();
           mbar_arrive_warp(bar_p_full + 8 * g);
           s_ready = __all_sync(0xffffffffu, s_ready);
+          if (FLAT && t == 0 && lds1(flat_s) != 0.f) {
+            t += kGroups;
+            break;
+          }
         }
         if (FLAT) {
           const float2 scale2 = make_float2(scale, scale);
@@ -866,7 +905,8 @@ attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CU
                            : "memory");
           }
           mbar_arrive_warp(bar_xchg);
-          ok = mbar_wait_warp(bar_xchg, n_done & 1, abort_flag, c.status) && ok;
+          // (nor is this given up with the others: after a time-out too the warps go from item to item together)
+          ok = mbar_wait_warp(bar_xchg, n_done & 1, done_flag, c.status, 2 * kWaitLimitNs) && ok;
           tc_fence_after();
         }
         const int r = (warp & 3) * 32 + lane;         // from here on a thread owns one row, 32 of its columns

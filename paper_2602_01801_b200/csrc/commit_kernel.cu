@@ -243,7 +243,6 @@ __global__ void __launch_bounds__(kCommitThreads) commit_kernel(const CacheView 
 #pragma unroll
       for (int o = LPR / 2; o >= 1; o >>= 1) ss += __shfl_xor_sync(mask, ss, o);
       rn = ss > 0.f ? 1.f / sqrtf(ss) : 0.f;
-      if (__float_as_uint(ss) > c.bound[h].key) atomicMax(&c.bound[h].key, __float_as_uint(ss));      // (rounding may lift a mean above the keys)
       // sign-random-projection code: bit u of table t = [<k, R[t*B + u]> > 0].  Every lane forms its part of all 32
       // projections, then a reduce-scatter over the row's lanes (each step halves the values a lane keeps) leaves
       // 32 / LPR complete sums per lane: 30 shuffles instead of 128.

@@ -25,12 +25,16 @@ struct PlanRec {          // per head, written by the planning kernel of an upda
   int32_t pad[2];
 };
 
-// What the rows of a head's slots do not exceed: bounds over all that came since the last reset, so they only rise.  The first is the word
-// of a float that is not negative, and these words are in the floats' order; one that is not finite, or no number, is above all that are.
-struct HeadBound {
-  uint32_t key;           // |k|^2 (squares below the smallest float are not in it)
-  int32_t count;          // m
+// What the live slots of a key block do not exceed, written by the last kernel of every update.  Infinite where a key is not finite.
+struct BlockBound {
+  float norm;             // |k| (0 where the squares are below the smallest float)
+  float log2m;
+  float joint;            // kJoint |k| + log2 m
+  float pad;
 };
+// A logit, in binary orders, is at most a |k| + log2 m with a = |q| log2(e) / sqrt(d), and the longest key is hardly the one that most tokens have
+// merged into.  kJoint is a for |q| = sqrt(d); for a beyond it a |k| + log2 m is at most joint + (a - kJoint) norm.
+constexpr float kJoint = 1.4426950408889634f;
 constexpr int kSegParts = 128;     // parts of the tokens of an un-cached segment whose bounds the attention puts together
 
 struct CacheView {
@@ -54,7 +58,7 @@ struct CacheView {
   uint32_t* kcode;                 // [H][CAP]   table t in byte t
   __nv_bfloat16* hk;               // [H][CAPB][hist_cols]
   int32_t* len;                    // [H]
-  HeadBound* bound;                // [H]
+  BlockBound* bound;               // [H][CAPB]
   int32_t* now;                    // [1]
   int32_t* status;                 // [1]
   __nv_bfloat16* lsh;              // [T*B][D]

@@ -145,7 +145,7 @@ size_t carve(const fastar_cache_desc& d, uint8_t* base, CacheView* v) {
   t.kcode = reinterpret_cast<uint32_t*>(take(H * CAP * 4));
   t.hk = reinterpret_cast<__nv_bfloat16*>(take(H * t.CAPB * t.hist_cols * 2));
   t.len = reinterpret_cast<int32_t*>(take(H * 4));
-  t.bound = reinterpret_cast<HeadBound*>(take(H * sizeof(HeadBound)));
+  t.bound = reinterpret_cast<BlockBound*>(take(H * t.CAPB * sizeof(BlockBound)));
   t.now = reinterpret_cast<int32_t*>(take(4));
   t.status = reinterpret_cast<int32_t*>(take(4));
   t.lsh = reinterpret_cast<__nv_bfloat16*>(take(32 * D * 2));
@@ -257,7 +257,7 @@ int make_range(fastar_cache* c, int h0, int count, HeadRange* out) {
   v.count += cap; v.stamp += cap; v.log2m += cap; v.rnorm += cap; v.kcode += cap; v.cnt += cap; v.cur += cap;
   v.hk += h * v.CAPB * v.hist_cols;
   v.len += h;
-  v.bound += h;
+  v.bound += h * v.CAPB;
   v.seg_bound += h * kSegParts;
   v.best += mt; v.segslot += mt; v.ulist += mt; v.rnorm_new += mt; v.code_new += mt; v.match += mt; v.sim += mt; v.order += mt;
   v.dest += mt; v.victims += mt; v.code_q_ca += mt; v.code_q_sa += mt;
@@ -543,6 +543,22 @@ int fastar_cache_export_probe_codes(fastar_cache_t* c, uint8_t* host_probe_codes
                               static_cast<size_t>(n) * 128, v.H, cudaMemcpyDeviceToHost, st) == cudaSuccess;
   ok &= cudaStreamSynchronize(st) == cudaSuccess;
   return ok ? FASTAR_OK : FASTAR_ERR_CUDA;
+}
+
+int fastar_cache_export_bounds(fastar_cache_t* c, float* host_norm, float* host_log2m, float* host_joint, void* stream) {
+  if (!c || !host_norm || !host_log2m || !host_joint) return FASTAR_ERR_INVALID_ARG;
+  DeviceGuard guard(c->desc.device);
+  cudaStream_t st = static_cast<cudaStream_t>(stream);
+  const CacheView& v = c->v;
+  std::vector<BlockBound> b(static_cast<size_t>(v.H) * v.CAPB);
+  if (cudaMemcpyAsync(b.data(), v.bound, b.size() * sizeof(BlockBound), cudaMemcpyDeviceToHost, st) != cudaSuccess || cudaStreamSynchronize(st) != cudaSuccess)
+    return FASTAR_ERR_CUDA;
+  for (int i = 0; i < v.H * v.CAPB; ++i) {
+    host_norm[i] = b[i].norm;
+    host_log2m[i] = b[i].log2m;
+    host_joint[i] = b[i].joint;
+  }
+  return FASTAR_OK;
 }
 
 int fastar_cache_export_annca_codes(fastar_cache_t* c, uint8_t* host_q_codes, uint8_t* host_prompt_codes, int32_t nq, int32_t np,

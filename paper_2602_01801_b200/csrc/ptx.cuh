@@ -150,8 +150,9 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatil
 
 // The same wait by a whole converged warp: a warp-uniform answer, so that the code behind it stays converged.
 template <uint32_t HINT_NS = 0>
-__device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity, volatile int* abort_flag, int* status) {
-  return __all_sync(0xffffffffu, mbar_wait<HINT_NS>(bar, parity, abort_flag, status));
+__device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity, volatile int* abort_flag, int* status,
+                                               uint64_t limit_ns = kWaitLimitNs) {
+  return __all_sync(0xffffffffu, mbar_wait<HINT_NS>(bar, parity, abort_flag, status, limit_ns));
 }
 
 // ---------------------------------------------------------------------------------------------

@@ -128,7 +128,7 @@ template <int D, int ROWS, bool F32>
 __global__ void __launch_bounds__(256, 2) prep_kernel(const __nv_bfloat16* __restrict__ x, int H, int n, int64_t hs, int64_t ts,
                                                    const __nv_bfloat16* __restrict__ lsh, int T, int B,
                                                    uint32_t* __restrict__ code_out, float* __restrict__ rnorm_out,
-                                                   int64_t out_stride, HeadBound* bound, UpdateScratch clear, BlockHist bh, const ConvertArgs conv) {
+                                                   int64_t out_stride, UpdateScratch clear, BlockHist bh, const ConvertArgs conv) {
   constexpr bool BLOCKS = ROWS > 0;
   constexpr int per_block = BLOCKS ? ROWS / 16 : 1, blocks_a_pass = BLOCKS ? 8 / per_block : 1;
   __shared__ __align__(16) int hist[BLOCKS ? 2 : 1][blocks_a_pass][BLOCKS ? 1024 : 4];      // [pass & 1][block of the pass]
@@ -216,7 +216,6 @@ __global__ void __launch_bounds__(256, 2) prep_kernel(const __nv_bfloat16* __res
     const int h = grp / groups_per_head;
     const int r0 = (grp - h * groups_per_head) * 16;
     const bool more = grp + stride < total_groups;
-    const uint32_t had = !BLOCKS && bound ? bound[h].key : 0xFFFFFFFFu;
     if (more) rows(grp + stride);
     if (!BLOCKS || grp < total_groups) {         // (the last pass may have a block less)
       float acc[4][4];
@@ -262,7 +261,6 @@ __global__ void __launch_bounds__(256, 2) prep_kernel(const __nv_bfloat16* __res
         sqa += __shfl_xor_sync(0xffffffffu, sqa, o);
         sqb += __shfl_xor_sync(0xffffffffu, sqb, o);
       }
-      if (!BLOCKS && bound) raise_bound_warp(&bound[h].key, had, max(__float_as_uint(sqa), __float_as_uint(sqb)));
       uint32_t ca = 0, cb = 0;
       for (int tt = 0; tt < T; ++tt) {
         ca |= ((ma >> (tt * B)) & ((1u << B) - 1u)) << (8 * tt);
@@ -309,7 +307,6 @@ static int launch_prep_generic(const CacheView& c, const __nv_bfloat16* x, int n
                                float* rnorm_out, int64_t out_stride, cudaStream_t st, const UpdateScratch& clear = UpdateScratch{},
                                const ConvertArgs& conv = ConvertArgs{}) {
   if (n <= 0) return 0;
-  HeadBound* bound = rnorm_out ? c.bound : nullptr;               // cached keys, or keys that will be
   const int groups = ((n + 15) / 16) * c.H;                      // 16 rows per warp pass
   // CTAs for the rows (eight warps of 16 a pass) or for the zeros (32 KB each), whichever needs more: a few tokens against many heads
   // with long caches leave far more to clear than to hash (40 heads x 65536 slots, 1 to 16 tokens: an update of 81 us with CTAs for
@@ -318,7 +315,7 @@ static int launch_prep_generic(const CacheView& c, const __nv_bfloat16* x, int n
   if (conv.count > 1) want = max(want, static_cast<int64_t>(conv.count - 1) * c.H * n * c.D / 4 / 256);      // four numbers a thread
   const dim3 grid(static_cast<unsigned>(max(static_cast<int64_t>(1), min(want, static_cast<int64_t>(2 * 148)))));
   auto launch = [&](auto kernel) {
-    launch_chained(kernel, grid, 256, 0, st, x, c.H, n, hs, ts, c.lsh, c.T, c.B, code_out, rnorm_out, out_stride, bound, clear, BlockHist{}, conv);
+    launch_chained(kernel, grid, 256, 0, st, x, c.H, n, hs, ts, c.lsh, c.T, c.B, code_out, rnorm_out, out_stride, clear, BlockHist{}, conv);
   };
   if (c.D == 128) conv.count > 0 ? launch(prep_kernel<128, 0, true>) : launch(prep_kernel<128, 0, false>);
   else conv.count > 0 ? launch(prep_kernel<64, 0, true>) : launch(prep_kernel<64, 0, false>);
@@ -330,7 +327,7 @@ int launch_query_blocks(const CacheView& c, const __nv_bfloat16* q, int nq, int6
   const int64_t groups = static_cast<int64_t>((nq + block_q - 1) / block_q) * c.H * (block_q / 16);
   const int grid = static_cast<int>(min((groups + 7) / 8, static_cast<int64_t>(2 * 148)));
   auto launch = [&](auto kernel) {
-    launch_chained(kernel, grid, 256, 0, st, q, c.H, nq, hs, ts, c.lsh, c.T, c.B, c.code_q_sa, nullptr, c.max_tokens, nullptr, UpdateScratch{}, BlockHist{c.hq, c.max_qb, c.hist_cols}, conv);
+    launch_chained(kernel, grid, 256, 0, st, q, c.H, nq, hs, ts, c.lsh, c.T, c.B, c.code_q_sa, nullptr, c.max_tokens, UpdateScratch{}, BlockHist{c.hq, c.max_qb, c.hist_cols}, conv);
   };
   if (conv.count > 0) {
     if (c.D == 128) block_q == 128 ? launch(prep_kernel<128, 128, true>) : launch(prep_kernel<128, 64, true>);
@@ -944,24 +941,55 @@ int launch_plan(const CacheView& c, int n, float tau, const UpdateOut& out, cuda
 // One CTA of 128 threads per block: a slot per thread, then 16 bytes of the histogram per thread.  A block's row is 2 KB of bf16 for
 // at most 128 codes, so what bounds it is writing the rows (40 heads x 512 blocks: 42 MB, 6.4 us) and the CTAs' starts; with 2-byte
 // stores by 256 threads 39 -> 29 us, 12 heads x 256 blocks 6.8 -> 5.5.
-__global__ void __launch_bounds__(128) key_hist_kernel(const CacheView c, int use_plan, fastar_update_stats* stats_out,
+// It has every live slot in hand, so the bounds of a block's keys and multiplicities come from here: exact, and gone with the slot that set them.
+// (Bounds of a head that only rise, where keys and counts are written, would keep it out of the attention's flat items long after the eviction of
+// a key far longer than the rest, and m would be bounded by all that ever matched.)  12 heads x 256 blocks 5.8 -> 6.3 us, 40 x 512 30 -> 35, of
+// which the hash and the commit, which raised them, have lost 1.1 and 7; by atomics into one place per head it took 7.3 to 50.
+// A key without a reciprocal norm: |k|^2 is zero (or below the smallest float), infinite or no number.
+__device__ __forceinline__ bool key_is_zero(const __nv_bfloat16* k, int D) {
+  float sq = 0.f;
+#pragma unroll 1
+  for (int e = 0; e < D; e += 8) sq = square_sum8(*reinterpret_cast<const uint4*>(k + e), sq);
+  return sq <= 0.f;
+}
+__global__ void __launch_bounds__(128, 16) key_hist_kernel(const CacheView c, int use_plan, fastar_update_stats* stats_out,
                                                        int advance_clock) {
   chain_wait();
   extern __shared__ __align__(16) int hist[];          // hist_cols counters, a multiple of 64
+  __shared__ uint3 bound_s[4];
   const int b = blockIdx.x, h = blockIdx.y;
   const int L = use_plan ? c.plan[h].len_new : c.len[h];
   for (int q = threadIdx.x; q < c.hist_cols / 4; q += blockDim.x) reinterpret_cast<int4*>(hist)[q] = make_int4(0, 0, 0, 0);
   __syncthreads();
   const int s0 = b * c.PT, s1 = min(L, s0 + c.PT);
   const int nb = 1 << c.B;
+  float norm = 0.f, log2m = 0.f, joint = 0.f;          // the largest of the slots
   // weighted histograms (a selector option): a slot counts m times, as its merged tokens would; an entry saturates
   // at 65535 and is stored as two 8-bit digits, each exact in bf16, that S3 contracts separately
   for (int s = s0 + threadIdx.x; s < s1; s += blockDim.x) {
-    const uint32_t code = c.kcode[static_cast<int64_t>(h) * c.CAP + s];
-    const int wgt = c.hist_weighted ? min(c.count[static_cast<int64_t>(h) * c.CAP + s], 65535) : 1;
+    const int64_t q = static_cast<int64_t>(h) * c.CAP + s;
+    const uint32_t code = c.kcode[q];
+    const float rn = c.rnorm[q];
+    const int wgt = c.hist_weighted ? min(c.count[q], 65535) : 1;
+    const float lm = c.log2m[q];
+    float x = __fdividef(1.f, rn);
+    if (rn == 0.f && key_is_zero(c.pool_k + slot_row_offset(c, c.page_table + static_cast<int64_t>(h) * c.CAPB, s), c.D)) x = 0.f;
+    norm = fmaxf(norm, x);
+    log2m = fmaxf(log2m, lm);
+    joint = fmaxf(joint, fmaf(kJoint, x, lm));
     for (int t = 0; t < c.T; ++t) atomicAdd(&hist[t * nb + ((code >> (8 * t)) & 0xFFu)], wgt);
   }
+  // (none is negative, so their words are in the floats' order)
+  const uint32_t norm_w = __reduce_max_sync(0xffffffffu, __float_as_uint(norm)), log2m_w = __reduce_max_sync(0xffffffffu, __float_as_uint(log2m));
+  const uint32_t joint_w = __reduce_max_sync(0xffffffffu, __float_as_uint(joint));
+  if ((threadIdx.x & 31) == 0) bound_s[threadIdx.x >> 5] = make_uint3(norm_w, log2m_w, joint_w);
   __syncthreads();
+  if (threadIdx.x == 0) {
+    uint3 w = bound_s[0];
+#pragma unroll
+    for (int i = 1; i < 4; ++i) w = make_uint3(max(w.x, bound_s[i].x), max(w.y, bound_s[i].y), max(w.z, bound_s[i].z));
+    c.bound[static_cast<int64_t>(h) * c.CAPB + b] = BlockBound{__uint_as_float(w.x), __uint_as_float(w.y), __uint_as_float(w.z), 0.f};
+  }
   const int64_t ho = (static_cast<int64_t>(h) * c.CAPB + b) * c.hist_cols;
   for (int q = threadIdx.x; q < c.hist_cols / 8; q += blockDim.x) {
     int v[8];
@@ -977,7 +1005,6 @@ __global__ void __launch_bounds__(128) key_hist_kernel(const CacheView c, int us
   if (b == 0 && threadIdx.x == 0 && use_plan) {
     const PlanRec pr = c.plan[h];
     c.len[h] = pr.len_new;
-    c.bound[h].count = min(max(c.bound[h].count, 1) + pr.n_matched, 1 << 30);          // a slot of m takes no more than all that matched
     if (c.pool_shared && pr.pages_granted > 0) atomicAdd(c.next_free, pr.pages_granted);
     if (stats_out) {
       fastar_update_stats s;
@@ -1030,7 +1057,8 @@ __device__ __forceinline__ void segment_part(const CacheView& c, const SegArgs& 
       most = max(most, __float_as_uint(sq));
     }
   }
-  raise_bound_warp(&bound, 0, most);
+  most = __reduce_max_sync(0xffffffffu, most);
+  if ((threadIdx.x & 31) == 0) atomicMax(&bound, most);
   __syncthreads();
   if (threadIdx.x == 0) c.seg_bound[h * kSegParts + part] = bound;
 }
@@ -1181,9 +1209,9 @@ __global__ void reset_meta_kernel(const CacheView c) {
     c.kcode[q] = 0;
     // one full set of pages per head: the identity; a shared pool: no page handed out yet (entries of pages a head
     // does not hold stay at page 0, a valid address that only masked-out slots ever read)
+    if (q < static_cast<int64_t>(c.H) * c.CAPB) c.bound[q] = BlockBound{};
     if (q < static_cast<int64_t>(c.H) * c.CAPB) c.page_table[q] = c.pool_shared ? 0 : static_cast<int32_t>(q);
     if (q < c.H) c.len[q] = 0;
-    if (q < c.H) c.bound[q] = HeadBound{0u, 0};
     if (q == 0) { *c.now = 0; *c.status = 0; *c.next_free = 0; }
   }
 }
@@ -1204,10 +1232,8 @@ __global__ void import_fix_kernel(const CacheView c) {
   const int L = c.len[h];
   const int lane = threadIdx.x & 31;
   const int32_t* pt_h = c.page_table + static_cast<int64_t>(h) * c.CAPB;
-  int cmost = 1;
   for (int s = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); s < c.CAP; s += gridDim.x * (blockDim.x >> 5)) {
     const int64_t q = static_cast<int64_t>(h) * c.CAP + s;
-    if (s < L) cmost = max(cmost, c.count[q]);
     if (s >= L) {
       const int64_t ro = slot_row_offset(c, pt_h, s);
       for (int e = lane * 2; e < D; e += 64) {
@@ -1219,7 +1245,6 @@ __global__ void import_fix_kernel(const CacheView c) {
       c.log2m[q] = log2f(static_cast<float>(max(1, c.count[q])));
     }
   }
-  if (lane == 0) atomicMax(&c.bound[h].count, cmost);
 }
 int launch_import_derive(const CacheView& c, cudaStream_t st) {
   // codes and reciprocal norms of every slot (the pools are [H][CAP][D] under the identity page table)

@@ -47,6 +47,7 @@ SIGNATURES = {
     "fastar_cache_export_search_codes": (C.c_int, [_vp, _vp, _vp, _i32, _vp]),
     "fastar_cache_export_probe_codes": (C.c_int, [_vp, _vp, _i32, _vp]),
     "fastar_cache_export_annca_codes": (C.c_int, [_vp, _vp, _vp, _i32, _i32, _vp]),
+    "fastar_cache_export_bounds": (C.c_int, [_vp, _vp, _vp, _vp, _vp]),
     "fastar_cache_import": (C.c_int, [_vp, _vp, _vp, _vp, _vp, _vp, _i32, _vp]),
     "fastar_tempcache_update": (C.c_int, [_vp, _vp, _vp, _i32, _i32, _i64, _i64, _f32, _vp, _vp, _vp, _vp, _vp]),
     "fastar_tempcache_update_probe": (C.c_int, [_vp, _vp, _vp, _vp, _i32, _i32, _i64, _i64, _f32, _vp, _vp, _vp, _vp, _vp]),
@@ -223,6 +224,14 @@ class Cache:
         with self.torch.cuda.device(self.device):
             _check(self.lib.fastar_cache_export_annca_codes(self.handle, out["q"].ctypes.data, out["prompt"].ctypes.data, nq,
                                                             n_prompt, _stream()), "fastar_cache_export_annca_codes")
+        return out
+
+    def export_bounds(self) -> Dict[str, np.ndarray]:
+        """The largest |k|, log2 m and log2(e) |k| + log2 m of the live slots of every key block, by which AnnSA bounds its logits; [H][blocks] each."""
+        out = {x: np.empty((self.H, self.CAP // self.PT), np.float32) for x in ("norm", "log2m", "joint")}
+        with self.torch.cuda.device(self.device):
+            _check(self.lib.fastar_cache_export_bounds(self.handle, out["norm"].ctypes.data, out["log2m"].ctypes.data, out["joint"].ctypes.data,
+                                                       _stream()), "fastar_cache_export_bounds")
         return out
 
     def import_state(self, k_bits: np.ndarray, v_bits: np.ndarray, length: np.ndarray, count: Optional[np.ndarray] = None,

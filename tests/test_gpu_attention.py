@@ -294,7 +294,7 @@ def test_items_of_caches_that_are_not_full(d, pt, H, nqb, tiles, lens, seg):
 @pytest.mark.parametrize("d,pt", [(64, 64), (64, 128), (128, 64), (128, 128)])
 @pytest.mark.parametrize("tiles", [7, 8, 9, 21])
 def test_bounds_of_the_logits(d, pt, tiles):
-    """Heads whose largest norms, values and multiplicities bound every logit near an item's first ones, and heads where they do not: a last key
+    """Heads whose largest norms and multiplicities bound every logit near an item's first ones, and heads where they do not: a last key
     that towers over the others, values near the end of bf16's range, rows of very unequal norms, keys and values of zero.  The same for keys
     that came by updates, by an import, and as a segment."""
     import torch
@@ -376,3 +376,47 @@ def test_items_without_maxima_are_as_exact_as_with(d, pt, size):
         errors.append(float((out - want).norm() / want.norm()))
     # the same probabilities up to the exponentials' 2e-7, which round to another bf16 number once in some ten thousand times
     assert errors[0] <= 1.001 * errors[1]
+
+
+@pytest.mark.parametrize("d,pt", [(64, 64), (64, 128), (128, 64), (128, 128)])
+@pytest.mark.parametrize("source", ["import", "update", "merge", "segment"])
+def test_a_late_key_that_only_its_bound_gives_away(d, pt, source):
+    """One key, behind all others, 200 binary orders above the first logits: without its bound the item would not look for a maximum, and the
+    exponential would leave fp32's range.  The key comes by an import, by a second update, by a merge (in the place of a short key of its
+    direction), or with a segment."""
+    import torch
+    from paper_2602_01801_b200 import fastar
+    rng = np.random.default_rng(d + pt)
+    H, n, nq = 2, 13 * 64, 200
+    order = math.sqrt(d) / math.log2(math.e) / 8.0         # q = 8 e0: so much of a key's first component is one binary order
+    q = 0.01 * rng.standard_normal((H, nq, d))
+    q[:, :, 0] = 8.0
+    k, v = 0.3 * rng.standard_normal((H, n, d)), rng.standard_normal((H, n, d))
+    k[:, :, 0] = rng.uniform(-0.5, 0.5, (H, n)) * order
+    k[:, n - 1] = 0.0
+    k[:, n - 1, 0] = 200.0 * order
+    q, k, v = (synth.round_bf16(x.astype(np.float32)) for x in (q, k, v))
+    assert (8.0 * k[:, n - 1, 0] / math.sqrt(d) * math.log2(math.e) > 150.0).all()        # 2^150 and more, relative to the others
+    cap = n + 192
+    cache = fastar.Cache(H, d, cap // 128 * 128, pt, rng.standard_normal((32, d)).astype(np.float32), max_tokens=n)
+    dk, dv, blocks = fastar.to_device(k), fastar.to_device(v), cap // 128 * 128 // pt
+    if source == "import":
+        cache.import_state(fastar.bf16_bits(k), fastar.bf16_bits(v), np.full(H, n))
+    elif source == "merge":
+        short = k.copy()
+        short[:, n - 1, 0] = 1.0
+        cache.update(fastar.to_device(short), dv, n, 2.0)
+        assert (cache.update(dk[:, n - 64:], dv[:, n - 64:], 64, 0.999)["match"] >= 0).all()
+    else:
+        cache.update(dk[:, :n - 64], dv[:, :n - 64], n, 2.0)
+        if source == "update":
+            cache.update(dk[:, n - 64:], dv[:, n - 64:], 64, 2.0)
+    if source == "segment":
+        out = cache.annsa_segment(fastar.to_device(q), dk[:, n - 64:], dv[:, n - 64:], 128, blocks)["out"]
+    else:
+        out = cache.annsa(fastar.to_device(q), 128, blocks)["out"]
+    assert cache.status() == 0
+    out = out.float().cpu().numpy()
+    assert np.isfinite(out).all()
+    # nothing else has any weight (2^-150), and a mean of equal values is that value
+    assert np.array_equal(out, np.broadcast_to(v[:, n - 1:], out.shape))
