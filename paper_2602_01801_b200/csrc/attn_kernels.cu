@@ -689,18 +689,21 @@ attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CU
           mbar_arrive_warp(sbase + SM::bar_off + 8);
         }
         const uint32_t looked = bar_s_full + 184 + 8 * (warp & 3);
-        bool looks = true;
+        bool flat = false;
         if (FLAT && ns >= kFlatMin && t > 0) {            // the first sub-tile's warp says whether the item is flat
           // (not given up with the other waits: all warps of the rows have to go the same way, and the one that says which gets there)
           ok = mbar_wait_warp(looked, n_done & 1, done_flag, c.status, 2 * kWaitLimitNs) && ok;
-          looks = lds1(flat_s) == 0.f;
-          if (!looks) {
+          flat = lds1(flat_s) != 0.f;
+          if (flat) {
             const float4 ref = lds4(max_s);
             m[0] = ref.x; m[1] = ref.y; m[2] = ref.z; m[3] = ref.w;
           }
         }
-        if (looks)                                        // (a condition of its own: in the loop's it costs a twentieth)
-        for (; t < ns; t += kGroups) {
+        // A sub-tile whose maximum is looked for.  An item's first one is code of its own: inside the loop, what only it does took a twentieth of the
+        // loop's time.  Items that all look, before there were flat ones, with that in the loop, now: 12 heads x 4680 queries on 32 of 220 blocks
+        // 103-105, 110, 105 us, 8 x 4096 on 16384 keys 228, 240, 225, d = 64, 64 of 1 024 blocks 116, 124, 117.
+        auto look = [&](auto way) {
+          constexpr bool FIRST = decltype(way)::value;
           const int tg = sub0 + t, jg = tg / SUB;
           const uint32_t sb = SM::QT ? tg % SM::NSB : 0;
           if (!s_ready) ok = ok && mbar_wait_warp(full, (tg / kGroups) & 1, abort_flag, c.status);
@@ -714,8 +717,8 @@ attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CU
           float2 bias[8];
 #pragma unroll
           for (int k = 0; k < 8; ++k) bias[k] = lds2(bp + 32 * k);
-          if (t > 0) named_barrier_sync(heard, 64);
-          const float4 seen = t > 0 ? lds4(max_s) : make_float4(-INFINITY, -INFINITY, -INFINITY, -INFINITY);
+          if (!FIRST) named_barrier_sync(heard, 64);
+          const float4 seen = FIRST ? make_float4(-INFINITY, -INFINITY, -INFINITY, -INFINITY) : lds4(max_s);
           bool p_free = tg < kGroups || mbar_test_wait(bar_pv_done + 8 * g, (tg / kGroups - 1) & 1);
           tmem_wait_ld();
           tc_fence_before();
@@ -737,18 +740,20 @@ attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CU
           // raises it waits for P V of all sub-tiles before.
           // The first sub-tile's warp always goes the long way: it puts the maxima where the others read them, also those of a sub-tile
           // without a live key (-inf; what lies there is an earlier item's).
-          bool may = t == 0;
+          bool may = FIRST;
+          if (!FIRST) {
 #pragma unroll
-          for (int q = 0; q < 4; ++q) may |= mx[q] > m[q] + kTop;
-          may = __any_sync(0xffffffffu, may);
+            for (int q = 0; q < 4; ++q) may |= mx[q] > m[q] + kTop;
+            may = __any_sync(0xffffffffu, may);
+          }
           if (!may && t + 1 < ns) named_barrier_arrive(told, 64);
           const float cur[4] = {seen.x, seen.y, seen.z, seen.w};
-          bool change = t == 0;
+          bool change = FIRST;
 #pragma unroll
           for (int q = 0; q < 4; ++q) change |= mx[q] > cur[q] + kTop || cur[q] != m[q];
           if (__any_sync(0xffffffffu, change)) {
             float alpha[4];
-            bool raised = t == 0;
+            bool raised = FIRST;
 #pragma unroll
             for (int q = 0; q < 4; ++q) {
               // the same for the four threads of a row
@@ -769,8 +774,7 @@ attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CU
               }
               m[q] = top;
             }
-            bool flat = false;
-            if (FLAT && t == 0) {
+            if (FLAT && FIRST) {
               if (ns >= kFlatMin) {
                 const float4 need = lds4(max_s);
                 flat = need.x <= m[0] && need.y <= m[1] && need.z <= m[2] && need.w <= m[3] && fminf(fminf(m[0], m[1]), fminf(m[2], m[3])) > -INFINITY;
@@ -779,7 +783,7 @@ attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CU
               if (lane == 0) asm volatile("st.shared.f32 [%0], %1;" ::"r"(flat_s), "f"(flat ? 1.f : 0.f) : "memory");
             }
             if (__any_sync(0xffffffffu, raised)) {
-              if (t > 0) {
+              if (!FIRST) {
                 // O is relative to the old maxima: P V of the sub-tile before must be in it, that of this one follows its P.
                 // (A parity tells only two phases apart, so the phase before has to be over: P V of sub-tile t - 4, which this group
                 // has to see done in any case, comes after that of t - 5.)
@@ -803,9 +807,9 @@ attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CU
               }
               if ((lane & 3) == 0) sts4(max_s, m);
               __syncwarp();
-              if (FLAT && t == 0) mbar_arrive_warp(looked);
+              if (FLAT && FIRST) mbar_arrive_warp(looked);
             }
-            if (flat) may = false;                         // nobody hands on in a flat item
+            if (FLAT && FIRST && flat) may = false;        // nobody hands on in a flat item
           }
           if (may && t + 1 < ns) named_barrier_arrive(told, 64);
           // P is free once P V of the group's last sub-tile has read it
@@ -836,11 +840,13 @@ attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CU
           tc_fence_before();
           mbar_arrive_warp(bar_p_full + 8 * g);
           s_ready = __all_sync(0xffffffffu, s_ready);
-          if (FLAT && t == 0 && lds1(flat_s) != 0.f) {
-            t += kGroups;
-            break;
-          }
+        };
+        if (t == 0 && ns > 0) {
+          look(std::true_type{});
+          t += kGroups;
         }
+        if (!flat)                                        // (a condition of its own: in the loop's it costs a twentieth)
+          for (; t < ns; t += kGroups) look(std::false_type{});
         if (FLAT) {
           const float2 scale2 = make_float2(scale, scale);
           for (; t < ns; t += kGroups) {
