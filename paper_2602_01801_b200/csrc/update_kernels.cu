@@ -79,6 +79,27 @@ __device__ __forceinline__ void convert_rows(const ConvertArgs::Tensor& x, int h
     *reinterpret_cast<uint2*>(x.dst + (static_cast<int64_t>(h) * x.n + row) * D + col) = o;
   }
 }
+// The rows of all heads by all threads of a launch, four loads of each under way.  (Head by head, each from the first thread on, the heads
+// followed one another and most threads had none.  Hash and conversion, d = 128, by two launches, so, now: 40 heads x 64 rows 9.4, 17.8, 6.3 us;
+// 40 x 600 32, 33.5, 13.5; 12 x 4680 66, 33, 25; 1 x 256 6.5, 6.6, 6.0.)
+template <int D>
+__device__ __forceinline__ void convert_heads(const ConvertArgs::Tensor& x, int H, int thread, int threads) {
+  constexpr int B = 4;
+  const int total = H * x.n * (D / 4);               // below 2^25
+  for (int q0 = thread; q0 < total; q0 += B * threads) {
+    float4 v[B];
+#pragma unroll
+    for (int b = 0; b < B; ++b) {
+      const int q = q0 + b * threads, row = q / (D / 4), h = row / x.n;
+      if (q < total) v[b] = *reinterpret_cast<const float4*>(x.src + h * x.hs + (row - h * x.n) * x.ts + q % (D / 4) * 4);
+    }
+#pragma unroll
+    for (int b = 0; b < B; ++b) {
+      const int q = q0 + b * threads;
+      if (q < total) *reinterpret_cast<uint2*>(x.dst + static_cast<int64_t>(q) * 4) = make_uint2(pack_bf16x2(v[b].x, v[b].y), pack_bf16x2(v[b].z, v[b].w));
+    }
+  }
+}
 __global__ void convert_kernel(const ConvertArgs a, int D) {
   chain_wait();
   convert_rows(a.t[blockIdx.z], blockIdx.y, D, blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x, static_cast<int64_t>(gridDim.x) * blockDim.x);
@@ -119,7 +140,7 @@ __device__ __forceinline__ uint4 pack_counts(const int (&v)[8]) {
 // whose bucket histograms the CTA writes.  With four of eight warps idle for blocks of 64, 40 x 10800 rows took 45 us, with two blocks a pass 37
 // (d = 64 29 -> 22); with a launch of their own for the histograms 33 (26).  Blocks of 128: 34 (21) us, 31 (24) with that launch.
 // F32: the rows are fp32 (conv.t[0]); the kernel rounds them on their way, writes them where the kernels behind it read them, and converts
-// conv's other tensors too (an update's values): one head x 256 rows, d = 64, 2.2 + 3.4 -> 4.9 us and a launch less for the host.
+// conv's other tensors too (an update's values): one head x 256 rows, d = 64, 2.2 + 3.4 -> 4.7 us and a launch less for the host.
 struct BlockHist {
   __nv_bfloat16* hist;         // [H][max_qb][hist_cols]
   int max_qb, hist_cols;
@@ -297,10 +318,8 @@ __global__ void __launch_bounds__(256, 2) prep_kernel(const __nv_bfloat16* __res
     }
   }
   if constexpr (F32) {
-    if (conv.count > 1)
-      for (int h = 0; h < H; ++h) convert_rows(conv.t[1], h, D, thread, threads);
-    if (conv.count > 2)
-      for (int h = 0; h < H; ++h) convert_rows(conv.t[2], h, D, thread, threads);
+    if (conv.count > 1) convert_heads<D>(conv.t[1], H, static_cast<int>(thread), static_cast<int>(threads));      // (by constants: an index puts the array on the stack)
+    if (conv.count > 2) convert_heads<D>(conv.t[2], H, static_cast<int>(thread), static_cast<int>(threads));
   }
 }
 static int launch_prep_generic(const CacheView& c, const __nv_bfloat16* x, int n, int64_t hs, int64_t ts, uint32_t* code_out,
