@@ -103,10 +103,17 @@ def _ptr(t) -> Optional[int]:
     return None if t is None else t.data_ptr()
 
 
+_raw_stream = None
+
+
 def _stream() -> int:
     # The current stream's handle without a Stream object around it, which takes the host 3.4 us to make: three of a small step's 72.
+    # torch has that only under a private name; where it is not there, through the object.
+    global _raw_stream
     import torch
-    return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
+    if _raw_stream is None:
+        _raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None) or (lambda device: torch.cuda.current_stream(device).cuda_stream)
+    return _raw_stream(torch.cuda.current_device())
 
 
 class Cache:
