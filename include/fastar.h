@@ -269,7 +269,8 @@ int fastar_cache_set_similarity_kernel(fastar_cache_t* cache, int32_t kind);
  *   o_i = softmax over {live slots of the kept blocks, bias ln m_j} U {segment tokens, bias 0}.
  * The block selection is unchanged (it ranks cache blocks only); keep_blocks >= CAP/Bk gives dense
  * attention over the whole cache plus the segment; an empty cache gives dense attention over the
- * segment.  sel_in / nsel_in as above (may be NULL).  1 <= ns <= max_tokens. */
+ * segment.  sel_in / nsel_in as above (may be NULL).  1 <= ns <= max_tokens.  A misaligned segment is
+ * refused before anything of the call is launched but the conversion of fp32 queries. */
 int fastar_annsa_attention_segment(fastar_cache_t* cache, const void* q, const void* k_seg, const void* v_seg,
                                    void* out, int32_t nq, int32_t ns, int64_t head_stride, int64_t token_stride,
                                    int64_t seg_head_stride, int64_t seg_token_stride, int32_t block_q,

@@ -35,7 +35,8 @@
 //     an SM's instruction caches bear (stalls for instructions: a twentieth of a warp's time, and a sixth with a little more code in the
 //     kernel), so the cut is a variant of its own;
 //   - items whose logits a bound keeps near the first sub-tile's need no maximum at all (see kFlatMin): the loop for them is what the
-//     arithmetic needs, 270 instructions, and the exponentials and the tensor core bound it (0.74 and 0.73 of the time at d = 128);
+//     arithmetic needs, some 270 instructions, and the tensor core and the exponentials' units are at 0.76 and 0.67 of the time at d = 128, 0.40
+//     and 0.71 at 64;
 //   - the CTA stays for its items, and the copies and Q K^T run ahead into the next one, whose first logits are there when the
 //     output of the last has left.
 // TMEM columns: S 4 x 64, P 4 x 32, O D; with key tiles of 64: S 3 x 64, P, O and Q D / 2 (AttnSmem::QT).  K and V tiles have a TMA ring
@@ -95,8 +96,9 @@ __device__ __forceinline__ float lds1(uint32_t addr) {
   asm volatile("ld.shared.f32 %0, [%1];" : "=f"(v) : "r"(addr));
   return v;
 }
-// 2^u of two logits on the FMA units, u < 2^22; 0 from -127 down, as the special-function units give it for a logit of -inf.  2^f on
-// [-1/2, 1/2] by a polynomial of degree 5, fitted to the least relative error (9.2e-8; that of ex2.approx is 1.2e-7) with 2^0 = 1.
+// 2^u of two logits on the FMA units, u < 2^22; 0 from -127 down, as the special-function units give it for a logit of -inf.  Adding 1.5 x 2^23
+// rounds u to the nearest integer, which goes to the exponent; 2^f of the rest, on [-1/2, 1/2], by a polynomial of degree 5 fitted to the least
+// relative error with 2^0 = 1.  Error 1.1e-7 at most, 1.7e-7 as worked out in fp32 (ex2.approx 1.2e-7); rounding to bf16 is 2e-3.
 __device__ __forceinline__ float2 poly_exp2(float2 u) {
   auto both = [](float v) { return make_float2(v, v); };
   constexpr float kRound = 12582912.f;                     // 1.5 x 2^23: the sum's last bits are the nearest integer
@@ -128,8 +130,8 @@ __device__ __forceinline__ void add_bf16x2(float2& s, uint32_t b) {
 // m are bounded apart 0.01.
 constexpr int kFlatMin = 8;
 // Pairs of every sixteen whose exponentials the FMA units work out: the special-function units take 512 cycles for a sub-tile's, the tensor
-// core 270 at d = 64 and 540 at 128.  Kernel time with 0 / 2 / 4 of sixteen: d = 64, 256 items of 128 sub-tiles 97.9 / 94.1 / 95.0 us; d = 128, 256 of
-// 256 201 / 200 / 202.
+// core 270 at d = 64 and 540 at 128.  Kernel time with 0 / 2 / 4 of sixteen: d = 64, 256 items of 128 sub-tiles 97.9 / 94.1 / 95.0 us; at d = 128 it
+// makes no difference (256 of 256 201 / 200 / 202), and has the same two.
 constexpr int kPolyPairs = 2;
 
 template <int D, int BKT>
