@@ -285,6 +285,12 @@ attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CU
             const __grid_constant__ CUtensorMap tm_sv, const CacheView c, const AttnArgs a) {
   using SM = AttnSmem<D, BKT>;
   constexpr bool FLAT = !GATHER;                     // prompt tokens have no bounds, and few tiles
+  // An item's first sub-tile as code of its own: in the loop, what only it does takes a twentieth of the loop's time, but items that are flat
+  // then run through more code.  In the loop -> apart: 12 heads x 4680 queries on 32 of 220 blocks, all of whose items look 110 -> 105 us, flat 95.8 ->
+  // 95.9; 8 x 4096 on 16 384 keys 240 -> 225 and 200.9 -> 201.6.  At d = 64, 64 of 1 024 blocks 124 -> 117, but flat 89.4 -> 91.4, 16 of 160 41.3 -> 39.9 and
+  // 31.7 -> 32.1; where items are cut (12 x 1560, 16 of 110 blocks, flat) 36.6 -> 38.3.
+  constexpr bool kApart = FLAT && D == 128 && !CUT;
+  constexpr int kFirst = 1, kOther = 0, kAny = 2;
   constexpr int RS = SM::RS, RK = SM::RK, RV = SM::RV, NB = SM::NB, SUB = SM::SUB;
   extern __shared__ __align__(1024) uint8_t smem_raw[];
   const uint32_t sbase = smem_u32(smem_raw);
@@ -701,11 +707,10 @@ attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CU
             m[0] = ref.x; m[1] = ref.y; m[2] = ref.z; m[3] = ref.w;
           }
         }
-        // A sub-tile whose maximum is looked for.  An item's first one is code of its own: inside the loop, what only it does took a twentieth of the
-        // loop's time.  Items that all look, before there were flat ones, with that in the loop, now: 12 heads x 4680 queries on 32 of 220 blocks
-        // 103-105, 110, 105 us, 8 x 4096 on 16384 keys 228, 240, 225, d = 64, 64 of 1 024 blocks 116, 124, 117.
+        // A sub-tile whose maximum is looked for: an item's first one (kFirst), another one (kOther), or whichever it is.
         auto look = [&](auto way) {
-          constexpr bool FIRST = decltype(way)::value;
+          constexpr int WAY = decltype(way)::value;
+          const bool first = WAY == kAny ? t == 0 : WAY == kFirst;
           const int tg = sub0 + t, jg = tg / SUB;
           const uint32_t sb = SM::QT ? tg % SM::NSB : 0;
           if (!s_ready) ok = ok && mbar_wait_warp(full, (tg / kGroups) & 1, abort_flag, c.status);
@@ -719,8 +724,8 @@ attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CU
           float2 bias[8];
 #pragma unroll
           for (int k = 0; k < 8; ++k) bias[k] = lds2(bp + 32 * k);
-          if (!FIRST) named_barrier_sync(heard, 64);
-          const float4 seen = FIRST ? make_float4(-INFINITY, -INFINITY, -INFINITY, -INFINITY) : lds4(max_s);
+          if (!first) named_barrier_sync(heard, 64);
+          const float4 seen = first ? make_float4(-INFINITY, -INFINITY, -INFINITY, -INFINITY) : lds4(max_s);
           bool p_free = tg < kGroups || mbar_test_wait(bar_pv_done + 8 * g, (tg / kGroups - 1) & 1);
           tmem_wait_ld();
           tc_fence_before();
@@ -742,20 +747,20 @@ attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CU
           // raises it waits for P V of all sub-tiles before.
           // The first sub-tile's warp always goes the long way: it puts the maxima where the others read them, also those of a sub-tile
           // without a live key (-inf; what lies there is an earlier item's).
-          bool may = FIRST;
-          if (!FIRST) {
+          bool may = first;
+          if (WAY != kFirst) {
 #pragma unroll
             for (int q = 0; q < 4; ++q) may |= mx[q] > m[q] + kTop;
             may = __any_sync(0xffffffffu, may);
           }
           if (!may && t + 1 < ns) named_barrier_arrive(told, 64);
           const float cur[4] = {seen.x, seen.y, seen.z, seen.w};
-          bool change = FIRST;
+          bool change = first, becomes_flat = false;
 #pragma unroll
           for (int q = 0; q < 4; ++q) change |= mx[q] > cur[q] + kTop || cur[q] != m[q];
           if (__any_sync(0xffffffffu, change)) {
             float alpha[4];
-            bool raised = FIRST;
+            bool raised = first;
 #pragma unroll
             for (int q = 0; q < 4; ++q) {
               // the same for the four threads of a row
@@ -776,16 +781,16 @@ attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CU
               }
               m[q] = top;
             }
-            if (FLAT && FIRST) {
+            if (FLAT && first) {
               if (ns >= kFlatMin) {
                 const float4 need = lds4(max_s);
-                flat = need.x <= m[0] && need.y <= m[1] && need.z <= m[2] && need.w <= m[3] && fminf(fminf(m[0], m[1]), fminf(m[2], m[3])) > -INFINITY;
-                flat = __all_sync(0xffffffffu, flat);
+                becomes_flat = need.x <= m[0] && need.y <= m[1] && need.z <= m[2] && need.w <= m[3] && fminf(fminf(m[0], m[1]), fminf(m[2], m[3])) > -INFINITY;
+                becomes_flat = __all_sync(0xffffffffu, becomes_flat);
               }
-              if (lane == 0) asm volatile("st.shared.f32 [%0], %1;" ::"r"(flat_s), "f"(flat ? 1.f : 0.f) : "memory");
+              if (lane == 0) asm volatile("st.shared.f32 [%0], %1;" ::"r"(flat_s), "f"(becomes_flat ? 1.f : 0.f) : "memory");
             }
             if (__any_sync(0xffffffffu, raised)) {
-              if (!FIRST) {
+              if (!first) {
                 // O is relative to the old maxima: P V of the sub-tile before must be in it, that of this one follows its P.
                 // (A parity tells only two phases apart, so the phase before has to be over: P V of sub-tile t - 4, which this group
                 // has to see done in any case, comes after that of t - 5.)
@@ -809,9 +814,9 @@ attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CU
               }
               if ((lane & 3) == 0) sts4(max_s, m);
               __syncwarp();
-              if (FLAT && FIRST) mbar_arrive_warp(looked);
+              if (FLAT && first) mbar_arrive_warp(looked);
             }
-            if (FLAT && FIRST && flat) may = false;        // nobody hands on in a flat item
+            if (becomes_flat) may = false;                 // nobody hands on in a flat item
           }
           if (may && t + 1 < ns) named_barrier_arrive(told, 64);
           // P is free once P V of the group's last sub-tile has read it
@@ -842,13 +847,24 @@ attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CU
           tc_fence_before();
           mbar_arrive_warp(bar_p_full + 8 * g);
           s_ready = __all_sync(0xffffffffu, s_ready);
+          if (WAY == kFirst) flat = becomes_flat;
         };
-        if (t == 0 && ns > 0) {
-          look(std::true_type{});
-          t += kGroups;
+        if (kApart) {
+          if (t == 0 && ns > 0) {
+            look(std::integral_constant<int, kFirst>{});
+            t += kGroups;
+          }
+          if (!flat)                                      // (a condition of its own: in the loop's it costs a twentieth)
+            for (; t < ns; t += kGroups) look(std::integral_constant<int, kOther>{});
+        } else if (!flat) {
+          for (; t < ns; t += kGroups) {
+            look(std::integral_constant<int, kAny>{});
+            if (FLAT && t == 0 && lds1(flat_s) != 0.f) {
+              t += kGroups;
+              break;
+            }
+          }
         }
-        if (!flat)                                        // (a condition of its own: in the loop's it costs a twentieth)
-          for (; t < ns; t += kGroups) look(std::false_type{});
         if (FLAT) {
           const float2 scale2 = make_float2(scale, scale);
           for (; t < ns; t += kGroups) {
