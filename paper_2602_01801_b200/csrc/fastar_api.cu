@@ -1045,8 +1045,8 @@ int fastar_attention_step_host(fastar_cache_t* c, const void* k_new_host, const 
   //   attend  : (planned, values up) commit, (hashed) AnnSA
   //   down    : AnnCA's outputs, AnnSA's outputs (two streams in turn, by slice)
   // 12 heads x 4680 tokens against 28 080 keys, bf16, four slices: 1 368 -> 1 150 to 1 210 us (46.3 MB up and 28.8 down take 952 at once).  With one
-  // stream for the downloads the call depends on when the kernels between them end: 1 235 to 1 310, but 1 173 to 1 193 with a search that takes
-  // 4 % longer.  (Means of 240 calls; single ones vary by 50 either way.)  Two streams against one, by shape: the same with 8-bit search 0.94, by the
+  // stream for the downloads the call depends on when the kernels between them end: on one box 1 235 to 1 310, but 1 173 to 1 193 with a search
+  // that takes 4 % longer; on another 1 180, and 1 214 with that search, where it is 1 187 with two.  (Means of 240 calls; single ones vary by 50.)  Two streams against one, by shape: the same with 8-bit search 0.94, by the
   // probe 0.94, 4 blocks kept of 147 0.94, 11 heads x 1 120 in fp32 0.94, 25 and 40 heads 1.00, 6 and 8 heads 1.01 and 1.015.  With two: slices
   // of 4, 4, 2 and 2 heads 1 214, of 4, 3, 3 and 2 1 221, three of 4 1 191; a stream for each download 1 145 to 1 160.  With one, against 1 190: 1 277
   // with two slices, 1 274 with six; 1 225 with the queries before the keys, 1 277 with AnnCA's output in one copy, 1 345 with the queries in
