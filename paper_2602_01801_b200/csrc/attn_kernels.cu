@@ -125,9 +125,10 @@ __device__ __forceinline__ void add_bf16x2(float2& s, uint32_t b) {
 // lie just below a power of two, where bf16 is finest: error against 64 bits 0.00230 -> 0.00233.  Nor may the bound be further above: with 96, as
 // far as fp32 sums bear, items stay flat in which the other loop would have raised, and behind a raise the row's largest probability is a power
 // of two.  Keys in the order of their clusters, logits of 1.5 to 4 times the usual size: 0.00209-0.00230 where the maximum is looked for,
-// 0.00224-0.00233 so.)  Items of fewer sub-tiles than kFlatMin don't ask.  The bounds are of the item's own blocks: where tokens have merged into
-// its slots thousands of times (12 heads, 8-bit search, m up to 2^10) 0.89 of the items are flat, by the bounds of a head 0.60, and if |k| and
-// m are bounded apart 0.01.
+// 0.00224-0.00233 so.)  Items of fewer sub-tiles than kFlatMin don't ask; with as many it pays (64 and 444 items of eight, d = 128: 10.6 and 26.6 us,
+// looking 11.5 and 28.8; d = 64: 9.4 and 22.4, 10.9 and 25.3).  The bounds are of the item's own blocks: where tokens have merged into its slots
+// thousands of times (12 heads, 8-bit search, m up to 2^10) 0.89 of the items are flat, by the bounds of a head 0.60, and if |k| and m are
+// bounded apart 0.01.
 constexpr int kFlatMin = 8;
 // Pairs of every sixteen whose exponentials the FMA units work out: the special-function units take 512 cycles for a sub-tile's, the tensor
 // core 270 at d = 64 and 540 at 128.  Kernel time with 0 / 2 / 4 of sixteen: d = 64, 256 items of 128 sub-tiles 97.9 / 94.1 / 95.0 us; at d = 128 it
